@@ -9,7 +9,7 @@
 //   warps 21, 22     one store warp per epilogue group: resolves the tile's stream offset by
 //                    look-back and copies the group's staging buffer out, while the group
 //                    already works on its next tile
-//   warps 16-19      loaders: cp.async NCHW -> shared memory in the MMA's MN-major layout
+//   warps 16-19      loaders: cp.async NCHW -> shared memory in the MMA's MN-major layout (128-byte swizzle)
 //   warp 20          one thread issues tcgen05.mma:  D[pixel][coef] = X_tile[pixel][c] * T[coef][c]
 // The basis T (bf16, K x C) stays resident in shared memory; the X tile streams through a ring
 // of 64-channel panels; the fp32 accumulators are double-buffered in tensor memory so that the
@@ -30,7 +30,8 @@ constexpr int kStages = 4;
 constexpr int kStageBytes = kPanelCh * TC_TILE_PIXELS * 2;   // 16 KB
 constexpr int kLag = 2;                           // cp.async groups kept in flight per loader thread; the
                                                   // remaining ring stage absorbs the MMA's latency
-constexpr int kStagingBytes = 15360;              // packed-bit staging per epilogue group (15 KB)
+constexpr int kStaticSmem = 1024;                 // the static shared variables, up to the ring's alignment
+constexpr int kStagingBytes = 15104;              // packed-bit staging per epilogue group (14.75 KB)
 constexpr int kEpiWarps = 16;                     // 2 groups x (2 column halves x 4 lane quarters)
 constexpr int kLoaderWarp0 = kEpiWarps, kMmaWarp = kEpiWarps + 4;
 constexpr int kStoreWarp0 = kMmaWarp + 1;         // two store warps follow
@@ -136,7 +137,7 @@ __device__ __forceinline__ void quantise_bits2(uint32_t acc0, uint32_t acc1, flo
 template <bool kPerChannel, bool kDebug, bool kPair, bool kHist>
 __global__ void __launch_bounds__(kThreads, 1) encode_tc_kernel(EncodeArgs a)
 {
-    extern __shared__ __align__(128) unsigned char smem[];
+    extern __shared__ __align__(1024) unsigned char smem[];      // swizzled ring stages: aligned to their 1 KB atoms
     __shared__ __align__(8) unsigned long long s_full[kStages], s_empty[kStages], s_tfull[2], s_tempty[2];
     __shared__ uint32_t s_tmem_base;
     __shared__ unsigned int s_warp_sums[2][4];
@@ -213,35 +214,41 @@ __global__ void __launch_bounds__(kThreads, 1) encode_tc_kernel(EncodeArgs a)
 
     if (warp >= kLoaderWarp0 && warp < kMmaWarp) {
         // ================= loaders =================
-        const int lw = warp - kLoaderWarp0, kk = lane & 7;
+        // A copy instruction of a warp moves whole runs of a channel's row -- 32 groups of 4 pixels of
+        // one channel, or, where rows allow 16 bytes, 16 groups of 8 pixels of two channels -- and
+        // touches two to four cache lines.  (Eight channels x 32 bytes per instruction, which the
+        // unswizzled operand layout asks for to spread over the banks, touched eight or more and held
+        // the whole kernel to 1.85 TB/s of input: 222 us for 256x14x14 x 4096 with the MMAs and the
+        // epilogue's work taken out.)  In the swizzled layout 64 pixels of a channel are 128 contiguous
+        // bytes, the 16-byte pieces exchanged by XOR with the channel modulo 8: no bank conflicts.
+        const int lw = warp - kLoaderWarp0;
+        const bool wide = (a.hw & 7) == 0 && ((uintptr_t)a.x & 15u) == 0;      // 16 bytes per copy
+        const int px = wide ? 8 * (lane & 15) : 4 * lane;          // first pixel of this lane's group in the tile
+        const int ch0 = wide ? 2 * lw + (lane >> 4) : lw;          // this lane's first channel of a panel, then every 8th / 4th
+        const uint32_t dst0 = (uint32_t)((px >> 6) * (kStageBytes / 2) + (px & 7) * 2);
+        const uint32_t piece = (uint32_t)((px & 63) >> 3);
         const __nv_bfloat16 *xin = reinterpret_cast<const __nv_bfloat16 *>(a.x);
         int it = 0;
         bool alive = true;
         for (long long tl = 0; tl < my_tiles && alive; ++tl) {
-            const long long tile = blockIdx.x + tl * gridDim.x;
-            const __nv_bfloat16 *src[2];
-            uint32_t dst_off[2], nbytes[2];
-#pragma unroll
-            for (int g = 0; g < 2; ++g) {
-                const int mg = 8 * lw + (lane >> 3) + 4 * g;          // group of 4 pixels
-                const long long p0 = tile * TC_TILE_PIXELS + 4 * mg;
-                const bool valid = p0 < a.pixels;
-                const long long img = valid ? p0 / a.hw : 0;
-                const long long s = valid ? p0 - img * a.hw : 0;
-                src[g] = xin + img * a.c * (long long)a.hw + s;
-                nbytes[g] = valid ? 8u : 0u;
-                dst_off[g] = (uint32_t)((mg >> 1) * 128 + kk * 16 + (mg & 1) * 8);
-            }
+            const long long p0 = (blockIdx.x + tl * gridDim.x) * TC_TILE_PIXELS + px;
+            const bool valid = p0 < a.pixels;
+            const long long img = valid ? p0 / a.hw : 0;
+            const __nv_bfloat16 *src = xin + img * a.c * (long long)a.hw + (valid ? p0 - img * a.hw : 0) + (long long)ch0 * a.hw;
+            const uint32_t nbytes = valid ? (wide ? 16u : 8u) : 0u;
             for (int kp = 0; kp < n_panels; ++kp, ++it) {
                 const int s = it % kStages;
                 if (!mbar_wait(smem_u32(&s_empty[s]), ((it / kStages) & 1) ^ 1)) { alive = false; break; }
-                const int k0 = kp * kPanelCh;
-                const int nk8 = min(kPanelCh, a.c - k0) >> 3;
-                const uint32_t stage = ring_addr + s * kStageBytes;
-                for (int k8 = 0; k8 < nk8; ++k8) {
-                    const long long ch_off = (long long)(k0 + 8 * k8 + kk) * a.hw;
-#pragma unroll
-                    for (int g = 0; g < 2; ++g) cp_async_8(stage + k8 * 2048 + dst_off[g], src[g] + ch_off, nbytes[g]);
+                const int nch = min(kPanelCh, a.c - kp * kPanelCh);
+                const uint32_t stage = ring_addr + s * kStageBytes + dst0;
+                if (wide) {
+#pragma unroll 4
+                    for (int ch = ch0; ch < nch; ch += 8, src += 8 * a.hw)
+                        cp_async_16(stage + (uint32_t)ch * 128u + ((piece ^ (uint32_t)(ch & 7)) << 4), src, nbytes);
+                } else {
+#pragma unroll 4
+                    for (int ch = ch0; ch < nch; ch += 4, src += 4 * a.hw)
+                        cp_async_8(stage + (uint32_t)ch * 128u + ((piece ^ (uint32_t)(ch & 7)) << 4), src, nbytes);
                 }
                 cp_async_commit();
                 if (it >= kLag) {
@@ -281,7 +288,7 @@ __global__ void __launch_bounds__(kThreads, 1) encode_tc_kernel(EncodeArgs a)
                     const int k0 = kp * kPanelCh;
                     const int nk16 = min(kPanelCh, a.c - k0) >> 4;
                     for (int q = 0; q < nk16; ++q) {
-                        const uint64_t adesc = make_smem_desc(ring_addr + s * kStageBytes + q * 4096, 2048, 128);
+                        const uint64_t adesc = make_smem_desc_mn_sw128(ring_addr + s * kStageBytes + q * 2048, kStageBytes / 2, 1024);
                         const uint64_t bdesc = make_smem_desc(basis_addr + ((k0 + 16 * q) >> 3) * 128, 128, b_sbo);
                         mma_bf16_ss_guarded(d_tmem, adesc, bdesc, idesc, (kp | q) != 0 ? 1u : 0u, issuer);
                     }
@@ -644,7 +651,7 @@ bool tc_encode_tc_supported(const tc_ctx *ctx, const EncodeArgs &a)
     if (a.splits != 1 && !(a.splits == 2 && a.k % 32 == 0) && !(a.splits == 4 && a.k % 64 == 0 && a.chunk_pixels == 1)) return false;
     if (a.groups != 1 && a.groups != a.k) return false;
     const SmemLayout l = smem_layout(a.c, a.k, enc_table_entries(a));
-    return (int)l.total + 512 <= ctx->max_smem_optin;       // leaves room for the static shared variables
+    return (int)l.total + kStaticSmem <= ctx->max_smem_optin;       // leaves room for the static shared variables
 }
 
 tc_status tc_launch_encode_tc(const tc_ctx *ctx, const EncodeArgs &a, cudaStream_t s)

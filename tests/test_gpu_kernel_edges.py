@@ -1,0 +1,46 @@
+"""Kernel branches that the parity cases do not separate, each at the sizes where it can go wrong."""
+import pytest
+import torch
+
+import paper_1905_10830_b200 as tc
+from synth import featuremaps as fm
+from tests import helpers as H
+from tests.test_gpu_parity import check_stream_against_oracle, check_symbols
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def ctx():
+    c = tc.tc_create(0)
+    yield c
+    c.close()
+
+
+def _same_stream(a, b):
+    n = a.total_bits() // 8
+    return a.total_bits() == b.total_bits() and torch.equal(a.words[:n], b.words[:n]) and torch.equal(a.tile_off, b.tile_off) \
+        and torch.equal(a.chunk_len[:a.layout.n_chunks], b.chunk_len[:b.layout.n_chunks])
+
+
+# Resident-basis encoder.  Rows of 8 k elements in a 16-byte aligned tensor are copied 16 bytes at a
+# time, others 8; the last tile is partly or nearly empty; panels of 64 channels end in remainders.
+@pytest.mark.parametrize("offset", [0, 4, 8])
+@pytest.mark.parametrize("c,h,w,n,bits", [(16, 4, 2, 1, 4), (80, 8, 8, 3, 5), (208, 12, 12, 2, 4), (256, 14, 14, 1, 6), (48, 2, 10, 13, 8)])
+def test_resident_encoder_copies(ctx, c, h, w, n, bits, offset):
+    spec = fm.LayerSpec(c, h, w, 0.9, None, 11000 + c + h)
+    o = H.oracle_side(spec, bits, max(3, 2 * c // (h * w) + 1), n, torch.bfloat16, False)
+    m = H.import_model(tc, ctx, o["model"], torch.bfloat16)
+    cb = tc.tc_codebook_import(ctx, o["lengths"], bits)
+    buf = torch.empty(o["x"].numel() + 16, dtype=torch.bfloat16, device="cuda")
+    x = buf[offset:offset + o["x"].numel()].view(o["x"].shape)
+    x.copy_(o["x"])
+    enc = tc.tc_encode(ctx, m, cb, x, debug=True)
+    assert tc.tc_get_status(ctx) == 0 and tc.tc_last_path(ctx) == 1
+    q = enc.symbols.cpu().numpy()
+    check_symbols(q, o, exact=False)
+    check_stream_against_oracle(enc, q, o["lengths"], bits)
+    # the kernel without the debug outputs writes the same stream
+    assert _same_stream(tc.tc_encode(ctx, m, cb, x), enc)
+    assert tc.tc_get_status(ctx) == 0
+    m.close(); cb.close()
