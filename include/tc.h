@@ -238,9 +238,9 @@ tc_status tc_host_huffman_lengths(const uint64_t *counts, int32_t nsym, int32_t 
 /* The fit's device eigensolver on its own (Section 3.1, "Linear transform": the PCA matrix is
  * the eigenvector matrix of the calibration covariance): `a` is a symmetric n x n matrix in DEVICE memory
  * (fp64, row-major, left untouched), evals [n] and evecs [n][n] DEVICE arrays, with the same
- * conventions as tc_host_eigh.  One-sided Jacobi, one launch per round of n / 2 disjoint
- * column pairs; synchronises the stream once per sweep.  *sweeps (HOST, may be NULL) receives
- * the number of sweeps.  Errors: INVALID_ARG, NOT_CONVERGED (150 sweeps), CUDA. */
+ * conventions as tc_host_eigh.  One-sided Jacobi in one cooperative launch;
+ * synchronises the stream.  *sweeps (HOST, may be NULL) receives the number of sweeps.
+ * Errors: INVALID_ARG, NOT_CONVERGED (150 sweeps), TIMEOUT, CUDA. */
 tc_status tc_device_eigh(tc_ctx *ctx, const double *a, int32_t n, double *evals, double *evecs, int32_t *sweeps,
                          void *cuda_stream);
 /* Host eigensolver (TC_EIG_HOST): eigendecomposition of a symmetric n x n matrix `a`

@@ -3,12 +3,14 @@
 // running moments to the covariance, its eigendecomposition, the rounded basis and the constants
 // the codec kernels read -- without moving a C x C matrix to the host.
 //
-// Eigensolver: one-sided Jacobi (Hestenes).  With G = A and V = I, plane rotations applied to
-// the same pair of columns of G and V make the columns of G mutually orthogonal; then G = A V,
-// the columns of V are eigenvectors and, for a symmetric A, v_i . (A v_i) the eigenvalues.  The
-// n / 2 column pairs of a round of a round-robin tournament are disjoint, so one launch rotates
-// them all, one block per pair; n - 1 rounds visit every pair once (a sweep).  Columns are stored
-// as rows (A is symmetric), so a block reads and writes contiguous memory.
+// Eigensolver: one-sided Jacobi (Hestenes) on the shifted matrix G = A / |A|_F + s I.  Plane
+// rotations of pairs of columns make the columns of G mutually orthogonal; then G = U S and, G
+// being positive definite (s > 1), the columns of U are the eigenvectors of A.  Columns are stored
+// as rows (A is symmetric).  All columns of G have norms within [s - 1, s + 1], which the method
+// profits from three times: the eigenvectors are the normalised columns (no second matrix is
+// rotated), inner products compare against relative bounds, and the gaps between the squared
+// singular values are linear, not quadratic, in the eigenvalue gaps (a graded covariance: 13
+// instead of 16 sweeps, a geometric spectrum over 12 decades 24 instead of 40).
 #include "tc_internal.h"
 
 #include <cuda_bf16.h>
@@ -22,9 +24,10 @@
 namespace {
 
 constexpr int kPairThreads = 128;
-// A covariance with a steeply graded spectrum takes 20 to 40 sweeps (the method works on the
-// squared spectrum); an ordinary matrix under 10.
+// A covariance with a steeply graded spectrum takes 13 to 25 sweeps, an ordinary matrix under 10.
 constexpr int kMaxSweeps = 150;
+constexpr double kShift = 1.25;                        // of |A|_F: no eigenvalue of G is below 0.25
+constexpr unsigned long long kBarrierLimitNs = 2000000000ull;
 
 __device__ __forceinline__ double block_sum(double v, double *s_red)
 {
@@ -64,19 +67,35 @@ __global__ void scale_mirror_kernel(double *cov, int c, double denom)
     cov[(size_t)b * c + a] = v;
 }
 
-__global__ void jacobi_init_kernel(const double *a, int c, double *g, double *vt, double *frob2)
+// device bookkeeping of one decomposition, zeroed before use
+struct JacobiState {
+    double frob2;
+    unsigned int arrived;                              // grid barrier: blocks that have come, over all barriers
+    unsigned int failed;                               // a bounded wait ran out
+    unsigned int sweeps;                               // sweeps done; the last one found nothing to rotate
+    unsigned int converged;
+    unsigned int rotations[kMaxSweeps];                // per sweep
+};
+
+__global__ void frobenius_kernel(const double *a, int c, JacobiState *st)
 {
     __shared__ double s_red[kPairThreads / 32];
-    const int r = blockIdx.x;
     double acc = 0.0;
     for (int j = threadIdx.x; j < c; j += blockDim.x) {
-        const double v = a[(size_t)r * c + j];
-        g[(size_t)r * c + j] = v;
-        vt[(size_t)r * c + j] = (j == r) ? 1.0 : 0.0;
+        const double v = a[(size_t)blockIdx.x * c + j];
         acc += v * v;
     }
     acc = block_sum(acc, s_red);
-    if (threadIdx.x == 0) atomicAdd(frob2, acc);
+    if (threadIdx.x == 0) atomicAdd(&st->frob2, acc);
+}
+
+// g = a / |a|_F + s I, rows padded to `ld` with zeros; rows past c are zero (nothing rotates them)
+__global__ void jacobi_init_kernel(const double *a, int c, double *g, int ld, const JacobiState *st)
+{
+    const int r = blockIdx.x;
+    const double f2 = st->frob2, inv = f2 > 0.0 ? 1.0 / sqrt(f2) : 0.0;
+    for (int j = threadIdx.x; j < ld; j += blockDim.x)
+        g[(size_t)r * ld + j] = (r < c && j < c) ? a[(size_t)r * c + j] * inv + (j == r ? kShift : 0.0) : 0.0;
 }
 
 // The pair of round `round` played at table `t` (n even): player n - 1 stays, the others rotate.
@@ -88,57 +107,221 @@ __device__ __forceinline__ void round_robin_pair(int n, int round, int t, int &p
     if (p > q) { const int x = p; p = q; q = x; }
 }
 
-__global__ void jacobi_round_kernel(double *g, double *vt, int c, int n_even, int round, double tol, const double *frob2,
-                                    unsigned int *rotations)
+// All blocks of a cooperative launch have come `n`-th time; false if the wait ran out (or one of
+// another block did): everyone leaves then.
+__device__ __forceinline__ bool grid_barrier(JacobiState *st, unsigned int n)
 {
-    __shared__ double s_red[kPairThreads / 32];
-    int p, q;
-    round_robin_pair(n_even, round, blockIdx.x, p, q);
-    if (q >= c) return;                                 // the bye of an odd n
-    double *gp = g + (size_t)p * c, *gq = g + (size_t)q * c;
-    double alpha = 0.0, beta = 0.0, gamma = 0.0;
-    for (int j = threadIdx.x; j < c; j += blockDim.x) {
-        const double x = gp[j], y = gq[j];
-        alpha += x * x; beta += y * y; gamma += x * y;
+    __shared__ bool s_ok;
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        bool ok = true;
+        const unsigned int target = n * gridDim.x;
+        atomicAdd(&st->arrived, 1u);
+        unsigned long long t0, t1;
+        asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t0));
+        unsigned int seen;
+        while (true) {
+            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(&st->arrived) : "memory");
+            if (seen >= target) break;
+            asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t1));
+            if (t1 - t0 > kBarrierLimitNs) { ok = false; atomicExch(&st->failed, 1u); break; }
+        }
+        s_ok = ok;
     }
-    alpha = block_sum(alpha, s_red);
-    beta = block_sum(beta, s_red);
-    gamma = block_sum(gamma, s_red);
-    // The columns carry an absolute error of about eps |A| (every rotation with a large column
-    // leaves that much in a small one), so their inner product is known to eps |A| times the
-    // larger norm, whatever the smaller one: below that a rotation would only chase noise.  (The
-    // eigenvectors of A are not determined any better than that by A itself.)
-    const double bigger = sqrt(fmax(alpha, beta));
-    if (fabs(gamma) <= tol * sqrt(*frob2) * bigger) return;
-    const double zeta = (beta - alpha) / (2.0 * gamma);
-    const double t = (zeta >= 0.0 ? 1.0 : -1.0) / (fabs(zeta) + sqrt(1.0 + zeta * zeta));
-    const double cs = 1.0 / sqrt(1.0 + t * t), sn = cs * t;
-    double *vp = vt + (size_t)p * c, *vq = vt + (size_t)q * c;
-    for (int j = threadIdx.x; j < c; j += blockDim.x) {
-        const double x = gp[j], y = gq[j];
-        gp[j] = cs * x - sn * y;
-        gq[j] = sn * x + cs * y;
-        const double u = vp[j], w = vq[j];
-        vp[j] = cs * u - sn * w;
-        vq[j] = sn * u + cs * w;
-    }
-    if (threadIdx.x == 0) atomicAdd(rotations, 1u);
+    __syncthreads();
+    return s_ok;
 }
 
-// eigenvalue of row i of vt against the untouched matrix: v^T A v
-__global__ void rayleigh_kernel(const double *a, const double *vt, int c, double *lambda)
+__device__ __forceinline__ double warp_sum(double v)
+{
+#pragma unroll
+    for (int d = 16; d > 0; d >>= 1) v += __shfl_xor_sync(0xffffffffu, v, d);
+    return v;
+}
+
+template <int R>
+__device__ __forceinline__ double norm2(const double2 (&x)[R])
+{
+    double a = 0.0, b = 0.0;
+#pragma unroll
+    for (int i = 0; i < R; ++i) { a += x[i].x * x[i].x; b += x[i].y * x[i].y; }
+    return warp_sum(a + b);
+}
+
+// Makes the columns x and y (2 R elements per lane, squared norms al and be) orthogonal; false if
+// they already are, to rounding: below `tol2` (squared) of the norms a rotation would only chase noise.
+// The angle is computed in fp32 -- the rotations' angles steer the iteration, an error of 1e-7 of
+// one leaves 1e-7 of the inner product for the next sweep -- but the matrix applied is a rotation
+// to fp64: cosine and tan(angle / 2) follow from that tangent by a cubic correction of the
+// fp32 reciprocal (square root), and the update x -= s (y + u x), y += s (x - u y) rounds in
+// proportion to the angle.
+template <int R>
+__device__ __forceinline__ bool rotate_pair(double2 (&x)[R], double2 (&y)[R], double &al, double &be, double tol2)
+{
+    double g0 = 0.0, g1 = 0.0;
+#pragma unroll
+    for (int i = 0; i < R; ++i) { g0 += x[i].x * y[i].x; g1 += x[i].y * y[i].y; }
+    const double ga = warp_sum(g0 + g1);
+    if (ga * ga <= tol2 * al * be) return false;
+    // t = tan of the smaller angle that annuls the inner product; norms lie within [1/16, 6], and the
+    // inner product is above the tolerance: no square below leaves the range of fp32
+    const float d = (float)(be - al), g2 = (float)(2.0 * ga), h = sqrtf(d * d + g2 * g2);
+    const double t = (double)__fdividef(g2, d + (d >= 0.f ? h : -h));
+    const double q = fma(t, t, 1.0);
+    const double r0 = (double)rsqrtf((float)q), re = fma(-q * r0, r0, 1.0);
+    const double cs = fma(r0 * re, fma(re, 0.375, 0.5), r0);              // 1 / sqrt(q)
+    const double k = 1.0 + cs, k0 = (double)__frcp_rn((float)k), ke = fma(-k, k0, 1.0);
+    const double sn = cs * t, u = sn * fma(k0 * ke, 1.0 + ke, k0);         // sin / (1 + cos)
+#pragma unroll
+    for (int i = 0; i < R; ++i) {
+        const double2 v = x[i], w = y[i];
+        x[i] = make_double2(fma(-sn, fma(u, v.x, w.x), v.x), fma(-sn, fma(u, v.y, w.y), v.y));
+        y[i] = make_double2(fma(sn, fma(-u, w.x, v.x), w.x), fma(sn, fma(-u, w.y, v.y), w.y));
+    }
+    al = fma(-t, ga, al);
+    be = fma(t, ga, be);
+    return true;
+}
+
+// The columns are dealt into blocks of B.  A thread block plays the block pairs of one table of a
+// round-robin tournament over the column blocks: it holds the first column block in registers
+// (warp w: column w), the second in shared memory, and in B inner rounds rotates every column of
+// the one against every column of the other (warp w takes column w + r).  The first round of a
+// sweep also rotates the pairs inside both column blocks.  Between rounds the blocks change
+// tables through global memory (L2), behind a grid barrier.
+// What bounds it: the latency of an inner round -- loads, the inner product's shuffles, the angle,
+// a block barrier: 960 cycles at 64 rows -- then, from about 256 rows on (1480 cycles), the shared
+// memory and the fp64 pipe; a table change costs 6500 cycles.  So columns' norms are carried
+// through the inner rounds instead of recomputed, and one launch does the whole decomposition:
+// with a launch per round of single pairs (6.3 us each) n = 256 took 24 ms, now 3.2.  B = 16 halves
+// the table changes of B = 8; from 512 rows on the registers only hold B = 8.
+template <int R, int B>
+__global__ void __launch_bounds__(B * 32, 1) jacobi_kernel(double *g, int n_blocks, double tol2, JacobiState *st)
+{
+    constexpr int ld = 64 * R;
+    extern __shared__ __align__(16) double s_col[];    // [2][B][ld]; the first half only for the pairs inside a block
+    __shared__ double s_norm[B];                       // squared norms of the second block's columns
+    __shared__ unsigned int s_rot;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    double *s_first = s_col, *s_second = s_col + (size_t)B * ld;
+    auto column = [&](double *base, int i) { return reinterpret_cast<double2 *>(base + (size_t)i * ld) + lane; };
+    double2 x[R], y[R];
+    unsigned int barriers = 0;
+    for (int sweep = 0; sweep < kMaxSweeps; ++sweep) {
+        unsigned int rotated = 0;
+        for (int round = 0; round < n_blocks - 1; ++round) {
+            int bi, bj;
+            round_robin_pair(n_blocks, round, blockIdx.x, bi, bj);
+            const double2 *gi = column(g, bi * B + warp), *gj = column(g, bj * B + warp);
+#pragma unroll
+            for (int i = 0; i < R; ++i) { x[i] = __ldcg(gi + 32 * i); y[i] = __ldcg(gj + 32 * i); }
+#pragma unroll
+            for (int i = 0; i < R; ++i) column(s_second, warp)[32 * i] = y[i];
+            if (round == 0) {
+                // the pairs inside the two column blocks: warps 0 .. B/2 - 1 the first block's, the others the second's
+#pragma unroll
+                for (int i = 0; i < R; ++i) column(s_first, warp)[32 * i] = x[i];
+                double *half = warp < B / 2 ? s_first : s_second;
+#pragma unroll 1
+                for (int r = 0; r < B - 1; ++r) {
+                    __syncthreads();
+                    int p, q;
+                    round_robin_pair(B, r, warp & (B / 2 - 1), p, q);
+#pragma unroll
+                    for (int i = 0; i < R; ++i) { x[i] = column(half, p)[32 * i]; y[i] = column(half, q)[32 * i]; }
+                    double al = norm2<R>(x), be = norm2<R>(y);
+                    if (rotate_pair<R>(x, y, al, be, tol2)) {
+                        ++rotated;
+#pragma unroll
+                        for (int i = 0; i < R; ++i) { column(half, p)[32 * i] = x[i]; column(half, q)[32 * i] = y[i]; }
+                    }
+                }
+                __syncthreads();
+#pragma unroll
+                for (int i = 0; i < R; ++i) { x[i] = column(s_first, warp)[32 * i]; y[i] = column(s_second, warp)[32 * i]; }
+            }
+            double al = norm2<R>(x);
+            const double own = norm2<R>(y);
+            if (lane == 0) s_norm[warp] = own;
+#pragma unroll 1
+            for (int r = 0; r < B; ++r) {
+                __syncthreads();
+                const int qi = (warp + r) & (B - 1);
+                double2 *cq = column(s_second, qi);
+                double be = s_norm[qi];
+#pragma unroll
+                for (int i = 0; i < R; ++i) y[i] = cq[32 * i];
+                if (rotate_pair<R>(x, y, al, be, tol2)) {
+                    ++rotated;
+                    __syncwarp();
+                    if (lane == 0) s_norm[qi] = be;
+#pragma unroll
+                    for (int i = 0; i < R; ++i) cq[32 * i] = y[i];
+                }
+            }
+            __syncthreads();
+            double2 *oi = column(g, bi * B + warp), *oj = column(g, bj * B + warp);
+#pragma unroll
+            for (int i = 0; i < R; ++i) { __stcg(oi + 32 * i, x[i]); __stcg(oj + 32 * i, column(s_second, warp)[32 * i]); }
+            if (round == n_blocks - 2) {
+                if (threadIdx.x == 0) s_rot = 0;
+                __syncthreads();
+                if (lane == 0 && rotated) atomicAdd(&s_rot, rotated);
+                __syncthreads();
+                if (threadIdx.x == 0 && s_rot) atomicAdd(&st->rotations[sweep], s_rot);
+            }
+            if (!grid_barrier(st, ++barriers)) return;
+        }
+        if (__ldcg(&st->rotations[sweep]) == 0) {
+            if (blockIdx.x == 0 && threadIdx.x == 0) { st->sweeps = sweep + 1; st->converged = 1; }
+            return;
+        }
+    }
+    if (blockIdx.x == 0 && threadIdx.x == 0) st->sweeps = kMaxSweeps;
+}
+
+// Normalises kVec columns of g into rows of vt and takes their Rayleigh quotients v^T A v against the
+// untouched matrix.  A thread owns columns j of A and reads them row by row (coalesced) once for
+// all kVec vectors.
+constexpr int kVec = 4;
+__global__ void rayleigh_kernel(const double *a, const double *g, int ld, int c, double *vt, double *lambda)
 {
     __shared__ double s_red[kPairThreads / 32];
-    const double *v = vt + (size_t)blockIdx.x * c;
-    double acc = 0.0;
-    for (int r = threadIdx.x; r < c; r += blockDim.x) {
-        const double *row = a + (size_t)r * c;
-        double w = 0.0;
-        for (int j = 0; j < c; ++j) w += row[j] * v[j];
-        acc += v[r] * w;
+    __shared__ double s_v[kVec][TC_MAX_C];
+    const int first = blockIdx.x * kVec;
+    for (int k = 0; k < kVec; ++k) {
+        const int i = first + k;
+        double acc = 0.0;
+        for (int j = threadIdx.x; j < c; j += blockDim.x) {
+            const double v = i < c ? g[(size_t)i * ld + j] : 0.0;
+            s_v[k][j] = v;
+            acc += v * v;
+        }
+        const double norm = sqrt(block_sum(acc, s_red));
+        for (int j = threadIdx.x; j < c && i < c; j += blockDim.x) {
+            const double v = s_v[k][j] / norm;
+            s_v[k][j] = v;
+            vt[(size_t)i * c + j] = v;
+        }
     }
-    acc = block_sum(acc, s_red);
-    if (threadIdx.x == 0) lambda[blockIdx.x] = acc;
+    __syncthreads();
+    double acc[kVec] = {};
+    for (int j = threadIdx.x; j < c; j += blockDim.x) {
+        double w[kVec] = {};
+#pragma unroll 4
+        for (int r = 0; r < c; ++r) {
+            const double ar = a[(size_t)r * c + j];
+#pragma unroll
+            for (int k = 0; k < kVec; ++k) w[k] += ar * s_v[k][r];
+        }
+#pragma unroll
+        for (int k = 0; k < kVec; ++k) acc[k] += w[k] * s_v[k][j];
+    }
+    for (int k = 0; k < kVec; ++k) {
+        const double t = block_sum(acc[k], s_red);
+        if (threadIdx.x == 0 && first + k < c) lambda[first + k] = t;
+    }
 }
 
 // Descending eigenvalues (equal ones in their original order); each vector signed so that its
@@ -146,21 +329,36 @@ __global__ void rayleigh_kernel(const double *a, const double *vt, int c, double
 __global__ void order_sign_kernel(const double *vt, const double *lambda, int c, double *evals, double *evecs)
 {
     __shared__ int s_rank, s_big;
-    const int i = blockIdx.x;
+    __shared__ double s_mag[kPairThreads / 32];
+    __shared__ int s_at[kPairThreads / 32];
+    const int i = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const double *v = vt + (size_t)i * c;
+    const double li = lambda[i];
+    if (threadIdx.x == 0) s_rank = 0;
+    __syncthreads();
+    int before = 0, at = c;
+    double mag = -1.0;
+    for (int j = threadIdx.x; j < c; j += blockDim.x) {
+        const double lj = lambda[j], m = fabs(v[j]);
+        before += (lj > li || (lj == li && j < i)) ? 1 : 0;
+        if (m > mag) { mag = m; at = j; }
+    }
+    before = __reduce_add_sync(0xffffffffu, before);
+#pragma unroll
+    for (int d = 16; d > 0; d >>= 1) {
+        const double om = __shfl_xor_sync(0xffffffffu, mag, d);
+        const int oa = __shfl_xor_sync(0xffffffffu, at, d);
+        if (om > mag || (om == mag && oa < at)) { mag = om; at = oa; }
+    }
+    if (lane == 0) { s_mag[warp] = mag; s_at[warp] = at; atomicAdd(&s_rank, before); }
+    __syncthreads();
     if (threadIdx.x == 0) {
-        const double li = lambda[i];
-        int rank = 0;
-        for (int j = 0; j < c; ++j) rank += (lambda[j] > li || (lambda[j] == li && j < i)) ? 1 : 0;
-        const double *v = vt + (size_t)i * c;
-        int big = 0;
-        for (int j = 1; j < c; ++j)
-            if (fabs(v[j]) > fabs(v[big])) big = j;
-        s_rank = rank;
-        s_big = big;
-        evals[rank] = li;
+        for (int w = 1; w < kPairThreads / 32; ++w)
+            if (s_mag[w] > mag || (s_mag[w] == mag && s_at[w] < at)) { mag = s_mag[w]; at = s_at[w]; }
+        s_big = min(at, c - 1);
+        evals[s_rank] = li;
     }
     __syncthreads();
-    const double *v = vt + (size_t)i * c;
     const double sgn = v[s_big] < 0.0 ? -1.0 : 1.0;
     for (int j = threadIdx.x; j < c; j += blockDim.x) evecs[(size_t)s_rank * c + j] = sgn * v[j];
 }
@@ -257,34 +455,59 @@ tc_status tc_launch_scale_mirror(double *cov, int c, double denom, cudaStream_t 
     return cudaGetLastError() == cudaSuccess ? TC_OK : TC_ERR_CUDA;
 }
 
-size_t tc_eigh_device_workspace_bytes(int c) { return (2 * (size_t)c * c + (size_t)c + 2) * sizeof(double); }
+// Column blocks and padding of the Jacobi kernel for c columns: rows of 64 R elements, blocks of B
+// columns, an even number of them.
+struct JacobiShape { int r, b, n_blocks, ld; };
+static JacobiShape jacobi_shape(int c)
+{
+    JacobiShape j;
+    const int need = (c + 63) / 64;
+    j.r = need <= 2 ? need : need <= 4 ? 4 : need <= 6 ? 6 : need <= 8 ? 8 : need <= 12 ? 12 : 16;
+    j.b = j.r <= 8 ? 16 : 8;
+    j.ld = 64 * j.r;
+    j.n_blocks = 2 * ((c + 2 * j.b - 1) / (2 * j.b));
+    return j;
+}
+
+size_t tc_eigh_device_workspace_bytes(int c)
+{
+    const JacobiShape j = jacobi_shape(c);
+    return ((size_t)j.n_blocks * j.b * j.ld + (size_t)c * c + (size_t)c) * sizeof(double) + sizeof(JacobiState);
+}
 
 // a: [c][c] symmetric, DEVICE, left untouched.  evals [c], evecs [c][c] (row j = eigenvector of
 // evals[j]), DEVICE.  `work`: tc_eigh_device_workspace_bytes(c) bytes, DEVICE.  Synchronises the
-// stream once per sweep (a 4-byte read of the rotation count).
+// stream once (the number of sweeps comes back).
 tc_status tc_eigh_device(const double *a, int c, double *evals, double *evecs, void *work, int *sweeps_out, cudaStream_t s)
 {
-    if (c < 1) return TC_ERR_INVALID_ARG;
-    double *g = static_cast<double *>(work), *vt = g + (size_t)c * c, *lambda = vt + (size_t)c * c, *frob2 = lambda + c;
-    unsigned int *rotations = reinterpret_cast<unsigned int *>(frob2 + 1);
-    TC_CUDA(cudaMemsetAsync(frob2, 0, 2 * sizeof(double), s));
-    jacobi_init_kernel<<<c, kPairThreads, 0, s>>>(a, c, g, vt, frob2);
-    const int n_even = (c + 1) & ~1;
-    const double tol = (double)(c < 16 ? 16 : c) * DBL_EPSILON;
-    int sweeps = 0;
-    bool converged = c == 1;
-    for (; sweeps < kMaxSweeps && !converged; ++sweeps) {
-        TC_CUDA(cudaMemsetAsync(rotations, 0, sizeof(unsigned int), s));
-        for (int round = 0; round < n_even - 1; ++round)
-            jacobi_round_kernel<<<n_even / 2, kPairThreads, 0, s>>>(g, vt, c, n_even, round, tol, frob2, rotations);
-        unsigned int n_rot = 0;
-        TC_CUDA(cudaMemcpyAsync(&n_rot, rotations, sizeof(n_rot), cudaMemcpyDeviceToHost, s));
-        TC_CUDA(cudaStreamSynchronize(s));
-        converged = n_rot == 0;
-    }
-    if (sweeps_out) *sweeps_out = sweeps;
-    if (!converged) return TC_ERR_NOT_CONVERGED;
-    rayleigh_kernel<<<c, kPairThreads, 0, s>>>(a, vt, c, lambda);
+    if (c < 1 || c > TC_MAX_C) return TC_ERR_INVALID_ARG;
+    const JacobiShape js = jacobi_shape(c);
+    double *g = static_cast<double *>(work), *vt = g + (size_t)js.n_blocks * js.b * js.ld, *lambda = vt + (size_t)c * c;
+    JacobiState *st = reinterpret_cast<JacobiState *>(lambda + c);
+    TC_CUDA(cudaMemsetAsync(st, 0, sizeof(JacobiState), s));
+    frobenius_kernel<<<c, kPairThreads, 0, s>>>(a, c, st);
+    jacobi_init_kernel<<<js.n_blocks * js.b, kPairThreads, 0, s>>>(a, c, g, js.ld, st);
+    // (the rounding of an inner product and of the columns since their rotation grows like sqrt(c);
+    // a cluster of m equal eigenvalues is only resolved to m times the bound)
+    const double tol = 8.0 * sqrt((double)(c < 16 ? 16 : c)) * DBL_EPSILON;
+    double tol2 = tol * tol;
+    int n_blocks = js.n_blocks;
+    const void *kernel = js.r == 1 ? (const void *)jacobi_kernel<1, 16> : js.r == 2 ? (const void *)jacobi_kernel<2, 16>
+                       : js.r == 4 ? (const void *)jacobi_kernel<4, 16> : js.r == 6 ? (const void *)jacobi_kernel<6, 16>
+                       : js.r == 8 ? (const void *)jacobi_kernel<8, 16> : js.r == 12 ? (const void *)jacobi_kernel<12, 8>
+                                   : (const void *)jacobi_kernel<16, 8>;
+    const size_t smem = 2 * (size_t)js.b * js.ld * sizeof(double);
+    TC_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    void *params[] = {&g, &n_blocks, &tol2, &st};
+    // cooperative: the blocks wait for one another between rounds
+    TC_CUDA(cudaLaunchCooperativeKernel(kernel, dim3(js.n_blocks / 2), dim3(js.b * 32), params, smem, s));
+    JacobiState got;
+    TC_CUDA(cudaMemcpyAsync(&got, st, sizeof(got), cudaMemcpyDeviceToHost, s));
+    TC_CUDA(cudaStreamSynchronize(s));
+    if (sweeps_out) *sweeps_out = (int)got.sweeps;
+    if (got.failed) return TC_ERR_TIMEOUT;
+    if (!got.converged) return TC_ERR_NOT_CONVERGED;
+    rayleigh_kernel<<<(c + kVec - 1) / kVec, kPairThreads, 0, s>>>(a, g, js.ld, c, vt, lambda);
     order_sign_kernel<<<c, kPairThreads, 0, s>>>(vt, lambda, c, evals, evecs);
     return cudaGetLastError() == cudaSuccess ? TC_OK : TC_ERR_CUDA;
 }

@@ -1,4 +1,5 @@
 """Kernel branches that the parity cases do not separate, each at the sizes where it can go wrong."""
+import numpy as np
 import pytest
 import torch
 
@@ -44,3 +45,23 @@ def test_resident_encoder_copies(ctx, c, h, w, n, bits, offset):
     assert _same_stream(tc.tc_encode(ctx, m, cb, x), enc)
     assert tc.tc_get_status(ctx) == 0
     m.close(); cb.close()
+
+
+# Device eigensolver: every row / block shape of its kernel (blocks of 16 columns up to 512 rows, of 8
+# beyond; 33 and 65 columns leave column blocks that are empty), and spectra that reach below zero.
+@pytest.mark.parametrize("n,shift", [(16, 0.0), (31, 0.5), (33, 0.0), (65, 0.3), (130, 0.0), (300, 0.5), (384, 0.0), (513, 0.4), (640, 0.0)])
+def test_device_eigh_block_shapes_and_indefinite(ctx, n, shift):
+    rng = np.random.default_rng(300 + n)
+    q, _ = np.linalg.qr(rng.standard_normal((n, n)))
+    lam = np.sort(rng.uniform(0.0, 1.0, n) - shift)[::-1]
+    a = (q * lam) @ q.T
+    a = (a + a.T) / 2
+    evals, evecs, sweeps = tc.tc_device_eigh(ctx, torch.from_numpy(a).cuda())
+    evals, evecs = evals.cpu().numpy(), evecs.cpu().numpy()
+    assert 1 <= sweeps <= 40
+    # off-diagonal inner products stop at 8 sqrt(n) eps of the norms; (1.25 |A|_F + |A|) of it in V A V^T
+    tol = 8 * np.sqrt(max(n, 16)) * 2.0 ** -52
+    frob = np.linalg.norm(a)
+    assert np.abs(evecs @ evecs.T - np.eye(n)).max() <= 2 * tol
+    assert np.abs(evecs @ a @ evecs.T - np.diag(evals)).max() <= 6 * tol * frob
+    assert np.abs(evals - np.linalg.eigvalsh(a)[::-1]).max() <= tol * frob
