@@ -449,17 +449,23 @@ __global__ void __launch_bounds__(kThreads, 1) decode_tc_kernel(DecodeArgs a)
                 // a chunk must end exactly where its recorded length says
                 if (active && r.consumed(seg_addr, chunk_start) != chunk_bits) bad = true;
             } else if (cur.ok && cur.staged) {
-                // per-channel tables (global memory), stream from shared memory
+                // per-channel codes: bounds loaded ahead (they do not depend on the stream), lengths by
+                // comparison, symbols off the critical path; stream from shared memory
                 SmemWindowReader r;
                 if (active) r.init(seg_addr, chunk_start);
                 else { r.hi = r.lo = r.ahead = 0; r.avail = 64; r.next_addr = seg_addr; }
                 decode_chunk(by_pairs([&](int j) -> uint32_t {
+                    const uint32_t *c = a.canon + (size_t)j * kCanonWords;
+                    const CanonBounds b0 = canon_bounds(c), b1 = canon_bounds(c + kCanonWords);
                     r.refill();
-                    const uint32_t e0 = __ldg(a.lut32 + (size_t)j * lut_size + r.peek(a.lut_bits));
-                    r.skip_entry(e0);
-                    const uint32_t e1 = __ldg(a.lut32 + (size_t)(j + 1) * lut_size + r.peek(a.lut_bits));
-                    r.skip_entry(e1);
-                    return __byte_perm(centre(e0), centre(e1), 0x7632);
+                    const uint32_t h0 = r.hi, l0 = canon_length(h0, b0);
+                    r.skip_entry(l0);
+                    const uint32_t h1 = r.hi, l1 = canon_length(h1, b1);
+                    r.skip_entry(l1);
+                    const uint8_t *order = a.sorted + ((size_t)j << a.bits);
+                    const uint32_t q0 = canon_symbol(h0, l0, reinterpret_cast<const uint16_t *>(c + 6), order);
+                    const uint32_t q1 = canon_symbol(h1, l1, reinterpret_cast<const uint16_t *>(c + 6 + kCanonWords), order + (1u << a.bits));
+                    return __byte_perm(centre(q0 << 8), centre(q1 << 8), 0x7632);
                 }));
                 if (active && r.consumed(seg_addr, chunk_start) != chunk_bits) bad = true;
             } else {

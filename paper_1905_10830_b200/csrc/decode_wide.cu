@@ -241,14 +241,20 @@ __global__ void __launch_bounds__(Roles<G>::kThreads, 1) decode_wide_kernel(Deco
                             uint32_t v0, v1, len0, len1;
                             if constexpr (kPerChannel) {
                                 const int j = k_first + k8 * 8 + 2 * i;
-                                const uint32_t e0 = __ldg(a.lut32 + (size_t)j * lut_size + r.peek(a.lut_bits));
-                                len0 = e0 & 0xffu;
+                                // (bounds instead of a table of all bit patterns: see canon_length)
+                                const uint32_t *c = a.canon + (size_t)j * kCanonWords;
+                                const uint8_t *order = a.sorted + ((size_t)j << a.bits);
+                                const CanonBounds b0 = canon_bounds(c), b1 = canon_bounds(c + kCanonWords);
+                                const uint32_t h0 = r.hi;
+                                len0 = canon_length(h0, b0);
                                 r.skip((int)len0);
-                                const uint32_t e1 = __ldg(a.lut32 + (size_t)(j + 1) * lut_size + r.peek(a.lut_bits));
-                                len1 = e1 & 0xffu;
+                                const uint32_t h1 = r.hi;
+                                len1 = canon_length(h1, b1);
                                 r.skip((int)len1);
-                                v0 = __float_as_uint((float)((int)((e0 >> 8) & 0xffu) - a.center));
-                                v1 = __float_as_uint((float)((int)((e1 >> 8) & 0xffu) - a.center));
+                                const uint32_t q0 = canon_symbol(h0, len0, reinterpret_cast<const uint16_t *>(c + 6), order);
+                                const uint32_t q1 = canon_symbol(h1, len1, reinterpret_cast<const uint16_t *>(c + 6 + kCanonWords), order + (1u << a.bits));
+                                v0 = __float_as_uint((float)((int)q0 - a.center));
+                                v1 = __float_as_uint((float)((int)q1 - a.center));
                             } else {
                                 v0 = s_lut[r.peek(a.lut_bits)];
                                 len0 = v0 & 0xffu;

@@ -170,6 +170,36 @@ struct BitWriter {
     }
 };
 
+// Decoding with the bounds of a canonical code instead of a table of all bit patterns, for per-channel
+// codes.  A table of 2^12 entries per channel lives in global memory (2 MB at 256 channels), and the
+// length of a symbol -- which the next symbol waits for -- took a load from L2 each time.  The bounds
+// are 24 bytes per channel at an address that does not depend on the stream, so they are loaded
+// ahead; the length follows from eleven comparisons, two per packed add; the symbol itself
+// (canon_symbol) is off the critical path.
+struct CanonBounds {
+    uint4 a;
+    uint2 b;
+};
+__device__ __forceinline__ CanonBounds canon_bounds(const uint32_t *table)      // global memory, 16-byte aligned
+{
+    return {__ldg(reinterpret_cast<const uint4 *>(table)), __ldg(reinterpret_cast<const uint2 *>(table + 4))};
+}
+// length of the code that `window` starts with (left-aligned, at least 12 valid bits)
+__device__ __forceinline__ uint32_t canon_length(uint32_t window, const CanonBounds &c)
+{
+    // a half-word's sum reaches bit 15 when the pattern lies past the codes of up to l bits
+    const uint32_t v = (window >> 17) * 0x00010001u, m = 0x80008000u;
+    const uint32_t s = ((v + c.a.x) & m) | (((v + c.a.y) & m) >> 1) | (((v + c.a.z) & m) >> 2) | (((v + c.a.w) & m) >> 3) |
+                       (((v + c.b.x) & m) >> 4) | (((v + c.b.y) & m) >> 5);
+    return 1u + (uint32_t)__popc(s);
+}
+// its symbol: `bases` = the code's half-words of bases, `sorted` = its symbols in code order
+__device__ __forceinline__ uint32_t canon_symbol(uint32_t window, uint32_t len, const uint16_t *bases, const uint8_t *sorted)
+{
+    const uint32_t place = ((uint32_t)bases[len - 1] + (window >> (32 - len))) & 0xffffu;
+    return __ldg(sorted + place);
+}
+
 // MSB-first reader over 32-bit words with a 64-bit window held in two registers.  Words at or
 // past `end` read as zero, so a corrupt offset can never cause an out-of-bounds load.
 // kShared: the words lie in shared memory (a staged segment) instead of global memory.

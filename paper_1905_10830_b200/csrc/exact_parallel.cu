@@ -93,35 +93,38 @@ __global__ void __launch_bounds__(kPx * kOut) project_quantise_kernel(EncodeArgs
 template <typename TOut>
 __global__ void __launch_bounds__(kPx * kOut) reconstruct_kernel(DecodeArgs a, const uint8_t *sym)
 {
-    // symbols of the block's pixels, coefficient-major ([K][kPx]: a warp reads 32 neighbouring bytes)
-    extern __shared__ __align__(16) unsigned char s_sym[];
-    __shared__ double s_t[kRed][kOut];                 // basis entries of kRed coefficients x the block's channels
+    // operands of kRed terms of every sum of the block: dequantised coefficients and basis entries, each
+    // computed or fetched once (a thread used to dequantise every symbol for itself: two of its four
+    // double operations per term)
+    __shared__ double s_yh[kRed][kPx + 1];
+    __shared__ double s_t[kRed][kOut];
     const int tx = threadIdx.x, ty = threadIdx.y, t = ty * kPx + tx;
     const long long p0 = (long long)blockIdx.x * kPx;
     const int n_px = (int)min((long long)kPx, a.pixels - p0);
-    for (int i = t; i < n_px * a.k; i += kPx * kOut) {
-        const int px = i / a.k, j = i - px * a.k;
-        s_sym[j * kPx + px] = sym[p0 * a.k + i];
-    }
     const long long p = p0 + tx;
     const int c = blockIdx.y * kOut + ty;
-    // staging role: thread t fetches the basis entry (coef, ch) = (t / 16, t % 16) of a step
-    const int lj = t / kOut, lc = blockIdx.y * kOut + (t % kOut);
-    auto fetch = [&](int j0) { return (j0 + lj < a.k && lc < a.c) ? __ldg(a.basis64 + (long long)(j0 + lj) * a.c + lc) : 0.0; };
-    double acc = 0.0, tv = fetch(0);
+    // staging roles: thread t fetches the symbols (px, coef) = (t / 16, 2 (t % 16)) and the next one,
+    // and the basis entry (coef, ch) = (t / 16, t % 16) of a step
+    const int lr = t / kOut, lx = t % kOut, lc = blockIdx.y * kOut + lx;
+    const uint8_t *src = sym + (p0 + lr) * a.k;
+    auto symbol = [&](int j) { return (lr < n_px && j < a.k) ? src[j] : (uint8_t)0; };
+    auto entry = [&](int j0) { return (j0 + lr < a.k && lc < a.c) ? __ldg(a.basis64 + (long long)(j0 + lr) * a.c + lc) : 0.0; };
+    double acc = 0.0, tv = entry(0);
+    uint8_t q0 = symbol(2 * lx), q1 = symbol(2 * lx + 1);
     for (int j0 = 0; j0 < a.k; j0 += kRed) {
-        __syncthreads();                               // symbols staged (first step); the previous step's entries used
-        s_t[lj][t % kOut] = tv;
+        __syncthreads();                               // the previous step's operands have been used
+        s_t[lr][lx] = tv;
+        s_yh[2 * lx][lr] = __dadd_rn(a.lo, __dmul_rn((double)q0, a.step));
+        s_yh[2 * lx + 1][lr] = __dadd_rn(a.lo, __dmul_rn((double)q1, a.step));
         __syncthreads();
-        if (j0 + kRed < a.k) tv = fetch(j0 + kRed);
-        const int n = min(kRed, a.k - j0);
-        if (tx < n_px) {
-#pragma unroll 8
-            for (int jj = 0; jj < n; ++jj) {
-                const double yh = __dadd_rn(a.lo, __dmul_rn((double)s_sym[(j0 + jj) * kPx + tx], a.step));
-                acc = __dadd_rn(acc, __dmul_rn(s_t[jj][ty], yh));
-            }
+        if (j0 + kRed < a.k) {                         // in flight while this step is added up
+            tv = entry(j0 + kRed);
+            q0 = symbol(j0 + kRed + 2 * lx);
+            q1 = symbol(j0 + kRed + 2 * lx + 1);
         }
+        const int n = min(kRed, a.k - j0);
+#pragma unroll 8
+        for (int jj = 0; jj < n; ++jj) acc = __dadd_rn(acc, __dmul_rn(s_t[jj][ty], s_yh[jj][tx]));
     }
     if (tx >= n_px || c >= a.c) return;
     double v = __dadd_rn(acc, __ldg(a.mean64 + c));
@@ -250,51 +253,70 @@ __global__ void __launch_bounds__(TC_TILE_PIXELS * kMaxParts) pack_symbols_kerne
 // its tile and consumed to exactly its recorded length.
 constexpr int kUnpackThreads = 512;
 
-struct GlobalBitReader {
-    const uint32_t *words;
-    unsigned long long window;   // upcoming bits, left-aligned
-    int avail;
-    unsigned long long next_word, end_word;
-    uint32_t ahead;              // the word behind the window, already loaded: a refill never waits for memory
+// MSB-first reader with a 64-bit window hi:lo (left-aligned) and the word behind it already loaded: a
+// refill never waits for memory.  Words at or past `end` read as zero.
+struct AheadReader {
+    const uint32_t *next, *end;
+    uint32_t hi, lo, ahead;
+    int avail;                   // valid bits in the window
+
     __device__ __forceinline__ uint32_t fetch()
     {
-        const uint32_t v = (next_word < end_word) ? __ldg(words + next_word) : 0u;   // past the end: zeros, never a load
-        ++next_word;
+        const uint32_t v = next < end ? __ldg(next) : 0u;
+        ++next;
         return v;
     }
     __device__ __forceinline__ void init(const uint32_t *base, unsigned long long bitpos, unsigned long long end_bits)
     {
-        words = base;
-        next_word = bitpos >> 5;
-        end_word = end_bits >> 5;
-        const unsigned long long hi = fetch(), lo = fetch();
+        next = base + (bitpos >> 5);
+        end = base + (end_bits >> 5);
+        const uint32_t w0 = fetch(), w1 = fetch();
         ahead = fetch();
         const int sh = (int)(bitpos & 31);
-        window = ((hi << 32) | lo) << sh;
+        hi = __funnelshift_l(w1, w0, sh);
+        lo = w1 << sh;
         avail = 64 - sh;
     }
-    __device__ __forceinline__ uint32_t peek(int nbits) const { return (uint32_t)(window >> (64 - nbits)); }
-    __device__ __forceinline__ void skip(int nbits)
+    __device__ __forceinline__ void skip(uint32_t nbits)         // below 32
     {
-        window <<= nbits;
-        avail -= nbits;
+        hi = __funnelshift_l(lo, hi, nbits);
+        lo <<= nbits;
+        avail -= (int)nbits;
+    }
+    // more than 32 valid bits: enough for two codes
+    __device__ __forceinline__ void refill()
+    {
         if (avail <= 32) {
-            window |= (unsigned long long)ahead << (32 - avail);
+            const int s = 32 - avail;                 // 0..31
+            hi |= __funnelshift_l(ahead, 0u, s);
+            lo |= ahead << s;
             avail += 32;
             ahead = fetch();
         }
     }
 };
 
+// What bounds it: the chain length -> shift -> length of a chunk's symbols, with a handful of warps on
+// the chip (a 256x14x14 map has two tiles).  Per-layer tables are staged in shared memory; of
+// per-channel codes the bounds are (K x 48 bytes, read ahead of the symbol), the symbols come from
+// global memory off the chain.  The threads of a warp walk the same run of coefficients of
+// neighbouring pixels, and symbols leave 16 bytes at a time.  Measured with the inverse transform
+// and the launches, 256x14x14 at 6 bits: 64.5 us with a 2^12-entry table per channel in global
+// memory and a byte stored per symbol.
 __global__ void __launch_bounds__(kUnpackThreads) unpack_symbols_kernel(DecodeArgs a, uint8_t *sym)
 {
     __shared__ unsigned int s_warp_sums[kUnpackThreads / 32];
-    extern __shared__ uint16_t s_lut[];                 // a per-layer table is staged (the launch sizes this to it, or to nothing)
+    __shared__ unsigned int s_start[kUnpackThreads];
+    extern __shared__ __align__(16) unsigned char s_tables[];   // the per-layer table, or the bounds and bases of every channel's code
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
-    const int lut_size = 1 << a.lut_bits;
-    const bool lut_staged = a.groups == 1;
-    if (lut_staged)
+    const int lut_size = 1 << a.lut_bits, nsym = 1 << a.bits;
+    const bool per_layer = a.groups == 1;
+    uint16_t *s_lut = reinterpret_cast<uint16_t *>(s_tables);
+    uint32_t *s_canon = reinterpret_cast<uint32_t *>(s_tables);
+    if (per_layer)
         for (int i = t; i < lut_size; i += kUnpackThreads) s_lut[i] = a.lut[i];
+    else
+        for (int i = t; i < a.k * kCanonWords; i += kUnpackThreads) s_canon[i] = a.canon[i];
     const long long tile = blockIdx.x;
     const unsigned long long base = a.tile_off[tile], end = a.tile_off[tile + 1];
     const bool tile_ok = (base & 127ull) == 0 && (end & 127ull) == 0 && base <= end && end <= a.stream_bits;
@@ -303,11 +325,10 @@ __global__ void __launch_bounds__(kUnpackThreads) unpack_symbols_kernel(DecodeAr
         return;
     }
     const int chunks_per_tile = a.splits * TC_TILE_PIXELS / a.chunk_pixels;      // at most 512
-    const long long ch = tile * chunks_per_tile + t;
-    const bool mine = t < chunks_per_tile && ch < a.n_chunks;
-    const unsigned int want = mine ? a.chunk_len[ch] : 0u;
-    // where the chunk starts: the lengths of the tile's earlier chunks
-    unsigned int inc = want;
+    // where every chunk of the tile starts: the lengths of its earlier chunks
+    const long long scan_ch = tile * chunks_per_tile + t;
+    const unsigned int len_t = (t < chunks_per_tile && scan_ch < a.n_chunks) ? a.chunk_len[scan_ch] : 0u;
+    unsigned int inc = len_t;
 #pragma unroll
     for (int d = 1; d < 32; d <<= 1) {
         const unsigned int up = __shfl_up_sync(0xffffffffu, inc, d);
@@ -315,34 +336,68 @@ __global__ void __launch_bounds__(kUnpackThreads) unpack_symbols_kernel(DecodeAr
     }
     if (lane == 31) s_warp_sums[warp] = inc;
     __syncthreads();
-    unsigned int off = inc - want;
-    for (int w = 0; w < warp; ++w) off += s_warp_sums[w];
-    bool bad = false;
-    if (mine) {
-        bad = base + off + want > end;
-        if (!bad) {
-            GlobalBitReader r;
-            r.init(a.stream, base + off, end);
-            unsigned int used = 0;
-            // the chunk's symbols: chunk_pixels whole pixels, or one of `splits` runs of one pixel
-            const int run = a.k / a.splits;
-            const int first_px = a.splits > 1 ? t / a.splits : t * a.chunk_pixels;
-            const int j_first = a.splits > 1 ? (t % a.splits) * run : 0;
-            for (int lp = first_px; lp < first_px + (a.splits > 1 ? 1 : a.chunk_pixels); ++lp) {
-                const long long p = tile * TC_TILE_PIXELS + lp;
-                if (p >= a.pixels) break;
-                uint8_t *dst = sym + p * a.k;
+    unsigned int off_t = inc - len_t;
+    for (int w = 0; w < warp; ++w) off_t += s_warp_sums[w];
+    s_start[t] = off_t;
+    __syncthreads();
+    // this thread's chunk: chunk_pixels whole pixels, or one of `splits` runs of one pixel
+    const int part = a.splits > 1 ? t / TC_TILE_PIXELS : 0;
+    const int in_tile = a.splits > 1 ? (t % TC_TILE_PIXELS) * a.splits + part : t;
+    const long long ch = tile * chunks_per_tile + in_tile;
+    if (t >= chunks_per_tile || ch >= a.n_chunks) return;
+    const unsigned int want = a.chunk_len[ch], off = s_start[in_tile];
+    bool bad = base + off + want > end;
+    if (!bad) {
+        AheadReader r;
+        r.init(a.stream, base + off, end);
+        unsigned int used = 0;
+        const int run = a.k / a.splits, j_first = part * run;
+        const int first_px = a.splits > 1 ? t % TC_TILE_PIXELS : t * a.chunk_pixels;
+        // decodes kN symbols from coefficient j on into v (one per element)
+        auto decode = [&](int j, auto &v) {
+            constexpr int kN = sizeof(v) / sizeof(v[0]);
+#pragma unroll
+            for (int i = 0; i < kN; ++i) {
+                if ((i & 1) == 0) r.refill();
+                uint32_t len;
+                if (per_layer) {
+                    const uint32_t e = s_lut[r.hi >> (32 - a.lut_bits)];
+                    len = e & 0xffu;
+                    v[i] = e >> 8;
+                } else {
+                    const uint32_t *c = s_canon + (j + i) * kCanonWords;
+                    const CanonBounds cb{*reinterpret_cast<const uint4 *>(c), *reinterpret_cast<const uint2 *>(c + 4)};
+                    len = canon_length(r.hi, cb);
+                    v[i] = canon_symbol(r.hi, len, reinterpret_cast<const uint16_t *>(c + 6), a.sorted + (size_t)(j + i) * nsym);
+                }
+                r.skip(len);
+                used += len;
+            }
+        };
+        const bool by16 = a.k % 16 == 0 && run % 16 == 0;
+        for (int lp = first_px; lp < first_px + (a.splits > 1 ? 1 : a.chunk_pixels); ++lp) {
+            const long long p = tile * TC_TILE_PIXELS + lp;
+            if (p >= a.pixels) break;
+            uint8_t *dst = sym + p * a.k;
+            if (by16) {
+#pragma unroll 1
+                for (int j = j_first; j < j_first + run; j += 16) {
+                    uint32_t v[16], w[4];
+                    decode(j, v);
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) w[i] = v[4 * i] | (v[4 * i + 1] << 8) | (v[4 * i + 2] << 16) | (v[4 * i + 3] << 24);
+                    *reinterpret_cast<uint4 *>(dst + j) = make_uint4(w[0], w[1], w[2], w[3]);
+                }
+            } else {
+#pragma unroll 1
                 for (int j = j_first; j < j_first + run; ++j) {
-                    const uint32_t e = lut_staged ? s_lut[r.peek(a.lut_bits)] : __ldg(a.lut + (size_t)j * lut_size + r.peek(a.lut_bits));
-                    const int len = (int)(e & 0xffu);
-                    dst[j] = (uint8_t)(e >> 8);
-                    r.skip(len);
-                    used += len;
-                    if (len == 0) bad = true;
+                    uint32_t v[1];
+                    decode(j, v);
+                    dst[j] = (uint8_t)v[0];
                 }
             }
-            if (used != want) bad = true;
         }
+        if (used != want) bad = true;
     }
     if (bad) tc_dev_set_status(a.status, TC_ERR_CORRUPT_STREAM);
 }
@@ -362,9 +417,8 @@ tc_status tc_launch_reconstruct(const DecodeArgs &a, int dtype, const uint8_t *s
 {
     if (a.pixels <= 0) return TC_OK;
     const dim3 block(kPx, kOut), grid((unsigned int)((a.pixels + kPx - 1) / kPx), (unsigned int)((a.c + kOut - 1) / kOut));
-    const size_t smem = (size_t)kPx * a.k;
-    if (dtype == TC_F32) reconstruct_kernel<float><<<grid, block, smem, s>>>(a, sym);
-    else reconstruct_kernel<__nv_bfloat16><<<grid, block, smem, s>>>(a, sym);
+    if (dtype == TC_F32) reconstruct_kernel<float><<<grid, block, 0, s>>>(a, sym);
+    else reconstruct_kernel<__nv_bfloat16><<<grid, block, 0, s>>>(a, sym);
     return cudaGetLastError() == cudaSuccess ? TC_OK : TC_ERR_CUDA;
 }
 
@@ -392,7 +446,9 @@ tc_status tc_launch_unpack_symbols(const DecodeArgs &a, uint8_t *sym, cudaStream
 {
     if (a.n_tiles <= 0) return TC_OK;
     if (a.splits * TC_TILE_PIXELS / a.chunk_pixels > kUnpackThreads) return TC_ERR_UNSUPPORTED;
-    const size_t smem = a.groups == 1 ? ((size_t)2 << a.lut_bits) : 0;
+    const size_t smem = a.groups == 1 ? ((size_t)2 << a.lut_bits) : (size_t)a.k * kCanonWords * 4;      // at most 48 KB
+    if (cudaFuncSetAttribute(unpack_symbols_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, TC_MAX_C * kCanonWords * 4) != cudaSuccess)
+        return TC_ERR_CUDA;
     unpack_symbols_kernel<<<(unsigned int)a.n_tiles, kUnpackThreads, smem, s>>>(a, sym);
     return cudaGetLastError() == cudaSuccess ? TC_OK : TC_ERR_CUDA;
 }

@@ -199,10 +199,26 @@ tc_status finish_codebook(tc_codebook *cb)
     std::vector<uint32_t> enc((size_t)cb->groups * nsym);
     std::vector<uint16_t> lut((size_t)cb->groups << cb->lut_bits);
     std::vector<uint32_t> lut32((size_t)cb->groups << cb->lut_bits);
-    std::vector<uint32_t> code(nsym);
+    std::vector<uint32_t> code(nsym), canon((size_t)cb->groups * kCanonWords);
+    std::vector<uint8_t> sorted((size_t)cb->groups * nsym);
     for (int g = 0; g < cb->groups; ++g) {
         const uint8_t *len = cb->lengths.data() + (size_t)g * nsym;
         tc_canonical_codes_host(len, nsym, code.data());
+        // The code as its canonical order: the codes of length l are consecutive numbers, and followed
+        // by the longer ones.  Half-word l - 1 of the first six words: 2^15 minus the first 15-bit
+        // pattern past the codes of up to l bits; half-word l - 1 of the last six: what turns a code of
+        // l bits into its place in the order.
+        uint16_t *half = reinterpret_cast<uint16_t *>(canon.data() + (size_t)g * kCanonWords);
+        uint32_t past = 0, place = 0;
+        for (int l = 1; l <= TC_MAX_CODE_LEN; ++l) {
+            uint32_t first = past >> (15 - l), n = 0;      // a code of l bits starts where the shorter ones end
+            for (int s = 0; s < nsym; ++s)
+                if (len[s] == l) sorted[(size_t)g * nsym + place + n++] = (uint8_t)s;
+            half[TC_MAX_CODE_LEN + l - 1] = (uint16_t)(place - first);
+            place += n;
+            past += n << (15 - l);
+            half[l - 1] = l < TC_MAX_CODE_LEN ? (uint16_t)(0x8000u - past) : (uint16_t)0;
+        }
         for (int s = 0; s < nsym; ++s) {
             enc[(size_t)g * nsym + s] = (code[s] << 8) | len[s];
             // every table index whose leading bits equal the code decodes to this symbol
@@ -220,6 +236,8 @@ tc_status finish_codebook(tc_codebook *cb)
     tc_status st;
     if ((st = upload(&cb->d_enc, enc)) != TC_OK) return st;
     if ((st = upload(&cb->d_lut32, lut32)) != TC_OK) return st;
+    if ((st = upload(&cb->d_canon, canon)) != TC_OK) return st;
+    if ((st = upload(&cb->d_sorted, sorted)) != TC_OK) return st;
     return upload(&cb->d_lut, lut);
 }
 
@@ -743,6 +761,8 @@ void tc_codebook_free(tc_codebook *cb)
     cudaFree(cb->d_enc);
     cudaFree(cb->d_lut);
     cudaFree(cb->d_lut32);
+    cudaFree(cb->d_canon);
+    cudaFree(cb->d_sorted);
     delete cb;
 }
 
@@ -907,7 +927,7 @@ static tc_status decode_with_scratch(tc_ctx *ctx, const tc_model *m, const tc_co
     a.chunk_pixels = cs.cp; a.lut_bits = cb->lut_bits; a.lut = cb->d_lut;
     a.basis64 = m->d_basis64; a.mean64 = m->d_mean64; a.lo = m->lo; a.step = m->step; a.basis_scale = m->basis_scale;
     a.xhat = x_hat->data; a.status = ctx->d_status;
-    a.lut32 = cb->d_lut32; a.basis_t_bf16 = m->d_basis_t_bf16; a.dec_bias = m->d_dec_bias; a.center = m->center;
+    a.lut32 = cb->d_lut32; a.canon = cb->d_canon; a.sorted = cb->d_sorted; a.basis_t_bf16 = m->d_basis_t_bf16; a.dec_bias = m->d_dec_bias; a.center = m->center;
     a.relu = (params && params->relu) ? 1 : 0;
     a.basis_t_map = m->has_basis_t_map ? &m->basis_t_map : nullptr;
     a.modal = cb->modal;

@@ -15,6 +15,8 @@ constexpr int TC_MAX_C = 1024;
 constexpr int TC_MAX_CODE_LEN = 12;
 constexpr int kMaxRoundtripChunks = 64;   // longest code the decode lookup table covers
 
+constexpr int kCanonWords = 12;               // words per table of a canonical code's bounds (6) and bases (6)
+
 // Device status word: first error wins.
 __device__ __forceinline__ void tc_dev_set_status(unsigned int *status, unsigned int code)
 {
@@ -77,6 +79,8 @@ struct tc_codebook {
     uint32_t *d_enc = nullptr;              // [groups][2^bits]  (code << 8) | length
     uint16_t *d_lut = nullptr;              // [groups][2^lut_bits]  (symbol << 8) | length
     uint32_t *d_lut32 = nullptr;            // [groups][2^lut_bits]  bf16(symbol) << 16 | symbol << 8 | length
+    uint32_t *d_canon = nullptr;            // [groups][kCanonWords]  bounds and bases of the canonical code (tcdev::canon_length)
+    uint8_t *d_sorted = nullptr;            // [groups][2^bits]  symbols in the order of their codes
 };
 
 // ---- kernel argument blocks -------------------------------------------------------------
@@ -129,6 +133,8 @@ struct DecodeArgs {
     int lut_bits;
     const uint16_t *lut;
     const uint32_t *lut32;              // tensor-core path
+    const uint32_t *canon;              // [groups][kCanonWords], see tc_codebook
+    const uint8_t *sorted;              // [groups][2^bits]
     const __nv_bfloat16 *basis_t_bf16;  // [c][k]
     const CUtensorMap *basis_t_map;     // HOST pointer to the model's tensor map of basis_t_bf16, or null
     const float *dec_bias;              // [c]

@@ -3,6 +3,7 @@ import numpy as np
 import pytest
 import torch
 
+import oracle
 import paper_1905_10830_b200 as tc
 from synth import featuremaps as fm
 from tests import helpers as H
@@ -65,3 +66,46 @@ def test_device_eigh_block_shapes_and_indefinite(ctx, n, shift):
     assert np.abs(evecs @ evecs.T - np.eye(n)).max() <= 2 * tol
     assert np.abs(evecs @ a @ evecs.T - np.diag(evals)).max() <= 6 * tol * frob
     assert np.abs(evals - np.linalg.eigvalsh(a)[::-1]).max() <= tol * frob
+
+
+# Per-channel codes decoded from their bounds: one-symbol-dominated, flat and maximum-length (12 bit)
+# tables side by side, every kernel that reads them (fp64 kernels with 1, 2 and 4 chunks a pixel and
+# runs that are no multiple of 16, resident and streaming tensor-core decoders).
+@pytest.mark.parametrize("c,k,s,n,bits,dtype,cp,splits,mode", [
+    (16, 16, 3, 1, 8, torch.float32, 0, 0, 0), (40, 24, 9, 2, 6, torch.float32, 0, 0, 0), (256, 256, 7, 2, 5, torch.float32, 0, 0, 0),
+    (512, 512, 4, 1, 8, torch.float32, 0, 0, 0), (64, 64, 9, 2, 1, torch.float32, 4, 1, 0), (48, 48, 9, 2, 7, torch.bfloat16, 0, 0, 0),
+    (256, 256, 14, 1, 6, torch.bfloat16, 0, 0, 0), (128, 128, 7, 3, 8, torch.bfloat16, 0, 0, 2), (320, 320, 5, 2, 4, torch.bfloat16, 0, 0, 0)])
+def test_per_channel_codes_from_bounds(ctx, c, k, s, n, bits, dtype, cp, splits, mode):
+    spec = fm.LayerSpec(c, s, s, 0.9, None, 12000 + c + bits)
+    o = H.oracle_side(spec, bits, max(3, 2 * c // (s * s) + 1), n, dtype, True, k=k)
+    lengths, nsym = o["lengths"].copy(), 1 << bits
+    flat = np.full(nsym, bits, dtype=np.uint8)
+    # the longest code a table can hold: 1, 2, 3, ... bits down to `deep` symbols of one length
+    steep = np.sort(np.r_[np.arange(1, nsym), nsym - 1]).astype(np.uint8) if nsym <= 8 else None
+    if steep is None:
+        counts = np.array([4 ** max(0, 14 - i) for i in range(nsym)], dtype=np.uint64)
+        steep = tc.tc_host_huffman_lengths(counts, 12)
+        assert steep.max() == 12
+    for j in range(0, k, 3):
+        lengths[j] = flat if j % 2 else steep[::-1]
+    m = H.import_model(tc, ctx, o["model"], dtype)
+    cb = tc.tc_codebook_import(ctx, lengths, bits)
+    x = o["x"].cuda()
+    tc.tc_force_exact_path(ctx, mode)
+    try:
+        enc = tc.tc_encode(ctx, m, cb, x, chunk_pixels=cp, pixel_splits=splits, debug=True, k=k)
+        xhat = tc.tc_decode(ctx, m, cb, enc, x.shape, dtype)
+        assert tc.tc_get_status(ctx) == 0
+        q = enc.symbols.cpu().numpy()
+        ref = check_stream_against_oracle(enc, q, lengths, bits)
+        assert np.array_equal(oracle.decode_symbols(ref, lengths, bits), q)
+        want = oracle.reconstruct(o["model"], q, tuple(x.shape), out_bf16=dtype == torch.bfloat16)
+        got = xhat.float().cpu().numpy()
+        if dtype == torch.float32:
+            assert np.array_equal(got, want)
+        else:                                       # fp32 accumulation: the parity cases' bound
+            flips, expected = H.count_output_flips(got, want), H.expected_output_flips(o["model"], q)
+            assert flips <= H.flip_allowance(expected)
+    finally:
+        tc.tc_force_exact_path(ctx, 0)
+    m.close(); cb.close()
