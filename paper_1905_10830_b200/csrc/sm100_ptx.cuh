@@ -51,11 +51,13 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, uint32_
     if (mbar_try_wait(bar, parity, 0u)) return true;
     unsigned long long t0, t1;
     asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t0));
+    // (one compact loop: with the inner loop of 64 attempts it had before, which the compiler unrolled at
+    // every call, the waits were a quarter of the kernels' code, and instruction fetch is what a
+    // kernel of one or two tiles per SM spends most of its time on)
+#pragma unroll 1
     while (true) {
-        for (int i = 0; i < 64; ++i) {
-            __nanosleep(sleep_ns);
-            if (mbar_try_wait(bar, parity, 100000u)) return true;
-        }
+        __nanosleep(sleep_ns);
+        if (mbar_try_wait(bar, parity, 100000u)) return true;
         asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t1));
         if (t1 - t0 > 2000000000ull) return false;
     }
