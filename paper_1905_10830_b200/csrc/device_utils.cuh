@@ -101,7 +101,7 @@ __device__ __forceinline__ unsigned long long lookback_resolve(unsigned long lon
             s = ld_volatile_u64(state + mine);
             while ((s >> 62) == 0) {
                 if (global_timer_ns() - t0 > kWaitLimitNs) break;
-                __nanosleep(64);
+                __nanosleep(200);          // (a polling warp takes issue slots from the block's working warps)
                 s = ld_volatile_u64(state + mine);
             }
         }

@@ -14,8 +14,10 @@
 // The basis T (bf16, K x C) stays resident in shared memory; the X tile streams through a ring
 // of 64-channel panels; the fp32 accumulators are double-buffered in tensor memory so that the
 // epilogue of one tile overlaps the loads and MMAs of the next.
+#include <algorithm>
 #include <cstdio>
 #include <cstdlib>
+#include <type_traits>
 
 #include "device_utils.cuh"
 #include "sm100_ptx.cuh"
@@ -25,37 +27,50 @@ namespace {
 using namespace tcdev;
 using namespace sm100;
 
-constexpr int kPanelCh = 64;                      // channels per ring stage
-constexpr int kStages = 4;
-constexpr int kStageBytes = kPanelCh * TC_TILE_PIXELS * 2;   // 16 KB
-constexpr int kLag = 2;                           // cp.async groups kept in flight per loader thread; the
-                                                  // remaining ring stage absorbs the MMA's latency
+constexpr int kPanelCh = 32;                      // channels per ring stage
+constexpr int kMaxStages = 8;                     // ring stages (six where the staging buffers need the room)
+constexpr int kStageBytes = kPanelCh * TC_TILE_PIXELS * 2;   // 8 KB
 constexpr int kStaticSmem = 1024;                 // the static shared variables, up to the ring's alignment
-constexpr int kStagingBytes = 15104;              // packed-bit staging per epilogue group (14.75 KB)
+constexpr int kSlots = 4;                         // packed tiles of a group that may wait in its staging buffer
+constexpr int kMaxStagingBytes = 49152;           // a tile of 256 coefficients of 12 bits
 constexpr int kEpiWarps = 16;                     // 2 groups x (2 column halves x 4 lane quarters)
 constexpr int kLoaderWarp0 = kEpiWarps, kMmaWarp = kEpiWarps + 4;
 constexpr int kStoreWarp0 = kMmaWarp + 1;         // two store warps follow
 constexpr int kThreads = (kEpiWarps + 7) * 32;
-constexpr int kMaxHalfCols = 128;                 // coefficients per epilogue thread (K <= 256)
 constexpr int kTmemCols = 512;
+constexpr int kSetupBar = 3;                      // named barrier of all warps but the loaders (1, 2: the epilogue groups)
 constexpr int kAccCols = 256;
-constexpr int kPairMaxBits = 4;                   // symbols of up to 4 bits are coded two at a time (256-entry tables)
+constexpr int kPairMaxBits = 6;                   // symbols of up to 6 bits can be coded two at a time (tables of up to 4096 entries)
+constexpr int kRunStep = 512;                     // bytes between a thread's words in the private runs (128 threads of a half)
 
-struct SmemLayout {
-    uint32_t basis, ring, staging, enc, len8, bias, xch, total;
+// How a launch uses the block: chosen on the host.
+struct Plan {
+    int stages;                // ring stages
+    uint32_t staging_bytes;    // per epilogue group, a multiple of 16; 0: does not fit
+    int run_words[2];          // words of a thread's private run, first and second half's threads; 0: two passes
+    int split_blk;             // blocks of 16 coefficients of the first half's threads
+    int skip_blk;              // blocks from here on are tested for holding nothing but the modal symbol
+    int entries;               // of the code table in shared memory
 };
 
-__host__ __device__ inline SmemLayout smem_layout(int c, int k, int enc_entries)
+struct SmemLayout {
+    uint32_t basis, ring, staging, runs, run_bytes, enc, len8, bias, bias_mid, xch, total;
+};
+
+__host__ __device__ inline SmemLayout smem_layout(int c, int k, const Plan &pl)
 {
     SmemLayout l;
     l.basis = 0;
     l.ring = (uint32_t)(((size_t)k * c * 2 + 1023) & ~(size_t)1023);
-    l.staging = l.ring + kStages * kStageBytes;
-    l.enc = l.staging + 2 * kStagingBytes;
-    l.len8 = l.enc + (uint32_t)enc_entries * 8;          // code lengths as bytes (per-layer table)
-    l.bias = (l.len8 + (enc_entries ? 256u : 0u) + 15u) & ~15u;
-    l.xch = l.bias + (uint32_t)k * 4;                   // code lengths exchanged between the halves: [2 groups][2][128] u16
-    l.total = l.xch + 2u * 2u * 128u * 2u;
+    l.staging = l.ring + (uint32_t)pl.stages * kStageBytes;
+    l.runs = l.staging + 2u * pl.staging_bytes;
+    l.run_bytes = (uint32_t)(pl.run_words[0] + pl.run_words[1]) * kRunStep;      // per group
+    l.enc = l.runs + 2u * l.run_bytes;
+    l.len8 = l.enc + (uint32_t)pl.entries * 8;           // code lengths as bytes
+    l.bias = (l.len8 + (uint32_t)pl.entries + 15u) & ~15u;
+    l.bias_mid = l.bias + (uint32_t)k * 4;
+    l.xch = l.bias_mid + (uint32_t)k * 4;               // per group: [2 halves][128] prefix and bits of every pixel, [3][128] chunk boundaries
+    l.total = l.xch + 2u * (2u * 128u * 4u + 3u * 128u * 2u);
     return l;
 }
 
@@ -65,47 +80,70 @@ __host__ __device__ inline SmemLayout smem_layout(int c, int k, int enc_entries)
 constexpr float kMagic = 12582912.0f;
 constexpr uint32_t kMagicBits = 0x4B400000u;
 
-// Bit writer into the shared-memory staging buffer.  A word is stored (plain, predicated
-// store) by the writer that supplies its last bit; bits that other writers own in that word
-// are zero in the stored value.  What is left after the last full word -- a writer's tail --
-// is merged afterwards with one shared-memory OR per writer (finish()), behind a barrier, so
-// that it cannot be overwritten by the store of the word's last writer.  A put adds fewer
+// Bit writer into shared memory, words kStep bytes apart.  A word is stored (plain, predicated store)
+// by the writer that supplies its last bit, nothing at or past `limit`; bits that other writers own
+// in that word are zero in the stored value.  What is left after the last full word -- a
+// writer's tail -- is merged afterwards with one shared-memory OR per writer (finish()), behind a
+// barrier, so that it cannot be overwritten by the store of the word's last writer.  A put adds fewer
 // than 32 bits (the pending count stays below 32 between puts).
+template <int kStep>
 struct SmemBitWriter {
-    uint32_t addr;             // shared address of the word being filled
+    uint32_t addr, limit;      // shared addresses: of the word being filled, past the last word
     uint32_t lo, hi;           // pending bits, right-aligned in hi:lo (bits above `pending` are stale)
     int pending;
-    __device__ __forceinline__ void init(uint32_t base_addr, unsigned int bitpos)
+    __device__ __forceinline__ void init(uint32_t base_addr, uint32_t end_addr, unsigned int bitpos)
     {
-        addr = base_addr + (bitpos >> 5) * 4u;
+        addr = base_addr + (bitpos >> 5) * (uint32_t)kStep;
+        limit = end_addr;
         pending = (int)(bitpos & 31u);
         lo = hi = 0;
     }
     __device__ __forceinline__ void put(uint32_t code, int len)
     {
         // hi:lo <<= len; lo |= code; pending += len; if (pending >= 32) { store bits
-        // [pending-32, pending) of hi:lo; addr += 4; pending -= 32; }  (the funnel shift takes
+        // [pending-32, pending) of hi:lo; addr += step; pending -= 32; }  (the funnel shift takes
         // its amount modulo 32, so `pending` itself serves as pending - 32)
         asm volatile(
-            "{\n\t.reg .pred p;\n\t.reg .b32 t, o;\n\t"
+            "{\n\t.reg .pred p, q;\n\t.reg .b32 t, o;\n\t"
             "shf.l.wrap.b32 %1, %0, %1, %5;\n\t"
             "shl.b32 t, %0, %5;\n\t"
             "or.b32 %0, t, %4;\n\t"
             "add.s32 %2, %2, %5;\n\t"
             "setp.ge.s32 p, %2, 32;\n\t"
+            "setp.lt.and.u32 q, %3, %6, p;\n\t"
             "shf.r.wrap.b32 o, %0, %1, %2;\n\t"
-            "@p st.shared.u32 [%3], o;\n\t"
-            "@p add.s32 %3, %3, 4;\n\t"
+            "@q st.shared.u32 [%3], o;\n\t"
+            "@p add.s32 %3, %3, %7;\n\t"
             "@p add.s32 %2, %2, -32;\n\t}"
             : "+r"(lo), "+r"(hi), "+r"(pending), "+r"(addr)
-            : "r"(code), "r"(len));
+            : "r"(code), "r"(len), "r"(limit), "n"(kStep));
+    }
+    // 32 bits at once: the pending count stays
+    __device__ __forceinline__ void put_word(uint32_t bits)
+    {
+        const uint32_t out = __funnelshift_r(bits, lo, pending);       // the pending bits, then the first of the new ones
+        if (addr < limit) asm volatile("st.shared.u32 [%0], %1;" ::"r"(addr), "r"(out) : "memory");
+        addr += kStep;
+        lo = bits;
+        hi = 0;
     }
     // call after a barrier that follows every writer's puts
     __device__ __forceinline__ void finish()
     {
         const uint32_t out = pending > 0 ? (lo << (32 - pending)) : 0u;
-        if (out) asm volatile("red.shared.or.b32 [%0], %1;" ::"r"(addr), "r"(out) : "memory");
+        if (out && addr < limit) asm volatile("red.shared.or.b32 [%0], %1;" ::"r"(addr), "r"(out) : "memory");
     }
+};
+
+// Sinks of a thread's codes that are not written to shared memory: only counted, or packed into global memory.
+struct CountSink {
+    unsigned int bits;
+};
+struct GlobalSink {
+    BitWriter w;
+    bool on;
+    __device__ __forceinline__ void put(uint32_t code, int len) { if (on) w.put(code, len); }
+    __device__ __forceinline__ void put_word(uint32_t bits) { put(bits >> 16, 16); put(bits & 0xffffu, 16); }
 };
 
 // Two coefficients at once.  The position on the quantiser's grid is computed as a fraction of
@@ -128,63 +166,105 @@ __device__ __forceinline__ void quantise_bits2(uint32_t acc0, uint32_t acc1, flo
         : "=r"(q0), "=r"(q1) : "f"(t0), "f"(t1), "f"(top), "f"(kMagic));
 }
 
-// kPair (per-layer tables, b <= 4): the code tables are indexed by two neighbouring symbols at
-// once (q0 | q1 << b, at most 256 entries), which halves the lookups of both passes.
+// Raises `far` to the larger distance of two coefficients from the modal symbol's level, as fractions of
+// the quantiser's range (`mid`: the bias seen from that level): one packed multiply-add, one
+// three-input maximum.
+__device__ __forceinline__ void farthest2(float &far, uint32_t acc0, uint32_t acc1, float inv_range, float mid0, float mid1)
+{
+    asm("{\n\t.reg .b64 v, s, m;\n\t.reg .f32 u0, u1;\n\t"
+        "mov.b64 v, {%1, %2};\n\t"
+        "mov.b64 s, {%3, %3};\n\t"
+        "mov.b64 m, {%4, %5};\n\t"
+        "fma.rn.f32x2 v, v, s, m;\n\t"
+        "mov.b64 {u0, u1}, v;\n\t"
+        "max.NaN.abs.f32 %0, %0, u0, u1;\n\t}"
+        : "+f"(far) : "r"(acc0), "r"(acc1), "f"(inv_range), "f"(mid0), "f"(mid1));
+}
+
+// The epilogue's two ways (kRuns):
+//   one pass: every thread packs the codes of its coefficients, as they are quantised, into a private
+//     run of words in shared memory (word w of all threads side by side: no bank conflicts); when
+//     the tile's bit offsets are known the few words are shifted to their place in the staging buffer.
+//     Nothing but the packed bits is kept, so the loop over the coefficients stays rolled.
+//   two passes, where runs and staging do not both fit (near-lossless codes of wide layers): code
+//     lengths first, then the coefficients are quantised again and packed straight to their place; the
+//     accumulator is held until then.
+// What bounded the epilogue before (symbols in registers between a length pass and a pack pass, both
+// unrolled over 128 coefficients): 117 KB of straight-line code per tile -- instruction fetch -- and a
+// second table lookup per symbol.
+// Blocks of 16 coefficients from skip_blk on are first tested, by the whole warp, for holding nothing
+// but the modal symbol (the single bit 0): sixteen zero bits then.
+// kPair (per-layer tables, b <= 6): the code tables are indexed by two neighbouring symbols at once
+// (q0 | q1 << b), which halves the lookups.
 // kHist (statistics, Section 3.1 "Variable length coding": the entropy needs the distribution of
 // the symbols): every symbol is also counted, per coefficient channel, into a.hist.  The lanes of
 // a warp hold one coefficient of 32 pixels; the symbol most of them hold (the zero level) is
 // counted once per warp from a ballot, the others one atomic each.
-template <bool kPerChannel, bool kDebug, bool kPair, bool kHist>
-__global__ void __launch_bounds__(kThreads, 1) encode_tc_kernel(EncodeArgs a)
+template <bool kPerChannel, bool kDebug, bool kPair, bool kHist, bool kRuns>
+__global__ void __launch_bounds__(kThreads, 1) encode_tc_kernel(EncodeArgs a, Plan pl)
 {
     extern __shared__ __align__(1024) unsigned char smem[];      // swizzled ring stages: aligned to their 1 KB atoms
-    __shared__ __align__(8) unsigned long long s_full[kStages], s_empty[kStages], s_tfull[2], s_tempty[2];
+    __shared__ __align__(8) unsigned long long s_full[kMaxStages], s_empty[kMaxStages], s_tfull[2], s_tempty[2];
     __shared__ uint32_t s_tmem_base;
-    __shared__ unsigned int s_warp_sums[2][4];
+    __shared__ unsigned int s_warp_sums[2][2][4], s_overflow[2];
+    __shared__ int s_go[2];                    // per group: its polling warp's waits for the tile have succeeded
     __shared__ unsigned long long s_base[2];
     __shared__ int s_write_ok[2];
-    __shared__ __align__(8) unsigned long long s_stg_full[2], s_stg_free[2];   // staging hand-over to the store warp
-    __shared__ unsigned long long s_padded[2];
-    __shared__ int s_store_cmd[2];             // 1: copy the staged tile out, 2: nothing to copy, 3: stop
+    // staging hand-over to the store warp: slot n % kSlots for a group's n-th tile
+    __shared__ __align__(8) unsigned long long s_stg_full[2][kSlots], s_stg_free[2][kSlots];
+    __shared__ unsigned int s_padded[2][kSlots], s_stg_at[2][kSlots];   // bits of the tile, its place in the staging buffer
+    __shared__ int s_store_cmd[2][kSlots];     // 1: copy the staged tile out, 2: nothing to copy, 3: stop
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int nsym = 1 << a.bits;
     constexpr bool enc_in_smem = !kPerChannel;
-    const int enc_entries = enc_in_smem ? (kPair ? nsym * nsym : nsym) : 0;
-    const SmemLayout L = smem_layout(a.c, a.k, enc_entries);
+    constexpr bool kCanSkip = !kPerChannel && !kDebug && !kHist;     // blocks of modal symbols are passed over
+    const int enc_entries = pl.entries;
+    const SmemLayout L = smem_layout(a.c, a.k, pl);
+    const int n_stages = pl.stages;
     unsigned char *s_basis = smem + L.basis;
     uint32_t *s_enc = reinterpret_cast<uint32_t *>(smem + L.enc);
-    float *s_bias = reinterpret_cast<float *>(smem + L.bias);
+    float *s_bias = reinterpret_cast<float *>(smem + L.bias), *s_bias_mid = reinterpret_cast<float *>(smem + L.bias_mid);
     const uint32_t ring_addr = smem_u32(smem + L.ring);
     const uint32_t basis_addr = smem_u32(s_basis);
     const int n_panels = (a.c + kPanelCh - 1) / kPanelCh;
 
     // ---- set-up ---------------------------------------------------------------------
+    if (tid < 2) s_overflow[tid] = 0;
     if (tid == 0) {
-        for (int s = 0; s < kStages; ++s) { mbar_init(smem_u32(&s_full[s]), 128); mbar_init(smem_u32(&s_empty[s]), 1); }
+        for (int s = 0; s < n_stages; ++s) { mbar_init(smem_u32(&s_full[s]), 128); mbar_init(smem_u32(&s_empty[s]), 1); }
         for (int b = 0; b < 2; ++b) {
             mbar_init(smem_u32(&s_tfull[b]), 1);
-            mbar_init(smem_u32(&s_tempty[b]), 256);
-            mbar_init(smem_u32(&s_stg_full[b]), 256);
-            mbar_init(smem_u32(&s_stg_free[b]), 1);
+            mbar_init(smem_u32(&s_tempty[b]), 8);                 // one arrival per warp of the group
+            for (int i = 0; i < kSlots; ++i) { mbar_init(smem_u32(&s_stg_full[b][i]), 8); mbar_init(smem_u32(&s_stg_free[b][i]), 1); }
         }
         mbar_fence_init();
     }
+    const long long my_tiles = (a.n_tiles > blockIdx.x) ? (a.n_tiles - blockIdx.x + gridDim.x - 1) / gridDim.x : 0;
+    __syncthreads();
+    // the loaders start with the first tile at once, the others lay out the basis and the tables meanwhile
+    const bool loader = warp >= kLoaderWarp0 && warp < kMmaWarp;
+    const int setup_tid = warp < kLoaderWarp0 ? tid : tid - 128;
+    constexpr int kSetupThreads = kThreads - 128;
     if (warp == kMmaWarp) { tmem_alloc(smem_u32(&s_tmem_base), kTmemCols); tmem_relinquish(); }
-    // basis -> K-major core-matrix layout: element (j, ch) at (j/8)*sbo + (ch/8)*128 + (j%8)*16 + (ch%8)*2
-    {
+    if (!loader) {
+        // basis -> K-major core-matrix layout: element (j, ch) at (j/8)*sbo + (ch/8)*128 + (j%8)*16 + (ch%8)*2
         const uint32_t sbo = (uint32_t)(a.c / 8) * 128u;
         const int chunks_per_row = a.c / 8;
         const uint4 *src = reinterpret_cast<const uint4 *>(a.basis_bf16);
         // (asynchronous copies: all of a thread's pieces are in flight at once)
-        for (int i = tid; i < a.k * chunks_per_row; i += kThreads) {
+        for (int i = setup_tid; i < a.k * chunks_per_row; i += kSetupThreads) {
             const int j = i / chunks_per_row, c8 = i - j * chunks_per_row;
             cp_async_16(basis_addr + (j >> 3) * sbo + c8 * 128 + (j & 7) * 16, src + i, 16u);
         }
         cp_async_commit();
-        for (int i = tid; i < a.k; i += kThreads) s_bias[i] = a.enc_bias[i] / (float)(nsym - 1);   // as a fraction of the range
+        for (int i = setup_tid; i < a.k; i += kSetupThreads) {
+            const float b = a.enc_bias[i] / (float)(nsym - 1);   // as a fraction of the range
+            s_bias[i] = b;
+            s_bias_mid[i] = b - (float)(a.modal < 0 ? 0 : a.modal) / (float)(nsym - 1);   // the same, seen from the modal symbol's level
+        }
         if (enc_in_smem)
-            for (int i = tid; i < enc_entries; i += kThreads) {
+            for (int i = setup_tid; i < enc_entries; i += kSetupThreads) {
                 // per-layer table: (1 << length, code) pairs, so that appending a code to a register is
                 // one multiply-add, and the lengths once more as bytes.  In pair mode entry
                 // q0 | q1 << b holds the two codes joined (q0's first), at most 24 bits.
@@ -202,67 +282,78 @@ __global__ void __launch_bounds__(kThreads, 1) encode_tc_kernel(EncodeArgs a)
                 s_enc[2 * i + 1] = code;
                 (smem + L.len8)[i] = (unsigned char)len;
             }
+        cp_async_wait<0>();
+        fence_proxy_async_smem();
+        tc_fence_before_sync();
+        named_bar_sync(kSetupBar, kSetupThreads);
+        tc_fence_after_sync();
     }
-    cp_async_wait<0>();
-    fence_proxy_async_smem();
-    tc_fence_before_sync();
-    __syncthreads();
-    tc_fence_after_sync();
     const uint32_t tmem_base = s_tmem_base;
-
-    const long long my_tiles = (a.n_tiles > blockIdx.x) ? (a.n_tiles - blockIdx.x + gridDim.x - 1) / gridDim.x : 0;
 
     if (warp >= kLoaderWarp0 && warp < kMmaWarp) {
         // ================= loaders =================
-        // A copy instruction of a warp moves whole runs of a channel's row -- 32 groups of 4 pixels of
-        // one channel, or, where rows allow 16 bytes, 16 groups of 8 pixels of two channels -- and
-        // touches two to four cache lines.  (Eight channels x 32 bytes per instruction, which the
-        // unswizzled operand layout asks for to spread over the banks, touched eight or more and held
-        // the whole kernel to 1.85 TB/s of input: 222 us for 256x14x14 x 4096 with the MMAs and the
-        // epilogue's work taken out.)  In the swizzled layout 64 pixels of a channel are 128 contiguous
-        // bytes, the 16-byte pieces exchanged by XOR with the channel modulo 8: no bank conflicts.
+        // A lane moves groups of 8 pixels of every eighth channel: one copy of 16 bytes where the group starts
+        // on a 16-byte boundary of global memory and lies in one image, else two of 8.  With H*W an odd
+        // multiple of 4 the groups of the channels of one parity are aligned (the parity changes from image
+        // to image), so a warp takes channels of one parity only: its lanes agree up to an image
+        // boundary.  What bounds the loads is the copy unit, by lanes rather than bytes: 8-byte copies
+        // alone reach 3.3 TB/s of input (123 us for 256x14x14 x 4096 and nothing else), this mix
+        // 4.6 TB/s, 16-byte copies 6.4 TB/s.  (Eight channels x 32 bytes per instruction, which the
+        // unswizzled operand layout asks for, reached 1.85 TB/s.)  In the swizzled layout 64 pixels of a
+        // channel are 128 contiguous bytes, the 16-byte pieces exchanged by XOR with the channel modulo 8.
         const int lw = warp - kLoaderWarp0;
-        const bool wide = (a.hw & 7) == 0 && ((uintptr_t)a.x & 15u) == 0;      // 16 bytes per copy
-        const int px = wide ? 8 * (lane & 15) : 4 * lane;          // first pixel of this lane's group in the tile
-        const int ch0 = wide ? 2 * lw + (lane >> 4) : lw;          // this lane's first channel of a panel, then every 8th / 4th
-        const uint32_t dst0 = (uint32_t)((px >> 6) * (kStageBytes / 2) + (px & 7) * 2);
-        const uint32_t piece = (uint32_t)((px & 63) >> 3);
+        const int px = 8 * (lane & 15);                            // first pixel of this lane's group in the tile
+        const int ch0 = (lw & 1) + 2 * (lane >> 4) + 4 * (lw >> 1);  // channels ch0, ch0 + 8, ... of a panel
+        const uint32_t dst0 = (uint32_t)((px >> 6) * (kStageBytes / 2) + ch0 * 128 + ((((px & 63) >> 3) ^ ch0) << 4));
         const __nv_bfloat16 *xin = reinterpret_cast<const __nv_bfloat16 *>(a.x);
-        int it = 0;
+        const uint32_t row8 = 16u * (uint32_t)a.hw;   // bytes from a channel to the eighth after it
+        static_assert(kPanelCh == 32, "a lane copies four channels of a panel");
+        int s = 0;                                 // ring stage of the next panel
+        uint32_t phase = 1;
         bool alive = true;
         for (long long tl = 0; tl < my_tiles && alive; ++tl) {
             const long long p0 = (blockIdx.x + tl * gridDim.x) * TC_TILE_PIXELS + px;
-            const bool valid = p0 < a.pixels;
-            const long long img = valid ? p0 / a.hw : 0;
-            const __nv_bfloat16 *src = xin + img * a.c * (long long)a.hw + (valid ? p0 - img * a.hw : 0) + (long long)ch0 * a.hw;
-            const uint32_t nbytes = valid ? (wide ? 16u : 8u) : 0u;
-            for (int kp = 0; kp < n_panels; ++kp, ++it) {
-                const int s = it % kStages;
-                if (!mbar_wait(smem_u32(&s_empty[s]), ((it / kStages) & 1) ^ 1)) { alive = false; break; }
-                const int nch = min(kPanelCh, a.c - kp * kPanelCh);
-                const uint32_t stage = ring_addr + s * kStageBytes + dst0;
-                if (wide) {
-#pragma unroll 4
-                    for (int ch = ch0; ch < nch; ch += 8, src += 8 * a.hw)
-                        cp_async_16(stage + (uint32_t)ch * 128u + ((piece ^ (uint32_t)(ch & 7)) << 4), src, nbytes);
+            const long long img = p0 < a.pixels ? p0 / a.hw : 0;
+            const int sp = p0 < a.pixels ? (int)(p0 - img * a.hw) : 0;
+            const bool split = sp + 4 >= a.hw;                 // the second four pixels start the next image
+            const char *src = reinterpret_cast<const char *>(xin + (img * a.c + ch0) * (long long)a.hw + sp);
+            const uint32_t n1 = p0 < a.pixels ? 8u : 0u, n2 = p0 + 4 < a.pixels ? 8u : 0u;
+            const char *src2 = n2 == 0u ? src : src + (split ? ((long long)a.c * a.hw - a.hw + 4) * 2 : 8);    // the second four pixels
+            const bool whole = !split && n2 != 0u && ((uintptr_t)src & 15u) == 0;
+            for (int kp = 0; kp < n_panels; ++kp) {
+                if (!mbar_wait(smem_u32(&s_empty[s]), phase, 200u)) { alive = false; break; }
+                const uint32_t dst = ring_addr + s * kStageBytes + dst0;
+                const bool full = (kp + 1) * kPanelCh <= a.c;              // else half a panel (C is a multiple of 16)
+                if (whole) {
+                    cp_async_16(dst, src, 16u);
+                    cp_async_16(dst + 1024u, src + row8, 16u);
+                    if (full) {
+                        cp_async_16(dst + 2048u, src + 2u * row8, 16u);
+                        cp_async_16(dst + 3072u, src + 3u * row8, 16u);
+                    }
                 } else {
-#pragma unroll 4
-                    for (int ch = ch0; ch < nch; ch += 4, src += 4 * a.hw)
-                        cp_async_8(stage + (uint32_t)ch * 128u + ((piece ^ (uint32_t)(ch & 7)) << 4), src, nbytes);
+                    cp_async_8(dst, src, n1);
+                    cp_async_8(dst + 8u, src2, n2);
+                    cp_async_8(dst + 1024u, src + row8, n1);
+                    cp_async_8(dst + 1032u, src2 + row8, n2);
+                    if (full) {
+                        cp_async_8(dst + 2048u, src + 2u * row8, n1);
+                        cp_async_8(dst + 2056u, src2 + 2u * row8, n2);
+                        cp_async_8(dst + 3072u, src + 3u * row8, n1);
+                        cp_async_8(dst + 3080u, src2 + 3u * row8, n2);
+                    }
                 }
-                cp_async_commit();
-                if (it >= kLag) {
-                    cp_async_wait<kLag>();
-                    fence_proxy_async_smem();
-                    mbar_arrive(smem_u32(&s_full[(it - kLag) % kStages]));
-                }
+                src += 4u * row8;
+                src2 += 4u * row8;
+                // the stage's barrier gets this thread's arrival when its copies have landed: the thread goes
+                // on to the next stage, so that all free stages are in flight (with a wait for the panel
+                // before the last the loads were bound by their latency, two panels at a time)
+                cp_async_arrive_noinc(smem_u32(&s_full[s]));
+                if (++s == n_stages) { s = 0; phase ^= 1u; }
             }
         }
-        if (alive) {
-            if (it >= 2) { cp_async_wait<1>(); fence_proxy_async_smem(); mbar_arrive(smem_u32(&s_full[(it - 2) % kStages])); }
-            if (it >= 1) { cp_async_wait<0>(); fence_proxy_async_smem(); mbar_arrive(smem_u32(&s_full[(it - 1) % kStages])); }
-        } else {
-            cp_async_wait<0>();
+        if (!alive) {
+            cp_async_wait_all();
             tc_dev_set_status(a.status, TC_ERR_TIMEOUT);
         }
     } else if (warp == kMmaWarp) {
@@ -273,26 +364,29 @@ __global__ void __launch_bounds__(kThreads, 1) encode_tc_kernel(EncodeArgs a)
         {
             const uint32_t issuer = lane == 0 ? 1u : 0u;
             const uint32_t idesc = make_idesc_bf16(TC_TILE_PIXELS, a.k, /*A MN-major*/ true, /*B K-major*/ false);
-            const uint32_t b_sbo = (uint32_t)(a.c / 8) * 128u;
-            int it = 0;
+            const uint64_t a_desc = make_smem_desc_mn_sw128(ring_addr, kStageBytes / 2, 1024);
+            const uint64_t b_desc = make_smem_desc(basis_addr, 128, (uint32_t)(a.c / 8) * 128u);
+            const uint32_t a_desc_lo = (uint32_t)a_desc, a_desc_hi = (uint32_t)(a_desc >> 32), b_desc_hi = (uint32_t)(b_desc >> 32);
+            int s = 0;
+            uint32_t phase = 0;
             bool alive = true;
             for (long long tl = 0; tl < my_tiles && alive; ++tl) {
                 const int acc = (int)(tl & 1);
                 if (!mbar_wait(smem_u32(&s_tempty[acc]), (uint32_t)(((tl >> 1) & 1) ^ 1))) { alive = false; break; }
                 tc_fence_after_sync();
                 const uint32_t d_tmem = tmem_base + acc * kAccCols;
-                for (int kp = 0; kp < n_panels; ++kp, ++it) {
-                    const int s = it % kStages;
-                    if (!mbar_wait(smem_u32(&s_full[s]), (it / kStages) & 1)) { alive = false; break; }
+                uint32_t b_lo = (uint32_t)b_desc;
+                for (int kp = 0; kp < n_panels; ++kp) {
+                    if (!mbar_wait(smem_u32(&s_full[s]), phase)) { alive = false; break; }
+                    fence_proxy_async_smem();            // the loaders' copies, made visible to the tensor core
                     tc_fence_after_sync();
-                    const int k0 = kp * kPanelCh;
-                    const int nk16 = min(kPanelCh, a.c - k0) >> 4;
-                    for (int q = 0; q < nk16; ++q) {
-                        const uint64_t adesc = make_smem_desc_mn_sw128(ring_addr + s * kStageBytes + q * 2048, kStageBytes / 2, 1024);
-                        const uint64_t bdesc = make_smem_desc(basis_addr + ((k0 + 16 * q) >> 3) * 128, 128, b_sbo);
-                        mma_bf16_ss_guarded(d_tmem, adesc, bdesc, idesc, (kp | q) != 0 ? 1u : 0u, issuer);
-                    }
+                    const uint32_t a_lo = a_desc_lo + (uint32_t)s * (kStageBytes >> 4);
+                    mma_bf16_ss_guarded(d_tmem, a_lo, a_desc_hi, b_lo, b_desc_hi, idesc, kp ? 1u : 0u, issuer);
+                    if ((kp + 1) * kPanelCh <= a.c)          // else half a panel
+                        mma_bf16_ss_guarded(d_tmem, a_lo + (2048u >> 4), a_desc_hi, b_lo + (256u >> 4), b_desc_hi, idesc, 1u, issuer);
+                    b_lo += (kPanelCh / 8) * (128u >> 4);
                     mma_commit_guarded(smem_u32(&s_empty[s]), issuer);
+                    if (++s == n_stages) { s = 0; phase ^= 1u; }
                 }
                 if (alive) mma_commit_guarded(smem_u32(&s_tfull[acc]), issuer);
             }
@@ -301,15 +395,17 @@ __global__ void __launch_bounds__(kThreads, 1) encode_tc_kernel(EncodeArgs a)
     } else if (warp >= kStoreWarp0) {
         // ================= store warps =================
         const int grp = warp - kStoreWarp0;
-        const uint32_t stg_addr = smem_u32(smem + L.staging + grp * kStagingBytes);
+        const uint32_t stg_addr = smem_u32(smem + L.staging + (uint32_t)grp * pl.staging_bytes);
         long long n = 0;
         for (long long tl = grp; tl < my_tiles; tl += 2, ++n) {
             const long long tile = blockIdx.x + tl * gridDim.x;
-            if (!mbar_wait(smem_u32(&s_stg_full[grp]), (uint32_t)(n & 1))) { if (lane == 0) tc_dev_set_status(a.status, TC_ERR_TIMEOUT); break; }
-            const int cmd = s_store_cmd[grp];
+            const int slot = (int)(n % kSlots);
+            if (!mbar_wait(smem_u32(&s_stg_full[grp][slot]), (uint32_t)((n / kSlots) & 1), 400u)) { if (lane == 0) tc_dev_set_status(a.status, TC_ERR_TIMEOUT); break; }
+            const int cmd = s_store_cmd[grp][slot];
             if (cmd == 3) break;
             if (cmd == 1) {
-                const unsigned long long padded = s_padded[grp];
+                const unsigned long long padded = s_padded[grp][slot];
+                const uint32_t src = stg_addr + s_stg_at[grp][slot];
                 bool ok;
                 const unsigned long long base = lookback_resolve(a.tile_state, tile, padded, a.status, ok);
                 const bool fits = base + padded <= a.capacity_bits;
@@ -319,7 +415,7 @@ __global__ void __launch_bounds__(kThreads, 1) encode_tc_kernel(EncodeArgs a)
                     for (unsigned int i = lane; i < (unsigned int)(padded >> 7); i += 32) {
                         uint4 v;
                         asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];"
-                                     : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(stg_addr + i * 16u));
+                                     : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(src + i * 16u));
                         dst[i] = v;
                     }
                 }
@@ -329,31 +425,41 @@ __global__ void __launch_bounds__(kThreads, 1) encode_tc_kernel(EncodeArgs a)
                 }
             }
             __syncwarp();
-            if (lane == 0) mbar_arrive(smem_u32(&s_stg_free[grp]));
+            if (lane == 0) mbar_arrive(smem_u32(&s_stg_free[grp][slot]));
         }
     } else {
         // ================= epilogue groups =================
         const int grp = warp >> 3;                 // 0 or 1
         const int wg = warp & 7;
-        const int half = wg >> 2;                  // which half of the coefficients
+        const int half = wg >> 2;                  // which part of the coefficients
         const int wq = wg & 3;                     // TMEM lane quarter
         const int m = wq * 32 + lane;              // pixel within the tile = TMEM lane
         const int tg = (tid & 255);                // thread within the group
-        const int half_cols = ((a.k + 31) / 32) * 16;              // columns of half 0 (multiple of 16)
-        const int col0 = half * half_cols;
-        const int ncols = half ? a.k - half_cols : half_cols;      // multiple of 16, may be 0
-        unsigned char *stg = smem + L.staging + grp * kStagingBytes;
-        const uint32_t stg_addr = smem_u32(stg);
+        const int n_blk = a.k >> 4;                // blocks of 16 coefficients: the first split_blk belong to the first half's threads
+        const int blk0 = half ? pl.split_blk : 0, blk1 = half ? n_blk : pl.split_blk;
+        const int chunk_blks = a.splits > 1 ? n_blk / a.splits : n_blk;    // blocks per chunk of a pixel
+        const int bound0 = max(1, (blk0 + chunk_blks - 1) / chunk_blks);   // the first chunk boundary that lies before one of this thread's blocks
+        const uint32_t stg_addr = smem_u32(smem + L.staging + (uint32_t)grp * pl.staging_bytes);
         const uint32_t enc_addr = smem_u32(s_enc);
-        const uint32_t len8_rel = smem_u32(smem + L.len8) - kMagicBits;   // + (kMagicBits + q) = address of len8[q]
-        const uint32_t pair_len_rel = smem_u32(smem + L.len8) - kMagicBits * (1u + (1u << a.bits));   // same for a pair sum
-        unsigned short *xch = reinterpret_cast<unsigned short *>(smem + L.xch) + grp * 256;   // [2][128] lengths exchanged between the halves
-        long long n_done = 0;                      // tiles this group has handed to its store warp
+        const uint32_t len8_addr = smem_u32(smem + L.len8);
+        const uint32_t run_addr = smem_u32(smem + L.runs) + (uint32_t)grp * L.run_bytes + (half ? (uint32_t)pl.run_words[0] * kRunStep : 0u) + (uint32_t)m * 4u;
+        const uint32_t run_end = run_addr + (uint32_t)pl.run_words[half] * kRunStep;
+        uint32_t *xch = reinterpret_cast<uint32_t *>(smem + L.xch + grp * (2 * 128 * 4 + 3 * 128 * 2));   // [2][128]: prefix in the warp << 12 | bits
+        unsigned short *bound = reinterpret_cast<unsigned short *>(xch + 256);                            // [3][128]: bits before chunk boundary 1 ..., from its thread's start
+        // The staging buffer is a ring; the place [prev_at, prev_end) of the newest tile handed to the store
+        // warp may still be in use, those before it are free (the polling warp has waited for that).
+        unsigned int prev_at = 0, prev_end = 0;
+        unsigned int n_done = 0;                   // tiles this group has handed to its store warp
         const float inv_range = (float)(a.basis_scale / (a.step * (double)(nsym - 1)));   // the operand holds basis / basis_scale
         const float top = (float)(nsym - 1);
         const float coef_scale = (float)a.basis_scale;
         const int bar_id = 1 + grp;
         bool alive = true;
+        [[maybe_unused]] const int skip_blk = pl.skip_blk;
+        // a position nearer to the modal level than this rounds to it, whatever the last bits of the
+        // two ways to compute it (they agree to 1e-6 of a level)
+        [[maybe_unused]] const float skip_dist = 0.499f / top;
+        const uint32_t trow = tmem_base + grp * kAccCols + ((uint32_t)(wq * 32) << 16);
 
         auto resolve_base = [&](long long tile, unsigned long long padded) {
             if (wg == 0) {
@@ -372,83 +478,186 @@ __global__ void __launch_bounds__(kThreads, 1) encode_tc_kernel(EncodeArgs a)
             const long long tile = blockIdx.x + tl * gridDim.x;
             const long long p = tile * TC_TILE_PIXELS + m;
             const bool valid = p < a.pixels;
-            if (!mbar_wait(smem_u32(&s_tfull[grp]), (uint32_t)((tl >> 1) & 1))) { alive = false; break; }
+            // One warp of the group waits -- for the accumulator, and for the store warp to be done with the
+            // tile before the last -- and lets the others in through a hardware barrier: a parked warp
+            // issues nothing, whereas polling warps took two thirds of the SM's instructions.
+            if (wg == 0) {
+                bool go = mbar_wait(smem_u32(&s_tfull[grp]), (uint32_t)((tl >> 1) & 1), 200u);
+                if (n_done >= 2) go = go && mbar_wait(smem_u32(&s_stg_free[grp][(n_done - 2) % kSlots]), ((n_done - 2) / kSlots) & 1u);
+                if (lane == 0) s_go[grp] = go;
+                tc_fence_before_sync();
+            }
+            named_bar_sync(bar_id, 256);
             tc_fence_after_sync();
-            const uint32_t trow = tmem_base + grp * kAccCols + ((uint32_t)(wq * 32) << 16) + col0;
-
-            // pass 1: quantise, keep the symbols (one byte each) in registers, add up code lengths
-            uint32_t sym[kPair ? kMaxHalfCols / 8 : kMaxHalfCols / 4];   // one byte per symbol, or per pair of symbols
-            uint32_t blk_bits[kMaxHalfCols / 64] = {};          // code bits of each block of 16 symbols, one byte each
-            unsigned int my_bits = 0, bits_first = 0;          // bits_first: the first half of this thread's coefficients
+            if (!s_go[grp]) { alive = false; break; }
             [[maybe_unused]] unsigned int n_clamped = 0;       // statistics mode: coefficients outside the quantiser's range
+
+            // Quantises and codes block `blk` of 16 coefficients, which are on their way into r; `first`: the
+            // tile's first pass (counts for the statistics, debug outputs).  The next block's load is
+            // issued as soon as r has been read: a load waited for at once took 700 cycles beside the MMAs'
+            // traffic, more than the coding.  All lanes of the warp call it together.
+            auto code_block = [&](int blk, uint32_t (&r)[16], auto &sink, auto first) {
+                constexpr bool kCount = std::is_same<std::decay_t<decltype(sink)>, CountSink>::value;
+                constexpr bool kKeep = decltype(first)::value && (kHist || kDebug);        // r is needed once more
+                tmem_ld_wait(r);
+                const uint32_t next = trow + min(blk + 1, blk1 - 1) * 16;
+                uint32_t qv[16];
 #pragma unroll
-            for (int blk = 0; blk < kMaxHalfCols / 16; ++blk) {
-                if (blk * 16 < ncols) {
-                    if (blk * 32 == ncols) bits_first = my_bits;
-                    const unsigned int bits_before = my_bits;
-                    uint32_t r[16];
-                    tmem_ld_32x32b_x16(trow + blk * 16, r);
-                    float4 bias4[4];
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) bias4[i] = *reinterpret_cast<const float4 *>(s_bias + col0 + blk * 16 + 4 * i);
-                    const float *biasv = reinterpret_cast<const float *>(bias4);
-                    tmem_ld_wait();
-                    uint32_t qv[16];
-#pragma unroll
-                    for (int i = 0; i < 16; i += 2) quantise_bits2(r[i], r[i + 1], inv_range, biasv[i], biasv[i + 1], top, qv[i], qv[i + 1]);
-                    if constexpr (kHist) {
-                        // every symbol other than the zero level is counted; the zero level's count is what
-                        // is left of the pixels, which the caller works out
-                        const uint32_t modal_bits = kMagicBits + (uint32_t)a.hist_modal;
-#pragma unroll
-                        for (int i = 0; i < 16; ++i) {
-                            const int j = col0 + blk * 16 + i;
-                            if (valid && qv[i] != modal_bits) atomicAdd(a.hist + (size_t)j * nsym + (qv[i] & 0xffu), 1ull);
-                            // outside the quantiser's range [lo, lo + (2^b - 1) step]
-                            const float t = fmaf(__uint_as_float(r[i]), inv_range, biasv[i]);
-                            n_clamped += (valid && (t < 0.f || t > 1.f)) ? 1u : 0u;
-                        }
-                    }
+                for (int i = 0; i < 16; i += 4) {
+                    const float4 b4 = *reinterpret_cast<const float4 *>(s_bias + blk * 16 + i);
+                    quantise_bits2(r[i], r[i + 1], inv_range, b4.x, b4.y, top, qv[i], qv[i + 1]);
+                    quantise_bits2(r[i + 2], r[i + 3], inv_range, b4.z, b4.w, top, qv[i + 2], qv[i + 3]);
+                }
+                if constexpr (!kKeep) tmem_ld_32x32b_x16(next, r);
+                if constexpr (kKeep) {
 #pragma unroll
                     for (int i = 0; i < 16; ++i) {
-                        const int j = col0 + blk * 16 + i;
-                        const uint32_t vb = qv[i];
-                        if constexpr (kPerChannel) my_bits += __ldg(a.enc + j * nsym + (vb & 0xffu)) & 0xffu;
-                        else if constexpr (!kPair) {
-                            uint32_t l;
-                            asm("ld.shared.u8 %0, [%1];" : "=r"(l) : "r"(vb + len8_rel));
-                            my_bits += l;
+                        const int j = blk * 16 + i;
+                        if constexpr (kHist) {
+                            // every symbol other than the zero level is counted; the zero level's count is what
+                            // is left of the pixels, which the caller works out
+                            if (valid && qv[i] != kMagicBits + (uint32_t)a.hist_modal) atomicAdd(a.hist + (size_t)j * nsym + (qv[i] & 0xffu), 1ull);
+                            // outside the quantiser's range [lo, lo + (2^b - 1) step]
+                            const float t = fmaf(__uint_as_float(r[i]), inv_range, s_bias[j]);
+                            n_clamped += (valid && (t < 0.f || t > 1.f)) ? 1u : 0u;
                         }
                         if constexpr (kDebug) {
                             if (valid && a.dbg_coef) a.dbg_coef[p * a.k + j] = fmaf(__uint_as_float(r[i]), coef_scale, -a.tmu32[j]);
-                            if (valid && a.dbg_sym) a.dbg_sym[p * a.k + j] = (uint8_t)(vb & 0xffu);
+                            if (valid && a.dbg_sym) a.dbg_sym[p * a.k + j] = (uint8_t)(qv[i] & 0xffu);
                         }
-                        r[i] = vb;
                     }
-                    if constexpr (kPair) {
-                        // pair index in the low byte of vb0 + (vb1 << b) (the magic constants have a zero
-                        // low byte); the same sum, rebased, addresses the pair-length table
+                }
+                if constexpr (kKeep) tmem_ld_32x32b_x16(next, r);
+                if constexpr (kCount) {
 #pragma unroll
-                        for (int i = 0; i < 16; i += 2) {
-                            r[i] = r[i] + (r[i + 1] << a.bits);
-                            uint32_t l;
-                            asm("ld.shared.u8 %0, [%1];" : "=r"(l) : "r"(r[i] + pair_len_rel));
-                            my_bits += l;
+                    for (int i = 0; i < 16; i += kPair ? 2 : 1) {
+                        uint32_t l;
+                        if constexpr (kPerChannel) l = __ldg(a.enc + (blk * 16 + i) * nsym + (qv[i] & 0xffu)) & 0xffu;
+                        else {
+                            // (the magic constant is zero in the low bits; its upper bits fall out of the address)
+                            uint32_t idx = qv[i] - kMagicBits;
+                            if constexpr (kPair) idx += (qv[i + 1] - kMagicBits) << a.bits;
+                            asm("ld.shared.u8 %0, [%1];" : "=r"(l) : "r"(len8_addr + idx));
                         }
+                        sink.bits += l;
+                    }
+                } else {
+                    // two symbols a piece: (1 << length, code), at most 24 bits
+                    uint32_t mul[8], code[8];
 #pragma unroll
-                        for (int i = 0; i < 16; i += 8)      // low bytes of four pairs -> one register
-                            sym[blk * 2 + i / 8] = __byte_perm(__byte_perm(r[i], r[i + 2], 0x0040), __byte_perm(r[i + 4], r[i + 6], 0x0040), 0x5410);
+                    for (int i = 0; i < 8; ++i) {
+                        if constexpr (kPair) {
+                            const uint32_t idx = (qv[2 * i] - kMagicBits) + ((qv[2 * i + 1] - kMagicBits) << a.bits);
+                            asm("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(mul[i]), "=r"(code[i]) : "r"(enc_addr + idx * 8u));
+                        } else {
+                            uint32_t m0, c0, m1, c1;
+                            if constexpr (kPerChannel) {
+                                const int j = blk * 16 + 2 * i;
+                                const uint32_t e0 = __ldg(a.enc + j * nsym + (qv[2 * i] & 0xffu)), e1 = __ldg(a.enc + (j + 1) * nsym + (qv[2 * i + 1] & 0xffu));
+                                m0 = 1u << (e0 & 0xffu); c0 = e0 >> 8; m1 = 1u << (e1 & 0xffu); c1 = e1 >> 8;
+                            } else {
+                                asm("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(m0), "=r"(c0) : "r"(enc_addr + (qv[2 * i] - kMagicBits) * 8u));
+                                asm("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(m1), "=r"(c1) : "r"(enc_addr + (qv[2 * i + 1] - kMagicBits) * 8u));
+                            }
+                            mul[i] = m0 * m1;
+                            code[i] = c0 * m1 + c1;
+                        }
+                    }
+                    // How many symbols are joined before they are appended is chosen for the whole warp (lanes
+                    // that go different ways run one after the other): sixteen or eight where every lane's
+                    // codes of them fit 31 bits -- a product of powers of two that reaches 2^32 is zero --
+                    // else four, else two.  Joining is a multiply-add, appending costs ten instructions.
+                    uint32_t m4[4], c4[4];
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) { m4[i] = mul[2 * i] * mul[2 * i + 1]; c4[i] = code[2 * i] * mul[2 * i + 1] + code[2 * i + 1]; }
+                    const uint32_t m8a = m4[0] * m4[1], m8b = m4[2] * m4[3];
+                    if (__all_sync(0xffffffffu, m8a != 0u && m8b != 0u)) {
+                        const uint32_t c8a = c4[0] * m4[1] + c4[1], c8b = c4[2] * m4[3] + c4[3], m16 = m8a * m8b;
+                        if (__all_sync(0xffffffffu, m16 != 0u)) sink.put(c8a * m8b + c8b, 31 - __clz((int)m16));
+                        else { sink.put(c8a, 31 - __clz((int)m8a)); sink.put(c8b, 31 - __clz((int)m8b)); }
                     } else {
 #pragma unroll
-                        for (int i = 0; i < 16; i += 4)      // low bytes of four values -> one register
-                            sym[blk * 4 + i / 4] = __byte_perm(__byte_perm(r[i], r[i + 1], 0x0040), __byte_perm(r[i + 2], r[i + 3], 0x0040), 0x5410);
+                        for (int i = 0; i < 4; ++i) {
+                            if (__all_sync(0xffffffffu, m4[i] != 0u)) sink.put(c4[i], 31 - __clz((int)m4[i]));
+                            else { sink.put(code[2 * i], 31 - __clz((int)mul[2 * i])); sink.put(code[2 * i + 1], 31 - __clz((int)mul[2 * i + 1])); }
+                        }
                     }
-                    blk_bits[blk >> 2] |= (my_bits - bits_before) << (8 * (blk & 3));      // at most 16 * 12 = 192
                 }
+            };
+
+            // The thread's blocks in order; `mark(i)` is called where the i-th chunk boundary of the pixel
+            // (1 ...) lies before a block.  From skip_blk on two blocks at a time are tested for holding nothing
+            // but the modal symbol.
+            auto code_blocks = [&](auto &sink, auto first, auto &&mark) {
+                constexpr bool kCount = std::is_same<std::decay_t<decltype(sink)>, CountSink>::value;
+                if (blk0 >= blk1) return;
+                int blk = blk0, bound_i = bound0, bound_blk = bound0 * chunk_blks;
+                auto at = [&] {
+                    if (blk == bound_blk) { mark(bound_i); ++bound_i; bound_blk += chunk_blks; }
+                };
+                // blocks up to `end` one by one
+                auto one_by_one = [&](int end) {
+                    if (blk >= end) return;
+                    uint32_t r[16];
+                    tmem_ld_32x32b_x16(trow + blk * 16, r);
+#pragma unroll 1
+                    do {
+                        at();
+                        code_block(blk, r, sink, first);
+                    } while (++blk < end);
+                    tmem_ld_wait(r);
+                };
+                if constexpr (!kCanSkip) one_by_one(blk1);
+                else {
+#pragma unroll 1
+                    while (blk < blk1) {
+                        int plain = min(max(skip_blk, blk), blk1);           // this far without the test
+                        if (plain + 2 > blk1) plain = blk1;
+                        one_by_one(plain);
+#pragma unroll 1
+                        while (blk + 2 <= blk1 && bound_blk != blk + 1) {
+                            uint32_t r0[16], r1[16];
+                            tmem_ld_32x32b_x16(trow + blk * 16, r0);
+                            tmem_ld_32x32b_x16(trow + blk * 16 + 16, r1);
+                            float4 mid[8];
+#pragma unroll
+                            for (int i = 0; i < 8; ++i) mid[i] = *reinterpret_cast<const float4 *>(s_bias_mid + blk * 16 + 4 * i);
+                            tmem_ld_wait(r0);
+                            tmem_ld_wait(r1);
+                            // farthest of the 32 positions from the modal level (not a number: stays one, fails the test)
+                            float far[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+                            for (int i = 0; i < 4; ++i) {
+                                farthest2(far[0], r0[4 * i], r0[4 * i + 1], inv_range, mid[i].x, mid[i].y);
+                                farthest2(far[1], r0[4 * i + 2], r0[4 * i + 3], inv_range, mid[i].z, mid[i].w);
+                                farthest2(far[2], r1[4 * i], r1[4 * i + 1], inv_range, mid[4 + i].x, mid[4 + i].y);
+                                farthest2(far[3], r1[4 * i + 2], r1[4 * i + 3], inv_range, mid[4 + i].z, mid[4 + i].w);
+                            }
+                            if (!__all_sync(0xffffffffu, (far[0] < skip_dist) & (far[1] < skip_dist) & (far[2] < skip_dist) & (far[3] < skip_dist))) break;
+                            at();
+                            if constexpr (kCount) sink.bits += 32;             // 32 times the code 0 (one bit)
+                            else sink.put_word(0u);
+                            blk += 2;
+                        }
+                        if (blk < blk1) one_by_one(min(blk + 2, blk1));
+                    }
+                }
+            };
+
+            // first pass: code lengths, and with private runs the codes
+            unsigned int my_bits;
+            [[maybe_unused]] SmemBitWriter<kRunStep> run;
+            if constexpr (kRuns) {
+                run.init(run_addr, run_end, 0u);
+                auto bits_so_far = [&] { return (run.addr - run_addr) / (kRunStep / 32) + (unsigned int)run.pending; };
+                code_blocks(run, std::true_type{}, [&](int i) { bound[(i - 1) * 128 + m] = (unsigned short)bits_so_far(); });
+                my_bits = bits_so_far();
+                if (__any_sync(0xffffffffu, run.addr > run_end) && lane == 0) s_overflow[grp] = n_done + 1;
+            } else {
+                CountSink count{0u};
+                code_blocks(count, std::true_type{}, [&](int i) { bound[(i - 1) * 128 + m] = (unsigned short)count.bits; });
+                my_bits = count.bits;
             }
-            // the accumulator buffer is free for the tile after next
-            tc_fence_before_sync();
-            mbar_arrive(smem_u32(&s_tempty[grp]));
             if constexpr (kHist) {
                 if (a.clamped) {
 #pragma unroll
@@ -458,166 +667,155 @@ __global__ void __launch_bounds__(kThreads, 1) encode_tc_kernel(EncodeArgs a)
             }
             if (!valid) my_bits = 0;
 
-            // bit offsets: pixel-major, first half before second half
-            xch[half * 128 + m] = (unsigned short)my_bits;     // at most 128 * 12 bits
-            named_bar_sync(bar_id, 256);
-            const unsigned int other = xch[(half ^ 1) * 128 + m];
-            const unsigned int pair = my_bits + other;
-            unsigned int inc = pair;
+            // bit offsets: pixel-major, first half before second half.  Each warp scans its own half's bits of
+            // its 32 pixels; a pixel's offset is the sum of both halves' prefixes.
+            unsigned int inc = my_bits;
 #pragma unroll
             for (int d = 1; d < 32; d <<= 1) {
                 const unsigned int up = __shfl_up_sync(0xffffffffu, inc, d);
                 if (lane >= d) inc += up;
             }
-            if (lane == 31 && half == 0) s_warp_sums[grp][wq] = inc;
+            xch[half * 128 + m] = ((inc - my_bits) << 12) | my_bits;       // at most 31 * 256 * 12 bits before, 256 * 12 own
+            if (lane == 31) s_warp_sums[grp][half][wq] = inc;
             named_bar_sync(bar_id, 256);
-            unsigned int before = 0, tile_bits = 0;
+            const uint32_t theirs = xch[(half ^ 1) * 128 + m];
+            const unsigned int other = theirs & 0xfffu, pixel_bits = my_bits + other;
+            unsigned int before = 0, tile_bits = 0, warp_bits = 0;
 #pragma unroll
             for (int w = 0; w < 4; ++w) {
-                const unsigned int sw = s_warp_sums[grp][w];
+                const unsigned int sw = s_warp_sums[grp][0][w] + s_warp_sums[grp][1][w];
                 if (w < wq) before += sw;
+                if (w == wq) warp_bits = sw;
                 tile_bits += sw;
             }
-            const unsigned int pixel_off = before + inc - pair;
+            const unsigned int pixel_off = before + (inc - my_bits) + (theirs >> 12);
             const unsigned int my_off = pixel_off + (half ? other : 0u);
-            // end of the chunk that starts at this pixel (chunks of several pixels): the offset of
-            // the pixel chunk_pixels further on, which sits in this warp, or is a sum of warp totals
-            unsigned int chunk_end = 0;
+            // chunk lengths.  Chunks of several pixels: a chunk ends at the offset of the pixel chunk_pixels
+            // further on, which sits in this warp, or is a sum of warp totals.  Several chunks per pixel:
+            // from the bits before their boundaries.
             if (a.chunk_pixels > 1) {
                 const int cpx = a.chunk_pixels;
+                unsigned int chunk_end = 0;
                 if (cpx < 32) {
                     const unsigned int further = __shfl_down_sync(0xffffffffu, pixel_off, cpx);
-                    chunk_end = (lane + cpx < 32) ? further : before + s_warp_sums[grp][wq];
+                    chunk_end = (lane + cpx < 32) ? further : before + warp_bits;
                 } else {
 #pragma unroll
                     for (int w = 0; w < 4; ++w)
-                        if (w < wq + (cpx >> 5)) chunk_end += s_warp_sums[grp][w];
+                        if (w < wq + (cpx >> 5)) chunk_end += s_warp_sums[grp][0][w] + s_warp_sums[grp][1][w];
+                }
+                if (valid && half == 0 && (m & (cpx - 1)) == 0) a.chunk_len[p >> (__ffs(cpx) - 1)] = (uint16_t)(chunk_end - pixel_off);
+            } else if (valid && half == 0) {
+                if (a.splits == 1) a.chunk_len[p] = (uint16_t)pixel_bits;
+                else {
+                    // start of chunk s in the pixel: a boundary among the second half's blocks counts from my_bits on
+                    auto starts = [&](int sc) { return bound[(sc - 1) * 128 + m] + (sc * chunk_blks >= pl.split_blk ? my_bits : 0u); };
+                    uint32_t *dst = reinterpret_cast<uint32_t *>(a.chunk_len + a.splits * p);
+                    const unsigned int s1 = starts(1);
+                    if (a.splits == 2) dst[0] = s1 | ((pixel_bits - s1) << 16);
+                    else {
+                        const unsigned int s2 = starts(2), s3 = starts(3);
+                        dst[0] = s1 | ((s2 - s1) << 16);
+                        dst[1] = (s3 - s2) | ((pixel_bits - s3) << 16);
+                    }
                 }
             }
             const unsigned long long padded = ((unsigned long long)tile_bits + 127ull) & ~127ull;
             if (tg == 0) lookback_publish(a.tile_state, tile, padded);
-            const bool staged = padded <= (unsigned long long)kStagingBytes * 8ull;
-            // the store warp must be done with the previous tile before staging is written again
-            if (n_done > 0 && !mbar_wait(smem_u32(&s_stg_free[grp]), (uint32_t)((n_done - 1) & 1))) { alive = false; break; }
+            const bool staged = padded <= (unsigned long long)pl.staging_bytes * 8ull && !(kRuns && s_overflow[grp] == n_done + 1);
+            if (kRuns && staged) {                 // the accumulator is free for the tile after next
+                tc_fence_before_sync();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(smem_u32(&s_tempty[grp]));
+            }
+            // place in the staging ring: behind the newest tile, or at the buffer's start if it would not
+            // fit before the end
+            const unsigned int tile_bytes = staged ? (unsigned int)(padded >> 3) : 0u;
+            const unsigned int stg_at = prev_end + tile_bytes > pl.staging_bytes ? 0u : prev_end;
+            if (n_done >= 1 && stg_at < prev_end && prev_at < stg_at + tile_bytes &&
+                !mbar_wait(smem_u32(&s_stg_free[grp][(n_done - 1) % kSlots]), ((n_done - 1) / kSlots) & 1u)) { alive = false; break; }
+            prev_at = stg_at;
+            prev_end = stg_at + tile_bytes;
+            const uint32_t tile_addr = stg_addr + stg_at;
 
             if (staged) {
                 // every word below tile_bits / 32 is stored by the writer of its last bit; the last
                 // partial word and the padding up to the 128-bit boundary start as zero
                 const unsigned int first_open = tile_bits >> 5, end_word = (unsigned int)(padded >> 5);
                 if ((unsigned int)tg < end_word - first_open)
-                    asm volatile("st.shared.u32 [%0], %1;" ::"r"(stg_addr + (first_open + tg) * 4u), "r"(0u) : "memory");
+                    asm volatile("st.shared.u32 [%0], %1;" ::"r"(tile_addr + (first_open + tg) * 4u), "r"(0u) : "memory");
+                if constexpr (kRuns) {
+                    // the run's words, shifted to the thread's offset
+                    const int sh = (int)(my_off & 31u);
+                    const unsigned int n_words = my_bits >> 5;
+                    uint32_t dst = tile_addr + (my_off >> 5) * 4u, src = run_addr, prev = 0;
+                    const unsigned int most = __reduce_max_sync(0xffffffffu, n_words);
+#pragma unroll 2
+                    for (unsigned int i = 0; i < most; ++i) {
+                        if (i < n_words) {
+                            uint32_t w;
+                            asm volatile("ld.shared.u32 %0, [%1];" : "=r"(w) : "r"(src));
+                            asm volatile("st.shared.u32 [%0], %1;" ::"r"(dst), "r"(__funnelshift_r(w, prev, sh)) : "memory");
+                            prev = w;
+                            src += kRunStep;
+                            dst += 4;
+                        }
+                    }
+                    const int rest = valid ? run.pending : 0;
+                    const uint32_t last = rest ? run.lo << (32 - rest) : 0u;
+                    uint32_t tail = __funnelshift_r(last, prev, sh);
+                    if (sh + rest >= 32) {
+                        asm volatile("st.shared.u32 [%0], %1;" ::"r"(dst), "r"(tail) : "memory");
+                        dst += 4;
+                        tail = last << (32 - sh);
+                    }
+                    named_bar_sync(bar_id, 256);      // all full words stored
+                    if (tail && valid) asm volatile("red.shared.or.b32 [%0], %1;" ::"r"(dst), "r"(tail) : "memory");
+                } else {
+                    SmemBitWriter<4> w;
+                    w.init(valid ? tile_addr : 0u, valid ? tile_addr + tile_bytes : 0u, valid ? my_off : 0u);
+                    code_blocks(w, std::false_type{}, [](int) {});
+                    tc_fence_before_sync();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(smem_u32(&s_tempty[grp]));
+                    named_bar_sync(bar_id, 256);
+                    w.finish();
+                }
+                if (tg == 0) { s_padded[grp][n_done % kSlots] = (unsigned int)padded; s_stg_at[grp][n_done % kSlots] = stg_at; s_store_cmd[grp][n_done % kSlots] = 1; }
             } else {
-                // rare: the tile does not fit the staging buffer -> resolve its position first and
-                // pack straight into (zeroed) global memory
+                // rare: the tile (or a run) does not fit -> resolve its position first and pack straight
+                // into (zeroed) global memory
                 resolve_base(tile, padded);
                 named_bar_sync(bar_id, 256);
                 if (s_write_ok[grp]) {
                     uint4 *z = reinterpret_cast<uint4 *>(a.stream + (s_base[grp] >> 5));
                     for (unsigned int i = tg; i < (unsigned int)(padded >> 7); i += 256) z[i] = make_uint4(0u, 0u, 0u, 0u);
                 }
-            }
-            named_bar_sync(bar_id, 256);
-
-            // pass 2: look up the codes of the kept symbols and pack; two symbols are joined in
-            // registers and appended as one piece of at most 24 bits
-            const bool do_pack = valid && (staged || s_write_ok[grp]);
-            auto pack_tile = [&](auto &w) {
-                if (!do_pack) return;
-#pragma unroll
-                for (int blk = 0; blk < kMaxHalfCols / 16; ++blk) {
-                    if (blk * 16 < ncols) {
-#pragma unroll
-                        const int nbits = (int)((blk_bits[blk >> 2] >> (8 * (blk & 3))) & 0xffu);
-                        if (!kPerChannel && nbits < 32) {
-                            // the whole block fits one register: acc = acc * 2^len + code per symbol (or pair)
-                            uint32_t acc = 0;
-                            if constexpr (kPair) {
-#pragma unroll
-                                for (int i = 0; i < 8; ++i) {
-                                    const uint32_t q = (sym[blk * 2 + i / 4] >> (8 * (i & 3))) & 0xffu;
-                                    uint32_t mul, code;
-                                    asm("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(mul), "=r"(code) : "r"(enc_addr + q * 8u));
-                                    acc = acc * mul + code;
-                                }
-                            } else {
-#pragma unroll
-                                for (int i = 0; i < 16; ++i) {
-                                    const uint32_t q = (sym[blk * 4 + i / 4] >> (8 * (i & 3))) & 0xffu;
-                                    uint32_t mul, code;
-                                    asm("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(mul), "=r"(code) : "r"(enc_addr + q * 8u));
-                                    acc = acc * mul + code;
-                                }
-                            }
-                            w.put(acc, nbits);
-                        } else if constexpr (kPair) {
-#pragma unroll
-                            for (int i = 0; i < 8; ++i) {         // pair by pair: at most 24 bits each
-                                const uint32_t q = (sym[blk * 2 + i / 4] >> (8 * (i & 3))) & 0xffu;
-                                uint32_t code, l;
-                                asm("ld.shared.u32 %0, [%1];" : "=r"(code) : "r"(enc_addr + q * 8u + 4u));
-                                asm("ld.shared.u8 %0, [%1];" : "=r"(l) : "r"(len8_rel + kMagicBits + q));
-                                w.put(code, (int)l);
-                            }
-                        } else {
-#pragma unroll
-                            for (int i = 0; i < 16; i += 2) {
-                                const uint32_t word = sym[blk * 4 + i / 4];
-                                const uint32_t q0 = (word >> (8 * (i & 3))) & 0xffu, q1 = (word >> (8 * ((i + 1) & 3))) & 0xffu;
-                                uint32_t c0, c1, l0, l1;
-                                if constexpr (kPerChannel) {
-                                    const int j = col0 + blk * 16 + i;
-                                    const uint32_t e0 = __ldg(a.enc + j * nsym + q0), e1 = __ldg(a.enc + (j + 1) * nsym + q1);
-                                    c0 = e0 >> 8; l0 = e0 & 0xffu; c1 = e1 >> 8; l1 = e1 & 0xffu;
-                                } else {
-                                    asm("ld.shared.u32 %0, [%1];" : "=r"(c0) : "r"(enc_addr + q0 * 8u + 4u));
-                                    asm("ld.shared.u32 %0, [%1];" : "=r"(c1) : "r"(enc_addr + q1 * 8u + 4u));
-                                    asm("ld.shared.u8 %0, [%1];" : "=r"(l0) : "r"(len8_rel + kMagicBits + q0));
-                                    asm("ld.shared.u8 %0, [%1];" : "=r"(l1) : "r"(len8_rel + kMagicBits + q1));
-                                }
-                                w.put((c0 << l1) | c1, (int)(l0 + l1));
-                            }
-                        }
-                    }
-                }
-            };
-            if (staged) {
-                SmemBitWriter ws;
-                ws.init(stg_addr, my_off);
-                pack_tile(ws);
-                named_bar_sync(bar_id, 256);      // all full words stored
-                if (do_pack) ws.finish();
-                if (tg == 0) { s_padded[grp] = padded; s_store_cmd[grp] = 1; }
-            } else {
-                BitWriter wgl;
-                wgl.init(a.stream, s_base[grp] + my_off);
-                pack_tile(wgl);
-                if (do_pack) wgl.finish();
+                named_bar_sync(bar_id, 256);
+                GlobalSink g;
+                g.on = valid && s_write_ok[grp];
+                g.w.init(a.stream, s_base[grp] + my_off);
+                code_blocks(g, std::false_type{}, [](int) {});
+                if (g.on) g.w.finish();
+                tc_fence_before_sync();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(smem_u32(&s_tempty[grp]));
                 if (tg == 0) {
                     const unsigned long long base = s_base[grp];
                     a.tile_off[tile] = base;
                     if (tile == a.n_tiles - 1) a.tile_off[a.n_tiles] = base + padded;
-                    s_store_cmd[grp] = 2;
+                    s_store_cmd[grp][n_done % kSlots] = 2;
                 }
             }
-            // hand the tile to the store warp (each thread's arrival releases its own writes)
-            mbar_arrive(smem_u32(&s_stg_full[grp]));
+            // hand the tile to the store warp (a warp's arrival releases its lanes' writes)
+            __syncwarp();
+            if (lane == 0) mbar_arrive(smem_u32(&s_stg_full[grp][n_done % kSlots]));
             ++n_done;
-            // chunk lengths: with four chunks per pixel each thread writes the two of its half
-            // (one aligned word); otherwise the first half's thread of a pixel writes them
-            if (valid && a.splits == 4)
-                *reinterpret_cast<uint32_t *>(a.chunk_len + 4 * p + 2 * half) = bits_first | ((my_bits - bits_first) << 16);
-            else if (valid && half == 0) {
-                if (a.splits == 2)                        // one chunk per half: both lengths in one aligned word
-                    *reinterpret_cast<uint32_t *>(a.chunk_len + 2 * p) = my_bits | (other << 16);
-                else if (a.chunk_pixels == 1)
-                    a.chunk_len[p] = (uint16_t)pair;
-                else if ((p % a.chunk_pixels) == 0)
-                    a.chunk_len[p / a.chunk_pixels] = (uint16_t)(chunk_end - pixel_off);
-            }
         }
         if (!alive) {
-            if (tg == 0) { tc_dev_set_status(a.status, TC_ERR_TIMEOUT); s_store_cmd[grp] = 3; }
-            mbar_arrive(smem_u32(&s_stg_full[grp]));   // lets the store warp leave
+            if (tg == 0) { tc_dev_set_status(a.status, TC_ERR_TIMEOUT); s_store_cmd[grp][n_done % kSlots] = 3; }
+            __syncwarp();
+            if (lane == 0) mbar_arrive(smem_u32(&s_stg_full[grp][n_done % kSlots]));   // lets the store warp leave
         }
     }
 
@@ -632,12 +830,55 @@ __global__ void __launch_bounds__(kThreads, 1) encode_tc_kernel(EncodeArgs a)
 
 }  // namespace
 
-// entries of the code table held in shared memory: none (per-channel tables stay in global
-// memory), one per symbol, or one per pair of symbols
-static int enc_table_entries(const EncodeArgs &a)
+// What a launch does with the shared memory that the basis leaves, from the code lengths to expect of
+// the model's coefficients (a code without a one-bit symbol: b bits for each).  A tile's size varies
+// by a few per cent about its mean, a thread's run by its symbols that are not the zero level.  A tile
+// that breaks the estimate is coded at about a quarter of the speed (straight into global memory).
+// Preferred, in this order: symbol pairs before single symbols, private runs before two passes, eight
+// ring stages before six.
+static Plan make_plan(const tc_ctx *ctx, const EncodeArgs &a)
 {
-    if (a.groups != 1) return 0;
-    return a.bits <= kPairMaxBits ? (1 << (2 * a.bits)) : (1 << a.bits);
+    const int n_blk = a.k / 16;
+    const bool modal = a.groups == 1 && a.modal >= 0;
+    auto blk_bits = [&](int b) { return modal || a.groups != 1 ? a.blk_bits[b] : std::max(a.blk_bits[b], 16.f * a.bits); };
+    Plan best{};
+    // A test of 32 coefficients x 32 pixels pays from a success in three on: fewer than about one other
+    // symbol expected in it.
+    best.skip_blk = n_blk;
+    while (modal && best.skip_blk > 0 && 64.f * a.blk_odd[best.skip_blk - 1] < 1.2f) --best.skip_blk;
+    // blocks of the two threads of a pixel: equal work, a coded block counted as three passed over
+    auto cost = [&](int b0, int b1) { return 3 * std::max(0, std::min(b1, best.skip_blk) - b0) + (b1 - std::max(b0, std::min(b1, best.skip_blk))); };
+    best.split_blk = 1;
+    for (int x = 2; x <= n_blk; ++x)
+        if (std::max(cost(0, x), cost(x, n_blk)) < std::max(cost(0, best.split_blk), cost(best.split_blk, n_blk))) best.split_blk = x;
+    double tile_bits = 0.0;
+    int want_words[2];
+    for (int h = 0; h < 2; ++h) {
+        double bits = 0.0, odd = 0.0;
+        const int b0 = h ? best.split_blk : 0, b1 = h ? n_blk : best.split_blk;
+        for (int b = b0; b < b1; ++b) { bits += blk_bits(b); odd += a.blk_odd[b]; }
+        tile_bits += TC_TILE_PIXELS * bits;
+        // (the largest of 10^5 threads' runs: about 10 standard deviations' worth of other symbols)
+        want_words[h] = b1 > b0 ? std::min((int)((bits + 11.0 * std::sqrt(odd)) / 32.0) + 2, (b1 - b0) * 6) : 0;
+    }
+    const uint32_t want_staging = (uint32_t)(1.08 * tile_bits / 8.0) + 128u;
+    const int budget = ctx->max_smem_optin - kStaticSmem;
+    for (int t = 0; t < 8; ++t) {
+        Plan pl = best;
+        const bool pair = !(t & 4), runs = !(t & 2);
+        if (pair && (a.groups != 1 || a.bits > kPairMaxBits)) continue;
+        pl.stages = (t & 1) ? 6 : 8;
+        pl.entries = a.groups != 1 ? 0 : pair ? 1 << (2 * a.bits) : 1 << a.bits;
+        for (int h = 0; h < 2; ++h) pl.run_words[h] = runs ? want_words[h] : 0;
+        pl.staging_bytes = 0;
+        const long long left = (long long)budget - smem_layout(a.c, a.k, pl).total;
+        const long long per_group = (left / 2) & ~15ll;
+        if (per_group < 4096 || (per_group < (long long)want_staging && t != 7)) continue;
+        pl.staging_bytes = (uint32_t)std::min<long long>(per_group, kMaxStagingBytes);
+        return pl;
+    }
+    best.staging_bytes = 0;
+    return best;
 }
 
 bool tc_encode_tc_supported(const tc_ctx *ctx, const EncodeArgs &a)
@@ -646,30 +887,37 @@ bool tc_encode_tc_supported(const tc_ctx *ctx, const EncodeArgs &a)
     if (a.c % 16 != 0 || a.k % 16 != 0 || a.k < 16 || a.k > a.c || a.c > 256 || a.hw % 4 != 0) return false;
     // the loaders copy groups of four pixels with 8-byte cp.async: the tensor must start on an 8-byte boundary
     if (((uintptr_t)a.x & 7u) != 0) return false;
-    // two chunks per pixel must coincide with the two halves the epilogue threads work on
-    // (four chunks: each half splits once more in its middle)
+    // chunks are whole blocks of 16 coefficients
     if (a.splits != 1 && !(a.splits == 2 && a.k % 32 == 0) && !(a.splits == 4 && a.k % 64 == 0 && a.chunk_pixels == 1)) return false;
     if (a.groups != 1 && a.groups != a.k) return false;
-    const SmemLayout l = smem_layout(a.c, a.k, enc_table_entries(a));
-    return (int)l.total + kStaticSmem <= ctx->max_smem_optin;       // leaves room for the static shared variables
+    return make_plan(ctx, a).staging_bytes > 0;
+}
+
+template <bool kPerChannel, bool kPair, bool kRuns>
+static void (*pick_kernel(bool debug, bool hist))(EncodeArgs, Plan)
+{
+    if constexpr (!kPerChannel)
+        if (hist) return encode_tc_kernel<false, false, kPair, true, kRuns>;
+    return debug ? encode_tc_kernel<kPerChannel, true, kPair, false, kRuns> : encode_tc_kernel<kPerChannel, false, kPair, false, kRuns>;
 }
 
 tc_status tc_launch_encode_tc(const tc_ctx *ctx, const EncodeArgs &a, cudaStream_t s)
 {
     if (a.n_tiles <= 0) return TC_OK;
-    const SmemLayout l = smem_layout(a.c, a.k, enc_table_entries(a));
-    const bool per_channel = a.groups != 1, debug = a.dbg_coef || a.dbg_sym, pair = !per_channel && a.bits <= kPairMaxBits;
+    const bool per_channel = a.groups != 1, debug = a.dbg_coef || a.dbg_sym;
     if (a.hist && (per_channel || debug)) return TC_ERR_UNSUPPORTED;      // statistics run with a per-layer table
-    void (*kernel)(EncodeArgs) =
-        a.hist      ? (pair ? encode_tc_kernel<false, false, true, true> : encode_tc_kernel<false, false, false, true>)
-        : per_channel ? (debug ? encode_tc_kernel<true, true, false, false> : encode_tc_kernel<true, false, false, false>)
-        : pair      ? (debug ? encode_tc_kernel<false, true, true, false> : encode_tc_kernel<false, false, true, false>)
-                    : (debug ? encode_tc_kernel<false, true, false, false> : encode_tc_kernel<false, false, false, false>);
+    Plan pl = make_plan(ctx, a);
+    if (pl.staging_bytes == 0) return TC_ERR_UNSUPPORTED;
+    const bool pair = !per_channel && pl.entries > (1 << a.bits), runs = pl.run_words[0] > 0;
+    const SmemLayout l = smem_layout(a.c, a.k, pl);
+    void (*kernel)(EncodeArgs, Plan) = per_channel ? (runs ? pick_kernel<true, false, true>(debug, false) : pick_kernel<true, false, false>(debug, false))
+                                     : pair        ? (runs ? pick_kernel<false, true, true>(debug, a.hist) : pick_kernel<false, true, false>(debug, a.hist))
+                                                   : (runs ? pick_kernel<false, false, true>(debug, a.hist) : pick_kernel<false, false, false>(debug, a.hist));
     if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)l.total) != cudaSuccess)
         return TC_ERR_CUDA;
     const unsigned int grid = (unsigned int)((a.n_tiles < ctx->sm_count) ? a.n_tiles : ctx->sm_count);
     EncodeArgs args = a;
-    void *params[] = {&args};
+    void *params[] = {&args, &pl};
     // cooperative launch: the grid must be co-resident, which is what makes the look-back safe
     const cudaError_t err = cudaLaunchCooperativeKernel((void *)kernel, dim3(grid), dim3(kThreads), params, l.total, s);
     if (err != cudaSuccess) {

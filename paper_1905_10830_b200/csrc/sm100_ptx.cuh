@@ -51,13 +51,15 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, uint32_
     if (mbar_try_wait(bar, parity, 0u)) return true;
     unsigned long long t0, t1;
     asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t0));
-    // (one compact loop: with the inner loop of 64 attempts it had before, which the compiler unrolled at
-    // every call, the waits were a quarter of the kernels' code, and instruction fetch is what a
-    // kernel of one or two tiles per SM spends most of its time on)
-#pragma unroll 1
+    // (rolled: with the 64 attempts unrolled at every call the waits were a quarter of the kernels' code;
+    // the clock is read once per 64 attempts: a waiting warp's instructions come out of the issue
+    // slots of the warps that work)
     while (true) {
-        __nanosleep(sleep_ns);
-        if (mbar_try_wait(bar, parity, 100000u)) return true;
+#pragma unroll 1
+        for (int i = 0; i < 64; ++i) {
+            __nanosleep(sleep_ns);
+            if (mbar_try_wait(bar, parity, 100000u)) return true;
+        }
         asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t1));
         if (t1 - t0 > 2000000000ull) return false;
     }
@@ -106,6 +108,13 @@ __device__ __forceinline__ void cp_async_wait()
 {
     asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
 }
+__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+// The barrier gets one of its expected arrivals when every cp.async this thread has issued so far has
+// landed; the thread does not wait.
+__device__ __forceinline__ void cp_async_arrive_noinc(uint32_t bar)
+{
+    asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(bar) : "memory");
+}
 
 // ---- tensor memory ------------------------------------------------------------------------
 __device__ __forceinline__ void tmem_alloc(uint32_t smem_result, uint32_t columns)
@@ -147,6 +156,14 @@ __device__ __forceinline__ void tmem_ld_32x32b_x16(uint32_t taddr, uint32_t (&r)
         : "memory");
 }
 __device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
+// The same, with the loaded registers named, so that nothing that reads them can be moved above it.
+__device__ __forceinline__ void tmem_ld_wait(uint32_t (&r)[16])
+{
+    asm volatile("tcgen05.wait::ld.sync.aligned;"
+                 : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]),
+                   "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15])
+                 :: "memory");
+}
 // The store that mirrors tmem_ld_32x32b_x16: thread i of the warp writes 16 consecutive 32-bit
 // columns of row (lane base + i).
 __device__ __forceinline__ void tmem_st_32x32b_x16(uint32_t taddr, const uint32_t (&r)[16])
@@ -319,6 +336,20 @@ __device__ __forceinline__ void mma_bf16_ss_guarded(uint32_t d_tmem, uint64_t a_
         "setp.ne.b32 g, %5, 0;\n\t"
         "@g tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
         ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate), "r"(issue)
+        : "memory");
+}
+// (both descriptors as their two halves, so that a caller steps the start addresses with 32-bit adds)
+__device__ __forceinline__ void mma_bf16_ss_guarded(uint32_t d_tmem, uint32_t a_lo, uint32_t a_hi, uint32_t b_lo, uint32_t b_hi,
+                                                    uint32_t idesc, uint32_t accumulate, uint32_t issue)
+{
+    asm volatile(
+        "{\n\t.reg .pred p, g;\n\t.reg .b64 ad, bd;\n\t"
+        "mov.b64 ad, {%1, %2};\n\t"
+        "mov.b64 bd, {%3, %4};\n\t"
+        "setp.ne.b32 p, %6, 0;\n\t"
+        "setp.ne.b32 g, %7, 0;\n\t"
+        "@g tcgen05.mma.cta_group::1.kind::f16 [%0], ad, bd, %5, p;\n\t}"
+        ::"r"(d_tmem), "r"(a_lo), "r"(a_hi), "r"(b_lo), "r"(b_hi), "r"(idesc), "r"(accumulate), "r"(issue)
         : "memory");
 }
 __device__ __forceinline__ void mma_commit_guarded(uint32_t bar, uint32_t issue)

@@ -136,6 +136,22 @@ tc_status finish_model(tc_model *m)
     // x_hat = step * sum_j T[j][c] (q_j - center) + mu_c + (lo + center*step) * sum_j T[j][c]
     const double top = (double)((1 << m->bits) - 1);
     m->center = (int)std::min(top, std::max(0.0, std::nearbyint(-m->lo / m->step)));
+    // What to expect of the symbols, coefficient j taken as Gaussian with the variance eig[j] (without
+    // eigenvalues: as dense): the share that is not the zero level, 1 - p0, and the code length with
+    // one bit for the zero level and 2.5 + log2(1 + 2 sigma / step) for the others -- 1.0 to 1.25
+    // times what the fitted layers' codes take.
+    m->blk_bits.assign((size_t)(k + 15) / 16, 0.f);
+    m->blk_odd.assign((size_t)(k + 15) / 16, 0.f);
+    for (int j = 0; j < k; ++j) {
+        double bits = m->bits + 0.5, odd = 1.0;
+        if (!m->eig.empty()) {
+            const double sigma = std::sqrt(std::max(0.0, m->eig[j])) / m->step;
+            odd = 1.0 - std::erf(0.5 / (std::sqrt(2.0) * sigma + 1e-30));
+            bits = std::min(12.0, 1.0 + odd * (1.5 + std::log2(1.0 + 2.0 * sigma)));
+        }
+        m->blk_bits[j / 16] += (float)bits;
+        m->blk_odd[j / 16] += (float)odd;
+    }
     tc_status st;
     if (!m->d_basis64 && (st = upload(&m->d_basis64, m->basis)) != TC_OK) return st;
     if (!m->d_mean64 && (st = upload(&m->d_mean64, m->mean)) != TC_OK) return st;
@@ -798,6 +814,8 @@ tc_status tc_encode_with_scratch(tc_ctx *ctx, const tc_model *m, const tc_codebo
     a.basis_bf16 = m->d_basis_bf16; a.enc_bias = m->d_enc_bias; a.tmu32 = m->d_tmu32;
     a.basis_map = m->has_basis_map ? &m->basis_map : nullptr;
     a.hist = hist; a.hist_modal = m->center;
+    a.modal = cb->modal;
+    a.blk_bits = m->blk_bits.data(); a.blk_odd = m->blk_odd.data();
     if (hist && !((ctx->force_exact == 0 || ctx->force_exact == 3) && x->dtype == TC_BF16 && tc_encode_tc_supported(ctx, a)))
         return TC_ERR_UNSUPPORTED;                      // only the resident-basis tensor-core encoder counts symbols
     if ((ctx->force_exact == 0 || ctx->force_exact == 3) && x->dtype == TC_BF16 && tc_encode_tc_supported(ctx, a)) {

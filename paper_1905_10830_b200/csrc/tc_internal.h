@@ -56,6 +56,7 @@ struct tc_model {
     // from d_basis64 the first time the host needs it (export, folding)
     mutable std::vector<double> basis;      // [c][c], or empty
     std::vector<double> mean, eig;          // [c]
+    std::vector<float> blk_bits, blk_odd;   // [(k + 15) / 16]  see finish_model
     int device = 0;
     // device copies
     double *d_basis64 = nullptr;            // [c][c] exact values of the (rounded) basis
@@ -116,6 +117,8 @@ struct EncodeArgs {
     uint8_t *sym_park;                // streaming encoder: non-null = leave the symbols [P][K] here and stop (the entropy coder runs as a kernel of its own)
     unsigned long long *hist;         // tensor-core encoder, statistics: non-null = per-coefficient counts [K][2^bits] of every symbol but hist_modal are added here
     int hist_modal;                   // the symbol of the zero level, which most coefficients hold: statistics mode counts all the others
+    int modal;                        // per-layer table: the symbol whose code is the single bit 0, or -1 if no code has one bit
+    const float *blk_bits, *blk_odd;  // HOST, per block of 16 coefficients: expected code bits, expected number of symbols that are not the zero level
 };
 
 struct DecodeArgs {
