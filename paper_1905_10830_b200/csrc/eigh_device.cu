@@ -425,8 +425,10 @@ __global__ void model_consts_kernel(const double *basis, const double *mean, int
     }
 }
 
-// bf16 operand copies: b[j][a] and its transpose bt[a][j] (an 8-bit basis as its integers)
-__global__ void basis_bf16_kernel(const double *basis, int c, int k, double scale_or_zero, __nv_bfloat16 *b, __nv_bfloat16 *bt)
+// bf16 operand copies: b[j][a], its transpose bt[a][j] and, unless null, bc: b in core matrices of 8 x 8
+// elements (128 contiguous bytes), those of the same eight rows side by side (an 8-bit basis as its integers)
+__global__ void basis_bf16_kernel(const double *basis, int c, int k, double scale_or_zero, __nv_bfloat16 *b, __nv_bfloat16 *bt,
+                                  __nv_bfloat16 *bc)
 {
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= (long long)k * c) return;
@@ -436,6 +438,7 @@ __global__ void basis_bf16_kernel(const double *basis, int c, int k, double scal
     const __nv_bfloat16 h = __float2bfloat16(f);
     b[i] = h;
     bt[(size_t)a * k + j] = h;
+    if (bc) bc[((size_t)(j >> 3) * (c >> 3) + (a >> 3)) * 64 + (j & 7) * 8 + (a & 7)] = h;
 }
 
 }  // namespace
@@ -530,10 +533,12 @@ tc_status tc_launch_model_consts(const double *basis, const double *mean, int c,
     return cudaGetLastError() == cudaSuccess ? TC_OK : TC_ERR_CUDA;
 }
 
-tc_status tc_launch_basis_bf16(const double *basis, int c, int k, double basis_scale, bool int8, void *b, void *bt, cudaStream_t s)
+tc_status tc_launch_basis_bf16(const double *basis, int c, int k, double basis_scale, bool int8, void *b, void *bt, void *bc,
+                               cudaStream_t s)
 {
     const long long n = (long long)k * c;
     basis_bf16_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(basis, c, k, int8 ? basis_scale : 0.0,
-                                                                 static_cast<__nv_bfloat16 *>(b), static_cast<__nv_bfloat16 *>(bt));
+                                                                 static_cast<__nv_bfloat16 *>(b), static_cast<__nv_bfloat16 *>(bt),
+                                                                 static_cast<__nv_bfloat16 *>(bc));
     return cudaGetLastError() == cudaSuccess ? TC_OK : TC_ERR_CUDA;
 }

@@ -260,6 +260,13 @@ __device__ __forceinline__ void tma_load_2d(uint32_t smem_dst, const void *tenso
         : "memory");
 }
 
+// Contiguous bulk copy global -> shared: both addresses 16-byte aligned, the size a multiple of 16.
+__device__ __forceinline__ void bulk_load(uint32_t smem_dst, const void *src, uint32_t bytes, uint32_t bar)
+{
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+                 ::"r"(smem_dst), "l"(src), "r"(bytes), "r"(bar) : "memory");
+}
+
 // Instruction descriptor for kind::f16 with bf16 operands and fp32 accumulation.
 __device__ __forceinline__ uint32_t make_idesc_bf16(int m, int n, bool a_mn_major, bool b_mn_major)
 {

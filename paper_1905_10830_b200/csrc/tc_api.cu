@@ -165,8 +165,10 @@ tc_status finish_model(tc_model *m)
         // folded into their quantiser and dequantiser constants
         TC_CUDA(cudaMalloc((void **)&m->d_basis_bf16, sizeof(__nv_bfloat16) * (size_t)k * c));
         TC_CUDA(cudaMalloc((void **)&m->d_basis_t_bf16, sizeof(__nv_bfloat16) * (size_t)k * c));
+        if (c <= 256 && c % 16 == 0 && k % 16 == 0)
+            TC_CUDA(cudaMalloc((void **)&m->d_basis_core, sizeof(__nv_bfloat16) * (size_t)k * c));
         if ((st = tc_launch_basis_bf16(m->d_basis64, c, k, m->basis_scale, m->basis_dtype == TC_INT8, m->d_basis_bf16,
-                                       m->d_basis_t_bf16, nullptr)) != TC_OK) return st;
+                                       m->d_basis_t_bf16, m->d_basis_core, nullptr)) != TC_OK) return st;
         // Tensor map for the kernels that stream the basis: boxes of 256 coefficient rows x 32
         // channels (64 bytes), written with the 64-byte swizzle the MMA descriptor names.  Needs
         // rows of a multiple of 16 bytes; without a map those kernels copy the basis with cp.async.
@@ -419,7 +421,7 @@ void tc_model_free(tc_model *m)
     if (!m) return;
     DeviceGuard guard(m->device);
     cudaFree(m->d_basis64); cudaFree(m->d_mean64); cudaFree(m->d_basis_bf16);
-    cudaFree(m->d_basis_t_bf16); cudaFree(m->d_enc_bias); cudaFree(m->d_dec_bias); cudaFree(m->d_tmu32);
+    cudaFree(m->d_basis_core); cudaFree(m->d_basis_t_bf16); cudaFree(m->d_enc_bias); cudaFree(m->d_dec_bias); cudaFree(m->d_tmu32);
     delete m;
 }
 
@@ -811,7 +813,7 @@ tc_status tc_encode_with_scratch(tc_ctx *ctx, const tc_model *m, const tc_codebo
     a.ticket = (unsigned int *)scratch;
     a.tile_state = (unsigned long long *)((char *)scratch + kEncodeScratchHeader);
     a.status = ctx->d_status; a.clamped = clamped; a.emit = 1;
-    a.basis_bf16 = m->d_basis_bf16; a.enc_bias = m->d_enc_bias; a.tmu32 = m->d_tmu32;
+    a.basis_bf16 = m->d_basis_bf16; a.basis_core = m->d_basis_core; a.enc_bias = m->d_enc_bias; a.tmu32 = m->d_tmu32;
     a.basis_map = m->has_basis_map ? &m->basis_map : nullptr;
     a.hist = hist; a.hist_modal = m->center;
     a.modal = cb->modal;

@@ -62,6 +62,7 @@ struct tc_model {
     double *d_basis64 = nullptr;            // [c][c] exact values of the (rounded) basis
     double *d_mean64 = nullptr;             // [c]
     __nv_bfloat16 *d_basis_bf16 = nullptr;  // [k][c]   bf16 basis, or the integers of an 8-bit basis (exact in bf16)
+    __nv_bfloat16 *d_basis_core = nullptr;  // the same in the MMA's shared-memory order (8 x 8 core matrices); layers of up to 256 channels
     __nv_bfloat16 *d_basis_t_bf16 = nullptr;// [c][k]   transpose, for the inverse projection
     float *d_enc_bias = nullptr;            // [k]  -(T mu + lo)_j / step
     float *d_dec_bias = nullptr;            // [c]  mu_c + (lo + center*step) * sum_j T[j][c]
@@ -96,6 +97,7 @@ struct EncodeArgs {
     const double *basis64;      // [c][c]
     const double *mean64;       // [c]
     const __nv_bfloat16 *basis_bf16;   // [k][c]  (tensor-core path)
+    const __nv_bfloat16 *basis_core;   // basis_bf16 in 8 x 8 core matrices, or null
     const CUtensorMap *basis_map;      // HOST pointer to the model's tensor map of basis_bf16, or null
     const float *enc_bias;      // [k]  -(T mu + lo)_j / step
     const float *tmu32;         // [k]  (T mu)_j
@@ -216,4 +218,4 @@ tc_status tc_eigh_device(const double *a, int c, double *evals, double *evecs, v
 tc_status tc_launch_round_basis(double *basis, int c, int dtype, double *scale_slot, cudaStream_t s);
 tc_status tc_launch_model_consts(const double *basis, const double *mean, int c, int k, double lo, double step, double center,
                                  float *enc_bias, float *tmu32, float *dec_bias, cudaStream_t s);
-tc_status tc_launch_basis_bf16(const double *basis, int c, int k, double basis_scale, bool int8, void *b, void *bt, cudaStream_t s);
+tc_status tc_launch_basis_bf16(const double *basis, int c, int k, double basis_scale, bool int8, void *b, void *bt, void *bc, cudaStream_t s);
