@@ -59,15 +59,12 @@ double round_to_dtype(double v, int dtype)
     return std::ldexp(std::nearbyint(std::ldexp(f, shift)), e - shift);
 }
 
-template <typename T>
-tc_status upload(T **dst, const std::vector<T> &src)
-{
-    *dst = nullptr;
-    if (src.empty()) return TC_OK;
-    TC_CUDA(cudaMalloc((void **)dst, src.size() * sizeof(T)));
-    TC_CUDA(cudaMemcpy(*dst, src.data(), src.size() * sizeof(T), cudaMemcpyHostToDevice));
-    return TC_OK;
-}
+// Lays several device arrays out in one allocation (an allocation costs tens of microseconds next to a
+// busy device, and a model or code table is several small arrays).
+struct Layout {
+    size_t bytes = 0;
+    size_t add(size_t n) { const size_t at = bytes; bytes += (n + 255) & ~(size_t)255; return at; }
+};
 
 bool valid_tensor(const tc_tensor *t)
 {
@@ -153,20 +150,34 @@ tc_status finish_model(tc_model *m)
         m->blk_odd[j / 16] += (float)odd;
     }
     tc_status st;
-    if (!m->d_basis64 && (st = upload(&m->d_basis64, m->basis)) != TC_OK) return st;
-    if (!m->d_mean64 && (st = upload(&m->d_mean64, m->mean)) != TC_OK) return st;
-    TC_CUDA(cudaMalloc((void **)&m->d_enc_bias, sizeof(float) * k));
-    TC_CUDA(cudaMalloc((void **)&m->d_tmu32, sizeof(float) * k));
-    TC_CUDA(cudaMalloc((void **)&m->d_dec_bias, sizeof(float) * c));
+    const bool bf16 = m->basis_dtype == TC_BF16 || m->basis_dtype == TC_INT8, imported = !m->d_basis64;
+    const bool core = bf16 && c <= 256 && c % 16 == 0 && k % 16 == 0;
+    Layout lay;
+    const size_t basis64_at = lay.add(imported ? sizeof(double) * (size_t)c * c : 0), mean64_at = lay.add(imported ? sizeof(double) * c : 0);
+    const size_t enc_bias_at = lay.add(sizeof(float) * k), tmu_at = lay.add(sizeof(float) * k), dec_bias_at = lay.add(sizeof(float) * c);
+    const size_t operand = sizeof(__nv_bfloat16) * (size_t)k * c;
+    const size_t b_at = lay.add(bf16 ? operand : 0), bt_at = lay.add(bf16 ? operand : 0), bc_at = lay.add(core ? operand : 0);
+    char *mem = nullptr;
+    TC_CUDA(cudaMalloc((void **)&mem, lay.bytes));
+    m->d_block = mem;
+    if (imported) {
+        m->d_basis64 = (double *)(mem + basis64_at);
+        m->d_mean64 = (double *)(mem + mean64_at);
+        m->owns64 = false;
+        TC_CUDA(cudaMemcpy(m->d_basis64, m->basis.data(), sizeof(double) * (size_t)c * c, cudaMemcpyHostToDevice));
+        TC_CUDA(cudaMemcpy(m->d_mean64, m->mean.data(), sizeof(double) * c, cudaMemcpyHostToDevice));
+    }
+    m->d_enc_bias = (float *)(mem + enc_bias_at);
+    m->d_tmu32 = (float *)(mem + tmu_at);
+    m->d_dec_bias = (float *)(mem + dec_bias_at);
     if ((st = tc_launch_model_consts(m->d_basis64, m->d_mean64, c, k, m->lo, m->step, (double)m->center, m->d_enc_bias,
                                      m->d_tmu32, m->d_dec_bias, nullptr)) != TC_OK) return st;
-    if (m->basis_dtype == TC_BF16 || m->basis_dtype == TC_INT8) {
+    if (bf16) {
         // an 8-bit basis goes to the bf16 kernels as its integers (exact in bf16); the scale is
         // folded into their quantiser and dequantiser constants
-        TC_CUDA(cudaMalloc((void **)&m->d_basis_bf16, sizeof(__nv_bfloat16) * (size_t)k * c));
-        TC_CUDA(cudaMalloc((void **)&m->d_basis_t_bf16, sizeof(__nv_bfloat16) * (size_t)k * c));
-        if (c <= 256 && c % 16 == 0 && k % 16 == 0)
-            TC_CUDA(cudaMalloc((void **)&m->d_basis_core, sizeof(__nv_bfloat16) * (size_t)k * c));
+        m->d_basis_bf16 = (__nv_bfloat16 *)(mem + b_at);
+        m->d_basis_t_bf16 = (__nv_bfloat16 *)(mem + bt_at);
+        m->d_basis_core = core ? (__nv_bfloat16 *)(mem + bc_at) : nullptr;
         if ((st = tc_launch_basis_bf16(m->d_basis64, c, k, m->basis_scale, m->basis_dtype == TC_INT8, m->d_basis_bf16,
                                        m->d_basis_t_bf16, m->d_basis_core, nullptr)) != TC_OK) return st;
         // Tensor map for the kernels that stream the basis: boxes of 256 coefficient rows x 32
@@ -251,12 +262,25 @@ tc_status finish_codebook(tc_codebook *cb)
             }
         }
     }
-    tc_status st;
-    if ((st = upload(&cb->d_enc, enc)) != TC_OK) return st;
-    if ((st = upload(&cb->d_lut32, lut32)) != TC_OK) return st;
-    if ((st = upload(&cb->d_canon, canon)) != TC_OK) return st;
-    if ((st = upload(&cb->d_sorted, sorted)) != TC_OK) return st;
-    return upload(&cb->d_lut, lut);
+    Layout lay;
+    auto bytes = [](const auto &v) { return v.size() * sizeof(v[0]); };
+    const size_t enc_at = lay.add(bytes(enc)), lut32_at = lay.add(bytes(lut32)), canon_at = lay.add(bytes(canon)), sorted_at = lay.add(bytes(sorted)),
+                 lut_at = lay.add(bytes(lut));
+    std::vector<char> host(lay.bytes);
+    std::memcpy(host.data() + enc_at, enc.data(), bytes(enc));
+    std::memcpy(host.data() + lut32_at, lut32.data(), bytes(lut32));
+    std::memcpy(host.data() + canon_at, canon.data(), bytes(canon));
+    std::memcpy(host.data() + sorted_at, sorted.data(), bytes(sorted));
+    std::memcpy(host.data() + lut_at, lut.data(), bytes(lut));
+    TC_CUDA(cudaMalloc(&cb->d_block, lay.bytes));
+    char *mem = (char *)cb->d_block;
+    TC_CUDA(cudaMemcpy(mem, host.data(), lay.bytes, cudaMemcpyHostToDevice));
+    cb->d_enc = (uint32_t *)(mem + enc_at);
+    cb->d_lut32 = (uint32_t *)(mem + lut32_at);
+    cb->d_canon = (uint32_t *)(mem + canon_at);
+    cb->d_sorted = (uint8_t *)(mem + sorted_at);
+    cb->d_lut = (uint16_t *)(mem + lut_at);
+    return TC_OK;
 }
 
 bool kraft_complete(const uint8_t *len, int nsym, int lmax)
@@ -302,12 +326,17 @@ tc_status tc_create(tc_ctx **out, int device)
     tc_ctx *ctx = new (std::nothrow) tc_ctx();
     if (!ctx) return TC_ERR_CUDA;
     ctx->device = device;
-    cudaDeviceProp prop;
-    if (cudaGetDeviceProperties(&prop, device) != cudaSuccess) { delete ctx; return TC_ERR_CUDA; }
-    ctx->sm_count = prop.multiProcessorCount;
-    ctx->max_smem_optin = (int)prop.sharedMemPerBlockOptin;
-    if (cudaMalloc((void **)&ctx->d_status, 64) != cudaSuccess || cudaMemset(ctx->d_status, 0, 64) != cudaSuccess) {
+    if (cudaDeviceGetAttribute(&ctx->sm_count, cudaDevAttrMultiProcessorCount, device) != cudaSuccess ||
+        cudaDeviceGetAttribute(&ctx->max_smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, device) != cudaSuccess) {
         cudaGetLastError();
+        delete ctx;
+        return TC_ERR_CUDA;
+    }
+    // (the arena at its smallest size, so that a first call does not stop for an allocation)
+    if (cudaMalloc((void **)&ctx->d_status, 64) != cudaSuccess || cudaMemset(ctx->d_status, 0, 64) != cudaSuccess ||
+        ensure_scratch(ctx, 1) != TC_OK) {
+        cudaGetLastError();
+        cudaFree(ctx->d_status);
         delete ctx;
         return TC_ERR_CUDA;
     }
@@ -420,8 +449,8 @@ void tc_model_free(tc_model *m)
 {
     if (!m) return;
     DeviceGuard guard(m->device);
-    cudaFree(m->d_basis64); cudaFree(m->d_mean64); cudaFree(m->d_basis_bf16);
-    cudaFree(m->d_basis_core); cudaFree(m->d_basis_t_bf16); cudaFree(m->d_enc_bias); cudaFree(m->d_dec_bias); cudaFree(m->d_tmu32);
+    if (m->owns64) { cudaFree(m->d_basis64); cudaFree(m->d_mean64); }
+    cudaFree(m->d_block);
     delete m;
 }
 
@@ -776,11 +805,7 @@ void tc_codebook_free(tc_codebook *cb)
 {
     if (!cb) return;
     DeviceGuard guard(cb->device);
-    cudaFree(cb->d_enc);
-    cudaFree(cb->d_lut);
-    cudaFree(cb->d_lut32);
-    cudaFree(cb->d_canon);
-    cudaFree(cb->d_sorted);
+    cudaFree(cb->d_block);
     delete cb;
 }
 

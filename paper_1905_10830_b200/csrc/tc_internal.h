@@ -58,7 +58,9 @@ struct tc_model {
     std::vector<double> mean, eig;          // [c]
     std::vector<float> blk_bits, blk_odd;   // [(k + 15) / 16]  see finish_model
     int device = 0;
-    // device copies
+    // device copies, all but the first two (of a fitted model: owns64) inside one allocation
+    void *d_block = nullptr;
+    bool owns64 = true;
     double *d_basis64 = nullptr;            // [c][c] exact values of the (rounded) basis
     double *d_mean64 = nullptr;             // [c]
     __nv_bfloat16 *d_basis_bf16 = nullptr;  // [k][c]   bf16 basis, or the integers of an 8-bit basis (exact in bf16)
@@ -78,6 +80,7 @@ struct tc_codebook {
     int modal = -1;                         // per-layer table: the symbol coded by the single bit 0 (-1: none)
     std::vector<uint8_t> lengths;           // host [groups][2^bits]
     int device = 0;
+    void *d_block = nullptr;                // one allocation that holds the arrays below
     uint32_t *d_enc = nullptr;              // [groups][2^bits]  (code << 8) | length
     uint16_t *d_lut = nullptr;              // [groups][2^lut_bits]  (symbol << 8) | length
     uint32_t *d_lut32 = nullptr;            // [groups][2^lut_bits]  bf16(symbol) << 16 | symbol << 8 | length
