@@ -10,9 +10,12 @@
 // the decoded symbols are then written into it one by one.
 //
 // One persistent block per SM.  Warp roles:
-//   warps 0-7, 8-15    two VLD groups on alternating tiles of 128 pixels, each with its own operand
-//                      buffer (all K coefficients of the tile, K-major).  One or two threads per
-//                      pixel walk the pixel's chunks.
+//   warps 0-15         VLD groups of as many warps as a tile has chunks for -- eight with two chunks per
+//                      pixel, four with one, two with a chunk of two pixels -- on tiles of 128 pixels in
+//                      turn, each group with its own operand buffer (all K coefficients of the tile,
+//                      K-major).  One or two threads per pixel walk the pixel's chunks.  A group's time
+//                      per tile is the latency of its chunks' symbols, so the groups in flight set the
+//                      rate: with two groups whatever their size 64x56x56 x 64 took 62 us, with eight 24.
 //   warps 16-23        epilogue, all eight warps on every work item: TMEM -> registers,
 //                      x_hat = step * acc + bias, round to bf16, NCHW stores through warp-private
 //                      transpose blocks (the accumulator is held transposed: lane = channel)
@@ -38,7 +41,7 @@ namespace {
 using namespace tcdev;
 using namespace sm100;
 
-constexpr int kGroupWarps = 8, kEpiWarp0 = 2 * kGroupWarps, kMmaWarp = kEpiWarp0 + 8;
+constexpr int kVldWarps = 16, kMaxGroups = 8, kEpiWarp0 = kVldWarps, kMmaWarp = kEpiWarp0 + 8;
 constexpr int kThreads = (kMmaWarp + 2) * 32;                  // two MMA warps, one per accumulator
 constexpr int kTmemCols = 512;
 constexpr int kAccBase = 256, kAccCols = 128;                 // two accumulators behind the basis columns
@@ -50,39 +53,54 @@ constexpr int kDenseBits128 = 224;                            // tiles above 1.7
 // bits, whatever the bits say; the slack after the last buffer keeps those reads inside the
 // block's shared memory even for a corrupt stream (the buffers lie back to back).
 constexpr int kStreamSlack = 1024;
-constexpr int kTrWarpBytes = 1024;                            // epilogue transpose block of one warp: 32 channel rows x 16 pixels
+constexpr int kStaticSmem = 1536;                             // room for the kernel's static shared variables
+constexpr int kTrWarpBytes = 2048;                            // epilogue transpose block of one warp: 32 channel rows x 32 pixels
 // Named barriers.  Hand-overs between warps that both run ordinary instructions use them instead
 // of mbarriers: the waiting side is parked by the hardware, whereas a warp polling an mbarrier
 // keeps issuing and takes issue slots from the warps that work.  (mbarriers remain where the
 // tensor core signals: accumulator ready, operand panel consumed.)
 constexpr int kBarGroup = 1;                                  // + group: the VLD threads of a group, once per tile
-constexpr int kBarFull = 3;                                   // + group: operand complete, VLD threads -> MMA warp
-constexpr int kBarAccFree = 5;                                // + accumulator: drained, epilogue warps -> MMA warp
-constexpr int kBarEpi = 7;                                    // accumulator ready, polling epilogue warp -> the other seven
+constexpr int kBarAccFree = kBarGroup + kMaxGroups;           // + accumulator: drained, epilogue warps -> MMA warp
+constexpr int kBarEpi = kBarAccFree + 2;                      // accumulator ready, polling epilogue warp -> the other seven
 
 struct SmemLayout {
     uint32_t lut, opnd, tbuf, sbuf, total;
     uint32_t opnd_bytes;                                      // one operand buffer (one per VLD group)
     uint32_t stream_buf;                                      // bytes per staged stream buffer (two per group; 0: does not fit)
+    int groups;                                               // VLD groups
 };
 
-__host__ __device__ inline SmemLayout smem_layout(int k, int lut_entries, int budget)
+// group_warps: warps of a VLD group.  As many groups as warps and shared memory allow beside stream
+// buffers for tiles of 2.5 bits per symbol (two groups: for what is left, at least 4 KB).
+inline SmemLayout smem_layout(int k, int lut_entries, int group_warps, int budget)
 {
     SmemLayout l;
     l.lut = 0;                                                // 32-bit entries: bf16(symbol - center) << 16 | length
     l.opnd = ((uint32_t)lut_entries * 4u + 1023u) & ~1023u;
     l.opnd_bytes = (uint32_t)k * TC_TILE_PIXELS * 2;
-    l.tbuf = l.opnd + 2u * l.opnd_bytes;
-    l.sbuf = l.tbuf + 8u * kTrWarpBytes;
+    const int most = kVldWarps / group_warps < kMaxGroups ? kVldWarps / group_warps : kMaxGroups;
+    const uint32_t want_kb = ((uint32_t)k * 40u + 1023u) / 1024u;
     l.stream_buf = 0;
     l.total = 0;
-    for (uint32_t kb = 16; kb >= 4; --kb)
-        if ((long long)l.sbuf + 4ll * kb * 1024 + kStreamSlack <= (long long)budget) {
-            l.stream_buf = kb * 1024;
-            l.total = l.sbuf + 4u * l.stream_buf + kStreamSlack;
-            break;
-        }
+    for (l.groups = most; l.groups >= 2; --l.groups) {
+        l.tbuf = l.opnd + (uint32_t)l.groups * l.opnd_bytes;
+        l.sbuf = l.tbuf + 8u * kTrWarpBytes;
+        const long long left = (long long)budget - l.sbuf - kStreamSlack;
+        long long kb = left / (2ll * l.groups * 1024);
+        if (kb > 16) kb = 16;
+        if (kb < 4 || (kb < (long long)want_kb && l.groups > 2)) continue;
+        l.stream_buf = (uint32_t)kb * 1024u;
+        l.total = l.sbuf + 2u * (uint32_t)l.groups * l.stream_buf + kStreamSlack;
+        break;
+    }
+    if (l.groups < 2) l.groups = 2;
     return l;
+}
+
+// Threads of a VLD group: one per chunk, or two per pixel with more than one chunk per pixel.
+__host__ __device__ inline int group_work(int splits, int chunk_pixels)
+{
+    return chunk_pixels > 1 ? TC_TILE_PIXELS / chunk_pixels : TC_TILE_PIXELS * (splits >= 2 ? 2 : 1);
 }
 
 __device__ __forceinline__ uint32_t lds_u32(uint32_t addr)
@@ -184,36 +202,36 @@ struct BitReader {
 };
 
 template <bool kRelu>
-__global__ void __launch_bounds__(kThreads, 1) decode_runs_kernel(DecodeArgs a)
+__global__ void __launch_bounds__(kThreads, 1) decode_runs_kernel(DecodeArgs a, SmemLayout L)
 {
     extern __shared__ __align__(128) unsigned char smem[];
-    __shared__ __align__(8) unsigned long long s_empty[2][kMaxPanels], s_tfull[2];
+    __shared__ __align__(8) unsigned long long s_empty[kMaxGroups][kMaxPanels], s_bfull[kMaxGroups], s_tfull[2];
     __shared__ uint32_t s_tmem_base;
     // [group][tile parity][thread set][warp]: bits per warp, for the start positions.  Two copies: a warp
     // that is done with its tile early writes the next tile's sum while a slower warp may still
     // be reading this tile's; the group's barrier (one per tile) only orders the write after next.
-    __shared__ unsigned int s_wsum[2][2][2][4];
+    __shared__ unsigned int s_wsum[kMaxGroups][2][2][4];
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int lut_size = 1 << a.lut_bits;
-    const SmemLayout L = smem_layout(a.k, lut_size, a.smem_budget);
-    constexpr int nbuf = 2;
+    const int S = a.splits, cp = a.chunk_pixels;
+    const int tpp = S >= 2 ? 2 : 1;                            // threads per pixel
+    const int chunks_per_thread = S / tpp;                     // 1, or 2 with four chunks per pixel
+    const int n_work = group_work(S, cp);                      // threads of a group that own chunks
+    const int group_warps = (n_work + 31) / 32, n_thr = group_warps * 32;     // whole warps take part in the group's barriers
+    const int G = L.groups;
     const uint32_t lut_addr = smem_u32(smem + L.lut);
     const uint32_t opnd_addr = smem_u32(smem + L.opnd);
     const int n_blocks = (a.c + 127) / 128;                    // blocks of 128 channels
     const int items = n_blocks;                                // work items per tile: halves of 64 pixels with two channel blocks
-    const int S = a.splits, cp = a.chunk_pixels;
-    const int tpp = S >= 2 ? 2 : 1;                            // threads per pixel
-    const int chunks_per_thread = S / tpp;                     // 1, or 2 with four chunks per pixel
-    const int n_work = cp > 1 ? TC_TILE_PIXELS / cp : TC_TILE_PIXELS * tpp;   // threads of a group that own chunks
-    const int n_thr = ((n_work + 31) / 32) * 32;               // whole warps take part in the group's barriers
 
     // ---- set-up ---------------------------------------------------------------------
     if (tid == 0) {
-        for (int g = 0; g < 2; ++g) {
+        for (int g = 0; g < G; ++g) {
             for (int p = 0; p < kMaxPanels; ++p) mbar_init(smem_u32(&s_empty[g][p]), (uint32_t)items);   // one commit per item of the tile
-            mbar_init(smem_u32(&s_tfull[g]), 1);
+            mbar_init(smem_u32(&s_bfull[g]), (uint32_t)group_warps);                                     // operand complete: one arrival per warp
         }
+        for (int w = 0; w < 2; ++w) mbar_init(smem_u32(&s_tfull[w]), 1);
         mbar_fence_init();
     }
     if (warp == kMmaWarp) { tmem_alloc(smem_u32(&s_tmem_base), kTmemCols); tmem_relinquish(); }
@@ -271,9 +289,9 @@ __global__ void __launch_bounds__(kThreads, 1) decode_runs_kernel(DecodeArgs a)
 
     if (warp < kEpiWarp0) {
         // ================= VLD groups =================
-        const int grp = warp >> 3;
-        const int tg = tid & 255;                // thread within the group
-        if (tg < n_thr) {
+        const int grp = warp / group_warps;
+        const int tg = tid - grp * n_thr;        // thread within the group
+        if (grp < G) {
             const int set = cp > 1 ? 0 : tg >> 7;    // which thread of the pixel (warp-uniform)
             const int t = cp > 1 ? tg : (tg & 127);  // pixel within the tile, or chunk within the tile (cp > 1)
             const int wq = (t >> 5) & 3;
@@ -327,12 +345,12 @@ __global__ void __launch_bounds__(kThreads, 1) decode_runs_kernel(DecodeArgs a)
                 cp_async_commit();
             };
 
-            TileInfo cur = tile_info(grp), nxt = tile_info(grp + nbuf);
+            TileInfo cur = tile_info(grp), nxt = tile_info(grp + G);
             stage_tile(cur, 0);
             int li = 0;
             // (a thread whose wait ran out keeps walking the tiles without decoding: the group's
             // barriers and the hand-over to the MMA thread need every thread's arrival)
-            for (long long tl = grp; tl < my_tiles; tl += nbuf, ++li) {
+            for (long long tl = grp; tl < my_tiles; tl += G, ++li) {
                 const long long tile = blockIdx.x + tl * gridDim.x;
                 // start of every chunk = sum of the lengths before it in the tile (chunk order: pixel,
                 // then part of the pixel): scan over the pixels' totals
@@ -350,7 +368,7 @@ __global__ void __launch_bounds__(kThreads, 1) decode_runs_kernel(DecodeArgs a)
                 // with the tile before: its stream buffer may take the next tile's segment
                 named_bar_sync(bar_id, n_thr);
                 stage_tile(nxt, (li + 1) & 1);
-                const TileInfo after = tile_info(tl + 2 * nbuf);   // offsets two tiles ahead: their latency hides behind the decode
+                const TileInfo after = tile_info(tl + 2 * G);   // offsets two tiles ahead: their latency hides behind the decode
                 unsigned int before = 0, tile_total = 0;
                 const int n_wq = (n_work / tpp + 31) / 32;          // warps of one thread set
 #pragma unroll
@@ -461,7 +479,8 @@ __global__ void __launch_bounds__(kThreads, 1) decode_runs_kernel(DecodeArgs a)
                     decode_tile(r);
                 }
                 // (the issuing thread makes the operand visible to the tensor core's proxy)
-                named_bar_arrive(kBarFull + grp, n_thr + 32 * items);
+                __syncwarp();
+                if (lane == 0) mbar_arrive(smem_u32(&s_bfull[grp]));
                 if (bad) tc_dev_set_status(a.status, TC_ERR_CORRUPT_STREAM);
                 cur = nxt;
                 nxt = after;
@@ -490,13 +509,16 @@ __global__ void __launch_bounds__(kThreads, 1) decode_runs_kernel(DecodeArgs a)
         const bool vec = (a.hw & 3) == 0 && ((uintptr_t)a.xhat & 7u) == 0;
         const long long img_stride = (long long)a.c * a.hw;
         const int ch_base = blk * 128 + wq * 32;            // first channel of this warp
-        // transpose block: row = channel (32 bytes = 16 pixels); the two 16-byte halves of a row are
-        // swapped in rows 4-7, 12-15, ... so that neither the row writes nor the reads below collide
+        // Transpose block: row = channel (64 bytes = 32 pixels); the four 16-byte pieces of a row are exchanged
+        // by XOR with (row / 2) % 4, so that neither the row writes nor the reads below collide.
         const uint32_t tb = smem_u32(smem + L.tbuf) + (uint32_t)(warp - kEpiWarp0) * kTrWarpBytes;
-        const uint32_t sw_wr = (uint32_t)((lane >> 2) & 1);
-        const uint32_t tb_wr = tb + (uint32_t)lane * 32u;
-        const int r_sub = lane >> 2, piece = lane & 3;      // read phase: channel row r_sub (+ 8, 16, 24), pixels 4 * piece ...
-        const uint32_t tb_rd = tb + (uint32_t)r_sub * 32u + ((((uint32_t)piece >> 1) ^ ((uint32_t)(r_sub >> 2) & 1u)) << 4) + ((uint32_t)piece & 1u) * 8u;
+        const uint32_t tb_wr = tb + (uint32_t)lane * 64u, sw_wr = (uint32_t)((lane >> 1) & 3);
+        // Read phase: rows leave 8 pixels a lane (eight rows an instruction) where every group of 8 pixels is
+        // 16-byte aligned and inside one image, else 4 pixels a lane (four rows an instruction).
+        const bool vec8 = (a.hw & 7) == 0 && ((uintptr_t)a.xhat & 15u) == 0;
+        const int px_lane = vec8 ? 8 * (lane & 3) : 4 * (lane & 7);         // first pixel of this lane in a pass
+        const int r_sub = vec8 ? lane >> 2 : lane >> 3, r_step = vec8 ? 8 : 4;
+        const uint32_t tb_rd0 = tb + (uint32_t)r_sub * 64u, piece = (uint32_t)(px_lane >> 3), in_piece = (uint32_t)(px_lane & 7) * 2u;
         // two accumulator values -> two bf16: x_hat = step * acc + bias (one packed fused multiply-add)
         auto convert = [&](uint32_t x0, uint32_t x1) {
             float f0, f1;
@@ -511,14 +533,18 @@ __global__ void __launch_bounds__(kThreads, 1) decode_runs_kernel(DecodeArgs a)
             const __nv_bfloat162 h = __floats2bfloat162_rn(f0, f1);
             return *reinterpret_cast<const uint32_t *>(&h);
         };
-        // the four channel rows this lane stores in the read phase of a pass: offsets inside an image
-        int row_off[4];
-        bool row_ok[4];
-#pragma unroll
-        for (int it = 0; it < 4; ++it) {
-            row_ok[it] = ch_base + 8 * it + r_sub < a.c;
-            row_off[it] = (ch_base + 8 * it + r_sub) * a.hw;
-        }
+        // Position of this lane's pixels: image and offset inside it of the block's first tile, moved on from
+        // tile to tile by a constant number of pixels (a division of 64-bit numbers per item was a fifth of
+        // the epilogue's instructions).
+        const long long tile_step = (long long)gridDim.x * TC_TILE_PIXELS;
+        const long long img_step = tile_step / a.hw;
+        const int sp_step = (int)(tile_step - img_step * a.hw);
+        const long long first_px = (long long)blockIdx.x * TC_TILE_PIXELS + col_first + px_lane;
+        long long tile_img = first_px / a.hw;
+        int tile_sp = (int)(first_px - tile_img * a.hw);
+        const int rows_left = min(32, a.c - ch_base) - r_sub;               // rows r_sub + k r_step below it exist
+        __nv_bfloat16 *const out_row = out + (long long)(ch_base + r_sub) * a.hw;
+        const uint32_t row_stride = (uint32_t)(r_step * a.hw);              // elements between the rows of two instructions
         bool alive = true;
         const long long n_items = my_tiles * items;
         // (after a wait that ran out the warps keep walking the items: the MMA warp waits for their arrivals)
@@ -539,28 +565,50 @@ __global__ void __launch_bounds__(kThreads, 1) decode_runs_kernel(DecodeArgs a)
             tc_fence_after_sync();
             const uint32_t trow = tmem_base + kAccBase + acc * kAccCols + (n_blocks == 2 ? blk * 64 : 0) + ((uint32_t)(wq * 32) << 16) + col_first;
             if (vec) {
-                // position of this lane's pixel group (4 pixels) in the first pass
-                const long long pg = p_first + 4 * piece;
-                long long img = pg < a.pixels ? pg / a.hw : 0;
-                int sp = pg < a.pixels ? (int)(pg - img * a.hw) : 0;
-                for (int c0 = 0; c0 < col_count; c0 += 16) {
-                    uint32_t r[16];
-                    tmem_ld_32x32b_x16(trow + c0, r);
-                    tmem_ld_wait();
-                    sts_v4(tb_wr + (sw_wr << 4), convert(r[0], r[1]), convert(r[2], r[3]), convert(r[4], r[5]), convert(r[6], r[7]));
-                    sts_v4(tb_wr + ((sw_wr ^ 1u) << 4), convert(r[8], r[9]), convert(r[10], r[11]), convert(r[12], r[13]), convert(r[14], r[15]));
-                    __syncwarp();
-                    const bool px_ok = c0 + 4 * piece < n_valid;
-                    __nv_bfloat16 *px_ptr = out + img * img_stride + sp;
+                long long img = tile_img;
+                int sp = tile_sp + item * 64;
+                while (sp >= a.hw) { sp -= a.hw; ++img; }
+#pragma unroll 1
+                for (int c0 = 0; c0 < col_count; c0 += 32) {
+                    uint32_t r[32];
+                    tmem_ld_32x32b_x32(trow + c0, r);
+                    tmem_ld_wait(r);
 #pragma unroll
-                    for (int it = 0; it < 4; ++it) {
-                        uint32_t lo2, hi2;
-                        asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(lo2), "=r"(hi2) : "r"(tb_rd + it * 256));
-                        if (px_ok && row_ok[it]) *reinterpret_cast<uint2 *>(px_ptr + row_off[it]) = make_uint2(lo2, hi2);
+                    for (int q = 0; q < 4; ++q)
+                        sts_v4(tb_wr + (((uint32_t)q ^ sw_wr) << 4), convert(r[8 * q], r[8 * q + 1]), convert(r[8 * q + 2], r[8 * q + 3]),
+                               convert(r[8 * q + 4], r[8 * q + 5]), convert(r[8 * q + 6], r[8 * q + 7]));
+                    __syncwarp();
+                    const int rows = c0 + px_lane < n_valid ? rows_left : 0;
+                    __nv_bfloat16 *dst = out_row + img * img_stride + sp;
+                    if (vec8) {
+#pragma unroll
+                        for (int k = 0; k < 4; ++k) {
+                            uint32_t v[4];
+                            const uint32_t row = (uint32_t)(r_sub + 8 * k);
+                            asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3])
+                                         : "r"(tb_rd0 + k * 512u + ((piece ^ ((row >> 1) & 3u)) << 4)));
+                            if (8 * k < rows) *reinterpret_cast<uint4 *>(dst) = make_uint4(v[0], v[1], v[2], v[3]);
+                            dst += row_stride;
+                        }
+                    } else {
+#pragma unroll
+                        for (int k = 0; k < 8; ++k) {
+                            uint32_t lo2, hi2;
+                            const uint32_t row = (uint32_t)(r_sub + 4 * k);
+                            asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(lo2), "=r"(hi2)
+                                         : "r"(tb_rd0 + k * 256u + ((piece ^ ((row >> 1) & 3u)) << 4) + in_piece));
+                            if (4 * k < rows) *reinterpret_cast<uint2 *>(dst) = make_uint2(lo2, hi2);
+                            dst += row_stride;
+                        }
                     }
-                    sp += 16;
+                    sp += 32;
                     while (sp >= a.hw) { sp -= a.hw; ++img; }
                     __syncwarp();                                   // the block may be overwritten
+                }
+                if (items == 1 || item == 1) {
+                    tile_img += img_step;
+                    tile_sp += sp_step;
+                    if (tile_sp >= a.hw) { tile_sp -= a.hw; ++tile_img; }
                 }
             } else {
                 // position of the first pixel; from there on it moves incrementally
@@ -604,11 +652,14 @@ __global__ void __launch_bounds__(kThreads, 1) decode_runs_kernel(DecodeArgs a)
         const uint32_t a_blk1 = (uint32_t)(a.k / 2);               // columns between the two channel blocks of the basis
         const int n_k16 = a.k >> 4;
         const uint32_t d_tmem = tmem_base + kAccBase + w * kAccCols;
+        int buf = items == 2 ? 0 : w % G;                         // operand buffer (VLD group) of the tile, and the parity of its turn
+        uint32_t turn = items == 2 ? 0u : (uint32_t)(w / G) & 1u;
+        bool alive = true;
         for (long long tl = items == 2 ? 0 : w; tl < my_tiles; tl += items == 2 ? 1 : 2) {
-            const int buf = (int)(tl & 1);
             const long long it = items == 2 ? 2 * tl + w : tl;       // index of the work item: item it uses accumulator it % 2 = w
+            // (after a wait that ran out the warp keeps walking the items: the epilogue waits for its commits)
+            if (alive) alive = mbar_wait(smem_u32(&s_bfull[buf]), turn);     // the group's VLD threads have arrived
             __syncwarp();
-            named_bar_sync(kBarFull + buf, n_thr + 32 * items);       // the group's VLD threads have arrived
             // the operand was written with ordinary stores by threads that have arrived on the
             // barrier: one proxy fence here, between that synchronisation and the MMA's
             // operand reads, orders them for all writers
@@ -631,7 +682,10 @@ __global__ void __launch_bounds__(kThreads, 1) decode_runs_kernel(DecodeArgs a)
                 a_col += 8;
             }
             mma_commit_guarded(smem_u32(&s_tfull[w]), issuer);
+            buf += items == 2 ? 1 : 2;
+            if (buf >= G) { buf -= G; turn ^= 1u; }
         }
+        if (!alive && issuer) tc_dev_set_status(a.status, TC_ERR_TIMEOUT);
     }
 
     // ---- teardown ---------------------------------------------------------------------
@@ -645,6 +699,11 @@ __global__ void __launch_bounds__(kThreads, 1) decode_runs_kernel(DecodeArgs a)
 
 }  // namespace
 
+static SmemLayout runs_layout(const tc_ctx *ctx, const DecodeArgs &a)
+{
+    return smem_layout(a.k, 1 << a.lut_bits, (group_work(a.splits, a.chunk_pixels) + 31) / 32, ctx->max_smem_optin - kStaticSmem);
+}
+
 bool tc_decode_runs_supported(const tc_ctx *ctx, const DecodeArgs &a)
 {
     // K <= C leading components (PCA truncation): K is the reduction dimension of the MMA
@@ -653,27 +712,25 @@ bool tc_decode_runs_supported(const tc_ctx *ctx, const DecodeArgs &a)
     if (a.lut_bits > TC_MAX_CODE_LEN) return false;
     if (a.chunk_pixels > 1 ? a.splits != 1 : (a.splits != 1 && a.splits != 2 && a.splits != 4)) return false;
     if (a.splits > 1 && (a.k % a.splits != 0 || (a.k / a.splits) % 8 != 0)) return false;
-    return smem_layout(a.k, 1 << a.lut_bits, ctx->max_smem_optin - 512).stream_buf > 0;
+    return runs_layout(ctx, a).stream_buf > 0;
 }
 
 // Bytes of a tile's stream segment this kernel stages in shared memory; longer segments are read
 // from global memory, word by word.
 size_t tc_decode_runs_staging_bytes(const tc_ctx *ctx, const DecodeArgs &a)
 {
-    return smem_layout(a.k, 1 << a.lut_bits, ctx->max_smem_optin - 512).stream_buf;
+    return runs_layout(ctx, a).stream_buf;
 }
 
 tc_status tc_launch_decode_runs(const tc_ctx *ctx, const DecodeArgs &a, cudaStream_t s)
 {
     if (a.n_tiles <= 0) return TC_OK;
-    const SmemLayout l = smem_layout(a.k, 1 << a.lut_bits, ctx->max_smem_optin - 512);
+    const SmemLayout l = runs_layout(ctx, a);
     if (l.stream_buf == 0) return TC_ERR_UNSUPPORTED;
-    void (*kernel)(DecodeArgs) = a.relu ? decode_runs_kernel<true> : decode_runs_kernel<false>;
-    DecodeArgs args = a;
-    args.smem_budget = ctx->max_smem_optin - 512;
+    void (*kernel)(DecodeArgs, SmemLayout) = a.relu ? decode_runs_kernel<true> : decode_runs_kernel<false>;
     if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)l.total) != cudaSuccess)
         return TC_ERR_CUDA;
     const unsigned int grid = (unsigned int)((a.n_tiles < ctx->sm_count) ? a.n_tiles : ctx->sm_count);
-    kernel<<<grid, kThreads, l.total, s>>>(args);
+    kernel<<<grid, kThreads, l.total, s>>>(a, l);
     return cudaGetLastError() == cudaSuccess ? TC_OK : TC_ERR_CUDA;
 }

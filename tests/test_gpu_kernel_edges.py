@@ -109,3 +109,29 @@ def test_per_channel_codes_from_bounds(ctx, c, k, s, n, bits, dtype, cp, splits,
     finally:
         tc.tc_force_exact_path(ctx, 0)
     m.close(); cb.close()
+
+
+# Run-skipping decoder: one to eight warps per group, two to eight groups per block, every group with
+# several tiles (more than eight tiles a block), rows that allow 16-byte stores and rows that do not;
+# against the fp64 kernels on the same stream.
+@pytest.mark.parametrize("c,k,h,w,bits", [(16, 16, 56, 56, 4), (32, 32, 14, 14, 5), (64, 64, 56, 56, 4), (96, 48, 28, 28, 6), (144, 144, 14, 14, 5),
+                                          (192, 192, 8, 8, 3), (256, 256, 14, 14, 4), (256, 96, 27, 28, 8), (80, 80, 9, 7, 4)])
+def test_run_skipping_decoder_groups(ctx, c, k, h, w, bits):
+    params = fm.layer_params(fm.LayerSpec(c, h, w, 0.9, None, 13000 + c + k))
+    cal = fm.make_maps(params, max(4, 30000 // (h * w)), calib=True, dtype=torch.bfloat16, device="cuda")
+    x = fm.make_maps(params, 148 * 9 * 128 // (h * w) + 3, dtype=torch.bfloat16, device="cuda")
+    m = tc.tc_fit_pca(ctx, cal, bits, k=k)
+    cb = tc.tc_build_codebook(ctx, m, tc.tc_stats(ctx, m, None, cal).hist)
+    enc = tc.tc_encode(ctx, m, cb, x)
+    got = tc.tc_decode(ctx, m, cb, enc, x.shape, x.dtype)
+    assert tc.tc_get_status(ctx) == 0 and tc.tc_last_path(ctx, True) == 1
+    tc.tc_force_exact_path(ctx, 1)
+    want = tc.tc_decode(ctx, m, cb, enc, x.shape, x.dtype)
+    assert tc.tc_get_status(ctx) == 0
+    tc.tc_force_exact_path(ctx, 0)
+    # one rounding to bf16 on each side of the same value: neighbours at most, and for 0.1 % of the values
+    # (the cap of the parity cases)
+    a, b = got.float(), want.float()
+    assert bool(((a - b).abs() <= 2.0 ** -7 * b.abs() + 1e-6 * float(b.abs().max())).all())
+    assert float((a != b).double().mean()) <= 1e-3
+    m.close(); cb.close()
