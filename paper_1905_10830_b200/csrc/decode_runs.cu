@@ -61,7 +61,8 @@ constexpr int kTrWarpBytes = 2048;                            // epilogue transp
 // tensor core signals: accumulator ready, operand panel consumed.)
 constexpr int kBarGroup = 1;                                  // + group: the VLD threads of a group, once per tile
 constexpr int kBarAccFree = kBarGroup + kMaxGroups;           // + accumulator: drained, epilogue warps -> MMA warp
-constexpr int kBarEpi = kBarAccFree + 2;                      // accumulator ready, polling epilogue warp -> the other seven
+constexpr int kBarBasis = kBarAccFree + 2;                    // basis in tensor memory, epilogue warps -> MMA warps, once
+constexpr int kBarEpi = kBarAccFree + 3;                      // accumulator ready, polling epilogue warp -> the other seven
 
 struct SmemLayout {
     uint32_t lut, opnd, tbuf, sbuf, total;
@@ -226,20 +227,20 @@ __global__ void __launch_bounds__(kThreads, 1) decode_runs_kernel(DecodeArgs a, 
     const int items = n_blocks;                                // work items per tile: halves of 64 pixels with two channel blocks
 
     // ---- set-up ---------------------------------------------------------------------
-    if (tid == 0) {
-        for (int g = 0; g < G; ++g) {
-            for (int p = 0; p < kMaxPanels; ++p) mbar_init(smem_u32(&s_empty[g][p]), (uint32_t)items);   // one commit per item of the tile
-            mbar_init(smem_u32(&s_bfull[g]), (uint32_t)group_warps);                                     // operand complete: one arrival per warp
-        }
-        for (int w = 0; w < 2; ++w) mbar_init(smem_u32(&s_tfull[w]), 1);
+    if (tid < G * (kMaxPanels + 1)) {
+        const int g = tid / (kMaxPanels + 1), p = tid - g * (kMaxPanels + 1);
+        if (p < kMaxPanels) mbar_init(smem_u32(&s_empty[g][p]), (uint32_t)items);       // one commit per item of the tile
+        else mbar_init(smem_u32(&s_bfull[g]), (uint32_t)group_warps);                   // operand complete: one arrival per warp
+        if (tid < 2) mbar_init(smem_u32(&s_tfull[tid]), 1);
         mbar_fence_init();
     }
     if (warp == kMmaWarp) { tmem_alloc(smem_u32(&s_tmem_base), kTmemCols); tmem_relinquish(); }
     {
         // per-layer table: bf16(symbol - center) << 16 | code length
         uint32_t *s_lut = reinterpret_cast<uint32_t *>(smem + L.lut);
+#pragma unroll 5
         for (int i = tid; i < lut_size; i += kThreads) {
-            const uint32_t e = a.lut32[i];
+            const uint32_t e = __ldg(a.lut32 + i);
             const float f = (float)((int)((e >> 8) & 0xffu) - a.center);
             s_lut[i] = (__float_as_uint(f) & 0xffff0000u) | (e & 0xffu);
         }
@@ -259,6 +260,7 @@ __global__ void __launch_bounds__(kThreads, 1) decode_runs_kernel(DecodeArgs a, 
             const int ch = blk * 128 + wq * 32 + lane;
             const uint32_t *row = src + (size_t)(ch < a.c ? ch : 0) * (a.k / 2);
             const uint32_t trow = tmem_base + ((uint32_t)(wq * 32) << 16) + (uint32_t)(blk * (a.k / 2));
+#pragma unroll 2
             for (int j = 0; j < a.k / 2; j += 16) {
                 if (a.k / 2 - j >= 16) {
                     uint32_t r[16];
@@ -280,10 +282,10 @@ __global__ void __launch_bounds__(kThreads, 1) decode_runs_kernel(DecodeArgs a, 
             }
         }
         tmem_st_wait();
+        // (only the MMA warps wait for the basis; the VLD groups are on their first tiles meanwhile)
+        tc_fence_before_sync();
+        named_bar_arrive(kBarBasis, 256 + 64);
     }
-    tc_fence_before_sync();
-    __syncthreads();
-    tc_fence_after_sync();
 
     const long long my_tiles = (a.n_tiles > blockIdx.x) ? (a.n_tiles - blockIdx.x + gridDim.x - 1) / gridDim.x : 0;
 
@@ -645,6 +647,8 @@ __global__ void __launch_bounds__(kThreads, 1) decode_runs_kernel(DecodeArgs a, 
         // (no branch around an MMA).
         // A = transposed basis in tensor memory (128 channels per instruction), B = the decoded
         // symbols of the item's pixels (rows of the group's operand buffer).
+        named_bar_sync(kBarBasis, 256 + 64);
+        tc_fence_after_sync();
         const int w = warp - kMmaWarp;
         const uint32_t issuer = lane == 0 ? 1u : 0u;
         const int np = items == 2 ? 64 : TC_TILE_PIXELS;          // pixels per work item
