@@ -9,6 +9,8 @@
 // unfused double operations as the per-pixel kernels, so the results are bit-identical to theirs
 // (and to the definition evaluated in fp64); the entropy coder then runs in the per-pixel kernels
 // on the symbols these kernels leave in memory.
+#include <algorithm>
+
 #include "device_utils.cuh"
 
 namespace {
@@ -134,17 +136,23 @@ __global__ void __launch_bounds__(kPx * kOut) reconstruct_kernel(DecodeArgs a, c
     store_rounded(out + img * a.c * (long long)a.hw + (long long)c * a.hw + (p - img * a.hw), v);
 }
 
-// Entropy coder on symbols that already sit in memory ([P][K] bytes), for tensors of few pixels:
-// one block per tile of 128 pixels, `parts` threads per pixel, each coding a run of K / parts
-// consecutive coefficients (a multiple of 16, so that a thread fetches its symbols in 16-byte
+// Entropy coder on symbols that already sit in memory ([P][K] bytes, row 0 = the first pixel of tile
+// `first_tile`): one block per tile of 128 pixels, `parts` threads per pixel, each coding a run of
+// K / parts consecutive coefficients (a multiple of 8, so that a thread fetches its symbols in 8-byte
 // pieces and a chunk -- one of 1, 2 or 4 runs of a pixel -- is a whole number of thread runs).
 // Code lengths first (the lookups of a run are independent loads), then the bit offsets -- runs
-// inside a pixel, pixels inside the tile, the tile inside the stream by look-back -- then every
-// thread packs its run into the zeroed words of the tile.  Same stream, chunk lengths and tile
-// offsets as the one-thread-per-pixel coder.
+// inside a pixel, pixels inside the tile -- then every thread packs its run into zeroed words in
+// shared memory with an atomic OR at its ends, while the tile's place in the stream is found by
+// look-back; the words leave 16 bytes at a time.  A tile that does not fit the staging buffer is packed
+// into zeroed global memory.  Same stream, chunk lengths and tile offsets as the
+// one-thread-per-pixel coder.
+// What bounds it: instructions, about ten per symbol, and for few tiles the one block's latency -- hence
+// up to eight threads a pixel and a per-layer table in shared memory (960x7x7 x 128: 45 us with four
+// threads, tables and packed words in global memory, 13 like this).
 constexpr int kMaxParts = 8;
 
-__global__ void __launch_bounds__(TC_TILE_PIXELS * kMaxParts) pack_symbols_kernel(EncodeArgs a, const uint8_t *sym, int parts)
+__global__ void __launch_bounds__(TC_TILE_PIXELS * kMaxParts) pack_symbols_kernel(EncodeArgs a, const uint8_t *sym, int parts, long long first_tile,
+                                                                                  unsigned int staging_bytes)
 {
     __shared__ long long s_tile;
     __shared__ unsigned int s_run_bits[TC_TILE_PIXELS * kMaxParts];
@@ -152,57 +160,52 @@ __global__ void __launch_bounds__(TC_TILE_PIXELS * kMaxParts) pack_symbols_kerne
     __shared__ unsigned int s_pixel_off[TC_TILE_PIXELS + 1];
     __shared__ unsigned long long s_base;
     __shared__ int s_write_ok;
+    __shared__ uint32_t s_enc[256];
+    extern __shared__ __align__(16) uint32_t s_words[];
     const int t = threadIdx.x;
     const int nsym = 1 << a.bits;
+    const bool per_layer = a.groups == 1;
     if (t == 0) s_tile = (long long)atomicAdd(a.ticket, 1u);
+    if (per_layer)
+        for (int i = t; i < nsym; i += blockDim.x) s_enc[i] = __ldg(a.enc + i);
     __syncthreads();
     const long long tile = s_tile;
     const int px = t / parts, part = t - px * parts;          // the threads of a pixel are neighbours
     const long long p = tile * TC_TILE_PIXELS + px;
     const bool valid = p < a.pixels;
     const int run = a.k / parts, j0 = part * run;
-    const uint8_t *src = sym + p * a.k + j0;
+    const uint8_t *src = sym + (p - first_tile * TC_TILE_PIXELS) * a.k + j0;
+    // code << 8 | length of the symbol in byte b of w, coefficient j
+    auto entry = [&](uint32_t w, int b, int j) {
+        const uint32_t q = (w >> (8 * b)) & 0xffu;
+        return per_layer ? s_enc[q] : __ldg(a.enc + j * nsym + q);
+    };
 
     unsigned int my_bits = 0;
     if (valid)
-        for (int i = 0; i < run; i += 16) {
-            const uint4 v = __ldg(reinterpret_cast<const uint4 *>(src + i));
-            const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll 2
+        for (int i = 0; i < run; i += 8) {
+            const uint2 v = __ldg(reinterpret_cast<const uint2 *>(src + i));
 #pragma unroll
-            for (int b = 0; b < 16; ++b) {
-                const int j = j0 + i + b;
-                const uint32_t q = (w[b >> 2] >> (8 * (b & 3))) & 0xffu;
-                my_bits += __ldg(a.enc + (a.groups == 1 ? 0 : j) * nsym + q) & 0xffu;
-            }
+            for (int b = 0; b < 8; ++b) my_bits += entry(b < 4 ? v.x : v.y, b & 3, j0 + i + b) & 0xffu;
         }
     s_run_bits[t] = my_bits;
     __syncthreads();
     // pixel totals, scanned by the first 128 threads
-    unsigned int tile_bits = 0;
     if (t < TC_TILE_PIXELS) {
-        unsigned int pixel_bits = 0;
+        unsigned int pixel_bits = 0, total = 0;
         for (int r = 0; r < parts; ++r) pixel_bits += s_run_bits[t * parts + r];
-        const unsigned int off = group_exclusive_scan_128(pixel_bits, s_warp_sums, t, 1, tile_bits);
+        const unsigned int off = group_exclusive_scan_128(pixel_bits, s_warp_sums, t, 1, total);
         s_pixel_off[t] = off;
-        if (t == 0) s_pixel_off[TC_TILE_PIXELS] = tile_bits;
-        const unsigned long long padded = ((unsigned long long)tile_bits + 127ull) & ~127ull;
-        if (t < 32) {
-            bool ok;
-            const unsigned long long base = tile_lookback(a.tile_state, tile, padded, a.status, ok);
-            if (t == 0) {
-                const bool fits = base + padded <= a.capacity_bits;
-                if (ok && !fits) tc_dev_set_status(a.status, TC_ERR_BUFFER_TOO_SMALL);
-                s_base = base;
-                s_write_ok = (ok && fits) ? 1 : 0;
-                a.tile_off[tile] = base;
-                if (tile == a.n_tiles - 1) a.tile_off[a.n_tiles] = base + padded;
-            }
+        if (t == 0) {
+            s_pixel_off[TC_TILE_PIXELS] = total;
+            lookback_publish(a.tile_state, tile, ((unsigned long long)total + 127ull) & ~127ull);
         }
     }
     __syncthreads();
-    const unsigned long long base = s_base;
-    tile_bits = s_pixel_off[TC_TILE_PIXELS];
+    const unsigned int tile_bits = s_pixel_off[TC_TILE_PIXELS];
     const unsigned long long padded = ((unsigned long long)tile_bits + 127ull) & ~127ull;
+    const bool staged = padded <= (unsigned long long)staging_bytes * 8ull;
     unsigned int my_off = s_pixel_off[px];
     for (int r = 0; r < part; ++r) my_off += s_run_bits[px * parts + r];
     // chunk lengths: a chunk is chunk_pixels pixels, or one of `splits` runs of one pixel
@@ -219,34 +222,61 @@ __global__ void __launch_bounds__(TC_TILE_PIXELS * kMaxParts) pack_symbols_kerne
             a.chunk_len[p / a.chunk_pixels] = (uint16_t)(s_pixel_off[last] - s_pixel_off[px]);
         }
     }
-    if (!s_write_ok) return;
-    {
-        uint4 *dst = reinterpret_cast<uint4 *>(a.stream + (base >> 5));
-        const unsigned int n16 = (unsigned int)(padded >> 7);
-        for (unsigned int i = t; i < n16; i += blockDim.x) dst[i] = make_uint4(0u, 0u, 0u, 0u);
-    }
-    __syncthreads();
-    if (valid) {
-        BitWriter w;
-        w.init(a.stream, base + my_off);
-        for (int i = 0; i < run; i += 16) {
-            const uint4 v = __ldg(reinterpret_cast<const uint4 *>(src + i));
-            const uint32_t wd[4] = {v.x, v.y, v.z, v.w};
-            uint32_t e[16];
-#pragma unroll
-            for (int b = 0; b < 16; ++b) {
-                const int j = j0 + i + b;
-                const uint32_t q = (wd[b >> 2] >> (8 * (b & 3))) & 0xffu;
-                e[b] = __ldg(a.enc + (a.groups == 1 ? 0 : j) * nsym + q);
+    // the tile's place in the stream (one warp; without staging everyone needs it first)
+    auto resolve = [&] {
+        if (t < 32) {
+            bool ok;
+            const unsigned long long base = lookback_resolve(a.tile_state, tile, padded, a.status, ok);
+            if (t == 0) {
+                const bool fits = base + padded <= a.capacity_bits;
+                if (ok && !fits) tc_dev_set_status(a.status, TC_ERR_BUFFER_TOO_SMALL);
+                s_base = base;
+                s_write_ok = (ok && fits) ? 1 : 0;
+                a.tile_off[tile] = base;
+                if (tile == a.n_tiles - 1) a.tile_off[a.n_tiles] = base + padded;
             }
+        }
+    };
+    auto pack = [&](uint32_t *words, unsigned long long at) {
+        if (!valid) return;
+        BitWriter w;
+        w.init(words, at);
+#pragma unroll 1
+        for (int i = 0; i < run; i += 8) {
+            const uint2 v = __ldg(reinterpret_cast<const uint2 *>(src + i));
 #pragma unroll
-            for (int b = 0; b < 16; ++b) w.put(e[b] >> 8, (int)(e[b] & 0xffu));
+            for (int b = 0; b < 8; b += 2) {                  // two codes a piece, at most 24 bits
+                const uint32_t x = b < 4 ? v.x : v.y;
+                const uint32_t e0 = entry(x, b & 3, j0 + i + b), e1 = entry(x, (b & 3) + 1, j0 + i + b + 1);
+                w.put(((e0 >> 8) << (e1 & 0xffu)) | (e1 >> 8), (int)((e0 & 0xffu) + (e1 & 0xffu)));
+            }
         }
         w.finish();
+    };
+    const unsigned int n16 = (unsigned int)(padded >> 7);
+    if (staged) {
+        for (unsigned int i = t; i < n16; i += blockDim.x) reinterpret_cast<uint4 *>(s_words)[i] = make_uint4(0u, 0u, 0u, 0u);
+        __syncthreads();
+        pack(s_words, my_off);
+        resolve();
+        __syncthreads();
+        if (!s_write_ok) return;
+        uint4 *dst = reinterpret_cast<uint4 *>(a.stream + (s_base >> 5));
+        for (unsigned int i = t; i < n16; i += blockDim.x) dst[i] = reinterpret_cast<const uint4 *>(s_words)[i];
+    } else {
+        resolve();
+        __syncthreads();
+        if (!s_write_ok) return;
+        uint4 *dst = reinterpret_cast<uint4 *>(a.stream + (s_base >> 5));
+        for (unsigned int i = t; i < n16; i += blockDim.x) dst[i] = make_uint4(0u, 0u, 0u, 0u);
+        __syncthreads();
+        pack(a.stream, s_base + my_off);
     }
 }
 
-// Entropy decoder that leaves the symbols in memory ([P][K] bytes), for tensors of few pixels:
+// Entropy decoder that leaves the symbols in memory, row 0 = the first pixel of tile `first_tile`: as bytes
+// ([P][K], for the fp64 inverse of tensors of few pixels), or centred and as bf16 (kOperand: the
+// operand of the tensor cores' inverse transform):
 // one block per tile, one thread per chunk (up to 512 per tile), so that every chunk of the tile is
 // walked at the same time; the inverse transform then runs in reconstruct_kernel.  Same checks as
 // the per-pixel decoder: tile offsets aligned, ordered and inside the stream, every chunk inside
@@ -302,8 +332,10 @@ struct AheadReader {
 // global memory off the chain.  The threads of a warp walk the same run of coefficients of
 // neighbouring pixels, and symbols leave 16 bytes at a time.  Measured with the inverse transform
 // and the launches, 256x14x14 at 6 bits: 64.5 us with a 2^12-entry table per channel in global
-// memory and a byte stored per symbol.
-__global__ void __launch_bounds__(kUnpackThreads) unpack_symbols_kernel(DecodeArgs a, uint8_t *sym)
+// memory and a byte stored per symbol,
+// 40 us with the loop unrolled over sixteen symbols (16 KB of code, fetched once per launch).
+template <bool kOperand>
+__global__ void __launch_bounds__(kUnpackThreads) unpack_symbols_kernel(DecodeArgs a, void *out, long long first_tile)
 {
     __shared__ unsigned int s_warp_sums[kUnpackThreads / 32];
     __shared__ unsigned int s_start[kUnpackThreads];
@@ -311,13 +343,17 @@ __global__ void __launch_bounds__(kUnpackThreads) unpack_symbols_kernel(DecodeAr
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
     const int lut_size = 1 << a.lut_bits, nsym = 1 << a.bits;
     const bool per_layer = a.groups == 1;
-    uint16_t *s_lut = reinterpret_cast<uint16_t *>(s_tables);
-    uint32_t *s_canon = reinterpret_cast<uint32_t *>(s_tables);
+    // per-layer table: value << 16 | length, the value being the symbol or its centred bf16
+    uint32_t *s_lut = reinterpret_cast<uint32_t *>(s_tables), *s_canon = s_lut;
+    auto value = [&](uint32_t q) { return kOperand ? __float_as_uint((float)((int)q - a.center)) >> 16 : q; };
     if (per_layer)
-        for (int i = t; i < lut_size; i += kUnpackThreads) s_lut[i] = a.lut[i];
+        for (int i = t; i < lut_size; i += blockDim.x) {
+            const uint32_t e = __ldg(a.lut + i);
+            s_lut[i] = (value(e >> 8) << 16) | (e & 0xffu);
+        }
     else
-        for (int i = t; i < a.k * kCanonWords; i += kUnpackThreads) s_canon[i] = a.canon[i];
-    const long long tile = blockIdx.x;
+        for (int i = t; i < a.k * kCanonWords; i += blockDim.x) s_canon[i] = a.canon[i];
+    const long long tile = first_tile + blockIdx.x;
     const unsigned long long base = a.tile_off[tile], end = a.tile_off[tile + 1];
     const bool tile_ok = (base & 127ull) == 0 && (end & 127ull) == 0 && base <= end && end <= a.stream_bits;
     if (!tile_ok) {
@@ -363,37 +399,41 @@ __global__ void __launch_bounds__(kUnpackThreads) unpack_symbols_kernel(DecodeAr
                 if (per_layer) {
                     const uint32_t e = s_lut[r.hi >> (32 - a.lut_bits)];
                     len = e & 0xffu;
-                    v[i] = e >> 8;
+                    v[i] = e >> 16;
                 } else {
                     const uint32_t *c = s_canon + (j + i) * kCanonWords;
                     const CanonBounds cb{*reinterpret_cast<const uint4 *>(c), *reinterpret_cast<const uint2 *>(c + 4)};
                     len = canon_length(r.hi, cb);
-                    v[i] = canon_symbol(r.hi, len, reinterpret_cast<const uint16_t *>(c + 6), a.sorted + (size_t)(j + i) * nsym);
+                    v[i] = value(canon_symbol(r.hi, len, reinterpret_cast<const uint16_t *>(c + 6), a.sorted + (size_t)(j + i) * nsym));
                 }
                 r.skip(len);
                 used += len;
             }
         };
-        const bool by16 = a.k % 16 == 0 && run % 16 == 0;
+        const bool by8 = a.k % 8 == 0 && run % 8 == 0;
         for (int lp = first_px; lp < first_px + (a.splits > 1 ? 1 : a.chunk_pixels); ++lp) {
             const long long p = tile * TC_TILE_PIXELS + lp;
             if (p >= a.pixels) break;
-            uint8_t *dst = sym + p * a.k;
-            if (by16) {
+            const long long row = (p - first_tile * TC_TILE_PIXELS) * a.k;
+            if (by8) {
 #pragma unroll 1
-                for (int j = j_first; j < j_first + run; j += 16) {
-                    uint32_t v[16], w[4];
+                for (int j = j_first; j < j_first + run; j += 8) {
+                    uint32_t v[8];
                     decode(j, v);
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) w[i] = v[4 * i] | (v[4 * i + 1] << 8) | (v[4 * i + 2] << 16) | (v[4 * i + 3] << 24);
-                    *reinterpret_cast<uint4 *>(dst + j) = make_uint4(w[0], w[1], w[2], w[3]);
+                    if constexpr (kOperand)
+                        *reinterpret_cast<uint4 *>((uint16_t *)out + row + j) =
+                            make_uint4(v[0] | (v[1] << 16), v[2] | (v[3] << 16), v[4] | (v[5] << 16), v[6] | (v[7] << 16));
+                    else
+                        *reinterpret_cast<uint2 *>((uint8_t *)out + row + j) =
+                            make_uint2(v[0] | (v[1] << 8) | (v[2] << 16) | (v[3] << 24), v[4] | (v[5] << 8) | (v[6] << 16) | (v[7] << 24));
                 }
             } else {
 #pragma unroll 1
                 for (int j = j_first; j < j_first + run; ++j) {
                     uint32_t v[1];
                     decode(j, v);
-                    dst[j] = (uint8_t)v[0];
+                    if constexpr (kOperand) ((uint16_t *)out)[row + j] = (uint16_t)v[0];
+                    else ((uint8_t *)out)[row + j] = (uint8_t)v[0];
                 }
             }
         }
@@ -423,32 +463,47 @@ tc_status tc_launch_reconstruct(const DecodeArgs &a, int dtype, const uint8_t *s
 }
 
 // How many threads per pixel the parallel coder would use for K coefficients and `splits` chunks
-// per pixel: the largest of 8, 4, 2, 1 that gives every thread a multiple of 16 coefficients and
+// per pixel: the largest of 8, 4, 2, 1 that gives every thread a multiple of 8 coefficients and
 // every chunk a whole number of threads (0: none, use the one-thread-per-pixel coder).
 int tc_pack_symbols_parts(const EncodeArgs &a)
 {
     if (((uintptr_t)a.stream & 15u) != 0) return 0;
     for (int parts = kMaxParts; parts >= 1; parts >>= 1)
-        if (a.k % (16 * parts) == 0 && parts % a.splits == 0) return parts;
+        if (a.k % (8 * parts) == 0 && parts % a.splits == 0) return parts;
     return 0;
 }
 
-tc_status tc_launch_pack_symbols(const EncodeArgs &a, const uint8_t *sym, cudaStream_t s)
+tc_status tc_launch_pack_symbols(const EncodeArgs &a, const uint8_t *sym, long long first_tile, long long end_tile, cudaStream_t s)
 {
-    if (a.n_tiles <= 0) return TC_OK;
+    if (end_tile <= first_tile) return TC_OK;
     const int parts = tc_pack_symbols_parts(a);
-    if (parts == 0 || ((uintptr_t)sym & 15u) != 0) return TC_ERR_UNSUPPORTED;
-    pack_symbols_kernel<<<(unsigned int)a.n_tiles, TC_TILE_PIXELS * parts, 0, s>>>(a, sym, parts);
+    if (parts == 0 || ((uintptr_t)sym & 7u) != 0) return TC_ERR_UNSUPPORTED;
+    // staging for four bits per symbol, at most 96 KB: two blocks of 1024 threads still fit an SM
+    const unsigned int staging = (unsigned int)std::min<long long>((long long)a.k * TC_TILE_PIXELS / 2, 96 * 1024);
+    if (cudaFuncSetAttribute(pack_symbols_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024) != cudaSuccess) return TC_ERR_CUDA;
+    pack_symbols_kernel<<<(unsigned int)(end_tile - first_tile), TC_TILE_PIXELS * parts, staging, s>>>(a, sym, parts, first_tile, staging);
+    return cudaGetLastError() == cudaSuccess ? TC_OK : TC_ERR_CUDA;
+}
+
+template <bool kOperand>
+static tc_status launch_unpack(const DecodeArgs &a, void *out, long long first_tile, long long end_tile, cudaStream_t s)
+{
+    if (end_tile <= first_tile) return TC_OK;
+    const int chunks = a.splits * TC_TILE_PIXELS / a.chunk_pixels;
+    if (chunks > kUnpackThreads) return TC_ERR_UNSUPPORTED;
+    const size_t smem = a.groups == 1 ? ((size_t)4 << a.lut_bits) : (size_t)a.k * kCanonWords * 4;      // at most 48 KB
+    if (cudaFuncSetAttribute(unpack_symbols_kernel<kOperand>, cudaFuncAttributeMaxDynamicSharedMemorySize, TC_MAX_C * kCanonWords * 4) != cudaSuccess)
+        return TC_ERR_CUDA;
+    unpack_symbols_kernel<kOperand><<<(unsigned int)(end_tile - first_tile), (chunks + 31) / 32 * 32, smem, s>>>(a, out, first_tile);
     return cudaGetLastError() == cudaSuccess ? TC_OK : TC_ERR_CUDA;
 }
 
 tc_status tc_launch_unpack_symbols(const DecodeArgs &a, uint8_t *sym, cudaStream_t s)
 {
-    if (a.n_tiles <= 0) return TC_OK;
-    if (a.splits * TC_TILE_PIXELS / a.chunk_pixels > kUnpackThreads) return TC_ERR_UNSUPPORTED;
-    const size_t smem = a.groups == 1 ? ((size_t)2 << a.lut_bits) : (size_t)a.k * kCanonWords * 4;      // at most 48 KB
-    if (cudaFuncSetAttribute(unpack_symbols_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, TC_MAX_C * kCanonWords * 4) != cudaSuccess)
-        return TC_ERR_CUDA;
-    unpack_symbols_kernel<<<(unsigned int)a.n_tiles, kUnpackThreads, smem, s>>>(a, sym);
-    return cudaGetLastError() == cudaSuccess ? TC_OK : TC_ERR_CUDA;
+    return launch_unpack<false>(a, sym, 0, a.n_tiles, s);
+}
+
+tc_status tc_launch_unpack_operand(const DecodeArgs &a, void *operand, long long first_tile, long long end_tile, cudaStream_t s)
+{
+    return launch_unpack<true>(a, operand, first_tile, end_tile, s);
 }

@@ -29,6 +29,17 @@ static EncodeTiledFn encode_tiled_fn()
     return fn;
 }
 
+bool tc_tensor_map_sw128(CUtensorMap *map, const void *base, long long rows, int cols, int box_rows)
+{
+    const EncodeTiledFn fn = encode_tiled_fn();
+    if (!fn) return false;
+    const cuuint64_t dims[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
+    const cuuint64_t strides[1] = {(cuuint64_t)cols * 2};
+    const cuuint32_t box[2] = {64u, (cuuint32_t)box_rows};
+    const cuuint32_t elem[2] = {1u, 1u};
+    return fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void *>(base), dims, strides, box, elem, CU_TENSOR_MAP_INTERLEAVE_NONE,
+              CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
 
 #define TC_CUDA(call)                                   \
     do {                                                \
@@ -197,16 +208,8 @@ tc_status finish_model(tc_model *m)
         }
         // and for the decoder: the transposed basis in boxes of 128 channel rows x 64 coefficients
         m->has_basis_t_map = false;
-        if (encode_tiled && k % 16 == 0) {
-            const cuuint64_t dims[2] = {(cuuint64_t)k, (cuuint64_t)c};
-            const cuuint64_t strides[1] = {(cuuint64_t)k * 2};
-            const cuuint32_t box[2] = {64u, 128u};
-            const cuuint32_t elem[2] = {1u, 1u};
-            const CUresult rc = encode_tiled(&m->basis_t_map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, m->d_basis_t_bf16, dims,
-                                                       strides, box, elem, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
-                                                       CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-            m->has_basis_t_map = rc == CUDA_SUCCESS;
-        }
+        if (k % 16 == 0) m->has_basis_t_map = tc_tensor_map_sw128(&m->basis_t_map, m->d_basis_t_bf16, c, k, 128);
+        if (c % 16 == 0) m->has_basis_gemm_map = tc_tensor_map_sw128(&m->basis_gemm_map, m->d_basis_bf16, k, c, 32);
     }
     TC_CUDA(cudaStreamSynchronize(nullptr));
     return TC_OK;
@@ -813,12 +816,29 @@ void tc_codebook_free(tc_codebook *cb)
 
 }  // extern "C"
 
+// bf16 tensors the resident-basis encoder does not take because of their width, map size or alignment
+// (the streaming kernels' share, see tc_force_exact_path)
+static bool wide_encode(const tc_ctx *ctx, const tc_model *m, const tc_tensor *x)
+{
+    return x->dtype == TC_BF16 && ctx->force_exact != 1 && m->c % 16 == 0 && m->k % 16 == 0 &&
+           (m->c > 256 || (x->h * x->w) % 4 != 0 || ((uintptr_t)x->data & 7u) != 0);
+}
+
+// Bytes of workspace an encode of `x` makes use of: the rows and symbols of a wide layer, or the symbols
+// of a tensor of few tiles on the exact kernels.
+static size_t encode_work_bytes(const tc_ctx *ctx, const tc_model *m, const tc_tensor *x)
+{
+    const long long pixels = (long long)x->n * x->h * x->w, n_tiles = (pixels + TC_TILE_PIXELS - 1) / TC_TILE_PIXELS;
+    if (wide_encode(ctx, m, x)) return tc_encode_wide_workspace(m->c, m->k, n_tiles);
+    return n_tiles < (long long)kExactParallelTilesPerSm * ctx->sm_count ? (((size_t)pixels * m->k + 255) & ~(size_t)255) : 0;
+}
+
 // Argument block and kernel choice shared by tc_encode and tc_encode_noalloc.  `scratch` is
 // kEncodeScratchHeader bytes (ticket counter) followed by one 64-bit look-back word per tile;
 // it is cleared on the stream here, whoever owns it.
 tc_status tc_encode_with_scratch(tc_ctx *ctx, const tc_model *m, const tc_codebook *cb, const tc_tensor *x, int chunk_pixels,
                                  int splits, void *stream_out, size_t capacity, uint16_t *chunk_len, uint64_t *tile_off,
-                                 const tc_debug_out *debug, void *scratch, uint8_t *sym_scratch, cudaStream_t s,
+                                 const tc_debug_out *debug, void *scratch, void *work, cudaStream_t s,
                                  unsigned long long *hist, unsigned long long *clamped, bool scratch_is_zero)
 {
     const long long pixels = (long long)x->n * x->h * x->w;
@@ -840,6 +860,7 @@ tc_status tc_encode_with_scratch(tc_ctx *ctx, const tc_model *m, const tc_codebo
     a.status = ctx->d_status; a.clamped = clamped; a.emit = 1;
     a.basis_bf16 = m->d_basis_bf16; a.basis_core = m->d_basis_core; a.enc_bias = m->d_enc_bias; a.tmu32 = m->d_tmu32;
     a.basis_map = m->has_basis_map ? &m->basis_map : nullptr;
+    a.basis_gemm_map = m->has_basis_gemm_map ? &m->basis_gemm_map : nullptr;
     a.hist = hist; a.hist_modal = m->center;
     a.modal = cb->modal;
     a.blk_bits = m->blk_bits.data(); a.blk_odd = m->blk_odd.data();
@@ -851,15 +872,9 @@ tc_status tc_encode_with_scratch(tc_ctx *ctx, const tc_model *m, const tc_codebo
     }
     if (ctx->force_exact != 1 && x->dtype == TC_BF16 && tc_encode_wide_supported(ctx, a)) {   // wide layers, unaligned rows
         ctx->last_encode_path = 3;
-        if (sym_scratch && n_tiles < ctx->sm_count && ((uintptr_t)sym_scratch & 15u) == 0 && tc_pack_symbols_parts(a) > 0) {
-            // fewer tiles than SMs: the projection is dealt over the SMs by blocks of coefficients and leaves
-            // the symbols in the arena, the entropy coder follows as a kernel of its own (same stream)
-            a.sym_park = sym_scratch;
-            const tc_status st = tc_launch_encode_wide(ctx, a, s);
-            if (st != TC_OK) return st;
-            a.sym_park = nullptr;
-            return tc_launch_pack_symbols(a, sym_scratch, s);
-        }
+        // with workspace: projection as a tiled product, the entropy coder as a kernel of its own
+        if (work && !debug && wide_encode(ctx, m, x) && a.basis_gemm_map && tc_pack_symbols_parts(a) > 0)
+            return tc_launch_encode_wide_gemm(ctx, a, a.basis_gemm_map, work, s);
         return tc_launch_encode_wide(ctx, a, s);
     }
     if (ctx->force_exact != 1 && x->dtype == TC_BF16 && x->c % 2 == 0) {      // shapes the tensor-core kernel does not take
@@ -867,13 +882,14 @@ tc_status tc_encode_with_scratch(tc_ctx *ctx, const tc_model *m, const tc_codebo
         return tc_launch_encode_simt_fp32(ctx, a, s);
     }
     ctx->last_encode_path = 0;
-    if (sym_scratch && n_tiles < (long long)kExactParallelTilesPerSm * ctx->sm_count) {
+    if (work && n_tiles < (long long)kExactParallelTilesPerSm * ctx->sm_count) {
+        uint8_t *const sym_scratch = (uint8_t *)work;
         // few pixels: projection and quantiser with one thread per (pixel, coefficient), then the
         // entropy coder of the per-pixel kernel on those symbols -- same arithmetic, same results
         tc_status st = tc_launch_project_quantise(a, x->dtype, sym_scratch, s);
         if (st != TC_OK) return st;
         if (tc_pack_symbols_parts(a) > 0 && ((uintptr_t)sym_scratch & 15u) == 0)
-            return tc_launch_pack_symbols(a, sym_scratch, s);      // several threads per pixel code the symbols
+            return tc_launch_pack_symbols(a, sym_scratch, 0, a.n_tiles, s);      // several threads per pixel code the symbols
         a.sym_in = sym_scratch;
     }
     return tc_launch_encode_simt(ctx, a, x->dtype, s);
@@ -932,20 +948,24 @@ tc_status tc_encode(tc_ctx *ctx, const tc_model *m, const tc_codebook *cb, const
         return TC_OK;
     }
     const size_t lookback = (kEncodeScratchHeader + (size_t)n_tiles * sizeof(unsigned long long) + 255) & ~(size_t)255;
-    // small tensors on the exact kernels also park their symbols in the arena (P * K bytes)
-    const bool parallel_exact = n_tiles < (long long)kExactParallelTilesPerSm * ctx->sm_count;
-    const size_t scratch = lookback + (parallel_exact ? (size_t)pixels * m->k : 0);
-    if ((st = ensure_scratch(ctx, scratch)) != TC_OK) return st;
+    const size_t work = encode_work_bytes(ctx, m, x);
+    if ((st = ensure_scratch(ctx, lookback + work)) != TC_OK) return st;
     return tc_encode_with_scratch(ctx, m, cb, x, cs.cp, cs.splits, stream_out, capacity, chunk_len, tile_off, debug,
-                                  ctx->scratch, parallel_exact ? (uint8_t *)ctx->scratch + lookback : nullptr, s);
+                                  ctx->scratch, work ? (char *)ctx->scratch + lookback : nullptr, s);
 }
 
-// Bytes of symbol scratch a decode of `x_hat` may need: small tensors on the exact kernels park
-// their symbols there (whether that route is taken is decided at launch).
+static bool wide_decode(const tc_ctx *ctx, const tc_model *m, const tc_tensor *x_hat)
+{
+    return x_hat->dtype == TC_BF16 && ctx->force_exact != 1 && m->c % 16 == 0 && m->k % 16 == 0 && m->c > 256;
+}
+
+// Bytes of workspace a decode of `x_hat` may need: the centred symbols of a wide layer, or the symbols of
+// a tensor of few tiles on the exact kernels (whether that route is taken is decided at launch).
 static size_t decode_scratch_bytes(const tc_ctx *ctx, const tc_model *m, const tc_tensor *x_hat)
 {
     const long long pixels = (long long)x_hat->n * x_hat->h * x_hat->w;
     const long long n_tiles = (pixels + TC_TILE_PIXELS - 1) / TC_TILE_PIXELS;
+    if (wide_decode(ctx, m, x_hat)) return tc_decode_wide_workspace(m->k, n_tiles);
     return n_tiles < (long long)kExactParallelTilesPerSm * ctx->sm_count ? (((size_t)pixels * m->k + 255) & ~(size_t)255) : 0;
 }
 
@@ -1002,6 +1022,9 @@ static tc_status decode_with_scratch(tc_ctx *ctx, const tc_model *m, const tc_co
     }
     if (ctx->force_exact != 1 && x_hat->dtype == TC_BF16 && tc_decode_wide_supported(ctx, a)) {   // wide layers
         ctx->last_decode_path = 3;
+        // with workspace: the entropy decoder as a kernel of its own, the inverse as a tiled product
+        if (sym_scratch && wide_decode(ctx, m, x_hat) && a.basis_t_map)
+            return tc_launch_decode_wide_gemm(ctx, a, sym_scratch, (cudaStream_t)cuda_stream);
         return tc_launch_decode_wide(ctx, a, (cudaStream_t)cuda_stream);
     }
     if (ctx->force_exact != 1 && x_hat->dtype == TC_BF16 && x_hat->c % 2 == 0) {  // shapes the tensor-core kernel does not take
@@ -1085,9 +1108,10 @@ tc_status tc_encode_many(tc_ctx *ctx, const tc_encode_item *items, int32_t n_ite
         const tc_encode_item &it = items[i];
         const long long pixels = (long long)it.x->n * it.x->h * it.x->w;
         const long long n_tiles = (pixels + TC_TILE_PIXELS - 1) / TC_TILE_PIXELS;
-        if (n_tiles > 0 && n_tiles < (long long)kExactParallelTilesPerSm * ctx->sm_count) {
+        const size_t bytes = n_tiles > 0 ? encode_work_bytes(ctx, it.model, it.x) : 0;
+        if (bytes) {
             symbols_at[i] = total;
-            total += ((size_t)pixels * it.model->k + 255) & ~(size_t)255;
+            total += bytes;
         }
     }
     tc_status st = ensure_scratch(ctx, total);
@@ -1108,7 +1132,7 @@ tc_status tc_encode_many(tc_ctx *ctx, const tc_encode_item *items, int32_t n_ite
         if (pixels == 0) { if (cudaMemsetAsync(it.tile_off, 0, sizeof(uint64_t), ws) != cudaSuccess && first_error == TC_OK) first_error = TC_ERR_CUDA; continue; }
         st = tc_encode_with_scratch(ctx, it.model, it.codebook, it.x, shape[i].cp, shape[i].splits, it.stream_out, it.capacity,
                                     it.chunk_len, it.tile_off, nullptr, (char *)ctx->scratch + lookback_at[i],
-                                    symbols_at[i] ? (uint8_t *)ctx->scratch + symbols_at[i] : nullptr, ws, nullptr, nullptr, true);
+                                    symbols_at[i] ? (char *)ctx->scratch + symbols_at[i] : nullptr, ws, nullptr, nullptr, true);
         if (st != TC_OK && first_error == TC_OK) first_error = st;
     }
     for (int j = 0; j < n_streams; ++j) {

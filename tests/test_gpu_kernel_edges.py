@@ -135,3 +135,40 @@ def test_run_skipping_decoder_groups(ctx, c, k, h, w, bits):
     assert bool(((a - b).abs() <= 2.0 ** -7 * b.abs() + 1e-6 * float(b.abs().max())).all())
     assert float((a != b).double().mean()) <= 1e-3
     m.close(); cb.close()
+
+
+# Wide layers as tiled products: blocks of coefficients and channels with remainders, pixel rows of 1, 2 and
+# 4-element alignment, fewer units than SMs and more, several passes over the workspace, every chunk
+# shape, both table granularities.  Against the fused kernel (debug outputs take it), whose symbols the
+# parity cases check, and the fp64 kernels.
+@pytest.mark.parametrize("c,k,h,w,n,bits,tables,offset", [
+    (272, 272, 3, 3, 1, 4, 1, 0), (320, 320, 5, 5, 40, 5, 1, 0), (576, 576, 14, 14, 9, 5, 1, 0), (960, 960, 7, 7, 30, 5, 1, 0),
+    (1024, 1024, 12, 12, 160, 2, 1, 0), (512, 512, 7, 7, 64, 8, 1, 0), (400, 208, 6, 6, 50, 6, 208, 0), (960, 16, 7, 7, 5, 8, 1, 0),
+    (80, 48, 27, 19, 37, 6, 48, 0), (64, 64, 9, 9, 1, 4, 1, 0), (256, 256, 7, 9, 90, 3, 1, 0), (128, 128, 14, 14, 6, 4, 1, 1), (48, 32, 5, 3, 700, 7, 1, 0)])
+def test_wide_layers_as_tiled_products(ctx, c, k, h, w, n, bits, tables, offset):
+    params = fm.layer_params(fm.LayerSpec(c, h, w, 0.95, None, 14000 + c + k + h))
+    cal = fm.make_maps(params, max(4, 4 * c // (h * w) + 1), calib=True, dtype=torch.bfloat16, device="cuda")
+    m = tc.tc_fit_pca(ctx, cal, bits, k=k)
+    cb = tc.tc_build_codebook(ctx, m, tc.tc_stats(ctx, m, None, cal, groups=tables).hist, groups=tables)
+    maps = fm.make_maps(params, n, dtype=torch.bfloat16, device="cuda")
+    buf = torch.empty(maps.numel() + 8, dtype=torch.bfloat16, device="cuda")
+    x = buf[offset:offset + maps.numel()].view(maps.shape)
+    x.copy_(maps)
+    fused = tc.tc_encode(ctx, m, cb, x, debug=True, k=k)
+    assert tc.tc_get_status(ctx) == 0 and tc.tc_last_path(ctx) == 3
+    enc = tc.tc_encode(ctx, m, cb, x)
+    assert tc.tc_get_status(ctx) == 0 and tc.tc_last_path(ctx) == 3
+    assert _same_stream(enc, fused)
+    got = tc.tc_decode(ctx, m, cb, enc, x.shape, x.dtype, relu=True)
+    assert tc.tc_get_status(ctx) == 0
+    if c > 256:
+        assert tc.tc_last_path(ctx, True) == 3
+    tc.tc_force_exact_path(ctx, 1)
+    want = tc.tc_decode(ctx, m, cb, enc, x.shape, x.dtype, relu=True)
+    assert tc.tc_get_status(ctx) == 0
+    tc.tc_force_exact_path(ctx, 0)
+    # (neighbouring bf16 numbers for at most 0.1 % of the values: the parity cases' cap)
+    a, b = got.float(), want.float()
+    assert bool(((a - b).abs() <= 2.0 ** -7 * b.abs() + 1e-6 * float(b.abs().max())).all())
+    assert float((a != b).double().mean()) <= 1e-3
+    m.close(); cb.close()
