@@ -80,61 +80,6 @@ __host__ __device__ inline SmemLayout smem_layout(int c, int k, const Plan &pl)
 constexpr float kMagic = 12582912.0f;
 constexpr uint32_t kMagicBits = 0x4B400000u;
 
-// Bit writer into shared memory, words kStep bytes apart.  A word is stored (plain, predicated store)
-// by the writer that supplies its last bit, nothing at or past `limit`; bits that other writers own
-// in that word are zero in the stored value.  What is left after the last full word -- a
-// writer's tail -- is merged afterwards with one shared-memory OR per writer (finish()), behind a
-// barrier, so that it cannot be overwritten by the store of the word's last writer.  A put adds fewer
-// than 32 bits (the pending count stays below 32 between puts).
-template <int kStep>
-struct SmemBitWriter {
-    uint32_t addr, limit;      // shared addresses: of the word being filled, past the last word
-    uint32_t lo, hi;           // pending bits, right-aligned in hi:lo (bits above `pending` are stale)
-    int pending;
-    __device__ __forceinline__ void init(uint32_t base_addr, uint32_t end_addr, unsigned int bitpos)
-    {
-        addr = base_addr + (bitpos >> 5) * (uint32_t)kStep;
-        limit = end_addr;
-        pending = (int)(bitpos & 31u);
-        lo = hi = 0;
-    }
-    __device__ __forceinline__ void put(uint32_t code, int len)
-    {
-        // hi:lo <<= len; lo |= code; pending += len; if (pending >= 32) { store bits
-        // [pending-32, pending) of hi:lo; addr += step; pending -= 32; }  (the funnel shift takes
-        // its amount modulo 32, so `pending` itself serves as pending - 32)
-        asm volatile(
-            "{\n\t.reg .pred p, q;\n\t.reg .b32 t, o;\n\t"
-            "shf.l.wrap.b32 %1, %0, %1, %5;\n\t"
-            "shl.b32 t, %0, %5;\n\t"
-            "or.b32 %0, t, %4;\n\t"
-            "add.s32 %2, %2, %5;\n\t"
-            "setp.ge.s32 p, %2, 32;\n\t"
-            "setp.lt.and.u32 q, %3, %6, p;\n\t"
-            "shf.r.wrap.b32 o, %0, %1, %2;\n\t"
-            "@q st.shared.u32 [%3], o;\n\t"
-            "@p add.s32 %3, %3, %7;\n\t"
-            "@p add.s32 %2, %2, -32;\n\t}"
-            : "+r"(lo), "+r"(hi), "+r"(pending), "+r"(addr)
-            : "r"(code), "r"(len), "r"(limit), "n"(kStep));
-    }
-    // 32 bits at once: the pending count stays
-    __device__ __forceinline__ void put_word(uint32_t bits)
-    {
-        const uint32_t out = __funnelshift_r(bits, lo, pending);       // the pending bits, then the first of the new ones
-        if (addr < limit) asm volatile("st.shared.u32 [%0], %1;" ::"r"(addr), "r"(out) : "memory");
-        addr += kStep;
-        lo = bits;
-        hi = 0;
-    }
-    // call after a barrier that follows every writer's puts
-    __device__ __forceinline__ void finish()
-    {
-        const uint32_t out = pending > 0 ? (lo << (32 - pending)) : 0u;
-        if (out && addr < limit) asm volatile("red.shared.or.b32 [%0], %1;" ::"r"(addr), "r"(out) : "memory");
-    }
-};
-
 // Sinks of a thread's codes that are not written to shared memory: only counted, or packed into global memory.
 struct CountSink {
     unsigned int bits;

@@ -141,16 +141,18 @@ __global__ void __launch_bounds__(kPx * kOut) reconstruct_kernel(DecodeArgs a, c
 // K / parts consecutive coefficients (a multiple of 8, so that a thread fetches its symbols in 8-byte
 // pieces and a chunk -- one of 1, 2 or 4 runs of a pixel -- is a whole number of thread runs).
 // Code lengths first (the lookups of a run are independent loads), then the bit offsets -- runs
-// inside a pixel, pixels inside the tile -- then every thread packs its run into zeroed words in
-// shared memory with an atomic OR at its ends, while the tile's place in the stream is found by
-// look-back; the words leave 16 bytes at a time.  A tile that does not fit the staging buffer is packed
-// into zeroed global memory.  Same stream, chunk lengths and tile offsets as the
+// inside a pixel, pixels inside the tile -- then every thread packs its run into words in
+// shared memory (whole words by plain stores, its tail by an atomic OR), then the tile's place in the
+// stream is found by look-back and the words leave 16 bytes at a time.  A tile that does not fit the
+// staging buffer is packed into zeroed global memory.  Same stream, chunk lengths and tile offsets as the
 // one-thread-per-pixel coder.
 // What bounds it: instructions, about ten per symbol, and for few tiles the one block's latency -- hence
-// up to eight threads a pixel and a per-layer table in shared memory (960x7x7 x 128: 45 us with four
-// threads, tables and packed words in global memory, 13 like this).
+// up to eight threads a pixel, a per-layer table in shared memory and two codes a piece (960x7x7 x 128
+// from a cold cache: 45 us with four threads, tables and packed words in global memory, 42 staged with an
+// atomic OR a word, 22 like this).
 constexpr int kMaxParts = 8;
 
+template <bool kPerLayer>
 __global__ void __launch_bounds__(TC_TILE_PIXELS * kMaxParts) pack_symbols_kernel(EncodeArgs a, const uint8_t *sym, int parts, long long first_tile,
                                                                                   unsigned int staging_bytes)
 {
@@ -164,9 +166,8 @@ __global__ void __launch_bounds__(TC_TILE_PIXELS * kMaxParts) pack_symbols_kerne
     extern __shared__ __align__(16) uint32_t s_words[];
     const int t = threadIdx.x;
     const int nsym = 1 << a.bits;
-    const bool per_layer = a.groups == 1;
     if (t == 0) s_tile = (long long)atomicAdd(a.ticket, 1u);
-    if (per_layer)
+    if constexpr (kPerLayer)
         for (int i = t; i < nsym; i += blockDim.x) s_enc[i] = __ldg(a.enc + i);
     __syncthreads();
     const long long tile = s_tile;
@@ -178,12 +179,13 @@ __global__ void __launch_bounds__(TC_TILE_PIXELS * kMaxParts) pack_symbols_kerne
     // code << 8 | length of the symbol in byte b of w, coefficient j
     auto entry = [&](uint32_t w, int b, int j) {
         const uint32_t q = (w >> (8 * b)) & 0xffu;
-        return per_layer ? s_enc[q] : __ldg(a.enc + j * nsym + q);
+        if constexpr (kPerLayer) return s_enc[q];
+        else return __ldg(a.enc + j * nsym + q);
     };
 
     unsigned int my_bits = 0;
     if (valid)
-#pragma unroll 2
+#pragma unroll 4
         for (int i = 0; i < run; i += 8) {
             const uint2 v = __ldg(reinterpret_cast<const uint2 *>(src + i));
 #pragma unroll
@@ -237,13 +239,12 @@ __global__ void __launch_bounds__(TC_TILE_PIXELS * kMaxParts) pack_symbols_kerne
             }
         }
     };
-    auto pack = [&](uint32_t *words, unsigned long long at) {
-        if (!valid) return;
-        BitWriter w;
-        w.init(words, at);
+    auto pack = [&](auto &w) {
+        uint2 next = __ldg(reinterpret_cast<const uint2 *>(src));
 #pragma unroll 1
         for (int i = 0; i < run; i += 8) {
-            const uint2 v = __ldg(reinterpret_cast<const uint2 *>(src + i));
+            const uint2 v = next;
+            if (i + 8 < run) next = __ldg(reinterpret_cast<const uint2 *>(src + i + 8));
 #pragma unroll
             for (int b = 0; b < 8; b += 2) {                  // two codes a piece, at most 24 bits
                 const uint32_t x = b < 4 ? v.x : v.y;
@@ -251,13 +252,18 @@ __global__ void __launch_bounds__(TC_TILE_PIXELS * kMaxParts) pack_symbols_kerne
                 w.put(((e0 >> 8) << (e1 & 0xffu)) | (e1 >> 8), (int)((e0 & 0xffu) + (e1 & 0xffu)));
             }
         }
-        w.finish();
     };
     const unsigned int n16 = (unsigned int)(padded >> 7);
     if (staged) {
-        for (unsigned int i = t; i < n16; i += blockDim.x) reinterpret_cast<uint4 *>(s_words)[i] = make_uint4(0u, 0u, 0u, 0u);
+        // every word below tile_bits / 32 is stored by the writer of its last bit; the rest starts as zero
+        const unsigned int first_open = tile_bits >> 5, end_word = n16 * 4;
+        const uint32_t words = (uint32_t)__cvta_generic_to_shared(s_words);
+        if (t < end_word - first_open) s_words[first_open + t] = 0u;
+        SmemBitWriter<4> w;
+        w.init(words, words + end_word * 4u, my_off);
+        if (valid) pack(w);
         __syncthreads();
-        pack(s_words, my_off);
+        if (valid) w.finish();
         resolve();
         __syncthreads();
         if (!s_write_ok) return;
@@ -270,7 +276,12 @@ __global__ void __launch_bounds__(TC_TILE_PIXELS * kMaxParts) pack_symbols_kerne
         uint4 *dst = reinterpret_cast<uint4 *>(a.stream + (s_base >> 5));
         for (unsigned int i = t; i < n16; i += blockDim.x) dst[i] = make_uint4(0u, 0u, 0u, 0u);
         __syncthreads();
-        pack(a.stream, s_base + my_off);
+        if (valid) {
+            BitWriter w;
+            w.init(a.stream, s_base + my_off);
+            pack(w);
+            w.finish();
+        }
     }
 }
 
@@ -326,16 +337,65 @@ struct AheadReader {
     }
 };
 
+// The same over a segment staged in shared memory, without a branch: `used` counts the bits taken since the
+// window last moved on by a word.
+struct StagedReader {
+    uint32_t next, end;          // shared addresses
+    uint32_t hi, lo, ahead, used;
+
+    __device__ __forceinline__ uint32_t fetch()
+    {
+        uint32_t v = 0;
+        if (next < end) asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(next));
+        next += 4;
+        return v;
+    }
+    __device__ __forceinline__ void init(uint32_t base, unsigned int bitpos, uint32_t end_addr)
+    {
+        next = base + (bitpos >> 5) * 4u;
+        end = end_addr;
+        const uint32_t w0 = fetch(), w1 = fetch();
+        ahead = fetch();
+        used = bitpos & 31u;
+        hi = __funnelshift_l(w1, w0, used);
+        lo = w1 << used;
+    }
+    __device__ __forceinline__ void skip(uint32_t nbits)
+    {
+        hi = __funnelshift_l(lo, hi, nbits);
+        lo = __funnelshift_l(0u, lo, nbits);
+        used += nbits;
+    }
+    __device__ __forceinline__ void refill()
+    {
+        asm volatile(
+            "{\n\t.reg .pred p, q;\n\t.reg .b32 t, u;\n\t"
+            "setp.ge.u32 p, %3, 32;\n\t"
+            "setp.lt.and.u32 q, %4, %5, p;\n\t"
+            "shf.l.wrap.b32 t, %2, 0, %3;\n\t"      // ahead >> (32 - (used - 32)); the shifts take their amount modulo 32
+            "shf.l.wrap.b32 u, 0, %2, %3;\n\t"
+            "@p or.b32 %0, %0, t;\n\t"
+            "@p or.b32 %1, %1, u;\n\t"
+            "@p add.u32 %3, %3, -32;\n\t"
+            "@p mov.b32 %2, 0;\n\t"
+            "@q ld.shared.u32 %2, [%4];\n\t"
+            "@p add.u32 %4, %4, 4;\n\t}"
+            : "+r"(hi), "+r"(lo), "+r"(ahead), "+r"(used), "+r"(next) : "r"(end));
+    }
+};
+
 // What bounds it: the chain length -> shift -> length of a chunk's symbols, with a handful of warps on
 // the chip (a 256x14x14 map has two tiles).  Per-layer tables are staged in shared memory; of
 // per-channel codes the bounds are (K x 48 bytes, read ahead of the symbol), the symbols come from
-// global memory off the chain.  The threads of a warp walk the same run of coefficients of
-// neighbouring pixels, and symbols leave 16 bytes at a time.  Measured with the inverse transform
-// and the launches, 256x14x14 at 6 bits: 64.5 us with a 2^12-entry table per channel in global
-// memory and a byte stored per symbol,
-// 40 us with the loop unrolled over sixteen symbols (16 KB of code, fetched once per launch).
+// global memory off the chain.  The tile's segment is staged too: read from global memory, a word
+// ahead or not, any lane's refill waits for the last lane's load, which is in the same register.  The
+// threads of a warp walk the same run of coefficients of neighbouring pixels, and symbols leave
+// eight at a time.  256x14x14 f32 at 6 bits, with the inverse transform and the launches: 64.5 us with a
+// 2^12-entry table per channel in global memory and a byte stored per symbol, 40 with bounds, 35 with the
+// staged segment.
 template <bool kOperand>
-__global__ void __launch_bounds__(kUnpackThreads) unpack_symbols_kernel(DecodeArgs a, void *out, long long first_tile)
+__global__ void __launch_bounds__(kUnpackThreads) unpack_symbols_kernel(DecodeArgs a, void *out, long long first_tile, unsigned int table_bytes,
+                                                                         unsigned int segment_bytes)
 {
     __shared__ unsigned int s_warp_sums[kUnpackThreads / 32];
     __shared__ unsigned int s_start[kUnpackThreads];
@@ -360,6 +420,11 @@ __global__ void __launch_bounds__(kUnpackThreads) unpack_symbols_kernel(DecodeAr
         if (t == 0) tc_dev_set_status(a.status, TC_ERR_CORRUPT_STREAM);
         return;
     }
+    const bool staged = end - base <= (unsigned long long)segment_bytes * 8ull;
+    const uint32_t seg = (uint32_t)__cvta_generic_to_shared(s_tables) + table_bytes;
+    if (staged)
+        for (unsigned int i = t; i < (unsigned int)((end - base) >> 7); i += blockDim.x)
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(seg + i * 16u), "l"(reinterpret_cast<const uint4 *>(a.stream + (base >> 5)) + i) : "memory");
     const int chunks_per_tile = a.splits * TC_TILE_PIXELS / a.chunk_pixels;      // at most 512
     // where every chunk of the tile starts: the lengths of its earlier chunks
     const long long scan_ch = tile * chunks_per_tile + t;
@@ -371,6 +436,7 @@ __global__ void __launch_bounds__(kUnpackThreads) unpack_symbols_kernel(DecodeAr
         if (lane >= d) inc += up;
     }
     if (lane == 31) s_warp_sums[warp] = inc;
+    asm volatile("cp.async.wait_all;" ::: "memory");
     __syncthreads();
     unsigned int off_t = inc - len_t;
     for (int w = 0; w < warp; ++w) off_t += s_warp_sums[w];
@@ -383,9 +449,7 @@ __global__ void __launch_bounds__(kUnpackThreads) unpack_symbols_kernel(DecodeAr
     if (t >= chunks_per_tile || ch >= a.n_chunks) return;
     const unsigned int want = a.chunk_len[ch], off = s_start[in_tile];
     bool bad = base + off + want > end;
-    if (!bad) {
-        AheadReader r;
-        r.init(a.stream, base + off, end);
+    auto walk = [&](auto &r) {
         unsigned int used = 0;
         const int run = a.k / a.splits, j_first = part * run;
         const int first_px = a.splits > 1 ? t % TC_TILE_PIXELS : t * a.chunk_pixels;
@@ -438,6 +502,15 @@ __global__ void __launch_bounds__(kUnpackThreads) unpack_symbols_kernel(DecodeAr
             }
         }
         if (used != want) bad = true;
+    };
+    if (!bad && staged) {
+        StagedReader r;
+        r.init(seg, off, seg + (uint32_t)((end - base) >> 3));
+        walk(r);
+    } else if (!bad) {
+        AheadReader r;
+        r.init(a.stream, base + off, end);
+        walk(r);
     }
     if (bad) tc_dev_set_status(a.status, TC_ERR_CORRUPT_STREAM);
 }
@@ -480,8 +553,9 @@ tc_status tc_launch_pack_symbols(const EncodeArgs &a, const uint8_t *sym, long l
     if (parts == 0 || ((uintptr_t)sym & 7u) != 0) return TC_ERR_UNSUPPORTED;
     // staging for four bits per symbol, at most 96 KB: two blocks of 1024 threads still fit an SM
     const unsigned int staging = (unsigned int)std::min<long long>((long long)a.k * TC_TILE_PIXELS / 2, 96 * 1024);
-    if (cudaFuncSetAttribute(pack_symbols_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024) != cudaSuccess) return TC_ERR_CUDA;
-    pack_symbols_kernel<<<(unsigned int)(end_tile - first_tile), TC_TILE_PIXELS * parts, staging, s>>>(a, sym, parts, first_tile, staging);
+    void (*kernel)(EncodeArgs, const uint8_t *, int, long long, unsigned int) = a.groups == 1 ? pack_symbols_kernel<true> : pack_symbols_kernel<false>;
+    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024) != cudaSuccess) return TC_ERR_CUDA;
+    kernel<<<(unsigned int)(end_tile - first_tile), TC_TILE_PIXELS * parts, staging, s>>>(a, sym, parts, first_tile, staging);
     return cudaGetLastError() == cudaSuccess ? TC_OK : TC_ERR_CUDA;
 }
 
@@ -491,10 +565,12 @@ static tc_status launch_unpack(const DecodeArgs &a, void *out, long long first_t
     if (end_tile <= first_tile) return TC_OK;
     const int chunks = a.splits * TC_TILE_PIXELS / a.chunk_pixels;
     if (chunks > kUnpackThreads) return TC_ERR_UNSUPPORTED;
-    const size_t smem = a.groups == 1 ? ((size_t)4 << a.lut_bits) : (size_t)a.k * kCanonWords * 4;      // at most 48 KB
-    if (cudaFuncSetAttribute(unpack_symbols_kernel<kOperand>, cudaFuncAttributeMaxDynamicSharedMemorySize, TC_MAX_C * kCanonWords * 4) != cudaSuccess)
+    // beside the tables (at most 48 KB) room for a segment of three bits per symbol, at most 48 KB
+    const unsigned int tables = (unsigned int)(a.groups == 1 ? ((size_t)4 << a.lut_bits) : (size_t)a.k * kCanonWords * 4);
+    const unsigned int segment = (unsigned int)std::min<long long>((long long)a.k * TC_TILE_PIXELS * 3 / 8, 48 * 1024);
+    if (cudaFuncSetAttribute(unpack_symbols_kernel<kOperand>, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024) != cudaSuccess)
         return TC_ERR_CUDA;
-    unpack_symbols_kernel<kOperand><<<(unsigned int)(end_tile - first_tile), (chunks + 31) / 32 * 32, smem, s>>>(a, out, first_tile);
+    unpack_symbols_kernel<kOperand><<<(unsigned int)(end_tile - first_tile), (chunks + 31) / 32 * 32, tables + segment, s>>>(a, out, first_tile, tables, segment);
     return cudaGetLastError() == cudaSuccess ? TC_OK : TC_ERR_CUDA;
 }
 

@@ -11,7 +11,8 @@
 // coefficients (channels) of a tile, the units are dealt over all SMs, both operands arrive by
 // tiled TMA copies with 128-byte swizzle, and the coder's chunks run side by side over the chip.
 // The workspace traffic (2 bytes per value written and read) stays in the 126 MB L2 for the most part.
-// 576x14x14 x 128 decode: 108 -> 45 us; 960x7x7 x 128 encode: 135 -> 53 us.
+// 576x14x14 x 128: encode 132 -> 63 us, decode 108 -> 65;
+// 960x7x7 x 128: encode 140 -> 52, decode 140 -> 53; 512x7x7 x 64: encode 52 -> 30, decode 46 -> 27.
 //
 // Arithmetic as in the streaming kernels: bf16 products, fp32 accumulation over steps of 16 channels
 // (coefficients) in ascending order, the same quantiser and dequantiser expressions.
@@ -238,14 +239,36 @@ __global__ void __launch_bounds__(256) pixel_rows_kernel(const __nv_bfloat16 *x,
     __shared__ __nv_bfloat16 s[kTurn][kTurn + 2];             // [channel][pixel]; the padding keeps the column reads apart
     const int c0 = blockIdx.y * kTurn, t = threadIdx.x;
     const long long p0 = p_first + (long long)blockIdx.x * kTurn;
-    const int px = t & 63, cr = t >> 6;
-    const long long p = p0 + px;
-    if (p < p_end) {
-        const long long img = p / hw;
-        const __nv_bfloat16 *src = x + img * c * (long long)hw + (p - img * hw);
+    if ((hw & 3) == 0 && ((uintptr_t)x & 7u) == 0) {          // four pixels a load
+        const int px = (t & 15) * 4, cr = t >> 4;
+        const long long p = p0 + px;
+        if (p < p_end) {
+            const long long img = p / hw;
+            const __nv_bfloat16 *src = x + img * c * (long long)hw + (p - img * hw);
+            uint2 v[kTurn / 16];
 #pragma unroll
-        for (int i = 0; i < kTurn; i += 4)
-            if (c0 + cr + i < c) s[cr + i][px] = __ldg(src + (long long)(c0 + cr + i) * hw);
+            for (int i = 0; i < kTurn / 16; ++i)
+                if (c0 + cr + 16 * i < c) v[i] = __ldg(reinterpret_cast<const uint2 *>(src + (long long)(c0 + cr + 16 * i) * hw));
+#pragma unroll
+            for (int i = 0; i < kTurn / 16; ++i) {
+                uint32_t *d = reinterpret_cast<uint32_t *>(&s[cr + 16 * i][px]);
+                d[0] = v[i].x;
+                d[1] = v[i].y;
+            }
+        }
+    } else {
+        const int px = t & 63, cr = t >> 6;
+        const long long p = p0 + px;
+        if (p < p_end) {
+            const long long img = p / hw;
+            const __nv_bfloat16 *src = x + img * c * (long long)hw + (p - img * hw);
+            __nv_bfloat16 v[kTurn / 4];
+#pragma unroll
+            for (int i = 0; i < kTurn / 4; ++i)
+                if (c0 + cr + 4 * i < c) v[i] = __ldg(src + (long long)(c0 + cr + 4 * i) * hw);
+#pragma unroll
+            for (int i = 0; i < kTurn / 4; ++i) s[cr + 4 * i][px] = v[i];
+        }
     }
     __syncthreads();
     // a thread writes 8 channels of a pixel (16 bytes); C is a multiple of 16
