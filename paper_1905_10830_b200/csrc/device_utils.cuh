@@ -249,10 +249,13 @@ __device__ __forceinline__ uint32_t canon_length(uint32_t window, const CanonBou
     return 1u + (uint32_t)__popc(s);
 }
 // its symbol: `bases` = the code's half-words of bases, `sorted` = its symbols in code order
+__device__ __forceinline__ uint32_t canon_place(uint32_t window, uint32_t len, const uint16_t *bases)
+{
+    return ((uint32_t)bases[len - 1] + (window >> (32 - len))) & 0xffffu;
+}
 __device__ __forceinline__ uint32_t canon_symbol(uint32_t window, uint32_t len, const uint16_t *bases, const uint8_t *sorted)
 {
-    const uint32_t place = ((uint32_t)bases[len - 1] + (window >> (32 - len))) & 0xffffu;
-    return __ldg(sorted + place);
+    return __ldg(sorted + canon_place(window, len, bases));
 }
 
 // MSB-first reader over 32-bit words with a 64-bit window held in two registers.  Words at or

@@ -386,14 +386,17 @@ struct StagedReader {
 
 // What bounds it: the chain length -> shift -> length of a chunk's symbols, with a handful of warps on
 // the chip (a 256x14x14 map has two tiles).  Per-layer tables are staged in shared memory; of
-// per-channel codes the bounds are (K x 48 bytes, read ahead of the symbol), the symbols come from
-// global memory off the chain.  The tile's segment is staged too: read from global memory, a word
+// per-channel codes the bounds are (K x 48 bytes, read ahead of the symbol), and the symbols in code
+// order while they are few.  These are looked up eight at a time behind the chain: one lookup after each
+// symbol made every step wait for a load from L2, which shares its scoreboard with the chain's
+// shared-memory loads.  The tile's segment is staged too: read from global memory, a word
 // ahead or not, any lane's refill waits for the last lane's load, which is in the same register.  The
 // threads of a warp walk the same run of coefficients of neighbouring pixels, and symbols leave
 // eight at a time.  256x14x14 f32 at 6 bits, with the inverse transform and the launches: 64.5 us with a
 // 2^12-entry table per channel in global memory and a byte stored per symbol, 40 with bounds, 35 with the
-// staged segment.
-template <bool kOperand>
+// staged segment, 27 with the symbols looked up behind the chain and per-channel codes in an
+// instantiation of their own (the choice inside the loop kept the bounds from being read ahead).
+template <bool kOperand, bool kPerLayer>
 __global__ void __launch_bounds__(kUnpackThreads) unpack_symbols_kernel(DecodeArgs a, void *out, long long first_tile, unsigned int table_bytes,
                                                                          unsigned int segment_bytes)
 {
@@ -402,17 +405,25 @@ __global__ void __launch_bounds__(kUnpackThreads) unpack_symbols_kernel(DecodeAr
     extern __shared__ __align__(16) unsigned char s_tables[];   // the per-layer table, or the bounds and bases of every channel's code
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
     const int lut_size = 1 << a.lut_bits, nsym = 1 << a.bits;
-    const bool per_layer = a.groups == 1;
     // per-layer table: value << 16 | length, the value being the symbol or its centred bf16
     uint32_t *s_lut = reinterpret_cast<uint32_t *>(s_tables), *s_canon = s_lut;
     auto value = [&](uint32_t q) { return kOperand ? __float_as_uint((float)((int)q - a.center)) >> 16 : q; };
-    if (per_layer)
+    const uint32_t tables = (uint32_t)__cvta_generic_to_shared(s_tables);
+    const uint32_t s_sorted = tables + (uint32_t)a.k * kCanonWords * 4u;          // of per-channel codes, when there is room
+    const bool sorted_staged = !kPerLayer && table_bytes > (unsigned int)a.k * kCanonWords * 4u;
+    auto stage = [&](uint32_t dst, const void *src, unsigned int n16) {           // pieces of 16 bytes
+        for (unsigned int i = t; i < n16; i += blockDim.x)
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + i * 16u), "l"(reinterpret_cast<const uint4 *>(src) + i) : "memory");
+    };
+    if constexpr (kPerLayer) {
         for (int i = t; i < lut_size; i += blockDim.x) {
             const uint32_t e = __ldg(a.lut + i);
             s_lut[i] = (value(e >> 8) << 16) | (e & 0xffu);
         }
-    else
-        for (int i = t; i < a.k * kCanonWords; i += blockDim.x) s_canon[i] = a.canon[i];
+    } else {
+        stage(tables, a.canon, (unsigned int)a.k * kCanonWords / 4u);
+        if (sorted_staged) stage(s_sorted, a.sorted, (unsigned int)(a.k * nsym) / 16u);
+    }
     const long long tile = first_tile + blockIdx.x;
     const unsigned long long base = a.tile_off[tile], end = a.tile_off[tile + 1];
     const bool tile_ok = (base & 127ull) == 0 && (end & 127ull) == 0 && base <= end && end <= a.stream_bits;
@@ -421,10 +432,8 @@ __global__ void __launch_bounds__(kUnpackThreads) unpack_symbols_kernel(DecodeAr
         return;
     }
     const bool staged = end - base <= (unsigned long long)segment_bytes * 8ull;
-    const uint32_t seg = (uint32_t)__cvta_generic_to_shared(s_tables) + table_bytes;
-    if (staged)
-        for (unsigned int i = t; i < (unsigned int)((end - base) >> 7); i += blockDim.x)
-            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(seg + i * 16u), "l"(reinterpret_cast<const uint4 *>(a.stream + (base >> 5)) + i) : "memory");
+    const uint32_t seg = tables + table_bytes;
+    if (staged) stage(seg, a.stream + (base >> 5), (unsigned int)((end - base) >> 7));
     const int chunks_per_tile = a.splits * TC_TILE_PIXELS / a.chunk_pixels;      // at most 512
     // where every chunk of the tile starts: the lengths of its earlier chunks
     const long long scan_ch = tile * chunks_per_tile + t;
@@ -460,7 +469,7 @@ __global__ void __launch_bounds__(kUnpackThreads) unpack_symbols_kernel(DecodeAr
             for (int i = 0; i < kN; ++i) {
                 if ((i & 1) == 0) r.refill();
                 uint32_t len;
-                if (per_layer) {
+                if constexpr (kPerLayer) {
                     const uint32_t e = s_lut[r.hi >> (32 - a.lut_bits)];
                     len = e & 0xffu;
                     v[i] = e >> 16;
@@ -468,10 +477,22 @@ __global__ void __launch_bounds__(kUnpackThreads) unpack_symbols_kernel(DecodeAr
                     const uint32_t *c = s_canon + (j + i) * kCanonWords;
                     const CanonBounds cb{*reinterpret_cast<const uint4 *>(c), *reinterpret_cast<const uint2 *>(c + 4)};
                     len = canon_length(r.hi, cb);
-                    v[i] = value(canon_symbol(r.hi, len, reinterpret_cast<const uint16_t *>(c + 6), a.sorted + (size_t)(j + i) * nsym));
+                    v[i] = canon_place(r.hi, len, reinterpret_cast<const uint16_t *>(c + 6));
                 }
                 r.skip(len);
                 used += len;
+            }
+            if constexpr (!kPerLayer) {
+                if (sorted_staged) {
+#pragma unroll
+                    for (int i = 0; i < kN; ++i)
+                        asm volatile("ld.shared.u8 %0, [%1];" : "=r"(v[i]) : "r"(s_sorted + (uint32_t)((j + i) * nsym) + v[i]));
+                } else {
+#pragma unroll
+                    for (int i = 0; i < kN; ++i) v[i] = __ldg(a.sorted + (size_t)(j + i) * nsym + v[i]);
+                }
+#pragma unroll
+                for (int i = 0; i < kN; ++i) v[i] = value(v[i]);
             }
         };
         const bool by8 = a.k % 8 == 0 && run % 8 == 0;
@@ -559,27 +580,38 @@ tc_status tc_launch_pack_symbols(const EncodeArgs &a, const uint8_t *sym, long l
     return cudaGetLastError() == cudaSuccess ? TC_OK : TC_ERR_CUDA;
 }
 
+// Symbols of per-channel codes up to this size are staged with every tile; more of them cost a tile longer than
+// the lookups in L2 that they save.
+constexpr unsigned int kSortedStaged = 16 * 1024;
+
 template <bool kOperand>
-static tc_status launch_unpack(const DecodeArgs &a, void *out, long long first_tile, long long end_tile, cudaStream_t s)
+static tc_status launch_unpack(const DecodeArgs &a, void *out, long long first_tile, long long end_tile, int sm_count, cudaStream_t s)
 {
     if (end_tile <= first_tile) return TC_OK;
     const int chunks = a.splits * TC_TILE_PIXELS / a.chunk_pixels;
     if (chunks > kUnpackThreads) return TC_ERR_UNSUPPORTED;
-    // beside the tables (at most 48 KB) room for a segment of three bits per symbol, at most 48 KB
-    const unsigned int tables = (unsigned int)(a.groups == 1 ? ((size_t)4 << a.lut_bits) : (size_t)a.k * kCanonWords * 4);
+    // beside the tables (at most 48 KB and the symbols) room for a segment of three bits per symbol, at most 48 KB
+    unsigned int tables = (unsigned int)(a.groups == 1 ? ((size_t)4 << a.lut_bits) : (size_t)a.k * kCanonWords * 4);
+    if (a.groups != 1) {
+        const unsigned int sorted = (unsigned int)a.k << a.bits;                   // bytes
+        if (sorted % 16 == 0 && ((uintptr_t)a.sorted & 15u) == 0 && sorted <= kSortedStaged) tables += sorted;
+    }
     const unsigned int segment = (unsigned int)std::min<long long>((long long)a.k * TC_TILE_PIXELS * 3 / 8, 48 * 1024);
-    if (cudaFuncSetAttribute(unpack_symbols_kernel<kOperand>, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024) != cudaSuccess)
-        return TC_ERR_CUDA;
-    unpack_symbols_kernel<kOperand><<<(unsigned int)(end_tile - first_tile), (chunks + 31) / 32 * 32, tables + segment, s>>>(a, out, first_tile, tables, segment);
+    void (*kernel)(DecodeArgs, void *, long long, unsigned int, unsigned int) =
+        a.groups == 1 ? unpack_symbols_kernel<kOperand, true> : unpack_symbols_kernel<kOperand, false>;
+    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 112 * 1024) != cudaSuccess) return TC_ERR_CUDA;
+    // a block of few chunks has more threads for staging while all blocks are resident at once
+    const int threads = (chunks + 31) / 32 * 32, least = end_tile - first_tile < 4 * sm_count ? 256 : 32;
+    kernel<<<(unsigned int)(end_tile - first_tile), std::max(threads, least), tables + segment, s>>>(a, out, first_tile, tables, segment);
     return cudaGetLastError() == cudaSuccess ? TC_OK : TC_ERR_CUDA;
 }
 
-tc_status tc_launch_unpack_symbols(const DecodeArgs &a, uint8_t *sym, cudaStream_t s)
+tc_status tc_launch_unpack_symbols(const tc_ctx *ctx, const DecodeArgs &a, uint8_t *sym, cudaStream_t s)
 {
-    return launch_unpack<false>(a, sym, 0, a.n_tiles, s);
+    return launch_unpack<false>(a, sym, 0, a.n_tiles, ctx->sm_count, s);
 }
 
-tc_status tc_launch_unpack_operand(const DecodeArgs &a, void *operand, long long first_tile, long long end_tile, cudaStream_t s)
+tc_status tc_launch_unpack_operand(const tc_ctx *ctx, const DecodeArgs &a, void *operand, long long first_tile, long long end_tile, cudaStream_t s)
 {
-    return launch_unpack<true>(a, operand, first_tile, end_tile, s);
+    return launch_unpack<true>(a, operand, first_tile, end_tile, ctx->sm_count, s);
 }

@@ -209,7 +209,6 @@ tc_status finish_model(tc_model *m)
         // and for the decoder: the transposed basis in boxes of 128 channel rows x 64 coefficients
         m->has_basis_t_map = false;
         if (k % 16 == 0) m->has_basis_t_map = tc_tensor_map_sw128(&m->basis_t_map, m->d_basis_t_bf16, c, k, 128);
-        if (c % 16 == 0) m->has_basis_gemm_map = tc_tensor_map_sw128(&m->basis_gemm_map, m->d_basis_bf16, k, c, 32);
     }
     TC_CUDA(cudaStreamSynchronize(nullptr));
     return TC_OK;
@@ -862,7 +861,6 @@ tc_status tc_encode_with_scratch(tc_ctx *ctx, const tc_model *m, const tc_codebo
     a.status = ctx->d_status; a.clamped = clamped; a.emit = 1;
     a.basis_bf16 = m->d_basis_bf16; a.basis_core = m->d_basis_core; a.enc_bias = m->d_enc_bias; a.tmu32 = m->d_tmu32;
     a.basis_map = m->has_basis_map ? &m->basis_map : nullptr;
-    a.basis_gemm_map = m->has_basis_gemm_map ? &m->basis_gemm_map : nullptr;
     a.hist = hist; a.hist_modal = m->center;
     a.modal = cb->modal;
     a.blk_bits = m->blk_bits.data(); a.blk_odd = m->blk_odd.data();
@@ -875,8 +873,8 @@ tc_status tc_encode_with_scratch(tc_ctx *ctx, const tc_model *m, const tc_codebo
     if (ctx->force_exact != 1 && x->dtype == TC_BF16 && tc_encode_wide_supported(ctx, a)) {   // wide layers, unaligned rows
         ctx->last_encode_path = 3;
         // with workspace: projection as a tiled product, the entropy coder as a kernel of its own
-        if (work && !debug && wide_encode(ctx, m, x) && a.basis_gemm_map && tc_pack_symbols_parts(a) > 0)
-            return tc_launch_encode_wide_gemm(ctx, a, a.basis_gemm_map, work, s);
+        if (work && !debug && wide_encode(ctx, m, x) && m->has_basis_t_map && tc_pack_symbols_parts(a) > 0)
+            return tc_launch_encode_wide_gemm(ctx, a, work, s);
         return tc_launch_encode_wide(ctx, a, s);
     }
     if (ctx->force_exact != 1 && x->dtype == TC_BF16 && x->c % 2 == 0) {      // shapes the tensor-core kernel does not take
@@ -956,18 +954,23 @@ tc_status tc_encode(tc_ctx *ctx, const tc_model *m, const tc_codebook *cb, const
                                   ctx->scratch, work ? (char *)ctx->scratch + lookback : nullptr, s);
 }
 
-static bool wide_decode(const tc_ctx *ctx, const tc_model *m, const tc_tensor *x_hat)
+// bf16 tensors decoded by the entropy decoder and the tiled product in kernels of their own: wide layers, and per-channel
+// code tables, whose symbols cost so much more to find than the products that the warps of one resident block
+// cannot keep up (80x27x19 x 37 6 bits: 40 -> 23 us, 256x14x14 x 64 4 bits 51 -> 26, x 1024 265 -> 165, 8 bits
+// 284 -> 189, 64x56x56 x 64 114 -> 52, 16x112x112 x 128 690 -> 182, 96x112x112 x 64 437 -> 229)
+static bool wide_decode(const tc_ctx *ctx, const tc_model *m, const tc_codebook *cb, const tc_tensor *x_hat)
 {
-    return x_hat->dtype == TC_BF16 && ctx->force_exact != 1 && m->c % 16 == 0 && m->k % 16 == 0 && m->c > 256;
+    return x_hat->dtype == TC_BF16 && ctx->force_exact != 1 && m->c % 16 == 0 && m->k % 16 == 0 &&
+           (m->c > 256 || (cb->groups != 1 && ctx->force_exact == 0));
 }
 
 // Bytes of workspace a decode of `x_hat` may need: the centred symbols of a wide layer, or the symbols of
 // a tensor of few tiles on the exact kernels (whether that route is taken is decided at launch).
-static size_t decode_scratch_bytes(const tc_ctx *ctx, const tc_model *m, const tc_tensor *x_hat)
+static size_t decode_scratch_bytes(const tc_ctx *ctx, const tc_model *m, const tc_codebook *cb, const tc_tensor *x_hat)
 {
     const long long pixels = (long long)x_hat->n * x_hat->h * x_hat->w;
     const long long n_tiles = (pixels + TC_TILE_PIXELS - 1) / TC_TILE_PIXELS;
-    if (wide_decode(ctx, m, x_hat)) return tc_decode_wide_workspace(m->k, n_tiles);
+    if (wide_decode(ctx, m, cb, x_hat)) return tc_decode_wide_workspace(m->k, n_tiles);
     return n_tiles < (long long)kExactParallelTilesPerSm * ctx->sm_count ? (((size_t)pixels * m->k + 255) & ~(size_t)255) : 0;
 }
 
@@ -1020,12 +1023,14 @@ static tc_status decode_with_scratch(tc_ctx *ctx, const tc_model *m, const tc_co
         resident = false;
     if (resident) {
         ctx->last_decode_path = 1;
+        if (sym_scratch && wide_decode(ctx, m, cb, x_hat) && a.basis_t_map)
+            return tc_launch_decode_wide_gemm(ctx, a, sym_scratch, (cudaStream_t)cuda_stream);
         return tc_launch_decode_tc(ctx, a, (cudaStream_t)cuda_stream);
     }
     if (ctx->force_exact != 1 && x_hat->dtype == TC_BF16 && tc_decode_wide_supported(ctx, a)) {   // wide layers
         ctx->last_decode_path = 3;
         // with workspace: the entropy decoder as a kernel of its own, the inverse as a tiled product
-        if (sym_scratch && wide_decode(ctx, m, x_hat) && a.basis_t_map)
+        if (sym_scratch && wide_decode(ctx, m, cb, x_hat) && a.basis_t_map)
             return tc_launch_decode_wide_gemm(ctx, a, sym_scratch, (cudaStream_t)cuda_stream);
         return tc_launch_decode_wide(ctx, a, (cudaStream_t)cuda_stream);
     }
@@ -1037,7 +1042,7 @@ static tc_status decode_with_scratch(tc_ctx *ctx, const tc_model *m, const tc_co
     if (sym_scratch && a.n_tiles < (long long)kExactParallelTilesPerSm * ctx->sm_count) {
         // few pixels: the per-pixel kernel only decodes the symbols (into the context's arena), the
         // inverse transform runs with one thread per (pixel, channel) -- same arithmetic, same results
-        if ((st = tc_launch_unpack_symbols(a, sym_scratch, (cudaStream_t)cuda_stream)) != TC_OK) return st;
+        if ((st = tc_launch_unpack_symbols(ctx, a, sym_scratch, (cudaStream_t)cuda_stream)) != TC_OK) return st;
         return tc_launch_reconstruct(a, x_hat->dtype, sym_scratch, (cudaStream_t)cuda_stream);
     }
     return tc_launch_decode_simt(ctx, a, x_hat->dtype, (cudaStream_t)cuda_stream);
@@ -1049,7 +1054,7 @@ tc_status tc_decode(tc_ctx *ctx, const tc_model *m, const tc_codebook *cb, const
 {
     if (!ctx || !m || !valid_tensor(x_hat)) return TC_ERR_INVALID_ARG;
     DeviceGuard guard(ctx->device);
-    const size_t scratch = decode_scratch_bytes(ctx, m, x_hat);
+    const size_t scratch = decode_scratch_bytes(ctx, m, cb, x_hat);
     if (scratch) {
         const tc_status st = ensure_scratch(ctx, scratch);
         if (st != TC_OK) return st;
@@ -1163,7 +1168,7 @@ tc_status tc_decode_many(tc_ctx *ctx, const tc_decode_item *items, int32_t n_ite
         if (pixels > 0 && (!it.stream || !it.chunk_len || !it.tile_off || ((uintptr_t)it.stream & 15u) != 0 ||
                            ((uintptr_t)it.chunk_len & 3u) != 0))
             return TC_ERR_INVALID_ARG;
-        symbols_bytes[i] = decode_scratch_bytes(ctx, it.model, it.x_hat);
+        symbols_bytes[i] = decode_scratch_bytes(ctx, it.model, it.codebook, it.x_hat);
         symbols_at[i] = total;
         total += symbols_bytes[i];
         work[i] = (double)pixels * it.x_hat->c;

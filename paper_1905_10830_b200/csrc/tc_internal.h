@@ -71,8 +71,6 @@ struct tc_model {
     float *d_tmu32 = nullptr;               // [k]  (T mu)_j
     CUtensorMap basis_map;                  // d_basis_bf16 as a [k][c] tensor, boxes of 256 rows x 32 channels, 64-byte swizzle
     bool has_basis_map = false;
-    CUtensorMap basis_gemm_map;             // d_basis_bf16 in boxes of 32 rows x 64 channels, 128-byte swizzle
-    bool has_basis_gemm_map = false;
     CUtensorMap basis_t_map;                // d_basis_t_bf16 as a [c][k] tensor, boxes of 128 channel rows x 64 coefficients, 128-byte swizzle
     bool has_basis_t_map = false;
 };
@@ -103,7 +101,6 @@ struct EncodeArgs {
     const double *mean64;       // [c]
     const __nv_bfloat16 *basis_bf16;   // [k][c]  (tensor-core path)
     const __nv_bfloat16 *basis_core;   // basis_bf16 in 8 x 8 core matrices, or null
-    const CUtensorMap *basis_gemm_map; // HOST pointer to the map of basis_bf16 for the tiled product, or null
     const CUtensorMap *basis_map;      // HOST pointer to the model's tensor map of basis_bf16, or null
     const float *enc_bias;      // [k]  -(T mu + lo)_j / step
     const float *tmu32;         // [k]  (T mu)_j
@@ -179,16 +176,16 @@ tc_status tc_launch_encode_simt_fp32(const tc_ctx *ctx, const EncodeArgs &a, cud
 tc_status tc_launch_decode_simt_fp32(const tc_ctx *ctx, const DecodeArgs &a, cudaStream_t s);
 tc_status tc_launch_project_quantise(const EncodeArgs &a, int dtype, uint8_t *sym, cudaStream_t s);
 int tc_pack_symbols_parts(const EncodeArgs &a);
-tc_status tc_launch_unpack_symbols(const DecodeArgs &a, uint8_t *sym, cudaStream_t s);
+tc_status tc_launch_unpack_symbols(const tc_ctx *ctx, const DecodeArgs &a, uint8_t *sym, cudaStream_t s);
 tc_status tc_launch_pack_symbols(const EncodeArgs &a, const uint8_t *sym, long long first_tile, long long end_tile, cudaStream_t s);
-tc_status tc_launch_unpack_operand(const DecodeArgs &a, void *operand, long long first_tile, long long end_tile, cudaStream_t s);
+tc_status tc_launch_unpack_operand(const tc_ctx *ctx, const DecodeArgs &a, void *operand, long long first_tile, long long end_tile, cudaStream_t s);
 
 // Wide layers with workspace (wide_gemm.cu).  The workspace of one tensor is at most about kWideWorkspace:
 // larger tensors are worked through in passes.
 constexpr size_t kWideWorkspace = 64ull << 20;
 size_t tc_encode_wide_workspace(int c, int k, long long n_tiles);
 size_t tc_decode_wide_workspace(int k, long long n_tiles);
-tc_status tc_launch_encode_wide_gemm(const tc_ctx *ctx, const EncodeArgs &a, const CUtensorMap *basis_map, void *workspace, cudaStream_t s);
+tc_status tc_launch_encode_wide_gemm(const tc_ctx *ctx, const EncodeArgs &a, void *workspace, cudaStream_t s);
 tc_status tc_launch_decode_wide_gemm(const tc_ctx *ctx, const DecodeArgs &a, void *workspace, cudaStream_t s);
 // Tensor map of a bf16 matrix [rows][cols] (cols a multiple of 8): boxes of 64 columns x box_rows rows, 128-byte swizzle.
 bool tc_tensor_map_sw128(CUtensorMap *map, const void *base, long long rows, int cols, int box_rows);

@@ -11,8 +11,10 @@
 // coefficients (channels) of a tile, the units are dealt over all SMs, both operands arrive by
 // tiled TMA copies with 128-byte swizzle, and the coder's chunks run side by side over the chip.
 // The workspace traffic (2 bytes per value written and read) stays in the 126 MB L2 for the most part.
-// 576x14x14 x 128: encode 132 -> 63 us, decode 108 -> 65;
-// 960x7x7 x 128: encode 140 -> 52, decode 140 -> 53; 512x7x7 x 64: encode 52 -> 30, decode 46 -> 27.
+// 576x14x14 x 128: encode 132 -> 62 us, decode 108 -> 62;
+// 960x7x7 x 128: encode 140 -> 52, decode 140 -> 49; 512x7x7 x 64: encode 52 -> 30, decode 46 -> 27.
+// The product itself is bound by the operands' way from L2 (48 KB per 64 of the depth, at about 32 bytes a cycle
+// and SM); one copy per operand and stage, since a producer thread issues one in about 100 cycles.
 //
 // Arithmetic as in the streaming kernels: bf16 products, fp32 accumulation over steps of 16 channels
 // (coefficients) in ascending order, the same quantiser and dequantiser expressions.
@@ -29,9 +31,10 @@ constexpr int kStageA = 128 * kPanelK * 2;                    // 16 KB: 128 rows
 constexpr int kMaxN = 256;                                    // columns of an accumulator
 constexpr int kStageBytes = kStageA + kMaxN * kPanelK * 2;    // 48 KB
 constexpr int kStages = 4;
-constexpr int kBoxRows = 32;                                  // rows of a TMA box of the second operand
-constexpr int kEpiWarps = 8, kProducerWarp = 8, kMmaWarp = 9;
-constexpr int kThreads = 10 * 32;
+// four epilogue warps per quarter of TMEM's lanes: with two, layers of few channels (little to multiply) took longer
+// (80x27x19 x 37 decode 25.2 against 23.3 us, 16x112x112 x 128 206 against 182)
+constexpr int kEpiWarps = 16, kProducerWarp = kEpiWarps, kMmaWarp = kEpiWarps + 1;
+constexpr int kThreads = (kEpiWarps + 2) * 32;
 constexpr int kTrWarpBytes = 2048;                            // decode: transpose block of a warp, 32 channel rows x 32 pixels
 constexpr int kTmemCols = 512;
 constexpr float kMagic = 12582912.0f;                         // 1.5 * 2^23: adding it rounds to the nearest integer, ties to even
@@ -90,7 +93,7 @@ __global__ void __launch_bounds__(kThreads, 1) wide_gemm_kernel(GemmArgs a, cons
                     const uint32_t bar = smem_u32(&s_full[s]), dst = ring + (uint32_t)s * kStageBytes;
                     mbar_arrive_expect_tx(bar, (uint32_t)(kStageA + a.n_cols * kPanelK * 2));
                     tma_load_2d(dst, &map_a, kp * kPanelK, row_a, bar);
-                    for (int b = 0; b < a.n_cols; b += kBoxRows) tma_load_2d(dst + kStageA + b * (kPanelK * 2), &map_b, kp * kPanelK, row_b + b, bar);
+                    tma_load_2d(dst + kStageA, &map_b, kp * kPanelK, row_b, bar);
                     if (++s == kStages) { s = 0; phase ^= 1u; }
                 }
             }
@@ -122,8 +125,10 @@ __global__ void __launch_bounds__(kThreads, 1) wide_gemm_kernel(GemmArgs a, cons
         }
         if (!alive && issuer) tc_dev_set_status(a.status, TC_ERR_TIMEOUT);
     } else {
-        const int set = warp >> 2, wq = warp & 3;              // which half of the columns; TMEM lane quarter
-        const int half = a.n_cols / 2;                         // a multiple of 16 (decode: of 32)
+        const int set = warp >> 2, wq = warp & 3;              // which part of the columns; TMEM lane quarter
+        constexpr int kSets = kEpiWarps / 4, kStep = kEncode ? 16 : 32;
+        const int part = (a.n_cols / kStep + kSets - 1) / kSets * kStep;
+        const int col_first = set * part, cols = min(part, a.n_cols - col_first);     // none for the last sets of a narrow unit
         bool alive = true;
         int n = 0;
         for (long long u = blockIdx.x; u < a.units; u += gridDim.x, ++n) {
@@ -131,10 +136,10 @@ __global__ void __launch_bounds__(kThreads, 1) wide_gemm_kernel(GemmArgs a, cons
             if (!mbar_wait(smem_u32(&s_tfull[acc]), (uint32_t)((n >> 1) & 1))) { alive = false; break; }
             tc_fence_after_sync();
             const int tile = tile_of(u), block = block_of(u, tile);
-            const uint32_t trow = tmem_base + acc * kMaxN + ((uint32_t)(wq * 32) << 16) + set * half;
+            const uint32_t trow = tmem_base + acc * kMaxN + ((uint32_t)(wq * 32) << 16) + col_first;
             if constexpr (kEncode) {
                 const long long p = a.p_first + (long long)tile * 128 + wq * 32 + lane;
-                const int j_first = block * a.n_cols + set * half, j_end = min(j_first + half, a.k);
+                const int j_first = block * a.n_cols + col_first, j_end = min(j_first + cols, a.k);
                 uint8_t *dst = a.sym + (p - a.p_first) * a.k;
 #pragma unroll 1
                 for (int j0 = j_first; j0 < j_end; j0 += 16) {
@@ -161,7 +166,7 @@ __global__ void __launch_bounds__(kThreads, 1) wide_gemm_kernel(GemmArgs a, cons
                 const float floor_v = a.relu ? 0.f : __int_as_float((int)0xff800000u);
                 const int rows = min(32, a.c - (block * 128 + wq * 32));          // channel rows of this warp that exist
                 const uint32_t tb = ring + kStages * kStageBytes + (uint32_t)warp * kTrWarpBytes;
-                const long long p_unit = a.p_first + (long long)tile * a.n_cols + set * half;
+                const long long p_unit = a.p_first + (long long)tile * a.n_cols + col_first;
                 const bool vec = (a.hw & 3) == 0 && ((uintptr_t)a.xhat & 7u) == 0;
                 // This lane's pixels in a pass of 32: four of them with 8-byte stores (eight lanes a row, four
                 // rows an instruction), else one (a row an instruction).
@@ -170,7 +175,7 @@ __global__ void __launch_bounds__(kThreads, 1) wide_gemm_kernel(GemmArgs a, cons
                 long long img = p / a.hw;
                 int sp = (int)(p - img * a.hw);
                 const long long img_stride = (long long)a.c * a.hw;
-                for (int c0 = 0; c0 < half && rows > 0; c0 += 32, p += 32) {
+                for (int c0 = 0; c0 < cols && rows > 0; c0 += 32, p += 32) {
                     uint32_t r[32];
                     tmem_ld_32x32b_x32(trow + c0, r);
                     tmem_ld_wait(r);
@@ -331,7 +336,7 @@ size_t tc_decode_wide_workspace(int k, long long n_tiles)
     return up((size_t)tiles_per_pass(n_tiles, (size_t)TC_TILE_PIXELS * 2 * k) * TC_TILE_PIXELS * k * 2);
 }
 
-tc_status tc_launch_encode_wide_gemm(const tc_ctx *ctx, const EncodeArgs &a, const CUtensorMap *basis_map, void *workspace, cudaStream_t s)
+tc_status tc_launch_encode_wide_gemm(const tc_ctx *ctx, const EncodeArgs &a, void *workspace, cudaStream_t s)
 {
     const long long per_pass = tiles_per_pass(a.n_tiles, (size_t)TC_TILE_PIXELS * (2 * a.c + a.k));
     __nv_bfloat16 *rows = (__nv_bfloat16 *)workspace;
@@ -341,13 +346,13 @@ tc_status tc_launch_encode_wide_gemm(const tc_ctx *ctx, const EncodeArgs &a, con
         const long long p0 = t0 * TC_TILE_PIXELS, p1 = t1 * TC_TILE_PIXELS < a.pixels ? t1 * TC_TILE_PIXELS : a.pixels;
         const dim3 grid((unsigned int)((p1 - p0 + kTurn - 1) / kTurn), (unsigned int)((a.c + kTurn - 1) / kTurn));
         pixel_rows_kernel<<<grid, 256, 0, s>>>((const __nv_bfloat16 *)a.x, a.c, a.hw, p0, p1, rows);
-        CUtensorMap map_x;
-        if (!tc_tensor_map_sw128(&map_x, rows, p1 - p0, a.c, 128)) return TC_ERR_CUDA;
         GemmArgs g{};
         g.n_panels = (a.c + kPanelK - 1) / kPanelK;
         g.k_depth = a.c;
         g.n_cols = best_columns(t1 - t0, a.k, ctx->sm_count);
         g.blocks = (a.k + g.n_cols - 1) / g.n_cols;
+        CUtensorMap map_x, map_t;
+        if (!tc_tensor_map_sw128(&map_x, rows, p1 - p0, a.c, 128) || !tc_tensor_map_sw128(&map_t, a.basis_bf16, a.k, a.c, g.n_cols)) return TC_ERR_CUDA;
         g.units = (t1 - t0) * g.blocks;
         g.p_first = p0; g.p_end = p1;
         g.k = a.k;
@@ -356,7 +361,7 @@ tc_status tc_launch_encode_wide_gemm(const tc_ctx *ctx, const EncodeArgs &a, con
         g.bias = a.enc_bias;
         g.sym = sym;
         g.status = a.status;
-        tc_status st = launch_gemm<true>(ctx, g, map_x, *basis_map, s);
+        tc_status st = launch_gemm<true>(ctx, g, map_x, map_t, s);
         if (st != TC_OK) return st;
         if ((st = tc_launch_pack_symbols(a, sym, t0, t1, s)) != TC_OK) return st;
     }
@@ -370,10 +375,8 @@ tc_status tc_launch_decode_wide_gemm(const tc_ctx *ctx, const DecodeArgs &a, voi
     for (long long t0 = 0; t0 < a.n_tiles; t0 += per_pass) {
         const long long t1 = t0 + per_pass < a.n_tiles ? t0 + per_pass : a.n_tiles;
         const long long p0 = t0 * TC_TILE_PIXELS, p1 = t1 * TC_TILE_PIXELS < a.pixels ? t1 * TC_TILE_PIXELS : a.pixels;
-        tc_status st = tc_launch_unpack_operand(a, q, t0, t1, s);
+        tc_status st = tc_launch_unpack_operand(ctx, a, q, t0, t1, s);
         if (st != TC_OK) return st;
-        CUtensorMap map_q;
-        if (!tc_tensor_map_sw128(&map_q, q, p1 - p0, a.k, kBoxRows)) return TC_ERR_CUDA;
         GemmArgs g{};
         g.n_panels = (a.k + kPanelK - 1) / kPanelK;
         g.k_depth = a.k;
@@ -382,6 +385,8 @@ tc_status tc_launch_decode_wide_gemm(const tc_ctx *ctx, const DecodeArgs &a, voi
         g.n_cols = kMaxN;
         while (g.n_cols > 64 && ((p1 - p0 + g.n_cols - 1) / g.n_cols) * g.blocks < ctx->sm_count) g.n_cols /= 2;
         g.units = ((p1 - p0 + g.n_cols - 1) / g.n_cols) * g.blocks;
+        CUtensorMap map_q;
+        if (!tc_tensor_map_sw128(&map_q, q, p1 - p0, a.k, g.n_cols)) return TC_ERR_CUDA;
         g.p_first = p0; g.p_end = p1;
         g.c = a.c; g.hw = a.hw; g.relu = a.relu;
         g.step = (float)(a.step * a.basis_scale);              // the operand holds basis / basis_scale
