@@ -31,6 +31,12 @@ __device__ __forceinline__ unsigned long long global_timer_ns()
     return t;
 }
 
+// Kernels of one call that follow each other (launch_chained): a kernel lets the next one start setting up as soon
+// as all its own blocks run, and waits for what the one before it wrote -- and everything before that -- ahead of the
+// first access to it.  What it reads from the kernel before it does not go through the read-only path.
+__device__ __forceinline__ void chain_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 __device__ __forceinline__ double load_as_double(const float *p) { return (double)__ldg(p); }
 __device__ __forceinline__ double load_as_double(const __nv_bfloat16 *p)
 {

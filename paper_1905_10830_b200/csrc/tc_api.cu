@@ -836,7 +836,8 @@ static size_t encode_work_bytes(const tc_ctx *ctx, const tc_model *m, const tc_t
 
 // Argument block and kernel choice shared by tc_encode and tc_encode_noalloc.  `scratch` is
 // kEncodeScratchHeader bytes (ticket counter) followed by one 64-bit look-back word per tile;
-// it is cleared on the stream here, whoever owns it.
+// it is cleared on the stream here, whoever owns it: by the kernel that precedes the entropy coder where
+// there is one (a memset of its own costs the stream two microseconds).
 tc_status tc_encode_with_scratch(tc_ctx *ctx, const tc_model *m, const tc_codebook *cb, const tc_tensor *x, int chunk_pixels,
                                  int splits, void *stream_out, size_t capacity, uint16_t *chunk_len, uint64_t *tile_off,
                                  const tc_debug_out *debug, void *scratch, void *work, cudaStream_t s,
@@ -844,9 +845,7 @@ tc_status tc_encode_with_scratch(tc_ctx *ctx, const tc_model *m, const tc_codebo
 {
     const long long pixels = (long long)x->n * x->h * x->w;
     const long long n_tiles = (pixels + TC_TILE_PIXELS - 1) / TC_TILE_PIXELS;
-    if (!scratch_is_zero)
-        TC_CUDA(cudaMemsetAsync(scratch, 0, kEncodeScratchHeader + (size_t)n_tiles * sizeof(unsigned long long), s));
-
+    const size_t scratch_bytes = kEncodeScratchHeader + (size_t)n_tiles * sizeof(unsigned long long);
     EncodeArgs a{};
     a.x = x->data; a.n = x->n; a.c = x->c; a.hw = x->h * x->w; a.k = m->k; a.bits = m->bits; a.groups = cb->groups;
     a.pixels = pixels; a.n_tiles = n_tiles; a.chunk_pixels = chunk_pixels; a.splits = splits;
@@ -868,17 +867,22 @@ tc_status tc_encode_with_scratch(tc_ctx *ctx, const tc_model *m, const tc_codebo
         return TC_ERR_UNSUPPORTED;                      // only the resident-basis tensor-core encoder counts symbols
     if ((ctx->force_exact == 0 || ctx->force_exact == 3) && x->dtype == TC_BF16 && tc_encode_tc_supported(ctx, a)) {
         ctx->last_encode_path = 1;
+        if (!scratch_is_zero) TC_CUDA(cudaMemsetAsync(scratch, 0, scratch_bytes, s));
         return tc_launch_encode_tc(ctx, a, s);
     }
     if (ctx->force_exact != 1 && x->dtype == TC_BF16 && tc_encode_wide_supported(ctx, a)) {   // wide layers, unaligned rows
         ctx->last_encode_path = 3;
         // with workspace: projection as a tiled product, the entropy coder as a kernel of its own
-        if (work && !debug && wide_encode(ctx, m, x) && m->has_basis_t_map && tc_pack_symbols_parts(a) > 0)
+        if (work && !debug && wide_encode(ctx, m, x) && m->has_basis_t_map && tc_pack_symbols_parts(a) > 0) {
+            a.clear_words = scratch_is_zero ? 0 : (long long)(scratch_bytes / 8);
             return tc_launch_encode_wide_gemm(ctx, a, work, s);
+        }
+        if (!scratch_is_zero) TC_CUDA(cudaMemsetAsync(scratch, 0, scratch_bytes, s));
         return tc_launch_encode_wide(ctx, a, s);
     }
     if (ctx->force_exact != 1 && x->dtype == TC_BF16 && x->c % 2 == 0) {      // shapes the tensor-core kernel does not take
         ctx->last_encode_path = 2;
+        if (!scratch_is_zero) TC_CUDA(cudaMemsetAsync(scratch, 0, scratch_bytes, s));
         return tc_launch_encode_simt_fp32(ctx, a, s);
     }
     ctx->last_encode_path = 0;
@@ -886,12 +890,14 @@ tc_status tc_encode_with_scratch(tc_ctx *ctx, const tc_model *m, const tc_codebo
         uint8_t *const sym_scratch = (uint8_t *)work;
         // few pixels: projection and quantiser with one thread per (pixel, coefficient), then the
         // entropy coder of the per-pixel kernel on those symbols -- same arithmetic, same results
+        a.clear_words = scratch_is_zero ? 0 : (long long)(scratch_bytes / 8);
         tc_status st = tc_launch_project_quantise(a, x->dtype, sym_scratch, s);
         if (st != TC_OK) return st;
         if (tc_pack_symbols_parts(a) > 0 && ((uintptr_t)sym_scratch & 15u) == 0)
-            return tc_launch_pack_symbols(a, sym_scratch, 0, a.n_tiles, s);      // several threads per pixel code the symbols
+            return tc_launch_pack_symbols(ctx, a, sym_scratch, 0, a.n_tiles, s);      // several threads per pixel code the symbols
         a.sym_in = sym_scratch;
-    }
+    } else if (!scratch_is_zero)
+        TC_CUDA(cudaMemsetAsync(scratch, 0, scratch_bytes, s));
     return tc_launch_encode_simt(ctx, a, x->dtype, s);
 }
 

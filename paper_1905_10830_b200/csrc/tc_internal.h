@@ -6,6 +6,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <utility>
 #include <vector>
 
 #include "tc.h"
@@ -114,7 +115,8 @@ struct EncodeArgs {
     float *dbg_coef;            // nullable
     uint8_t *dbg_sym;           // nullable
     unsigned long long *tile_state;   // look-back state, zeroed before launch
-    unsigned int *ticket;             // zeroed before launch
+    unsigned int *ticket;             // zeroed before launch; the look-back words follow it
+    long long clear_words;            // 64-bit words from `ticket` on that the first of several kernels zeroes (0: they are zero)
     unsigned int *status;
     unsigned long long *clamped;      // nullable: counts coefficients outside the range
     int emit;                         // 0: symbols only (statistics mode)
@@ -161,6 +163,22 @@ struct DecodeArgs {
 };
 
 // ---- encode dispatch shared by tc_encode and tc_encode_noalloc (tc_api.cu) --------------------
+// Launch of a kernel that may be set up while the one before it in the stream still runs (it calls chain_wait).  Only for
+// the second and later kernels of one call: its first one starts after everything that the stream held before.
+template <typename... P, typename... A>
+inline cudaError_t launch_chained(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A &&...args)
+{
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = s;
+    cfg.attrs = &attr; cfg.numAttrs = 1;
+    const cudaError_t err = cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...);
+    if (err != cudaSuccess) cudaGetLastError();
+    return err;
+}
+
 constexpr size_t kEncodeScratchHeader = 64;   // ticket counter, padded; the per-tile look-back words follow
 tc_status tc_encode_with_scratch(tc_ctx *ctx, const tc_model *m, const tc_codebook *cb, const tc_tensor *x, int chunk_pixels,
                                  int splits, void *stream_out, size_t capacity, uint16_t *chunk_len, uint64_t *tile_off,
@@ -177,7 +195,7 @@ tc_status tc_launch_decode_simt_fp32(const tc_ctx *ctx, const DecodeArgs &a, cud
 tc_status tc_launch_project_quantise(const EncodeArgs &a, int dtype, uint8_t *sym, cudaStream_t s);
 int tc_pack_symbols_parts(const EncodeArgs &a);
 tc_status tc_launch_unpack_symbols(const tc_ctx *ctx, const DecodeArgs &a, uint8_t *sym, cudaStream_t s);
-tc_status tc_launch_pack_symbols(const EncodeArgs &a, const uint8_t *sym, long long first_tile, long long end_tile, cudaStream_t s);
+tc_status tc_launch_pack_symbols(const tc_ctx *ctx, const EncodeArgs &a, const uint8_t *sym, long long first_tile, long long end_tile, cudaStream_t s);
 tc_status tc_launch_unpack_operand(const tc_ctx *ctx, const DecodeArgs &a, void *operand, long long first_tile, long long end_tile, cudaStream_t s);
 
 // Wide layers with workspace (wide_gemm.cu).  The workspace of one tensor is at most about kWideWorkspace:

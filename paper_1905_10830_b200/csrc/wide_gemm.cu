@@ -66,6 +66,7 @@ __global__ void __launch_bounds__(kThreads, 1) wide_gemm_kernel(GemmArgs a, cons
     __shared__ uint32_t s_tmem_base;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const uint32_t ring = smem_u32(smem);
+    chain_next();
     if (tid == 0) {
         for (int s = 0; s < kStages; ++s) { mbar_init(smem_u32(&s_full[s]), 1); mbar_init(smem_u32(&s_empty[s]), 1); }
         for (int b = 0; b < 2; ++b) { mbar_init(smem_u32(&s_tfull[b]), 1); mbar_init(smem_u32(&s_tempty[b]), kEpiWarps); }
@@ -76,6 +77,7 @@ __global__ void __launch_bounds__(kThreads, 1) wide_gemm_kernel(GemmArgs a, cons
     __syncthreads();
     tc_fence_after_sync();
     const uint32_t tmem_base = s_tmem_base;
+    chain_wait();                                             // the workspace operand; earlier readers of what this kernel writes
     // rows of both operands of unit u: (tile of pixels, block)
     auto tile_of = [&](long long u) { return (int)(u / a.blocks); };
     auto block_of = [&](long long u, int tile) { return (int)(u - (long long)tile * a.blocks); };
@@ -239,8 +241,12 @@ __global__ void __launch_bounds__(kThreads, 1) wide_gemm_kernel(GemmArgs a, cons
 // Pixels [p_first, p_end) of an NCHW tensor as rows of C channels.  A block turns 64 pixels x 64 channels
 // through shared memory; bound by the memory it moves (L2 for the rows).
 constexpr int kTurn = 64;
-__global__ void __launch_bounds__(256) pixel_rows_kernel(const __nv_bfloat16 *x, int c, int hw, long long p_first, long long p_end, __nv_bfloat16 *rows)
+__global__ void __launch_bounds__(256) pixel_rows_kernel(const __nv_bfloat16 *x, int c, int hw, long long p_first, long long p_end, __nv_bfloat16 *rows,
+                                                         unsigned long long *clear, long long clear_words)
 {
+    chain_next();
+    for (long long i = (blockIdx.y * (long long)gridDim.x + blockIdx.x) * 256 + threadIdx.x; i < clear_words; i += (long long)gridDim.x * gridDim.y * 256)
+        clear[i] = 0ull;                                      // the coder's look-back state
     __shared__ __nv_bfloat16 s[kTurn][kTurn + 2];             // [channel][pixel]; the padding keeps the column reads apart
     const int c0 = blockIdx.y * kTurn, t = threadIdx.x;
     const long long p0 = p_first + (long long)blockIdx.x * kTurn;
@@ -308,8 +314,7 @@ tc_status launch_gemm(const tc_ctx *ctx, const GemmArgs &g, const CUtensorMap &m
     const size_t smem = (size_t)kStages * kStageBytes + (kEncode ? 0 : kEpiWarps * kTrWarpBytes);
     if (cudaFuncSetAttribute(wide_gemm_kernel<kEncode>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return TC_ERR_CUDA;
     const unsigned int grid = (unsigned int)(g.units < ctx->sm_count ? g.units : ctx->sm_count);
-    wide_gemm_kernel<kEncode><<<grid, kThreads, smem, s>>>(g, map_a, map_b);
-    return cudaGetLastError() == cudaSuccess ? TC_OK : TC_ERR_CUDA;
+    return launch_chained(wide_gemm_kernel<kEncode>, grid, kThreads, smem, s, g, map_a, map_b) == cudaSuccess ? TC_OK : TC_ERR_CUDA;
 }
 
 // Tiles of a pass over a tensor whose workspace would exceed the cap.
@@ -345,7 +350,8 @@ tc_status tc_launch_encode_wide_gemm(const tc_ctx *ctx, const EncodeArgs &a, voi
         const long long t1 = t0 + per_pass < a.n_tiles ? t0 + per_pass : a.n_tiles;
         const long long p0 = t0 * TC_TILE_PIXELS, p1 = t1 * TC_TILE_PIXELS < a.pixels ? t1 * TC_TILE_PIXELS : a.pixels;
         const dim3 grid((unsigned int)((p1 - p0 + kTurn - 1) / kTurn), (unsigned int)((a.c + kTurn - 1) / kTurn));
-        pixel_rows_kernel<<<grid, 256, 0, s>>>((const __nv_bfloat16 *)a.x, a.c, a.hw, p0, p1, rows);
+        pixel_rows_kernel<<<grid, 256, 0, s>>>((const __nv_bfloat16 *)a.x, a.c, a.hw, p0, p1, rows, (unsigned long long *)a.ticket,
+                                               t0 == 0 ? a.clear_words : 0);
         GemmArgs g{};
         g.n_panels = (a.c + kPanelK - 1) / kPanelK;
         g.k_depth = a.c;
@@ -363,7 +369,7 @@ tc_status tc_launch_encode_wide_gemm(const tc_ctx *ctx, const EncodeArgs &a, voi
         g.status = a.status;
         tc_status st = launch_gemm<true>(ctx, g, map_x, map_t, s);
         if (st != TC_OK) return st;
-        if ((st = tc_launch_pack_symbols(a, sym, t0, t1, s)) != TC_OK) return st;
+        if ((st = tc_launch_pack_symbols(ctx, a, sym, t0, t1, s)) != TC_OK) return st;
     }
     return TC_OK;
 }
