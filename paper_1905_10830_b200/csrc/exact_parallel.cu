@@ -611,7 +611,7 @@ tc_status tc_launch_reconstruct(const DecodeArgs &a, int dtype, const uint8_t *s
     if (a.pixels <= 0) return TC_OK;
     const dim3 block(kPx, kRows), grid((unsigned int)((a.pixels + kPx - 1) / kPx), (unsigned int)((a.c + kOut - 1) / kOut));
     void (*kernel)(DecodeArgs, const uint8_t *) = dtype == TC_F32 ? reconstruct_kernel<float> : reconstruct_kernel<__nv_bfloat16>;
-    return launch_chained(kernel, grid, block, 0, s, a, sym) == cudaSuccess ? TC_OK : TC_ERR_CUDA;
+    return launch_chained(a.alone, kernel, grid, block, 0, s, a, sym) == cudaSuccess ? TC_OK : TC_ERR_CUDA;
 }
 
 // How many threads per pixel the parallel coder would use for K coefficients and `splits` chunks
@@ -641,8 +641,8 @@ tc_status tc_launch_pack_symbols(const tc_ctx *ctx, const EncodeArgs &a, const u
     // memory each -- small blocks that arrive early all pile onto the first SMs that have room (960x7x7 x 128, 49
     // blocks: 49 us unchained, 65 chained, 48 chained and spread; 64x56x56 f32 17.2 unchained, 14.9 chained and spread).
     // More blocks than that start when the SMs are free (80x27x19 x 37: 20 us, chained 26).
-    if (end_tile - first_tile <= ctx->sm_count)
-        return launch_chained(kernel, grid, block, std::max(staging, kSpreadBytes), s, a, sym, parts, first_tile, staging) == cudaSuccess ? TC_OK : TC_ERR_CUDA;
+    if (a.alone && end_tile - first_tile <= ctx->sm_count)
+        return launch_chained(true, kernel, grid, block, std::max(staging, kSpreadBytes), s, a, sym, parts, first_tile, staging) == cudaSuccess ? TC_OK : TC_ERR_CUDA;
     kernel<<<grid, block, staging, s>>>(a, sym, parts, first_tile, staging);
     return cudaGetLastError() == cudaSuccess ? TC_OK : TC_ERR_CUDA;
 }

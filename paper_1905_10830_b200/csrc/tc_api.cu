@@ -861,6 +861,7 @@ tc_status tc_encode_with_scratch(tc_ctx *ctx, const tc_model *m, const tc_codebo
     a.basis_bf16 = m->d_basis_bf16; a.basis_core = m->d_basis_core; a.enc_bias = m->d_enc_bias; a.tmu32 = m->d_tmu32;
     a.basis_map = m->has_basis_map ? &m->basis_map : nullptr;
     a.hist = hist; a.hist_modal = m->center;
+    a.alone = !scratch_is_zero;                         // tensors of a list share one cleared scratch and run on several streams
     a.modal = cb->modal;
     a.blk_bits = m->blk_bits.data(); a.blk_odd = m->blk_odd.data();
     if (hist && !((ctx->force_exact == 0 || ctx->force_exact == 3) && x->dtype == TC_BF16 && tc_encode_tc_supported(ctx, a)))
@@ -983,7 +984,7 @@ static size_t decode_scratch_bytes(const tc_ctx *ctx, const tc_model *m, const t
 // tc_decode with the symbol scratch named by the caller (decode_scratch_bytes of it, or nullptr)
 static tc_status decode_with_scratch(tc_ctx *ctx, const tc_model *m, const tc_codebook *cb, const void *stream, size_t stream_bytes,
                                      const uint16_t *chunk_len, const uint64_t *tile_off, const tc_encode_params *params,
-                                     const tc_tensor *x_hat, uint8_t *sym_scratch, void *cuda_stream)
+                                     const tc_tensor *x_hat, uint8_t *sym_scratch, bool alone, void *cuda_stream)
 {
     if (!ctx) return TC_ERR_INVALID_ARG;
     tc_status st = check_codec_args(m, cb, x_hat);
@@ -1005,6 +1006,7 @@ static tc_status decode_with_scratch(tc_ctx *ctx, const tc_model *m, const tc_co
     a.xhat = x_hat->data; a.status = ctx->d_status;
     a.lut32 = cb->d_lut32; a.canon = cb->d_canon; a.sorted = cb->d_sorted; a.basis_t_bf16 = m->d_basis_t_bf16; a.dec_bias = m->d_dec_bias; a.center = m->center;
     a.relu = (params && params->relu) ? 1 : 0;
+    a.alone = alone;
     a.basis_t_map = m->has_basis_t_map ? &m->basis_t_map : nullptr;
     a.modal = cb->modal;
     a.mean_tile_bytes = (params && params->mean_tile_bytes > 0) ? params->mean_tile_bytes : 0;
@@ -1066,7 +1068,7 @@ tc_status tc_decode(tc_ctx *ctx, const tc_model *m, const tc_codebook *cb, const
         if (st != TC_OK) return st;
     }
     return decode_with_scratch(ctx, m, cb, stream, stream_bytes, chunk_len, tile_off, params, x_hat,
-                               scratch ? (uint8_t *)ctx->scratch : nullptr, cuda_stream);
+                               scratch ? (uint8_t *)ctx->scratch : nullptr, true, cuda_stream);
 }
 
 // ---- several tensors per call --------------------------------------------------------------------
@@ -1192,7 +1194,7 @@ tc_status tc_decode_many(tc_ctx *ctx, const tc_decode_item *items, int32_t n_ite
         const tc_decode_item &it = items[i];
         st = decode_with_scratch(ctx, it.model, it.codebook, it.stream, it.stream_bytes, it.chunk_len, it.tile_off, it.params,
                                  it.x_hat, symbols_bytes[i] ? (uint8_t *)ctx->scratch + symbols_at[i] : nullptr,
-                                 ctx->many_streams[r % n_streams]);
+                                 false, ctx->many_streams[r % n_streams]);
         if (st != TC_OK && first_error == TC_OK) first_error = st;
     }
     for (int j = 0; j < n_streams; ++j) {

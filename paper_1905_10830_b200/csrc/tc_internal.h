@@ -116,6 +116,7 @@ struct EncodeArgs {
     uint8_t *dbg_sym;           // nullable
     unsigned long long *tile_state;   // look-back state, zeroed before launch
     unsigned int *ticket;             // zeroed before launch; the look-back words follow it
+    bool alone;                       // no other stream of this call (see launch_chained)
     long long clear_words;            // 64-bit words from `ticket` on that the first of several kernels zeroes (0: they are zero)
     unsigned int *status;
     unsigned long long *clamped;      // nullable: counts coefficients outside the range
@@ -145,6 +146,7 @@ struct DecodeArgs {
     const uint32_t *canon;              // [groups][kCanonWords], see tc_codebook
     const uint8_t *sorted;              // [groups][2^bits]
     const __nv_bfloat16 *basis_t_bf16;  // [c][k]
+    bool alone;                         // no other stream of this call (see launch_chained)
     const CUtensorMap *basis_t_map;     // HOST pointer to the model's tensor map of basis_t_bf16, or null
     const float *dec_bias;              // [c]
     int center;                         // subtracted from every symbol before the MMA
@@ -164,16 +166,18 @@ struct DecodeArgs {
 
 // ---- encode dispatch shared by tc_encode and tc_encode_noalloc (tc_api.cu) --------------------
 // Launch of a kernel that may be set up while the one before it in the stream still runs (it calls chain_wait).  Only for
-// the second and later kernels of one call: its first one starts after everything that the stream held before.
+// the second and later kernels of one call: its first one starts after everything that the stream held before.  Not with
+// other streams of the call at work (`early` false): a product's blocks that wait hold shared memory their kernels could
+// use (decode of a network's 16 layers 274 us, 250 without).
 template <typename... P, typename... A>
-inline cudaError_t launch_chained(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A &&...args)
+inline cudaError_t launch_chained(bool early, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A &&...args)
 {
     cudaLaunchAttribute attr{};
     attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr.val.programmaticStreamSerializationAllowed = 1;
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = s;
-    cfg.attrs = &attr; cfg.numAttrs = 1;
+    cfg.attrs = &attr; cfg.numAttrs = early ? 1 : 0;
     const cudaError_t err = cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...);
     if (err != cudaSuccess) cudaGetLastError();
     return err;

@@ -309,12 +309,12 @@ int best_columns(long long tiles, int k, int sm_count)
 }
 
 template <bool kEncode>
-tc_status launch_gemm(const tc_ctx *ctx, const GemmArgs &g, const CUtensorMap &map_a, const CUtensorMap &map_b, cudaStream_t s)
+tc_status launch_gemm(const tc_ctx *ctx, bool early, const GemmArgs &g, const CUtensorMap &map_a, const CUtensorMap &map_b, cudaStream_t s)
 {
     const size_t smem = (size_t)kStages * kStageBytes + (kEncode ? 0 : kEpiWarps * kTrWarpBytes);
     if (cudaFuncSetAttribute(wide_gemm_kernel<kEncode>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return TC_ERR_CUDA;
     const unsigned int grid = (unsigned int)(g.units < ctx->sm_count ? g.units : ctx->sm_count);
-    return launch_chained(wide_gemm_kernel<kEncode>, grid, kThreads, smem, s, g, map_a, map_b) == cudaSuccess ? TC_OK : TC_ERR_CUDA;
+    return launch_chained(early, wide_gemm_kernel<kEncode>, grid, kThreads, smem, s, g, map_a, map_b) == cudaSuccess ? TC_OK : TC_ERR_CUDA;
 }
 
 // Tiles of a pass over a tensor whose workspace would exceed the cap.
@@ -367,7 +367,7 @@ tc_status tc_launch_encode_wide_gemm(const tc_ctx *ctx, const EncodeArgs &a, voi
         g.bias = a.enc_bias;
         g.sym = sym;
         g.status = a.status;
-        tc_status st = launch_gemm<true>(ctx, g, map_x, map_t, s);
+        tc_status st = launch_gemm<true>(ctx, a.alone, g, map_x, map_t, s);
         if (st != TC_OK) return st;
         if ((st = tc_launch_pack_symbols(ctx, a, sym, t0, t1, s)) != TC_OK) return st;
     }
@@ -399,7 +399,7 @@ tc_status tc_launch_decode_wide_gemm(const tc_ctx *ctx, const DecodeArgs &a, voi
         g.bias = a.dec_bias;
         g.xhat = (__nv_bfloat16 *)a.xhat;
         g.status = a.status;
-        if ((st = launch_gemm<false>(ctx, g, *a.basis_t_map, map_q, s)) != TC_OK) return st;
+        if ((st = launch_gemm<false>(ctx, a.alone, g, *a.basis_t_map, map_q, s)) != TC_OK) return st;
     }
     return TC_OK;
 }
