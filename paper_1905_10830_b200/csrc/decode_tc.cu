@@ -688,7 +688,7 @@ tc_status tc_launch_decode_tc(const tc_ctx *ctx, const DecodeArgs &a, cudaStream
     args.smem_budget = ctx->max_smem_optin - 512;
     if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)l.total) != cudaSuccess)
         return TC_ERR_CUDA;
-    const unsigned int grid = (unsigned int)((a.n_tiles < ctx->sm_count) ? a.n_tiles : ctx->sm_count);
+    const unsigned int grid = (unsigned int)((a.n_tiles < a.sms) ? a.n_tiles : a.sms);
     kernel<<<grid, kThreads, l.total, s>>>(args);
     return cudaGetLastError() == cudaSuccess ? TC_OK : TC_ERR_CUDA;
 }

@@ -859,7 +859,7 @@ tc_status tc_launch_encode_tc(const tc_ctx *ctx, const EncodeArgs &a, cudaStream
                                                    : (runs ? pick_kernel<false, false, true>(debug, a.hist) : pick_kernel<false, false, false>(debug, a.hist));
     if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)l.total) != cudaSuccess)
         return TC_ERR_CUDA;
-    const unsigned int grid = (unsigned int)((a.n_tiles < ctx->sm_count) ? a.n_tiles : ctx->sm_count);
+    const unsigned int grid = (unsigned int)((a.n_tiles < a.sms) ? a.n_tiles : a.sms);
     EncodeArgs args = a;
     void *params[] = {&args, &pl};
     // cooperative launch: the grid must be co-resident, which is what makes the look-back safe

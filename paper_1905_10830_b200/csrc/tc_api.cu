@@ -113,7 +113,7 @@ tc_status ensure_scratch(tc_ctx *ctx, size_t bytes)
 {
     if (bytes <= ctx->scratch_bytes) return TC_OK;
     if (ctx->scratch) { TC_CUDA(cudaDeviceSynchronize()); cudaFree(ctx->scratch); ctx->scratch = nullptr; ctx->scratch_bytes = 0; }
-    size_t want = std::max<size_t>(bytes, 1 << 20);
+    size_t want = std::max<size_t>(bytes, 8 << 20);
     TC_CUDA(cudaMalloc(&ctx->scratch, want));
     ctx->scratch_bytes = want;
     return TC_OK;
@@ -361,7 +361,7 @@ void tc_destroy(tc_ctx *ctx)
         if (ctx->ev_out[i]) cudaEventDestroy(ctx->ev_out[i]);
     }
     if (ctx->chunk_bits) cudaFreeHost(ctx->chunk_bits);
-    for (int i = 0; i < 4; ++i) {
+    for (int i = 0; i < kManyStreams; ++i) {
         if (ctx->many_streams[i]) cudaStreamDestroy(ctx->many_streams[i]);
         if (ctx->many_join[i]) cudaEventDestroy(ctx->many_join[i]);
     }
@@ -841,10 +841,11 @@ static size_t encode_work_bytes(const tc_ctx *ctx, const tc_model *m, const tc_t
 tc_status tc_encode_with_scratch(tc_ctx *ctx, const tc_model *m, const tc_codebook *cb, const tc_tensor *x, int chunk_pixels,
                                  int splits, void *stream_out, size_t capacity, uint16_t *chunk_len, uint64_t *tile_off,
                                  const tc_debug_out *debug, void *scratch, void *work, cudaStream_t s,
-                                 unsigned long long *hist, unsigned long long *clamped, bool scratch_is_zero)
+                                 unsigned long long *hist, unsigned long long *clamped, int list_sms)
 {
     const long long pixels = (long long)x->n * x->h * x->w;
     const long long n_tiles = (pixels + TC_TILE_PIXELS - 1) / TC_TILE_PIXELS;
+    const bool scratch_is_zero = list_sms != 0;
     const size_t scratch_bytes = kEncodeScratchHeader + (size_t)n_tiles * sizeof(unsigned long long);
     EncodeArgs a{};
     a.x = x->data; a.n = x->n; a.c = x->c; a.hw = x->h * x->w; a.k = m->k; a.bits = m->bits; a.groups = cb->groups;
@@ -861,7 +862,8 @@ tc_status tc_encode_with_scratch(tc_ctx *ctx, const tc_model *m, const tc_codebo
     a.basis_bf16 = m->d_basis_bf16; a.basis_core = m->d_basis_core; a.enc_bias = m->d_enc_bias; a.tmu32 = m->d_tmu32;
     a.basis_map = m->has_basis_map ? &m->basis_map : nullptr;
     a.hist = hist; a.hist_modal = m->center;
-    a.alone = !scratch_is_zero;                         // tensors of a list share one cleared scratch and run on several streams
+    a.alone = list_sms == 0;
+    a.sms = list_sms ? list_sms : ctx->sm_count;
     a.modal = cb->modal;
     a.blk_bits = m->blk_bits.data(); a.blk_odd = m->blk_odd.data();
     if (hist && !((ctx->force_exact == 0 || ctx->force_exact == 3) && x->dtype == TC_BF16 && tc_encode_tc_supported(ctx, a)))
@@ -984,7 +986,7 @@ static size_t decode_scratch_bytes(const tc_ctx *ctx, const tc_model *m, const t
 // tc_decode with the symbol scratch named by the caller (decode_scratch_bytes of it, or nullptr)
 static tc_status decode_with_scratch(tc_ctx *ctx, const tc_model *m, const tc_codebook *cb, const void *stream, size_t stream_bytes,
                                      const uint16_t *chunk_len, const uint64_t *tile_off, const tc_encode_params *params,
-                                     const tc_tensor *x_hat, uint8_t *sym_scratch, bool alone, void *cuda_stream)
+                                     const tc_tensor *x_hat, uint8_t *sym_scratch, int list_sms, void *cuda_stream)
 {
     if (!ctx) return TC_ERR_INVALID_ARG;
     tc_status st = check_codec_args(m, cb, x_hat);
@@ -1006,7 +1008,8 @@ static tc_status decode_with_scratch(tc_ctx *ctx, const tc_model *m, const tc_co
     a.xhat = x_hat->data; a.status = ctx->d_status;
     a.lut32 = cb->d_lut32; a.canon = cb->d_canon; a.sorted = cb->d_sorted; a.basis_t_bf16 = m->d_basis_t_bf16; a.dec_bias = m->d_dec_bias; a.center = m->center;
     a.relu = (params && params->relu) ? 1 : 0;
-    a.alone = alone;
+    a.alone = list_sms == 0;
+    a.sms = list_sms ? list_sms : ctx->sm_count;
     a.basis_t_map = m->has_basis_t_map ? &m->basis_t_map : nullptr;
     a.modal = cb->modal;
     a.mean_tile_bytes = (params && params->mean_tile_bytes > 0) ? params->mean_tile_bytes : 0;
@@ -1068,7 +1071,7 @@ tc_status tc_decode(tc_ctx *ctx, const tc_model *m, const tc_codebook *cb, const
         if (st != TC_OK) return st;
     }
     return decode_with_scratch(ctx, m, cb, stream, stream_bytes, chunk_len, tile_off, params, x_hat,
-                               scratch ? (uint8_t *)ctx->scratch : nullptr, true, cuda_stream);
+                               scratch ? (uint8_t *)ctx->scratch : nullptr, 0, cuda_stream);
 }
 
 // ---- several tensors per call --------------------------------------------------------------------
@@ -1076,13 +1079,27 @@ tc_status tc_decode(tc_ctx *ctx, const tc_model *m, const tc_codebook *cb, const
 static tc_status ensure_many_streams(tc_ctx *ctx)
 {
     if (ctx->many_fork) return TC_OK;
-    for (int i = 0; i < 4; ++i) {
+    for (int i = 0; i < kManyStreams; ++i) {
         TC_CUDA(cudaStreamCreateWithFlags(&ctx->many_streams[i], cudaStreamNonBlocking));
         TC_CUDA(cudaEventCreateWithFlags(&ctx->many_join[i], cudaEventDisableTiming));
     }
     TC_CUDA(cudaEventCreateWithFlags(&ctx->many_fork, cudaEventDisableTiming));
     return TC_OK;
 }
+
+// SMs that the persistent kernels of tensor i of a list take: a quarter of them, more where the tensor is more than that
+// of the list's work.  A kernel's first tile costs a block 10 to 15 us (basis, tensor memory, first copies) and a further one
+// 2 to 4, so a grid over all SMs with a tile or two for each block spends the chip on set-up; the other streams'
+// kernels fill the rest.  16 layers of a residual network, four streams: encode 257 us on all SMs, 206 on half, 205 on a
+// quarter, 224 on 28; decode 252, 212, 202, 238; eight streams on a quarter: 201 and 179.
+static int list_share(int sm_count, int n_streams, const std::vector<double> &work, int i)
+{
+    double total = 0.0;
+    for (double w : work) total += w;
+    const int least = sm_count / std::min(4, n_streams);
+    return total > 0.0 ? std::min(sm_count, std::max(least, (int)std::ceil(sm_count * work[i] / total))) : least;
+}
+
 
 // Items in descending order of work: the large ones start first, each on its own stream.
 static std::vector<int> by_descending_work(int n, const std::vector<double> &work)
@@ -1135,7 +1152,7 @@ tc_status tc_encode_many(tc_ctx *ctx, const tc_encode_item *items, int32_t n_ite
     // one clear for the look-back state of all items, then the items fan out over the streams
     TC_CUDA(cudaMemsetAsync(ctx->scratch, 0, lookback_total, s));
     TC_CUDA(cudaEventRecord(ctx->many_fork, s));
-    const int n_streams = std::min(4, (int)n_items);
+    const int n_streams = std::min(kManyStreams, (int)n_items);
     for (int j = 0; j < n_streams; ++j) TC_CUDA(cudaStreamWaitEvent(ctx->many_streams[j], ctx->many_fork, 0));
     const std::vector<int> order = by_descending_work(n_items, work);
     tc_status first_error = TC_OK;
@@ -1143,11 +1160,12 @@ tc_status tc_encode_many(tc_ctx *ctx, const tc_encode_item *items, int32_t n_ite
         const int i = order[r];
         const tc_encode_item &it = items[i];
         cudaStream_t ws = ctx->many_streams[r % n_streams];
+        const int list_sms = list_share(ctx->sm_count, n_streams, work, i);
         const long long pixels = (long long)it.x->n * it.x->h * it.x->w;
         if (pixels == 0) { if (cudaMemsetAsync(it.tile_off, 0, sizeof(uint64_t), ws) != cudaSuccess && first_error == TC_OK) first_error = TC_ERR_CUDA; continue; }
         st = tc_encode_with_scratch(ctx, it.model, it.codebook, it.x, shape[i].cp, shape[i].splits, it.stream_out, it.capacity,
                                     it.chunk_len, it.tile_off, nullptr, (char *)ctx->scratch + lookback_at[i],
-                                    symbols_at[i] ? (char *)ctx->scratch + symbols_at[i] : nullptr, ws, nullptr, nullptr, true);
+                                    symbols_at[i] ? (char *)ctx->scratch + symbols_at[i] : nullptr, ws, nullptr, nullptr, list_sms);
         if (st != TC_OK && first_error == TC_OK) first_error = st;
     }
     for (int j = 0; j < n_streams; ++j) {
@@ -1185,16 +1203,17 @@ tc_status tc_decode_many(tc_ctx *ctx, const tc_decode_item *items, int32_t n_ite
     if (total && (st = ensure_scratch(ctx, total)) != TC_OK) return st;
     if ((st = ensure_many_streams(ctx)) != TC_OK) return st;
     TC_CUDA(cudaEventRecord(ctx->many_fork, s));
-    const int n_streams = std::min(4, (int)n_items);
+    const int n_streams = std::min(kManyStreams, (int)n_items);
     for (int j = 0; j < n_streams; ++j) TC_CUDA(cudaStreamWaitEvent(ctx->many_streams[j], ctx->many_fork, 0));
     const std::vector<int> order = by_descending_work(n_items, work);
     tc_status first_error = TC_OK;
     for (int r = 0; r < n_items; ++r) {
         const int i = order[r];
         const tc_decode_item &it = items[i];
+        const int list_sms = list_share(ctx->sm_count, n_streams, work, i);
         st = decode_with_scratch(ctx, it.model, it.codebook, it.stream, it.stream_bytes, it.chunk_len, it.tile_off, it.params,
                                  it.x_hat, symbols_bytes[i] ? (uint8_t *)ctx->scratch + symbols_at[i] : nullptr,
-                                 false, ctx->many_streams[r % n_streams]);
+                                 list_sms, ctx->many_streams[r % n_streams]);
         if (st != TC_OK && first_error == TC_OK) first_error = st;
     }
     for (int j = 0; j < n_streams; ++j) {

@@ -16,6 +16,7 @@ constexpr int TC_MAX_C = 1024;
 constexpr int TC_MAX_CODE_LEN = 12;
 constexpr int kMaxRoundtripChunks = 64;   // longest code the decode lookup table covers
 
+constexpr int kManyStreams = 8;               // streams that a list of tensors is spread over
 constexpr int kCanonWords = 12;               // words per table of a canonical code's bounds (6) and bases (6)
 
 // Device status word: first error wins.
@@ -40,8 +41,8 @@ struct tc_ctx {
     cudaEvent_t ev_in[2] = {nullptr, nullptr}, ev_done[2] = {nullptr, nullptr}, ev_out[2] = {nullptr, nullptr};
     unsigned long long *chunk_bits = nullptr;   // pinned HOST [kMaxRoundtripChunks]
     // tc_encode_many / tc_decode_many spread their items over these streams (created at first use)
-    cudaStream_t many_streams[4] = {nullptr, nullptr, nullptr, nullptr};
-    cudaEvent_t many_fork = nullptr, many_join[4] = {nullptr, nullptr, nullptr, nullptr};
+    cudaStream_t many_streams[kManyStreams] = {};
+    cudaEvent_t many_fork = nullptr, many_join[kManyStreams] = {};
     int force_exact = 0;                  // 1: route every tensor through the fp64 kernels; 2: skip the resident-basis kernels; 3: skip the run-skipping decoder
     int last_encode_path = 0;             // 0 = fp64 kernels, 1 = tensor-core kernels (resident basis), 2 = fp32 kernels, 3 = tensor-core kernels (streamed basis)
     int last_decode_path = 0;
@@ -117,6 +118,7 @@ struct EncodeArgs {
     unsigned long long *tile_state;   // look-back state, zeroed before launch
     unsigned int *ticket;             // zeroed before launch; the look-back words follow it
     bool alone;                       // no other stream of this call (see launch_chained)
+    int sms;                          // SMs that a persistent kernel takes at most
     long long clear_words;            // 64-bit words from `ticket` on that the first of several kernels zeroes (0: they are zero)
     unsigned int *status;
     unsigned long long *clamped;      // nullable: counts coefficients outside the range
@@ -147,6 +149,7 @@ struct DecodeArgs {
     const uint8_t *sorted;              // [groups][2^bits]
     const __nv_bfloat16 *basis_t_bf16;  // [c][k]
     bool alone;                         // no other stream of this call (see launch_chained)
+    int sms;                            // SMs that a persistent kernel takes at most
     const CUtensorMap *basis_t_map;     // HOST pointer to the model's tensor map of basis_t_bf16, or null
     const float *dec_bias;              // [c]
     int center;                         // subtracted from every symbol before the MMA
@@ -187,7 +190,7 @@ constexpr size_t kEncodeScratchHeader = 64;   // ticket counter, padded; the per
 tc_status tc_encode_with_scratch(tc_ctx *ctx, const tc_model *m, const tc_codebook *cb, const tc_tensor *x, int chunk_pixels,
                                  int splits, void *stream_out, size_t capacity, uint16_t *chunk_len, uint64_t *tile_off,
                                  const tc_debug_out *debug, void *scratch, void *work, cudaStream_t s,
-                                 unsigned long long *hist = nullptr, unsigned long long *clamped = nullptr, bool scratch_is_zero = false);
+                                 unsigned long long *hist = nullptr, unsigned long long *clamped = nullptr, int list_sms = 0);
 // tensors of fewer tiles than this many per SM take the one-thread-per-value exact kernels
 constexpr int kExactParallelTilesPerSm = 2;
 

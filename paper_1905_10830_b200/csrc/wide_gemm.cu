@@ -309,11 +309,11 @@ int best_columns(long long tiles, int k, int sm_count)
 }
 
 template <bool kEncode>
-tc_status launch_gemm(const tc_ctx *ctx, bool early, const GemmArgs &g, const CUtensorMap &map_a, const CUtensorMap &map_b, cudaStream_t s)
+tc_status launch_gemm(int sms, bool early, const GemmArgs &g, const CUtensorMap &map_a, const CUtensorMap &map_b, cudaStream_t s)
 {
     const size_t smem = (size_t)kStages * kStageBytes + (kEncode ? 0 : kEpiWarps * kTrWarpBytes);
     if (cudaFuncSetAttribute(wide_gemm_kernel<kEncode>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return TC_ERR_CUDA;
-    const unsigned int grid = (unsigned int)(g.units < ctx->sm_count ? g.units : ctx->sm_count);
+    const unsigned int grid = (unsigned int)(g.units < sms ? g.units : sms);
     return launch_chained(early, wide_gemm_kernel<kEncode>, grid, kThreads, smem, s, g, map_a, map_b) == cudaSuccess ? TC_OK : TC_ERR_CUDA;
 }
 
@@ -355,7 +355,7 @@ tc_status tc_launch_encode_wide_gemm(const tc_ctx *ctx, const EncodeArgs &a, voi
         GemmArgs g{};
         g.n_panels = (a.c + kPanelK - 1) / kPanelK;
         g.k_depth = a.c;
-        g.n_cols = best_columns(t1 - t0, a.k, ctx->sm_count);
+        g.n_cols = best_columns(t1 - t0, a.k, a.sms);
         g.blocks = (a.k + g.n_cols - 1) / g.n_cols;
         CUtensorMap map_x, map_t;
         if (!tc_tensor_map_sw128(&map_x, rows, p1 - p0, a.c, 128) || !tc_tensor_map_sw128(&map_t, a.basis_bf16, a.k, a.c, g.n_cols)) return TC_ERR_CUDA;
@@ -367,7 +367,7 @@ tc_status tc_launch_encode_wide_gemm(const tc_ctx *ctx, const EncodeArgs &a, voi
         g.bias = a.enc_bias;
         g.sym = sym;
         g.status = a.status;
-        tc_status st = launch_gemm<true>(ctx, a.alone, g, map_x, map_t, s);
+        tc_status st = launch_gemm<true>(a.sms, a.alone, g, map_x, map_t, s);
         if (st != TC_OK) return st;
         if ((st = tc_launch_pack_symbols(ctx, a, sym, t0, t1, s)) != TC_OK) return st;
     }
@@ -389,7 +389,7 @@ tc_status tc_launch_decode_wide_gemm(const tc_ctx *ctx, const DecodeArgs &a, voi
         g.blocks = (a.c + 127) / 128;
         // 256 pixels a unit; 128 or 64 while that leaves SMs without one
         g.n_cols = kMaxN;
-        while (g.n_cols > 64 && ((p1 - p0 + g.n_cols - 1) / g.n_cols) * g.blocks < ctx->sm_count) g.n_cols /= 2;
+        while (g.n_cols > 64 && ((p1 - p0 + g.n_cols - 1) / g.n_cols) * g.blocks < a.sms) g.n_cols /= 2;
         g.units = ((p1 - p0 + g.n_cols - 1) / g.n_cols) * g.blocks;
         CUtensorMap map_q;
         if (!tc_tensor_map_sw128(&map_q, q, p1 - p0, a.k, g.n_cols)) return TC_ERR_CUDA;
@@ -399,7 +399,7 @@ tc_status tc_launch_decode_wide_gemm(const tc_ctx *ctx, const DecodeArgs &a, voi
         g.bias = a.dec_bias;
         g.xhat = (__nv_bfloat16 *)a.xhat;
         g.status = a.status;
-        if ((st = launch_gemm<false>(ctx, a.alone, g, *a.basis_t_map, map_q, s)) != TC_OK) return st;
+        if ((st = launch_gemm<false>(a.sms, a.alone, g, *a.basis_t_map, map_q, s)) != TC_OK) return st;
     }
     return TC_OK;
 }
