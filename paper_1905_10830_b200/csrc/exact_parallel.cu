@@ -351,6 +351,9 @@ __global__ void __launch_bounds__(TC_TILE_PIXELS * kMaxParts) pack_symbols_kerne
 // the per-pixel decoder: tile offsets aligned, ordered and inside the stream, every chunk inside
 // its tile and consumed to exactly its recorded length.
 constexpr int kUnpackThreads = 512;
+constexpr int kFirstBits = 6;                                  // of a per-layer code: lengths that the first table resolves
+constexpr uint32_t kRowBytes = 80;                            // 32 symbols of a row, padded: the lanes' 16-byte pieces fall into all banks
+constexpr uint32_t kRowsWarpBytes = 32 * kRowBytes;
 
 // MSB-first reader with a 64-bit window hi:lo (left-aligned) and the word behind it already loaded: a
 // refill never waits for memory.  Words at or past `end` read as zero.
@@ -454,10 +457,16 @@ struct StagedReader {
 // 2^12-entry table per channel in global memory and a byte stored per symbol, 40 with bounds, 35 with the
 // staged segment, 27 with the symbols looked up behind the chain and per-channel codes in an
 // instantiation of their own (the choice inside the loop kept the bounds from being read ahead).
-template <bool kOperand, bool kPerLayer>
+// kFull: with many warps on an SM the shared-memory pipe bounds it instead, eleven wavefronts a step of a warp:
+// bank conflicts of the 2^12-entry table (seven), and the stores, a row each per lane (four).  Codes of up to six bits then
+// come from a table that every lane has in a bank of its own, and rows leave 64 bytes at a time.  576x14x14 x 1024
+// decode 376 -> 341 us, x 128 (21 warps an SM) 60.5 -> 57.1; 384x14x14 x 128 (5 warps) would lose, 39.1 -> 41.5, to the
+// second lookup in the chain, 512x7x7 x 64 (25 tiles) 23.3 -> 27.3.
+template <bool kOperand, bool kPerLayer, bool kFull>
 __global__ void __launch_bounds__(kUnpackThreads) unpack_symbols_kernel(DecodeArgs a, void *out, long long first_tile, unsigned int table_bytes,
                                                                          unsigned int segment_bytes)
 {
+    __shared__ uint32_t s_first[kFull ? (32 << kFirstBits) : 1];
     __shared__ unsigned int s_warp_sums[kUnpackThreads / 32];
     __shared__ unsigned int s_start[kUnpackThreads];
     extern __shared__ __align__(16) unsigned char s_tables[];   // the per-layer table, or the bounds and bases of every channel's code
@@ -479,6 +488,12 @@ __global__ void __launch_bounds__(kUnpackThreads) unpack_symbols_kernel(DecodeAr
             const uint32_t e = __ldg(a.lut + i);
             s_lut[i] = (value(e >> 8) << 16) | (e & 0xffu);
         }
+        // the codes of up to kFirstBits bits, every lane's copy in a bank of its own; longer ones: 0
+        if constexpr (kFull)
+            for (int i = warp; i < (1 << kFirstBits); i += blockDim.x / 32) {
+                const uint32_t e = __ldg(a.lut + (a.lut_bits >= kFirstBits ? i << (a.lut_bits - kFirstBits) : i >> (kFirstBits - a.lut_bits)));
+                s_first[i * 32 + lane] = (e & 0xffu) <= kFirstBits ? (value(e >> 8) << 16) | (e & 0xffu) : 0u;
+            }
     } else {
         stage(tables, a.canon, (unsigned int)a.k * kCanonWords / 4u);
         if (sorted_staged) stage(s_sorted, a.sorted, (unsigned int)(a.k * nsym) / 16u);
@@ -514,8 +529,11 @@ __global__ void __launch_bounds__(kUnpackThreads) unpack_symbols_kernel(DecodeAr
     const int part = a.splits > 1 ? t / TC_TILE_PIXELS : 0;
     const int in_tile = a.splits > 1 ? (t % TC_TILE_PIXELS) * a.splits + part : t;
     const long long ch = tile * chunks_per_tile + in_tile;
-    if (t >= chunks_per_tile || ch >= a.n_chunks) return;
-    const unsigned int want = a.chunk_len[ch], off = s_start[in_tile];
+    if (warp * 32 >= chunks_per_tile) return;
+    // a lane without a chunk walks zeros beside its warp where the warp's rows leave together
+    const bool mine = t < chunks_per_tile && ch < a.n_chunks;
+    if (!kFull && !mine) return;
+    const unsigned int want = mine ? a.chunk_len[ch] : 0u, off = mine ? s_start[in_tile] : 0u;
     bool bad = base + off + want > end;
     auto walk = [&](auto &r) {
         unsigned int used = 0;
@@ -529,7 +547,13 @@ __global__ void __launch_bounds__(kUnpackThreads) unpack_symbols_kernel(DecodeAr
                 if ((i & 1) == 0) r.refill();
                 uint32_t len;
                 if constexpr (kPerLayer) {
-                    const uint32_t e = s_lut[r.hi >> (32 - a.lut_bits)];
+                    uint32_t e;
+                    if constexpr (kFull) {
+                        e = s_first[(r.hi >> (32 - kFirstBits)) * 32 + lane];
+                        asm volatile("{\n\t.reg .pred p;\n\tsetp.eq.u32 p, %0, 0;\n\t@p ld.shared.u32 %0, [%1];\n\t}"
+                                     : "+r"(e) : "r"(tables + (r.hi >> (32 - a.lut_bits)) * 4u));
+                    } else
+                        e = s_lut[r.hi >> (32 - a.lut_bits)];
                     len = e & 0xffu;
                     v[i] = e >> 16;
                 } else {
@@ -554,42 +578,78 @@ __global__ void __launch_bounds__(kUnpackThreads) unpack_symbols_kernel(DecodeAr
                 for (int i = 0; i < kN; ++i) v[i] = value(v[i]);
             }
         };
-        const bool by8 = a.k % 8 == 0 && run % 8 == 0;
-        for (int lp = first_px; lp < first_px + (a.splits > 1 ? 1 : a.chunk_pixels); ++lp) {
-            const long long p = tile * TC_TILE_PIXELS + lp;
-            if (p >= a.pixels) break;
-            const long long row = (p - first_tile * TC_TILE_PIXELS) * a.k;
-            if (by8) {
+        if constexpr (kFull) {
+            // runs are multiples of 8; 32 symbols of the warp's 32 rows are turned through shared memory, so that a
+            // store covers 64 bytes of a row
+            const uint32_t rows = tables + table_bytes + segment_bytes + (uint32_t)warp * kRowsWarpBytes;
+            const int per_lane = a.splits > 1 ? 1 : a.chunk_pixels, px0 = a.splits > 1 ? (warp * 32) % TC_TILE_PIXELS : warp * 32 * per_lane;
+            for (int lp = 0; lp < per_lane; ++lp) {
+                const unsigned int used_before = used;
 #pragma unroll 1
-                for (int j = j_first; j < j_first + run; j += 8) {
-                    uint32_t v[8];
-                    decode(j, v);
-                    if constexpr (kOperand)
-                        *reinterpret_cast<uint4 *>((uint16_t *)out + row + j) =
-                            make_uint4(v[0] | (v[1] << 16), v[2] | (v[3] << 16), v[4] | (v[5] << 16), v[6] | (v[7] << 16));
-                    else
-                        *reinterpret_cast<uint2 *>((uint8_t *)out + row + j) =
-                            make_uint2(v[0] | (v[1] << 8) | (v[2] << 16) | (v[3] << 24), v[4] | (v[5] << 8) | (v[6] << 16) | (v[7] << 24));
+                for (int j = j_first; j < j_first + run; j += 32) {
+                    const int n8 = min(4, (j_first + run - j) >> 3);
+#pragma unroll 1
+                    for (int g = 0; g < n8; ++g) {
+                        uint32_t v[8];
+                        decode(j + 8 * g, v);
+                        asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(rows + lane * kRowBytes + g * 16u), "r"(v[0] | (v[1] << 16)),
+                                     "r"(v[2] | (v[3] << 16)), "r"(v[4] | (v[5] << 16)), "r"(v[6] | (v[7] << 16)) : "memory");
+                    }
+                    __syncwarp();
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        const int row = (lane >> 2) + 8 * i, px = px0 + row * per_lane + lp;
+                        const long long p = tile * TC_TILE_PIXELS + px;
+                        uint4 q;
+                        asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(q.x), "=r"(q.y), "=r"(q.z), "=r"(q.w)
+                                     : "r"(rows + row * kRowBytes + (lane & 3) * 16u));
+                        if ((lane & 3) < n8 && px < TC_TILE_PIXELS && p < a.pixels)
+                            *reinterpret_cast<uint4 *>((uint16_t *)out + (p - first_tile * TC_TILE_PIXELS) * a.k + j + (lane & 3) * 8) = q;
+                    }
+                    __syncwarp();
                 }
-            } else {
+                if (tile * TC_TILE_PIXELS + first_px + lp >= a.pixels) used = used_before;        // a pixel that does not exist
+            }
+        } else {
+            const bool by8 = a.k % 8 == 0 && run % 8 == 0;
+            for (int lp = first_px; lp < first_px + (a.splits > 1 ? 1 : a.chunk_pixels); ++lp) {
+                const long long p = tile * TC_TILE_PIXELS + lp;
+                if (p >= a.pixels) break;
+                const long long row = (p - first_tile * TC_TILE_PIXELS) * a.k;
+                if (by8) {
 #pragma unroll 1
-                for (int j = j_first; j < j_first + run; ++j) {
-                    uint32_t v[1];
-                    decode(j, v);
-                    if constexpr (kOperand) ((uint16_t *)out)[row + j] = (uint16_t)v[0];
-                    else ((uint8_t *)out)[row + j] = (uint8_t)v[0];
+                    for (int j = j_first; j < j_first + run; j += 8) {
+                        uint32_t v[8];
+                        decode(j, v);
+                        if constexpr (kOperand)
+                            *reinterpret_cast<uint4 *>((uint16_t *)out + row + j) =
+                                make_uint4(v[0] | (v[1] << 16), v[2] | (v[3] << 16), v[4] | (v[5] << 16), v[6] | (v[7] << 16));
+                        else
+                            *reinterpret_cast<uint2 *>((uint8_t *)out + row + j) =
+                                make_uint2(v[0] | (v[1] << 8) | (v[2] << 16) | (v[3] << 24), v[4] | (v[5] << 8) | (v[6] << 16) | (v[7] << 24));
+                    }
+                } else {
+#pragma unroll 1
+                    for (int j = j_first; j < j_first + run; ++j) {
+                        uint32_t v[1];
+                        decode(j, v);
+                        if constexpr (kOperand) ((uint16_t *)out)[row + j] = (uint16_t)v[0];
+                        else ((uint8_t *)out)[row + j] = (uint8_t)v[0];
+                    }
                 }
             }
         }
-        if (used != want) bad = true;
+        if (mine && used != want) bad = true;
     };
-    if (!bad && staged) {
+    const bool walks = mine && !bad;
+    if (!kFull && !walks) {
+    } else if (staged) {
         StagedReader r;
-        r.init(seg, off, seg + (uint32_t)((end - base) >> 3));
+        r.init(seg, walks ? off : 0u, walks ? seg + (uint32_t)((end - base) >> 3) : seg);
         walk(r);
-    } else if (!bad) {
+    } else {
         AheadReader r;
-        r.init(a.stream, base + off, end);
+        r.init(a.stream, base + (walks ? off : 0u), walks ? end : base);
         walk(r);
     }
     if (bad) tc_dev_set_status(a.status, TC_ERR_CORRUPT_STREAM);
@@ -658,18 +718,22 @@ static tc_status launch_unpack(const DecodeArgs &a, void *out, long long first_t
     const int chunks = a.splits * TC_TILE_PIXELS / a.chunk_pixels;
     if (chunks > kUnpackThreads) return TC_ERR_UNSUPPORTED;
     // beside the tables (at most 48 KB and the symbols) room for a segment of three bits per symbol, at most 48 KB
-    unsigned int tables = (unsigned int)(a.groups == 1 ? ((size_t)4 << a.lut_bits) : (size_t)a.k * kCanonWords * 4);
+    unsigned int tables = (unsigned int)(a.groups == 1 ? std::max<size_t>((size_t)4 << a.lut_bits, 16) : (size_t)a.k * kCanonWords * 4);
     if (a.groups != 1) {
         const unsigned int sorted = (unsigned int)a.k << a.bits;                   // bytes
         if (sorted % 16 == 0 && ((uintptr_t)a.sorted & 15u) == 0 && sorted <= kSortedStaged) tables += sorted;
     }
     const unsigned int segment = (unsigned int)std::min<long long>((long long)a.k * TC_TILE_PIXELS * 3 / 8, 48 * 1024);
-    void (*kernel)(DecodeArgs, void *, long long, unsigned int, unsigned int) =
-        a.groups == 1 ? unpack_symbols_kernel<kOperand, true> : unpack_symbols_kernel<kOperand, false>;
-    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 112 * 1024) != cudaSuccess) return TC_ERR_CUDA;
     // a block of few chunks has more threads for staging while all blocks are resident at once
     const int threads = (chunks + 31) / 32 * 32, least = end_tile - first_tile < 4 * sm_count ? 256 : 32;
-    kernel<<<(unsigned int)(end_tile - first_tile), std::max(threads, least), tables + segment, s>>>(a, out, first_tile, tables, segment);
+    // from 16 warps an SM on the shared-memory pipe is what bounds a per-layer decoder (see the kernel)
+    const bool full = kOperand && a.groups == 1 && (end_tile - first_tile) * threads >= 16 * 32 * (long long)sm_count;
+    void (*kernel)(DecodeArgs, void *, long long, unsigned int, unsigned int) =
+        a.groups != 1 ? unpack_symbols_kernel<kOperand, false, false>
+        : full ? unpack_symbols_kernel<kOperand, true, kOperand> : unpack_symbols_kernel<kOperand, true, false>;
+    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024) != cudaSuccess) return TC_ERR_CUDA;
+    const size_t rows = full ? (size_t)(threads / 32) * kRowsWarpBytes : 0;
+    kernel<<<(unsigned int)(end_tile - first_tile), std::max(threads, least), tables + segment + rows, s>>>(a, out, first_tile, tables, segment);
     return cudaGetLastError() == cudaSuccess ? TC_OK : TC_ERR_CUDA;
 }
 

@@ -139,12 +139,13 @@ def test_run_skipping_decoder_groups(ctx, c, k, h, w, bits):
 
 # Wide layers as tiled products: blocks of coefficients and channels with remainders, pixel rows of 1, 2 and
 # 4-element alignment, fewer units than SMs and more, several passes over the workspace, every chunk
-# shape, both table granularities.  Against the fused kernel (debug outputs take it), whose symbols the
+# shape, both table granularities, few and many decoder warps an SM.  Against the fused kernel (debug outputs take it), whose symbols the
 # parity cases check, and the fp64 kernels.
 @pytest.mark.parametrize("c,k,h,w,n,bits,tables,offset", [
     (272, 272, 3, 3, 1, 4, 1, 0), (320, 320, 5, 5, 40, 5, 1, 0), (576, 576, 14, 14, 9, 5, 1, 0), (960, 960, 7, 7, 30, 5, 1, 0),
     (1024, 1024, 12, 12, 160, 2, 1, 0), (512, 512, 7, 7, 64, 8, 1, 0), (400, 208, 6, 6, 50, 6, 208, 0), (960, 16, 7, 7, 5, 8, 1, 0),
-    (80, 48, 27, 19, 37, 6, 48, 0), (64, 64, 9, 9, 1, 4, 1, 0), (256, 256, 7, 9, 90, 3, 1, 0), (128, 128, 14, 14, 6, 4, 1, 1), (48, 32, 5, 3, 700, 7, 1, 0)])
+    (80, 48, 27, 19, 37, 6, 48, 0), (64, 64, 9, 9, 1, 4, 1, 0), (256, 256, 7, 9, 90, 3, 1, 0), (128, 128, 14, 14, 6, 4, 1, 1), (48, 32, 5, 3, 700, 7, 1, 0),
+    (272, 112, 28, 28, 97, 5, 1, 0), (272, 48, 28, 28, 194, 5, 1, 0)])
 def test_wide_layers_as_tiled_products(ctx, c, k, h, w, n, bits, tables, offset):
     params = fm.layer_params(fm.LayerSpec(c, h, w, 0.95, None, 14000 + c + k + h))
     cal = fm.make_maps(params, max(4, 4 * c // (h * w) + 1), calib=True, dtype=torch.bfloat16, device="cuda")
