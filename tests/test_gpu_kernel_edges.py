@@ -173,3 +173,25 @@ def test_wide_layers_as_tiled_products(ctx, c, k, h, w, n, bits, tables, offset)
     assert bool(((a - b).abs() <= 2.0 ** -7 * b.abs() + 1e-6 * float(b.abs().max())).all())
     assert float((a != b).double().mean()) <= 1e-3
     m.close(); cb.close()
+
+
+# Covariance of the fit in 64 x 64 blocks of channel pairs over slabs of 32 pixels: one block, blocks with
+# remainders, a single partial slab, slabs that cross images.  The basis rows are rounded to fp32
+# (2^-24 of an entry), so the covariance put together from the model is off by at most
+# 2 * 2^-24 * sum_j eig_j |b_ja| |b_jb| <= 2^-23 * max(eig); as much again for the sums' order and the
+# eigenvectors' residual.
+@pytest.mark.parametrize("c,h,w,n,dtype", [(2, 3, 3, 1, torch.float32), (33, 5, 7, 3, torch.float32), (64, 14, 14, 2, torch.float32),
+                                           (65, 4, 8, 9, torch.float32), (200, 7, 7, 30, torch.float32)])
+def test_covariance_blocks(ctx, c, h, w, n, dtype):
+    g = torch.Generator(device="cuda").manual_seed(c)
+    x = torch.randn(n, c, h, w, generator=g, device="cuda", dtype=torch.float64) * torch.linspace(2.0, 0.5, c, device="cuda", dtype=torch.float64).view(1, c, 1, 1)
+    x = (x + 3.0 + 0.5 * x.mean(1, keepdim=True)).to(dtype)
+    m = tc.tc_fit_pca(ctx, x, 6)
+    e = tc.tc_model_export(m)
+    v = x.double().transpose(0, 1).reshape(c, -1).cpu().numpy()
+    v = v - v.mean(1, keepdims=True)
+    want = v @ v.T / (v.shape[1] - 1)
+    basis, eig = np.asarray(e["basis"], dtype=np.float64).reshape(c, c), np.asarray(e["eig"], dtype=np.float64)
+    got = basis.T @ (eig[:, None] * basis)
+    assert np.abs(got - want).max() <= 2.0 ** -22 * eig.max()
+    m.close()
