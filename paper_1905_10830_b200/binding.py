@@ -155,6 +155,11 @@ def _stream_ptr(device) -> int:
     return torch.cuda.current_stream(device).cuda_stream
 
 
+def _tensor_stream(device: int) -> int:
+    """The same for calls that have a CUDA tensor (CUDA is initialised): 0.1 us a call instead of 1.3."""
+    return torch._C._cuda_getCurrentRawStream(device)
+
+
 class _Handle:
     _free = None
 
@@ -437,9 +442,10 @@ def tc_encode(ctx: Context, model: Model, cb: Codebook, x: torch.Tensor, *, chun
               k: int | None = None) -> EncodedStream:
     """Encode `x`.  Buffers are allocated with torch (worst-case size) unless `out` is given."""
     t = _tensor(x)
-    lay = tc_encode_bound(model, cb, x, chunk_pixels, pixel_splits)
     dev = x.device
-    if out is None:
+    if out is None:              # the library resolves the chunk shape by itself: 2.5 us a call less with `out`
+        lay = tc_encode_bound(model, cb, x, chunk_pixels, pixel_splits)
+        chunk_pixels, pixel_splits = lay.chunk_pixels, lay.pixel_splits
         nbytes = lay.stream_bytes if capacity is None else capacity
         out = EncodedStream(torch.empty(max(nbytes, 16), dtype=torch.uint8, device=dev),
                             torch.empty(max(lay.n_chunks + (lay.n_chunks & 1), 2), dtype=torch.int16, device=dev),
@@ -451,11 +457,11 @@ def tc_encode(ctx: Context, model: Model, cb: Codebook, x: torch.Tensor, *, chun
         out.coefficients = torch.empty(pixels, kk, dtype=torch.float32, device=dev)
         out.symbols = torch.empty(pixels, kk, dtype=torch.uint8, device=dev)
         dbg = _DebugOut(out.coefficients.data_ptr(), out.symbols.data_ptr())
-    p = _EncodeParams(lay.chunk_pixels, lay.pixel_splits)
+    p = _EncodeParams(chunk_pixels, pixel_splits)
     cap = out.words.numel() if capacity is None else min(capacity, out.words.numel())
     _check(load_library().tc_encode(ctx.ptr, model.ptr, cb.ptr, C.byref(t), C.byref(p), out.words.data_ptr(), cap,
                                     out.chunk_len.data_ptr(), out.tile_off.data_ptr(),
-                                    C.byref(dbg) if dbg is not None else None, _stream_ptr(ctx.device)), "tc_encode")
+                                    C.byref(dbg) if dbg is not None else None, _tensor_stream(ctx.device)), "tc_encode")
     return out
 
 
@@ -490,7 +496,7 @@ def tc_decode(ctx: Context, model: Model, cb: Codebook, enc: EncodedStream, shap
     nbytes = enc.words.numel() if stream_bytes is None else stream_bytes
     _check(load_library().tc_decode(ctx.ptr, model.ptr, cb.ptr, enc.words.data_ptr(), nbytes,
                                     enc.chunk_len.data_ptr(), enc.tile_off.data_ptr(), C.byref(p), C.byref(t),
-                                    _stream_ptr(ctx.device)), "tc_decode")
+                                    _tensor_stream(ctx.device)), "tc_decode")
     return out
 
 
@@ -512,14 +518,15 @@ def tc_encode_many(ctx: Context, layers, *, outs=None):
     result = []
     for i, (model, cb, x) in enumerate(layers):
         t = _tensor(x)
-        lay = tc_encode_bound(model, cb, x, 0, 0)
+        p = _EncodeParams(0, 0)
         if outs is not None:
             out = outs[i]
         else:
+            lay = tc_encode_bound(model, cb, x, 0, 0)
+            p = _EncodeParams(lay.chunk_pixels, lay.pixel_splits)
             out = EncodedStream(torch.empty(max(lay.stream_bytes, 16), dtype=torch.uint8, device=x.device),
                                 torch.empty(max(lay.n_chunks + (lay.n_chunks & 1), 2), dtype=torch.int16, device=x.device),
                                 torch.empty(lay.n_tiles + 1, dtype=torch.int64, device=x.device), lay)
-        p = _EncodeParams(lay.chunk_pixels, lay.pixel_splits)
         tensors.append(t); params.append(p); result.append(out)
         items[i] = _EncodeItem(model.ptr, cb.ptr, C.addressof(t), C.addressof(p), out.words.data_ptr(), out.words.numel(),
                                out.chunk_len.data_ptr(), out.tile_off.data_ptr())
