@@ -16,7 +16,8 @@
  *   - `cuda_stream` is a cudaStream_t passed as void* (NULL = the default stream).  Calls that
  *     take one are asynchronous on it unless stated otherwise.
  *   - A context serves one stream at a time: its scratch arena (the cross-tile bookkeeping of
- *     tc_encode, the buffers of tc_stats and tc_roundtrip_host) and its status word are shared by
+ *     tc_encode, the workspaces of fits and of entropy coders that run as kernels of their own, the
+ *     buffers of tc_stats and tc_roundtrip_host) and its status word are shared by
  *     all calls made on it, so two calls on the same context that could overlap on the GPU --
  *     different streams, no dependency between them -- corrupt each other's output.  Use one
  *     context per concurrent stream; models and codebooks may be shared between contexts of the

@@ -456,6 +456,15 @@ void tc_model_free(tc_model *m)
     delete m;
 }
 
+// Workspace of a fit in the context's arena (an allocation and its release cost about 0.1 ms each): mean and
+// covariance, then the eigensolver's, then eigenvalues, scale and the blocks' ranges of coefficient 0.
+static size_t fit_head_bytes(int c) { return (((size_t)c + (size_t)c * c) * sizeof(double) + 255) & ~(size_t)255; }
+static size_t fit_scratch_bytes(int c, long long range_pixels)
+{
+    return fit_head_bytes(c) + ((tc_eigh_device_workspace_bytes(c) + 255) & ~(size_t)255) +
+           ((size_t)c + 1 + 2 * (size_t)tc_range0_max_blocks(range_pixels)) * sizeof(double);
+}
+
 static tc_status finish_fit(tc_ctx *ctx, const tc_tensor *range_maps, const tc_fit_params *params, int k,
                             const double *d_mean, const double *d_cov, tc_model **out, cudaStream_t s);
 
@@ -480,13 +489,12 @@ tc_status tc_fit_pca(tc_ctx *ctx, const tc_tensor *calib, const tc_fit_params *p
     cudaStream_t s = (cudaStream_t)cuda_stream;
 
     const size_t n_doubles = (size_t)c + (size_t)c * c;
-    double *d_buf = nullptr;
-    TC_CUDA(cudaMalloc((void **)&d_buf, n_doubles * sizeof(double)));
-    double *d_mean = d_buf, *d_cov = d_buf + c;
-    struct Free { double *p; ~Free() { cudaFree(p); } } freer{d_buf};
+    tc_status st = ensure_scratch(ctx, fit_scratch_bytes(c, m_samples));
+    if (st != TC_OK) return st;
+    double *const d_buf = (double *)ctx->scratch, *d_mean = d_buf, *d_cov = d_buf + c;
     TC_CUDA(cudaMemsetAsync(d_buf, 0, n_doubles * sizeof(double), s));
 
-    tc_status st = tc_launch_channel_sums(calib->data, calib->dtype, n, c, hw, d_mean, s);
+    st = tc_launch_channel_sums(calib->data, calib->dtype, n, c, hw, d_mean, s);
     if (st != TC_OK) return st;
     std::vector<double> mean(c);
     TC_CUDA(cudaMemcpyAsync(mean.data(), d_mean, sizeof(double) * c, cudaMemcpyDeviceToHost, s));
@@ -512,13 +520,15 @@ static tc_status finish_fit(tc_ctx *ctx, const tc_tensor *range_maps, const tc_f
     const int range_blocks = tc_range0_max_blocks(m_samples);
     const size_t cc = (size_t)c * c;
     // small: eigenvalues [c], scale [1], min / max per block [2 * range_blocks]
-    double *d_small = nullptr, *d_basis = nullptr, *d_mean_copy = nullptr;
-    void *d_work = nullptr;
+    double *d_basis = nullptr, *d_mean_copy = nullptr;
     struct Free {
-        double **a, **b, **m; void **w;
-        ~Free() { cudaFree(*a); cudaFree(*b); cudaFree(*m); cudaFree(*w); }
-    } freer{&d_small, &d_basis, &d_mean_copy, &d_work};
-    TC_CUDA(cudaMalloc((void **)&d_small, ((size_t)c + 1 + 2 * (size_t)range_blocks) * sizeof(double)));
+        double **a, **b;
+        ~Free() { cudaFree(*a); cudaFree(*b); }
+    } freer{&d_basis, &d_mean_copy};
+    // behind mean and covariance in the arena (fit_scratch_bytes)
+    char *const rest = (char *)ctx->scratch + fit_head_bytes(c);
+    void *const d_work = rest;
+    double *const d_small = (double *)(rest + ((tc_eigh_device_workspace_bytes(c) + 255) & ~(size_t)255));
     TC_CUDA(cudaMalloc((void **)&d_basis, cc * sizeof(double)));
     TC_CUDA(cudaMalloc((void **)&d_mean_copy, (size_t)c * sizeof(double)));
     double *d_eig = d_small, *d_scale = d_small + c, *d_minmax = d_scale + 1;
@@ -533,7 +543,6 @@ static tc_status finish_fit(tc_ctx *ctx, const tc_tensor *range_maps, const tc_f
         TC_CUDA(cudaMemcpyAsync(d_eig, eig.data(), sizeof(double) * c, cudaMemcpyHostToDevice, s));
         TC_CUDA(cudaStreamSynchronize(s));
     } else {
-        TC_CUDA(cudaMalloc(&d_work, tc_eigh_device_workspace_bytes(c)));
         if ((st = tc_eigh_device(d_cov, c, d_eig, d_basis, d_work, nullptr, s)) != TC_OK) return st;
     }
     if ((st = tc_launch_round_basis(d_basis, c, params->basis_dtype, d_scale, s)) != TC_OK) return st;
@@ -661,11 +670,10 @@ tc_status tc_fit_state_finish(tc_ctx *ctx, const tc_fit_state *st, const tc_tens
     DeviceGuard guard(ctx->device);
     cudaStream_t s = (cudaStream_t)cuda_stream;
     // mean = s / M, covariance = (S - s s^T / M) / (M - 1), on the device
-    double *d_buf = nullptr;
-    TC_CUDA(cudaMalloc((void **)&d_buf, ((size_t)c + (size_t)c * c) * sizeof(double)));
-    struct Free { double *p; ~Free() { cudaFree(p); } } freer{d_buf};
-    double *d_mean = d_buf, *d_cov = d_buf + c;
-    tc_status rc = tc_launch_moments_to_cov(st->d_sum, st->d_outer, st->count, c, d_mean, d_cov, s);
+    tc_status rc = ensure_scratch(ctx, fit_scratch_bytes(c, (long long)range_maps->n * range_maps->h * range_maps->w));
+    if (rc != TC_OK) return rc;
+    double *d_mean = (double *)ctx->scratch, *d_cov = d_mean + c;
+    rc = tc_launch_moments_to_cov(st->d_sum, st->d_outer, st->count, c, d_mean, d_cov, s);
     if (rc != TC_OK) return rc;
     return finish_fit(ctx, range_maps, params, k, d_mean, d_cov, out, s);
 }
