@@ -2,17 +2,18 @@
 //
 // One persistent block per SM walks tiles of 128 consecutive pixels.  Warp roles:
 //   warps 0-7, 8-15  two epilogue groups (alternating tiles).  Within a group warps 0-3 own the
-//                    first half of the coefficients of the tile's 128 pixels and warps 4-7 the
-//                    second half: TMEM -> registers, quantise, code lengths, bit offsets (scan +
-//                    tile look-back), pack, 128-bit stores.  The symbols stay packed in
-//                    registers between the length pass and the packing pass.
+//                    leading coefficients of the tile's 128 pixels and warps 4-7 the others, split
+//                    where the expected work of both is the same: TMEM -> registers, quantise, code.  A
+//                    thread packs its codes into a run of its own in shared memory, in one pass, and the
+//                    runs are joined once the tile's bit offsets are known (scan); tiles whose runs
+//                    would not fit take two passes over the accumulator, lengths first.
 //   warps 21, 22     one store warp per epilogue group: resolves the tile's stream offset by
 //                    look-back and copies the group's staging buffer out, while the group
 //                    already works on its next tile
-//   warps 16-19      loaders: cp.async NCHW -> shared memory in the MMA's MN-major layout (128-byte swizzle)
+//   warps 16-19      loaders: 16- and 8-byte cp.async NCHW -> shared memory in the MMA's MN-major layout (128-byte swizzle)
 //   warp 20          one thread issues tcgen05.mma:  D[pixel][coef] = X_tile[pixel][c] * T[coef][c]
 // The basis T (bf16, K x C) stays resident in shared memory; the X tile streams through a ring
-// of 64-channel panels; the fp32 accumulators are double-buffered in tensor memory so that the
+// of 32-channel panels; the fp32 accumulators are double-buffered in tensor memory so that the
 // epilogue of one tile overlaps the loads and MMAs of the next.
 #include <algorithm>
 #include <cstdio>

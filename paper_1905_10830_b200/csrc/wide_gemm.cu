@@ -11,8 +11,8 @@
 // coefficients (channels) of a tile, the units are dealt over all SMs, both operands arrive by
 // tiled TMA copies with 128-byte swizzle, and the coder's chunks run side by side over the chip.
 // The workspace traffic (2 bytes per value written and read) stays in the 126 MB L2 for the most part.
-// 576x14x14 x 128: encode 132 -> 62 us, decode 108 -> 62;
-// 960x7x7 x 128: encode 140 -> 52, decode 140 -> 49; 512x7x7 x 64: encode 52 -> 30, decode 46 -> 27.
+// 576x14x14 x 128: encode 132 -> 60 us, decode 108 -> 56;
+// 960x7x7 x 128: encode 140 -> 48, decode 140 -> 45; 512x7x7 x 64: encode 52 -> 25, decode 46 -> 21.
 // The product itself is bound by the operands' way from L2 (48 KB per 64 of the depth, at about 32 bytes a cycle
 // and SM); one copy per operand and stage, since a producer thread issues one in about 100 cycles.
 //
@@ -308,6 +308,21 @@ int best_columns(long long tiles, int k, int sm_count)
     return best;
 }
 
+// Pixels per unit of the inverse: 64 to 256 in steps of a transposed pass, where the rounds of the grid are cheapest.  A unit
+// costs what its operands bring from L2, its pixels and 128 channels.  Against 256, or 128 or 64 while that left SMs
+// idle: 512x7x7 x 64 (one round of 96 instead of two of 64) 23.2 -> 21.1 us, 960x7x7 x 128 46.9 -> 45.2, 576x14x14 x 128
+// 56.5 -> 56.0, 128x28x28 x 64 per channel 29.3 -> 27.4.
+int best_pixels(long long pixels, int blocks, int sm_count)
+{
+    int best = 0;
+    long long best_cost = 0;
+    for (int n = kMaxN; n >= 64; n -= 32) {
+        const long long units = (pixels + n - 1) / n * blocks, cost = (units + sm_count - 1) / sm_count * (n + 128);
+        if (best == 0 || cost < best_cost) { best = n; best_cost = cost; }
+    }
+    return best;
+}
+
 template <bool kEncode>
 tc_status launch_gemm(int sms, bool early, const GemmArgs &g, const CUtensorMap &map_a, const CUtensorMap &map_b, cudaStream_t s)
 {
@@ -387,9 +402,7 @@ tc_status tc_launch_decode_wide_gemm(const tc_ctx *ctx, const DecodeArgs &a, voi
         g.n_panels = (a.k + kPanelK - 1) / kPanelK;
         g.k_depth = a.k;
         g.blocks = (a.c + 127) / 128;
-        // 256 pixels a unit; 128 or 64 while that leaves SMs without one
-        g.n_cols = kMaxN;
-        while (g.n_cols > 64 && ((p1 - p0 + g.n_cols - 1) / g.n_cols) * g.blocks < a.sms) g.n_cols /= 2;
+        g.n_cols = best_pixels(p1 - p0, g.blocks, a.sms);
         g.units = ((p1 - p0 + g.n_cols - 1) / g.n_cols) * g.blocks;
         CUtensorMap map_q;
         if (!tc_tensor_map_sw128(&map_q, q, p1 - p0, a.k, g.n_cols)) return TC_ERR_CUDA;
