@@ -1118,6 +1118,21 @@ static std::vector<int> by_descending_work(int n, const std::vector<double> &wor
     return order;
 }
 
+// Workspaces of a list's tensors: the tensors of one stream follow each other and share one, as large as the largest of
+// them wants, so that a list of any length holds at most kManyStreams workspaces.  at[i] = byte offset; returns the end.
+static size_t stream_workspaces(const std::vector<int> &order, int n_streams, const std::vector<size_t> &bytes, size_t base, std::vector<size_t> &at)
+{
+    for (int j = 0; j < n_streams; ++j) {
+        size_t most = 0;
+        for (size_t r = j; r < order.size(); r += n_streams) {
+            most = std::max(most, bytes[order[r]]);
+            at[order[r]] = base;
+        }
+        base += (most + 255) & ~(size_t)255;
+    }
+    return base;
+}
+
 tc_status tc_encode_many(tc_ctx *ctx, const tc_encode_item *items, int32_t n_items, void *cuda_stream)
 {
     if (!ctx || n_items < 0 || (n_items > 0 && !items)) return TC_ERR_INVALID_ARG;
@@ -1126,9 +1141,9 @@ tc_status tc_encode_many(tc_ctx *ctx, const tc_encode_item *items, int32_t n_ite
     cudaStream_t s = (cudaStream_t)cuda_stream;
     // every item is checked before anything is launched
     std::vector<ChunkShape> shape(n_items);
-    std::vector<size_t> lookback_at(n_items), symbols_at(n_items, 0);
+    std::vector<size_t> lookback_at(n_items), symbols_at(n_items, 0), symbols_bytes(n_items, 0);
     std::vector<double> work(n_items);
-    size_t lookback_total = 0, total = 0;
+    size_t lookback_total = 0;
     for (int i = 0; i < n_items; ++i) {
         const tc_encode_item &it = items[i];
         if (!it.tile_off) return TC_ERR_INVALID_ARG;
@@ -1143,26 +1158,16 @@ tc_status tc_encode_many(tc_ctx *ctx, const tc_encode_item *items, int32_t n_ite
         lookback_total += (kEncodeScratchHeader + (size_t)n_tiles * sizeof(unsigned long long) + 255) & ~(size_t)255;
         work[i] = (double)pixels * it.x->c;
     }
-    total = lookback_total;
-    for (int i = 0; i < n_items; ++i) {
-        const tc_encode_item &it = items[i];
-        const long long pixels = (long long)it.x->n * it.x->h * it.x->w;
-        const long long n_tiles = (pixels + TC_TILE_PIXELS - 1) / TC_TILE_PIXELS;
-        const size_t bytes = n_tiles > 0 ? encode_work_bytes(ctx, it.model, it.x) : 0;
-        if (bytes) {
-            symbols_at[i] = total;
-            total += bytes;
-        }
-    }
-    tc_status st = ensure_scratch(ctx, total);
+    const int n_streams = std::min(kManyStreams, (int)n_items);
+    const std::vector<int> order = by_descending_work(n_items, work);
+    for (int i = 0; i < n_items; ++i) symbols_bytes[i] = work[i] > 0.0 ? encode_work_bytes(ctx, items[i].model, items[i].x) : 0;
+    tc_status st = ensure_scratch(ctx, stream_workspaces(order, n_streams, symbols_bytes, lookback_total, symbols_at));
     if (st != TC_OK) return st;
     if ((st = ensure_many_streams(ctx)) != TC_OK) return st;
     // one clear for the look-back state of all items, then the items fan out over the streams
     TC_CUDA(cudaMemsetAsync(ctx->scratch, 0, lookback_total, s));
     TC_CUDA(cudaEventRecord(ctx->many_fork, s));
-    const int n_streams = std::min(kManyStreams, (int)n_items);
     for (int j = 0; j < n_streams; ++j) TC_CUDA(cudaStreamWaitEvent(ctx->many_streams[j], ctx->many_fork, 0));
-    const std::vector<int> order = by_descending_work(n_items, work);
     tc_status first_error = TC_OK;
     for (int r = 0; r < n_items; ++r) {
         const int i = order[r];
@@ -1173,7 +1178,7 @@ tc_status tc_encode_many(tc_ctx *ctx, const tc_encode_item *items, int32_t n_ite
         if (pixels == 0) { if (cudaMemsetAsync(it.tile_off, 0, sizeof(uint64_t), ws) != cudaSuccess && first_error == TC_OK) first_error = TC_ERR_CUDA; continue; }
         st = tc_encode_with_scratch(ctx, it.model, it.codebook, it.x, shape[i].cp, shape[i].splits, it.stream_out, it.capacity,
                                     it.chunk_len, it.tile_off, nullptr, (char *)ctx->scratch + lookback_at[i],
-                                    symbols_at[i] ? (char *)ctx->scratch + symbols_at[i] : nullptr, ws, nullptr, nullptr, list_sms);
+                                    symbols_bytes[i] ? (char *)ctx->scratch + symbols_at[i] : nullptr, ws, nullptr, nullptr, list_sms);
         if (st != TC_OK && first_error == TC_OK) first_error = st;
     }
     for (int j = 0; j < n_streams; ++j) {
@@ -1191,7 +1196,6 @@ tc_status tc_decode_many(tc_ctx *ctx, const tc_decode_item *items, int32_t n_ite
     cudaStream_t s = (cudaStream_t)cuda_stream;
     std::vector<size_t> symbols_at(n_items, 0), symbols_bytes(n_items, 0);
     std::vector<double> work(n_items);
-    size_t total = 0;
     for (int i = 0; i < n_items; ++i) {
         const tc_decode_item &it = items[i];
         const tc_status st = check_codec_args(it.model, it.codebook, it.x_hat);
@@ -1203,17 +1207,16 @@ tc_status tc_decode_many(tc_ctx *ctx, const tc_decode_item *items, int32_t n_ite
                            ((uintptr_t)it.chunk_len & 3u) != 0))
             return TC_ERR_INVALID_ARG;
         symbols_bytes[i] = decode_scratch_bytes(ctx, it.model, it.codebook, it.x_hat);
-        symbols_at[i] = total;
-        total += symbols_bytes[i];
         work[i] = (double)pixels * it.x_hat->c;
     }
     tc_status st;
+    const int n_streams = std::min(kManyStreams, (int)n_items);
+    const std::vector<int> order = by_descending_work(n_items, work);
+    const size_t total = stream_workspaces(order, n_streams, symbols_bytes, 0, symbols_at);
     if (total && (st = ensure_scratch(ctx, total)) != TC_OK) return st;
     if ((st = ensure_many_streams(ctx)) != TC_OK) return st;
     TC_CUDA(cudaEventRecord(ctx->many_fork, s));
-    const int n_streams = std::min(kManyStreams, (int)n_items);
     for (int j = 0; j < n_streams; ++j) TC_CUDA(cudaStreamWaitEvent(ctx->many_streams[j], ctx->many_fork, 0));
-    const std::vector<int> order = by_descending_work(n_items, work);
     tc_status first_error = TC_OK;
     for (int r = 0; r < n_items; ++r) {
         const int i = order[r];
