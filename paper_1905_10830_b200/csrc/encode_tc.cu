@@ -250,7 +250,7 @@ __global__ void __launch_bounds__(kThreads, 1) encode_tc_kernel(EncodeArgs a, Pl
         const int ch0 = (lw & 1) + 2 * (lane >> 4) + 4 * (lw >> 1);  // channels ch0, ch0 + 8, ... of a panel
         const uint32_t dst0 = (uint32_t)((px >> 6) * (kStageBytes / 2) + ch0 * 128 + ((((px & 63) >> 3) ^ ch0) << 4));
         const __nv_bfloat16 *xin = reinterpret_cast<const __nv_bfloat16 *>(a.x);
-        const uint32_t row8 = 16u * (uint32_t)a.hw;   // bytes from a channel to the eighth after it
+        const size_t row8 = 16 * (size_t)a.hw;        // bytes from a channel to the eighth after it; a panel (four of them) passes 4 GB at 2^26 pixels a map
         static_assert(kPanelCh == 32, "a lane copies four channels of a panel");
         int s = 0;                                 // ring stage of the next panel
         uint32_t phase = 1;
@@ -272,8 +272,8 @@ __global__ void __launch_bounds__(kThreads, 1) encode_tc_kernel(EncodeArgs a, Pl
                     cp_async_16(dst, src, 16u);
                     cp_async_16(dst + 1024u, src + row8, 16u);
                     if (full) {
-                        cp_async_16(dst + 2048u, src + 2u * row8, 16u);
-                        cp_async_16(dst + 3072u, src + 3u * row8, 16u);
+                        cp_async_16(dst + 2048u, src + 2 * row8, 16u);
+                        cp_async_16(dst + 3072u, src + 3 * row8, 16u);
                     }
                 } else {
                     cp_async_8(dst, src, n1);
@@ -281,14 +281,14 @@ __global__ void __launch_bounds__(kThreads, 1) encode_tc_kernel(EncodeArgs a, Pl
                     cp_async_8(dst + 1024u, src + row8, n1);
                     cp_async_8(dst + 1032u, src2 + row8, n2);
                     if (full) {
-                        cp_async_8(dst + 2048u, src + 2u * row8, n1);
-                        cp_async_8(dst + 2056u, src2 + 2u * row8, n2);
-                        cp_async_8(dst + 3072u, src + 3u * row8, n1);
-                        cp_async_8(dst + 3080u, src2 + 3u * row8, n2);
+                        cp_async_8(dst + 2048u, src + 2 * row8, n1);
+                        cp_async_8(dst + 2056u, src2 + 2 * row8, n2);
+                        cp_async_8(dst + 3072u, src + 3 * row8, n1);
+                        cp_async_8(dst + 3080u, src2 + 3 * row8, n2);
                     }
                 }
-                src += 4u * row8;
-                src2 += 4u * row8;
+                src += 4 * row8;
+                src2 += 4 * row8;
                 // the stage's barrier gets this thread's arrival when its copies have landed: the thread goes
                 // on to the next stage, so that all free stages are in flight (with a wait for the panel
                 // before the last the loads were bound by their latency, two panels at a time)

@@ -195,3 +195,25 @@ def test_covariance_blocks(ctx, c, h, w, n, dtype):
     got = basis.T @ (eig[:, None] * basis)
     assert np.abs(got - want).max() <= 2.0 ** -22 * eig.max()
     m.close()
+
+
+# One map of 2^26 pixels: the channels that a loader copies together lie further apart than 32 bits count.  The
+# same pixels as sixteen maps are the same stream.
+def test_channels_more_than_4_gb_apart(ctx):
+    c, side, parts = 48, 8192, 16
+    g = torch.Generator(device="cuda").manual_seed(17)
+    x = torch.empty(1, c, side, side, dtype=torch.bfloat16, device="cuda")
+    for i in range(c):
+        x[0, i] = torch.randn(side, side, generator=g, device="cuda")
+    cal = x[:, :, :64, :64].contiguous()
+    m = tc.tc_fit_pca(ctx, cal, 4)
+    cb = tc.tc_build_codebook(ctx, m, tc.tc_stats(ctx, m, None, cal).hist)
+    enc = tc.tc_encode(ctx, m, cb, x)
+    assert tc.tc_get_status(ctx) == 0 and tc.tc_last_path(ctx) == 1
+    y = x.view(c, parts, side // parts, side).permute(1, 0, 2, 3).contiguous()
+    assert _same_stream(enc, tc.tc_encode(ctx, m, cb, y))
+    a = tc.tc_decode(ctx, m, cb, enc, x.shape, x.dtype)
+    b = tc.tc_decode(ctx, m, cb, enc, y.shape, y.dtype)
+    assert tc.tc_get_status(ctx) == 0
+    assert torch.equal(a.view(c, parts, side // parts, side).permute(1, 0, 2, 3), b)
+    m.close(); cb.close()
