@@ -400,9 +400,18 @@ __global__ void __launch_bounds__(kThreads, 1) encode_tc_kernel(EncodeArgs a, Pl
         const int bar_id = 1 + grp;
         bool alive = true;
         [[maybe_unused]] const int skip_blk = pl.skip_blk;
-        // a position nearer to the modal level than this rounds to it, whatever the last bits of the
-        // two ways to compute it (they agree to 1e-6 of a level)
-        [[maybe_unused]] const float skip_dist = 0.499f / top;
+        // A position nearer to the modal level than this rounds to it, whichever of the two ways it is computed:
+        // they differ by the rounding of s_bias_mid and of the two results, together at most 2^-24 of the
+        // bias's size plus three; four times that is kept clear.  (At 8 bits and a mean of a thousand ranges that is
+        // 0.06 of a level; a fixed 0.001 let symbols one off the quantiser's pass for the modal one there.)
+        [[maybe_unused]] float skip_dist = 0.f;
+        if constexpr (kCanSkip) {
+            float most = 0.f;
+            for (int i = lane; i < a.k; i += 32) most = fmaxf(most, fabsf(s_bias[i]));
+#pragma unroll
+            for (int d = 16; d > 0; d >>= 1) most = fmaxf(most, __shfl_xor_sync(0xffffffffu, most, d));
+            skip_dist = 0.499f / top - (most + 1.f) * 2.4e-7f;
+        }
         const uint32_t trow = tmem_base + grp * kAccCols + ((uint32_t)(wq * 32) << 16);
 
         auto resolve_base = [&](long long tile, unsigned long long padded) {

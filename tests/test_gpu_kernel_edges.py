@@ -217,3 +217,26 @@ def test_channels_more_than_4_gb_apart(ctx):
     assert tc.tc_get_status(ctx) == 0
     assert torch.equal(a.view(c, parts, side // parts, side).permute(1, 0, 2, 3), b)
     m.close(); cb.close()
+
+
+# Blocks of modal symbols are passed over after a test that adds the bias up differently from the quantiser.  With a mean of
+# 2048 quantiser ranges (identity basis, channel 5 `d` of a level above the modal one) fp32 places the two up to
+# 0.03 of a level apart: a position next to the rounding boundary must not pass as the modal symbol.  The debug
+# outputs switch the passing over off.
+@pytest.mark.parametrize("d", [0.486, 0.499, 0.501, 0.515])
+def test_passing_over_modal_blocks_far_from_zero_mean(ctx, d):
+    c, bits, modal, offset = 64, 8, 127, 2048.0
+    mean = np.full(c, offset)
+    mean[5] -= d / 255
+    m = tc.tc_model_import(ctx, basis=np.eye(c), mean=mean, lo=-modal / 255, step=1 / 255, bits=bits, basis_dtype=1, eig=np.full(c, 1e-12))
+    counts = np.ones(256, dtype=np.uint64)
+    counts[modal] = 1 << 30
+    cb = tc.tc_codebook_import(ctx, tc.tc_host_huffman_lengths(counts, 12), bits)
+    x = torch.full((2, c, 16, 16), offset, dtype=torch.bfloat16, device="cuda")
+    enc = tc.tc_encode(ctx, m, cb, x)
+    dbg = tc.tc_encode(ctx, m, cb, x, debug=True)
+    assert tc.tc_get_status(ctx) == 0 and tc.tc_last_path(ctx) == 1
+    q = dbg.symbols.cpu().numpy()
+    assert np.all(np.delete(q, 5, axis=1) == modal) and np.all((q[:, 5] == modal) | (q[:, 5] == modal + 1))
+    assert _same_stream(enc, dbg)
+    m.close(); cb.close()
