@@ -1071,7 +1071,9 @@ tc_status tc_decode(tc_ctx *ctx, const tc_model *m, const tc_codebook *cb, const
                     const uint16_t *chunk_len, const uint64_t *tile_off, const tc_encode_params *params,
                     const tc_tensor *x_hat, void *cuda_stream)
 {
-    if (!ctx || !m || !valid_tensor(x_hat)) return TC_ERR_INVALID_ARG;
+    if (!ctx) return TC_ERR_INVALID_ARG;
+    const tc_status args = check_codec_args(m, cb, x_hat);      // ahead of the workspace, whose size depends on them
+    if (args != TC_OK) return args;
     DeviceGuard guard(ctx->device);
     const size_t scratch = decode_scratch_bytes(ctx, m, cb, x_hat);
     if (scratch) {

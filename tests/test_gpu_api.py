@@ -346,3 +346,25 @@ def test_stats_on_the_tensor_core_kernels(ctx, c, s, n, bits, with_cb):
     for h in (m, cb, cb_any):
         if h is not None:
             h.close()
+
+
+def test_decode_without_a_handle_or_tensor_is_refused(ctx):
+    # the C ABI's own checks: a missing model, code table or tensor is an invalid argument on every route
+    import ctypes as C
+    lib = tc.load_library()
+    for c, dtype in ((64, torch.bfloat16), (320, torch.bfloat16), (64, torch.float32)):
+        spec = fm.LayerSpec(c, 7, 7, 0.9, None, 530 + c)
+        o = H.oracle_side(spec, 4, 2 * c // 49 + 1, 2, dtype, False)
+        m = H.import_model(tc, ctx, o["model"], dtype)
+        cb = tc.tc_codebook_import(ctx, o["lengths"], 4)
+        x = o["x"].cuda()
+        enc = tc.tc_encode(ctx, m, cb, x)
+        out = torch.empty_like(x)
+        t = tc.binding._tensor(out)
+        args = [ctx.ptr, m.ptr, cb.ptr, enc.words.data_ptr(), enc.words.numel(), enc.chunk_len.data_ptr(), enc.tile_off.data_ptr(), None,
+                C.byref(t), None]
+        assert lib.tc_decode(*args) == 0
+        for missing in (0, 1, 2, 3, 5, 6, 8):
+            assert lib.tc_decode(*[None if i == missing else a for i, a in enumerate(args)]) == 1
+        assert tc.tc_get_status(ctx) == 0
+        m.close(); cb.close()
