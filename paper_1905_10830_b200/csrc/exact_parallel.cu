@@ -501,7 +501,18 @@ __global__ void __launch_bounds__(kUnpackThreads) unpack_symbols_kernel(DecodeAr
     const long long tile = first_tile + blockIdx.x;
     const unsigned long long base = a.tile_off[tile], end = a.tile_off[tile + 1];
     const bool tile_ok = (base & 127ull) == 0 && (end & 127ull) == 0 && base <= end && end <= a.stream_bits;
+    // Rows that are not decoded hold the zero level (centred: 0; with kFull, whose lanes keep step, what zero bits
+    // decode to), not what the workspace held before.
+    const long long row0 = (tile - first_tile) * TC_TILE_PIXELS;
+    auto clear = [&](int px, int j, int n) {                  // n coefficients from j on of a pixel of the tile
+        for (int i = j; i < j + n; ++i) {
+            if constexpr (kOperand) ((uint16_t *)out)[(row0 + px) * a.k + i] = 0;
+            else ((uint8_t *)out)[(row0 + px) * a.k + i] = (uint8_t)a.center;
+        }
+    };
+    const int n_px = (int)min((long long)TC_TILE_PIXELS, a.pixels - tile * TC_TILE_PIXELS);
     if (!tile_ok) {
+        for (int px = t; px < n_px; px += blockDim.x) clear(px, 0, a.k);
         if (t == 0) tc_dev_set_status(a.status, TC_ERR_CORRUPT_STREAM);
         return;
     }
@@ -643,6 +654,9 @@ __global__ void __launch_bounds__(kUnpackThreads) unpack_symbols_kernel(DecodeAr
     };
     const bool walks = mine && !bad;
     if (!kFull && !walks) {
+        if (a.splits > 1) clear(t % TC_TILE_PIXELS, part * (a.k / a.splits), a.k / a.splits);
+        else
+            for (int px = t * a.chunk_pixels; px < min((t + 1) * a.chunk_pixels, n_px); ++px) clear(px, 0, a.k);
     } else if (staged) {
         StagedReader r;
         r.init(seg, walks ? off : 0u, walks ? seg + (uint32_t)((end - base) >> 3) : seg);

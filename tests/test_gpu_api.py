@@ -368,3 +368,34 @@ def test_decode_without_a_handle_or_tensor_is_refused(ctx):
             assert lib.tc_decode(*[None if i == missing else a for i, a in enumerate(args)]) == 1
         assert tc.tc_get_status(ctx) == 0
         m.close(); cb.close()
+
+
+@pytest.mark.parametrize("c,s,n,dtype,per_channel", [(320, 7, 9, torch.bfloat16, False), (64, 14, 9, torch.bfloat16, True),
+                                                     (320, 14, 500, torch.bfloat16, False), (512, 7, 4, torch.float32, True),
+                                                     (48, 9, 7, torch.float32, False)])
+def test_corrupt_tiles_show_nothing_of_earlier_calls(c, s, n, dtype, per_channel):
+    # tiles whose offsets or chunk lengths cannot be valid are reported, and what is decoded in their place does not
+    # depend on what the context's workspace held: two contexts with different pasts return the same tensor
+    params = fm.layer_params(fm.LayerSpec(c, s, s, 0.9, None, 540 + c))
+    cal = fm.make_maps(params, max(8, 2 * c // (s * s) + 1), calib=True, dtype=dtype, device="cuda")
+    x = fm.make_maps(params, n, dtype=dtype, device="cuda")
+    outs = []
+    for past in (0, 1):
+        own = tc.tc_create(0)
+        m = tc.tc_fit_pca(own, cal, 4, eigensolver=tc.TC_EIG_HOST)
+        groups = c if per_channel else 1
+        cb = tc.tc_build_codebook(own, m, tc.tc_stats(own, m, None, cal, groups=groups).hist, groups=groups)
+        enc = tc.tc_encode(own, m, cb, x)
+        before = x.flip(0).contiguous() if past else torch.full_like(x, 3.0)
+        tc.tc_decode(own, m, cb, tc.tc_encode(own, m, cb, before), x.shape, dtype)
+        assert tc.tc_get_status(own) == 0
+        broken = tc.EncodedStream(enc.words, enc.chunk_len.clone(), enc.tile_off.clone(), enc.layout)
+        broken.tile_off[1] += 64                               # the first two tiles
+        broken.chunk_len[enc.layout.n_chunks - 1] = 30000      # and the last chunk
+        out = tc.tc_decode(own, m, cb, broken, x.shape, dtype)
+        assert tc.tc_get_status(own) == 5
+        assert bool(torch.isfinite(out.float()).all())
+        outs.append(out)
+        for h in (m, cb, own):
+            h.close()
+    assert torch.equal(outs[0], outs[1])
