@@ -685,8 +685,16 @@ __global__ void __launch_bounds__(kThreads, 1) encode_tc_kernel(EncodeArgs a, Pl
             // fit before the end
             const unsigned int tile_bytes = staged ? (unsigned int)(padded >> 3) : 0u;
             const unsigned int stg_at = prev_end + tile_bytes > pl.staging_bytes ? 0u : prev_end;
-            if (n_done >= 1 && stg_at < prev_end && prev_at < stg_at + tile_bytes &&
-                !mbar_wait(smem_u32(&s_stg_free[grp][(n_done - 1) % kSlots]), ((n_done - 1) / kSlots) & 1u)) { alive = false; break; }
+            if (n_done >= 1 && stg_at < prev_end && prev_at < stg_at + tile_bytes) {
+                // one warp waits for all (the condition is the same in every thread): warps whose waits end
+                // differently would leave the others at the group's barriers
+                if (wg == 0) {
+                    const bool go = mbar_wait(smem_u32(&s_stg_free[grp][(n_done - 1) % kSlots]), ((n_done - 1) / kSlots) & 1u);
+                    if (lane == 0) s_go[grp] = go;
+                }
+                named_bar_sync(bar_id, 256);
+                if (!s_go[grp]) { alive = false; break; }
+            }
             prev_at = stg_at;
             prev_end = stg_at + tile_bytes;
             const uint32_t tile_addr = stg_addr + stg_at;

@@ -240,3 +240,28 @@ def test_passing_over_modal_blocks_far_from_zero_mean(ctx, d):
     assert np.all(np.delete(q, 5, axis=1) == modal) and np.all((q[:, 5] == modal) | (q[:, 5] == modal + 1))
     assert _same_stream(enc, dbg)
     m.close(); cb.close()
+
+
+# Resident-basis encoder with several tiles per group and staging buffers that hold one, one and a half or many of
+# them: the place of a new tile has to wait for the copy of the one before.  The same maps in pieces of one tile per
+# block write the same words.
+@pytest.mark.parametrize("c,bits,ratio", [(256, 8, 0.9), (256, 8, 0.99), (256, 6, 0.97), (208, 7, 0.98), (64, 8, 0.98)])
+def test_staging_ring_of_the_resident_encoder(ctx, c, bits, ratio):
+    params = fm.layer_params(fm.LayerSpec(c, 14, 14, ratio, None, 15000 + c + bits))
+    cal = fm.make_maps(params, 256, calib=True, dtype=torch.bfloat16, device="cuda")
+    m = tc.tc_fit_pca(ctx, cal, bits)
+    cb = tc.tc_build_codebook(ctx, m, tc.tc_stats(ctx, m, None, cal).hist)
+    x = fm.make_maps(params, 32 * 40, dtype=torch.bfloat16, device="cuda")             # 1960 tiles, pieces of 49
+    enc = tc.tc_encode(ctx, m, cb, x)
+    assert tc.tc_get_status(ctx) == 0 and tc.tc_last_path(ctx) == 1
+    base, chunks = 0, 0
+    for i in range(0, x.shape[0], 32):
+        part = tc.tc_encode(ctx, m, cb, x[i:i + 32])
+        assert tc.tc_get_status(ctx) == 0
+        n, bits_n, t0 = part.total_bits() // 8, part.total_bits(), i // 32 * 49
+        assert torch.equal(enc.words[base // 8: base // 8 + n], part.words[:n])
+        assert torch.equal(enc.tile_off[t0:t0 + 50] - base, part.tile_off)
+        assert torch.equal(enc.chunk_len[chunks:chunks + part.layout.n_chunks], part.chunk_len[:part.layout.n_chunks])
+        base, chunks = base + bits_n, chunks + part.layout.n_chunks
+    assert base == enc.total_bits()
+    m.close(); cb.close()
