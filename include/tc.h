@@ -22,6 +22,11 @@
  *     different streams, no dependency between them -- corrupt each other's output.  Use one
  *     context per concurrent stream; models and codebooks may be shared between contexts of the
  *     same device.
+ *   - tc_encode, tc_decode and their list forms may be captured into a CUDA graph, also as the first call of a
+ *     context: a captured call takes its scratch from the graph (stream-ordered allocation and release
+ *     inside it), not from the arena, so that later calls of the context do not disturb a replay.  A graph's
+ *     replays and other calls on the same context follow the rule above as far as the status word is
+ *     concerned; two replays of one graph must not overlap.
  *   - Errors are return codes.  Argument errors are found on the host before any launch.
  *     Conditions only the device can see (corrupt stream, output capacity exceeded at run
  *     time, a bounded wait that ran out) are recorded in a per-context status word and

@@ -119,6 +119,34 @@ tc_status ensure_scratch(tc_ctx *ctx, size_t bytes)
     return TC_OK;
 }
 
+// The memory one call's kernels share: the context's arena, or -- while the stream is being captured -- memory of
+// the graph's own.  A captured call is replayed long after the arena may have moved to make room for a larger tensor, and
+// the arena cannot grow during a capture.
+struct CallScratch {
+    char *at = nullptr;
+    cudaStream_t stream = nullptr;
+    bool of_graph = false;
+    ~CallScratch() { if (of_graph && cudaFreeAsync(at, stream) != cudaSuccess) cudaGetLastError(); }
+};
+
+tc_status call_scratch(tc_ctx *ctx, size_t bytes, cudaStream_t s, CallScratch *out)
+{
+    if (bytes == 0) return TC_OK;
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &capture) != cudaSuccess) cudaGetLastError();
+    if (capture == cudaStreamCaptureStatusNone) {
+        const tc_status st = ensure_scratch(ctx, bytes);
+        out->at = (char *)ctx->scratch;
+        return st;
+    }
+    void *mem = nullptr;
+    TC_CUDA(cudaMallocAsync(&mem, bytes, s));
+    out->at = (char *)mem;
+    out->stream = s;
+    out->of_graph = true;
+    return TC_OK;
+}
+
 // The host copy of a model's basis, fetched from the device at first use.
 const std::vector<double> *host_basis(const tc_model *m)
 {
@@ -966,9 +994,10 @@ tc_status tc_encode(tc_ctx *ctx, const tc_model *m, const tc_codebook *cb, const
     }
     const size_t lookback = (kEncodeScratchHeader + (size_t)n_tiles * sizeof(unsigned long long) + 255) & ~(size_t)255;
     const size_t work = encode_work_bytes(ctx, m, x);
-    if ((st = ensure_scratch(ctx, lookback + work)) != TC_OK) return st;
+    CallScratch scratch;
+    if ((st = call_scratch(ctx, lookback + work, s, &scratch)) != TC_OK) return st;
     return tc_encode_with_scratch(ctx, m, cb, x, cs.cp, cs.splits, stream_out, capacity, chunk_len, tile_off, debug,
-                                  ctx->scratch, work ? (char *)ctx->scratch + lookback : nullptr, s);
+                                  scratch.at, work ? scratch.at + lookback : nullptr, s);
 }
 
 // bf16 tensors decoded by the entropy decoder and the tiled product in kernels of their own: wide layers, and per-channel
@@ -1075,13 +1104,10 @@ tc_status tc_decode(tc_ctx *ctx, const tc_model *m, const tc_codebook *cb, const
     const tc_status args = check_codec_args(m, cb, x_hat);      // ahead of the workspace, whose size depends on them
     if (args != TC_OK) return args;
     DeviceGuard guard(ctx->device);
-    const size_t scratch = decode_scratch_bytes(ctx, m, cb, x_hat);
-    if (scratch) {
-        const tc_status st = ensure_scratch(ctx, scratch);
-        if (st != TC_OK) return st;
-    }
-    return decode_with_scratch(ctx, m, cb, stream, stream_bytes, chunk_len, tile_off, params, x_hat,
-                               scratch ? (uint8_t *)ctx->scratch : nullptr, 0, cuda_stream);
+    CallScratch scratch;
+    const tc_status st = call_scratch(ctx, decode_scratch_bytes(ctx, m, cb, x_hat), (cudaStream_t)cuda_stream, &scratch);
+    if (st != TC_OK) return st;
+    return decode_with_scratch(ctx, m, cb, stream, stream_bytes, chunk_len, tile_off, params, x_hat, (uint8_t *)scratch.at, 0, cuda_stream);
 }
 
 // ---- several tensors per call --------------------------------------------------------------------
@@ -1163,11 +1189,12 @@ tc_status tc_encode_many(tc_ctx *ctx, const tc_encode_item *items, int32_t n_ite
     const int n_streams = std::min(kManyStreams, (int)n_items);
     const std::vector<int> order = by_descending_work(n_items, work);
     for (int i = 0; i < n_items; ++i) symbols_bytes[i] = work[i] > 0.0 ? encode_work_bytes(ctx, items[i].model, items[i].x) : 0;
-    tc_status st = ensure_scratch(ctx, stream_workspaces(order, n_streams, symbols_bytes, lookback_total, symbols_at));
+    tc_status st = ensure_many_streams(ctx);
     if (st != TC_OK) return st;
-    if ((st = ensure_many_streams(ctx)) != TC_OK) return st;
+    CallScratch scratch;
+    if ((st = call_scratch(ctx, stream_workspaces(order, n_streams, symbols_bytes, lookback_total, symbols_at), s, &scratch)) != TC_OK) return st;
     // one clear for the look-back state of all items, then the items fan out over the streams
-    TC_CUDA(cudaMemsetAsync(ctx->scratch, 0, lookback_total, s));
+    TC_CUDA(cudaMemsetAsync(scratch.at, 0, lookback_total, s));
     TC_CUDA(cudaEventRecord(ctx->many_fork, s));
     for (int j = 0; j < n_streams; ++j) TC_CUDA(cudaStreamWaitEvent(ctx->many_streams[j], ctx->many_fork, 0));
     tc_status first_error = TC_OK;
@@ -1179,8 +1206,8 @@ tc_status tc_encode_many(tc_ctx *ctx, const tc_encode_item *items, int32_t n_ite
         const long long pixels = (long long)it.x->n * it.x->h * it.x->w;
         if (pixels == 0) { if (cudaMemsetAsync(it.tile_off, 0, sizeof(uint64_t), ws) != cudaSuccess && first_error == TC_OK) first_error = TC_ERR_CUDA; continue; }
         st = tc_encode_with_scratch(ctx, it.model, it.codebook, it.x, shape[i].cp, shape[i].splits, it.stream_out, it.capacity,
-                                    it.chunk_len, it.tile_off, nullptr, (char *)ctx->scratch + lookback_at[i],
-                                    symbols_bytes[i] ? (char *)ctx->scratch + symbols_at[i] : nullptr, ws, nullptr, nullptr, list_sms);
+                                    it.chunk_len, it.tile_off, nullptr, scratch.at + lookback_at[i],
+                                    symbols_bytes[i] ? scratch.at + symbols_at[i] : nullptr, ws, nullptr, nullptr, list_sms);
         if (st != TC_OK && first_error == TC_OK) first_error = st;
     }
     for (int j = 0; j < n_streams; ++j) {
@@ -1214,9 +1241,9 @@ tc_status tc_decode_many(tc_ctx *ctx, const tc_decode_item *items, int32_t n_ite
     tc_status st;
     const int n_streams = std::min(kManyStreams, (int)n_items);
     const std::vector<int> order = by_descending_work(n_items, work);
-    const size_t total = stream_workspaces(order, n_streams, symbols_bytes, 0, symbols_at);
-    if (total && (st = ensure_scratch(ctx, total)) != TC_OK) return st;
     if ((st = ensure_many_streams(ctx)) != TC_OK) return st;
+    CallScratch scratch;
+    if ((st = call_scratch(ctx, stream_workspaces(order, n_streams, symbols_bytes, 0, symbols_at), s, &scratch)) != TC_OK) return st;
     TC_CUDA(cudaEventRecord(ctx->many_fork, s));
     for (int j = 0; j < n_streams; ++j) TC_CUDA(cudaStreamWaitEvent(ctx->many_streams[j], ctx->many_fork, 0));
     tc_status first_error = TC_OK;
@@ -1225,7 +1252,7 @@ tc_status tc_decode_many(tc_ctx *ctx, const tc_decode_item *items, int32_t n_ite
         const tc_decode_item &it = items[i];
         const int list_sms = list_share(ctx->sm_count, n_streams, work, i);
         st = decode_with_scratch(ctx, it.model, it.codebook, it.stream, it.stream_bytes, it.chunk_len, it.tile_off, it.params,
-                                 it.x_hat, symbols_bytes[i] ? (uint8_t *)ctx->scratch + symbols_at[i] : nullptr,
+                                 it.x_hat, symbols_bytes[i] ? (uint8_t *)scratch.at + symbols_at[i] : nullptr,
                                  list_sms, ctx->many_streams[r % n_streams]);
         if (st != TC_OK && first_error == TC_OK) first_error = st;
     }

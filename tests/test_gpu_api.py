@@ -399,3 +399,63 @@ def test_corrupt_tiles_show_nothing_of_earlier_calls(c, s, n, dtype, per_channel
         for h in (m, cb, own):
             h.close()
     assert torch.equal(outs[0], outs[1])
+
+
+# (C, side, batch, dtype, one table per channel): resident-basis kernels, tiled products of more and of less than 8 MB of
+# workspace, per-channel codes, the fp64 kernels
+CAPTURED = [(64, 14, 40, torch.bfloat16, False), (960, 7, 128, torch.bfloat16, False), (320, 14, 6, torch.bfloat16, False),
+            (256, 14, 300, torch.bfloat16, True), (48, 12, 3, torch.float32, True)]
+
+
+def _fitted_layers(ctx, shapes):
+    layers = []
+    for c, s, n, dtype, per_channel in shapes:
+        params = fm.layer_params(fm.LayerSpec(c, s, s, 0.9, None, 560 + c))
+        cal = fm.make_maps(params, max(8, 2 * c // (s * s) + 1), calib=True, dtype=dtype, device="cuda")
+        m = tc.tc_fit_pca(ctx, cal, 4)
+        groups = c if per_channel else 1
+        cb = tc.tc_build_codebook(ctx, m, tc.tc_stats(ctx, m, None, cal, groups=groups).hist, groups=groups)
+        layers.append((m, cb, fm.make_maps(params, n, dtype=dtype, device="cuda")))
+    return layers
+
+
+@pytest.mark.parametrize("as_list", [False, True])
+def test_captured_calls_keep_their_scratch(ctx, as_list):
+    # the first calls of a context, captured; then calls that make its arena grow; then the graph once more, on new maps
+    layers = _fitted_layers(ctx, CAPTURED)
+    own = tc.tc_create(0)
+    static = [torch.empty_like(x) for *_, x in layers]
+    encs = [tc.tc_encode(ctx, m, cb, x) for m, cb, x in layers]          # buffers
+    outs = [torch.empty_like(x) for *_, x in layers]
+    for (*_, x), st in zip(layers, static):
+        st.copy_(x)
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        if as_list:
+            tc.tc_encode_many(own, [(m, cb, st) for (m, cb, _), st in zip(layers, static)], outs=encs)
+            tc.tc_decode_many(own, [(m, cb, e, st.shape, st.dtype) for (m, cb, _), e, st in zip(layers, encs, static)], outs=outs)
+        else:
+            for (m, cb, _), st, e, o in zip(layers, static, encs, outs):
+                tc.tc_encode(own, m, cb, st, out=e)
+                tc.tc_decode(own, m, cb, e, st.shape, st.dtype, out=o)
+    for turn in range(3):
+        want = []
+        for (m, cb, x), st in zip(layers, static):
+            st.copy_(x if turn == 0 else x.flip(0) if turn == 1 else x * 0.5)
+            e = tc.tc_encode(ctx, m, cb, st)
+            want.append((e, tc.tc_decode(ctx, m, cb, e, st.shape, st.dtype)))
+        assert tc.tc_get_status(ctx) == 0
+        graph.replay()
+        assert tc.tc_get_status(own) == 0
+        for (e, o), ge, go in zip(want, encs, outs):
+            n = e.total_bits() // 8
+            assert ge.total_bits() == e.total_bits() and torch.equal(ge.words[:n], e.words[:n]) and torch.equal(go, o)
+        # the arena of the captured calls' context moves
+        big = [layers[1], layers[1], layers[3], layers[3]] * (turn + 1) * 4
+        grown = tc.tc_encode_many(own, big)
+        tc.tc_decode_many(own, [(m, cb, e, x.shape, x.dtype) for (m, cb, x), e in zip(big, grown)])
+        assert tc.tc_get_status(own) == 0
+    del graph
+    own.close()
+    for m, cb, _ in layers:
+        m.close(); cb.close()
