@@ -12,7 +12,12 @@
  * Conventions
  *   - Every pointer says whether it is HOST or DEVICE memory.  Device pointers must belong to
  *     the device the context was created on.  The caller owns every buffer it passes in; the
- *     library owns only the opaque handles it returns and a small scratch arena per context.
+ *     library owns only the opaque handles it returns and a scratch arena per context.
+ *   - The arena is as large as the largest call so far: up to about 64 MB of workspace for a tensor (layers of more
+ *     than 256 channels, unaligned maps, per-channel code tables, few tiles), eight times that for a list,
+ *     besides 8 bytes per tile.  It grows inside the call that needs more, which stops the device while memory is
+ *     released and allocated.  If that memory cannot be had, tc_encode, tc_decode and their list forms run on kernels
+ *     that need no workspace (same stream; slower).
  *   - `cuda_stream` is a cudaStream_t passed as void* (NULL = the default stream).  Calls that
  *     take one are asynchronous on it unless stated otherwise.
  *   - A context serves one stream at a time: its scratch arena (the cross-tile bookkeeping of
@@ -89,7 +94,9 @@ tc_status tc_get_status(tc_ctx *ctx, void *cuda_stream);
  * multiples of 16) run on plain fp32 kernels with the same arithmetic.  fp32 tensors run on
  * kernels that evaluate the definition in fp64.  With `on` == 1 every tensor takes the fp64
  * kernels; with `on` == 2 bf16 tensors skip the resident-basis kernels, so that the streaming
- * kernels can be checked on the shapes both take; 0 restores the default. */
+ * kernels can be checked on the shapes both take; with `on` == 3 bf16 tensors skip the decoder that
+ * passes over runs of the zero level; with `on` == 4 calls run as if the memory for their workspaces could
+ * not be had, on the kernels that need none; 0 restores the default. */
 void tc_force_exact_path(tc_ctx *ctx, int on);
 /* Which kernels the last tc_encode (decode == 0) or tc_decode (decode != 0) of this context
  * launched: 0 = fp64 kernels, 1 = tensor-core kernels with the basis resident in shared

@@ -242,7 +242,8 @@ def tc_create(device: int = 0) -> Context:
 
 def tc_force_exact_path(ctx: Context, on) -> None:
     """0 / False: default routes; 1 / True: fp64 kernels for everything; 2: bf16 tensors skip the
-    resident-basis tensor-core kernels (validation of the streaming kernels)."""
+    resident-basis tensor-core kernels (validation of the streaming kernels); 3: they skip the run-skipping
+    decoder; 4: calls run as if the memory for their workspaces could not be had."""
     load_library().tc_force_exact_path(ctx.ptr, int(on))
 
 

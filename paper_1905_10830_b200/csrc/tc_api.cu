@@ -109,42 +109,58 @@ bool resolve_chunks(const tc_encode_params *p, int k, int max_len, ChunkShape *o
     return true;
 }
 
+// The context's arena, at least `bytes` of it.  If the memory cannot be had, the arena stays as large as it was.
 tc_status ensure_scratch(tc_ctx *ctx, size_t bytes)
 {
     if (bytes <= ctx->scratch_bytes) return TC_OK;
+    const size_t had = ctx->scratch_bytes;
+    auto take = [&](size_t want) {
+        if (cudaMalloc(&ctx->scratch, want) != cudaSuccess) { cudaGetLastError(); ctx->scratch = nullptr; ctx->scratch_bytes = 0; return false; }
+        ctx->scratch_bytes = want;
+        return true;
+    };
     if (ctx->scratch) { TC_CUDA(cudaDeviceSynchronize()); cudaFree(ctx->scratch); ctx->scratch = nullptr; ctx->scratch_bytes = 0; }
-    size_t want = std::max<size_t>(bytes, 8 << 20);
-    TC_CUDA(cudaMalloc(&ctx->scratch, want));
-    ctx->scratch_bytes = want;
-    return TC_OK;
+    if (take(std::max<size_t>(bytes, 8 << 20)) || (bytes < (8 << 20) && take(bytes))) return TC_OK;
+    if (had) take(had);
+    return TC_ERR_CUDA;
 }
 
 // The memory one call's kernels share: the context's arena, or -- while the stream is being captured -- memory of
 // the graph's own.  A captured call is replayed long after the arena may have moved to make room for a larger tensor, and
 // the arena cannot grow during a capture.
+// A call needs `least` bytes; with `most` it has its workspaces too, without them it takes the kernels that need none
+// (tc_encode_with_scratch, decode_with_scratch): `whole` says which.
 struct CallScratch {
     char *at = nullptr;
+    bool whole = false;
     cudaStream_t stream = nullptr;
     bool of_graph = false;
     ~CallScratch() { if (of_graph && cudaFreeAsync(at, stream) != cudaSuccess) cudaGetLastError(); }
 };
 
-tc_status call_scratch(tc_ctx *ctx, size_t bytes, cudaStream_t s, CallScratch *out)
+tc_status call_scratch(tc_ctx *ctx, size_t least, size_t most, cudaStream_t s, CallScratch *out)
 {
-    if (bytes == 0) return TC_OK;
+    if (ctx->no_workspace) most = least;
+    out->whole = !ctx->no_workspace;
+    if (most == 0) return TC_OK;
     cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(s, &capture) != cudaSuccess) cudaGetLastError();
-    if (capture == cudaStreamCaptureStatusNone) {
-        const tc_status st = ensure_scratch(ctx, bytes);
-        out->at = (char *)ctx->scratch;
-        return st;
-    }
-    void *mem = nullptr;
-    TC_CUDA(cudaMallocAsync(&mem, bytes, s));
-    out->at = (char *)mem;
-    out->stream = s;
-    out->of_graph = true;
-    return TC_OK;
+    auto take = [&](size_t bytes) {
+        if (capture == cudaStreamCaptureStatusNone) {
+            if (ensure_scratch(ctx, bytes) != TC_OK) return false;
+            out->at = (char *)ctx->scratch;
+            return true;
+        }
+        void *mem = nullptr;
+        if (cudaMallocAsync(&mem, bytes, s) != cudaSuccess) { cudaGetLastError(); return false; }
+        out->at = (char *)mem;
+        out->stream = s;
+        out->of_graph = true;
+        return true;
+    };
+    if (take(most)) return TC_OK;
+    out->whole = false;
+    return least == 0 || (least < most && take(least)) ? TC_OK : TC_ERR_CUDA;
 }
 
 // The host copy of a model's basis, fetched from the device at first use.
@@ -401,7 +417,9 @@ void tc_destroy(tc_ctx *ctx)
 
 void tc_force_exact_path(tc_ctx *ctx, int on)
 {
-    if (ctx) ctx->force_exact = (on == 2 || on == 3) ? on : (on ? 1 : 0);
+    if (!ctx) return;
+    ctx->no_workspace = on == 4;
+    ctx->force_exact = (on == 2 || on == 3) ? on : (on && on != 4 ? 1 : 0);
 }
 
 int tc_last_path(const tc_ctx *ctx, int decode)
@@ -995,9 +1013,9 @@ tc_status tc_encode(tc_ctx *ctx, const tc_model *m, const tc_codebook *cb, const
     const size_t lookback = (kEncodeScratchHeader + (size_t)n_tiles * sizeof(unsigned long long) + 255) & ~(size_t)255;
     const size_t work = encode_work_bytes(ctx, m, x);
     CallScratch scratch;
-    if ((st = call_scratch(ctx, lookback + work, s, &scratch)) != TC_OK) return st;
+    if ((st = call_scratch(ctx, lookback, lookback + work, s, &scratch)) != TC_OK) return st;
     return tc_encode_with_scratch(ctx, m, cb, x, cs.cp, cs.splits, stream_out, capacity, chunk_len, tile_off, debug,
-                                  scratch.at, work ? scratch.at + lookback : nullptr, s);
+                                  scratch.at, work && scratch.whole ? scratch.at + lookback : nullptr, s);
 }
 
 // bf16 tensors decoded by the entropy decoder and the tiled product in kernels of their own: wide layers, and per-channel
@@ -1105,7 +1123,7 @@ tc_status tc_decode(tc_ctx *ctx, const tc_model *m, const tc_codebook *cb, const
     if (args != TC_OK) return args;
     DeviceGuard guard(ctx->device);
     CallScratch scratch;
-    const tc_status st = call_scratch(ctx, decode_scratch_bytes(ctx, m, cb, x_hat), (cudaStream_t)cuda_stream, &scratch);
+    const tc_status st = call_scratch(ctx, 0, decode_scratch_bytes(ctx, m, cb, x_hat), (cudaStream_t)cuda_stream, &scratch);
     if (st != TC_OK) return st;
     return decode_with_scratch(ctx, m, cb, stream, stream_bytes, chunk_len, tile_off, params, x_hat, (uint8_t *)scratch.at, 0, cuda_stream);
 }
@@ -1192,7 +1210,7 @@ tc_status tc_encode_many(tc_ctx *ctx, const tc_encode_item *items, int32_t n_ite
     tc_status st = ensure_many_streams(ctx);
     if (st != TC_OK) return st;
     CallScratch scratch;
-    if ((st = call_scratch(ctx, stream_workspaces(order, n_streams, symbols_bytes, lookback_total, symbols_at), s, &scratch)) != TC_OK) return st;
+    if ((st = call_scratch(ctx, lookback_total, stream_workspaces(order, n_streams, symbols_bytes, lookback_total, symbols_at), s, &scratch)) != TC_OK) return st;
     // one clear for the look-back state of all items, then the items fan out over the streams
     TC_CUDA(cudaMemsetAsync(scratch.at, 0, lookback_total, s));
     TC_CUDA(cudaEventRecord(ctx->many_fork, s));
@@ -1207,7 +1225,7 @@ tc_status tc_encode_many(tc_ctx *ctx, const tc_encode_item *items, int32_t n_ite
         if (pixels == 0) { if (cudaMemsetAsync(it.tile_off, 0, sizeof(uint64_t), ws) != cudaSuccess && first_error == TC_OK) first_error = TC_ERR_CUDA; continue; }
         st = tc_encode_with_scratch(ctx, it.model, it.codebook, it.x, shape[i].cp, shape[i].splits, it.stream_out, it.capacity,
                                     it.chunk_len, it.tile_off, nullptr, scratch.at + lookback_at[i],
-                                    symbols_bytes[i] ? scratch.at + symbols_at[i] : nullptr, ws, nullptr, nullptr, list_sms);
+                                    symbols_bytes[i] && scratch.whole ? scratch.at + symbols_at[i] : nullptr, ws, nullptr, nullptr, list_sms);
         if (st != TC_OK && first_error == TC_OK) first_error = st;
     }
     for (int j = 0; j < n_streams; ++j) {
@@ -1243,7 +1261,7 @@ tc_status tc_decode_many(tc_ctx *ctx, const tc_decode_item *items, int32_t n_ite
     const std::vector<int> order = by_descending_work(n_items, work);
     if ((st = ensure_many_streams(ctx)) != TC_OK) return st;
     CallScratch scratch;
-    if ((st = call_scratch(ctx, stream_workspaces(order, n_streams, symbols_bytes, 0, symbols_at), s, &scratch)) != TC_OK) return st;
+    if ((st = call_scratch(ctx, 0, stream_workspaces(order, n_streams, symbols_bytes, 0, symbols_at), s, &scratch)) != TC_OK) return st;
     TC_CUDA(cudaEventRecord(ctx->many_fork, s));
     for (int j = 0; j < n_streams; ++j) TC_CUDA(cudaStreamWaitEvent(ctx->many_streams[j], ctx->many_fork, 0));
     tc_status first_error = TC_OK;
@@ -1252,7 +1270,7 @@ tc_status tc_decode_many(tc_ctx *ctx, const tc_decode_item *items, int32_t n_ite
         const tc_decode_item &it = items[i];
         const int list_sms = list_share(ctx->sm_count, n_streams, work, i);
         st = decode_with_scratch(ctx, it.model, it.codebook, it.stream, it.stream_bytes, it.chunk_len, it.tile_off, it.params,
-                                 it.x_hat, symbols_bytes[i] ? (uint8_t *)scratch.at + symbols_at[i] : nullptr,
+                                 it.x_hat, symbols_bytes[i] && scratch.at ? (uint8_t *)scratch.at + symbols_at[i] : nullptr,
                                  list_sms, ctx->many_streams[r % n_streams]);
         if (st != TC_OK && first_error == TC_OK) first_error = st;
     }

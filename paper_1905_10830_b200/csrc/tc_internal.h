@@ -44,6 +44,7 @@ struct tc_ctx {
     cudaStream_t many_streams[kManyStreams] = {};
     cudaEvent_t many_fork = nullptr, many_join[kManyStreams] = {};
     int force_exact = 0;                  // 1: route every tensor through the fp64 kernels; 2: skip the resident-basis kernels; 3: skip the run-skipping decoder
+    bool no_workspace = false;            // calls run as if no memory could be had for their workspaces
     int last_encode_path = 0;             // 0 = fp64 kernels, 1 = tensor-core kernels (resident basis), 2 = fp32 kernels, 3 = tensor-core kernels (streamed basis)
     int last_decode_path = 0;
     tc_codebook *stats_cb[9] = {};        // tc_stats: fixed-length code tables (one per bit width) for streams coded without a codebook

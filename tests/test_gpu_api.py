@@ -459,3 +459,28 @@ def test_captured_calls_keep_their_scratch(ctx, as_list):
     own.close()
     for m, cb, _ in layers:
         m.close(); cb.close()
+
+
+def test_without_memory_for_workspaces(ctx):
+    # the kernels that need no workspace (what a call falls back to when its allocation fails) write the same streams
+    # and tensors: wide layers, unaligned maps, per-channel codes, fp32 maps, singly and as a list
+    layers = _fitted_layers(ctx, CAPTURED + [(272, 5, 30, torch.bfloat16, False), (128, 9, 11, torch.bfloat16, True),
+                                             (1024, 4, 9, torch.bfloat16, False), (80, 15, 40, torch.bfloat16, True)])
+    own = tc.tc_create(0)
+    tc.tc_force_exact_path(own, 4)
+    encs = [tc.tc_encode(own, m, cb, x) for m, cb, x in layers]
+    outs = [tc.tc_decode(own, m, cb, e, x.shape, x.dtype) for (m, cb, x), e in zip(layers, encs)]
+    encs_list = tc.tc_encode_many(own, layers)
+    outs_list = tc.tc_decode_many(own, [(m, cb, e, x.shape, x.dtype) for (m, cb, x), e in zip(layers, encs_list)])
+    assert tc.tc_get_status(own) == 0
+    for (m, cb, x), e, o, el, ol in zip(layers, encs, outs, encs_list, outs_list):
+        want = tc.tc_encode(ctx, m, cb, x)
+        xhat = tc.tc_decode(ctx, m, cb, want, x.shape, x.dtype)
+        n = want.total_bits() // 8
+        for got, back in ((e, o), (el, ol)):
+            assert torch.equal(got.tile_off, want.tile_off) and torch.equal(got.words[:n], want.words[:n])
+            assert torch.equal(got.chunk_len[:want.layout.n_chunks], want.chunk_len[:want.layout.n_chunks])
+            assert torch.equal(back, xhat)
+        m.close(); cb.close()
+    assert tc.tc_get_status(ctx) == 0
+    own.close()
