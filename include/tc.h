@@ -13,11 +13,11 @@
  *   - Every pointer says whether it is HOST or DEVICE memory.  Device pointers must belong to
  *     the device the context was created on.  The caller owns every buffer it passes in; the
  *     library owns only the opaque handles it returns and a scratch arena per context.
- *   - The arena is as large as the largest call so far: up to about 64 MB of workspace for a tensor (layers of more
- *     than 256 channels, unaligned maps, per-channel code tables, few tiles), eight times that for a list,
- *     besides 8 bytes per tile.  It grows inside the call that needs more, which stops the device while memory is
- *     released and allocated.  If that memory cannot be had, tc_encode, tc_decode and their list forms run on kernels
- *     that need no workspace (same stream; slower).
+ *   - The arena starts with 72 MB, which is room for the workspace of any one tensor (layers of more than 256
+ *     channels, unaligned maps, per-channel code tables, few tiles: up to about 64 MB, in passes) and 8 bytes per tile of
+ *     about a million tiles; a list takes up to eight workspaces.  It grows inside the call that needs more, which
+ *     stops the device while memory is released and allocated.  If that memory cannot be had, tc_encode, tc_decode and
+ *     their list forms run on kernels that need no workspace (same stream; slower).
  *   - `cuda_stream` is a cudaStream_t passed as void* (NULL = the default stream).  Calls that
  *     take one are asynchronous on it unless stated otherwise.
  *   - A context serves one stream at a time: its scratch arena (the cross-tile bookkeeping of

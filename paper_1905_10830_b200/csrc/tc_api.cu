@@ -378,14 +378,16 @@ tc_status tc_create(tc_ctx **out, int device)
         delete ctx;
         return TC_ERR_CUDA;
     }
-    // (the arena at its smallest size, so that a first call does not stop for an allocation)
-    if (cudaMalloc((void **)&ctx->d_status, 64) != cudaSuccess || cudaMemset(ctx->d_status, 0, 64) != cudaSuccess ||
-        ensure_scratch(ctx, 1) != TC_OK) {
+    if (cudaMalloc((void **)&ctx->d_status, 64) != cudaSuccess || cudaMemset(ctx->d_status, 0, 64) != cudaSuccess) {
         cudaGetLastError();
         cudaFree(ctx->d_status);
         delete ctx;
         return TC_ERR_CUDA;
     }
+    // The arena is made here, so that a first call does not stop for it, with room for the workspace of any one tensor (72 MB
+    // take no longer to allocate than 8, about 360 us; growing costs a call that and a stop of the device).  Where memory
+    // is short it starts smaller, or empty.
+    if (ensure_scratch(ctx, kWideWorkspace + (8 << 20)) != TC_OK) ensure_scratch(ctx, 1);
     *out = ctx;
     return TC_OK;
 }

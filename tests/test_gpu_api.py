@@ -484,3 +484,23 @@ def test_without_memory_for_workspaces(ctx):
         m.close(); cb.close()
     assert tc.tc_get_status(ctx) == 0
     own.close()
+
+
+def test_first_calls_of_a_context_allocate_nothing(ctx):
+    # one tensor's workspace, whatever its size, fits the arena that a context is created with: what is free on the
+    # device does not change (kernels and output buffers are there from calls on another context)
+    layers = _fitted_layers(ctx, CAPTURED + [(576, 14, 1000, torch.bfloat16, False), (16, 112, 300, torch.bfloat16, True)])
+    encs = [tc.tc_encode(ctx, m, cb, x) for m, cb, x in layers]
+    outs = [tc.tc_decode(ctx, m, cb, e, x.shape, x.dtype) for (m, cb, x), e in zip(layers, encs)]
+    own = [tc.tc_create(0) for _ in layers]
+    torch.cuda.synchronize()
+    free = torch.cuda.mem_get_info()[0]
+    for c, (m, cb, x), e, o in zip(own, layers, encs, outs):
+        tc.tc_encode(c, m, cb, x, out=e)
+        tc.tc_decode(c, m, cb, e, x.shape, x.dtype, out=o)
+        assert tc.tc_get_status(c) == 0
+    assert torch.cuda.mem_get_info()[0] == free
+    for h in own:
+        h.close()
+    for m, cb, _ in layers:
+        m.close(); cb.close()
