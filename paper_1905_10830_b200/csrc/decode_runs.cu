@@ -661,6 +661,10 @@ __global__ void __launch_bounds__(kThreads, 1) decode_runs_kernel(DecodeArgs a, 
         bool alive = true;
         for (long long tl = items == 2 ? 0 : w; tl < my_tiles; tl += items == 2 ? 1 : 2) {
             const long long it = items == 2 ? 2 * tl + w : tl;       // index of the work item: item it uses accumulator it % 2 = w
+            // The accumulator first: the epilogue takes the items in order, so once it has drained the item before the last
+            // the MMAs of that tile and of all before it are done, and the wait for the operand cannot mistake an earlier
+            // turn of the buffer for this one (the two warps share the buffers where the groups are odd in number).
+            if (it >= 2) named_bar_sync(kBarAccFree + w, 256 + 32);   // the epilogue has drained the accumulator
             // (after a wait that ran out the warp keeps walking the items: the epilogue waits for its commits)
             if (alive) alive = mbar_wait(smem_u32(&s_bfull[buf]), turn);     // the group's VLD threads have arrived
             __syncwarp();
@@ -671,7 +675,6 @@ __global__ void __launch_bounds__(kThreads, 1) decode_runs_kernel(DecodeArgs a, 
             const uint64_t b_base = make_smem_desc(opnd_addr + (uint32_t)buf * L.opnd_bytes, 2048, 128);
             const uint32_t b_hi = (uint32_t)(b_base >> 32);
             __syncwarp();
-            if (it >= 2) named_bar_sync(kBarAccFree + w, 256 + 32);   // the epilogue has drained the accumulator
             tc_fence_after_sync();
             // rows 64 w ... of the buffer (two blocks): eight-row groups are 128 bytes apart; a step of 16
             // coefficients moves the start address on by two core-matrix columns of 2048 bytes
