@@ -33,6 +33,8 @@
 //
 // A tile whose stream is dense (more than kDenseBits128 / 128 bits per symbol) gains nothing
 // from run skipping; its threads then decode symbol by symbol, eight symbols per 16-byte store.
+#include <algorithm>
+
 #include "device_utils.cuh"
 #include "sm100_ptx.cuh"
 
@@ -72,25 +74,26 @@ struct SmemLayout {
 };
 
 // group_warps: warps of a VLD group.  As many groups as warps and shared memory allow beside stream
-// buffers for tiles of 2.5 bits per symbol (two groups: for what is left, at least 4 KB).
-inline SmemLayout smem_layout(int k, int lut_entries, int group_warps, int budget)
+// buffers of `want_bytes`, what a tile's segment is expected to take (two groups: for what is left, at least 4 KB).  A segment
+// that does not fit its buffer is read from global memory word by word, which costs more than a group less: with room
+// for 2.5 bits per symbol whatever the rate, 512 maps of 28x28 at 8 bits (4.8 to 4.3 bits per value) took 115 us at
+// 128 channels, 186 at 176 and 200 at 192; sized by the rate 95, 153 and 163, and 256 maps of 64x56x56 121 -> 101.
+inline SmemLayout smem_layout(int k, int lut_entries, int group_warps, uint32_t want_bytes, int budget)
 {
     SmemLayout l;
     l.lut = 0;                                                // 32-bit entries: bf16(symbol - center) << 16 | length
     l.opnd = ((uint32_t)lut_entries * 4u + 1023u) & ~1023u;
     l.opnd_bytes = (uint32_t)k * TC_TILE_PIXELS * 2;
     const int most = kVldWarps / group_warps < kMaxGroups ? kVldWarps / group_warps : kMaxGroups;
-    const uint32_t want_kb = ((uint32_t)k * 40u + 1023u) / 1024u;
     l.stream_buf = 0;
     l.total = 0;
     for (l.groups = most; l.groups >= 2; --l.groups) {
         l.tbuf = l.opnd + (uint32_t)l.groups * l.opnd_bytes;
         l.sbuf = l.tbuf + 8u * kTrWarpBytes;
         const long long left = (long long)budget - l.sbuf - kStreamSlack;
-        long long kb = left / (2ll * l.groups * 1024);
-        if (kb > 16) kb = 16;
-        if (kb < 4 || (kb < (long long)want_kb && l.groups > 2)) continue;
-        l.stream_buf = (uint32_t)kb * 1024u;
+        const long long room = (left / (2ll * l.groups)) & ~127ll;
+        if (room < 4096 || (room < (long long)want_bytes && l.groups > 2)) continue;
+        l.stream_buf = (uint32_t)std::min(room, std::max(16384ll, ((long long)want_bytes + 127) & ~127ll));
         l.total = l.sbuf + 2u * (uint32_t)l.groups * l.stream_buf + kStreamSlack;
         break;
     }
@@ -708,7 +711,10 @@ __global__ void __launch_bounds__(kThreads, 1) decode_runs_kernel(DecodeArgs a, 
 
 static SmemLayout runs_layout(const tc_ctx *ctx, const DecodeArgs &a)
 {
-    return smem_layout(a.k, 1 << a.lut_bits, (group_work(a.splits, a.chunk_pixels) + 31) / 32, ctx->max_smem_optin - kStaticSmem);
+    // (a dense tile's segment is at most 3 % longer than the mean)
+    const double tile_bytes = a.mean_tile_bytes > 0 ? a.mean_tile_bytes : std::max(2.5, (double)a.code_bits) * a.k * TC_TILE_PIXELS / 8;
+    const uint32_t want = (uint32_t)std::min(1.03 * tile_bytes, 1e6);
+    return smem_layout(a.k, 1 << a.lut_bits, (group_work(a.splits, a.chunk_pixels) + 31) / 32, want, ctx->max_smem_optin - kStaticSmem);
 }
 
 bool tc_decode_runs_supported(const tc_ctx *ctx, const DecodeArgs &a)
@@ -720,13 +726,6 @@ bool tc_decode_runs_supported(const tc_ctx *ctx, const DecodeArgs &a)
     if (a.chunk_pixels > 1 ? a.splits != 1 : (a.splits != 1 && a.splits != 2 && a.splits != 4)) return false;
     if (a.splits > 1 && (a.k % a.splits != 0 || (a.k / a.splits) % 8 != 0)) return false;
     return runs_layout(ctx, a).stream_buf > 0;
-}
-
-// Bytes of a tile's stream segment this kernel stages in shared memory; longer segments are read
-// from global memory, word by word.
-size_t tc_decode_runs_staging_bytes(const tc_ctx *ctx, const DecodeArgs &a)
-{
-    return runs_layout(ctx, a).stream_buf;
 }
 
 tc_status tc_launch_decode_runs(const tc_ctx *ctx, const DecodeArgs &a, cudaStream_t s)

@@ -271,6 +271,9 @@ tc_status finish_codebook(tc_codebook *cb)
     if (cb->groups == 1)
         for (int s = 0; s < nsym && cb->modal < 0; ++s)
             if (cb->lengths[s] == 1) cb->modal = s;
+    double mean_bits = 0.0;
+    for (uint8_t l : cb->lengths) mean_bits += std::ldexp((double)l, -(int)l);
+    cb->mean_bits = (float)(mean_bits / cb->groups);
     std::vector<uint32_t> enc((size_t)cb->groups * nsym);
     std::vector<uint16_t> lut((size_t)cb->groups << cb->lut_bits);
     std::vector<uint32_t> lut32((size_t)cb->groups << cb->lut_bits);
@@ -847,7 +850,12 @@ tc_status tc_build_codebook(tc_ctx *ctx, const tc_model *model, const uint64_t *
     for (int g = 0; g < groups; ++g)
         if (tc_huffman_lengths_host(h.data() + (size_t)g * nsym, nsym, lmax, lengths.data() + (size_t)g * nsym) != 0)
             return TC_ERR_INVALID_ARG;
-    return tc_codebook_import(ctx, model->bits, groups, lengths.data(), out);
+    const tc_status st = tc_codebook_import(ctx, model->bits, groups, lengths.data(), out);
+    if (st != TC_OK) return st;
+    double count = 0.0, bits = 0.0;
+    for (size_t i = 0; i < h.size(); ++i) { count += (double)h[i]; bits += (double)h[i] * lengths[i]; }
+    if (count > 0.0) (*out)->mean_bits = (float)(bits / count);
+    return TC_OK;
 }
 
 tc_status tc_codebook_export(const tc_codebook *cb, int32_t *bits, int32_t *groups, uint8_t *lengths)
@@ -1069,6 +1077,7 @@ static tc_status decode_with_scratch(tc_ctx *ctx, const tc_model *m, const tc_co
     a.sms = list_sms ? list_sms : ctx->sm_count;
     a.basis_t_map = m->has_basis_t_map ? &m->basis_t_map : nullptr;
     a.modal = cb->modal;
+    a.code_bits = cb->mean_bits;
     a.mean_tile_bytes = (params && params->mean_tile_bytes > 0) ? params->mean_tile_bytes : 0;
     // Coefficient j has standard deviation sqrt(eig[j]) on the calibration data; where that exceeds
     // about 0.45 steps more than a quarter of its symbols differ from the zero level and skipping

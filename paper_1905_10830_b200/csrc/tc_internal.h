@@ -81,6 +81,8 @@ struct tc_model {
 struct tc_codebook {
     int bits = 0, groups = 0, max_len = 0, lut_bits = 0;
     int modal = -1;                         // per-layer table: the symbol coded by the single bit 0 (-1: none)
+    float mean_bits = 0.f;                  // bits per symbol: of the counts it was built from, else for symbols of probability 2^-length
+                                            // (from 2.5 bits on within 10 % of the coded layers' rate)
     std::vector<uint8_t> lengths;           // host [groups][2^bits]
     int device = 0;
     void *d_block = nullptr;                // one allocation that holds the arrays below
@@ -155,6 +157,7 @@ struct DecodeArgs {
     const float *dec_bias;              // [c]
     int center;                         // subtracted from every symbol before the MMA
     int modal;                          // per-layer table: the symbol whose code is the single bit 0, or -1 if no code has one bit
+    float code_bits;                    // bits per symbol to expect (tc_codebook::mean_bits)
     int mean_tile_bytes;                // caller's hint: mean size of a tile's stream segment, 0 = not known
     int dense_head;                     // run-skipping decoder: leading coefficients that are too often non-modal for run skipping to pay
     int relu;                           // x_hat = max(x_hat, 0) before it is rounded to the tensor type
@@ -227,7 +230,6 @@ tc_status tc_launch_encode_wide(const tc_ctx *ctx, const EncodeArgs &a, cudaStre
 bool tc_decode_wide_supported(const tc_ctx *ctx, const DecodeArgs &a);
 tc_status tc_launch_decode_wide(const tc_ctx *ctx, const DecodeArgs &a, cudaStream_t s);
 size_t tc_decode_tc_staging_bytes(const tc_ctx *ctx, const DecodeArgs &a);     // per tile
-size_t tc_decode_runs_staging_bytes(const tc_ctx *ctx, const DecodeArgs &a);   // per tile
 size_t tc_decode_wide_staging_bytes(const tc_ctx *ctx, const DecodeArgs &a);   // per tile
 
 tc_status tc_launch_channel_sums(const void *x, int dtype, int n, int c, int hw, double *sums,

@@ -265,3 +265,34 @@ def test_staging_ring_of_the_resident_encoder(ctx, c, bits, ratio):
         base, chunks = base + bits_n, chunks + part.layout.n_chunks
     assert base == enc.total_bits()
     m.close(); cb.close()
+
+
+# Run-skipping decoder, stream buffers sized by the rate: three groups and one work item per tile (128 and 112
+# channels), buffers above 16 KB, segments that fit no buffer, and hints that are too small or too large -- the hint
+# changes how tiles are staged, never the tensor.  Against the fp64 kernels on the same stream.
+@pytest.mark.parametrize("c,h,w,bits,ratio,cp", [(128, 28, 28, 8, 0.9, 0), (112, 28, 28, 8, 0.98, 2), (160, 28, 28, 8, 0.9, 0), (208, 14, 14, 8, 0.98, 0),
+                                                 (224, 14, 14, 8, 0.98, 0), (80, 28, 28, 8, 0.9, 0), (64, 56, 56, 7, 0.95, 0), (144, 28, 28, 6, 0.9, 0)])
+def test_run_skipping_decoder_stream_buffers(ctx, c, h, w, bits, ratio, cp):
+    params = fm.layer_params(fm.LayerSpec(c, h, w, ratio, None, 16000 + c))
+    cal = fm.make_maps(params, max(4, 30000 // (h * w)), calib=True, dtype=torch.bfloat16, device="cuda")
+    x = fm.make_maps(params, 148 * 9 * 128 // (h * w) + 3, dtype=torch.bfloat16, device="cuda")
+    m = tc.tc_fit_pca(ctx, cal, bits)
+    cb = tc.tc_build_codebook(ctx, m, tc.tc_stats(ctx, m, None, cal).hist)
+    enc = tc.tc_encode(ctx, m, cb, x, chunk_pixels=cp)
+    got = tc.tc_decode(ctx, m, cb, enc, x.shape, x.dtype)
+    assert tc.tc_get_status(ctx) == 0 and tc.tc_last_path(ctx, True) == 1
+    for hint in (1, 5000, 12000, 60000, 2 ** 31 - 1):
+        assert torch.equal(got, tc.tc_decode(ctx, m, cb, enc, x.shape, x.dtype, mean_tile_bytes=hint))
+    again = tc.tc_codebook_import(ctx, tc.tc_codebook_export(cb), bits)          # without counts
+    assert torch.equal(got, tc.tc_decode(ctx, m, again, enc, x.shape, x.dtype))
+    assert tc.tc_get_status(ctx) == 0 and tc.tc_last_path(ctx, True) == 1
+    tc.tc_force_exact_path(ctx, 1)
+    want = tc.tc_decode(ctx, m, cb, enc, x.shape, x.dtype)
+    assert tc.tc_get_status(ctx) == 0
+    tc.tc_force_exact_path(ctx, 0)
+    # (neighbouring bf16 numbers for at most 0.1 % of the values: the parity cases' cap)
+    a, b = got.float(), want.float()
+    assert bool(((a - b).abs() <= 2.0 ** -7 * b.abs() + 1e-6 * float(b.abs().max())).all())
+    assert float((a != b).double().mean()) <= 1e-3
+    for h_ in (m, cb, again):
+        h_.close()
