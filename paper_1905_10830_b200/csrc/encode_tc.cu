@@ -51,6 +51,7 @@ struct Plan {
     int run_words[2];          // words of a thread's private run, first and second half's threads; 0: two passes
     int split_blk;             // blocks of 16 coefficients of the first half's threads
     int skip_blk;              // blocks from here on are tested for holding nothing but the modal symbol
+    float skip_dist;           // a position nearer to the modal level than this (as a fraction of the quantiser's range) rounds to it
     int entries;               // of the code table in shared memory
 };
 
@@ -400,18 +401,6 @@ __global__ void __launch_bounds__(kThreads, 1) encode_tc_kernel(EncodeArgs a, Pl
         const int bar_id = 1 + grp;
         bool alive = true;
         [[maybe_unused]] const int skip_blk = pl.skip_blk;
-        // A position nearer to the modal level than this rounds to it, whichever of the two ways it is computed:
-        // they differ by the rounding of s_bias_mid and of the two results, together at most 2^-24 of the
-        // bias's size plus three; four times that is kept clear.  (At 8 bits and a mean of a thousand ranges that is
-        // 0.06 of a level; a fixed 0.001 let symbols one off the quantiser's pass for the modal one there.)
-        [[maybe_unused]] float skip_dist = 0.f;
-        if constexpr (kCanSkip) {
-            float most = 0.f;
-            for (int i = lane; i < a.k; i += 32) most = fmaxf(most, fabsf(s_bias[i]));
-#pragma unroll
-            for (int d = 16; d > 0; d >>= 1) most = fmaxf(most, __shfl_xor_sync(0xffffffffu, most, d));
-            skip_dist = 0.499f / top - (most + 1.f) * 2.4e-7f;
-        }
         const uint32_t trow = tmem_base + grp * kAccCols + ((uint32_t)(wq * 32) << 16);
 
         auto resolve_base = [&](long long tile, unsigned long long padded) {
@@ -586,7 +575,7 @@ __global__ void __launch_bounds__(kThreads, 1) encode_tc_kernel(EncodeArgs a, Pl
                                 farthest2(far[2], r1[4 * i], r1[4 * i + 1], inv_range, mid[4 + i].x, mid[4 + i].y);
                                 farthest2(far[3], r1[4 * i + 2], r1[4 * i + 3], inv_range, mid[4 + i].z, mid[4 + i].w);
                             }
-                            if (!__all_sync(0xffffffffu, (far[0] < skip_dist) & (far[1] < skip_dist) & (far[2] < skip_dist) & (far[3] < skip_dist))) break;
+                            if (!__all_sync(0xffffffffu, (far[0] < pl.skip_dist) & (far[1] < pl.skip_dist) & (far[2] < pl.skip_dist) & (far[3] < pl.skip_dist))) break;
                             at();
                             if constexpr (kCount) sink.bits += 32;             // 32 times the code 0 (one bit)
                             else sink.put_word(0u);
@@ -803,6 +792,12 @@ static Plan make_plan(const tc_ctx *ctx, const EncodeArgs &a)
     const bool modal = a.groups == 1 && a.modal >= 0;
     auto blk_bits = [&](int b) { return modal || a.groups != 1 ? a.blk_bits[b] : std::max(a.blk_bits[b], 16.f * a.bits); };
     Plan best{};
+    // The test for modal blocks adds the bias up differently from the quantiser: the two positions differ by the rounding of s_bias_mid and
+    // of the two results, together at most 2^-24 of the largest bias plus three.  Four times that is kept clear, besides
+    // 0.001 of a level.  (At 8 bits and a mean of a thousand ranges that is 0.06 of a level; the 0.001 alone let symbols
+    // next to a rounding boundary pass for the modal one there.  Here and not from s_bias in the kernel, which cost the coder
+    // 2 to 3 %: 64x56x56 x 256 at 8 bits 107 -> 110 us.)
+    best.skip_dist = 0.499f / (float)((1 << a.bits) - 1) - (a.max_bias + 1.f) * 2.4e-7f;
     // A test of 32 coefficients x 32 pixels pays from a success in three on: fewer than about one other
     // symbol expected in it.
     best.skip_blk = n_blk;

@@ -254,7 +254,9 @@ tc_status finish_model(tc_model *m)
         m->has_basis_t_map = false;
         if (k % 16 == 0) m->has_basis_t_map = tc_tensor_map_sw128(&m->basis_t_map, m->d_basis_t_bf16, c, k, 128);
     }
-    TC_CUDA(cudaStreamSynchronize(nullptr));
+    std::vector<float> bias(k);
+    TC_CUDA(cudaMemcpy(bias.data(), m->d_enc_bias, sizeof(float) * k, cudaMemcpyDeviceToHost));      // (ends after the kernels above)
+    for (float b : bias) m->max_bias = std::max(m->max_bias, std::fabs(b) / (float)((1 << m->bits) - 1));
     return TC_OK;
 }
 
@@ -929,6 +931,7 @@ tc_status tc_encode_with_scratch(tc_ctx *ctx, const tc_model *m, const tc_codebo
     a.alone = list_sms == 0;
     a.sms = list_sms ? list_sms : ctx->sm_count;
     a.modal = cb->modal;
+    a.max_bias = m->max_bias;
     a.blk_bits = m->blk_bits.data(); a.blk_odd = m->blk_odd.data();
     if (hist && !((ctx->force_exact == 0 || ctx->force_exact == 3) && x->dtype == TC_BF16 && tc_encode_tc_supported(ctx, a)))
         return TC_ERR_UNSUPPORTED;                      // only the resident-basis tensor-core encoder counts symbols

@@ -60,6 +60,7 @@ struct tc_model {
     mutable std::vector<double> basis;      // [c][c], or empty
     std::vector<double> mean, eig;          // [c]
     std::vector<float> blk_bits, blk_odd;   // [(k + 15) / 16]  see finish_model
+    float max_bias = 0.f;                   // largest |d_enc_bias|, as a fraction of the quantiser's range
     int device = 0;
     // device copies, all but the first two (of a fitted model: owns64) inside one allocation
     void *d_block = nullptr;
@@ -130,6 +131,7 @@ struct EncodeArgs {
     unsigned long long *hist;         // tensor-core encoder, statistics: non-null = per-coefficient counts [K][2^bits] of every symbol but hist_modal are added here
     int hist_modal;                   // the symbol of the zero level, which most coefficients hold: statistics mode counts all the others
     int modal;                        // per-layer table: the symbol whose code is the single bit 0, or -1 if no code has one bit
+    float max_bias;                   // see tc_model
     const float *blk_bits, *blk_odd;  // HOST, per block of 16 coefficients: expected code bits, expected number of symbols that are not the zero level
 };
 
