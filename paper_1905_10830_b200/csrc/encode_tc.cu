@@ -56,7 +56,7 @@ struct Plan {
 };
 
 struct SmemLayout {
-    uint32_t basis, ring, staging, runs, run_bytes, enc, len8, bias, bias_mid, xch, total;
+    uint32_t basis, ring, staging, run_bytes, enc, len8, bias, bias_mid, xch, total;
 };
 
 __host__ __device__ inline SmemLayout smem_layout(int c, int k, const Plan &pl)
@@ -64,10 +64,9 @@ __host__ __device__ inline SmemLayout smem_layout(int c, int k, const Plan &pl)
     SmemLayout l;
     l.basis = 0;
     l.ring = (uint32_t)(((size_t)k * c * 2 + 1023) & ~(size_t)1023);
-    l.staging = l.ring + (uint32_t)pl.stages * kStageBytes;
-    l.runs = l.staging + 2u * pl.staging_bytes;
     l.run_bytes = (uint32_t)(pl.run_words[0] + pl.run_words[1]) * kRunStep;      // per group
-    l.enc = l.runs + 2u * l.run_bytes;
+    l.staging = l.ring + (uint32_t)pl.stages * kStageBytes;                     // per group: the buffer, then the runs
+    l.enc = l.staging + 2u * (pl.staging_bytes + l.run_bytes);
     l.len8 = l.enc + (uint32_t)pl.entries * 8;           // code lengths as bytes
     l.bias = (l.len8 + (uint32_t)pl.entries + 15u) & ~15u;
     l.bias_mid = l.bias + (uint32_t)k * 4;
@@ -126,6 +125,80 @@ __device__ __forceinline__ void farthest2(float &far, uint32_t acc0, uint32_t ac
         "mov.b64 {u0, u1}, v;\n\t"
         "max.NaN.abs.f32 %0, %0, u0, u1;\n\t}"
         : "+f"(far) : "r"(acc0), "r"(acc1), "f"(inv_range), "f"(mid0), "f"(mid1));
+}
+
+// The codes of a block's sixteen symbols, two a piece: (1 << length, code), at most 24 bits.
+template <bool kPerChannel, bool kPair>
+__device__ __forceinline__ void block_pieces(const uint32_t (&qv)[16], uint32_t enc_addr, const uint32_t *enc, int j0, int bits,
+                                             uint32_t (&mul)[8], uint32_t (&code)[8])
+{
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        if constexpr (kPair) {
+            const uint32_t idx = (qv[2 * i] - kMagicBits) + ((qv[2 * i + 1] - kMagicBits) << bits);
+            asm("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(mul[i]), "=r"(code[i]) : "r"(enc_addr + idx * 8u));
+        } else {
+            uint32_t m0, c0, m1, c1;
+            if constexpr (kPerChannel) {
+                const int j = j0 + 2 * i;
+                const uint32_t e0 = __ldg(enc + (j << bits) + (qv[2 * i] & 0xffu)), e1 = __ldg(enc + ((j + 1) << bits) + (qv[2 * i + 1] & 0xffu));
+                m0 = 1u << (e0 & 0xffu); c0 = e0 >> 8; m1 = 1u << (e1 & 0xffu); c1 = e1 >> 8;
+            } else {
+                asm("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(m0), "=r"(c0) : "r"(enc_addr + (qv[2 * i] - kMagicBits) * 8u));
+                asm("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(m1), "=r"(c1) : "r"(enc_addr + (qv[2 * i + 1] - kMagicBits) * 8u));
+            }
+            mul[i] = m0 * m1;
+            code[i] = c0 * m1 + c1;
+        }
+    }
+}
+
+// Appends them.  How many symbols are joined before they are appended is chosen for the whole warp (lanes
+// that go different ways run one after the other): sixteen or eight where every lane's
+// codes of them fit 31 bits -- a product of powers of two that reaches 2^32 is zero --
+// else four, else two.  Joining is a multiply-add, appending costs ten instructions.
+template <typename Sink>
+__device__ __forceinline__ void append_block(Sink &sink, const uint32_t (&mul)[8], const uint32_t (&code)[8])
+{
+    uint32_t m4[4], c4[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) { m4[i] = mul[2 * i] * mul[2 * i + 1]; c4[i] = code[2 * i] * mul[2 * i + 1] + code[2 * i + 1]; }
+    const uint32_t m8a = m4[0] * m4[1], m8b = m4[2] * m4[3];
+    if (__all_sync(0xffffffffu, m8a != 0u && m8b != 0u)) {
+        const uint32_t c8a = c4[0] * m4[1] + c4[1], c8b = c4[2] * m4[3] + c4[3], m16 = m8a * m8b;
+        if (__all_sync(0xffffffffu, m16 != 0u)) sink.put(c8a * m8b + c8b, 31 - __clz((int)m16));
+        else { sink.put(c8a, 31 - __clz((int)m8a)); sink.put(c8b, 31 - __clz((int)m8b)); }
+    } else {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            if (__all_sync(0xffffffffu, m4[i] != 0u)) sink.put(c4[i], 31 - __clz((int)m4[i]));
+            else { sink.put(code[2 * i], 31 - __clz((int)mul[2 * i])); sink.put(code[2 * i + 1], 31 - __clz((int)mul[2 * i + 1])); }
+        }
+    }
+}
+
+// A thread's blocks quantised and coded from the accumulator once more, for tiles that the plan does not fit.  A
+// function of its own, so that what it keeps in registers does not weigh on the loop that every tile goes through (inlined, it
+// cost that loop up to 7 %: 64x56x56 x 256 at 8 bits 103 -> 110 us).  All lanes of the warp call it together.
+template <bool kPerChannel, bool kPair, typename Sink>
+__device__ __noinline__ Sink code_again(Sink sink, uint32_t trow, int blk0, int blk1, float inv_range, float top, const float *s_bias,
+                                        uint32_t enc_addr, const uint32_t *enc, int bits)
+{
+#pragma unroll 1
+    for (int blk = blk0; blk < blk1; ++blk) {
+        uint32_t r[16], qv[16], mul[8], code[8];
+        tmem_ld_32x32b_x16(trow + blk * 16, r);
+        tmem_ld_wait(r);
+#pragma unroll
+        for (int i = 0; i < 16; i += 4) {
+            const float4 b4 = *reinterpret_cast<const float4 *>(s_bias + blk * 16 + i);
+            quantise_bits2(r[i], r[i + 1], inv_range, b4.x, b4.y, top, qv[i], qv[i + 1]);
+            quantise_bits2(r[i + 2], r[i + 3], inv_range, b4.z, b4.w, top, qv[i + 2], qv[i + 3]);
+        }
+        block_pieces<kPerChannel, kPair>(qv, enc_addr, enc, blk * 16, bits, mul, code);
+        append_block(sink, mul, code);
+    }
+    return sink;
 }
 
 // The epilogue's two ways (kRuns):
@@ -340,7 +413,7 @@ __global__ void __launch_bounds__(kThreads, 1) encode_tc_kernel(EncodeArgs a, Pl
     } else if (warp >= kStoreWarp0) {
         // ================= store warps =================
         const int grp = warp - kStoreWarp0;
-        const uint32_t stg_addr = smem_u32(smem + L.staging + (uint32_t)grp * pl.staging_bytes);
+        const uint32_t stg_addr = smem_u32(smem + L.staging + (uint32_t)grp * (pl.staging_bytes + L.run_bytes));
         long long n = 0;
         for (long long tl = grp; tl < my_tiles; tl += 2, ++n) {
             const long long tile = blockIdx.x + tl * gridDim.x;
@@ -384,10 +457,10 @@ __global__ void __launch_bounds__(kThreads, 1) encode_tc_kernel(EncodeArgs a, Pl
         const int blk0 = half ? pl.split_blk : 0, blk1 = half ? n_blk : pl.split_blk;
         const int chunk_blks = a.splits > 1 ? n_blk / a.splits : n_blk;    // blocks per chunk of a pixel
         const int bound0 = max(1, (blk0 + chunk_blks - 1) / chunk_blks);   // the first chunk boundary that lies before one of this thread's blocks
-        const uint32_t stg_addr = smem_u32(smem + L.staging + (uint32_t)grp * pl.staging_bytes);
+        const uint32_t stg_addr = smem_u32(smem + L.staging + (uint32_t)grp * (pl.staging_bytes + L.run_bytes));
         const uint32_t enc_addr = smem_u32(s_enc);
         const uint32_t len8_addr = smem_u32(smem + L.len8);
-        const uint32_t run_addr = smem_u32(smem + L.runs) + (uint32_t)grp * L.run_bytes + (half ? (uint32_t)pl.run_words[0] * kRunStep : 0u) + (uint32_t)m * 4u;
+        const uint32_t run_addr = stg_addr + pl.staging_bytes + (half ? (uint32_t)pl.run_words[0] * kRunStep : 0u) + (uint32_t)m * 4u;
         const uint32_t run_end = run_addr + (uint32_t)pl.run_words[half] * kRunStep;
         uint32_t *xch = reinterpret_cast<uint32_t *>(smem + L.xch + grp * (2 * 128 * 4 + 3 * 128 * 2));   // [2][128]: prefix in the warp << 12 | bits
         unsigned short *bound = reinterpret_cast<unsigned short *>(xch + 256);                            // [3][128]: bits before chunk boundary 1 ..., from its thread's start
@@ -425,7 +498,8 @@ __global__ void __launch_bounds__(kThreads, 1) encode_tc_kernel(EncodeArgs a, Pl
             // issues nothing, whereas polling warps took two thirds of the SM's instructions.
             if (wg == 0) {
                 bool go = mbar_wait(smem_u32(&s_tfull[grp]), (uint32_t)((tl >> 1) & 1), 200u);
-                if (n_done >= 2) go = go && mbar_wait(smem_u32(&s_stg_free[grp][(n_done - 2) % kSlots]), ((n_done - 2) / kSlots) & 1u);
+                const unsigned int back = prev_end > pl.staging_bytes ? 1u : 2u;      // (the tile before lies in the runs, too)
+                if (n_done >= back) go = go && mbar_wait(smem_u32(&s_stg_free[grp][(n_done - back) % kSlots]), ((n_done - back) / kSlots) & 1u);
                 if (lane == 0) s_go[grp] = go;
                 tc_fence_before_sync();
             }
@@ -484,46 +558,9 @@ __global__ void __launch_bounds__(kThreads, 1) encode_tc_kernel(EncodeArgs a, Pl
                         sink.bits += l;
                     }
                 } else {
-                    // two symbols a piece: (1 << length, code), at most 24 bits
                     uint32_t mul[8], code[8];
-#pragma unroll
-                    for (int i = 0; i < 8; ++i) {
-                        if constexpr (kPair) {
-                            const uint32_t idx = (qv[2 * i] - kMagicBits) + ((qv[2 * i + 1] - kMagicBits) << a.bits);
-                            asm("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(mul[i]), "=r"(code[i]) : "r"(enc_addr + idx * 8u));
-                        } else {
-                            uint32_t m0, c0, m1, c1;
-                            if constexpr (kPerChannel) {
-                                const int j = blk * 16 + 2 * i;
-                                const uint32_t e0 = __ldg(a.enc + j * nsym + (qv[2 * i] & 0xffu)), e1 = __ldg(a.enc + (j + 1) * nsym + (qv[2 * i + 1] & 0xffu));
-                                m0 = 1u << (e0 & 0xffu); c0 = e0 >> 8; m1 = 1u << (e1 & 0xffu); c1 = e1 >> 8;
-                            } else {
-                                asm("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(m0), "=r"(c0) : "r"(enc_addr + (qv[2 * i] - kMagicBits) * 8u));
-                                asm("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(m1), "=r"(c1) : "r"(enc_addr + (qv[2 * i + 1] - kMagicBits) * 8u));
-                            }
-                            mul[i] = m0 * m1;
-                            code[i] = c0 * m1 + c1;
-                        }
-                    }
-                    // How many symbols are joined before they are appended is chosen for the whole warp (lanes
-                    // that go different ways run one after the other): sixteen or eight where every lane's
-                    // codes of them fit 31 bits -- a product of powers of two that reaches 2^32 is zero --
-                    // else four, else two.  Joining is a multiply-add, appending costs ten instructions.
-                    uint32_t m4[4], c4[4];
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) { m4[i] = mul[2 * i] * mul[2 * i + 1]; c4[i] = code[2 * i] * mul[2 * i + 1] + code[2 * i + 1]; }
-                    const uint32_t m8a = m4[0] * m4[1], m8b = m4[2] * m4[3];
-                    if (__all_sync(0xffffffffu, m8a != 0u && m8b != 0u)) {
-                        const uint32_t c8a = c4[0] * m4[1] + c4[1], c8b = c4[2] * m4[3] + c4[3], m16 = m8a * m8b;
-                        if (__all_sync(0xffffffffu, m16 != 0u)) sink.put(c8a * m8b + c8b, 31 - __clz((int)m16));
-                        else { sink.put(c8a, 31 - __clz((int)m8a)); sink.put(c8b, 31 - __clz((int)m8b)); }
-                    } else {
-#pragma unroll
-                        for (int i = 0; i < 4; ++i) {
-                            if (__all_sync(0xffffffffu, m4[i] != 0u)) sink.put(c4[i], 31 - __clz((int)m4[i]));
-                            else { sink.put(code[2 * i], 31 - __clz((int)mul[2 * i])); sink.put(code[2 * i + 1], 31 - __clz((int)mul[2 * i + 1])); }
-                        }
-                    }
+                    block_pieces<kPerChannel, kPair>(qv, enc_addr, a.enc, blk * 16, a.bits, mul, code);
+                    append_block(sink, mul, code);
                 }
             };
 
@@ -551,11 +588,12 @@ __global__ void __launch_bounds__(kThreads, 1) encode_tc_kernel(EncodeArgs a, Pl
                 };
                 if constexpr (!kCanSkip) one_by_one(blk1);
                 else {
+                    int plain = min(max(skip_blk, blk), blk1);               // this far without the test
 #pragma unroll 1
-                    while (blk < blk1) {
-                        int plain = min(max(skip_blk, blk), blk1);           // this far without the test
+                    while (true) {
                         if (plain + 2 > blk1) plain = blk1;
                         one_by_one(plain);
+                        if (blk >= blk1) break;
 #pragma unroll 1
                         while (blk + 2 <= blk1 && bound_blk != blk + 1) {
                             uint32_t r0[16], r1[16];
@@ -581,7 +619,7 @@ __global__ void __launch_bounds__(kThreads, 1) encode_tc_kernel(EncodeArgs a, Pl
                             else sink.put_word(0u);
                             blk += 2;
                         }
-                        if (blk < blk1) one_by_one(min(blk + 2, blk1));
+                        plain = min(blk + 2, blk1);
                     }
                 }
             };
@@ -665,6 +703,7 @@ __global__ void __launch_bounds__(kThreads, 1) encode_tc_kernel(EncodeArgs a, Pl
             const unsigned long long padded = ((unsigned long long)tile_bits + 127ull) & ~127ull;
             if (tg == 0) lookback_publish(a.tile_state, tile, padded);
             const bool staged = padded <= (unsigned long long)pl.staging_bytes * 8ull && !(kRuns && s_overflow[grp] == n_done + 1);
+            const bool fits = staged || (kRuns && padded <= (unsigned long long)(pl.staging_bytes + L.run_bytes) * 8ull);    // coded again, where the runs are in the way
             if (kRuns && staged) {                 // the accumulator is free for the tile after next
                 tc_fence_before_sync();
                 __syncwarp();
@@ -672,7 +711,7 @@ __global__ void __launch_bounds__(kThreads, 1) encode_tc_kernel(EncodeArgs a, Pl
             }
             // place in the staging ring: behind the newest tile, or at the buffer's start if it would not
             // fit before the end
-            const unsigned int tile_bytes = staged ? (unsigned int)(padded >> 3) : 0u;
+            const unsigned int tile_bytes = fits ? (unsigned int)(padded >> 3) : 0u;
             const unsigned int stg_at = prev_end + tile_bytes > pl.staging_bytes ? 0u : prev_end;
             if (n_done >= 1 && stg_at < prev_end && prev_at < stg_at + tile_bytes) {
                 // one warp waits for all (the condition is the same in every thread): warps whose waits end
@@ -732,9 +771,22 @@ __global__ void __launch_bounds__(kThreads, 1) encode_tc_kernel(EncodeArgs a, Pl
                     w.finish();
                 }
                 if (tg == 0) { s_padded[grp][n_done % kSlots] = (unsigned int)padded; s_stg_at[grp][n_done % kSlots] = stg_at; s_store_cmd[grp][n_done % kSlots] = 1; }
+            } else if (kRuns && fits) {
+                // a run is longer than the plan allows for, or the tile than the staging buffer
+                const unsigned int first_open = tile_bits >> 5, end_word = (unsigned int)(padded >> 5);
+                if ((unsigned int)tg < end_word - first_open)
+                    asm volatile("st.shared.u32 [%0], %1;" ::"r"(tile_addr + (first_open + tg) * 4u), "r"(0u) : "memory");
+                SmemBitWriter<4> w;
+                w.init(valid ? tile_addr : 0u, valid ? tile_addr + tile_bytes : 0u, valid ? my_off : 0u);
+                w = code_again<kPerChannel, kPair>(w, trow, blk0, blk1, inv_range, top, s_bias, enc_addr, a.enc, a.bits);
+                tc_fence_before_sync();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(smem_u32(&s_tempty[grp]));
+                named_bar_sync(bar_id, 256);
+                w.finish();
+                if (tg == 0) { s_padded[grp][n_done % kSlots] = (unsigned int)padded; s_stg_at[grp][n_done % kSlots] = stg_at; s_store_cmd[grp][n_done % kSlots] = 1; }
             } else {
-                // rare: the tile (or a run) does not fit -> resolve its position first and pack straight
-                // into (zeroed) global memory
+                // rare: the tile does not fit -> resolve its position first and pack straight into (zeroed) global memory
                 resolve_base(tile, padded);
                 named_bar_sync(bar_id, 256);
                 if (s_write_ok[grp]) {
@@ -783,7 +835,9 @@ __global__ void __launch_bounds__(kThreads, 1) encode_tc_kernel(EncodeArgs a, Pl
 // What a launch does with the shared memory that the basis leaves, from the code lengths to expect of
 // the model's coefficients (a code without a one-bit symbol: b bits for each).  A tile's size varies
 // by a few per cent about its mean, a thread's run by its symbols that are not the zero level.  A tile
-// that breaks the estimate is coded at about a quarter of the speed (straight into global memory).
+// that breaks the estimate is coded once more, over the staging buffer and the runs behind it (256x14x14 x 4096, 4 bits, maps of
+// twice the calibration's spread: 243 us; 348 when such tiles went straight into global memory, as those still do that
+// fit neither).
 // Preferred, in this order: symbol pairs before single symbols, private runs before two passes, eight
 // ring stages before six.
 static Plan make_plan(const tc_ctx *ctx, const EncodeArgs &a)

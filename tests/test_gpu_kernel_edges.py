@@ -296,3 +296,32 @@ def test_run_skipping_decoder_stream_buffers(ctx, c, h, w, bits, ratio, cp):
     assert float((a != b).double().mean()) <= 1e-3
     for h_ in (m, cb, again):
         h_.close()
+
+
+# Resident-basis encoder, private runs shorter than the codes: a model whose eigenvalues say too little (or nothing) and
+# maps of more spread than the calibration's.  Tiles are then coded once more into the staging buffer, over the runs
+# behind it, or into global memory; the words are those of a plan that allows for everything (eigenvalues 100 times
+# too large), and those of the streaming kernels' coder on the same symbols.
+@pytest.mark.parametrize("c,bits,tables,spread", [(256, 4, 1, 1), (256, 4, 1, 2), (256, 4, 1, 6), (64, 4, 1, 5), (128, 6, 1, 3), (128, 8, 1, 1),
+                                                  (208, 5, 1, 3), (16, 2, 1, 4), (96, 4, 96, 3), (256, 3, 256, 5), (240, 8, 1, 8)])
+def test_runs_shorter_than_the_codes(ctx, c, bits, tables, spread):
+    params = fm.layer_params(fm.LayerSpec(c, 14, 14, 0.9, None, 17000 + c + bits))
+    cal = fm.make_maps(params, 256, calib=True, dtype=torch.bfloat16, device="cuda")
+    m = tc.tc_fit_pca(ctx, cal, bits)
+    cb = tc.tc_build_codebook(ctx, m, tc.tc_stats(ctx, m, None, cal, groups=tables).hist, groups=tables)
+    d = tc.tc_model_export(m)
+    mean = torch.from_numpy(d["mean"]).float().cuda().view(1, c, 1, 1)
+    x = ((fm.make_maps(params, 1500, dtype=torch.float32, device="cuda") - mean) * spread + mean).to(torch.bfloat16)      # several tiles a group
+    x[7] = cal[0]                                                     # tiles that do fit between those that do not
+    args = dict(basis=d["basis"], mean=d["mean"], lo=d["lo"], step=d["step"], bits=bits, basis_dtype=1, k=d["k"])
+    ample = tc.tc_model_import(ctx, eig=d["eig"] * 100, **args)
+    ref = tc.tc_encode(ctx, ample, cb, x, debug=True)
+    assert tc.tc_get_status(ctx) == 0 and tc.tc_last_path(ctx) == 1
+    check_stream_against_oracle(tc.tc_encode(ctx, ample, cb, x[:9], debug=True), ref.symbols[:9 * 196].cpu().numpy(), tc.tc_codebook_export(cb), bits)
+    for eig in (d["eig"], d["eig"] / 100, np.full(c, 1e-9), None):
+        own = tc.tc_model_import(ctx, eig=eig, **args)
+        assert _same_stream(tc.tc_encode(ctx, own, cb, x), ref)
+        assert tc.tc_get_status(ctx) == 0
+        own.close()
+    for h in (m, cb, ample):
+        h.close()
