@@ -325,3 +325,24 @@ def test_runs_shorter_than_the_codes(ctx, c, bits, tables, spread):
         own.close()
     for h in (m, cb, ample):
         h.close()
+
+
+# The decoder's side of it: eight channel rows of 2^29 pixels are further apart than 32 bits count.
+def test_decoded_rows_more_than_2_32_elements_apart(ctx):
+    c, h, w, parts = 16, 16384, 32768, 64
+    g = torch.Generator(device="cuda").manual_seed(18)
+    x = torch.empty(1, c, h, w, dtype=torch.bfloat16, device="cuda")
+    for i in range(c):
+        x[0, i] = torch.randn(h, w, generator=g, device="cuda")
+    cal = x[:, :, :256, :256].contiguous()
+    m = tc.tc_fit_pca(ctx, cal, 3)
+    cb = tc.tc_build_codebook(ctx, m, tc.tc_stats(ctx, m, None, cal).hist)
+    enc = tc.tc_encode(ctx, m, cb, x, capacity=6 << 30)
+    assert tc.tc_get_status(ctx) == 0
+    del x
+    a = tc.tc_decode(ctx, m, cb, enc, (1, c, h, w), torch.bfloat16)
+    b = tc.tc_decode(ctx, m, cb, enc, (parts, c, h // parts, w), torch.bfloat16)
+    assert tc.tc_get_status(ctx) == 0 and tc.tc_last_path(ctx, True) == 1
+    for i in range(c):
+        assert torch.equal(a[0, i].view(parts, h // parts, w), b[:, i])
+    m.close(); cb.close()
