@@ -198,13 +198,13 @@ tc_status tc_launch_channel_sums(const void *x, int dtype, int n, int c, int hw,
 }
 
 tc_status tc_launch_covariance(const void *x, int dtype, int n, int c, int hw, const double *mean, double *cov,
-                               cudaStream_t s)
+                               int sm_count, cudaStream_t s)
 {
     const int bpd = (c + kCovTile - 1) / kCovTile;
     const int pairs = bpd * (bpd + 1) / 2;
     const long long pixels = (long long)n * hw;
     long long slabs = (pixels + kCovSlab - 1) / kCovSlab;
-    const long long want = (592 + pairs - 1) / pairs;        // two rounds of two blocks for each of 148 SMs
+    const long long want = (4ll * sm_count + pairs - 1) / pairs;        // two rounds of two blocks for each SM
     if (slabs > want) slabs = want;
     if (slabs < 1) slabs = 1;
     dim3 grid((unsigned int)slabs, (unsigned int)pairs);

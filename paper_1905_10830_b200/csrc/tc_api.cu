@@ -552,7 +552,7 @@ tc_status tc_fit_pca(tc_ctx *ctx, const tc_tensor *calib, const tc_fit_params *p
     TC_CUDA(cudaStreamSynchronize(s));
     for (double &v : mean) v /= (double)m_samples;
     TC_CUDA(cudaMemcpyAsync(d_mean, mean.data(), sizeof(double) * c, cudaMemcpyHostToDevice, s));
-    st = tc_launch_covariance(calib->data, calib->dtype, n, c, hw, d_mean, d_cov, s);
+    st = tc_launch_covariance(calib->data, calib->dtype, n, c, hw, d_mean, d_cov, ctx->sm_count, s);
     if (st != TC_OK) return st;
     // centred sums in the upper triangle -> covariance, full symmetric, still on the device
     if ((st = tc_launch_scale_mirror(d_cov, c, (double)(m_samples - 1), s)) != TC_OK) return st;
@@ -672,7 +672,7 @@ tc_status tc_fit_state_update(tc_ctx *ctx, tc_fit_state *st, const tc_tensor *ma
     if ((long long)maps->n * hw == 0) return TC_OK;
     tc_status rc = tc_launch_channel_sums(maps->data, maps->dtype, maps->n, st->c, hw, st->d_sum, s);
     if (rc != TC_OK) return rc;
-    rc = tc_launch_covariance(maps->data, maps->dtype, maps->n, st->c, hw, st->d_zero, st->d_outer, s);
+    rc = tc_launch_covariance(maps->data, maps->dtype, maps->n, st->c, hw, st->d_zero, st->d_outer, ctx->sm_count, s);
     if (rc != TC_OK) return rc;
     st->count += (long long)maps->n * hw;
     return TC_OK;
