@@ -155,9 +155,8 @@ def _stream_ptr(device) -> int:
     return torch.cuda.current_stream(device).cuda_stream
 
 
-def _tensor_stream(device: int) -> int:
-    """The same for calls that have a CUDA tensor (CUDA is initialised): 0.1 us a call instead of 1.3."""
-    return torch._C._cuda_getCurrentRawStream(device)
+# The same for calls that have a CUDA tensor (CUDA is initialised): 0.1 us a call instead of 1.3, where this torch has it.
+_tensor_stream = getattr(torch._C, "_cuda_getCurrentRawStream", _stream_ptr)
 
 
 class _Handle:
