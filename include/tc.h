@@ -17,7 +17,8 @@
  *     channels, unaligned maps, per-channel code tables, few tiles: up to about 64 MB, in passes) and 8 bytes per tile of
  *     about a million tiles; a list takes up to eight workspaces.  It grows inside the call that needs more, which
  *     stops the device while memory is released and allocated.  If that memory cannot be had, tc_encode, tc_decode and
- *     their list forms run on kernels that need no workspace (same stream; slower).
+ *     their list forms run on kernels that need no workspace: slower, the same stream, tensors that may differ
+ *     in the rounding of the last bit.
  *   - `cuda_stream` is a cudaStream_t passed as void* (NULL = the default stream).  Calls that
  *     take one are asynchronous on it unless stated otherwise.
  *   - A context serves one stream at a time: its scratch arena (the cross-tile bookkeeping of
@@ -99,9 +100,10 @@ tc_status tc_get_status(tc_ctx *ctx, void *cuda_stream);
  * not be had, on the kernels that need none; 0 restores the default. */
 void tc_force_exact_path(tc_ctx *ctx, int on);
 /* Which kernels the last tc_encode (decode == 0) or tc_decode (decode != 0) of this context
- * launched: 0 = fp64 kernels, 1 = tensor-core kernels with the basis resident in shared
- * memory, 2 = fp32 kernels, 3 = tensor-core kernels that stream the basis; -1 for a NULL
- * context. */
+ * launched: 0 = fp64 kernels, 1 = tensor-core kernels for up to 256 channels (basis resident on the SM; decodes
+ * with per-channel code tables: the tiled product, where its workspace could be had), 2 = fp32 kernels,
+ * 3 = tensor-core kernels for wide layers and unaligned maps (basis streamed: tiled products, or fused
+ * kernels where the workspace could not be had or debug outputs were asked for); -1 for a NULL context. */
 int tc_last_path(const tc_ctx *ctx, int decode);
 
 /* ---------------------------------------------------------------------------------------
@@ -288,13 +290,15 @@ typedef struct {
     int32_t relu;         /* tc_decode / tc_roundtrip_host only: non-zero applies the layer's
                              non-linearity after the inverse transform (Section 3.1),
                              x_hat = max(T^T y_hat + mu, 0), before rounding to the tensor type */
-    int32_t mean_tile_bytes; /* tc_decode only, a hint that changes speed, never results: the mean size
-                             of a tile's stream segment in bytes (stream length / n_tiles), 0 = not
-                             known.  It matters for per-channel code tables on layers of up to 256
-                             channels: the decoder that keeps the basis in shared memory stages
-                             segments of up to about 14 KB there and reads longer ones from global
-                             memory word by word, the decoder that streams the basis stages up to
-                             32 KB; told that the segments are long, tc_decode picks the second.
+    int32_t mean_tile_bytes; /* tc_decode only, a hint that changes speed, not results (but for the rounding of the
+                             last bit, where it picks another kernel): the mean size of a tile's stream
+                             segment in bytes (stream length / n_tiles), 0 = not known.  The decoder for per-layer tables and up to 256 channels sizes the
+                             shared memory for segments by it (without it: by the counts the code table
+                             was built from, or its lengths): a segment that does not fit is read from global
+                             memory word by word.  For per-channel tables it matters only where the
+                             workspace could not be had: the decoder that keeps the basis in shared memory then
+                             stages segments of up to about 14 KB, the one that streams the basis
+                             up to 32 KB; told that the segments are long, tc_decode picks the second.
                              tc_decode never infers the rate from `stream_bytes` (which may be the
                              length of the stream or the capacity of its buffer).            */
 } tc_encode_params;

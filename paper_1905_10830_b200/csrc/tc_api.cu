@@ -1092,7 +1092,9 @@ static tc_status decode_with_scratch(tc_ctx *ctx, const tc_model *m, const tc_co
         return tc_launch_decode_runs(ctx, a, (cudaStream_t)cuda_stream);
     }
     bool resident = (ctx->force_exact == 0 || ctx->force_exact == 3) && x_hat->dtype == TC_BF16 && tc_decode_tc_supported(ctx, a);
-    // High-rate streams (params->mean_tile_bytes): a tile's segment that no longer fits the shared-memory
+    // with workspace: the entropy decoder as a kernel of its own, the inverse as a tiled product
+    const bool product = sym_scratch && wide_decode(ctx, m, cb, x_hat) && a.basis_t_map;
+    // Without it, high-rate streams (params->mean_tile_bytes; the route is named after it either way): a tile's segment that no longer fits the shared-memory
     // staging of the resident-basis decoder but still fits that of the streaming decoder is better
     // served by the latter (the former would read the stream from global memory word by word).
     const size_t hint = (params && params->mean_tile_bytes > 0) ? (size_t)params->mean_tile_bytes : 0;
@@ -1101,15 +1103,12 @@ static tc_status decode_with_scratch(tc_ctx *ctx, const tc_model *m, const tc_co
         resident = false;
     if (resident) {
         ctx->last_decode_path = 1;
-        if (sym_scratch && wide_decode(ctx, m, cb, x_hat) && a.basis_t_map)
-            return tc_launch_decode_wide_gemm(ctx, a, sym_scratch, (cudaStream_t)cuda_stream);
+        if (product) return tc_launch_decode_wide_gemm(ctx, a, sym_scratch, (cudaStream_t)cuda_stream);
         return tc_launch_decode_tc(ctx, a, (cudaStream_t)cuda_stream);
     }
     if (ctx->force_exact != 1 && x_hat->dtype == TC_BF16 && tc_decode_wide_supported(ctx, a)) {   // wide layers
         ctx->last_decode_path = 3;
-        // with workspace: the entropy decoder as a kernel of its own, the inverse as a tiled product
-        if (sym_scratch && wide_decode(ctx, m, cb, x_hat) && a.basis_t_map)
-            return tc_launch_decode_wide_gemm(ctx, a, sym_scratch, (cudaStream_t)cuda_stream);
+        if (product) return tc_launch_decode_wide_gemm(ctx, a, sym_scratch, (cudaStream_t)cuda_stream);
         return tc_launch_decode_wide(ctx, a, (cudaStream_t)cuda_stream);
     }
     if (ctx->force_exact != 1 && x_hat->dtype == TC_BF16 && x_hat->c % 2 == 0) {  // shapes the tensor-core kernel does not take

@@ -362,11 +362,12 @@ def test_streaming_kernels_on_narrow_layers(ctx_stream, c, s, n, bits, splits):
 
 
 def test_rate_hint_picks_the_decoder_for_per_channel_tables(ctx_tc):
-    # 256 channels at 8 bits with per-channel code tables.  tc_decode never reads a rate into
+    # 256 channels at 8 bits with per-channel code tables, without workspace (mode 4; with it the tiled product
+    # runs, whatever the hint says and the route is called).  tc_decode never reads a rate into
     # `stream_bytes`; told (tc_encode_params.mean_tile_bytes) that a tile's segment is longer than the
     # resident-basis decoder stages in shared memory, it picks the streaming kernel, which stages up
-    # to 32 KB; without the hint, or with a small one, the resident-basis decoder runs.  The hint
-    # changes speed only: all three calls return the same tensor.
+    # to 32 KB; without the hint, or with a small one, the resident-basis decoder runs.  All three meet the
+    # same bar; calls that run the same kernel return the same tensor.
     spec = fm.LayerSpec(256, 14, 14, 0.9, None, 6500)
     o = H.oracle_side(spec, 8, 6, 8, torch.bfloat16, True)
     model = H.import_model(tc, ctx_tc, o["model"], torch.bfloat16)
@@ -375,17 +376,19 @@ def test_rate_hint_picks_the_decoder_for_per_channel_tables(ctx_tc):
     enc = tc.tc_encode(ctx_tc, model, cb, x, debug=True)
     nbytes = enc.total_bits() // 8
     outs = []
-    for hint, route in ((30000, 3), (None, 1), (2000, 1)):
+    for mode, hint, route in ((4, 30000, 3), (4, None, 1), (4, 2000, 1), (0, 30000, 3), (0, None, 1), (0, 2000, 1)):
+        tc.tc_force_exact_path(ctx_tc, mode)
         outs.append(tc.tc_decode(ctx_tc, model, cb, enc, x.shape, torch.bfloat16, stream_bytes=nbytes if hint else None,
                                  mean_tile_bytes=hint))
         assert tc.tc_get_status(ctx_tc) == 0 and tc.tc_last_path(ctx_tc, True) == route
+        tc.tc_force_exact_path(ctx_tc, 0)
     want = oracle.reconstruct(o["model"], enc.symbols.cpu().numpy(), x.shape, out_bf16=True)
     expected = H.expected_output_flips(o["model"], enc.symbols.cpu().numpy())
     for got in (t.float().cpu().numpy() for t in outs):
         ulp = 2.0 ** (np.floor(np.log2(np.maximum(np.abs(want), 1e-30))) - 7)
         assert np.all(np.abs(got - want) <= np.maximum(1e-3 * np.maximum(np.abs(want), o["model"].step), ulp))
         assert H.count_output_flips(got, want) <= H.flip_allowance(expected)
-    assert torch.equal(outs[1], outs[2])
+    assert torch.equal(outs[1], outs[2]) and torch.equal(outs[3], outs[4]) and torch.equal(outs[4], outs[5])
     model.close(); cb.close()
 
 
