@@ -103,3 +103,45 @@ def test_many_reuses_buffers_and_rejects_a_bad_item_before_launching(ctx):
         tc.tc_encode_many(ctx, layers, outs=first[:-1] + [skewed])
     torch.cuda.synchronize()
     assert all(bool((e.words == 0x33).all()) for e in first)
+
+
+def test_tensors_that_share_a_stream_and_its_workspace(ctx):
+    # 24 items on eight streams, every one with workspace of another size: wide layers, unaligned maps, per-channel code tables,
+    # fp32 maps and one wide layer that takes several passes; three follow each other on a stream.  Byte for byte the
+    # single calls, twice (the second call meets the first one's leftovers) and in another order.
+    shapes = [(320, 7, 7, 40, torch.bfloat16, False), (576, 14, 14, 9, torch.bfloat16, False), (272, 28, 28, 200, torch.bfloat16, False),
+              (960, 7, 7, 30, torch.bfloat16, False), (80, 27, 19, 37, torch.bfloat16, True), (48, 5, 3, 300, torch.bfloat16, False),
+              (256, 14, 14, 60, torch.bfloat16, True), (64, 9, 9, 3, torch.bfloat16, True), (48, 12, 12, 3, torch.float32, True),
+              (128, 10, 10, 2, torch.float32, False), (1024, 4, 4, 5, torch.bfloat16, False), (16, 28, 28, 20, torch.bfloat16, True)]
+    items = []
+    for i, (c, h, w, n, dtype, per_channel) in enumerate(shapes):
+        params = fm.layer_params(fm.LayerSpec(c, h, w, 0.9, None, 8900 + i))
+        cal = fm.make_maps(params, max(8, 2 * c // (h * w) + 1), calib=True, dtype=dtype, device="cuda")
+        m = tc.tc_fit_pca(ctx, cal, 4 + i % 3)
+        groups = c if per_channel else 1
+        cb = tc.tc_build_codebook(ctx, m, tc.tc_stats(ctx, m, None, cal, groups=groups).hist, groups=groups)
+        x = fm.make_maps(params, n, dtype=dtype, device="cuda")
+        items += [(m, cb, x), (m, cb, x[: (n + 1) // 2].contiguous())]
+    want = []
+    for m, cb, x in items:
+        e = tc.tc_encode(ctx, m, cb, x)
+        want.append((e, tc.tc_decode(ctx, m, cb, e, x.shape, x.dtype)))
+    assert tc.tc_get_status(ctx) == 0
+    outs = decs = None
+    for order in (range(24), range(24), [5 * i % 24 for i in range(24)]):
+        outs = [outs[i] for i in order] if outs else None
+        decs = [torch.full_like(d, 7.0) for d in decs] if decs else None
+        decs = [decs[i] for i in order] if decs else None
+        if outs:
+            for e in outs:
+                e.words.fill_(0x5A)
+        outs = tc.tc_encode_many(ctx, [items[i] for i in order], outs=outs)
+        decs = tc.tc_decode_many(ctx, [(items[i][0], items[i][1], e, items[i][2].shape, items[i][2].dtype) for i, e in zip(order, outs)], outs=decs)
+        assert tc.tc_get_status(ctx) == 0
+        for i, e, d in zip(order, outs, decs):
+            n = want[i][0].total_bits() // 8
+            assert torch.equal(e.tile_off, want[i][0].tile_off) and torch.equal(e.words[:n], want[i][0].words[:n])
+            assert torch.equal(e.chunk_len[:e.layout.n_chunks], want[i][0].chunk_len[:e.layout.n_chunks])
+            assert torch.equal(d, want[i][1])
+    for m, cb, _ in items[::2]:
+        m.close(); cb.close()
