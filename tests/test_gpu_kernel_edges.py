@@ -70,11 +70,14 @@ def test_device_eigh_block_shapes_and_indefinite(ctx, n, shift):
 
 # Per-channel codes decoded from their bounds: one-symbol-dominated, flat and maximum-length (12 bit)
 # tables side by side, every kernel that reads them (fp64 kernels with 1, 2 and 4 chunks a pixel and
-# runs that are no multiple of 16, resident and streaming tensor-core decoders).
+# runs that are no multiple of 16, the tiled product's decoder, and -- without workspace (mode 4), or with the run-skipping
+# decoder left out (mode 3) -- the resident and streaming tensor-core decoders).
 @pytest.mark.parametrize("c,k,s,n,bits,dtype,cp,splits,mode", [
     (16, 16, 3, 1, 8, torch.float32, 0, 0, 0), (40, 24, 9, 2, 6, torch.float32, 0, 0, 0), (256, 256, 7, 2, 5, torch.float32, 0, 0, 0),
     (512, 512, 4, 1, 8, torch.float32, 0, 0, 0), (64, 64, 9, 2, 1, torch.float32, 4, 1, 0), (48, 48, 9, 2, 7, torch.bfloat16, 0, 0, 0),
-    (256, 256, 14, 1, 6, torch.bfloat16, 0, 0, 0), (128, 128, 7, 3, 8, torch.bfloat16, 0, 0, 2), (320, 320, 5, 2, 4, torch.bfloat16, 0, 0, 0)])
+    (256, 256, 14, 1, 6, torch.bfloat16, 0, 0, 0), (128, 128, 7, 3, 8, torch.bfloat16, 0, 0, 2), (320, 320, 5, 2, 4, torch.bfloat16, 0, 0, 0),
+    (256, 256, 14, 1, 6, torch.bfloat16, 0, 0, 3), (48, 48, 9, 2, 7, torch.bfloat16, 0, 0, 4), (128, 128, 7, 3, 8, torch.bfloat16, 0, 0, 4),
+    (320, 320, 5, 2, 4, torch.bfloat16, 0, 0, 4), (256, 256, 7, 2, 5, torch.float32, 0, 0, 4)])
 def test_per_channel_codes_from_bounds(ctx, c, k, s, n, bits, dtype, cp, splits, mode):
     spec = fm.LayerSpec(c, s, s, 0.9, None, 12000 + c + bits)
     o = H.oracle_side(spec, bits, max(3, 2 * c // (s * s) + 1), n, dtype, True, k=k)
