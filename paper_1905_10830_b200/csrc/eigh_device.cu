@@ -153,9 +153,10 @@ __device__ __forceinline__ double norm2(const double2 (&x)[R])
 // they already are, to rounding: below `tol2` (squared) of the norms a rotation would only chase noise.
 // The angle is computed in fp32 -- the rotations' angles steer the iteration, an error of 1e-7 of
 // one leaves 1e-7 of the inner product for the next sweep -- but the matrix applied is a rotation
-// to fp64: cosine and tan(angle / 2) follow from that tangent by a cubic correction of the
-// fp32 reciprocal (square root), and the update x -= s (y + u x), y += s (x - u y) rounds in
-// proportion to the angle.
+// to fp64: cosine and tan(angle / 2) follow from that tangent by one step of Householder's third-order
+// iteration from the fp32 reciprocal (square root) -- r (1 + e / 2 + 3 e^2 / 8) with e = 1 - q r^2 for
+// 1 / sqrt(q), r (1 + e + e^2) with e = 1 - k r for 1 / k; e is below 1e-6, the term left out below 1e-18 --
+// and the update x -= s (y + u x), y += s (x - u y) rounds in proportion to the angle.
 template <int R>
 __device__ __forceinline__ bool rotate_pair(double2 (&x)[R], double2 (&y)[R], double &al, double &be, double tol2)
 {

@@ -122,3 +122,19 @@ def test_online_fit_finishes_on_the_device(ctx):
         assert np.abs(online["basis"] - other["basis"]).max() <= 2.0 ** -8
         assert (online["basis"] == other["basis"]).mean() >= 0.999
         assert np.isclose(online["lo"], other["lo"], rtol=1e-6, atol=1e-6) and np.isclose(online["step"], other["step"], rtol=1e-6)
+
+
+@pytest.mark.parametrize("n", [2, 3, 5])
+def test_rotations_are_orthogonal_to_fp64(ctx, n):
+    # Few columns, angles of every size: cosine and tangent of a rotation start from fp32 (1e-7), and a rotation that is
+    # orthogonal to that only would leave 1e-7 |A| beside the diagonal.  Inner products stop at 8 sqrt(16) eps of the
+    # norms, which (1.25 + 1) |A|_F turns into at most 2.25 times that; as much again for the rounding of the sweeps.
+    rng = np.random.default_rng(70 + n)
+    for i in range(60):
+        a = rng.standard_normal((n, n)) * 10.0 ** rng.uniform(-6, 0, (n, n))
+        a = (a + a.T) / 2
+        evals, evecs, _ = tc.tc_device_eigh(ctx, torch.from_numpy(a).cuda())
+        evals, evecs = evals.cpu().numpy(), evecs.cpu().numpy()
+        bound = 4.5 * 8 * 4 * 2.0 ** -52
+        assert np.abs(evecs @ evecs.T - np.eye(n)).max() <= bound
+        assert np.abs(evecs @ a @ evecs.T - np.diag(evals)).max() <= bound * np.linalg.norm(a)
