@@ -349,6 +349,8 @@ tc_status tc_encode(tc_ctx *ctx, const tc_model *model, const tc_codebook *cb,
  * (about 0.5 MB on every GPU that loads the library, held until the process exits), and the
  * call runs no cudaMalloc, cudaFree or other allocating routine.
  *   - Same arguments, outputs, asynchrony and errors as tc_encode, minus the debug outputs.
+ *   - It runs on kernels that need no workspace: layers of more than 256 channels, unaligned maps and fp32
+ *     tensors of few tiles take two to three times as long as with tc_encode.
  *   - Tensors of more than TC_NOALLOC_MAX_TILES tiles of 128 pixels (N*H*W > 8 388 608
  *     pixels) are refused with TC_ERR_UNSUPPORTED; nothing is launched.
  *   - The first call on a device looks up the array's device address; make that first call

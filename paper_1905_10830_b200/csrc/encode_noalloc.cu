@@ -1,8 +1,8 @@
 // tc_encode_noalloc: tc_encode for callers that are not allowed to allocate device memory.
 //
 // tc_encode keeps the state of its cross-tile look-back (one 64-bit word per 128-pixel tile,
-// plus a ticket counter) in a scratch arena that the context grows with cudaMalloc when a
-// larger tensor arrives.  Some users of this library cannot accept that: a serving process
+// plus a ticket counter) and its workspaces in a scratch arena that the context grows with cudaMalloc when a
+// larger tensor or list arrives.  Some users of this library cannot accept that: a serving process
 // that reserves its whole memory budget at start-up and treats any later cudaMalloc as a bug;
 // a pipeline whose other streams must not be stalled by the device-wide synchronisation that
 // cudaMalloc / cudaFree imply; a plug-in running under a host application that owns the
@@ -76,8 +76,10 @@ extern "C" tc_status tc_encode_noalloc(tc_ctx *ctx, const tc_model *m, const tc_
     void *scratch = nullptr;
     if ((st = scratch_address(ctx->device, &scratch)) != TC_OK) return st;
     // The array still holds the previous call's tickets and tile states; the shared dispatch
-    // clears, on the stream, everything this call will read, then picks the same kernels as
-    // tc_encode (tensor-core kernels with the basis resident or streamed, fp32, fp64).
+    // clears, on the stream, everything this call will read, then picks among the kernels that need no
+    // workspace (tensor-core kernels with the basis resident or streamed, fp32, fp64): tc_encode's where
+    // it takes none either; on wide layers, unaligned maps and fp32 tensors of few tiles the fused ones, which
+    // take two to three times as long as its products and coder (960x7x7 x 128: 130 against 47 us).
     return tc_encode_with_scratch(ctx, m, cb, x, lay.chunk_pixels, lay.pixel_splits, stream_out, capacity, chunk_len, tile_off,
-                                  nullptr, scratch, /*no arena for symbols: the per-pixel exact kernels*/ nullptr, s);
+                                  nullptr, scratch, /*no workspace*/ nullptr, s);
 }

@@ -445,6 +445,18 @@ struct StagedReader {
     }
 };
 
+// The zero level in n coefficients from j on of the pixels px0, px0 + step, ... below px1 (a function of its own: nothing of it
+// in the registers of the tiles that decode).
+template <bool kOperand>
+__device__ __noinline__ void clear_rows(void *out, long long row0, int px0, int px1, int step, int k, int j, int n, int center)
+{
+    for (int px = px0; px < px1; px += step)
+        for (int i = j; i < j + n; ++i) {
+            if constexpr (kOperand) ((uint16_t *)out)[(row0 + px) * k + i] = 0;
+            else ((uint8_t *)out)[(row0 + px) * k + i] = (uint8_t)center;
+        }
+}
+
 // What bounds it: the chain length -> shift -> length of a chunk's symbols, with a handful of warps on
 // the chip (a 256x14x14 map has two tiles).  Per-layer tables are staged in shared memory; of
 // per-channel codes the bounds are (K x 48 bytes, read ahead of the symbol), and the symbols in code
@@ -503,16 +515,12 @@ __global__ void __launch_bounds__(kUnpackThreads) unpack_symbols_kernel(DecodeAr
     const bool tile_ok = (base & 127ull) == 0 && (end & 127ull) == 0 && base <= end && end <= a.stream_bits;
     // Rows that are not decoded hold the zero level (centred: 0; with kFull, whose lanes keep step, what zero bits
     // decode to), not what the workspace held before.
-    const long long row0 = (tile - first_tile) * TC_TILE_PIXELS;
-    auto clear = [&](int px, int j, int n) {                  // n coefficients from j on of a pixel of the tile
-        for (int i = j; i < j + n; ++i) {
-            if constexpr (kOperand) ((uint16_t *)out)[(row0 + px) * a.k + i] = 0;
-            else ((uint8_t *)out)[(row0 + px) * a.k + i] = (uint8_t)a.center;
-        }
+    auto clear = [&](int px0, int px1, int step, int j, int n) {       // n coefficients from j on of pixels of the tile
+        const int n_px = (int)min((long long)TC_TILE_PIXELS, a.pixels - tile * TC_TILE_PIXELS);
+        clear_rows<kOperand>(out, (tile - first_tile) * TC_TILE_PIXELS, px0, min(px1, n_px), step, a.k, j, n, a.center);
     };
-    const int n_px = (int)min((long long)TC_TILE_PIXELS, a.pixels - tile * TC_TILE_PIXELS);
     if (!tile_ok) {
-        for (int px = t; px < n_px; px += blockDim.x) clear(px, 0, a.k);
+        clear(t, TC_TILE_PIXELS, blockDim.x, 0, a.k);
         if (t == 0) tc_dev_set_status(a.status, TC_ERR_CORRUPT_STREAM);
         return;
     }
@@ -654,9 +662,8 @@ __global__ void __launch_bounds__(kUnpackThreads) unpack_symbols_kernel(DecodeAr
     };
     const bool walks = mine && !bad;
     if (!kFull && !walks) {
-        if (a.splits > 1) clear(t % TC_TILE_PIXELS, part * (a.k / a.splits), a.k / a.splits);
-        else
-            for (int px = t * a.chunk_pixels; px < min((t + 1) * a.chunk_pixels, n_px); ++px) clear(px, 0, a.k);
+        const int px = a.splits > 1 ? t % TC_TILE_PIXELS : t * a.chunk_pixels;
+        clear(px, px + a.chunk_pixels, 1, part * (a.k / a.splits), a.k / a.splits);
     } else if (staged) {
         StagedReader r;
         r.init(seg, walks ? off : 0u, walks ? seg + (uint32_t)((end - base) >> 3) : seg);
