@@ -60,7 +60,7 @@ struct tc_model {
     mutable std::vector<double> basis;      // [c][c], or empty
     std::vector<double> mean, eig;          // [c]
     std::vector<float> blk_bits, blk_odd;   // [(k + 15) / 16]  see finish_model
-    float max_bias = 0.f;                   // largest |d_enc_bias|, as a fraction of the quantiser's range
+    float max_bias = 0.f;                   // no |d_enc_bias| is larger, as a fraction of the quantiser's range
     int device = 0;
     // device copies, all but the first two (of a fitted model: owns64) inside one allocation
     void *d_block = nullptr;
