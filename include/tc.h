@@ -130,7 +130,7 @@ typedef struct {
                             a low-variance channel maps to a single value (Appendix E), with zero
                             between two levels it flips between both, which costs rate and
                             distortion.  0 keeps lo at the calibration minimum.                */
-    int32_t eigensolver; /* TC_EIG_DEVICE (0): one-sided Jacobi on the device, no C x C matrix
+    int32_t eigensolver; /* TC_EIG_DEVICE (0): solved on the device, no C x C matrix
                             crosses to the host during the fit.  TC_EIG_HOST (1): the
                             covariance is copied to the host and solved there (Householder
                             tridiagonalisation + implicit QR, tc_host_eigh).  Both return the
@@ -253,9 +253,10 @@ tc_status tc_host_huffman_lengths(const uint64_t *counts, int32_t nsym, int32_t 
 /* The fit's device eigensolver on its own (Section 3.1, "Linear transform": the PCA matrix is
  * the eigenvector matrix of the calibration covariance): `a` is a symmetric n x n matrix in DEVICE memory
  * (fp64, row-major, left untouched), evals [n] and evecs [n][n] DEVICE arrays, with the same
- * conventions as tc_host_eigh.  One-sided Jacobi in one cooperative launch;
- * synchronises the stream.  *sweeps (HOST, may be NULL) receives the number of sweeps.
- * Errors: INVALID_ARG, NOT_CONVERGED (150 sweeps), TIMEOUT, CUDA. */
+ * conventions as tc_host_eigh.  Up to 576 rows: Householder reduction and divide and conquer in thread-block
+ * clusters; beyond: one-sided Jacobi in one cooperative launch.  Synchronises the stream.  *sweeps (HOST, may be NULL)
+ * receives the number of passes: one and the levels of the division that coupled anything, or the sweeps.
+ * Errors: INVALID_ARG, NOT_CONVERGED (an element is not finite; 150 sweeps), TIMEOUT, CUDA. */
 tc_status tc_device_eigh(tc_ctx *ctx, const double *a, int32_t n, double *evals, double *evecs, int32_t *sweeps,
                          void *cuda_stream);
 /* Host eigensolver (TC_EIG_HOST): eigendecomposition of a symmetric n x n matrix `a`

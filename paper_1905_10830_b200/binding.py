@@ -404,7 +404,7 @@ def tc_host_huffman_lengths(counts: np.ndarray, max_length: int = 12) -> np.ndar
 
 
 def tc_device_eigh(ctx: Context, a: torch.Tensor):
-    """Eigenvalues (descending), eigenvectors (rows) and the number of Jacobi sweeps for a symmetric
+    """Eigenvalues (descending), eigenvectors (rows) and the solver's number of passes for a symmetric
     float64 CUDA matrix."""
     if a.dtype != torch.float64 or not a.is_cuda or a.dim() != 2 or a.shape[0] != a.shape[1]:
         raise ValueError("tc_device_eigh wants a square float64 CUDA tensor")

@@ -516,12 +516,12 @@ void tc_model_free(tc_model *m)
 }
 
 // Workspace of a fit in the context's arena (an allocation and its release cost about 0.1 ms each): mean and
-// covariance, then the eigensolver's, then eigenvalues, scale and the blocks' ranges of coefficient 0.
+// covariance, then the eigensolver's, then eigenvalues, its outcome, scale and the blocks' ranges of coefficient 0.
 static size_t fit_head_bytes(int c) { return (((size_t)c + (size_t)c * c) * sizeof(double) + 255) & ~(size_t)255; }
 static size_t fit_scratch_bytes(int c, long long range_pixels)
 {
     return fit_head_bytes(c) + ((tc_eigh_device_workspace_bytes(c) + 255) & ~(size_t)255) +
-           ((size_t)c + 1 + 2 * (size_t)tc_range0_max_blocks(range_pixels)) * sizeof(double);
+           ((size_t)c + 2 + 2 * (size_t)tc_range0_max_blocks(range_pixels)) * sizeof(double);
 }
 
 static tc_status finish_fit(tc_ctx *ctx, const tc_tensor *range_maps, const tc_fit_params *params, int k,
@@ -578,7 +578,7 @@ static tc_status finish_fit(tc_ctx *ctx, const tc_tensor *range_maps, const tc_f
     const long long m_samples = (long long)n * hw;
     const int range_blocks = tc_range0_max_blocks(m_samples);
     const size_t cc = (size_t)c * c;
-    // small: eigenvalues [c], scale [1], min / max per block [2 * range_blocks]
+    // small: eigenvalues [c], the solver's outcome [1], scale [1], min / max per block [2 * range_blocks]
     double *d_basis = nullptr, *d_mean_copy = nullptr;
     struct Free {
         double **a, **b;
@@ -590,7 +590,7 @@ static tc_status finish_fit(tc_ctx *ctx, const tc_tensor *range_maps, const tc_f
     double *const d_small = (double *)(rest + ((tc_eigh_device_workspace_bytes(c) + 255) & ~(size_t)255));
     TC_CUDA(cudaMalloc((void **)&d_basis, cc * sizeof(double)));
     TC_CUDA(cudaMalloc((void **)&d_mean_copy, (size_t)c * sizeof(double)));
-    double *d_eig = d_small, *d_scale = d_small + c, *d_minmax = d_scale + 1;
+    double *d_eig = d_small, *d_scale = d_small + c + 1, *d_minmax = d_scale + 1;
     TC_CUDA(cudaMemcpyAsync(d_mean_copy, d_mean, sizeof(double) * c, cudaMemcpyDeviceToDevice, s));
     tc_status st;
     if (params->eigensolver == TC_EIG_HOST) {
@@ -602,18 +602,19 @@ static tc_status finish_fit(tc_ctx *ctx, const tc_tensor *range_maps, const tc_f
         TC_CUDA(cudaMemcpyAsync(d_eig, eig.data(), sizeof(double) * c, cudaMemcpyHostToDevice, s));
         TC_CUDA(cudaStreamSynchronize(s));
     } else {
-        if ((st = tc_eigh_device(d_cov, c, d_eig, d_basis, d_work, nullptr, s)) != TC_OK) return st;
+        if ((st = tc_eigh_device(d_cov, c, d_eig, d_basis, d_work, s)) != TC_OK) return st;
     }
     if ((st = tc_launch_round_basis(d_basis, c, params->basis_dtype, d_scale, s)) != TC_OK) return st;
 
     int blocks = 0;
     st = tc_launch_range0(range_maps->data, range_maps->dtype, n, c, hw, d_mean_copy, d_basis, d_minmax, &blocks, s);
     if (st != TC_OK) return st;
-    std::vector<double> small((size_t)c + 1 + 2 * (size_t)blocks), mean(c);
+    std::vector<double> small((size_t)c + 2 + 2 * (size_t)blocks), mean(c);
     TC_CUDA(cudaMemcpyAsync(small.data(), d_small, sizeof(double) * small.size(), cudaMemcpyDeviceToHost, s));
     TC_CUDA(cudaMemcpyAsync(mean.data(), d_mean_copy, sizeof(double) * c, cudaMemcpyDeviceToHost, s));
     TC_CUDA(cudaStreamSynchronize(s));
-    const double *mm = small.data() + c + 1;
+    if (params->eigensolver == TC_EIG_DEVICE && (st = tc_eigh_outcome(small[c])) != TC_OK) return st;
+    const double *mm = small.data() + c + 2;
     double lo = INFINITY, hi = -INFINITY;
     for (int i = 0; i < blocks; ++i) { lo = std::min(lo, mm[2 * i]); hi = std::max(hi, mm[2 * i + 1]); }
     if (!(hi > lo)) return TC_ERR_INVALID_ARG;    // constant calibration data: no range to quantise
@@ -624,7 +625,7 @@ static tc_status finish_fit(tc_ctx *ctx, const tc_tensor *range_maps, const tc_f
     m->step = (hi - lo) / (double)((1 << params->bits) - 1);
     // zero_level: shift the grid so that y = 0 is a level (at most half a step; ties to even)
     m->lo = params->zero_level ? -m->step * std::nearbyint(-lo / m->step) : lo;
-    m->basis_scale = params->basis_dtype == TC_INT8 ? small[c] : 1.0;
+    m->basis_scale = params->basis_dtype == TC_INT8 ? small[c + 1] : 1.0;
     m->mean = mean;
     m->eig.assign(small.begin(), small.begin() + c);
     m->d_basis64 = d_basis; d_basis = nullptr;         // the model owns them from here
@@ -797,13 +798,20 @@ tc_status tc_device_eigh(tc_ctx *ctx, const double *a, int32_t n, double *evals,
     if (!ctx || !a || !evals || !evecs || n < 1 || n > TC_MAX_C) return TC_ERR_INVALID_ARG;
     DeviceGuard guard(ctx->device);
     cudaStream_t s = (cudaStream_t)cuda_stream;
-    void *work = nullptr;
-    TC_CUDA(cudaMalloc(&work, tc_eigh_device_workspace_bytes(n)));
-    int n_sweeps = 0;
-    const tc_status st = tc_eigh_device(a, n, evals, evecs, work, &n_sweeps, s);
-    cudaStreamSynchronize(s);
+    char *work = nullptr;                              // the solver's, then eigenvalues and outcome
+    const size_t bytes = (tc_eigh_device_workspace_bytes(n) + 255) & ~(size_t)255;
+    TC_CUDA(cudaMalloc((void **)&work, bytes + ((size_t)n + 1) * sizeof(double)));
+    double *const d_eig = (double *)(work + bytes);
+    double outcome = 0.0;
+    tc_status st = tc_eigh_device(a, n, d_eig, evecs, work, s);
+    if (st == TC_OK && (cudaMemcpyAsync(evals, d_eig, (size_t)n * sizeof(double), cudaMemcpyDeviceToDevice, s) != cudaSuccess ||
+                        cudaMemcpyAsync(&outcome, d_eig + n, sizeof(double), cudaMemcpyDeviceToHost, s) != cudaSuccess))
+        st = TC_ERR_CUDA;
+    if (cudaStreamSynchronize(s) != cudaSuccess && st == TC_OK) st = TC_ERR_CUDA;
     cudaFree(work);
-    if (sweeps) *sweeps = n_sweeps;
+    if (st == TC_ERR_CUDA) cudaGetLastError();
+    if (st == TC_OK) st = tc_eigh_outcome(outcome);
+    if (sweeps) *sweeps = outcome > 0.0 ? (int32_t)outcome : 0;
     return st;
 }
 

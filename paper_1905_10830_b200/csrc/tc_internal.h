@@ -257,7 +257,10 @@ tc_status tc_launch_moments_to_cov(const double *sum, const double *outer, long 
                                    cudaStream_t s);
 tc_status tc_launch_scale_mirror(double *cov, int c, double denom, cudaStream_t s);
 size_t tc_eigh_device_workspace_bytes(int c);
-tc_status tc_eigh_device(const double *a, int c, double *evals, double *evecs, void *work, int *sweeps_out, cudaStream_t s);
+tc_status tc_eigh_device(const double *a, int c, double *evals, double *evecs, void *work, cudaStream_t s);
+tc_status tc_eigh_outcome(double outcome);
+size_t tc_eigh_cluster_workspace_bytes(int n);   // eigh_cluster.cu
+tc_status tc_launch_eigh_cluster(const double *a, int n, void *work, double **vt, double **lambda, int **state, cudaStream_t s);
 tc_status tc_launch_round_basis(double *basis, int c, int dtype, double *scale_slot, cudaStream_t s);
 tc_status tc_launch_model_consts(const double *basis, const double *mean, int c, int k, double lo, double step, double center,
                                  float *enc_bias, float *tmu32, float *dec_bias, cudaStream_t s);

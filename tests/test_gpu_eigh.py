@@ -138,3 +138,53 @@ def test_rotations_are_orthogonal_to_fp64(ctx, n):
         bound = 4.5 * 8 * 4 * 2.0 ** -52
         assert np.abs(evecs @ evecs.T - np.eye(n)).max() <= bound
         assert np.abs(evecs @ a @ evecs.T - np.diag(evals)).max() <= bound * np.linalg.norm(a)
+
+
+# Edges of the cluster solver: lanes' elements and blocks of the cluster change at multiples of 64, groups of
+# eigenvectors at multiples of 16, halves of the division at powers of two; 576 rows are the last that fit, 577 take Jacobi.
+@pytest.mark.parametrize("n", [4, 5, 15, 16, 31, 32, 33, 63, 65, 127, 129, 191, 193, 257, 300, 384, 385, 320, 321, 512, 513, 575, 576, 577])
+def test_device_eigh_at_the_edges_of_its_kernels(ctx, n):
+    a, lam, _ = _sym(n, 4000 + n, 0.97)
+    a = (a + a.T) / 2
+    evals, evecs, sweeps = tc.tc_device_eigh(ctx, torch.from_numpy(a).cuda())
+    evals, evecs = evals.cpu().numpy(), evecs.cpu().numpy()
+    assert 1 <= sweeps <= 60
+    _check_conventions(a, evals, evecs)
+    assert np.abs(evals - np.linalg.eigvalsh(a)[::-1]).max() <= 1e-13 * max(1, n / 16) * lam.max()
+
+
+def _clustered(n):
+    q, _ = np.linalg.qr(np.random.default_rng(n).standard_normal((n, n)))
+    return (q * np.r_[np.ones(n // 2), 2 * np.ones(n // 3), np.arange(n - n // 2 - n // 3)]) @ q.T
+
+
+@pytest.mark.parametrize("a", [
+    np.ones((64, 64)),                                                                     # rank 1
+    np.diag(np.abs(np.arange(129) - 64.0)) + np.eye(129, k=1) + np.eye(129, k=-1),         # pairs that agree to rounding
+    2 * np.eye(200) - np.eye(200, k=1) - np.eye(200, k=-1),                                # equal halves at every cut
+    np.eye(100) + 1e-15 * (np.eye(100, k=1) + np.eye(100, k=-1)),                          # couplings at the rounding of the diagonal
+    np.diag(np.r_[np.zeros(70), np.arange(1.0, 31.0)]),                                    # diagonal, most of it zero
+    np.kron(np.eye(8), np.full((16, 16), 0.5)),                                            # uncoupled blocks
+    _clustered(150), np.zeros((40, 40)), 1e-200 * _clustered(70), 1e200 * _clustered(70),
+], ids=["ones", "wilkinson", "second difference", "tiny coupling", "diagonal", "blocks", "clusters", "zero", "small", "large"])
+def test_device_eigh_of_repeated_and_uncoupled_eigenvalues(ctx, a):
+    # Nothing is deflated: equal eigenvalues are set apart by one unit in the last place of |T| each, n of them by n / 2 eps |A| at
+    # a level, twice that over all levels (n, n / 2, ...); products and the reduction add a few sqrt(n) eps, n for good measure.
+    n = a.shape[0]
+    a = (a + a.T) / 2
+    evals, evecs, _ = tc.tc_device_eigh(ctx, torch.from_numpy(a).cuda())
+    evals, evecs = evals.cpu().numpy(), evecs.cpu().numpy()
+    norm = np.abs(np.linalg.eigvalsh(a)).max()
+    assert np.all(np.diff(evals) <= 0.0)
+    assert np.abs(evecs @ evecs.T - np.eye(n)).max() <= 2 * n * 2.0 ** -52
+    assert np.abs(evecs @ a @ evecs.T - np.diag(evals)).max() <= 4 * n * 2.0 ** -52 * norm
+    assert np.abs(evals - np.linalg.eigvalsh(a)[::-1]).max() <= 4 * n * 2.0 ** -52 * norm
+
+
+@pytest.mark.parametrize("n", [3, 100, 700])
+def test_device_eigh_refuses_what_is_not_finite(ctx, n):
+    for bad in (float("nan"), float("inf")):
+        a = torch.eye(n, dtype=torch.float64, device="cuda")
+        a[n - 1, n - 2] = a[n - 2, n - 1] = bad
+        with pytest.raises(tc.TcError):
+            tc.tc_device_eigh(ctx, a)
