@@ -317,4 +317,10 @@ struct WindowReaderT {
 };
 using WindowReader = WindowReaderT<false>;
 
+// c[8 x 8] += a[8 x 4] b[4 x 8]: a lane holds a[lane / 4][lane % 4], b[lane % 4][lane / 4] and c[lane / 4][2 (lane % 4) + 0, 1]
+__device__ __forceinline__ void mma_f64(double2 &c, double a, double b)
+{
+    asm("mma.sync.aligned.m8n8k4.row.col.f64.f64.f64.f64 {%0, %1}, {%2}, {%3}, {%0, %1};" : "+d"(c.x), "+d"(c.y) : "d"(a), "d"(b));
+}
+
 }  // namespace tcdev

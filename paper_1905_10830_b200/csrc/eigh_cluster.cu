@@ -6,11 +6,13 @@
 // Why this replaces the one-sided Jacobi method of eigh_device.cu wherever the matrix fits: Jacobi needs 13 to 28 sweeps
 // of n - 1 dependent rounds over all of the matrix; the reduction has n dependent steps in all, each a pass over what is
 // left of it, and dividing has log2(n) levels.
-#include "tc_internal.h"
+#include "device_utils.cuh"
 
 #include <cfloat>
 
 namespace {
+
+using tcdev::mma_f64;
 
 constexpr int kReduceWarps = 8, kReduceThreads = 32 * kReduceWarps;    // of a block that reduces: what every warp repeats costs issue slots
 constexpr int kWarps = 16, kThreads = 32 * kWarps;                      // of one that divides, or takes Rayleigh quotients
@@ -61,12 +63,6 @@ __device__ __forceinline__ uint32_t peer_address(const void *p, uint32_t rank)
     return out;
 }
 
-// c[8 x 8] += a[8 x 4] b[4 x 8]: a lane holds a[lane / 4][lane % 4], b[lane % 4][lane / 4] and c[lane / 4][2 (lane % 4) + 0, 1]
-__device__ __forceinline__ void mma_f64(double2 &c, double a, double b)
-{
-    asm("mma.sync.aligned.m8n8k4.row.col.f64.f64.f64.f64 {%0, %1}, {%2}, {%3}, {%0, %1};" : "+d"(c.x), "+d"(c.y) : "d"(a), "d"(b));
-}
-
 // 16 rows of `u` (shared memory, row pitch ld_u) times columns [col, col + 16) of `b` (global memory, row pitch ld_b),
 // terms [k0, k1) with k1 - k0 a multiple of 4; rows and columns of `b` past `last` read the last ones: `u` is zero there, and
 // so are its results' uses
@@ -75,16 +71,27 @@ __device__ __forceinline__ void tile_product(double2 (&acc)[2][2], const double 
 {
     const int lane = threadIdx.x & 31, lr = lane >> 2, lk = lane & 3;
     const double *left = b + min(col + lr, last), *right = b + min(col + lr + 8, last);
-#pragma unroll 8
-    for (int k = k0; k < k1; k += 4) {
-        const int row = k + lk;
-        const size_t at = (size_t)min(row, last) * ld_b;
-        const double a0 = u[lr * ld_u + row], a1 = u[(lr + 8) * ld_u + row];
-        const double b0 = __ldcg(left + at), b1 = __ldcg(right + at);
-        mma_f64(acc[0][0], a0, b0);
-        mma_f64(acc[0][1], a0, b1);
-        mma_f64(acc[1][0], a1, b0);
-        mma_f64(acc[1][1], a1, b1);
+    constexpr int kAhead = 8;                          // steps of four terms whose operands are on their way together
+#pragma unroll 1
+    for (int k = k0; k < k1; k += 4 * kAhead) {
+        double b0[kAhead], b1[kAhead];
+#pragma unroll
+        for (int i = 0; i < kAhead; ++i) {
+            const size_t at = (size_t)min(k + 4 * i + lk, last) * ld_b;
+            b0[i] = __ldcg(left + at); b1[i] = __ldcg(right + at);
+        }
+#pragma unroll
+        for (int i = 0; i < kAhead; ++i) asm volatile("" : "+d"(b0[i]), "+d"(b1[i]));       // (loads are not moved to their uses)
+#pragma unroll
+        for (int i = 0; i < kAhead; ++i) {
+            if (k + 4 * i >= k1) break;
+            const int row = k + 4 * i + lk;
+            const double a0 = u[lr * ld_u + row], a1 = u[(lr + 8) * ld_u + row];
+            mma_f64(acc[0][0], a0, b0[i]);
+            mma_f64(acc[0][1], a0, b1[i]);
+            mma_f64(acc[1][0], a1, b0[i]);
+            mma_f64(acc[1][1], a1, b1[i]);
+        }
     }
 }
 

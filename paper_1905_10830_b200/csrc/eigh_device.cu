@@ -407,23 +407,52 @@ __global__ void store_scale_kernel(double *abs_max) { *abs_max = __ddiv_rn(*abs_
 
 // The constants of a model from its basis and mean, in the summation order of a plain loop
 // (one thread per output, separate multiply and add):
-//   tmu[j] = sum_a T[j][a] mu[a], enc_bias[j] = -(tmu[j] + lo) / step,
-//   dec_bias[a] = mu[a] + (lo + center step) sum_{j<k} T[j][a]
-__global__ void model_consts_kernel(const double *basis, const double *mean, int c, int k, double lo, double step, double center,
-                                    float *enc_bias, float *tmu32, float *dec_bias)
+//   tmu[j] = sum_a T[j][a] mu[a], enc_bias[j] = -(tmu[j] + lo) / step      (blockIdx.y = 0)
+//   dec_bias[a] = mu[a] + (lo + center step) sum_{j<k} T[j][a]             (blockIdx.y = 1)
+// 32 outputs a block: all warps bring 64 terms of each through shared memory while the first adds up the 64 before.  With one thread
+// that read its own terms, the two sums one after the other: 38 us at 256 channels; 18.6 now.
+constexpr int kConstTerms = 64, kConstOutputs = 32;
+__global__ void __launch_bounds__(256) model_consts_kernel(const double *basis, const double *mean, int c, int k, double lo, double step, double center,
+                                                           float *enc_bias, float *tmu32, float *dec_bias)
 {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < k) {
-        double s = 0.0;
-        for (int a = 0; a < c; ++a) s = __dadd_rn(s, __dmul_rn(basis[(size_t)i * c + a], mean[a]));
-        enc_bias[i] = (float)__ddiv_rn(-__dadd_rn(s, lo), step);
-        tmu32[i] = (float)s;
+    __shared__ double s_terms[2][kConstTerms][kConstOutputs + 1];
+    const int first = blockIdx.x * kConstOutputs, t = threadIdx.x;
+    const bool rows = blockIdx.y == 0;                 // outputs are rows of the basis, terms run along them; else the columns
+    const int outputs = rows ? k : c, terms = rows ? c : k;
+    if (first >= outputs) return;
+    // element (term, output) that this thread brings, r = 0 .. 7; consecutive threads along a row of the basis
+    auto term_of = [&](int r) { return rows ? t % kConstTerms : t / kConstOutputs + 8 * r; };
+    auto output_of = [&](int r) { return rows ? t / kConstTerms + 4 * r : t % kConstOutputs; };
+    double got[8];
+    auto fetch = [&](int at) {
+#pragma unroll
+        for (int r = 0; r < 8; ++r) {
+            const int term = at + term_of(r), out = first + output_of(r);
+            got[r] = term < terms && out < outputs ? (rows ? basis[(size_t)out * c + term] : basis[(size_t)term * c + out]) : 0.0;
+        }
+    };
+    fetch(0);
+    double sum = 0.0;
+    for (int at = 0, buffer = 0; at < terms; at += kConstTerms, buffer ^= 1) {
+#pragma unroll
+        for (int r = 0; r < 8; ++r) s_terms[buffer][term_of(r)][output_of(r)] = got[r];
+        __syncthreads();                               // (the other buffer's sums are over: its reader has passed the barrier)
+        if (at + kConstTerms < terms) fetch(at + kConstTerms);
+        if (t < kConstOutputs) {
+            const int count = min(kConstTerms, terms - at);
+#pragma unroll 8
+            for (int i = 0; i < count; ++i) {
+                const double v = s_terms[buffer][i][t];
+                sum = __dadd_rn(sum, rows ? __dmul_rn(v, mean[at + i]) : v);
+            }
+        }
     }
-    if (i < c) {
-        double s = 0.0;
-        for (int j = 0; j < k; ++j) s = __dadd_rn(s, basis[(size_t)j * c + i]);
-        dec_bias[i] = (float)__dadd_rn(mean[i], __dmul_rn(__dadd_rn(lo, __dmul_rn(center, step)), s));
-    }
+    const int i = first + t;
+    if (t >= kConstOutputs || i >= outputs) return;
+    if (rows) {
+        enc_bias[i] = (float)__ddiv_rn(-__dadd_rn(sum, lo), step);
+        tmu32[i] = (float)sum;
+    } else dec_bias[i] = (float)__dadd_rn(mean[i], __dmul_rn(__dadd_rn(lo, __dmul_rn(center, step)), sum));
 }
 
 // bf16 operand copies: b[j][a], its transpose bt[a][j] and, unless null, bc: b in core matrices of 8 x 8
@@ -553,7 +582,7 @@ tc_status tc_launch_round_basis(double *basis, int c, int dtype, double *scale_s
 tc_status tc_launch_model_consts(const double *basis, const double *mean, int c, int k, double lo, double step, double center,
                                  float *enc_bias, float *tmu32, float *dec_bias, cudaStream_t s)
 {
-    model_consts_kernel<<<(c + 127) / 128, 128, 0, s>>>(basis, mean, c, k, lo, step, center, enc_bias, tmu32, dec_bias);
+    model_consts_kernel<<<dim3((unsigned)((c + kConstOutputs - 1) / kConstOutputs), 2), 256, 0, s>>>(basis, mean, c, k, lo, step, center, enc_bias, tmu32, dec_bias);
     return cudaGetLastError() == cudaSuccess ? TC_OK : TC_ERR_CUDA;
 }
 

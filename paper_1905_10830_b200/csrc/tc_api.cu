@@ -555,11 +555,7 @@ tc_status tc_fit_pca(tc_ctx *ctx, const tc_tensor *calib, const tc_fit_params *p
 
     st = tc_launch_channel_sums(calib->data, calib->dtype, n, c, hw, d_mean, s);
     if (st != TC_OK) return st;
-    std::vector<double> mean(c);
-    TC_CUDA(cudaMemcpyAsync(mean.data(), d_mean, sizeof(double) * c, cudaMemcpyDeviceToHost, s));
-    TC_CUDA(cudaStreamSynchronize(s));
-    for (double &v : mean) v /= (double)m_samples;
-    TC_CUDA(cudaMemcpyAsync(d_mean, mean.data(), sizeof(double) * c, cudaMemcpyHostToDevice, s));
+    if ((st = tc_launch_mean(d_mean, c, m_samples, s)) != TC_OK) return st;
     st = tc_launch_covariance(calib->data, calib->dtype, n, c, hw, d_mean, d_cov, ctx->sm_count, s);
     if (st != TC_OK) return st;
     // centred sums in the upper triangle -> covariance, full symmetric, still on the device

@@ -236,6 +236,7 @@ size_t tc_decode_wide_staging_bytes(const tc_ctx *ctx, const DecodeArgs &a);   /
 
 tc_status tc_launch_channel_sums(const void *x, int dtype, int n, int c, int hw, double *sums,
                                  cudaStream_t s);
+tc_status tc_launch_mean(double *sums, int c, long long pixels, cudaStream_t s);      // in place
 tc_status tc_launch_covariance(const void *x, int dtype, int n, int c, int hw, const double *mean,
                                double *cov, int sm_count, cudaStream_t s);
 tc_status tc_launch_range0(const void *x, int dtype, int n, int c, int hw, const double *mean,
