@@ -382,12 +382,14 @@ tc_status tc_decode(tc_ctx *ctx, const tc_model *model, const tc_codebook *cb, c
  * layers at a small batch are each too small to fill the GPU, and a call per layer pays the
  * launch and set-up time of its kernels one after the other.  These entry points take the
  * whole list: the items are checked first (nothing is launched if one is invalid), the
- * bookkeeping of all of them is cleared at once, and their kernels are spread, largest first,
- * over eight streams of the context so that small layers run beside one another; `cuda_stream`
+ * bookkeeping of all of them is cleared at once, and tensors that take the same kernel share its
+ * launch, each with blocks of its own; those whose route has several kernels are spread, largest
+ * first, over eight streams of the context.  `cuda_stream`
  * waits for all of them, so later work on it sees every output.  The results are those of
  * tc_encode / tc_decode called per item (same arguments, same errors; the first error is
  * returned after all items that could be launched have been).  Output buffers of different
- * items must not overlap.  tc_last_path reports the route of the item launched last. */
+ * items must not overlap.  tc_last_path reports the route of the item launched last (items that
+ * share launches come first). */
 typedef struct {
     const tc_model *model;
     const tc_codebook *codebook;

@@ -910,19 +910,13 @@ static size_t encode_work_bytes(const tc_ctx *ctx, const tc_model *m, const tc_t
     return n_tiles < (long long)kExactParallelTilesPerSm * ctx->sm_count ? (((size_t)pixels * m->k + 255) & ~(size_t)255) : 0;
 }
 
-// Argument block and kernel choice shared by tc_encode and tc_encode_noalloc.  `scratch` is
-// kEncodeScratchHeader bytes (ticket counter) followed by one 64-bit look-back word per tile;
-// it is cleared on the stream here, whoever owns it: by the kernel that precedes the entropy coder where
-// there is one (a memset of its own costs the stream two microseconds).
-tc_status tc_encode_with_scratch(tc_ctx *ctx, const tc_model *m, const tc_codebook *cb, const tc_tensor *x, int chunk_pixels,
-                                 int splits, void *stream_out, size_t capacity, uint16_t *chunk_len, uint64_t *tile_off,
-                                 const tc_debug_out *debug, void *scratch, void *work, cudaStream_t s,
-                                 unsigned long long *hist, unsigned long long *clamped, int list_sms)
+// Argument block of an encode.
+static EncodeArgs encode_args(const tc_ctx *ctx, const tc_model *m, const tc_codebook *cb, const tc_tensor *x, int chunk_pixels,
+                              int splits, void *stream_out, size_t capacity, uint16_t *chunk_len, uint64_t *tile_off,
+                              const tc_debug_out *debug, void *scratch, unsigned long long *hist, unsigned long long *clamped, int list_sms)
 {
     const long long pixels = (long long)x->n * x->h * x->w;
     const long long n_tiles = (pixels + TC_TILE_PIXELS - 1) / TC_TILE_PIXELS;
-    const bool scratch_is_zero = list_sms != 0;
-    const size_t scratch_bytes = kEncodeScratchHeader + (size_t)n_tiles * sizeof(unsigned long long);
     EncodeArgs a{};
     a.x = x->data; a.n = x->n; a.c = x->c; a.hw = x->h * x->w; a.k = m->k; a.bits = m->bits; a.groups = cb->groups;
     a.pixels = pixels; a.n_tiles = n_tiles; a.chunk_pixels = chunk_pixels; a.splits = splits;
@@ -943,9 +937,31 @@ tc_status tc_encode_with_scratch(tc_ctx *ctx, const tc_model *m, const tc_codebo
     a.modal = cb->modal;
     a.max_bias = m->max_bias;
     a.blk_bits = m->blk_bits.data(); a.blk_odd = m->blk_odd.data();
-    if (hist && !((ctx->force_exact == 0 || ctx->force_exact == 3) && x->dtype == TC_BF16 && tc_encode_tc_supported(ctx, a)))
-        return TC_ERR_UNSUPPORTED;                      // only the resident-basis tensor-core encoder counts symbols
-    if ((ctx->force_exact == 0 || ctx->force_exact == 3) && x->dtype == TC_BF16 && tc_encode_tc_supported(ctx, a)) {
+    return a;
+}
+
+// bf16 tensors that the resident-basis encoder takes.
+static bool resident_encode(const tc_ctx *ctx, const tc_tensor *x, const EncodeArgs &a)
+{
+    return (ctx->force_exact == 0 || ctx->force_exact == 3) && x->dtype == TC_BF16 && tc_encode_tc_supported(ctx, a);
+}
+
+// Kernel choice shared by tc_encode and tc_encode_noalloc.  `scratch` is
+// kEncodeScratchHeader bytes (ticket counter) followed by one 64-bit look-back word per tile;
+// it is cleared on the stream here, whoever owns it: by the kernel that precedes the entropy coder where
+// there is one (a memset of its own costs the stream two microseconds).
+tc_status tc_encode_with_scratch(tc_ctx *ctx, const tc_model *m, const tc_codebook *cb, const tc_tensor *x, int chunk_pixels,
+                                 int splits, void *stream_out, size_t capacity, uint16_t *chunk_len, uint64_t *tile_off,
+                                 const tc_debug_out *debug, void *scratch, void *work, cudaStream_t s,
+                                 unsigned long long *hist, unsigned long long *clamped, int list_sms)
+{
+    EncodeArgs a = encode_args(ctx, m, cb, x, chunk_pixels, splits, stream_out, capacity, chunk_len, tile_off, debug, scratch, hist, clamped, list_sms);
+    const long long n_tiles = a.n_tiles;
+    const bool scratch_is_zero = list_sms != 0;
+    const size_t scratch_bytes = kEncodeScratchHeader + (size_t)n_tiles * sizeof(unsigned long long);
+    const bool resident = resident_encode(ctx, x, a);
+    if (hist && !resident) return TC_ERR_UNSUPPORTED;   // only the resident-basis tensor-core encoder counts symbols
+    if (resident) {
         ctx->last_encode_path = 1;
         if (!scratch_is_zero) TC_CUDA(cudaMemsetAsync(scratch, 0, scratch_bytes, s));
         return tc_launch_encode_tc(ctx, a, s);
@@ -1061,21 +1077,12 @@ static size_t decode_scratch_bytes(const tc_ctx *ctx, const tc_model *m, const t
     return n_tiles < (long long)kExactParallelTilesPerSm * ctx->sm_count ? (((size_t)pixels * m->k + 255) & ~(size_t)255) : 0;
 }
 
-// tc_decode with the symbol scratch named by the caller (decode_scratch_bytes of it, or nullptr)
-static tc_status decode_with_scratch(tc_ctx *ctx, const tc_model *m, const tc_codebook *cb, const void *stream, size_t stream_bytes,
-                                     const uint16_t *chunk_len, const uint64_t *tile_off, const tc_encode_params *params,
-                                     const tc_tensor *x_hat, uint8_t *sym_scratch, int list_sms, void *cuda_stream)
+// Argument block of a decode.
+static DecodeArgs decode_args(const tc_ctx *ctx, const tc_model *m, const tc_codebook *cb, const void *stream, size_t stream_bytes,
+                              const uint16_t *chunk_len, const uint64_t *tile_off, const tc_encode_params *params, const ChunkShape &cs,
+                              const tc_tensor *x_hat, int list_sms)
 {
-    if (!ctx) return TC_ERR_INVALID_ARG;
-    tc_status st = check_codec_args(m, cb, x_hat);
-    if (st != TC_OK) return st;
-    ChunkShape cs;
-    if (!resolve_chunks(params, m->k, cb->max_len, &cs)) return TC_ERR_INVALID_ARG;
     const long long pixels = (long long)x_hat->n * x_hat->h * x_hat->w;
-    if (pixels == 0) return TC_OK;
-    if (!stream || !chunk_len || !tile_off || ((uintptr_t)stream & 15u) != 0 || ((uintptr_t)chunk_len & 3u) != 0)
-        return TC_ERR_INVALID_ARG;
-    DeviceGuard guard(ctx->device);
     DecodeArgs a{};
     a.stream = (const uint32_t *)stream; a.stream_bits = (unsigned long long)(stream_bytes & ~(size_t)3) * 8ull;
     a.chunk_len = chunk_len; a.splits = cs.splits; a.tile_off = (const unsigned long long *)tile_off; a.symbols = nullptr;
@@ -1098,8 +1105,32 @@ static tc_status decode_with_scratch(tc_ctx *ctx, const tc_model *m, const tc_co
     a.dense_head = 0;
     while (a.dense_head < m->k && a.dense_head < (int)m->eig.size() && std::sqrt(std::max(0.0, m->eig[a.dense_head])) > 0.45 * m->step)
         ++a.dense_head;
-    // per-layer code table, up to 256 channels: the run-skipping decoder (it also takes dense tiles)
-    if (ctx->force_exact == 0 && x_hat->dtype == TC_BF16 && tc_decode_runs_supported(ctx, a)) {
+    return a;
+}
+
+// bf16 tensors that the run-skipping decoder takes: per-layer code table, up to 256 channels.
+static bool runs_decode(const tc_ctx *ctx, const tc_tensor *x_hat, const DecodeArgs &a)
+{
+    return ctx->force_exact == 0 && x_hat->dtype == TC_BF16 && tc_decode_runs_supported(ctx, a);
+}
+
+// tc_decode with the symbol scratch named by the caller (decode_scratch_bytes of it, or nullptr)
+static tc_status decode_with_scratch(tc_ctx *ctx, const tc_model *m, const tc_codebook *cb, const void *stream, size_t stream_bytes,
+                                     const uint16_t *chunk_len, const uint64_t *tile_off, const tc_encode_params *params,
+                                     const tc_tensor *x_hat, uint8_t *sym_scratch, int list_sms, void *cuda_stream)
+{
+    if (!ctx) return TC_ERR_INVALID_ARG;
+    tc_status st = check_codec_args(m, cb, x_hat);
+    if (st != TC_OK) return st;
+    ChunkShape cs;
+    if (!resolve_chunks(params, m->k, cb->max_len, &cs)) return TC_ERR_INVALID_ARG;
+    const long long pixels = (long long)x_hat->n * x_hat->h * x_hat->w;
+    if (pixels == 0) return TC_OK;
+    if (!stream || !chunk_len || !tile_off || ((uintptr_t)stream & 15u) != 0 || ((uintptr_t)chunk_len & 3u) != 0)
+        return TC_ERR_INVALID_ARG;
+    DeviceGuard guard(ctx->device);
+    const DecodeArgs a = decode_args(ctx, m, cb, stream, stream_bytes, chunk_len, tile_off, params, cs, x_hat, list_sms);
+    if (runs_decode(ctx, x_hat, a)) {                   // (it also takes dense tiles)
         ctx->last_decode_path = 1;
         return tc_launch_decode_runs(ctx, a, (cudaStream_t)cuda_stream);
     }
@@ -1164,19 +1195,99 @@ static tc_status ensure_many_streams(tc_ctx *ctx)
     return TC_OK;
 }
 
-// SMs that the persistent kernels of tensor i of a list take: a quarter of them, more where the tensor is more than that
-// of the list's work.  A kernel's first tile costs a block 10 to 15 us (basis, tensor memory, first copies) and a further one
-// 2 to 4, so a grid over all SMs with a tile or two for each block spends the chip on set-up; the other streams'
-// kernels fill the rest.  16 layers of a residual network, four streams: encode 257 us on all SMs, 206 on half, 205 on a
-// quarter, 224 on 28; decode 252, 212, 202, 238; eight streams on a quarter: 201 and 179.
-static int list_share(int sm_count, int n_streams, const std::vector<double> &work, int i)
+}  // extern "C"
+
+void deal_blocks(std::vector<ListWork> &work, int sms)
 {
-    double total = 0.0;
-    for (double w : work) total += w;
-    const int least = sm_count / std::min(4, n_streams);
-    return total > 0.0 ? std::min(sm_count, std::max(least, (int)std::ceil(sm_count * work[i] / total))) : least;
+    // shortest time for which the blocks that the tensors then need are there; less than a tile's is not to be had
+    double least = 0.0, most = 0.0;
+    for (const ListWork &w : work) { least = std::max(least, w.tile_us); most = std::max(most, w.tile_us * (double)w.tiles); }
+    auto blocks_for = [](const ListWork &w, double us) {
+        const long long each = std::max(1ll, (long long)(us / w.tile_us));
+        return (int)std::min((w.tiles + each - 1) / each, 1ll << 20);
+    };
+    auto fits = [&](double us) {
+        long long sum = 0;
+        for (const ListWork &w : work) sum += blocks_for(w, us);
+        return sum <= sms;
+    };
+    if (!fits(least)) {
+        for (int i = 0; i < 24; ++i) {
+            const double us = 0.5 * (least + most);
+            if (fits(us)) most = us; else least = us;
+        }
+        least = most * (1.0 + 1e-9);                   // (`most` fits: one block each, for as many tensors as blocks)
+    }
+    for (ListWork &w : work) w.blocks = std::max(1, blocks_for(w, least));
 }
 
+// SMs for the tensors of a list that share a launch (`shared_us`: the work of all, in us of one SM), beside `others_us` of tensors with
+// kernels of their own: by their shares, at least eight for the others.
+static int shared_sms(int sm_count, double shared_us, double others_us)
+{
+    if (others_us <= 0.0) return sm_count;
+    return std::max(sm_count / 4, std::min(sm_count - 8, (int)(sm_count * shared_us / (shared_us + others_us))));
+}
+
+// us of one SM that a wide tensor takes, entropy coder and product (25 tiles of 512 channels at 4 bits: 960 to encode, 885 to decode).
+static double wide_us(long long pixels, int k) { return 0.075 * k * (double)((pixels + TC_TILE_PIXELS - 1) / TC_TILE_PIXELS); }
+
+// SMs that the persistent kernels of tensor i of those take that have launches of their own: a quarter of them, more where the tensor
+// is more than that of the list's work.  A kernel's first tile costs a block 10 to 15 us (basis, tensor memory, first copies) and a
+// further one 2 to 4, so a grid over all SMs with a tile or two for each block spends the chip on set-up; the other streams'
+// kernels fill the rest.
+static int list_share(int sm_count, int n_streams, double all, double mine)
+{
+    const int least = sm_count / std::min(4, n_streams);
+    return all > 0.0 ? std::min(sm_count, std::max(least, (int)std::ceil(sm_count * mine / all))) : least;
+}
+
+// The streams of a list beside the caller's: they start where it stands and it waits for them.
+struct ListStreams {
+    tc_ctx *ctx;
+    cudaStream_t s;
+    int used = 0;
+    tc_status fork(int n)
+    {
+        if (n == 0) return TC_OK;
+        const tc_status st = ensure_many_streams(ctx);
+        if (st != TC_OK) return st;
+        TC_CUDA(cudaEventRecord(ctx->many_fork, s));
+        for (int j = 0; j < n; ++j) TC_CUDA(cudaStreamWaitEvent(ctx->many_streams[j], ctx->many_fork, 0));
+        used = n;
+        return TC_OK;
+    }
+    tc_status join()
+    {
+        for (int j = 0; j < used; ++j) {
+            TC_CUDA(cudaEventRecord(ctx->many_join[j], ctx->many_streams[j]));
+            TC_CUDA(cudaStreamWaitEvent(s, ctx->many_join[j], 0));
+        }
+        return TC_OK;
+    }
+};
+
+// Tensors that share launches, by kernel: each kernel gets SMs by its share of the work.  The first runs on the caller's stream, the
+// others on the list's `n_streams` streams from `first_stream` on.
+template <typename Args, typename Launch>
+static tc_status launch_shared(tc_ctx *ctx, const std::vector<std::vector<Args>> &classes, const std::vector<double> &us, int sms,
+                               cudaStream_t s, int first_stream, int n_streams, Launch launch)
+{
+    double all = 0.0;
+    for (double u : us) all += u;
+    tc_status first_error = TC_OK;
+    int on = 0;
+    for (size_t j = 0; j < classes.size(); ++j) {
+        if (classes[j].empty()) continue;
+        const int mine = std::min(sms, std::max(1, (int)(sms * us[j] / all)));
+        const tc_status st = launch(classes[j], mine, on == 0 ? s : ctx->many_streams[(first_stream + on - 1) % n_streams]);
+        if (st != TC_OK && first_error == TC_OK) first_error = st;
+        ++on;
+    }
+    return first_error;
+}
+
+extern "C" {
 
 // Items in descending order of work: the large ones start first, each on its own stream.
 static std::vector<int> by_descending_work(int n, const std::vector<double> &work)
@@ -1227,34 +1338,63 @@ tc_status tc_encode_many(tc_ctx *ctx, const tc_encode_item *items, int32_t n_ite
         lookback_total += (kEncodeScratchHeader + (size_t)n_tiles * sizeof(unsigned long long) + 255) & ~(size_t)255;
         work[i] = (double)pixels * it.x->c;
     }
-    const int n_streams = std::min(kManyStreams, (int)n_items);
-    const std::vector<int> order = by_descending_work(n_items, work);
-    for (int i = 0; i < n_items; ++i) symbols_bytes[i] = work[i] > 0.0 ? encode_work_bytes(ctx, items[i].model, items[i].x) : 0;
-    tc_status st = ensure_many_streams(ctx);
-    if (st != TC_OK) return st;
+    // the resident-basis encoder takes its tensors in a launch per kernel, the others have kernels of their own
+    std::vector<EncodeArgs> args(n_items);
+    std::vector<int> kind(n_items, -1);
+    std::vector<std::vector<EncodeArgs>> classes(8);
+    std::vector<double> class_us(8, 0.0);
+    double shared_us = 0.0, others_us = 0.0, others = 0.0;
+    std::vector<int> order;
+    for (int i : by_descending_work(n_items, work)) {
+        const tc_encode_item &it = items[i];
+        if (work[i] > 0.0) {
+            args[i] = encode_args(ctx, it.model, it.codebook, it.x, shape[i].cp, shape[i].splits, it.stream_out, it.capacity, it.chunk_len,
+                                  it.tile_off, nullptr, nullptr, nullptr, nullptr, 0);
+            if (resident_encode(ctx, it.x, args[i])) kind[i] = tc_encode_tc_class(ctx, args[i]);
+        }
+        if (kind[i] >= 0) {
+            const double us = (double)args[i].n_tiles * tc_encode_tc_tile_us(args[i]);
+            class_us[kind[i]] += us;
+            shared_us += us;
+        } else {
+            order.push_back(i);
+            others += work[i];
+            others_us += wide_us((long long)it.x->n * it.x->h * it.x->w, it.model->k);
+            symbols_bytes[i] = work[i] > 0.0 ? encode_work_bytes(ctx, it.model, it.x) : 0;
+        }
+    }
+    const int n_streams = std::min(kManyStreams, (int)order.size());
+    tc_status st;
     CallScratch scratch;
     if ((st = call_scratch(ctx, lookback_total, stream_workspaces(order, n_streams, symbols_bytes, lookback_total, symbols_at), s, &scratch)) != TC_OK) return st;
+    for (int i = 0; i < n_items; ++i)
+        if (kind[i] >= 0) {
+            args[i].ticket = (unsigned int *)(scratch.at + lookback_at[i]);
+            args[i].tile_state = (unsigned long long *)(scratch.at + lookback_at[i] + kEncodeScratchHeader);
+            classes[kind[i]].push_back(args[i]);
+        }
+    const int n_classes = (int)std::count_if(classes.begin(), classes.end(), [](const auto &c) { return !c.empty(); });
+    const int sms = shared_sms(ctx->sm_count, shared_us, others_us);
     // one clear for the look-back state of all items, then the items fan out over the streams
     TC_CUDA(cudaMemsetAsync(scratch.at, 0, lookback_total, s));
-    TC_CUDA(cudaEventRecord(ctx->many_fork, s));
-    for (int j = 0; j < n_streams; ++j) TC_CUDA(cudaStreamWaitEvent(ctx->many_streams[j], ctx->many_fork, 0));
-    tc_status first_error = TC_OK;
-    for (int r = 0; r < n_items; ++r) {
+    ListStreams streams{ctx, s};
+    if ((st = streams.fork(std::min(kManyStreams, n_streams + std::max(0, n_classes - 1)))) != TC_OK) return st;
+    tc_status first_error = launch_shared(ctx, classes, class_us, sms, s, n_streams, streams.used, [&](const std::vector<EncodeArgs> &c, int mine, cudaStream_t on) {
+        return tc_launch_encode_tc_list(ctx, c, mine, on);
+    });
+    for (size_t r = 0; r < order.size(); ++r) {
         const int i = order[r];
         const tc_encode_item &it = items[i];
         cudaStream_t ws = ctx->many_streams[r % n_streams];
-        const int list_sms = list_share(ctx->sm_count, n_streams, work, i);
-        const long long pixels = (long long)it.x->n * it.x->h * it.x->w;
-        if (pixels == 0) { if (cudaMemsetAsync(it.tile_off, 0, sizeof(uint64_t), ws) != cudaSuccess && first_error == TC_OK) first_error = TC_ERR_CUDA; continue; }
+        const int list_sms = n_classes ? ctx->sm_count - sms : list_share(ctx->sm_count, n_streams, others, work[i]);
+        if (work[i] == 0.0) { if (cudaMemsetAsync(it.tile_off, 0, sizeof(uint64_t), ws) != cudaSuccess && first_error == TC_OK) first_error = TC_ERR_CUDA; continue; }
         st = tc_encode_with_scratch(ctx, it.model, it.codebook, it.x, shape[i].cp, shape[i].splits, it.stream_out, it.capacity,
                                     it.chunk_len, it.tile_off, nullptr, scratch.at + lookback_at[i],
                                     symbols_bytes[i] && scratch.whole ? scratch.at + symbols_at[i] : nullptr, ws, nullptr, nullptr, list_sms);
         if (st != TC_OK && first_error == TC_OK) first_error = st;
     }
-    for (int j = 0; j < n_streams; ++j) {
-        TC_CUDA(cudaEventRecord(ctx->many_join[j], ctx->many_streams[j]));
-        TC_CUDA(cudaStreamWaitEvent(s, ctx->many_join[j], 0));
-    }
+    if (order.empty()) ctx->last_encode_path = 1;
+    if ((st = streams.join()) != TC_OK) return st;
     return first_error;
 }
 
@@ -1279,28 +1419,49 @@ tc_status tc_decode_many(tc_ctx *ctx, const tc_decode_item *items, int32_t n_ite
         symbols_bytes[i] = decode_scratch_bytes(ctx, it.model, it.codebook, it.x_hat);
         work[i] = (double)pixels * it.x_hat->c;
     }
+    std::vector<std::vector<DecodeArgs>> classes(2);    // without and with a non-linearity behind the decoder
+    std::vector<double> class_us(2, 0.0);
+    double shared_us = 0.0, others_us = 0.0, others = 0.0;
+    std::vector<int> order;
+    for (int i : by_descending_work(n_items, work)) {
+        const tc_decode_item &it = items[i];
+        if (work[i] == 0.0) continue;
+        ChunkShape cs;
+        resolve_chunks(it.params, it.model->k, it.codebook->max_len, &cs);
+        const DecodeArgs a = decode_args(ctx, it.model, it.codebook, it.stream, it.stream_bytes, it.chunk_len, it.tile_off, it.params, cs, it.x_hat, 0);
+        if (runs_decode(ctx, it.x_hat, a)) {
+            const double us = (double)a.n_tiles * tc_decode_runs_tile_us(a);
+            classes[a.relu].push_back(a);
+            class_us[a.relu] += us;
+            shared_us += us;
+            symbols_bytes[i] = 0;
+        } else {
+            order.push_back(i);
+            others += work[i];
+            others_us += wide_us(a.pixels, a.k);
+        }
+    }
     tc_status st;
-    const int n_streams = std::min(kManyStreams, (int)n_items);
-    const std::vector<int> order = by_descending_work(n_items, work);
-    if ((st = ensure_many_streams(ctx)) != TC_OK) return st;
+    const int n_streams = std::min(kManyStreams, (int)order.size()), n_classes = (int)!classes[0].empty() + (int)!classes[1].empty();
     CallScratch scratch;
     if ((st = call_scratch(ctx, 0, stream_workspaces(order, n_streams, symbols_bytes, 0, symbols_at), s, &scratch)) != TC_OK) return st;
-    TC_CUDA(cudaEventRecord(ctx->many_fork, s));
-    for (int j = 0; j < n_streams; ++j) TC_CUDA(cudaStreamWaitEvent(ctx->many_streams[j], ctx->many_fork, 0));
-    tc_status first_error = TC_OK;
-    for (int r = 0; r < n_items; ++r) {
+    const int sms = shared_sms(ctx->sm_count, shared_us, others_us);
+    ListStreams streams{ctx, s};
+    if ((st = streams.fork(std::min(kManyStreams, n_streams + std::max(0, n_classes - 1)))) != TC_OK) return st;
+    tc_status first_error = launch_shared(ctx, classes, class_us, sms, s, n_streams, streams.used, [&](const std::vector<DecodeArgs> &c, int mine, cudaStream_t on) {
+        return tc_launch_decode_runs_list(ctx, c, mine, on);
+    });
+    for (size_t r = 0; r < order.size(); ++r) {
         const int i = order[r];
         const tc_decode_item &it = items[i];
-        const int list_sms = list_share(ctx->sm_count, n_streams, work, i);
+        const int list_sms = n_classes ? ctx->sm_count - sms : list_share(ctx->sm_count, n_streams, others, work[i]);
         st = decode_with_scratch(ctx, it.model, it.codebook, it.stream, it.stream_bytes, it.chunk_len, it.tile_off, it.params,
                                  it.x_hat, symbols_bytes[i] && scratch.at ? (uint8_t *)scratch.at + symbols_at[i] : nullptr,
                                  list_sms, ctx->many_streams[r % n_streams]);
         if (st != TC_OK && first_error == TC_OK) first_error = st;
     }
-    for (int j = 0; j < n_streams; ++j) {
-        TC_CUDA(cudaEventRecord(ctx->many_join[j], ctx->many_streams[j]));
-        TC_CUDA(cudaStreamWaitEvent(s, ctx->many_join[j], 0));
-    }
+    if (order.empty() && n_classes) ctx->last_decode_path = 1;
+    if ((st = streams.join()) != TC_OK) return st;
     return first_error;
 }
 

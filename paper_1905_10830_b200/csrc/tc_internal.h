@@ -192,6 +192,16 @@ inline cudaError_t launch_chained(bool early, void (*kernel)(P...), dim3 grid, d
     return err;
 }
 
+// ---- several tensors in one launch of a persistent kernel ------------------------------------
+constexpr int kListItems = 32;                // tensors of a launch (their arguments are kernel parameters)
+struct ListWork {
+    long long tiles;
+    double tile_us;                           // what a tile takes a block, after its first
+    int blocks;
+};
+// Deals `sms` blocks (at least one for each tensor) so that the slowest block is done as early as possible.
+void deal_blocks(std::vector<ListWork> &work, int sms);
+
 constexpr size_t kEncodeScratchHeader = 64;   // ticket counter, padded; the per-tile look-back words follow
 tc_status tc_encode_with_scratch(tc_ctx *ctx, const tc_model *m, const tc_codebook *cb, const tc_tensor *x, int chunk_pixels,
                                  int splits, void *stream_out, size_t capacity, uint16_t *chunk_len, uint64_t *tile_off,
@@ -223,10 +233,15 @@ bool tc_tensor_map_sw128(CUtensorMap *map, const void *base, long long rows, int
 tc_status tc_launch_reconstruct(const DecodeArgs &a, int dtype, const uint8_t *sym, cudaStream_t s);
 bool tc_encode_tc_supported(const tc_ctx *ctx, const EncodeArgs &a);
 tc_status tc_launch_encode_tc(const tc_ctx *ctx, const EncodeArgs &a, cudaStream_t s);
+int tc_encode_tc_class(const tc_ctx *ctx, const EncodeArgs &a);
+double tc_encode_tc_tile_us(const EncodeArgs &a);
+tc_status tc_launch_encode_tc_list(const tc_ctx *ctx, const std::vector<EncodeArgs> &tensors, int sms, cudaStream_t s);
 bool tc_decode_tc_supported(const tc_ctx *ctx, const DecodeArgs &a);
 tc_status tc_launch_decode_tc(const tc_ctx *ctx, const DecodeArgs &a, cudaStream_t s);
 bool tc_decode_runs_supported(const tc_ctx *ctx, const DecodeArgs &a);
 tc_status tc_launch_decode_runs(const tc_ctx *ctx, const DecodeArgs &a, cudaStream_t s);
+double tc_decode_runs_tile_us(const DecodeArgs &a);
+tc_status tc_launch_decode_runs_list(const tc_ctx *ctx, const std::vector<DecodeArgs> &tensors, int sms, cudaStream_t s);
 bool tc_encode_wide_supported(const tc_ctx *ctx, const EncodeArgs &a);
 tc_status tc_launch_encode_wide(const tc_ctx *ctx, const EncodeArgs &a, cudaStream_t s);
 bool tc_decode_wide_supported(const tc_ctx *ctx, const DecodeArgs &a);

@@ -145,3 +145,33 @@ def test_tensors_that_share_a_stream_and_its_workspace(ctx):
             assert torch.equal(d, want[i][1])
     for m, cb, _ in items[::2]:
         m.close(); cb.close()
+
+
+# Tensors that share launches: more than a launch holds, more kernels than one (symbol pairs up to 6 bits, private runs where they
+# fit, a table per channel, a non-linearity behind the decoder), tensors of one tile beside tensors of many, and beside them others that
+# have kernels of their own.
+def test_long_mixed_lists_equal_the_per_tensor_calls(ctx):
+    shapes = [(64, 14, 14, 5, 4, False), (16, 4, 2, 1, 3, False), (256, 14, 14, 3, 8, False), (48, 10, 6, 2, 7, False), (80, 12, 12, 2, 5, True),
+              (320, 7, 7, 3, 4, False), (96, 13, 13, 2, 4, False), (128, 28, 28, 2, 2, False)]
+    sides, items, relus = [], [], []
+    for i, (c, h, w, n, bits, per_channel) in enumerate(shapes):
+        o = H.oracle_side(fm.LayerSpec(c, h, w, 0.9, None, 8700 + i), bits, max(3, 2 * c // (h * w) + 1), n, torch.bfloat16, per_channel)
+        model = H.import_model(tc, ctx, o["model"], torch.bfloat16)
+        sides.append((model, tc.tc_codebook_import(ctx, o["lengths"], bits), o["x"].cuda()))
+    for j in range(70):
+        model, cb, x = sides[(j * 5) % len(sides)]
+        items.append((model, cb, x[:1 + j % x.shape[0]].contiguous()))
+        relus.append(j % 3 == 0)
+    encs = tc.tc_encode_many(ctx, items)
+    assert tc.tc_get_status(ctx) == 0
+    for relu in (False, True):
+        pick = [i for i in range(len(items)) if relus[i] == relu] if relu else list(range(len(items)))
+        outs = tc.tc_decode_many(ctx, [(*items[i][:2], encs[i], items[i][2].shape, torch.bfloat16) for i in pick], relu=relu)
+        assert tc.tc_get_status(ctx) == 0
+        for i, out in zip(pick, outs):
+            model, cb, x = items[i]
+            alone = tc.tc_encode(ctx, model, cb, x)
+            assert alone.total_bits() == encs[i].total_bits()
+            assert np.array_equal(H.stream_words(encs[i]), H.stream_words(alone)) and np.array_equal(H.chunk_len(encs[i]), H.chunk_len(alone))
+            assert torch.equal(out, tc.tc_decode(ctx, model, cb, alone, x.shape, torch.bfloat16, relu=relu))
+    assert tc.tc_get_status(ctx) == 0
