@@ -217,9 +217,8 @@ __device__ __noinline__ Sink code_again(Sink sink, uint32_t trow, int blk0, int 
 // kPair (per-layer tables, b <= 6): the code tables are indexed by two neighbouring symbols at once
 // (q0 | q1 << b), which halves the lookups.
 // kHist (statistics, Section 3.1 "Variable length coding": the entropy needs the distribution of
-// the symbols): every symbol is also counted, per coefficient channel, into a.hist.  The lanes of
-// a warp hold one coefficient of 32 pixels; the symbol most of them hold (the zero level) is
-// counted once per warp from a ballot, the others one atomic each.
+// the symbols): every symbol but the zero level is also counted, per coefficient channel, into one of the copies of a.hist, one
+// atomic each.
 // `block` of `blocks` that share the tensor's tiles.
 template <bool kPerChannel, bool kDebug, bool kPair, bool kHist, bool kRuns>
 __device__ __forceinline__ void encode_tiles(const EncodeArgs &a, const Plan &pl, unsigned int block, unsigned int blocks)
@@ -533,7 +532,7 @@ __device__ __forceinline__ void encode_tiles(const EncodeArgs &a, const Plan &pl
                         if constexpr (kHist) {
                             // every symbol other than the zero level is counted; the zero level's count is what
                             // is left of the pixels, which the caller works out
-                            if (valid && qv[i] != kMagicBits + (uint32_t)a.hist_modal) atomicAdd(a.hist + (size_t)j * nsym + (qv[i] & 0xffu), 1ull);
+                            if (valid && qv[i] != kMagicBits + (uint32_t)a.hist_modal) atomicAdd(a.hist + ((size_t)(block % kHistCopies) * a.k + j) * nsym + (qv[i] & 0xffu), 1ull);
                             // outside the quantiser's range [lo, lo + (2^b - 1) step]
                             const float t = fmaf(__uint_as_float(r[i]), inv_range, s_bias[j]);
                             n_clamped += (valid && (t < 0.f || t > 1.f)) ? 1u : 0u;

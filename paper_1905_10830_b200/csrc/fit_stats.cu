@@ -14,22 +14,6 @@ using namespace tcdev;
 __device__ __forceinline__ double as_double(float v) { return (double)v; }
 __device__ __forceinline__ double as_double(__nv_bfloat16 v) { return (double)__bfloat162float(v); }
 
-// The values are in registers from here on: without it the compiler moves each load to where its value is used, behind the
-// additions before it.
-__device__ __forceinline__ void keep(float &v) { asm volatile("" : "+f"(v)); }
-__device__ __forceinline__ void keep(__nv_bfloat16 &v)
-{
-    unsigned short raw = __bfloat16_as_ushort(v);
-    asm volatile("" : "+h"(raw));
-    v = __ushort_as_bfloat16(raw);
-}
-template <typename TIn, int N>
-__device__ __forceinline__ void keep_loads(TIn (&v)[N])
-{
-#pragma unroll
-    for (int i = 0; i < N; ++i) keep(v[i]);
-}
-
 // V elements that one load brings (V sizeof(TIn) is 2 to 16 bytes, and the address a multiple of it)
 template <typename TIn, int V>
 struct alignas(V * sizeof(TIn)) Vector { TIn v[V]; };
@@ -159,8 +143,8 @@ __global__ void __launch_bounds__(kCovThreads, 4) covariance_kernel(const TIn *x
 }
 
 // Per-block min and max of coefficient 0: y0 = sum_c T[0][c] (x_c - mu_c), summed in channel
-// order without contraction.  Bound by the latency of the loads, so 32 of them go ahead of the chain of additions, in small
-// blocks that fill the SMs evenly (a load at a time took 256x14x14 x 256 37 us).
+// order without contraction.  Bound by the latency of the loads, so 32 of them go ahead of the chain of additions (256x14x14 x 256:
+// 37 us with four ahead, 14.9 now, 118 where the compiler put every load beside its addition).
 constexpr int kRangeThreads = 128, kRangeAhead = 32;
 
 template <typename TIn>
@@ -172,7 +156,8 @@ __global__ void __launch_bounds__(kRangeThreads) range0_kernel(const TIn *x, int
     __syncthreads();
     const long long pixels = (long long)n * hw;
     double mn = INFINITY, mx = -INFINITY;
-    for (long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x; p < pixels; p += (long long)gridDim.x * blockDim.x) {
+    for (long long first = (long long)blockIdx.x * blockDim.x; first < pixels; first += (long long)gridDim.x * blockDim.x) {
+        const long long p = min(first + threadIdx.x, pixels - 1);      // threads past the end repeat the last pixel
         const long long img = p / hw, s = p - img * hw;
         const TIn *src = x + img * c * (long long)hw + s;
         double y = 0.0;
@@ -181,7 +166,7 @@ __global__ void __launch_bounds__(kRangeThreads) range0_kernel(const TIn *x, int
             TIn got[kRangeAhead];
 #pragma unroll
             for (int i = 0; i < kRangeAhead; ++i) got[i] = src[(long long)(cc + i) * hw];
-            keep_loads(got);
+            __syncwarp();                                              // (else the compiler moves each load to its addition)
 #pragma unroll
             for (int i = 0; i < kRangeAhead; ++i) y = __dadd_rn(y, __dmul_rn(s_rm[cc + i], __dsub_rn(as_double(got[i]), s_rm[c + cc + i])));
         }
@@ -297,6 +282,16 @@ void launch_sqerr(const TIn *x, const TIn *xhat, long long count, double *sum_sq
     else sqerr_kernel<TIn, 1><<<(unsigned)blocks, kErrThreads, 0, s>>>(x, xhat, count, sum_sq, zeros);
 }
 
+// copies[0][i] = the sum of copies[.][i]
+__global__ void fold_counts_kernel(unsigned long long *counts, int copies, int n)
+{
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    unsigned long long sum = 0;
+    for (int k = 0; k < copies; ++k) sum += counts[(size_t)k * n + i];
+    counts[i] = sum;
+}
+
 inline bool launched() { return cudaGetLastError() == cudaSuccess; }
 
 }  // namespace
@@ -368,5 +363,11 @@ tc_status tc_launch_sqerr(const void *x, const void *xhat, int dtype, long long 
 {
     if (dtype == TC_F32) launch_sqerr((const float *)x, (const float *)xhat, count, sum_sq, zeros, s);
     else launch_sqerr((const __nv_bfloat16 *)x, (const __nv_bfloat16 *)xhat, count, sum_sq, zeros, s);
+    return launched() ? TC_OK : TC_ERR_CUDA;
+}
+
+tc_status tc_launch_fold_counts(unsigned long long *counts, int copies, int n, cudaStream_t s)
+{
+    fold_counts_kernel<<<(n + 255) / 256, 256, 0, s>>>(counts, copies, n);
     return launched() ? TC_OK : TC_ERR_CUDA;
 }

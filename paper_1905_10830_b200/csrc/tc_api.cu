@@ -1600,7 +1600,7 @@ static tc_status stats_tensor_core(tc_ctx *ctx, const tc_model *m, const tc_code
     const size_t hist_bytes = (size_t)m->k * nsym * sizeof(unsigned long long);
     const size_t off_stream = up((size_t)chunk_n * image_bytes), off_chunk = off_stream + up(lay.stream_bytes),
                  off_tile = off_chunk + up(lay.chunk_len_bytes), off_hist = off_tile + up(lay.tile_off_bytes),
-                 off_small = off_hist + up(hist_bytes), total = off_small + 64;
+                 off_small = off_hist + up(hist_bytes * kHistCopies), total = off_small + 64;
     if (total > ctx->host_arena_bytes) {
         if (ctx->host_arena) { TC_CUDA(cudaDeviceSynchronize()); cudaFree(ctx->host_arena); ctx->host_arena = nullptr; ctx->host_arena_bytes = 0; }
         TC_CUDA(cudaMalloc(&ctx->host_arena, total));
@@ -1610,7 +1610,7 @@ static tc_status stats_tensor_core(tc_ctx *ctx, const tc_model *m, const tc_code
     unsigned long long *d_hist = (unsigned long long *)(base + off_hist);
     double *d_sq = (double *)(base + off_small);
     unsigned long long *d_zeros = (unsigned long long *)(base + off_small + 8), *d_clamped = (unsigned long long *)(base + off_small + 16);
-    TC_CUDA(cudaMemsetAsync(base + off_hist, 0, up(hist_bytes) + 64, s));
+    TC_CUDA(cudaMemsetAsync(base + off_hist, 0, up(hist_bytes * kHistCopies) + 64, s));
     const long long tiles_max = ((long long)chunk_n * hw + TC_TILE_PIXELS - 1) / TC_TILE_PIXELS;
     const size_t lookback = kEncodeScratchHeader + (size_t)tiles_max * sizeof(unsigned long long);
     if ((st = ensure_scratch(ctx, lookback)) != TC_OK) return st;
@@ -1628,6 +1628,7 @@ static tc_status stats_tensor_core(tc_ctx *ctx, const tc_model *m, const tc_code
         if (st != TC_OK) return st;
         if ((st = tc_launch_sqerr(xi.data, xh.data, x->dtype, (long long)cn * m->c * hw, d_sq, d_zeros, s)) != TC_OK) return st;
     }
+    if ((st = tc_launch_fold_counts(d_hist, kHistCopies, m->k * nsym, s)) != TC_OK) return st;
     hist.assign((size_t)m->k * nsym, 0ull);
     TC_CUDA(cudaMemcpyAsync(hist.data(), d_hist, hist_bytes, cudaMemcpyDeviceToHost, s));
     TC_CUDA(cudaMemcpyAsync(&sq, d_sq, 8, cudaMemcpyDeviceToHost, s));

@@ -128,7 +128,7 @@ struct EncodeArgs {
     unsigned long long *clamped;      // nullable: counts coefficients outside the range
     int emit;                         // 0: symbols only (statistics mode)
     const uint8_t *sym_in;            // exact kernels: non-null = the symbols [P][K] are given, skip the projection
-    unsigned long long *hist;         // tensor-core encoder, statistics: non-null = per-coefficient counts [K][2^bits] of every symbol but hist_modal are added here
+    unsigned long long *hist;         // tensor-core encoder, statistics: non-null = per-coefficient counts [kHistCopies][K][2^bits] of every symbol but hist_modal are added here
     int hist_modal;                   // the symbol of the zero level, which most coefficients hold: statistics mode counts all the others
     int modal;                        // per-layer table: the symbol whose code is the single bit 0, or -1 if no code has one bit
     float max_bias;                   // see tc_model
@@ -207,6 +207,9 @@ tc_status tc_encode_with_scratch(tc_ctx *ctx, const tc_model *m, const tc_codebo
                                  int splits, void *stream_out, size_t capacity, uint16_t *chunk_len, uint64_t *tile_off,
                                  const tc_debug_out *debug, void *scratch, void *work, cudaStream_t s,
                                  unsigned long long *hist = nullptr, unsigned long long *clamped = nullptr, int list_sms = 0);
+// Copies of the counts that the encoder's blocks share in statistics mode: the atomics of a leading coefficient all meet in one line of L2,
+// which takes one at a time (256x14x14 x 256: 96 us with one copy, 48 with eight).
+constexpr int kHistCopies = 8;
 // tensors of fewer tiles than this many per SM take the one-thread-per-value exact kernels
 constexpr int kExactParallelTilesPerSm = 2;
 
@@ -258,6 +261,7 @@ tc_status tc_launch_range0(const void *x, int dtype, int n, int c, int hw, const
                            const double *row0, double *block_minmax, int *n_blocks_out,
                            cudaStream_t s);
 int tc_range0_max_blocks(long long pixels);
+tc_status tc_launch_fold_counts(unsigned long long *counts, int copies, int n, cudaStream_t s);
 tc_status tc_launch_histogram(const uint8_t *sym, long long pixels, int k, int groups, int bits,
                               unsigned long long *hist, cudaStream_t s);
 tc_status tc_launch_sqerr(const void *x, const void *xhat, int dtype, long long count,
