@@ -570,10 +570,11 @@ def tc_roundtrip_host(ctx: Context, model: Model, cb: Codebook, x_host: torch.Te
 def tc_stats(ctx: Context, model: Model, cb: Codebook | None, x: torch.Tensor, *, groups: int = 1,
              want_hist: bool = True) -> Stats:
     t = _tensor(x)
-    exp = tc_model_export(model)
     hist = None
     if want_hist:
-        hist = torch.zeros(groups, 1 << exp["bits"], dtype=torch.int64, device=x.device)
+        desc = _ModelDesc()          # without its arrays: the basis stays on the device
+        _check(load_library().tc_model_export(model.ptr, C.byref(desc)), "tc_model_export")
+        hist = torch.zeros(groups, 1 << desc.bits, dtype=torch.int64, device=x.device)
     s = _StatsOut(groups, hist.data_ptr() if hist is not None else None, 0, 0, 0, 0, 0, 0)
     _check(load_library().tc_stats(ctx.ptr, model.ptr, cb.ptr if cb is not None else None, C.byref(t), C.byref(s),
                                    _stream_ptr(ctx.device)), "tc_stats")
