@@ -346,8 +346,9 @@ __global__ void __launch_bounds__(TC_TILE_PIXELS * kMaxParts) pack_symbols_kerne
 // Entropy decoder that leaves the symbols in memory, row 0 = the first pixel of tile `first_tile`: as bytes
 // ([P][K], for the fp64 inverse of tensors of few pixels), or centred and as bf16 (kOperand: the
 // operand of the tensor cores' inverse transform):
-// one block per tile, one thread per chunk (up to 512 per tile), so that every chunk of the tile is
-// walked at the same time; the inverse transform then runs in reconstruct_kernel.  Same checks as
+// one thread per chunk (up to 512 per tile), so that every chunk of the tile is
+// walked at the same time; the inverse transform then runs in reconstruct_kernel.  A tile's chunks may be dealt to
+// gridDim.y blocks, each with the pixels of its own.  Same checks as
 // the per-pixel decoder: tile offsets aligned, ordered and inside the stream, every chunk inside
 // its tile and consumed to exactly its recorded length.
 constexpr int kUnpackThreads = 512;
@@ -474,12 +475,14 @@ __device__ __noinline__ void clear_rows(void *out, long long row0, int px0, int 
 // come from a table that every lane has in a bank of its own, and rows leave 64 bytes at a time.  576x14x14 x 1024
 // decode 376 -> 341 us, x 128 (21 warps an SM) 60.5 -> 57.1; 384x14x14 x 128 (5 warps) would lose, 39.1 -> 41.5, to the
 // second lookup in the chain, 512x7x7 x 64 (25 tiles) 23.3 -> 27.3.
+// Two or four blocks a tile where that leaves no SM with two: the eight or sixteen warps of a tile share an SM's issue slots while others
+// idle (256x14x14 f32, per-channel codes, with the inverse 24.5 -> 20.5 us, 512x14x14 f32 45 -> 37, 768x7x7 x 16 26.7 -> 22.6).
 template <bool kOperand, bool kPerLayer, bool kFull>
 __global__ void __launch_bounds__(kUnpackThreads) unpack_symbols_kernel(DecodeArgs a, void *out, long long first_tile, unsigned int table_bytes,
                                                                          unsigned int segment_bytes)
 {
     __shared__ uint32_t s_first[kFull ? (32 << kFirstBits) : 1];
-    __shared__ unsigned int s_warp_sums[kUnpackThreads / 32];
+    __shared__ unsigned int s_warp_sums[kUnpackThreads / 32], s_before[kUnpackThreads / 32];
     __shared__ unsigned int s_start[kUnpackThreads];
     extern __shared__ __align__(16) unsigned char s_tables[];   // the per-layer table, or the bounds and bases of every channel's code
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
@@ -519,45 +522,52 @@ __global__ void __launch_bounds__(kUnpackThreads) unpack_symbols_kernel(DecodeAr
         const int n_px = (int)min((long long)TC_TILE_PIXELS, a.pixels - tile * TC_TILE_PIXELS);
         clear_rows<kOperand>(out, (tile - first_tile) * TC_TILE_PIXELS, px0, min(px1, n_px), step, a.k, j, n, a.center);
     };
+    // this block's chunks of the tile, and their pixels
+    const int chunks_per_tile = a.splits * TC_TILE_PIXELS / a.chunk_pixels;      // at most 512
+    const int per = chunks_per_tile / (int)gridDim.y, c_first = (int)blockIdx.y * per;
+    const int block_px = TC_TILE_PIXELS / (int)gridDim.y, px_first = (int)blockIdx.y * block_px;
     if (!tile_ok) {
-        clear(t, TC_TILE_PIXELS, blockDim.x, 0, a.k);
+        clear(px_first + t, px_first + block_px, blockDim.x, 0, a.k);
         if (t == 0) tc_dev_set_status(a.status, TC_ERR_CORRUPT_STREAM);
         return;
     }
     const bool staged = end - base <= (unsigned long long)segment_bytes * 8ull;
     const uint32_t seg = tables + table_bytes;
     if (staged) stage(seg, a.stream + (base >> 5), (unsigned int)((end - base) >> 7));
-    const int chunks_per_tile = a.splits * TC_TILE_PIXELS / a.chunk_pixels;      // at most 512
-    // where every chunk of the tile starts: the lengths of its earlier chunks
-    const long long scan_ch = tile * chunks_per_tile + t;
-    const unsigned int len_t = (t < chunks_per_tile && scan_ch < a.n_chunks) ? a.chunk_len[scan_ch] : 0u;
-    unsigned int inc = len_t;
+    // where every chunk of the block starts: the lengths of its tile's earlier chunks
+    const long long tile_ch = tile * chunks_per_tile;
+    const unsigned int len_t = (t < per && tile_ch + c_first + t < a.n_chunks) ? a.chunk_len[tile_ch + c_first + t] : 0u;
+    unsigned int inc = len_t, before = 0;
+    for (int i = t; i < c_first; i += blockDim.x) before += tile_ch + i < a.n_chunks ? a.chunk_len[tile_ch + i] : 0u;
+    before = __reduce_add_sync(0xffffffffu, before);
 #pragma unroll
     for (int d = 1; d < 32; d <<= 1) {
         const unsigned int up = __shfl_up_sync(0xffffffffu, inc, d);
         if (lane >= d) inc += up;
     }
-    if (lane == 31) s_warp_sums[warp] = inc;
+    if (lane == 31) { s_warp_sums[warp] = inc; s_before[warp] = before; }
     asm volatile("cp.async.wait_all;" ::: "memory");
     __syncthreads();
     unsigned int off_t = inc - len_t;
     for (int w = 0; w < warp; ++w) off_t += s_warp_sums[w];
+    if (c_first)
+        for (int w = 0; w < (int)blockDim.x / 32; ++w) off_t += s_before[w];
     s_start[t] = off_t;
     __syncthreads();
-    // this thread's chunk: chunk_pixels whole pixels, or one of `splits` runs of one pixel
-    const int part = a.splits > 1 ? t / TC_TILE_PIXELS : 0;
-    const int in_tile = a.splits > 1 ? (t % TC_TILE_PIXELS) * a.splits + part : t;
-    const long long ch = tile * chunks_per_tile + in_tile;
-    if (warp * 32 >= chunks_per_tile) return;
+    // this thread's chunk: chunk_pixels whole pixels, or one of `splits` runs of one pixel (the threads of a warp take the same run)
+    const int part = a.splits > 1 ? t / block_px : 0, my_px = a.splits > 1 ? px_first + t % block_px : px_first + t * a.chunk_pixels;
+    const int in_block = a.splits > 1 ? (t % block_px) * a.splits + part : t;
+    const long long ch = tile_ch + c_first + in_block;
+    if (warp * 32 >= per) return;
     // a lane without a chunk walks zeros beside its warp where the warp's rows leave together
-    const bool mine = t < chunks_per_tile && ch < a.n_chunks;
+    const bool mine = t < per && ch < a.n_chunks;
     if (!kFull && !mine) return;
-    const unsigned int want = mine ? a.chunk_len[ch] : 0u, off = mine ? s_start[in_tile] : 0u;
+    const unsigned int want = mine ? a.chunk_len[ch] : 0u, off = mine ? s_start[in_block] : 0u;
     bool bad = base + off + want > end;
     auto walk = [&](auto &r) {
         unsigned int used = 0;
         const int run = a.k / a.splits, j_first = part * run;
-        const int first_px = a.splits > 1 ? t % TC_TILE_PIXELS : t * a.chunk_pixels;
+        const int first_px = my_px;
         // decodes kN symbols from coefficient j on into v (one per element)
         auto decode = [&](int j, auto &v) {
             constexpr int kN = sizeof(v) / sizeof(v[0]);
@@ -601,7 +611,7 @@ __global__ void __launch_bounds__(kUnpackThreads) unpack_symbols_kernel(DecodeAr
             // runs are multiples of 8; 32 symbols of the warp's 32 rows are turned through shared memory, so that a
             // store covers 64 bytes of a row
             const uint32_t rows = tables + table_bytes + segment_bytes + (uint32_t)warp * kRowsWarpBytes;
-            const int per_lane = a.splits > 1 ? 1 : a.chunk_pixels, px0 = a.splits > 1 ? (warp * 32) % TC_TILE_PIXELS : warp * 32 * per_lane;
+            const int per_lane = a.splits > 1 ? 1 : a.chunk_pixels, px0 = px_first + (a.splits > 1 ? (warp * 32) % block_px : warp * 32 * per_lane);
             for (int lp = 0; lp < per_lane; ++lp) {
                 const unsigned int used_before = used;
 #pragma unroll 1
@@ -662,8 +672,7 @@ __global__ void __launch_bounds__(kUnpackThreads) unpack_symbols_kernel(DecodeAr
     };
     const bool walks = mine && !bad;
     if (!kFull && !walks) {
-        const int px = a.splits > 1 ? t % TC_TILE_PIXELS : t * a.chunk_pixels;
-        clear(px, px + a.chunk_pixels, 1, part * (a.k / a.splits), a.k / a.splits);
+        clear(my_px, my_px + a.chunk_pixels, 1, part * (a.k / a.splits), a.k / a.splits);
     } else if (staged) {
         StagedReader r;
         r.init(seg, walks ? off : 0u, walks ? seg + (uint32_t)((end - base) >> 3) : seg);
@@ -745,16 +754,21 @@ static tc_status launch_unpack(const DecodeArgs &a, void *out, long long first_t
         if (sorted % 16 == 0 && ((uintptr_t)a.sorted & 15u) == 0 && sorted <= kSortedStaged) tables += sorted;
     }
     const unsigned int segment = (unsigned int)std::min<long long>((long long)a.k * TC_TILE_PIXELS * 3 / 8, 48 * 1024);
+    // Two or four blocks a tile of 256 chunks and more, as long as every block has an SM (320x7x7 x 180, 69 tiles in four blocks each:
+    // 20.5 -> 22.6 us; 128x28x28 f32, two blocks of 64 chunks: 18.1 -> 18.5).
+    const long long tiles = end_tile - first_tile;
+    int parts = 1;
+    while (parts < 4 && chunks >= 256 && tiles * parts * 2 <= sm_count && chunks % (128 * parts) == 0) parts *= 2;
     // a block of few chunks has more threads for staging while all blocks are resident at once
-    const int threads = (chunks + 31) / 32 * 32, least = end_tile - first_tile < 4 * sm_count ? 256 : 32;
+    const int threads = (chunks / parts + 31) / 32 * 32, least = tiles * parts < 4 * sm_count ? 256 : 32;
     // from 16 warps an SM on the shared-memory pipe is what bounds a per-layer decoder (see the kernel)
-    const bool full = kOperand && a.groups == 1 && (end_tile - first_tile) * threads >= 16 * 32 * (long long)sm_count;
+    const bool full = kOperand && a.groups == 1 && tiles * ((chunks + 31) / 32) >= 16 * (long long)sm_count;
     void (*kernel)(DecodeArgs, void *, long long, unsigned int, unsigned int) =
         a.groups != 1 ? unpack_symbols_kernel<kOperand, false, false>
         : full ? unpack_symbols_kernel<kOperand, true, kOperand> : unpack_symbols_kernel<kOperand, true, false>;
     if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024) != cudaSuccess) return TC_ERR_CUDA;
     const size_t rows = full ? (size_t)(threads / 32) * kRowsWarpBytes : 0;
-    kernel<<<(unsigned int)(end_tile - first_tile), std::max(threads, least), tables + segment + rows, s>>>(a, out, first_tile, tables, segment);
+    kernel<<<dim3((unsigned int)tiles, (unsigned int)parts), std::max(threads, least), tables + segment + rows, s>>>(a, out, first_tile, tables, segment);
     return cudaGetLastError() == cudaSuccess ? TC_OK : TC_ERR_CUDA;
 }
 

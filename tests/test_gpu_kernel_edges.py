@@ -349,3 +349,51 @@ def test_decoded_rows_more_than_2_32_elements_apart(ctx):
     for i in range(c):
         assert torch.equal(a[0, i].view(parts, h // parts, w), b[:, i])
     m.close(); cb.close()
+
+
+# Entropy coder and decoder with a tile dealt to several blocks: tiles few enough for two and four blocks (and one more), last tiles
+# whose later blocks have a pixel or none, chunks of several pixels, one, two and four a pixel, tables per layer and per channel, codes
+# of one bit (blocks of a few words) and of twelve.  Against the one-thread-per-pixel kernels, which run without workspace.
+@pytest.mark.parametrize("c,pixels,bits,dtype,per_channel,cp,splits", [
+    (64, 1, 4, torch.float32, False, 0, 0), (64, 33, 4, torch.float32, False, 0, 0), (64, 128 * 37, 3, torch.float32, False, 4, 1),
+    (64, 128 * 37 + 1, 5, torch.float32, True, 0, 0), (96, 65, 8, torch.float32, True, 0, 0), (128, 128 * 74 - 31, 4, torch.float32, False, 0, 0),
+    (128, 128 * 74 + 97, 4, torch.float32, False, 0, 0), (64, 200, 2, torch.float32, False, 64, 1), (64, 200, 2, torch.float32, False, 32, 1),
+    (256, 96, 6, torch.float32, True, 0, 0), (256, 300, 1, torch.float32, False, 0, 0), (512, 129, 8, torch.float32, False, 0, 0),
+    (512, 128 * 5 + 34, 4, torch.float32, True, 0, 0), (320, 49 * 3, 4, torch.bfloat16, False, 0, 0), (320, 49 * 100, 8, torch.bfloat16, False, 0, 0),
+    (576, 49 * 7, 5, torch.bfloat16, False, 0, 0), (256, 49 * 3, 6, torch.bfloat16, True, 0, 0), (512, 49 * 500, 4, torch.bfloat16, False, 0, 0)])
+def test_a_tile_dealt_to_several_blocks(ctx, c, pixels, bits, dtype, per_channel, cp, splits):
+    rng = np.random.default_rng(c + pixels)
+    h, n = (7, pixels // 49) if dtype == torch.bfloat16 else (1, 1)
+    w = pixels // (n * h)
+    basis, _ = np.linalg.qr(rng.standard_normal((c, c)))
+    if dtype == torch.bfloat16:
+        basis = torch.from_numpy(basis).to(torch.bfloat16).double().numpy()
+    else:
+        basis = basis.astype(np.float32).astype(np.float64)
+    scale = 4.0 * 0.97 ** np.arange(c) + 1e-3
+    top = (1 << bits) - 1
+    step = 12.0 / top if bits > 1 else 6.0
+    lo = -step * round(6.0 / step)
+    x = torch.from_numpy(((rng.standard_normal((n * h * w, c)) * scale) @ basis).reshape(n, h * w, c).transpose(0, 2, 1).reshape(n, c, h, w).copy()).to(dtype).cuda()
+    counts = rng.integers(0, 50, (c if per_channel else 1, top + 1))
+    counts[..., top // 2] = 2000 if bits > 1 else 1
+    counts[..., 0] = 0
+    lengths = np.stack([tc.tc_host_huffman_lengths(row) for row in counts])
+    m = tc.tc_model_import(ctx, basis=basis, mean=np.zeros(c), lo=lo, step=step, bits=bits, basis_dtype=tc.binding.TC_BF16 if dtype == torch.bfloat16 else tc.binding.TC_F32,
+                           eig=scale ** 2)
+    cb = tc.tc_codebook_import(ctx, lengths, bits)
+    kw = dict(chunk_pixels=cp, pixel_splits=splits) if cp else {}
+    enc = tc.tc_encode(ctx, m, cb, x, **kw)
+    x_hat = tc.tc_decode(ctx, m, cb, enc, x.shape, dtype)
+    assert tc.tc_get_status(ctx) == 0
+    tc.tc_force_exact_path(ctx, 4)
+    want = tc.tc_encode(ctx, m, cb, x, **kw)
+    want_hat = tc.tc_decode(ctx, m, cb, enc, x.shape, dtype)
+    tc.tc_force_exact_path(ctx, 0)
+    assert tc.tc_get_status(ctx) == 0
+    if dtype == torch.float32:
+        assert _same_stream(enc, want) and torch.equal(x_hat, want_hat)
+    else:           # fp32 accumulation in another order: a symbol at a rounding tie, bf16 neighbours now and then
+        assert abs(enc.total_bits() - want.total_bits()) <= 1e-3 * want.total_bits() + 256
+        assert (x_hat != want_hat).double().mean() <= 1e-3 and (x_hat.double() - want_hat.double()).abs().max() <= 2.0 ** -7 * want_hat.double().abs().max()
+    m.close(); cb.close()
