@@ -12,7 +12,9 @@
 
 namespace {
 
+using tcdev::cluster_sync;
 using tcdev::mma_f64;
+using tcdev::peer_address;
 
 constexpr int kReduceWarps = 8, kReduceThreads = 32 * kReduceWarps;    // of a block that reduces: what every warp repeats costs issue slots
 constexpr int kWarps = 16, kThreads = 32 * kWarps;                      // of one that divides, or takes Rayleigh quotients
@@ -47,20 +49,6 @@ __device__ __forceinline__ uint32_t cluster_rank()
     uint32_t r;
     asm volatile("mov.u32 %0, %cluster_ctarank;" : "=r"(r));
     return r;
-}
-
-// every thread of the cluster has come; what they wrote (shared memory of any block, global memory) is visible
-__device__ __forceinline__ void cluster_sync()
-{
-    __syncwarp();
-    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-
-__device__ __forceinline__ uint32_t peer_address(const void *p, uint32_t rank)
-{
-    uint32_t out;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(out) : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(rank));
-    return out;
 }
 
 // 16 rows of `u` (shared memory, row pitch ld_u) times columns [col, col + 16) of `b` (global memory, row pitch ld_b),

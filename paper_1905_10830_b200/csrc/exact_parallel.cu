@@ -207,9 +207,13 @@ __global__ void __launch_bounds__(kPx * kRows) reconstruct_kernel(DecodeArgs a, 
 // up to eight threads a pixel, a per-layer table in shared memory and two codes a piece (960x7x7 x 128
 // from a cold cache: 45 us with four threads, tables and packed words in global memory, 42 staged with an
 // atomic OR a word, 22 like this).
-constexpr int kMaxParts = 8;
+// kCluster: a tile is dealt to the gridDim.y blocks of a cluster, each with the pixels of its own, where the tiles would leave most SMs
+// idle.  The first block takes the ticket and finds the tile's place in the stream; the blocks exchange their bits through
+// distributed shared memory, and a block hands the word that it shares with the block before to that one.
+// 960x7x7 x 128 47.1 -> 41.0 us with the kernels before, 512x14x14 f32 56 -> 44, 768x7x7 x 16 26.7 -> 21.6.
+constexpr int kMaxParts = 8, kMaxTileBlocks = 4;
 
-template <bool kPerLayer>
+template <bool kPerLayer, bool kCluster>
 __global__ void __launch_bounds__(TC_TILE_PIXELS * kMaxParts) pack_symbols_kernel(EncodeArgs a, const uint8_t *sym, int parts, long long first_tile,
                                                                                   unsigned int staging_bytes)
 {
@@ -220,17 +224,27 @@ __global__ void __launch_bounds__(TC_TILE_PIXELS * kMaxParts) pack_symbols_kerne
     __shared__ unsigned long long s_base;
     __shared__ int s_write_ok;
     __shared__ uint32_t s_enc[256];
+    __shared__ unsigned int s_totals[kMaxTileBlocks], s_head;  // bits of every block of the cluster; the word shared with the next block
     extern __shared__ __align__(16) uint32_t s_words[];
     const int t = threadIdx.x;
     const int nsym = 1 << a.bits;
+    const int blocks = kCluster ? (int)gridDim.y : 1, rank = kCluster ? (int)blockIdx.y : 0, block_px = TC_TILE_PIXELS / blocks;
+    if constexpr (kCluster) { cluster_sync(); }               // the others run: their shared memory may be written
     if constexpr (kPerLayer)
         for (int i = t; i < nsym; i += blockDim.x) s_enc[i] = __ldg(a.enc + i);
     chain_wait();                                             // the symbols and the cleared look-back state
-    if (t == 0) s_tile = (long long)atomicAdd(a.ticket, 1u);
-    __syncthreads();
+    if (t == 0 && rank == 0) {
+        s_tile = (long long)atomicAdd(a.ticket, 1u);
+        if constexpr (kCluster) {
+            for (int r = 1; r < blocks; ++r)
+                asm volatile("st.shared::cluster.u64 [%0], %1;" ::"r"(peer_address(&s_tile, r)), "l"(s_tile) : "memory");
+        }
+    }
+    if constexpr (kCluster) { cluster_sync(); }
+    else { __syncthreads(); }
     const long long tile = s_tile;
-    const int px = t / parts, part = t - px * parts;          // the threads of a pixel are neighbours
-    const long long p = tile * TC_TILE_PIXELS + px;
+    const int px = t / parts, part = t - px * parts;          // of the block's pixels; the threads of a pixel are neighbours
+    const long long p = tile * TC_TILE_PIXELS + rank * block_px + px;
     const bool valid = p < a.pixels;
     const int run = a.k / parts, j0 = part * run;
     const uint8_t *src = sym + (p - first_tile * TC_TILE_PIXELS) * a.k + j0;
@@ -254,19 +268,30 @@ __global__ void __launch_bounds__(TC_TILE_PIXELS * kMaxParts) pack_symbols_kerne
     // pixel totals, scanned by the first 128 threads
     if (t < TC_TILE_PIXELS) {
         unsigned int pixel_bits = 0, total = 0;
-        for (int r = 0; r < parts; ++r) pixel_bits += s_run_bits[t * parts + r];
+        for (int r = 0; r < parts && t < block_px; ++r) pixel_bits += s_run_bits[t * parts + r];
         const unsigned int off = group_exclusive_scan_128(pixel_bits, s_warp_sums, t, 1, total);
         s_pixel_off[t] = off;
-        if (t == 0) {
-            s_pixel_off[TC_TILE_PIXELS] = total;
-            lookback_publish(a.tile_state, tile, ((unsigned long long)total + 127ull) & ~127ull);
-        }
+        if (t == 0) s_pixel_off[TC_TILE_PIXELS] = total;
+        if constexpr (kCluster) {
+            if (t < blocks) asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(peer_address(s_totals + rank, t)), "r"(total) : "memory");
+        } else if (t == 0) lookback_publish(a.tile_state, tile, ((unsigned long long)total + 127ull) & ~127ull);
     }
-    __syncthreads();
-    const unsigned int tile_bits = s_pixel_off[TC_TILE_PIXELS];
+    unsigned int tile_bits, block_off = 0;                    // bits of the tile, and of its blocks before this one
+    if constexpr (kCluster) {
+        cluster_sync();
+        tile_bits = 0;
+        for (int r = 0; r < blocks; ++r) {
+            if (r < rank) block_off += s_totals[r];
+            tile_bits += s_totals[r];
+        }
+        if (t == 0 && rank == 0) lookback_publish(a.tile_state, tile, ((unsigned long long)tile_bits + 127ull) & ~127ull);
+    } else {
+        __syncthreads();
+        tile_bits = s_pixel_off[TC_TILE_PIXELS];
+    }
     const unsigned long long padded = ((unsigned long long)tile_bits + 127ull) & ~127ull;
     const bool staged = padded <= (unsigned long long)staging_bytes * 8ull;
-    unsigned int my_off = s_pixel_off[px];
+    unsigned int my_off = block_off + s_pixel_off[px];
     for (int r = 0; r < part; ++r) my_off += s_run_bits[px * parts + r];
     // chunk lengths: a chunk is chunk_pixels pixels, or one of `splits` runs of one pixel
     if (valid) {
@@ -278,7 +303,7 @@ __global__ void __launch_bounds__(TC_TILE_PIXELS * kMaxParts) pack_symbols_kerne
                 a.chunk_len[p * a.splits + part / per_chunk] = (uint16_t)bits;
             }
         } else if (part == 0 && (p % a.chunk_pixels) == 0) {
-            const int last = min(px + a.chunk_pixels, TC_TILE_PIXELS);
+            const int last = min(px + a.chunk_pixels, block_px);
             a.chunk_len[p / a.chunk_pixels] = (uint16_t)(s_pixel_off[last] - s_pixel_off[px]);
         }
     }
@@ -312,7 +337,61 @@ __global__ void __launch_bounds__(TC_TILE_PIXELS * kMaxParts) pack_symbols_kerne
         }
     };
     const unsigned int n16 = (unsigned int)(padded >> 7);
-    if (staged) {
+    // the place that the first block found, for all of its cluster
+    auto resolve_for_all = [&] {
+        if (rank != 0) return;
+        resolve();
+        if (t == 0) {
+            for (int r = 1; r < blocks; ++r) {
+                asm volatile("st.shared::cluster.u64 [%0], %1;" ::"r"(peer_address(&s_base, r)), "l"(s_base) : "memory");
+                asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(peer_address(&s_write_ok, r)), "r"(s_write_ok) : "memory");
+            }
+        }
+    };
+    if constexpr (kCluster) {
+        const unsigned int my_bits_all = s_totals[rank], next_off = block_off + my_bits_all, end_word = n16 * 4;
+        if (staged) {
+            // This block's words: from the first that starts in its bits to the first that starts in the next block's (the last block: to
+            // the tile's end).  Word w lies at s_words[w - from].
+            const unsigned int from = (block_off >> 5) & ~3u, w_lo = (block_off + 31) >> 5, w_hi = rank == blocks - 1 ? end_word : (next_off + 31) >> 5;
+            const uint32_t words = (uint32_t)__cvta_generic_to_shared(s_words) - from * 4u;
+            const unsigned int first_open = next_off >> 5;
+            if (first_open + t < w_hi) s_words[first_open + t - from] = 0u;
+            SmemBitWriter<4> w;
+            w.init(words, words + w_hi * 4u, my_off);
+            if (valid) pack(w);
+            __syncthreads();
+            if (valid) w.finish();
+            __syncthreads();
+            if (t == 0 && my_bits_all && (block_off & 31u) != 0)
+                asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(peer_address(&s_head, rank - 1)), "r"(s_words[(block_off >> 5) - from]) : "memory");
+            resolve_for_all();
+            cluster_sync();
+            if (!s_write_ok) return;
+            if (rank < blocks - 1 && (next_off & 31u) != 0 && s_totals[rank + 1]) {
+                if (t == 0) s_words[first_open - from] |= s_head;
+                __syncthreads();
+            }
+            uint32_t *dst = a.stream + (s_base >> 5);
+            for (unsigned int i = (w_lo & ~3u) + 4 * t; i < w_hi; i += 4 * blockDim.x) {
+                if (i >= w_lo && i + 4 <= w_hi) *reinterpret_cast<uint4 *>(dst + i) = *reinterpret_cast<const uint4 *>(s_words + (i - from));
+                else
+                    for (unsigned int k = max(i, w_lo); k < min(i + 4, w_hi); ++k) dst[k] = s_words[k - from];
+            }
+        } else {
+            resolve_for_all();
+            cluster_sync();
+            uint4 *dst = reinterpret_cast<uint4 *>(a.stream + (s_base >> 5));
+            for (unsigned int i = rank * blockDim.x + t; s_write_ok && i < n16; i += blocks * blockDim.x) dst[i] = make_uint4(0u, 0u, 0u, 0u);
+            cluster_sync();
+            if (s_write_ok && valid) {
+                BitWriter w;
+                w.init(a.stream, s_base + my_off);
+                pack(w);
+                w.finish();
+            }
+        }
+    } else if (staged) {
         // every word below tile_bits / 32 is stored by the writer of its last bit; the rest starts as zero
         const unsigned int first_open = tile_bits >> 5, end_word = n16 * 4;
         const uint32_t words = (uint32_t)__cvta_generic_to_shared(s_words);
@@ -476,7 +555,7 @@ __device__ __noinline__ void clear_rows(void *out, long long row0, int px0, int 
 // decode 376 -> 341 us, x 128 (21 warps an SM) 60.5 -> 57.1; 384x14x14 x 128 (5 warps) would lose, 39.1 -> 41.5, to the
 // second lookup in the chain, 512x7x7 x 64 (25 tiles) 23.3 -> 27.3.
 // Two or four blocks a tile where that leaves no SM with two: the eight or sixteen warps of a tile share an SM's issue slots while others
-// idle (256x14x14 f32, per-channel codes, with the inverse 24.5 -> 20.5 us, 512x14x14 f32 45 -> 37, 768x7x7 x 16 26.7 -> 22.6).
+// idle (256x14x14 f32, per-channel codes, with the inverse 23.8 -> 21.5 us, 512x14x14 f32 45 -> 37, 768x7x7 x 16 26.7 -> 22.6).
 template <bool kOperand, bool kPerLayer, bool kFull>
 __global__ void __launch_bounds__(kUnpackThreads) unpack_symbols_kernel(DecodeArgs a, void *out, long long first_tile, unsigned int table_bytes,
                                                                          unsigned int segment_bytes)
@@ -715,6 +794,9 @@ int tc_pack_symbols_parts(const EncodeArgs &a)
     return 0;
 }
 
+// Coefficients from which a tile is worth a cluster: its barriers cost 2 us (64x56x56 f32 14.3 -> 15.8 us, 128 to 256 coefficients
+// even, 384x7x7 x 64 20.5 -> 18.5).
+constexpr int kClusterCoefs = 384;
 constexpr unsigned int kSpreadBytes = 118 * 1024;             // two of these do not fit an SM
 
 tc_status tc_launch_pack_symbols(const tc_ctx *ctx, const EncodeArgs &a, const uint8_t *sym, long long first_tile, long long end_tile, cudaStream_t s)
@@ -724,14 +806,25 @@ tc_status tc_launch_pack_symbols(const tc_ctx *ctx, const EncodeArgs &a, const u
     if (parts == 0 || ((uintptr_t)sym & 7u) != 0) return TC_ERR_UNSUPPORTED;
     // staging for four bits per symbol, at most 96 KB: two blocks of 1024 threads still fit an SM
     const unsigned int staging = (unsigned int)std::min<long long>((long long)a.k * TC_TILE_PIXELS / 2, 96 * 1024);
-    void (*kernel)(EncodeArgs, const uint8_t *, int, long long, unsigned int) = a.groups == 1 ? pack_symbols_kernel<true> : pack_symbols_kernel<false>;
+    const long long tiles = end_tile - first_tile;
+    // Blocks of a tile: two or four while all of them fit the SMs side by side, each has the threads for the scan and no chunk reaches
+    // over a block's end.
+    int tile_blocks = 1;
+    while (tile_blocks < kMaxTileBlocks && a.alone && a.k >= kClusterCoefs && tiles * tile_blocks * 2 <= ctx->sm_count &&
+           TC_TILE_PIXELS / (2 * tile_blocks) * parts >= 128 && a.chunk_pixels <= TC_TILE_PIXELS / (2 * tile_blocks))
+        tile_blocks *= 2;
+    void (*kernel)(EncodeArgs, const uint8_t *, int, long long, unsigned int) =
+        tile_blocks > 1 ? (a.groups == 1 ? pack_symbols_kernel<true, true> : pack_symbols_kernel<false, true>)
+                        : (a.groups == 1 ? pack_symbols_kernel<true, false> : pack_symbols_kernel<false, false>);
     if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSpreadBytes) != cudaSuccess) return TC_ERR_CUDA;
-    const dim3 grid((unsigned int)(end_tile - first_tile)), block(TC_TILE_PIXELS * parts);
+    const dim3 grid((unsigned int)tiles, (unsigned int)tile_blocks), block(TC_TILE_PIXELS / tile_blocks * parts);
     // Up to a block per SM: set up while the kernel before is still at work, with more than half of an SM's shared
     // memory each -- small blocks that arrive early all pile onto the first SMs that have room (960x7x7 x 128, 49
     // blocks: 49 us unchained, 65 chained, 48 chained and spread; 64x56x56 f32 17.2 unchained, 14.9 chained and spread).
     // More blocks than that start when the SMs are free (80x27x19 x 37: 20 us, chained 26).
-    if (a.alone && end_tile - first_tile <= ctx->sm_count)
+    if (tile_blocks > 1)
+        return launch_chained_cluster(tile_blocks, kernel, grid, block, std::max(staging, kSpreadBytes), s, a, sym, parts, first_tile, staging) == cudaSuccess ? TC_OK : TC_ERR_CUDA;
+    if (a.alone && tiles <= ctx->sm_count)
         return launch_chained(true, kernel, grid, block, std::max(staging, kSpreadBytes), s, a, sym, parts, first_tile, staging) == cudaSuccess ? TC_OK : TC_ERR_CUDA;
     kernel<<<grid, block, staging, s>>>(a, sym, parts, first_tile, staging);
     return cudaGetLastError() == cudaSuccess ? TC_OK : TC_ERR_CUDA;

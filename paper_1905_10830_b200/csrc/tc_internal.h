@@ -192,6 +192,23 @@ inline cudaError_t launch_chained(bool early, void (*kernel)(P...), dim3 grid, d
     return err;
 }
 
+// The same, always early, in clusters of `blocks` along the grid's second dimension.
+template <typename... P, typename... A>
+inline cudaError_t launch_chained_cluster(int blocks, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A &&...args)
+{
+    cudaLaunchAttribute attr[2] = {};
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = 1; attr[1].val.clusterDim.y = (unsigned int)blocks; attr[1].val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = s;
+    cfg.attrs = attr; cfg.numAttrs = 2;
+    const cudaError_t err = cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...);
+    if (err != cudaSuccess) cudaGetLastError();
+    return err;
+}
+
 // ---- several tensors in one launch of a persistent kernel ------------------------------------
 constexpr int kListItems = 32;                // tensors of a launch (their arguments are kernel parameters)
 struct ListWork {
