@@ -283,6 +283,7 @@ __device__ __forceinline__ void encode_tiles(const EncodeArgs &a, const Plan &pl
             s_bias[i] = b;
             s_bias_mid[i] = b - (float)(a.modal < 0 ? 0 : a.modal) / (float)(nsym - 1);   // the same, seen from the modal symbol's level
         }
+        for (long long i = (long long)block * kSetupThreads + setup_tid; i < a.other_words; i += (long long)blocks * kSetupThreads) a.other_state[i] = 0ull;
         if (enc_in_smem)
             for (int i = setup_tid; i < enc_entries; i += kSetupThreads) {
                 // per-layer table: (1 << length, code) pairs, so that appending a code to a register is

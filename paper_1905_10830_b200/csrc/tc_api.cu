@@ -389,12 +389,15 @@ tc_status tc_create(tc_ctx **out, int device)
         delete ctx;
         return TC_ERR_CUDA;
     }
-    if (cudaMalloc((void **)&ctx->d_status, 64) != cudaSuccess || cudaMemset(ctx->d_status, 0, 64) != cudaSuccess) {
+    constexpr size_t lookback_words = kEncodeScratchHeader / 8 + kLookbackTiles, fixed_bytes = 64 + 2 * lookback_words * 8;
+    if (cudaMalloc((void **)&ctx->d_status, fixed_bytes) != cudaSuccess || cudaMemset(ctx->d_status, 0, fixed_bytes) != cudaSuccess ||
+        cudaStreamSynchronize(nullptr) != cudaSuccess) {
         cudaGetLastError();
         cudaFree(ctx->d_status);
         delete ctx;
         return TC_ERR_CUDA;
     }
+    for (int i = 0; i < 2; ++i) ctx->lookback[i] = (unsigned long long *)(ctx->d_status + 16) + i * lookback_words;
     // The arena is made here, so that a first call does not stop for it, with room for the workspace of any one tensor (72 MB
     // take no longer to allocate than 8, about 360 us; growing costs a call that and a stop of the device).  Where memory
     // is short it starts smaller, or empty.
@@ -1048,6 +1051,25 @@ tc_status tc_encode(tc_ctx *ctx, const tc_model *m, const tc_codebook *cb, const
     if (n_tiles == 0) {
         TC_CUDA(cudaMemsetAsync(tile_off, 0, sizeof(uint64_t), s));
         return TC_OK;
+    }
+    // The resident-basis encoder finds its look-back state zeroed by the call before: a memset ahead of the kernel cost every call 2 us
+    // of the stream's time (one 32x49x49 map LOOKBACK).  Not in a capture, whose replays would find what the last one left.
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &capture) != cudaSuccess) cudaGetLastError();
+    if (n_tiles <= kLookbackTiles && capture == cudaStreamCaptureStatusNone) {
+        const int now = ctx->lookback_next, other = now ^ 1;
+        EncodeArgs a = encode_args(ctx, m, cb, x, cs.cp, cs.splits, stream_out, capacity, chunk_len, tile_off, debug, ctx->lookback[now],
+                                   nullptr, nullptr, 0);
+        if (resident_encode(ctx, x, a)) {
+            a.other_state = ctx->lookback[other];
+            a.other_words = ctx->lookback_words[other];
+            if ((st = tc_launch_encode_tc(ctx, a, s)) != TC_OK) return st;
+            ctx->last_encode_path = 1;
+            ctx->lookback_words[other] = 0;
+            ctx->lookback_words[now] = (long long)(kEncodeScratchHeader / 8) + n_tiles;
+            ctx->lookback_next = other;
+            return TC_OK;
+        }
     }
     const size_t lookback = (kEncodeScratchHeader + (size_t)n_tiles * sizeof(unsigned long long) + 255) & ~(size_t)255;
     const size_t work = encode_work_bytes(ctx, m, x);

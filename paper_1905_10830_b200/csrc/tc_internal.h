@@ -31,6 +31,10 @@ struct tc_ctx {
     int max_smem_optin = 0;
     unsigned int *d_status = nullptr;     // device status word
     void *scratch = nullptr;              // look-back state, ticket counter
+    // Look-back state of the resident-basis encoder: two arrays in turn, each call clearing what the call before left in the other.
+    unsigned long long *lookback[2] = {};
+    long long lookback_words[2] = {};     // of each, from its start, that may not be zero
+    int lookback_next = 0;
     size_t scratch_bytes = 0;
     void *host_arena = nullptr;           // device staging of tc_roundtrip_host (grown on demand)
     size_t host_arena_bytes = 0;
@@ -124,6 +128,8 @@ struct EncodeArgs {
     bool alone;                       // no other stream of this call (see launch_chained)
     int sms;                          // SMs that a persistent kernel takes at most
     long long clear_words;            // 64-bit words from `ticket` on that the first of several kernels zeroes (0: they are zero)
+    unsigned long long *other_state;  // resident-basis encoder: look-back state that no tile of this call uses,
+    long long other_words;            // and how many words of it to zero for the next
     unsigned int *status;
     unsigned long long *clamped;      // nullable: counts coefficients outside the range
     int emit;                         // 0: symbols only (statistics mode)
@@ -219,6 +225,7 @@ struct ListWork {
 // Deals `sms` blocks (at least one for each tensor) so that the slowest block is done as early as possible.
 void deal_blocks(std::vector<ListWork> &work, int sms);
 
+constexpr long long kLookbackTiles = 32768;   // tiles that a context's two look-back arrays serve (a memset costs a larger call nothing that shows)
 constexpr size_t kEncodeScratchHeader = 64;   // ticket counter, padded; the per-tile look-back words follow
 tc_status tc_encode_with_scratch(tc_ctx *ctx, const tc_model *m, const tc_codebook *cb, const tc_tensor *x, int chunk_pixels,
                                  int splits, void *stream_out, size_t capacity, uint16_t *chunk_len, uint64_t *tile_off,
