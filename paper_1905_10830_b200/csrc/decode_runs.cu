@@ -716,7 +716,7 @@ __global__ void __launch_bounds__(kThreads, 1) decode_runs_kernel(DecodeArgs a, 
 }
 
 // Several tensors in one launch, each with blocks of its own (see encode_tc_list_kernel): 16 layers of a residual network at
-// batch 64 202 -> 162 us.
+// batch 64 199 -> 155 us, nine tensors of up to 50 000 values 62 -> 31.
 struct DecodeList {
     unsigned int first[kListItems + 1];        // block that each item starts at; past the last item 2^32 - 1
     struct { DecodeArgs a; SmemLayout l; } item[kListItems];
@@ -763,12 +763,12 @@ tc_status tc_launch_decode_runs(const tc_ctx *ctx, const DecodeArgs &a, cudaStre
     return cudaGetLastError() == cudaSuccess ? TC_OK : TC_ERR_CUDA;
 }
 
-// us that a tile takes a block: 1.9 with 64 coefficients at 1.1 bits each, 2.2 with 128, 4.9 with 256 (two VLD groups instead of four
-// and eight), 9.3 with 256 at 4.1 bits
+// us that a tile takes a block: 2.0 with 64 coefficients at 1.1 bits each, 2.55 with 128, 5.0 with 256 (two VLD groups instead of four
+// and eight), 10.7 with 256 at 4.1 bits (8 to 42 tiles a block, after the first)
 double tc_decode_runs_tile_us(const DecodeArgs &a)
 {
     const double bits = a.mean_tile_bytes > 0 ? a.mean_tile_bytes * 8.0 / TC_TILE_PIXELS : (double)a.code_bits * a.k;
-    return 1.4 + 0.014 * std::max(0, a.k - 128) + 0.0058 * bits;
+    return 1.42 + 0.011 * std::max(0, a.k - 128) + 0.0075 * bits;
 }
 
 // Decodes tensors that tc_decode_runs_supported takes, all with the same `relu`, on `sms` SMs, as many at a time as there are SMs and

@@ -839,7 +839,8 @@ __global__ void __launch_bounds__(kThreads, 1) encode_tc_kernel(EncodeArgs a, Pl
 
 // Several tensors in one launch, each with blocks of its own.  A block's set-up and first tile take 13 us and a launch on a stream
 // beside others 3 us of host time, so that a list of small tensors was bound by launches and one of large ones paid the set-up of
-// a quarter of the SMs for each: 16 layers of a residual network at batch 64 165 -> 154 us.
+// a quarter of the SMs for each: nine tensors of up to 50 000 values 72 -> 33 us, ten 76 -> 34, the 13 narrower layers of a residual
+// network at batch 64 143 -> 122, all 16 164 -> 148.
 struct EncodeList {
     unsigned int first[kListItems + 1];        // block that each item starts at; past the last item 2^32 - 1
     struct { EncodeArgs a; Plan pl; } item[kListItems];
@@ -945,13 +946,13 @@ static int kernel_class(const EncodeArgs &a, const Plan &pl)
 
 int tc_encode_tc_class(const tc_ctx *ctx, const EncodeArgs &a) { return tc_encode_tc_supported(ctx, a) ? kernel_class(a, make_plan(ctx, a)) : -1; }
 
-// us that a tile takes a block: 1.5 with 64 coefficients at 1.1 bits each, 2.0 with 128, 2.7 with 256, 2.5 with 96 at 2.8 bits, 6.5
-// with 256 at 4.1 (each 5 to 11 tiles a block, after the first)
+// us that a tile takes a block: 1.5 with 64 coefficients at 1.1 bits each, 2.1 with 128, 4.25 with 256, 2.3 with 96 at 2.8 bits, 7.5
+// with 256 at 4.1 (8 to 85 tiles a block, after the first)
 double tc_encode_tc_tile_us(const EncodeArgs &a)
 {
     double bits = 0.0;
     for (int b = 0; b < a.k / 16; ++b) bits += a.blk_bits[b];
-    return 1.1 + 0.0006 * a.k + 0.005 * bits;
+    return std::max(1.2, 0.0118 * a.k) + 0.0043 * bits;
 }
 
 // Encodes tensors of one class (tc_encode_tc_class) on `sms` SMs, as many at a time as there are SMs and places in a list.
