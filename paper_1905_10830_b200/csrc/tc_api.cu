@@ -390,8 +390,7 @@ tc_status tc_create(tc_ctx **out, int device)
         return TC_ERR_CUDA;
     }
     constexpr size_t lookback_words = kEncodeScratchHeader / 8 + kLookbackTiles, fixed_bytes = 64 + 2 * lookback_words * 8;
-    if (cudaMalloc((void **)&ctx->d_status, fixed_bytes) != cudaSuccess || cudaMemset(ctx->d_status, 0, fixed_bytes) != cudaSuccess ||
-        cudaStreamSynchronize(nullptr) != cudaSuccess) {
+    if (cudaMalloc((void **)&ctx->d_status, fixed_bytes) != cudaSuccess || cudaMemset(ctx->d_status, 0, 64) != cudaSuccess) {
         cudaGetLastError();
         cudaFree(ctx->d_status);
         delete ctx;
@@ -1053,7 +1052,7 @@ tc_status tc_encode(tc_ctx *ctx, const tc_model *m, const tc_codebook *cb, const
         return TC_OK;
     }
     // The resident-basis encoder finds its look-back state zeroed by the call before: a memset ahead of the kernel cost every call 2 us
-    // of the stream's time (one 32x49x49 map LOOKBACK).  Not in a capture, whose replays would find what the last one left.
+    // of the stream's time (one 32x48x48 map at 2 bits 10.5 -> 8.8, 256x14x14 x 8 14.4 -> 12.3).  Not in a capture, whose replays would find what the last one left.
     cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(s, &capture) != cudaSuccess) cudaGetLastError();
     if (n_tiles <= kLookbackTiles && capture == cudaStreamCaptureStatusNone) {
@@ -1061,6 +1060,10 @@ tc_status tc_encode(tc_ctx *ctx, const tc_model *m, const tc_codebook *cb, const
         EncodeArgs a = encode_args(ctx, m, cb, x, cs.cp, cs.splits, stream_out, capacity, chunk_len, tile_off, debug, ctx->lookback[now],
                                    nullptr, nullptr, 0);
         if (resident_encode(ctx, x, a)) {
+            if (!ctx->lookback_ready) {                 // here and not at creation: ahead of its first use on the stream that uses it
+                TC_CUDA(cudaMemsetAsync(ctx->lookback[0], 0, (size_t)((char *)ctx->lookback[1] - (char *)ctx->lookback[0]) * 2, s));
+                ctx->lookback_ready = true;
+            }
             a.other_state = ctx->lookback[other];
             a.other_words = ctx->lookback_words[other];
             if ((st = tc_launch_encode_tc(ctx, a, s)) != TC_OK) return st;

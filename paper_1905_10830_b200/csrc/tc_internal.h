@@ -35,6 +35,7 @@ struct tc_ctx {
     unsigned long long *lookback[2] = {};
     long long lookback_words[2] = {};     // of each, from its start, that may not be zero
     int lookback_next = 0;
+    bool lookback_ready = false;          // both have been zeroed once
     size_t scratch_bytes = 0;
     void *host_arena = nullptr;           // device staging of tc_roundtrip_host (grown on demand)
     size_t host_arena_bytes = 0;
@@ -225,7 +226,9 @@ struct ListWork {
 // Deals `sms` blocks (at least one for each tensor) so that the slowest block is done as early as possible.
 void deal_blocks(std::vector<ListWork> &work, int sms);
 
-constexpr long long kLookbackTiles = 32768;   // tiles that a context's two look-back arrays serve (a memset costs a larger call nothing that shows)
+// Tiles that a context's two look-back arrays serve: 128 KB (half a megabyte made tc_create 0.25 ms longer; a larger call's memset is
+// 1 % of it).
+constexpr long long kLookbackTiles = 8192;
 constexpr size_t kEncodeScratchHeader = 64;   // ticket counter, padded; the per-tile look-back words follow
 tc_status tc_encode_with_scratch(tc_ctx *ctx, const tc_model *m, const tc_codebook *cb, const tc_tensor *x, int chunk_pixels,
                                  int splits, void *stream_out, size_t capacity, uint16_t *chunk_len, uint64_t *tile_off,
