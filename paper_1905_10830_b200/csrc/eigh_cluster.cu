@@ -539,14 +539,15 @@ __global__ void __launch_bounds__(kThreads, 1) divide_kernel(const EighArgs args
         }
         __syncthreads();
         // poles at least `gap` apart (the running maximum of d_i - i gap): nothing is deflated, equal eigenvalues are told apart by
-        // rounding instead
+        // rounding instead.  They are multiples of `gap` before that, so that every sum here is exact: half a gap beside one, just below a
+        // power of two, sums rounded to even gave neighbours the same pole, and NaN for eigenvectors (eigenvalues 1 and 2, 64 of them).
         double mine[2];
 #pragma unroll
         for (int q = 0; q < 2; ++q) {
             const int pos = threadIdx.x + q * kThreads;
             if ((pos & ~31) >= n) break;
             const int at = pos & (size - 1), start = max(pos - at, pos & ~31) & 31;    // first lane of this block's in the warp
-            double x = pos < n ? dv.pole[pos] - at * gap : -INFINITY;
+            double x = pos < n ? rint(dv.pole[pos] / gap) * gap - at * gap : -INFINITY;
 #pragma unroll
             for (int d = 1; d < 32; d <<= 1) {
                 const double y = __shfl_up_sync(0xffffffffu, x, d);

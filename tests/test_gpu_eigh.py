@@ -153,9 +153,28 @@ def test_device_eigh_at_the_edges_of_its_kernels(ctx, n):
     assert np.abs(evals - np.linalg.eigvalsh(a)[::-1]).max() <= 1e-13 * max(1, n / 16) * lam.max()
 
 
+def _rotated(lam, seed):
+    q, _ = np.linalg.qr(np.random.default_rng(seed).standard_normal((len(lam), len(lam))))
+    return (q * lam) @ q.T
+
+
 def _clustered(n):
-    q, _ = np.linalg.qr(np.random.default_rng(n).standard_normal((n, n)))
-    return (q * np.r_[np.ones(n // 2), 2 * np.ones(n // 3), np.arange(n - n // 2 - n // 3)]) @ q.T
+    return _rotated(np.r_[np.ones(n // 2), 2 * np.ones(n // 3), np.arange(n - n // 2 - n // 3)], n)
+
+
+# Eigenvalues that agree but for rounding, most of them at or beside a power of two: spreading them apart has to leave no two equal.
+@pytest.mark.parametrize("n", [33, 64, 100, 150, 256, 384, 576])
+@pytest.mark.parametrize("values", [(1.0, 2.0), (2.0, 1.0, 0.0), (-1.0, 1.0), (1.0,), (3.0, 0.0), (1.0 - 2.0 ** -53, 0.25, 2.0 ** -20), (-2.0, -1.0)],
+                         ids=["1 2", "2 1 0", "-1 1", "1", "3 0", "below 1", "-2 -1"])
+def test_device_eigh_of_a_few_values(ctx, n, values):
+    a = _rotated(np.resize(np.array(values), n), n + len(values))
+    a = (a + a.T) / 2
+    evals, evecs, _ = tc.tc_device_eigh(ctx, torch.from_numpy(a).cuda())
+    evals, evecs = evals.cpu().numpy(), evecs.cpu().numpy()
+    norm = max(abs(v) for v in values)                  # bounds as in the next test
+    assert np.abs(evecs @ evecs.T - np.eye(n)).max() <= 2 * n * 2.0 ** -52
+    assert np.abs(evecs @ a @ evecs.T - np.diag(evals)).max() <= 4 * n * 2.0 ** -52 * norm
+    assert np.abs(evals - np.linalg.eigvalsh(a)[::-1]).max() <= 4 * n * 2.0 ** -52 * norm
 
 
 @pytest.mark.parametrize("a", [
