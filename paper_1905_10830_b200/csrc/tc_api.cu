@@ -1407,6 +1407,7 @@ tc_status tc_encode_many(tc_ctx *ctx, const tc_encode_item *items, int32_t n_ite
     tc_status first_error = launch_shared(ctx, classes, class_us, sms, s, n_streams, streams.used, [&](const std::vector<EncodeArgs> &c, int mine, cudaStream_t on) {
         return tc_launch_encode_tc_list(ctx, c, mine, on);
     });
+    if (n_classes) ctx->last_encode_path = 1;
     for (size_t r = 0; r < order.size(); ++r) {
         const int i = order[r];
         const tc_encode_item &it = items[i];
@@ -1418,7 +1419,6 @@ tc_status tc_encode_many(tc_ctx *ctx, const tc_encode_item *items, int32_t n_ite
                                     symbols_bytes[i] && scratch.whole ? scratch.at + symbols_at[i] : nullptr, ws, nullptr, nullptr, list_sms);
         if (st != TC_OK && first_error == TC_OK) first_error = st;
     }
-    if (order.empty()) ctx->last_encode_path = 1;
     if ((st = streams.join()) != TC_OK) return st;
     return first_error;
 }
@@ -1476,6 +1476,7 @@ tc_status tc_decode_many(tc_ctx *ctx, const tc_decode_item *items, int32_t n_ite
     tc_status first_error = launch_shared(ctx, classes, class_us, sms, s, n_streams, streams.used, [&](const std::vector<DecodeArgs> &c, int mine, cudaStream_t on) {
         return tc_launch_decode_runs_list(ctx, c, mine, on);
     });
+    if (n_classes) ctx->last_decode_path = 1;
     for (size_t r = 0; r < order.size(); ++r) {
         const int i = order[r];
         const tc_decode_item &it = items[i];
@@ -1485,7 +1486,6 @@ tc_status tc_decode_many(tc_ctx *ctx, const tc_decode_item *items, int32_t n_ite
                                  list_sms, ctx->many_streams[r % n_streams]);
         if (st != TC_OK && first_error == TC_OK) first_error = st;
     }
-    if (order.empty() && n_classes) ctx->last_decode_path = 1;
     if ((st = streams.join()) != TC_OK) return st;
     return first_error;
 }

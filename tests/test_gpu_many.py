@@ -175,3 +175,22 @@ def test_long_mixed_lists_equal_the_per_tensor_calls(ctx):
             assert np.array_equal(H.stream_words(encs[i]), H.stream_words(alone)) and np.array_equal(H.chunk_len(encs[i]), H.chunk_len(alone))
             assert torch.equal(out, tc.tc_decode(ctx, model, cb, alone, x.shape, torch.bfloat16, relu=relu))
     assert tc.tc_get_status(ctx) == 0
+
+
+# The route that a list reports: that of the item launched last, those that share launches first, and none by an empty tensor.
+def test_the_route_that_a_list_reports(ctx):
+    sides = {}
+    for c, dtype in ((64, torch.bfloat16), (320, torch.bfloat16), (48, torch.float32)):
+        o = H.oracle_side(fm.LayerSpec(c, 8, 8, 0.9, None, 8600 + c), 4, 2 * c // 64 + 3, 2, dtype, False)
+        sides[c] = H.import_model(tc, ctx, o["model"], dtype), tc.tc_codebook_import(ctx, o["lengths"], 4), o["x"].cuda()
+    encs = {c: tc.tc_encode(ctx, *sides[c]) for c in sides}
+    for lst, route in (([64], 1), ([64, -64], 1), ([-320, 64], 1), ([64, 320], 3), ([320, -64], 3), ([64, 48], 0), ([-48], None)):
+        own = tc.tc_create(0)
+        before = tc.tc_last_path(own), tc.tc_last_path(own, True)
+        items = [(sides[abs(c)][0], sides[abs(c)][1], sides[abs(c)][2][:2 if c > 0 else 0].contiguous()) for c in lst]
+        out = tc.tc_encode_many(own, items)
+        got = tc.tc_last_path(own)
+        tc.tc_decode_many(own, [(*i[:2], encs[c] if c > 0 else e, i[2].shape, i[2].dtype) for c, i, e in zip(lst, items, out)])
+        assert (got, tc.tc_last_path(own, True)) == (before if route is None else (route, route)), lst
+        assert tc.tc_get_status(own) == 0
+        own.close()
