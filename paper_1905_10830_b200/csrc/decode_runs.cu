@@ -771,17 +771,17 @@ double tc_decode_runs_tile_us(const DecodeArgs &a)
     return 1.42 + 0.011 * std::max(0, a.k - 128) + 0.0075 * bits;
 }
 
-// Decodes tensors that tc_decode_runs_supported takes, all with the same `relu`, on `sms` SMs, as many at a time as there are SMs and
-// places in a list.
+// Decodes tensors that tc_decode_runs_supported takes, all with the same `relu`, on `sms` SMs, in list_launches launches.
 tc_status tc_launch_decode_runs_list(const tc_ctx *ctx, const std::vector<DecodeArgs> &tensors, int sms, cudaStream_t s)
 {
-    for (size_t at = 0; at < tensors.size();) {
-        const int n = (int)std::min({tensors.size() - at, (size_t)kListItems, (size_t)sms});
+    const size_t launches = list_launches(tensors.size(), sms);
+    for (size_t r = 0; r < launches; ++r) {
+        const int n = (int)((tensors.size() - r + launches - 1) / launches);
         DecodeList list;
         std::vector<ListWork> work(n);
         uint32_t smem = 0;
         for (int i = 0; i < n; ++i) {
-            const DecodeArgs &a = tensors[at + i];
+            const DecodeArgs &a = tensors[r + i * launches];
             list.item[i].a = a;
             list.item[i].l = runs_layout(ctx, a);
             smem = std::max(smem, list.item[i].l.total);
@@ -794,11 +794,10 @@ tc_status tc_launch_decode_runs_list(const tc_ctx *ctx, const std::vector<Decode
             if (i < n) blocks += (unsigned int)work[i].blocks;
         }
         list.first[n] = ~0u;
-        const void *kernel = tensors[at].relu ? (const void *)decode_runs_list_kernel<true> : (const void *)decode_runs_list_kernel<false>;
+        const void *kernel = tensors[r].relu ? (const void *)decode_runs_list_kernel<true> : (const void *)decode_runs_list_kernel<false>;
         if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) { cudaGetLastError(); return TC_ERR_CUDA; }
         void *params[] = {&list};
         if (cudaLaunchKernel(kernel, dim3(blocks), dim3(kThreads), params, smem, s) != cudaSuccess) { cudaGetLastError(); return TC_ERR_CUDA; }
-        at += n;
     }
     return TC_OK;
 }

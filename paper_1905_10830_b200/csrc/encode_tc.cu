@@ -955,17 +955,19 @@ double tc_encode_tc_tile_us(const EncodeArgs &a)
     return std::max(1.2, 0.0118 * a.k) + 0.0043 * bits;
 }
 
-// Encodes tensors of one class (tc_encode_tc_class) on `sms` SMs, as many at a time as there are SMs and places in a list.
+// Encodes tensors of one class (tc_encode_tc_class) on `sms` SMs, in list_launches launches (40 of 128x14x14 x 32 in
+// two of 20 each: 57 us, in one of 32 and one of 8: 62).
 tc_status tc_launch_encode_tc_list(const tc_ctx *ctx, const std::vector<EncodeArgs> &tensors, int sms, cudaStream_t s)
 {
-    for (size_t at = 0; at < tensors.size();) {
-        const int n = (int)std::min({tensors.size() - at, (size_t)kListItems, (size_t)sms});
+    const size_t launches = list_launches(tensors.size(), sms);
+    for (size_t r = 0; r < launches; ++r) {
+        const int n = (int)((tensors.size() - r + launches - 1) / launches);
         EncodeList list;
         std::vector<ListWork> work(n);
         uint32_t smem = 0;
         int which = 0;
         for (int i = 0; i < n; ++i) {
-            const EncodeArgs &a = tensors[at + i];
+            const EncodeArgs &a = tensors[r + i * launches];
             list.item[i].a = a;
             list.item[i].pl = make_plan(ctx, a);
             which = kernel_class(a, list.item[i].pl);
@@ -986,7 +988,6 @@ tc_status tc_launch_encode_tc_list(const tc_ctx *ctx, const std::vector<EncodeAr
         void *params[] = {&list};
         // cooperative, as for one tensor: the blocks of a tensor look back at one another
         if (cudaLaunchCooperativeKernel(kernel, dim3(blocks), dim3(kThreads), params, smem, s) != cudaSuccess) { cudaGetLastError(); return TC_ERR_CUDA; }
-        at += n;
     }
     return TC_OK;
 }

@@ -1222,38 +1222,6 @@ static tc_status ensure_many_streams(tc_ctx *ctx)
 
 }  // extern "C"
 
-void deal_blocks(std::vector<ListWork> &work, int sms)
-{
-    // shortest time for which the blocks that the tensors then need are there; less than a tile's is not to be had
-    double least = 0.0, most = 0.0;
-    for (const ListWork &w : work) { least = std::max(least, w.tile_us); most = std::max(most, w.tile_us * (double)w.tiles); }
-    auto blocks_for = [](const ListWork &w, double us) {
-        const long long each = std::max(1ll, (long long)(us / w.tile_us));
-        return (int)std::min((w.tiles + each - 1) / each, 1ll << 20);
-    };
-    auto fits = [&](double us) {
-        long long sum = 0;
-        for (const ListWork &w : work) sum += blocks_for(w, us);
-        return sum <= sms;
-    };
-    if (!fits(least)) {
-        for (int i = 0; i < 24; ++i) {
-            const double us = 0.5 * (least + most);
-            if (fits(us)) most = us; else least = us;
-        }
-        least = most * (1.0 + 1e-9);                   // (`most` fits: one block each, for as many tensors as blocks)
-    }
-    for (ListWork &w : work) w.blocks = std::max(1, blocks_for(w, least));
-}
-
-// SMs for the tensors of a list that share a launch (`shared_us`: the work of all, in us of one SM), beside `others_us` of tensors with
-// kernels of their own: by their shares, at least eight for the others.
-static int shared_sms(int sm_count, double shared_us, double others_us)
-{
-    if (others_us <= 0.0) return sm_count;
-    return std::max(sm_count / 4, std::min(sm_count - 8, (int)(sm_count * shared_us / (shared_us + others_us))));
-}
-
 // us of one SM that a wide tensor takes, entropy coder and product (25 tiles of 512 channels at 4 bits: 960 to encode, 885 to decode).
 static double wide_us(long long pixels, int k) { return 0.075 * k * (double)((pixels + TC_TILE_PIXELS - 1) / TC_TILE_PIXELS); }
 
@@ -1292,20 +1260,17 @@ struct ListStreams {
     }
 };
 
-// Tensors that share launches, by kernel: each kernel gets SMs by its share of the work.  The first runs on the caller's stream, the
-// others on the list's `n_streams` streams from `first_stream` on.
+// Tensors that share launches, by kernel, each kernel on its SMs.  The first runs on the caller's stream, the others on the list's
+// `n_streams` streams from `first_stream` on.
 template <typename Args, typename Launch>
-static tc_status launch_shared(tc_ctx *ctx, const std::vector<std::vector<Args>> &classes, const std::vector<double> &us, int sms,
-                               cudaStream_t s, int first_stream, int n_streams, Launch launch)
+static tc_status launch_shared(tc_ctx *ctx, const std::vector<std::vector<Args>> &classes, const std::vector<int> &sms, cudaStream_t s,
+                               int first_stream, int n_streams, Launch launch)
 {
-    double all = 0.0;
-    for (double u : us) all += u;
     tc_status first_error = TC_OK;
     int on = 0;
     for (size_t j = 0; j < classes.size(); ++j) {
         if (classes[j].empty()) continue;
-        const int mine = std::min(sms, std::max(1, (int)(sms * us[j] / all)));
-        const tc_status st = launch(classes[j], mine, on == 0 ? s : ctx->many_streams[(first_stream + on - 1) % n_streams]);
+        const tc_status st = launch(classes[j], sms[j], on == 0 ? s : ctx->many_streams[(first_stream + on - 1) % n_streams]);
         if (st != TC_OK && first_error == TC_OK) first_error = st;
         ++on;
     }
@@ -1366,9 +1331,9 @@ tc_status tc_encode_many(tc_ctx *ctx, const tc_encode_item *items, int32_t n_ite
     // the resident-basis encoder takes its tensors in a launch per kernel, the others have kernels of their own
     std::vector<EncodeArgs> args(n_items);
     std::vector<int> kind(n_items, -1);
-    std::vector<std::vector<EncodeArgs>> classes(8);
-    std::vector<double> class_us(8, 0.0);
-    double shared_us = 0.0, others_us = 0.0, others = 0.0;
+    std::vector<std::vector<int>> members(8);
+    std::vector<std::vector<ListWork>> tiles(8);
+    double others_us = 0.0, others = 0.0;
     std::vector<int> order;
     for (int i : by_descending_work(n_items, work)) {
         const tc_encode_item &it = items[i];
@@ -1378,9 +1343,8 @@ tc_status tc_encode_many(tc_ctx *ctx, const tc_encode_item *items, int32_t n_ite
             if (resident_encode(ctx, it.x, args[i])) kind[i] = tc_encode_tc_class(ctx, args[i]);
         }
         if (kind[i] >= 0) {
-            const double us = (double)args[i].n_tiles * tc_encode_tc_tile_us(args[i]);
-            class_us[kind[i]] += us;
-            shared_us += us;
+            members[kind[i]].push_back(i);
+            tiles[kind[i]].push_back({args[i].n_tiles, tc_encode_tc_tile_us(args[i]), 0});
         } else {
             order.push_back(i);
             others += work[i];
@@ -1389,22 +1353,27 @@ tc_status tc_encode_many(tc_ctx *ctx, const tc_encode_item *items, int32_t n_ite
         }
     }
     const int n_streams = std::min(kManyStreams, (int)order.size());
+    const int n_own = (int)std::count_if(order.begin(), order.end(), [&](int i) { return work[i] > 0.0; });
     tc_status st;
     CallScratch scratch;
     if ((st = call_scratch(ctx, lookback_total, stream_workspaces(order, n_streams, symbols_bytes, lookback_total, symbols_at), s, &scratch)) != TC_OK) return st;
-    for (int i = 0; i < n_items; ++i)
-        if (kind[i] >= 0) {
+    std::vector<std::vector<EncodeArgs>> classes(8);
+    int n_classes = 0;
+    for (size_t j = 0; j < classes.size(); ++j) {
+        n_classes += !members[j].empty();
+        for (int i : members[j]) {
             args[i].ticket = (unsigned int *)(scratch.at + lookback_at[i]);
             args[i].tile_state = (unsigned long long *)(scratch.at + lookback_at[i] + kEncodeScratchHeader);
-            classes[kind[i]].push_back(args[i]);
+            classes[j].push_back(args[i]);
         }
-    const int n_classes = (int)std::count_if(classes.begin(), classes.end(), [](const auto &c) { return !c.empty(); });
-    const int sms = shared_sms(ctx->sm_count, shared_us, others_us);
+    }
+    std::vector<int> sms;
+    const int rest = deal_list(tiles, others_us, n_own, ctx->sm_count, sms);
     // one clear for the look-back state of all items, then the items fan out over the streams
     TC_CUDA(cudaMemsetAsync(scratch.at, 0, lookback_total, s));
     ListStreams streams{ctx, s};
     if ((st = streams.fork(std::min(kManyStreams, n_streams + std::max(0, n_classes - 1)))) != TC_OK) return st;
-    tc_status first_error = launch_shared(ctx, classes, class_us, sms, s, n_streams, streams.used, [&](const std::vector<EncodeArgs> &c, int mine, cudaStream_t on) {
+    tc_status first_error = launch_shared(ctx, classes, sms, s, n_streams, streams.used, [&](const std::vector<EncodeArgs> &c, int mine, cudaStream_t on) {
         return tc_launch_encode_tc_list(ctx, c, mine, on);
     });
     if (n_classes) ctx->last_encode_path = 1;
@@ -1412,7 +1381,7 @@ tc_status tc_encode_many(tc_ctx *ctx, const tc_encode_item *items, int32_t n_ite
         const int i = order[r];
         const tc_encode_item &it = items[i];
         cudaStream_t ws = ctx->many_streams[r % n_streams];
-        const int list_sms = n_classes ? ctx->sm_count - sms : list_share(ctx->sm_count, n_streams, others, work[i]);
+        const int list_sms = n_classes ? rest : list_share(ctx->sm_count, n_streams, others, work[i]);
         if (work[i] == 0.0) { if (cudaMemsetAsync(it.tile_off, 0, sizeof(uint64_t), ws) != cudaSuccess && first_error == TC_OK) first_error = TC_ERR_CUDA; continue; }
         st = tc_encode_with_scratch(ctx, it.model, it.codebook, it.x, shape[i].cp, shape[i].splits, it.stream_out, it.capacity,
                                     it.chunk_len, it.tile_off, nullptr, scratch.at + lookback_at[i],
@@ -1445,8 +1414,8 @@ tc_status tc_decode_many(tc_ctx *ctx, const tc_decode_item *items, int32_t n_ite
         work[i] = (double)pixels * it.x_hat->c;
     }
     std::vector<std::vector<DecodeArgs>> classes(2);    // without and with a non-linearity behind the decoder
-    std::vector<double> class_us(2, 0.0);
-    double shared_us = 0.0, others_us = 0.0, others = 0.0;
+    std::vector<std::vector<ListWork>> tiles(2);
+    double others_us = 0.0, others = 0.0;
     std::vector<int> order;
     for (int i : by_descending_work(n_items, work)) {
         const tc_decode_item &it = items[i];
@@ -1455,10 +1424,8 @@ tc_status tc_decode_many(tc_ctx *ctx, const tc_decode_item *items, int32_t n_ite
         resolve_chunks(it.params, it.model->k, it.codebook->max_len, &cs);
         const DecodeArgs a = decode_args(ctx, it.model, it.codebook, it.stream, it.stream_bytes, it.chunk_len, it.tile_off, it.params, cs, it.x_hat, 0);
         if (runs_decode(ctx, it.x_hat, a)) {
-            const double us = (double)a.n_tiles * tc_decode_runs_tile_us(a);
             classes[a.relu].push_back(a);
-            class_us[a.relu] += us;
-            shared_us += us;
+            tiles[a.relu].push_back({a.n_tiles, tc_decode_runs_tile_us(a), 0});
             symbols_bytes[i] = 0;
         } else {
             order.push_back(i);
@@ -1470,17 +1437,18 @@ tc_status tc_decode_many(tc_ctx *ctx, const tc_decode_item *items, int32_t n_ite
     const int n_streams = std::min(kManyStreams, (int)order.size()), n_classes = (int)!classes[0].empty() + (int)!classes[1].empty();
     CallScratch scratch;
     if ((st = call_scratch(ctx, 0, stream_workspaces(order, n_streams, symbols_bytes, 0, symbols_at), s, &scratch)) != TC_OK) return st;
-    const int sms = shared_sms(ctx->sm_count, shared_us, others_us);
+    std::vector<int> sms;
+    const int rest = deal_list(tiles, others_us, (int)order.size(), ctx->sm_count, sms);
     ListStreams streams{ctx, s};
     if ((st = streams.fork(std::min(kManyStreams, n_streams + std::max(0, n_classes - 1)))) != TC_OK) return st;
-    tc_status first_error = launch_shared(ctx, classes, class_us, sms, s, n_streams, streams.used, [&](const std::vector<DecodeArgs> &c, int mine, cudaStream_t on) {
+    tc_status first_error = launch_shared(ctx, classes, sms, s, n_streams, streams.used, [&](const std::vector<DecodeArgs> &c, int mine, cudaStream_t on) {
         return tc_launch_decode_runs_list(ctx, c, mine, on);
     });
     if (n_classes) ctx->last_decode_path = 1;
     for (size_t r = 0; r < order.size(); ++r) {
         const int i = order[r];
         const tc_decode_item &it = items[i];
-        const int list_sms = n_classes ? ctx->sm_count - sms : list_share(ctx->sm_count, n_streams, others, work[i]);
+        const int list_sms = n_classes ? rest : list_share(ctx->sm_count, n_streams, others, work[i]);
         st = decode_with_scratch(ctx, it.model, it.codebook, it.stream, it.stream_bytes, it.chunk_len, it.tile_off, it.params,
                                  it.x_hat, symbols_bytes[i] && scratch.at ? (uint8_t *)scratch.at + symbols_at[i] : nullptr,
                                  list_sms, ctx->many_streams[r % n_streams]);

@@ -223,8 +223,13 @@ struct ListWork {
     double tile_us;                           // what a tile takes a block, after its first
     int blocks;
 };
-// Deals `sms` blocks (at least one for each tensor) so that the slowest block is done as early as possible.
+// Deals `sms` blocks (at least one for each tensor; `sms` are no fewer) so that the slowest block is done as early as possible.
 void deal_blocks(std::vector<ListWork> &work, int sms);
+// Launches that `tensors` of one kernel take on `sms` SMs: tensors r, r + launches, ... go together.
+int list_launches(size_t tensors, int sms);
+// Deals the device to the kernels of a list that run at the same time: classes[j] share launches (tensors in descending order of
+// work), `others` tensors of `others_us` us of one SM have kernels of their own.  sms[j] = SMs of a class; returns those of the others.
+int deal_list(const std::vector<std::vector<ListWork>> &classes, double others_us, int others, int sm_count, std::vector<int> &sms);
 
 // Tiles that a context's two look-back arrays serve: 128 KB (half a megabyte made tc_create 0.25 ms longer; a larger call's memset is
 // 1 % of it).
