@@ -205,6 +205,9 @@ struct BitReader {
     }
 };
 
+// Rows leave in pieces of four pixels or eight, not pixel by pixel.
+__host__ __device__ inline bool vector_stores(const DecodeArgs &a) { return (a.hw & 3) == 0 && ((uintptr_t)a.xhat & 7u) == 0 && a.hw < (1 << 29); }
+
 // `block` of `blocks` that share the tensor's tiles.
 template <bool kRelu>
 __device__ __forceinline__ void decode_tiles(const DecodeArgs &a, const SmemLayout &L, unsigned int block, unsigned int blocks)
@@ -513,7 +516,7 @@ __device__ __forceinline__ void decode_tiles(const DecodeArgs &a, const SmemLayo
         // With H*W a multiple of 4 every aligned group of four pixels lies inside one image and is
         // 8-byte aligned (given an 8-byte aligned tensor); otherwise pixels are stored one by one.
         // (and eight rows of a map fit 32 bits: with the step in 64 bits 256x14x14 x 4096 took 236 us instead of 221)
-        const bool vec = (a.hw & 3) == 0 && ((uintptr_t)a.xhat & 7u) == 0 && a.hw < (1 << 29);
+        const bool vec = vector_stores(a);
         const long long img_stride = (long long)a.c * a.hw;
         const int ch_base = blk * 128 + wq * 32;            // first channel of this warp
         // Transpose block: row = channel (64 bytes = 32 pixels); the four 16-byte pieces of a row are exchanged
@@ -764,9 +767,10 @@ tc_status tc_launch_decode_runs(const tc_ctx *ctx, const DecodeArgs &a, cudaStre
 }
 
 // us that a tile takes a block: 2.0 with 64 coefficients at 1.1 bits each, 2.55 with 128, 5.0 with 256 (two VLD groups instead of four
-// and eight), 10.7 with 256 at 4.1 bits (8 to 42 tiles a block, after the first)
+// and eight), 10.7 with 256 at 4.1 bits (8 to 42 tiles a block, after the first); 7.0 with 32 and 43 with 256 where pixels are stored one by one
 double tc_decode_runs_tile_us(const DecodeArgs &a)
 {
+    if (!vector_stores(a)) return 2.0 + 0.165 * a.c;
     const double bits = a.mean_tile_bytes > 0 ? a.mean_tile_bytes * 8.0 / TC_TILE_PIXELS : (double)a.code_bits * a.k;
     return 1.42 + 0.011 * std::max(0, a.k - 128) + 0.0075 * bits;
 }

@@ -21,13 +21,21 @@ long long blocks_for(const ListWork &w, double us)
     return (w.tiles + each - 1) / each;
 }
 
+// us of one SM that the tensors take
+double all_us(const std::vector<ListWork> &work)
+{
+    double us = 0.0;
+    for (const ListWork &w : work) us += w.tile_us * (double)w.tiles;
+    return us;
+}
+
 // The least time (to 1 %) from `us` on for which fits(us); it fits some time.
 template <typename Fits>
 double least_time(double us, Fits fits)
 {
     if (fits(us)) return us;
-    double least = us, most = 2.0 * us;
-    while (!fits(most) && most < 1e12) { least = most; most *= 2.0; }
+    double least = us, most = 1.25 * us;
+    while (!fits(most) && most < 1e12) { least = most; most *= 1.5; }
     while (most - least > 0.01 * least) {
         const double mid = 0.5 * (least + most);
         if (fits(mid)) most = mid; else least = mid;
@@ -39,7 +47,7 @@ double least_time(double us, Fits fits)
 
 void deal_blocks(std::vector<ListWork> &work, int sms)
 {
-    const double us = least_time(13.0, [&](double t) {
+    const double us = least_time(std::max(13.0, all_us(work) / sms), [&](double t) {
         long long sum = 0;
         for (const ListWork &w : work) sum += blocks_for(w, t);
         return sum <= sms;
@@ -82,10 +90,12 @@ int deal_list(const std::vector<std::vector<ListWork>> &classes, double others_u
     // All done at the same time.  Beside others the shared launches have up to a quarter of the SMs all the same, which they leave early:
     // entropy coders fill those, while a launch on few SMs that starts late ends late (six layers of 128x28x28 x 64 with a table per channel and three
     // of 256x14x14 x 32, decode: 127 us with 37 SMs, 161 with 6).
-    double us = least_time(13.0, [&](double t) {
+    double total = others_us;
+    for (const auto &c : classes) total += all_us(c);
+    double us = least_time(std::max(13.0, total / sm_count), [&](double t) {
         return of_all(t) + std::max(others > 0 ? std::ceil(others_us / t) : 0.0, (double)(sm_count - shared)) <= sm_count;
     });
-    if (others > 0) us = std::min(us, least_time(13.0, [&](double t) { return of_all(t) <= sm_count / 4; }));
+    if (others > 0) us = std::min(us, least_time(std::max(13.0, 4.0 * (total - others_us) / sm_count), [&](double t) { return t >= us || of_all(t) <= sm_count / 4; }));
     int left = sm_count, largest = -1;
     for (size_t j = 0; j < classes.size(); ++j) {
         if (classes[j].empty()) continue;
@@ -96,6 +106,22 @@ int deal_list(const std::vector<std::vector<ListWork>> &classes, double others_u
     if (others > 0) return std::max(1, left);
     sms[largest] += std::max(0, left);
     return 0;
+}
+
+// us of one SM that a tensor with kernels of its own takes a tile where there are many (`bits` of code a pixel), within a third of
+// what 100 000 pixels took over 32 to 1024 channels: encodes on the tensor cores 6.0 with 32, 10.3 with 128, 24 with 320, 50 with 576, 96 with
+// 960; decodes 17 with 320, 36 with 576, 70 with 960; the bit width adds 2 to 20 %, a table per channel a quarter.  fp32 kernels 8.2 with 24, 22 with
+// 72, 104 with 200; exact ones 38 with 64, 130 with 128, 420 with 256, 1250 with 512.
+extern "C" double tc_list_own_us(long long tiles, int c, int k, double bits, bool per_channel, bool tensor_cores, bool exact, bool encode)
+{
+    double us;
+    if (exact) us = 0.0047 * c * k + 0.4 * k;
+    else if (!tensor_cores) us = 4.0 + 0.1 * k + 0.0019 * c * k;
+    else {
+        us = encode ? 2.0 + k * (0.045 + 5.5e-5 * c) : k * (0.043 + 3e-5 * c);
+        us = (us + 0.002 * bits) * (per_channel ? 1.25 : 1.0);
+    }
+    return us * (double)tiles;
 }
 
 // For the tests: `classes` lists of n_tensors[j] tensors each, one after the other in `tiles` and `tile_us`.

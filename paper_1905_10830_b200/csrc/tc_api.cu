@@ -1,6 +1,7 @@
 // Host side of the C ABI declared in include/tc.h: handles, argument checks, table building
 // and kernel launches.  No step of the coding path runs on the host.
 #include <algorithm>
+#include <numeric>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -1222,8 +1223,13 @@ static tc_status ensure_many_streams(tc_ctx *ctx)
 
 }  // extern "C"
 
-// us of one SM that a wide tensor takes, entropy coder and product (25 tiles of 512 channels at 4 bits: 960 to encode, 885 to decode).
-static double wide_us(long long pixels, int k) { return 0.075 * k * (double)((pixels + TC_TILE_PIXELS - 1) / TC_TILE_PIXELS); }
+// us of one SM of a tensor of a list that does not share launches.
+template <typename Args>
+static double own_us(const tc_ctx *ctx, const tc_tensor *x, const Args &a, double bits, bool encode)
+{
+    const bool bf16 = x->dtype == TC_BF16 && ctx->force_exact != 1;
+    return tc_list_own_us(a.n_tiles, a.c, a.k, bits, a.groups != 1, bf16 && a.c % 16 == 0 && a.k % 16 == 0, !bf16 || a.c % 2 != 0, encode);
+}
 
 // SMs that the persistent kernels of tensor i of those take that have launches of their own: a quarter of them, more where the tensor
 // is more than that of the list's work.  A kernel's first tile costs a block 10 to 15 us (basis, tensor memory, first copies) and a
@@ -1348,7 +1354,7 @@ tc_status tc_encode_many(tc_ctx *ctx, const tc_encode_item *items, int32_t n_ite
         } else {
             order.push_back(i);
             others += work[i];
-            others_us += wide_us((long long)it.x->n * it.x->h * it.x->w, it.model->k);
+            if (work[i] > 0.0) others_us += own_us(ctx, it.x, args[i], std::accumulate(it.model->blk_bits.begin(), it.model->blk_bits.end(), 0.0), true);
             symbols_bytes[i] = work[i] > 0.0 ? encode_work_bytes(ctx, it.model, it.x) : 0;
         }
     }
@@ -1430,7 +1436,7 @@ tc_status tc_decode_many(tc_ctx *ctx, const tc_decode_item *items, int32_t n_ite
         } else {
             order.push_back(i);
             others += work[i];
-            others_us += wide_us(a.pixels, a.k);
+            others_us += own_us(ctx, it.x_hat, a, (double)a.code_bits * a.k, false);
         }
     }
     tc_status st;

@@ -230,6 +230,7 @@ int list_launches(size_t tensors, int sms);
 // Deals the device to the kernels of a list that run at the same time: classes[j] share launches (tensors in descending order of
 // work), `others` tensors of `others_us` us of one SM have kernels of their own.  sms[j] = SMs of a class; returns those of the others.
 int deal_list(const std::vector<std::vector<ListWork>> &classes, double others_us, int others, int sm_count, std::vector<int> &sms);
+extern "C" double tc_list_own_us(long long tiles, int c, int k, double bits, bool per_channel, bool tensor_cores, bool exact, bool encode);
 
 // Tiles that a context's two look-back arrays serve: 128 KB (half a megabyte made tc_create 0.25 ms longer; a larger call's memset is
 // 1 % of it).
