@@ -99,6 +99,9 @@ tc_status tc_get_status(tc_ctx *ctx, void *cuda_stream);
  * passes over runs of the zero level; with `on` == 4 calls run as if the memory for their workspaces could
  * not be had, on the kernels that need none; 0 restores the default. */
 void tc_force_exact_path(tc_ctx *ctx, int on);
+/* Validation switch: with `on` != 0 the device eigensolver (fits and tc_device_eigh) takes the one-sided Jacobi method for matrices
+ * of any size, as on a device that cannot hold the clusters of the other one; 0 restores the default. */
+void tc_force_jacobi(tc_ctx *ctx, int on);
 /* Which kernels the last tc_encode (decode == 0) or tc_decode (decode != 0) of this context
  * launched: 0 = fp64 kernels, 1 = tensor-core kernels for up to 256 channels (basis resident on the SM; decodes
  * with per-channel code tables: the tiled product, where its workspace could be had), 2 = fp32 kernels,

@@ -65,7 +65,7 @@ class _StatsOut(C.Structure):
                 ("zero_fraction", C.c_double), ("energy_ratio_90", C.c_double)]
 
 
-EXPORTS = ["tc_create", "tc_destroy", "tc_status_string", "tc_get_status", "tc_force_exact_path", "tc_last_path", "tc_fit_pca",
+EXPORTS = ["tc_create", "tc_destroy", "tc_status_string", "tc_get_status", "tc_force_exact_path", "tc_force_jacobi", "tc_last_path", "tc_fit_pca",
            "tc_model_import", "tc_model_export", "tc_model_free", "tc_build_codebook",
            "tc_codebook_import", "tc_codebook_export", "tc_codebook_free",
            "tc_host_huffman_lengths", "tc_host_eigh", "tc_device_eigh", "tc_encode_bound", "tc_encode", "tc_encode_noalloc", "tc_decode", "tc_encode_many", "tc_decode_many", "tc_roundtrip_host",
@@ -97,6 +97,8 @@ def load_library() -> C.CDLL:
         lib.tc_get_status.argtypes = [vp, vp]
         lib.tc_force_exact_path.argtypes = [vp, C.c_int]
         lib.tc_force_exact_path.restype = None
+        lib.tc_force_jacobi.argtypes = [vp, C.c_int]
+        lib.tc_force_jacobi.restype = None
         lib.tc_last_path.argtypes = [vp, C.c_int]
         lib.tc_fit_pca.argtypes = [vp, P(_Tensor), P(_FitParams), P(vp), vp]
         lib.tc_model_import.argtypes = [vp, P(_ModelDesc), P(vp)]
@@ -244,6 +246,11 @@ def tc_force_exact_path(ctx: Context, on) -> None:
     resident-basis tensor-core kernels (validation of the streaming kernels); 3: they skip the run-skipping
     decoder; 4: calls run as if the memory for their workspaces could not be had."""
     load_library().tc_force_exact_path(ctx.ptr, int(on))
+
+
+def tc_force_jacobi(ctx: Context, on) -> None:
+    """Validation switch: the device eigensolver takes the Jacobi method for matrices of any size."""
+    load_library().tc_force_jacobi(ctx.ptr, int(on))
 
 
 def tc_last_path(ctx: Context, decode: bool = False) -> int:

@@ -546,16 +546,16 @@ static tc_status launch_jacobi(const double *a, int c, void *work, double **vt, 
 
 // a: [c][c] symmetric, DEVICE, left untouched.  evals [c + 1], evecs [c][c] (row j = eigenvector of
 // evals[j]), DEVICE; evals[c] is the outcome, for tc_eigh_outcome.  `work`: tc_eigh_device_workspace_bytes(c) bytes, DEVICE.
-// Only queues work.  Reduction and division wherever the matrix fits a cluster's shared memory (576 rows), Jacobi beyond that and on
-// devices that cannot hold the cluster.  tc_device_eigh on graded spectra, Jacobi against cluster: 64 rows 0.50 and 0.23 ms, 128 rows
+// Only queues work.  Reduction and division wherever the matrix fits a cluster's shared memory (576 rows), Jacobi beyond that, on
+// devices that cannot hold the cluster and where `jacobi` asks for it.  tc_device_eigh on graded spectra, Jacobi against cluster: 64 rows 0.50 and 0.23 ms, 128 rows
 // 1.5 and 0.42, 256 rows 5.9 and 1.3, 384 rows 12.9 and 1.8, 576 rows 20.6 and 3.8 (a third of a millisecond of it allocation);
 // orthogonality 1.4e-14 to 4.4e-14 and 1.2e-15 to 2.3e-15.
-tc_status tc_eigh_device(const double *a, int c, double *evals, double *evecs, void *work, cudaStream_t s)
+tc_status tc_eigh_device(const double *a, int c, double *evals, double *evecs, void *work, bool jacobi, cudaStream_t s)
 {
     if (c < 1 || c > TC_MAX_C) return TC_ERR_INVALID_ARG;
     double *vt, *lambda;
     int *outcome;
-    tc_status st = tc_launch_eigh_cluster(a, c, work, &vt, &lambda, &outcome, s);
+    tc_status st = jacobi ? TC_ERR_UNSUPPORTED : tc_launch_eigh_cluster(a, c, work, &vt, &lambda, &outcome, s);
     if (st == TC_ERR_UNSUPPORTED) st = launch_jacobi(a, c, work, &vt, &lambda, &outcome, s);
     if (st != TC_OK) return st;
     order_sign_kernel<<<c, kPairThreads, 0, s>>>(vt, lambda, c, outcome, evals, evecs);

@@ -431,6 +431,11 @@ void tc_destroy(tc_ctx *ctx)
     delete ctx;
 }
 
+void tc_force_jacobi(tc_ctx *ctx, int on)
+{
+    if (ctx) ctx->force_jacobi = on != 0;
+}
+
 void tc_force_exact_path(tc_ctx *ctx, int on)
 {
     if (!ctx) return;
@@ -601,7 +606,7 @@ static tc_status finish_fit(tc_ctx *ctx, const tc_tensor *range_maps, const tc_f
         TC_CUDA(cudaMemcpyAsync(d_eig, eig.data(), sizeof(double) * c, cudaMemcpyHostToDevice, s));
         TC_CUDA(cudaStreamSynchronize(s));
     } else {
-        if ((st = tc_eigh_device(d_cov, c, d_eig, d_basis, d_work, s)) != TC_OK) return st;
+        if ((st = tc_eigh_device(d_cov, c, d_eig, d_basis, d_work, ctx->force_jacobi, s)) != TC_OK) return st;
     }
     if ((st = tc_launch_round_basis(d_basis, c, params->basis_dtype, d_scale, s)) != TC_OK) return st;
 
@@ -802,7 +807,7 @@ tc_status tc_device_eigh(tc_ctx *ctx, const double *a, int32_t n, double *evals,
     TC_CUDA(cudaMalloc((void **)&work, bytes + ((size_t)n + 1) * sizeof(double)));
     double *const d_eig = (double *)(work + bytes);
     double outcome = 0.0;
-    tc_status st = tc_eigh_device(a, n, d_eig, evecs, work, s);
+    tc_status st = tc_eigh_device(a, n, d_eig, evecs, work, ctx->force_jacobi, s);
     if (st == TC_OK && (cudaMemcpyAsync(evals, d_eig, (size_t)n * sizeof(double), cudaMemcpyDeviceToDevice, s) != cudaSuccess ||
                         cudaMemcpyAsync(&outcome, d_eig + n, sizeof(double), cudaMemcpyDeviceToHost, s) != cudaSuccess))
         st = TC_ERR_CUDA;

@@ -50,6 +50,7 @@ struct tc_ctx {
     cudaEvent_t many_fork = nullptr, many_join[kManyStreams] = {};
     int force_exact = 0;                  // 1: route every tensor through the fp64 kernels; 2: skip the resident-basis kernels; 3: skip the run-skipping decoder
     bool no_workspace = false;            // calls run as if no memory could be had for their workspaces
+    bool force_jacobi = false;            // the eigensolver for devices that cannot hold the clusters
     int last_encode_path = 0;             // 0 = fp64 kernels, 1 = tensor-core kernels (resident basis), 2 = fp32 kernels, 3 = tensor-core kernels (streamed basis)
     int last_decode_path = 0;
     tc_codebook *stats_cb[9] = {};        // tc_stats: fixed-length code tables (one per bit width) for streams coded without a codebook
@@ -310,7 +311,7 @@ tc_status tc_launch_moments_to_cov(const double *sum, const double *outer, long 
                                    cudaStream_t s);
 tc_status tc_launch_scale_mirror(double *cov, int c, double denom, cudaStream_t s);
 size_t tc_eigh_device_workspace_bytes(int c);
-tc_status tc_eigh_device(const double *a, int c, double *evals, double *evecs, void *work, cudaStream_t s);
+tc_status tc_eigh_device(const double *a, int c, double *evals, double *evecs, void *work, bool jacobi, cudaStream_t s);
 tc_status tc_eigh_outcome(double outcome);
 size_t tc_eigh_cluster_workspace_bytes(int n);   // eigh_cluster.cu
 tc_status tc_launch_eigh_cluster(const double *a, int n, void *work, double **vt, double **lambda, int **state, cudaStream_t s);

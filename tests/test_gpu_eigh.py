@@ -124,8 +124,16 @@ def test_online_fit_finishes_on_the_device(ctx):
         assert np.isclose(online["lo"], other["lo"], rtol=1e-6, atol=1e-6) and np.isclose(online["step"], other["step"], rtol=1e-6)
 
 
+@pytest.fixture(params=[1])
+def jacobi(ctx, request):
+    tc.tc_force_jacobi(ctx, request.param)
+    yield
+    tc.tc_force_jacobi(ctx, 0)
+
+
+@pytest.mark.parametrize("jacobi", [0, 1], indirect=True, ids=["division", "jacobi"])
 @pytest.mark.parametrize("n", [2, 3, 5])
-def test_rotations_are_orthogonal_to_fp64(ctx, n):
+def test_rotations_are_orthogonal_to_fp64(ctx, jacobi, n):
     # Few columns, angles of every size: cosine and tangent of a rotation start from fp32 (1e-7), and a rotation that is
     # orthogonal to that only would leave 1e-7 |A| beside the diagonal.  Inner products stop at 8 sqrt(16) eps of the
     # norms, which (1.25 + 1) |A|_F turns into at most 2.25 times that; as much again for the rounding of the sweeps.
@@ -138,6 +146,30 @@ def test_rotations_are_orthogonal_to_fp64(ctx, n):
         bound = 4.5 * 8 * 4 * 2.0 ** -52
         assert np.abs(evecs @ evecs.T - np.eye(n)).max() <= bound
         assert np.abs(evecs @ a @ evecs.T - np.diag(evals)).max() <= bound * np.linalg.norm(a)
+
+
+# The method of devices that cannot hold the clusters, at the first and the last size of each of its kernels.
+@pytest.mark.parametrize("n", [1, 64, 65, 128, 129, 256, 257, 384, 385, 512, 513, 576])
+def test_jacobi_at_the_edges_of_its_kernels(ctx, jacobi, n):
+    a, lam, _ = _sym(n, 5000 + n, 0.97)
+    a = (a + a.T) / 2
+    evals, evecs, sweeps = tc.tc_device_eigh(ctx, torch.from_numpy(a).cuda())
+    evals, evecs = evals.cpu().numpy(), evecs.cpu().numpy()
+    assert sweeps >= 1
+    _check_conventions(a, evals, evecs)
+    assert np.abs(evals - np.linalg.eigvalsh(a)[::-1]).max() <= 1e-13 * max(1, n / 16) * lam.max()
+
+
+def test_fit_by_jacobi_matches_the_fit_by_division(ctx):
+    params = fm.layer_params(fm.LayerSpec(96, 8, 8, 0.92, None, 9200))
+    cal = fm.make_maps(params, 12, calib=True, dtype=torch.float32).cuda()
+    default = tc.tc_model_export(tc.tc_fit_pca(ctx, cal, 5))
+    tc.tc_force_jacobi(ctx, 1)
+    other = tc.tc_model_export(tc.tc_fit_pca(ctx, cal, 5))
+    tc.tc_force_jacobi(ctx, 0)
+    assert np.array_equal(default["mean"], other["mean"])
+    assert np.allclose(default["eig"], other["eig"], rtol=0, atol=1e-12 * default["eig"][0])
+    assert np.abs(default["basis"] - other["basis"]).max() <= 2.0 ** -23 and (default["basis"] == other["basis"]).mean() >= 0.99
 
 
 # Edges of the cluster solver: lanes' elements and blocks of the cluster change at multiples of 64, groups of
