@@ -761,7 +761,7 @@ tc_status tc_launch_decode_runs(const tc_ctx *ctx, const DecodeArgs &a, cudaStre
     void (*kernel)(DecodeArgs, SmemLayout) = a.relu ? decode_runs_kernel<true> : decode_runs_kernel<false>;
     if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)l.total) != cudaSuccess)
         return TC_ERR_CUDA;
-    const unsigned int grid = (unsigned int)((a.n_tiles < a.sms) ? a.n_tiles : a.sms);
+    const unsigned int grid = (unsigned int)((a.n_tiles < ctx->sm_count) ? a.n_tiles : ctx->sm_count);
     kernel<<<grid, kThreads, l.total, s>>>(a, l);
     return cudaGetLastError() == cudaSuccess ? TC_OK : TC_ERR_CUDA;
 }

@@ -936,15 +936,15 @@ static void (*pick_kernel(bool debug, bool hist))(EncodeArgs, Plan)
     return debug ? encode_tc_kernel<kPerChannel, true, kPair, false, kRuns> : encode_tc_kernel<kPerChannel, false, kPair, false, kRuns>;
 }
 
-// Which kernel codes the tensor: bit 0 a table per channel, bit 1 symbol pairs, bit 2 private runs; -1: not this file's.
+// Which kernel codes the tensor: bit 0 a table per channel, bit 1 symbol pairs, bit 2 private runs.
 static int kernel_class(const EncodeArgs &a, const Plan &pl)
 {
-    if (pl.staging_bytes == 0) return -1;
     const bool per_channel = a.groups != 1;
     return (per_channel ? 1 : 0) | (!per_channel && pl.entries > (1 << a.bits) ? 2 : 0) | (pl.run_words[0] > 0 ? 4 : 0);
 }
 
-int tc_encode_tc_class(const tc_ctx *ctx, const EncodeArgs &a) { return tc_encode_tc_supported(ctx, a) ? kernel_class(a, make_plan(ctx, a)) : -1; }
+// of a tensor that tc_encode_tc_supported takes
+int tc_encode_tc_class(const tc_ctx *ctx, const EncodeArgs &a) { return kernel_class(a, make_plan(ctx, a)); }
 
 // us that a tile takes a block: 1.5 with 64 coefficients at 1.1 bits each, 2.1 with 128, 4.25 with 256, 2.3 with 96 at 2.8 bits, 7.5
 // with 256 at 4.1 (8 to 85 tiles a block, after the first)
@@ -1006,7 +1006,7 @@ tc_status tc_launch_encode_tc(const tc_ctx *ctx, const EncodeArgs &a, cudaStream
                                                    : (runs ? pick_kernel<false, false, true>(debug, a.hist) : pick_kernel<false, false, false>(debug, a.hist));
     if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)l.total) != cudaSuccess)
         return TC_ERR_CUDA;
-    const unsigned int grid = (unsigned int)((a.n_tiles < a.sms) ? a.n_tiles : a.sms);
+    const unsigned int grid = (unsigned int)((a.n_tiles < ctx->sm_count) ? a.n_tiles : ctx->sm_count);
     EncodeArgs args = a;
     void *params[] = {&args, &pl};
     // cooperative launch: the grid must be co-resident, which is what makes the look-back safe

@@ -969,9 +969,9 @@ tc_status tc_encode_with_scratch(tc_ctx *ctx, const tc_model *m, const tc_codebo
     const size_t scratch_bytes = kEncodeScratchHeader + (size_t)n_tiles * sizeof(unsigned long long);
     const bool resident = resident_encode(ctx, x, a);
     if (hist && !resident) return TC_ERR_UNSUPPORTED;   // only the resident-basis tensor-core encoder counts symbols
-    if (resident) {
+    if (resident) {                                     // (in lists these share launches)
         ctx->last_encode_path = 1;
-        if (!scratch_is_zero) TC_CUDA(cudaMemsetAsync(scratch, 0, scratch_bytes, s));
+        TC_CUDA(cudaMemsetAsync(scratch, 0, scratch_bytes, s));
         return tc_launch_encode_tc(ctx, a, s);
     }
     if (ctx->force_exact != 1 && x->dtype == TC_BF16 && tc_encode_wide_supported(ctx, a)) {   // wide layers, unaligned rows
@@ -1161,7 +1161,7 @@ static tc_status decode_with_scratch(tc_ctx *ctx, const tc_model *m, const tc_co
         return TC_ERR_INVALID_ARG;
     DeviceGuard guard(ctx->device);
     const DecodeArgs a = decode_args(ctx, m, cb, stream, stream_bytes, chunk_len, tile_off, params, cs, x_hat, list_sms);
-    if (runs_decode(ctx, x_hat, a)) {                   // (it also takes dense tiles)
+    if (runs_decode(ctx, x_hat, a)) {                   // (it also takes dense tiles; in lists these share launches)
         ctx->last_decode_path = 1;
         return tc_launch_decode_runs(ctx, a, (cudaStream_t)cuda_stream);
     }

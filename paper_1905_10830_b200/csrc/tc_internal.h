@@ -128,7 +128,7 @@ struct EncodeArgs {
     unsigned long long *tile_state;   // look-back state, zeroed before launch
     unsigned int *ticket;             // zeroed before launch; the look-back words follow it
     bool alone;                       // no other stream of this call (see launch_chained)
-    int sms;                          // SMs that a persistent kernel takes at most
+    int sms;                          // SMs that a persistent kernel of its own takes at most in a list
     long long clear_words;            // 64-bit words from `ticket` on that the first of several kernels zeroes (0: they are zero)
     unsigned long long *other_state;  // resident-basis encoder: look-back state that no tile of this call uses,
     long long other_words;            // and how many words of it to zero for the next
@@ -162,7 +162,7 @@ struct DecodeArgs {
     const uint8_t *sorted;              // [groups][2^bits]
     const __nv_bfloat16 *basis_t_bf16;  // [c][k]
     bool alone;                         // no other stream of this call (see launch_chained)
-    int sms;                            // SMs that a persistent kernel takes at most
+    int sms;                            // SMs that a persistent kernel of its own takes at most in a list
     const CUtensorMap *basis_t_map;     // HOST pointer to the model's tensor map of basis_t_bf16, or null
     const float *dec_bias;              // [c]
     int center;                         // subtracted from every symbol before the MMA
