@@ -257,10 +257,10 @@ int piece_of(long long count, const void *a, const void *b)
 }
 
 template <typename TIn>
-void launch_channel_sums(const TIn *x, int n, int c, int hw, double *sums, cudaStream_t s)
+void launch_channel_sums(const TIn *x, int n, int c, int hw, double *sums, int sm_count, cudaStream_t s)
 {
     const unsigned channels = (unsigned)((c + kSumWarps - 1) / kSumWarps);
-    long long images = std::max(1u, 1184u / channels);                 // eight blocks an SM
+    long long images = std::max(1u, 8u * (unsigned)sm_count / channels);             // eight blocks an SM
     images = std::min(images, ((long long)n + kSumRows - 1) / kSumRows);
     const dim3 grid(channels, (unsigned)images);
     switch (piece_of<TIn>(hw, x, x)) {
@@ -272,12 +272,12 @@ void launch_channel_sums(const TIn *x, int n, int c, int hw, double *sums, cudaS
 }
 
 template <typename TIn>
-void launch_sqerr(const TIn *x, const TIn *xhat, long long count, double *sum_sq, unsigned long long *zeros, cudaStream_t s)
+void launch_sqerr(const TIn *x, const TIn *xhat, long long count, double *sum_sq, unsigned long long *zeros, int sm_count, cudaStream_t s)
 {
     constexpr int wide = 16 / sizeof(TIn);
     const bool aligned = (((uintptr_t)x | (uintptr_t)xhat) & 15u) == 0;
     long long blocks = (count + kErrThreads * wide - 1) / (kErrThreads * wide);
-    blocks = std::max(1ll, std::min(blocks, 1184ll));                  // eight an SM
+    blocks = std::max(1ll, std::min(blocks, 8ll * sm_count));          // eight an SM
     if (aligned) sqerr_kernel<TIn, wide><<<(unsigned)blocks, kErrThreads, 0, s>>>(x, xhat, count, sum_sq, zeros);
     else sqerr_kernel<TIn, 1><<<(unsigned)blocks, kErrThreads, 0, s>>>(x, xhat, count, sum_sq, zeros);
 }
@@ -296,11 +296,11 @@ inline bool launched() { return cudaGetLastError() == cudaSuccess; }
 
 }  // namespace
 
-tc_status tc_launch_channel_sums(const void *x, int dtype, int n, int c, int hw, double *sums, cudaStream_t s)
+tc_status tc_launch_channel_sums(const void *x, int dtype, int n, int c, int hw, double *sums, int sm_count, cudaStream_t s)
 {
     if (n == 0) return TC_OK;
-    if (dtype == TC_F32) launch_channel_sums((const float *)x, n, c, hw, sums, s);
-    else launch_channel_sums((const __nv_bfloat16 *)x, n, c, hw, sums, s);
+    if (dtype == TC_F32) launch_channel_sums((const float *)x, n, c, hw, sums, sm_count, s);
+    else launch_channel_sums((const __nv_bfloat16 *)x, n, c, hw, sums, sm_count, s);
     return launched() ? TC_OK : TC_ERR_CUDA;
 }
 
@@ -359,10 +359,10 @@ tc_status tc_launch_histogram(const uint8_t *sym, long long pixels, int k, int g
 }
 
 tc_status tc_launch_sqerr(const void *x, const void *xhat, int dtype, long long count, double *sum_sq,
-                          unsigned long long *zeros, cudaStream_t s)
+                          unsigned long long *zeros, int sm_count, cudaStream_t s)
 {
-    if (dtype == TC_F32) launch_sqerr((const float *)x, (const float *)xhat, count, sum_sq, zeros, s);
-    else launch_sqerr((const __nv_bfloat16 *)x, (const __nv_bfloat16 *)xhat, count, sum_sq, zeros, s);
+    if (dtype == TC_F32) launch_sqerr((const float *)x, (const float *)xhat, count, sum_sq, zeros, sm_count, s);
+    else launch_sqerr((const __nv_bfloat16 *)x, (const __nv_bfloat16 *)xhat, count, sum_sq, zeros, sm_count, s);
     return launched() ? TC_OK : TC_ERR_CUDA;
 }
 

@@ -561,7 +561,7 @@ tc_status tc_fit_pca(tc_ctx *ctx, const tc_tensor *calib, const tc_fit_params *p
     double *const d_buf = (double *)ctx->scratch, *d_mean = d_buf, *d_cov = d_buf + c;
     TC_CUDA(cudaMemsetAsync(d_buf, 0, n_doubles * sizeof(double), s));
 
-    st = tc_launch_channel_sums(calib->data, calib->dtype, n, c, hw, d_mean, s);
+    st = tc_launch_channel_sums(calib->data, calib->dtype, n, c, hw, d_mean, ctx->sm_count, s);
     if (st != TC_OK) return st;
     if ((st = tc_launch_mean(d_mean, c, m_samples, s)) != TC_OK) return st;
     st = tc_launch_covariance(calib->data, calib->dtype, n, c, hw, d_mean, d_cov, ctx->sm_count, s);
@@ -683,7 +683,7 @@ tc_status tc_fit_state_update(tc_ctx *ctx, tc_fit_state *st, const tc_tensor *ma
     cudaStream_t s = (cudaStream_t)cuda_stream;
     const int hw = maps->h * maps->w;
     if ((long long)maps->n * hw == 0) return TC_OK;
-    tc_status rc = tc_launch_channel_sums(maps->data, maps->dtype, maps->n, st->c, hw, st->d_sum, s);
+    tc_status rc = tc_launch_channel_sums(maps->data, maps->dtype, maps->n, st->c, hw, st->d_sum, ctx->sm_count, s);
     if (rc != TC_OK) return rc;
     rc = tc_launch_covariance(maps->data, maps->dtype, maps->n, st->c, hw, st->d_zero, st->d_outer, ctx->sm_count, s);
     if (rc != TC_OK) return rc;
@@ -1630,7 +1630,7 @@ static tc_status stats_tensor_core(tc_ctx *ctx, const tc_model *m, const tc_code
         st = tc_decode(ctx, m, code, base + off_stream, lay.stream_bytes, (const uint16_t *)(base + off_chunk),
                        (const uint64_t *)(base + off_tile), &prm, &xh, s);
         if (st != TC_OK) return st;
-        if ((st = tc_launch_sqerr(xi.data, xh.data, x->dtype, (long long)cn * m->c * hw, d_sq, d_zeros, s)) != TC_OK) return st;
+        if ((st = tc_launch_sqerr(xi.data, xh.data, x->dtype, (long long)cn * m->c * hw, d_sq, d_zeros, ctx->sm_count, s)) != TC_OK) return st;
     }
     if ((st = tc_launch_fold_counts(d_hist, kHistCopies, m->k * nsym, s)) != TC_OK) return st;
     hist.assign((size_t)m->k * nsym, 0ull);
@@ -1693,7 +1693,7 @@ static tc_status stats_exact(tc_ctx *ctx, const tc_model *m, const tc_tensor *x,
     d.basis64 = m->d_basis64; d.mean64 = m->d_mean64; d.lo = m->lo; d.step = m->step; d.basis_scale = m->basis_scale;
     d.xhat = d_xhat; d.status = ctx->d_status;
     if ((st = tc_launch_decode_simt(ctx, d, x->dtype, s)) != TC_OK) return st;
-    if ((st = tc_launch_sqerr(x->data, d_xhat, x->dtype, (long long)values, d_sq, d_zeros, s)) != TC_OK) return st;
+    if ((st = tc_launch_sqerr(x->data, d_xhat, x->dtype, (long long)values, d_sq, d_zeros, ctx->sm_count, s)) != TC_OK) return st;
 
     hist_out.assign((size_t)m->k * nsym, 0ull);
     TC_CUDA(cudaMemcpyAsync(hist_out.data(), d_hist, hist_bytes, cudaMemcpyDeviceToHost, s));

@@ -286,7 +286,7 @@ tc_status tc_launch_decode_wide(const tc_ctx *ctx, const DecodeArgs &a, cudaStre
 size_t tc_decode_tc_staging_bytes(const tc_ctx *ctx, const DecodeArgs &a);     // per tile
 size_t tc_decode_wide_staging_bytes(const tc_ctx *ctx, const DecodeArgs &a);   // per tile
 
-tc_status tc_launch_channel_sums(const void *x, int dtype, int n, int c, int hw, double *sums,
+tc_status tc_launch_channel_sums(const void *x, int dtype, int n, int c, int hw, double *sums, int sm_count,
                                  cudaStream_t s);
 tc_status tc_launch_mean(double *sums, int c, long long pixels, cudaStream_t s);      // in place
 tc_status tc_launch_covariance(const void *x, int dtype, int n, int c, int hw, const double *mean,
@@ -299,7 +299,7 @@ tc_status tc_launch_fold_counts(unsigned long long *counts, int copies, int n, c
 tc_status tc_launch_histogram(const uint8_t *sym, long long pixels, int k, int groups, int bits,
                               unsigned long long *hist, cudaStream_t s);
 tc_status tc_launch_sqerr(const void *x, const void *xhat, int dtype, long long count,
-                          double *sum_sq, unsigned long long *zeros, cudaStream_t s);
+                          double *sum_sq, unsigned long long *zeros, int sm_count, cudaStream_t s);
 
 // ---- host algorithms (host_algos.cpp) ---------------------------------------------------
 int tc_huffman_lengths_host(const uint64_t *counts, int nsym, int lmax, uint8_t *len);
