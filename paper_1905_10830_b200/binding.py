@@ -541,15 +541,19 @@ def tc_encode_many(ctx: Context, layers, *, outs=None):
     return result
 
 
-def tc_decode_many(ctx: Context, layers, *, outs=None, relu: bool = False):
-    """Decode several tensors in one call: `layers` is a list of (model, codebook, enc, shape, dtype)."""
+def tc_decode_many(ctx: Context, layers, *, outs=None, relu=False):
+    """Decode several tensors in one call: `layers` is a list of (model, codebook, enc, shape, dtype); `relu` is one flag
+    for all of them or a list of one each."""
     n = len(layers)
+    relus = relu if isinstance(relu, (list, tuple)) else [relu] * n
+    if len(relus) != n:
+        raise ValueError("relu: one flag, or one for each layer")
     tensors, params, items = [], [], (_DecodeItem * max(n, 1))()
     result = []
     for i, (model, cb, enc, shape, dtype) in enumerate(layers):
         out = outs[i] if outs is not None else torch.empty(shape, dtype=dtype, device=enc.words.device)
         t = _tensor(out)
-        p = _EncodeParams(enc.layout.chunk_pixels, enc.layout.pixel_splits, int(relu), 0)
+        p = _EncodeParams(enc.layout.chunk_pixels, enc.layout.pixel_splits, int(relus[i]), 0)
         tensors.append(t); params.append(p); result.append(out)
         items[i] = _DecodeItem(model.ptr, cb.ptr, enc.words.data_ptr(), enc.words.numel(), enc.chunk_len.data_ptr(),
                                enc.tile_off.data_ptr(), C.addressof(p), C.addressof(t))

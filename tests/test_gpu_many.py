@@ -164,16 +164,17 @@ def test_long_mixed_lists_equal_the_per_tensor_calls(ctx):
         relus.append(j % 3 == 0)
     encs = tc.tc_encode_many(ctx, items)
     assert tc.tc_get_status(ctx) == 0
-    for relu in (False, True):
-        pick = [i for i in range(len(items)) if relus[i] == relu] if relu else list(range(len(items)))
-        outs = tc.tc_decode_many(ctx, [(*items[i][:2], encs[i], items[i][2].shape, torch.bfloat16) for i in pick], relu=relu)
+    with pytest.raises(ValueError):
+        tc.tc_decode_many(ctx, [(*i[:2], e, i[2].shape, torch.bfloat16) for i, e in zip(items, encs)], relu=relus[1:])
+    for relu in (False, True, relus):
+        outs = tc.tc_decode_many(ctx, [(*i[:2], e, i[2].shape, torch.bfloat16) for i, e in zip(items, encs)], relu=relu)
         assert tc.tc_get_status(ctx) == 0
-        for i, out in zip(pick, outs):
+        for i, out in enumerate(outs):
             model, cb, x = items[i]
             alone = tc.tc_encode(ctx, model, cb, x)
             assert alone.total_bits() == encs[i].total_bits()
             assert np.array_equal(H.stream_words(encs[i]), H.stream_words(alone)) and np.array_equal(H.chunk_len(encs[i]), H.chunk_len(alone))
-            assert torch.equal(out, tc.tc_decode(ctx, model, cb, alone, x.shape, torch.bfloat16, relu=relu))
+            assert torch.equal(out, tc.tc_decode(ctx, model, cb, alone, x.shape, torch.bfloat16, relu=relus[i] if relu is relus else relu))
     assert tc.tc_get_status(ctx) == 0
 
 
