@@ -353,7 +353,8 @@ def test_decoded_rows_more_than_2_32_elements_apart(ctx):
 
 # Entropy coder and decoder with a tile dealt to several blocks: tiles few enough for two and four blocks (and one more), last tiles
 # whose later blocks have a pixel or none, chunks of several pixels, one, two and four a pixel, tables per layer and per channel, codes
-# of one bit (blocks of a few words) and of twelve.  Against the one-thread-per-pixel kernels, which run without workspace.
+# of one bit and of twelve.  (Most of them leave the coder, which deals from 384 coefficients on, one block a tile: more of its cases below.)
+# Against the one-thread-per-pixel kernels, which run without workspace.
 @pytest.mark.parametrize("c,pixels,bits,dtype,per_channel,cp,splits", [
     (64, 1, 4, torch.float32, False, 0, 0), (64, 33, 4, torch.float32, False, 0, 0), (64, 128 * 37, 3, torch.float32, False, 4, 1),
     (64, 128 * 37 + 1, 5, torch.float32, True, 0, 0), (96, 65, 8, torch.float32, True, 0, 0), (128, 128 * 74 - 31, 4, torch.float32, False, 0, 0),
@@ -362,6 +363,26 @@ def test_decoded_rows_more_than_2_32_elements_apart(ctx):
     (512, 128 * 5 + 34, 4, torch.float32, True, 0, 0), (320, 49 * 3, 4, torch.bfloat16, False, 0, 0), (320, 49 * 100, 8, torch.bfloat16, False, 0, 0),
     (576, 49 * 7, 5, torch.bfloat16, False, 0, 0), (256, 49 * 3, 6, torch.bfloat16, True, 0, 0), (512, 49 * 500, 4, torch.bfloat16, False, 0, 0)])
 def test_a_tile_dealt_to_several_blocks(ctx, c, pixels, bits, dtype, per_channel, cp, splits):
+    _deal_and_compare(ctx, c, pixels, bits, dtype, per_channel, cp, splits)
+
+
+# The coder deals a tile to a cluster from 384 coefficients on.  Two blocks a tile (38 and 74 tiles; 75 leave one) and four; last tiles that
+# leave the later blocks no pixel or one; chunks of several pixels, up to what a block has; codes of one bit, and codes of eight
+# throughout, which exceed the staging (four bits a symbol), so that the cluster clears the stream and writes to it.
+@pytest.mark.parametrize("c,pixels,bits,dtype,per_channel,cp,splits,flat", [
+    (512, 128 * 3 + 1, 1, torch.float32, False, 0, 0, False), (384, 128 * 2 + 33, 2, torch.float32, False, 4, 1, False),
+    (384, 128 + 97, 2, torch.float32, False, 32, 1, False), (384, 128 * 5, 1, torch.float32, False, 64, 1, False),
+    (512, 128 * 5 + 65, 3, torch.float32, False, 16, 1, False), (384, 128 * 37 + 1, 4, torch.float32, False, 0, 0, False),
+    (384, 128 * 37 + 64, 4, torch.float32, True, 0, 0, False), (384, 128 * 73 + 65, 3, torch.float32, False, 0, 0, False),
+    (384, 128 * 74 + 1, 3, torch.float32, False, 0, 0, False), (960, 49 * 100, 5, torch.bfloat16, False, 0, 0, False),
+    (512, 129, 8, torch.float32, False, 0, 0, True), (384, 128 * 2 + 34, 8, torch.float32, True, 0, 0, True), (384, 128 * 38 + 33, 8, torch.float32, False, 0, 0, True)])
+def test_a_tile_coded_by_a_cluster(ctx, c, pixels, bits, dtype, per_channel, cp, splits, flat):
+    enc = _deal_and_compare(ctx, c, pixels, bits, dtype, per_channel, cp, splits, flat)
+    if flat:
+        assert int(enc.tile_off[1] - enc.tile_off[0]) > 4 * 128 * c
+
+
+def _deal_and_compare(ctx, c, pixels, bits, dtype, per_channel, cp, splits, flat=False):
     rng = np.random.default_rng(c + pixels)
     h, n = (7, pixels // 49) if dtype == torch.bfloat16 else (1, 1)
     w = pixels // (n * h)
@@ -378,6 +399,8 @@ def test_a_tile_dealt_to_several_blocks(ctx, c, pixels, bits, dtype, per_channel
     counts = rng.integers(0, 50, (c if per_channel else 1, top + 1))
     counts[..., top // 2] = 2000 if bits > 1 else 1
     counts[..., 0] = 0
+    if flat:
+        counts[:] = 1
     lengths = np.stack([tc.tc_host_huffman_lengths(row) for row in counts])
     m = tc.tc_model_import(ctx, basis=basis, mean=np.zeros(c), lo=lo, step=step, bits=bits, basis_dtype=tc.binding.TC_BF16 if dtype == torch.bfloat16 else tc.binding.TC_F32,
                            eig=scale ** 2)
@@ -397,3 +420,56 @@ def test_a_tile_dealt_to_several_blocks(ctx, c, pixels, bits, dtype, per_channel
         assert abs(enc.total_bits() - want.total_bits()) <= 1e-3 * want.total_bits() + 256
         assert (x_hat != want_hat).double().mean() <= 1e-3 and (x_hat.double() - want_hat.double()).abs().max() <= 2.0 ** -7 * want_hat.double().abs().max()
     m.close(); cb.close()
+    return enc
+
+
+# The resident-basis encoder's look-back arrays, two of a context in turn, each cleared by the call that follows its use: calls large and small
+# on one context, with those in between that leave the arrays alone (over 8192 tiles, captured, a list) or end early (a buffer that is
+# too small).  Every stream that of a context of its own.
+def test_look_back_arrays_in_turn(ctx):
+    c, bits = 16, 4
+    basis = torch.linalg.qr(torch.randn(c, c, dtype=torch.float64, generator=torch.Generator().manual_seed(4)))[0].to(torch.bfloat16).double().numpy()
+    counts = np.full(16, 5)
+    counts[7] = 2000
+    m = tc.tc_model_import(ctx, basis=basis, mean=np.zeros(c), lo=-3.0, step=0.4, bits=bits, basis_dtype=tc.binding.TC_BF16, eig=4.0 * 0.7 ** np.arange(c))
+    cb = tc.tc_codebook_import(ctx, np.stack([tc.tc_host_huffman_lengths(counts)]), bits)
+    gen = torch.Generator(device="cuda").manual_seed(9)
+    maps = {tiles: torch.randn(1, c, tiles * 32, 4, device="cuda", generator=gen).to(torch.bfloat16) for tiles in (1, 3, 148, 700, 5000, 8192, 8193)}
+    want = {}
+    for tiles, x in maps.items():
+        own = tc.tc_create(0)
+        want[tiles] = tc.tc_encode(own, m, cb, x)
+        assert tc.tc_get_status(own) == 0 and tc.tc_last_path(own) == 1
+        own.close()
+
+    def check(enc, tiles):
+        n = want[tiles].total_bits() // 8
+        assert torch.equal(enc.tile_off, want[tiles].tile_off) and torch.equal(enc.words[:n], want[tiles].words[:n])
+        assert torch.equal(enc.chunk_len[:enc.layout.n_chunks], want[tiles].chunk_len[:enc.layout.n_chunks])
+
+    own = tc.tc_create(0)
+    for tiles in (5000, 3, 5000, 1, 1, 700, 8192, "short", 700, "short", 8192, 8193, 148, "graph", 5000, "list", 5000, "list", 3, "graph", 8192, 1, 8192):
+        if tiles == "short":
+            tc.tc_encode(own, m, cb, maps[700], capacity=want[700].total_bits() // 16)
+            assert tc.tc_get_status(own) == 3
+        elif tiles == "graph":
+            out = tc.tc_encode(own, m, cb, maps[700])
+            torch.cuda.synchronize()
+            graph, side = torch.cuda.CUDAGraph(), torch.cuda.Stream()
+            with torch.cuda.stream(side):
+                graph.capture_begin()
+                tc.tc_encode(own, m, cb, maps[700], out=out)
+                graph.capture_end()
+            torch.cuda.synchronize()
+            for _ in range(3):
+                out.words.zero_()
+                graph.replay()
+                torch.cuda.synchronize()
+                check(out, 700)
+        elif tiles == "list":
+            for t, enc in zip((148, 5000, 3), tc.tc_encode_many(own, [(m, cb, maps[t]) for t in (148, 5000, 3)])):
+                check(enc, t)
+        else:
+            check(tc.tc_encode(own, m, cb, maps[tiles]), tiles)
+    assert tc.tc_get_status(own) == 0
+    own.close()
