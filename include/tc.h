@@ -387,7 +387,7 @@ tc_status tc_decode(tc_ctx *ctx, const tc_model *model, const tc_codebook *cb, c
  * whole list: the items are checked first (nothing is launched if one is invalid), the
  * bookkeeping of all of them is cleared at once, and tensors that take the same kernel share its
  * launch, each with blocks of its own; those whose route has several kernels are spread, largest
- * first, over eight streams of the context.  `cuda_stream`
+ * first, over eight streams of the context.  The SMs are dealt so that all are done at about the same time.  `cuda_stream`
  * waits for all of them, so later work on it sees every output.  The results are those of
  * tc_encode / tc_decode called per item (same arguments, same errors; the first error is
  * returned after all items that could be launched have been).  Output buffers of different
