@@ -16,20 +16,24 @@
 //                      K-major).  One or two threads per pixel walk the pixel's chunks.  A group's time
 //                      per tile is the latency of its chunks' symbols, so the groups in flight set the
 //                      rate: with two groups whatever their size 64x56x56 x 64 took 62 us, with eight 24.
-//   warps 16-23        epilogue, all eight warps on every work item: TMEM -> registers,
-//                      x_hat = step * acc + bias, round to bf16, NCHW stores through warp-private
-//                      transpose blocks (the accumulator is held transposed: lane = channel)
-//   warps 24, 25       one thread each issues the tcgen05.mma of its accumulator's work items:
+//   warps 16-23        epilogue, four warps on each accumulator: TMEM -> registers,
+//                      x_hat = step * acc + bias, round to bf16, NCHW stores (the accumulator is held
+//                      transposed: lane = channel)
+//   warp 24            one thread issues the tcgen05.mma of the work items, a tile's blocks of 128 channels:
 //                      D[c][pixel] = T[j][c] * (Q[pixel][j] - center)
 // The transposed basis is the A operand and lives in TENSOR memory, not in shared memory: each
 // block of 128 channels takes K / 2 columns (two bf16 per column), 256 columns at C = K = 256,
 // loaded once per block with tcgen05.st.  That leaves shared memory to the symbols -- two whole
 // tiles in flight, 128 KB at K = 256 -- and takes the basis off the MMA's shared-memory reads.
-// The other 256 columns hold two accumulators of 128 columns: one tile of 128 pixels up to 128
-// channels; with two channel blocks a work item is half a tile (2 x 64 columns), so that the
-// epilogue of one item overlaps the MMAs of the next.
-// The operand is handed back in panels of 32 coefficients: the MMA thread commits a barrier per
-// panel, and a VLD thread of the group's next tile waits only for the panel it is about to touch.
+// The other 256 columns hold two accumulators of 128 pixels, so that the epilogue of one item overlaps the
+// MMAs of the next.
+// The operand is handed back in panels of 128 coefficients: the MMA thread commits a barrier per
+// panel, and a VLD thread of the group's next tile waits only for the panels that it writes.
+//
+// What bounds it is the VLD groups' instructions and their chains (256x14x14 x 4096 at 4 bits: 139 us with the products and the stores
+// left out, 163 in all; 218 before the items, stores and registers took their present form).  Every warp takes its turn at the issue
+// slots, an instruction in about twelve cycles, so that the MMA warp's loop is unrolled; and what does not fit the registers goes to local
+// memory and comes back from L2 (shared memory leaves the L1 no room): hence the split of the registers below.
 //
 // A tile whose stream is dense (more than kDenseBits128 / 128 bits per symbol) gains nothing
 // from run skipping; its threads then decode symbol by symbol, eight symbols per 16-byte store.
@@ -44,11 +48,13 @@ using namespace tcdev;
 using namespace sm100;
 
 constexpr int kVldWarps = 16, kMaxGroups = 8, kEpiWarp0 = kVldWarps, kMmaWarp = kEpiWarp0 + 8;
-constexpr int kThreads = (kMmaWarp + 2) * 32;                  // two MMA warps, one per accumulator
+constexpr int kThreads = (kMmaWarp + 4) * 32;                  // the MMA warp is one of a warpgroup of four, which leave registers to the VLD groups
 constexpr int kTmemCols = 512;
 constexpr int kAccBase = 256, kAccCols = 128;                 // two accumulators behind the basis columns
-constexpr int kPanelK = 32;                                   // coefficients per hand-over panel
-constexpr int kMaxPanels = 8;                                 // K <= 256
+// Coefficients per hand-over panel.  A commit keeps the issuing warp for some 400 cycles: with eight panels of 32 (and
+// a commit an item) VLD threads waited no less, and the commits held up the MMAs.
+constexpr int kPanelK = 128;
+constexpr int kMaxPanels = 2;                                 // K <= 256
 constexpr uint32_t kRunGuard = 0x800u;                        // bit 11 set: at most 20 zero bits are skipped per step (20 + 12 <= 32: one refill per step)
 constexpr int kDenseBits128 = 224;                            // tiles above 1.75 bits per symbol are decoded symbol by symbol
 // A chunk that starts inside a staged segment is read for at most (symbols of the chunk) x 12
@@ -56,15 +62,15 @@ constexpr int kDenseBits128 = 224;                            // tiles above 1.7
 // block's shared memory even for a corrupt stream (the buffers lie back to back).
 constexpr int kStreamSlack = 1024;
 constexpr int kStaticSmem = 1536;                             // room for the kernel's static shared variables
-constexpr int kTrWarpBytes = 2048;                            // epilogue transpose block of one warp: 32 channel rows x 32 pixels
+constexpr int kTrWarpBytes = 4096;                            // epilogue block of one warp: 16 channel rows x 128 pixels
 // Named barriers.  Hand-overs between warps that both run ordinary instructions use them instead
 // of mbarriers: the waiting side is parked by the hardware, whereas a warp polling an mbarrier
 // keeps issuing and takes issue slots from the warps that work.  (mbarriers remain where the
 // tensor core signals: accumulator ready, operand panel consumed.)
 constexpr int kBarGroup = 1;                                  // + group: the VLD threads of a group, once per tile
 constexpr int kBarAccFree = kBarGroup + kMaxGroups;           // + accumulator: drained, epilogue warps -> MMA warp
-constexpr int kBarBasis = kBarAccFree + 2;                    // basis in tensor memory, epilogue warps -> MMA warps, once
-constexpr int kBarEpi = kBarAccFree + 3;                      // accumulator ready, polling epilogue warp -> the other seven
+constexpr int kBarBasis = kBarAccFree + 2;                    // basis in tensor memory, epilogue warps -> MMA warp, once
+constexpr int kBarEpi = kBarAccFree + 3;                      // + accumulator: ready, polling epilogue warp -> its other three
 
 struct SmemLayout {
     uint32_t lut, opnd, tbuf, sbuf, total;
@@ -78,7 +84,7 @@ struct SmemLayout {
 // that does not fit its buffer is read from global memory word by word, which costs more than a group less: with room
 // for 2.5 bits per symbol whatever the rate, 512 maps of 28x28 at 8 bits (4.8 to 4.3 bits per value) took 115 us at
 // 128 channels, 186 at 176 and 200 at 192; sized by the rate 95, 153 and 163, and 256 maps of 64x56x56 121 -> 101.
-inline SmemLayout smem_layout(int k, int lut_entries, int group_warps, uint32_t want_bytes, int budget)
+inline SmemLayout smem_layout(int k, int lut_entries, int group_warps, uint32_t want_bytes, bool row_blocks, int budget)
 {
     SmemLayout l;
     l.lut = 0;                                                // 32-bit entries: bf16(symbol - center) << 16 | length
@@ -89,7 +95,7 @@ inline SmemLayout smem_layout(int k, int lut_entries, int group_warps, uint32_t 
     l.total = 0;
     for (l.groups = most; l.groups >= 2; --l.groups) {
         l.tbuf = l.opnd + (uint32_t)l.groups * l.opnd_bytes;
-        l.sbuf = l.tbuf + 8u * kTrWarpBytes;
+        l.sbuf = l.tbuf + (row_blocks ? 8u * kTrWarpBytes : 0u);
         const long long left = (long long)budget - l.sbuf - kStreamSlack;
         const long long room = (left / (2ll * l.groups)) & ~127ll;
         if (room < 4096 || (room < (long long)want_bytes && l.groups > 2)) continue;
@@ -205,8 +211,35 @@ struct BitReader {
     }
 };
 
-// Rows leave in pieces of four pixels or eight, not pixel by pixel.
-__host__ __device__ inline bool vector_stores(const DecodeArgs &a) { return (a.hw & 3) == 0 && ((uintptr_t)a.xhat & 7u) == 0 && a.hw < (1 << 29); }
+// How channel rows leave.  What a store costs is the lines of 128 bytes that it touches, 6.5 cycles each an SM, unless the store right
+// before it touched them too: 256x14x14 x 4096 written as 64 bytes of four rows an instruction takes 188 us and nothing else (what the
+// decoder did), 256 bytes of one row 109; 64x56x56 x 1024 as 64 bytes of eight rows 150, the same with the four pieces of a row one
+// after the other 73.  So a warp stores all 128 pixels of its 16 channels at a time:
+//   kRows16: every group of eight pixels is 16-byte aligned and inside one image: straight from the registers, 16 bytes a thread and
+//            64 of eight rows an instruction, a row's four pieces in succession;
+//   kRows8:  the same of groups of four: through a block of the warp in shared memory, a row an instruction, 8 bytes a thread;
+//   kRowsAny: rows that start anywhere (H*W no multiple of 4, an unaligned tensor): through the block, a pixel a thread, a row in four
+//            instructions in succession.
+enum { kRows16, kRows8, kRowsAny };
+__host__ __device__ inline int store_mode(const DecodeArgs &a)
+{
+    if ((a.hw & 3) != 0 || ((uintptr_t)a.xhat & 7u) != 0) return kRowsAny;
+    return (a.hw & 7) == 0 && ((uintptr_t)a.xhat & 15u) == 0 ? kRows16 : kRows8;
+}
+// The accumulator is read as matrix fragments: of 32 columns thread q of four gets 8 g + 2 q + {0, 1}, g = 0 ... 3.  Which pixel a column
+// stands for is free (the order of the operand's rows); so that a thread's columns are consecutive pixels, they are
+// pixels 8 q + 2 g + {0, 1}.
+__device__ __forceinline__ uint32_t column_of(uint32_t p) { return (p & ~31u) | ((p & 6u) << 2) | ((p >> 2) & 6u) | (p & 1u); }
+__device__ __forceinline__ uint32_t pixel_of(uint32_t n) { return (n & ~31u) | ((n & 6u) << 2) | ((n >> 2) & 6u) | (n & 1u); }
+
+// The thread's index, read anew: what a role derives from its own reading is not worked out ahead of the other roles and kept through them (with
+// registers as short as here such values went to local memory, that is to L2: L1 is what shared memory leaves of it).
+__device__ __forceinline__ int own_tid()
+{
+    int t;
+    asm volatile("mov.u32 %0, %%tid.x;" : "=r"(t));
+    return t;
+}
 
 // `block` of `blocks` that share the tensor's tiles.
 template <bool kRelu>
@@ -220,7 +253,8 @@ __device__ __forceinline__ void decode_tiles(const DecodeArgs &a, const SmemLayo
     // be reading this tile's; the group's barrier (one per tile) only orders the write after next.
     __shared__ unsigned int s_wsum[kMaxGroups][2][2][4];
 
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    // (taken from lane 0: the compiler knows that the branches between the roles are the same for a whole warp)
+    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
     const int lut_size = 1 << a.lut_bits;
     const int S = a.splits, cp = a.chunk_pixels;
     const int tpp = S >= 2 ? 2 : 1;                            // threads per pixel
@@ -231,12 +265,12 @@ __device__ __forceinline__ void decode_tiles(const DecodeArgs &a, const SmemLayo
     const uint32_t lut_addr = smem_u32(smem + L.lut);
     const uint32_t opnd_addr = smem_u32(smem + L.opnd);
     const int n_blocks = (a.c + 127) / 128;                    // blocks of 128 channels
-    const int items = n_blocks;                                // work items per tile: halves of 64 pixels with two channel blocks
+    const int items = n_blocks;                                // work items per tile: its channel blocks
 
     // ---- set-up ---------------------------------------------------------------------
     if (tid < G * (kMaxPanels + 1)) {
         const int g = tid / (kMaxPanels + 1), p = tid - g * (kMaxPanels + 1);
-        if (p < kMaxPanels) mbar_init(smem_u32(&s_empty[g][p]), (uint32_t)items);       // one commit per item of the tile
+        if (p < kMaxPanels) mbar_init(smem_u32(&s_empty[g][p]), 1);                     // the commit of the tile's last item
         else mbar_init(smem_u32(&s_bfull[g]), (uint32_t)group_warps);                   // operand complete: one arrival per warp
         if (tid < 2) mbar_init(smem_u32(&s_tfull[tid]), 1);
         mbar_fence_init();
@@ -255,7 +289,7 @@ __device__ __forceinline__ void decode_tiles(const DecodeArgs &a, const SmemLayo
     tc_fence_before_sync();
     __syncthreads();
     tc_fence_after_sync();
-    const uint32_t tmem_base = s_tmem_base;
+    const uint32_t tmem_base = __shfl_sync(0xffffffffu, s_tmem_base, 0);
     if (warp >= kEpiWarp0 && warp < kMmaWarp) {
         // Transposed basis -> tensor memory: row c of block b (channel 128 b + c) goes to lane c,
         // its K coefficients, two per 32-bit column in memory order, to columns b K/2 ... of the A
@@ -289,15 +323,18 @@ __device__ __forceinline__ void decode_tiles(const DecodeArgs &a, const SmemLayo
             }
         }
         tmem_st_wait();
-        // (only the MMA warps wait for the basis; the VLD groups are on their first tiles meanwhile)
+        // (only the MMA warp waits for the basis; the VLD groups are on their first tiles meanwhile)
         tc_fence_before_sync();
-        named_bar_arrive(kBarBasis, 256 + 64);
+        named_bar_arrive(kBarBasis, 256 + 32);
     }
 
-    const long long my_tiles = (a.n_tiles > block) ? (a.n_tiles - block + blocks - 1) / blocks : 0;
+    const int my_tiles = (a.n_tiles > block) ? (int)((a.n_tiles - block + blocks - 1) / blocks) : 0;
 
     if (warp < kEpiWarp0) {
         // ================= VLD groups =================
+        // 28 warps of 72 registers are launched: 16 of 80, 8 of 72 and 4 of 40 take as many
+        asm volatile("setmaxnreg.inc.sync.aligned.u32 80;");
+        const int tid = own_tid(), warp = tid >> 5, lane = tid & 31;
         const int grp = warp / group_warps;
         const int tg = tid - grp * n_thr;        // thread within the group
         if (grp < G) {
@@ -317,50 +354,72 @@ __device__ __forceinline__ void decode_tiles(const DecodeArgs &a, const SmemLayo
             const int lb = a.lut_bits;
             const int dense_head = (a.dense_head + 7) & ~7;    // leading coefficients decoded symbol by symbol
             const uint32_t modal2 = (__float_as_uint((float)((a.modal < 0 ? a.center : a.modal) - a.center)) >> 16) * 0x00010001u;   // two bf16 copies of the modal symbol's value
+            // The chunk that the thread decodes is not the one whose length it adds up: with one or two pixels a chunk the
+            // threads of a warp write neighbouring columns of the operand, free of bank conflicts.
+            const int src_lane = cp == 1 ? (int)pixel_of((uint32_t)lane) : cp == 2 ? (int)(pixel_of(2u * lane) >> 1) : lane;
+            const int tc = (t & ~31) | src_lane;
             bool alive = true;
 
-            // offsets of a tile, validated; a tile that cannot be valid decodes nothing.  `lens`
-            // holds the chunk lengths of this thread's pixel (up to four), or of its chunk.
-            struct TileInfo { unsigned long long base, bits; bool ok, staged; unsigned int l01, l23; };
-            auto tile_info = [&](long long tl) {
-                TileInfo ti{0, 0, false, false, 0, 0};
-                if (tl >= my_tiles) return ti;
-                const long long tile = block + tl * blocks;
-                const unsigned long long base = a.tile_off[tile], end = a.tile_off[tile + 1];
-                ti.ok = (base & 127ull) == 0 && (end & 127ull) == 0 && base <= end && end <= a.stream_bits;
-                if (!ti.ok) return ti;
-                ti.base = base;
-                ti.bits = end - base;
-                ti.staged = ti.bits <= (unsigned long long)sbuf_bytes * 8ull &&
-                            (cp * (k_last - k_first) * TC_MAX_CODE_LEN) / 8 + 16 <= kStreamSlack;
+            // Offsets of a tile and the chunk lengths of this thread's pixel (up to four) or of its chunk, as they
+            // lie in memory: read two tiles ahead and looked at (tile_info) a tile later.  Looked at at once, the
+            // offsets' way from memory stood in every tile's time: 6 000 of the 19 000 cycles that a tile of 256
+            // coefficients took a group.
+            // (even lanes hold a tile's start, odd lanes its end)
+            struct RawTile { unsigned long long at; unsigned int l01, l23; };
+            auto load_tile = [&](int tl) {
+                RawTile rt{1, 0, 0};                             // (no tile: not valid)
+                if (tl >= my_tiles) return rt;
+                const long long tile = block + (long long)tl * blocks;
+                rt.at = __ldg(a.tile_off + tile + (lane & 1));
                 if (owner) {
                     const long long ch = tile * chunks_per_tile + (long long)t * (cp > 1 ? 1 : S);
-                    if (cp > 1 || S == 1) { if (ch < a.n_chunks) ti.l01 = a.chunk_len[ch]; }
+                    if (cp > 1 || S == 1) { if (ch < a.n_chunks) rt.l01 = a.chunk_len[ch]; }
                     else if (ch < a.n_chunks) {      // S chunks of one pixel: an aligned word holds two lengths
-                        ti.l01 = *reinterpret_cast<const unsigned int *>(a.chunk_len + ch);
-                        if (S == 4) ti.l23 = *reinterpret_cast<const unsigned int *>(a.chunk_len + ch + 2);
+                        rt.l01 = *reinterpret_cast<const unsigned int *>(a.chunk_len + ch);
+                        if (S == 4) rt.l23 = *reinterpret_cast<const unsigned int *>(a.chunk_len + ch + 2);
                     }
                 }
+                return rt;
+            };
+            // validated; a tile that cannot be valid decodes nothing
+            // (room: buffers that the segment takes, 0 if it is read from global memory; landed: its copy was started a tile ahead)
+            struct TileInfo { unsigned int bits; bool ok, landed; int room; unsigned int l01, l23; };
+            auto tile_info = [&](const RawTile &rt, unsigned long long &base) {
+                TileInfo ti{0, false, false, 0, 0, 0};
+                base = __shfl_sync(0xffffffffu, rt.at, 0);
+                const unsigned long long end = __shfl_sync(0xffffffffu, rt.at, 1);
+                ti.ok = (base & 127ull) == 0 && (end & 127ull) == 0 && base <= end && end <= a.stream_bits;
+                if (!ti.ok) return ti;
+                ti.bits = (unsigned int)min(end - base, 0x7fffff80ull);           // (no tile's chunks take more)
+                if ((cp * (k_last - k_first) * TC_MAX_CODE_LEN) / 8 + 16 <= kStreamSlack) ti.room = ti.bits <= sbuf_bytes * 8u ? 1 : ti.bits <= sbuf_bytes * 16u ? 2 : 0;
+                ti.l01 = rt.l01;
+                ti.l23 = rt.l23;
                 return ti;
             };
-            // start the copy of a tile's segment into stream buffer `which` (16 bytes per cp.async)
-            auto stage_tile = [&](const TileInfo &ti, int which) {
-                if (ti.ok && ti.staged) {
+            // Starts the copy of a tile's segment into stream buffer `which` (16 bytes per cp.async): while the tile before
+            // is decoded, or, where one of the two takes both buffers, at the tile's own turn (encode and decode of 256x14x14 x 1024 at 8 bits 203 -> 171 us
+            // against reading such segments word by word from global memory).
+            auto stage_tile = [&](const TileInfo &ti, unsigned long long base, int which) {
+                if (ti.room) {
                     const uint32_t dst = sbuf_g + (uint32_t)which * sbuf_bytes;
-                    const unsigned char *src = reinterpret_cast<const unsigned char *>(a.stream) + (ti.base >> 3);
-                    const uint32_t n16 = (uint32_t)(ti.bits >> 7);
+                    const unsigned char *src = reinterpret_cast<const unsigned char *>(a.stream) + (base >> 3);
+                    const uint32_t n16 = ti.bits >> 7;
                     for (uint32_t i = tg; i < n16; i += n_thr) cp_async_16(dst + i * 16u, src + (size_t)i * 16u, 16u);
                 }
                 cp_async_commit();
             };
 
-            TileInfo cur = tile_info(grp), nxt = tile_info(grp + G);
-            stage_tile(cur, 0);
+            const RawTile first = load_tile(grp);
+            RawTile ahead = load_tile(grp + G);
+            unsigned long long tile_base;
+            TileInfo cur = tile_info(first, tile_base);
+            stage_tile(cur, tile_base, 0);
+            cur.landed = true;
             int li = 0;
             // (a thread whose wait ran out keeps walking the tiles without decoding: the group's
             // barriers and the hand-over to the MMA thread need every thread's arrival)
-            for (long long tl = grp; tl < my_tiles; tl += G, ++li) {
-                const long long tile = block + tl * blocks;
+            for (int tl = grp; tl < my_tiles; tl += G, ++li) {
+                const long long tile = block + (long long)tl * blocks;
                 // start of every chunk = sum of the lengths before it in the tile (chunk order: pixel,
                 // then part of the pixel): scan over the pixels' totals
                 const unsigned int len0 = cur.l01 & 0xffffu, len1 = cur.l01 >> 16, len2 = cur.l23 & 0xffffu, len3 = cur.l23 >> 16;
@@ -376,8 +435,15 @@ __device__ __forceinline__ void decode_tiles(const DecodeArgs &a, const SmemLayo
                 // every thread's part of this tile's segment has landed, and every thread is done
                 // with the tile before: its stream buffer may take the next tile's segment
                 named_bar_sync(bar_id, n_thr);
-                stage_tile(nxt, (li + 1) & 1);
-                const TileInfo after = tile_info(tl + 2 * G);   // offsets two tiles ahead: their latency hides behind the decode
+                if (!cur.landed) {
+                    if (cur.ok) stage_tile(cur, __ldg(a.tile_off + tile), cur.room == 2 ? 0 : li & 1);
+                    cp_async_wait<0>();
+                    named_bar_sync(bar_id, n_thr);
+                }
+                TileInfo nxt = tile_info(ahead, tile_base);
+                nxt.landed = cur.room + nxt.room <= 2;
+                if (nxt.landed) stage_tile(nxt, tile_base, nxt.room == 2 ? 0 : (li + 1) & 1);
+                ahead = load_tile(tl + 2 * G);
                 unsigned int before = 0, tile_total = 0;
                 const int n_wq = (n_work / tpp + 31) / 32;          // warps of one thread set
 #pragma unroll
@@ -393,17 +459,20 @@ __device__ __forceinline__ void decode_tiles(const DecodeArgs &a, const SmemLayo
                     if (S == 2) { chunk_start += len0; my_len0 = len1; }
                     else { chunk_start += len0 + len1; my_len0 = len2; my_len1 = len3; }
                 }
+                chunk_start = __shfl_sync(0xffffffffu, chunk_start, src_lane);
+                my_len0 = __shfl_sync(0xffffffffu, my_len0, src_lane);
+                if (S == 4) my_len1 = __shfl_sync(0xffffffffu, my_len1, src_lane);
 
-                const long long ch = tile * chunks_per_tile + (long long)t * (cp > 1 ? 1 : S);
+                const long long ch = tile * chunks_per_tile + (long long)tc * (cp > 1 ? 1 : S);
                 bool active = cur.ok && owner && ch < a.n_chunks;
-                bool bad = !cur.ok || (unsigned long long)tile_total > cur.bits;
+                bool bad = !cur.ok || tile_total > cur.bits;
                 if (bad) active = false;
-                const long long px0 = tile * TC_TILE_PIXELS + (long long)t * cp;
+                const long long px0 = tile * TC_TILE_PIXELS + (long long)tc * cp;
                 const int n_pix = active ? (int)min((long long)cp, a.pixels - px0) : 0;
-                const uint32_t seg_addr = sbuf_g + (uint32_t)(li & 1) * sbuf_bytes;
+                const uint32_t seg_addr = sbuf_g + (cur.room == 2 ? 0u : (uint32_t)(li & 1) * sbuf_bytes);
                 // dense tiles are decoded symbol by symbol
                 const bool runs = a.modal >= 0 &&
-                                  cur.bits * 128ull <= (unsigned long long)kDenseBits128 * (unsigned long long)a.k * TC_TILE_PIXELS;
+                                  cur.bits <= (unsigned int)(kDenseBits128 * TC_TILE_PIXELS / 128) * (unsigned int)a.k;
                 const uint32_t wait_parity = (uint32_t)((li & 1) ^ 1);   // the buffer's hand-back by the tile before this one
 
                 // Walks this thread's chunks.  Control flow is kept uniform across the warp: the lanes
@@ -415,7 +484,7 @@ __device__ __forceinline__ void decode_tiles(const DecodeArgs &a, const SmemLayo
                     uint32_t expect = 0;               // bits the chunks decoded so far should have taken
                     for (int pp = 0; pp < cp; ++pp) {
                         const bool decode = pp < n_pix;
-                        const uint32_t row = (uint32_t)(t * cp + pp);
+                        const uint32_t row = column_of((uint32_t)(tc * cp + pp));
                         const uint32_t row_addr = opnd_g + (row >> 3) * 128u + (row & 7u) * 16u;
                         int ready = p_first;           // panels [p_first, ready) of the warp's rows are handed back and filled
                         // waits for panel p to be handed back by the MMAs of the tile before, then fills this
@@ -446,8 +515,8 @@ __device__ __forceinline__ void decode_tiles(const DecodeArgs &a, const SmemLayo
                                 }
                                 if (decode) sts_v4(row_addr + (uint32_t)(k0 >> 3) * 2048u, pk[0], pk[1], pk[2], pk[3]);
                             }
+                            while (ready * kPanelK < ke) prepare(ready++, kd);
                             uint32_t pos = (uint32_t)kd, rem = decode ? (uint32_t)(ke - kd) : 0u;
-                            uint32_t ready_end = (uint32_t)(ready * kPanelK);
                             while (__any_sync(0xffffffffu, rem != 0u)) {
                                 r.refill();
                                 // a run of the modal symbol is a run of zero bits: at most 20 per step
@@ -458,7 +527,6 @@ __device__ __forceinline__ void decode_tiles(const DecodeArgs &a, const SmemLayo
                                 const bool sym = rem != 0u;            // a symbol follows the run
                                 const uint32_t e = lds_u32(lut_addr + (r.hi >> (32 - lb)) * 4u);
                                 r.take(sym ? e : 0u);
-                                while (__any_sync(0xffffffffu, sym && pos >= ready_end)) { prepare(ready++, kd); ready_end += kPanelK; }
                                 // coefficient pos of the row: core-matrix column pos / 8 (2048 bytes apart), 2 bytes per coefficient inside
                                 if (sym) sts_u16(row_addr + pos * 2u + (pos >> 3) * 2032u, e >> 16);
                                 pos += sym ? 1u : 0u;
@@ -472,9 +540,9 @@ __device__ __forceinline__ void decode_tiles(const DecodeArgs &a, const SmemLayo
                         }
                         while (ready < p_last) prepare(ready++, 0);
                     }
-                    if (cp > 1 && active && r.consumed() != len0) bad = true;
+                    if (cp > 1 && active && r.consumed() != my_len0) bad = true;
                 };
-                if (cur.ok && cur.staged) {
+                if (cur.room) {
                     BitReader<true> r;
                     if (active) r.init(seg_addr, nullptr, nullptr, chunk_start);
                     else r.idle();
@@ -482,7 +550,7 @@ __device__ __forceinline__ void decode_tiles(const DecodeArgs &a, const SmemLayo
                 } else {
                     BitReader<false> r;
                     if (active) {
-                        const uint32_t *seg = a.stream + (cur.base >> 5);
+                        const uint32_t *seg = a.stream + (__ldg(a.tile_off + tile) >> 5);
                         r.init(0u, seg, seg + (cur.bits >> 5), chunk_start);
                     } else r.idle();
                     decode_tile(r);
@@ -492,45 +560,24 @@ __device__ __forceinline__ void decode_tiles(const DecodeArgs &a, const SmemLayo
                 if (lane == 0) mbar_arrive(smem_u32(&s_bfull[grp]));
                 if (bad) tc_dev_set_status(a.status, TC_ERR_CORRUPT_STREAM);
                 cur = nxt;
-                nxt = after;
             }
             cp_async_wait<0>();
             if (!alive) tc_dev_set_status(a.status, TC_ERR_TIMEOUT);
         }
     } else if (warp < kMmaWarp) {
-        // ================= epilogue: all eight warps work on every item =================
-        // A thread owns one channel (its TMEM lane) of one block of 128 channels and 64 pixels of
-        // the item.  With two channel blocks an item is half a tile: warps 16-19 take the first
-        // block and warps 20-23 the second; with one block an item is a tile and the two warp sets
-        // split its pixels (TMEM columns) in halves.
-        const int set = (warp - kEpiWarp0) >> 2;
-        const int wq = warp & 3;                            // TMEM lane quarter of this warp
-        const int blk = n_blocks == 2 ? set : 0;
-        const int col_first = n_blocks == 2 ? 0 : 64 * set;
-        constexpr int col_count = 64;
-        const int ch = blk * 128 + wq * 32 + lane;
-        const bool ch_ok = ch < a.c;
+        // ================= epilogue =================
+        // An item is a tile's 128 pixels of one block of 128 channels.  Four warps serve each accumulator, so that the waits of one
+        // item run beside the work of another; a warp stores the 32 channels of its quarter of TMEM, 16 at a time.
+        const int warp = own_tid() >> 5, lane = own_tid() & 31;
+        const int mode = store_mode(a);
+        const int set = (warp - kEpiWarp0) >> 2, wq = warp & 3;
+        const int n_items = my_tiles * items;
+        const bool shared = n_items == 1;                         // one item only: half of the channels each
+        const int acc = shared ? 0 : set;
         const float step = (float)(a.step * a.basis_scale);        // the operand holds basis / basis_scale
-        const float bias = ch_ok ? a.dec_bias[ch] : 0.f;
         __nv_bfloat16 *out = reinterpret_cast<__nv_bfloat16 *>(a.xhat);
-        // With H*W a multiple of 4 every aligned group of four pixels lies inside one image and is
-        // 8-byte aligned (given an 8-byte aligned tensor); otherwise pixels are stored one by one.
-        // (and eight rows of a map fit 32 bits: with the step in 64 bits 256x14x14 x 4096 took 236 us instead of 221)
-        const bool vec = vector_stores(a);
-        const long long img_stride = (long long)a.c * a.hw;
-        const int ch_base = blk * 128 + wq * 32;            // first channel of this warp
-        // Transpose block: row = channel (64 bytes = 32 pixels); the four 16-byte pieces of a row are exchanged
-        // by XOR with (row / 2) % 4, so that neither the row writes nor the reads below collide.
-        const uint32_t tb = smem_u32(smem + L.tbuf) + (uint32_t)(warp - kEpiWarp0) * kTrWarpBytes;
-        const uint32_t tb_wr = tb + (uint32_t)lane * 64u, sw_wr = (uint32_t)((lane >> 1) & 3);
-        // Read phase: rows leave 8 pixels a lane (eight rows an instruction) where every group of 8 pixels is
-        // 16-byte aligned and inside one image, else 4 pixels a lane (four rows an instruction).
-        const bool vec8 = (a.hw & 7) == 0 && ((uintptr_t)a.xhat & 15u) == 0;
-        const int px_lane = vec8 ? 8 * (lane & 3) : 4 * (lane & 7);         // first pixel of this lane in a pass
-        const int r_sub = vec8 ? lane >> 2 : lane >> 3, r_step = vec8 ? 8 : 4;
-        const uint32_t tb_rd0 = tb + (uint32_t)r_sub * 64u, piece = (uint32_t)(px_lane >> 3), in_piece = (uint32_t)(px_lane & 7) * 2u;
         // two accumulator values -> two bf16: x_hat = step * acc + bias (one packed fused multiply-add)
-        auto convert = [&](uint32_t x0, uint32_t x1) {
+        auto convert = [&](uint32_t x0, uint32_t x1, float bias) {
             float f0, f1;
             asm("{\n\t.reg .b64 v, s, b;\n\t"
                 "mov.b64 v, {%2, %3};\n\t"
@@ -543,164 +590,184 @@ __device__ __forceinline__ void decode_tiles(const DecodeArgs &a, const SmemLayo
             const __nv_bfloat162 h = __floats2bfloat162_rn(f0, f1);
             return *reinterpret_cast<const uint32_t *>(&h);
         };
-        // Position of this lane's pixels: image and offset inside it of the block's first tile, moved on from
+        // Position of this lane's first pixel of a tile: image and offset inside it of the block's first tile, moved on from
         // tile to tile by a constant number of pixels (a division of 64-bit numbers per item was a fifth of
         // the epilogue's instructions).
-        const long long tile_step = (long long)blocks * TC_TILE_PIXELS;
-        const long long img_step = tile_step / a.hw;
-        const int sp_step = (int)(tile_step - img_step * a.hw);
-        const long long first_px = (long long)block * TC_TILE_PIXELS + col_first + px_lane;
-        long long tile_img = first_px / a.hw;
-        int tile_sp = (int)(first_px - tile_img * a.hw);
-        const int rows_left = min(32, a.c - ch_base) - r_sub;               // rows r_sub + k r_step below it exist
-        __nv_bfloat16 *const out_row = out + (long long)(ch_base + r_sub) * a.hw;
-        const uint32_t row_stride = (uint32_t)r_step * (uint32_t)a.hw;      // elements between the rows of two instructions
+        const int px_lane = mode == kRows16 ? 8 * (lane & 3) : mode == kRows8 ? 4 * lane : lane;
+        const unsigned int hw = (unsigned int)a.hw;
+        const long long px_step = (long long)blocks * TC_TILE_PIXELS * (items == 2 ? 1 : 2);
+        const unsigned int img_step = (unsigned int)(px_step / a.hw), sp_step = (unsigned int)(px_step - (long long)img_step * a.hw);
+        const long long first_px = ((long long)block + (items == 2 ? 0 : (long long)acc * blocks)) * TC_TILE_PIXELS + px_lane;
+        unsigned int tile_img = (unsigned int)(first_px / a.hw), tile_sp = (unsigned int)(first_px - (long long)tile_img * a.hw);
+        const int ch_base = (items == 2 ? set * 128 : 0) + wq * 32;         // first channel of this warp
+        const int h_first = shared ? set : 0, halves = min(shared ? set + 1 : 2, (a.c - ch_base) / 16);      // of 16 channels (C is a multiple of 16)
+        float bias[4];                                                      // of this thread's channels, eight apart
+#pragma unroll
+        for (int i = 0; i < 4; ++i) bias[i] = i < 2 * halves ? __ldg(a.dec_bias + ch_base + 8 * i + (lane >> 2)) : 0.f;
+        // The warp's block: row = channel (256 bytes); the halves of every 128 bytes of an odd row are exchanged, so that
+        // neither the row writes (two rows x 64 bytes a phase) nor the reads collide.
+        const uint32_t tb = smem_u32(smem + L.tbuf) + (uint32_t)(warp - kEpiWarp0) * kTrWarpBytes;
+        const uint32_t tb_wr = tb + (uint32_t)(lane >> 2) * 256u + (uint32_t)(lane & 3) * 16u, swap = (uint32_t)(lane & 4) << 4;
         bool alive = true;
-        const long long n_items = my_tiles * items;
+        const uint32_t trow = tmem_base + kAccBase + acc * kAccCols + ((uint32_t)(wq * 32) << 16);
         // (after a wait that ran out the warps keep walking the items: the MMA warp waits for their arrivals)
-        for (long long it = 0; it < n_items; ++it) {
-            const int acc = (int)(it & 1);
-            const long long tl = items == 2 ? (it >> 1) : it;
-            const int item = items == 2 ? (int)(it & 1) : 0;
-            const long long tile = block + tl * blocks;
-            const long long p_first = tile * TC_TILE_PIXELS + item * 64 + col_first;
-            const long long left = a.pixels - p_first;                       // pixels from this thread's first column on
-            const int n_valid = (int)(left < (long long)col_count ? (left < 0 ? 0 : left) : (long long)col_count);
-            // the first epilogue warp waits for the accumulator and lets the others in
-            if (warp == kEpiWarp0) {
-                if (alive) alive = mbar_wait(smem_u32(&s_tfull[acc]), (uint32_t)((it >> 1) & 1), 100u);
+        for (int it = acc; it < n_items; it += 2) {
+            const unsigned int tile = block + (unsigned int)(items == 2 ? it >> 1 : it) * blocks;
+            const int n_valid = tile == (unsigned int)a.n_tiles - 1u ? (int)(a.pixels - (a.n_tiles - 1) * TC_TILE_PIXELS) : TC_TILE_PIXELS;
+            // one warp waits for the accumulator and lets the others in
+            if (wq == 0) {
+                if (alive) alive = mbar_wait(smem_u32(&s_tfull[acc]), (uint32_t)((it >> 1) & 1), 50u);
                 tc_fence_before_sync();
             }
-            named_bar_sync(kBarEpi, 256);
+            named_bar_sync(kBarEpi + set, 128);
             tc_fence_after_sync();
-            const uint32_t trow = tmem_base + kAccBase + acc * kAccCols + (n_blocks == 2 ? blk * 64 : 0) + ((uint32_t)(wq * 32) << 16) + col_first;
-            if (vec) {
-                long long img = tile_img;
-                int sp = tile_sp + item * 64;
-                while (sp >= a.hw) { sp -= a.hw; ++img; }
+            uint32_t r[16];                                       // 32 pixels
+            if (h_first < halves) tmem_ld_16x256b_x4(trow + ((uint32_t)(16 * h_first) << 16), r);
+            auto hand_back = [&] {
+                tc_fence_before_sync();
+                if (!shared) named_bar_arrive(kBarAccFree + acc, 128 + 32);
+            };
+            if (h_first >= halves) hand_back();
 #pragma unroll 1
-                for (int c0 = 0; c0 < col_count; c0 += 32) {
-                    uint32_t r[32];
-                    tmem_ld_32x32b_x32(trow + c0, r);
+            for (int h = h_first; h < halves; ++h) {
+                const float bias0 = h ? bias[2] : bias[0], bias1 = h ? bias[3] : bias[1];
+                unsigned int img = tile_img, sp = tile_sp;
+                // this lane's place of the tensor in the first of the 16 channels, `pixels` further on each time
+                auto place = [&](unsigned int pixels) {
+                    __nv_bfloat16 *at = out + ((long long)img * a.c + (ch_base + 16 * h)) * a.hw + sp;
+                    sp += pixels;
+                    while (sp >= hw) { sp -= hw; ++img; }
+                    return at;
+                };
+#pragma unroll
+                for (int b = 0; b < 4; ++b) {
                     tmem_ld_wait(r);
+                    uint32_t w[2][4];                             // [row, eight apart][two pixels of eight]
 #pragma unroll
-                    for (int q = 0; q < 4; ++q)
-                        sts_v4(tb_wr + (((uint32_t)q ^ sw_wr) << 4), convert(r[8 * q], r[8 * q + 1]), convert(r[8 * q + 2], r[8 * q + 3]),
-                               convert(r[8 * q + 4], r[8 * q + 5]), convert(r[8 * q + 6], r[8 * q + 7]));
-                    __syncwarp();
-                    const int rows = c0 + px_lane < n_valid ? rows_left : 0;
-                    __nv_bfloat16 *dst = out_row + img * img_stride + sp;
-                    if (vec8) {
-#pragma unroll
-                        for (int k = 0; k < 4; ++k) {
-                            uint32_t v[4];
-                            const uint32_t row = (uint32_t)(r_sub + 8 * k);
-                            asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3])
-                                         : "r"(tb_rd0 + k * 512u + ((piece ^ ((row >> 1) & 3u)) << 4)));
-                            if (8 * k < rows) *reinterpret_cast<uint4 *>(dst) = make_uint4(v[0], v[1], v[2], v[3]);
-                            dst += row_stride;
-                        }
+                    for (int g = 0; g < 4; ++g) {
+                        w[0][g] = convert(r[4 * g], r[4 * g + 1], bias0);
+                        w[1][g] = convert(r[4 * g + 2], r[4 * g + 3], bias1);
+                    }
+                    // the next columns are on their way, or the accumulator handed back, while these are stored
+                    if (b < 3) tmem_ld_16x256b_x4(trow + ((uint32_t)(16 * h) << 16) + 32 * (b + 1), r);
+                    else if (h + 1 < halves) tmem_ld_16x256b_x4(trow + (16u << 16), r);
+                    else hand_back();
+                    if (mode == kRows16) {
+                        const bool ok = 32 * b + px_lane < n_valid;
+                        uint4 *at = reinterpret_cast<uint4 *>(place(32) + (long long)(lane >> 2) * a.hw);
+                        if (ok) *at = make_uint4(w[0][0], w[0][1], w[0][2], w[0][3]);
+                        if (ok) at[a.hw] = make_uint4(w[1][0], w[1][1], w[1][2], w[1][3]);          // eight rows on
                     } else {
+                        const uint32_t at = tb_wr + 128u * (b >> 1) + ((64u * (b & 1)) ^ swap);
+                        sts_v4(at, w[0][0], w[0][1], w[0][2], w[0][3]);
+                        sts_v4(at + 2048u, w[1][0], w[1][1], w[1][2], w[1][3]);
+                    }
+                }
+                if (mode == kRows8) {
+                    __syncwarp();
+                    __nv_bfloat16 *at = place(0);
+                    const bool ok = px_lane < n_valid;
+#pragma unroll 4
+                    for (int k = 0; k < 16; ++k) {
+                        uint32_t lo, hi;
+                        asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(lo), "=r"(hi) : "r"(tb + k * 256u + (((uint32_t)lane * 8u) ^ ((k & 1u) << 6))));
+                        if (ok) *reinterpret_cast<uint2 *>(at) = make_uint2(lo, hi);
+                        at += a.hw;
+                    }
+                    __syncwarp();                               // the block may be overwritten
+                } else if (mode == kRowsAny) {
+                    __syncwarp();
+                    __nv_bfloat16 *at[4];
 #pragma unroll
-                        for (int k = 0; k < 8; ++k) {
-                            uint32_t lo2, hi2;
-                            const uint32_t row = (uint32_t)(r_sub + 4 * k);
-                            asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(lo2), "=r"(hi2)
-                                         : "r"(tb_rd0 + k * 256u + ((piece ^ ((row >> 1) & 3u)) << 4) + in_piece));
-                            if (4 * k < rows) *reinterpret_cast<uint2 *>(dst) = make_uint2(lo2, hi2);
-                            dst += row_stride;
+                    for (int b = 0; b < 4; ++b) at[b] = place(32);
+#pragma unroll 1
+                    for (int k = 0; k < 16; ++k) {
+#pragma unroll
+                        for (int b = 0; b < 4; ++b) {
+                            unsigned short v;
+                            asm volatile("ld.shared.u16 %0, [%1];" : "=h"(v) : "r"(tb + k * 256u + (((uint32_t)lane * 2u + 64u * b) ^ ((k & 1u) << 6))));
+                            if (32 * b + lane < n_valid) *reinterpret_cast<unsigned short *>(at[b]) = v;
+                            at[b] += a.hw;
                         }
                     }
-                    sp += 32;
-                    while (sp >= a.hw) { sp -= a.hw; ++img; }
-                    __syncwarp();                                   // the block may be overwritten
-                }
-                if (items == 1 || item == 1) {
-                    tile_img += img_step;
-                    tile_sp += sp_step;
-                    if (tile_sp >= a.hw) { tile_sp -= a.hw; ++tile_img; }
-                }
-            } else {
-                // position of the first pixel; from there on it moves incrementally
-                const long long img0 = left > 0 ? p_first / a.hw : 0;
-                int s = left > 0 ? (int)(p_first - img0 * a.hw) : 0;
-                __nv_bfloat16 *dst = out + img0 * img_stride + (long long)(ch_ok ? ch : 0) * a.hw + s;
-                for (int c0 = 0; c0 < col_count; c0 += 16) {
-                    uint32_t r[16];
-                    tmem_ld_32x32b_x16(trow + c0, r);
-                    tmem_ld_wait();
-#pragma unroll
-                    for (int i = 0; i < 16; ++i) {
-                        float f = fmaf(__uint_as_float(r[i]), step, bias);
-                        if constexpr (kRelu) f = fmaxf(f, 0.f);
-                        if (ch_ok && c0 + i < n_valid) *dst = __float2bfloat16_rn(f);
-                        s += 1;
-                        const bool wrap = s == a.hw;            // the next pixel starts the next image
-                        dst += wrap ? 1 + img_stride - a.hw : 1;
-                        s = wrap ? 0 : s;
-                    }
+                    __syncwarp();
                 }
             }
-            tc_fence_before_sync();
-            named_bar_arrive(kBarAccFree + acc, 256 + 32);
+            tile_img += img_step;
+            tile_sp += sp_step;
+            if (tile_sp >= hw) { tile_sp -= hw; ++tile_img; }
         }
         if (!alive && lane == 0) tc_dev_set_status(a.status, TC_ERR_TIMEOUT);
     } else {
-        // ================= MMA issuers =================
-        // Two warps, one per accumulator: with two channel blocks warp w issues item w (pixels 64 w ...)
-        // of every tile, with one block the tiles alternate between the warps.  An MMA leaves its
-        // issuing thread about every 64 cycles at best and an item is K / 16 of them per channel block,
-        // so one warp alone would be the slowest stage of the kernel.  The whole warp walks the loop
-        // and waits on the barriers; lane 0 issues, through instructions that carry their own guard
-        // (no branch around an MMA).
-        // A = transposed basis in tensor memory (128 channels per instruction), B = the decoded
-        // symbols of the item's pixels (rows of the group's operand buffer).
-        named_bar_sync(kBarBasis, 256 + 64);
-        tc_fence_after_sync();
-        const int w = warp - kMmaWarp;
-        const uint32_t issuer = lane == 0 ? 1u : 0u;
-        const int np = items == 2 ? 64 : TC_TILE_PIXELS;          // pixels per work item
-        const uint32_t idesc = make_idesc_bf16(128, np, /*A K-major*/ false, /*B K-major*/ false);
-        const uint32_t a_blk1 = (uint32_t)(a.k / 2);               // columns between the two channel blocks of the basis
-        const int n_k16 = a.k >> 4;
-        const uint32_t d_tmem = tmem_base + kAccBase + w * kAccCols;
-        int buf = items == 2 ? 0 : w % G;                         // operand buffer (VLD group) of the tile, and the parity of its turn
-        uint32_t turn = items == 2 ? 0u : (uint32_t)(w / G) & 1u;
-        bool alive = true;
-        for (long long tl = items == 2 ? 0 : w; tl < my_tiles; tl += items == 2 ? 1 : 2) {
-            const long long it = items == 2 ? 2 * tl + w : tl;       // index of the work item: item it uses accumulator it % 2 = w
-            // The accumulator first: the epilogue takes the items in order, so once it has drained the item before the last
-            // the MMAs of that tile and of all before it are done, and the wait for the operand cannot mistake an earlier
-            // turn of the buffer for this one (the two warps share the buffers where the groups are odd in number).
-            if (it >= 2) named_bar_sync(kBarAccFree + w, 256 + 32);   // the epilogue has drained the accumulator
-            // (after a wait that ran out the warp keeps walking the items: the epilogue waits for its commits)
-            if (alive) alive = mbar_wait(smem_u32(&s_bfull[buf]), turn);     // the group's VLD threads have arrived
-            __syncwarp();
-            // the operand was written with ordinary stores by threads that have arrived on the
-            // barrier: one proxy fence here, between that synchronisation and the MMA's
-            // operand reads, orders them for all writers
-            fence_proxy_async_smem();
-            const uint64_t b_base = make_smem_desc(opnd_addr + (uint32_t)buf * L.opnd_bytes, 2048, 128);
-            const uint32_t b_hi = (uint32_t)(b_base >> 32);
-            __syncwarp();
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 40;");
+        if (warp == kMmaWarp) {
+            // ================= MMA issuer =================
+            // The items in order, on the two accumulators in turn.  The whole warp walks the loop
+            // and waits on the barriers; lane 0 issues, through instructions that carry their own guard
+            // (no branch around an MMA).  An MMA leaves its issuing thread every 64 cycles at best, with 64 columns as
+            // with 128: items of 64 pixels of both blocks took twice as many instructions (125 us for the products of
+            // 256x14x14 x 4096 alone) and a warp per accumulator.
+            // A = transposed basis in tensor memory (128 channels per instruction), B = the decoded
+            // symbols of the tile (the group's operand buffer).
+            named_bar_sync(kBarBasis, 256 + 32);
             tc_fence_after_sync();
-            // rows 64 w ... of the buffer (two blocks): eight-row groups are 128 bytes apart; a step of 16
-            // coefficients moves the start address on by two core-matrix columns of 2048 bytes
-            uint32_t b_lo = (uint32_t)b_base + (items == 2 ? (uint32_t)w * (1024u >> 4) : 0u);
-            uint32_t a_col = tmem_base;
-            for (int q = 0; q < n_k16; ++q) {
-                mma_bf16_ts_guarded(d_tmem, a_col, b_lo, b_hi, idesc, q ? 1u : 0u, issuer);
-                if (n_blocks == 2) mma_bf16_ts_guarded(d_tmem + 64, a_col + a_blk1, b_lo, b_hi, idesc, q ? 1u : 0u, issuer);
-                // a finished panel goes back to the VLD threads (when every item of the tile has read it)
-                if ((q & 1) || q == n_k16 - 1) mma_commit_guarded(smem_u32(&s_empty[buf][q >> 1]), issuer);
-                b_lo += 4096u >> 4;
-                a_col += 8;
+            const uint32_t issuer = (own_tid() & 31) == 0 ? 1u : 0u;
+            const uint32_t idesc = make_idesc_bf16(128, TC_TILE_PIXELS, /*A K-major*/ false, /*B K-major*/ false);
+            const int n_k16 = a.k >> 4;
+            int buf = 0;                                              // operand buffer (VLD group) of the tile, and the parity of its turn
+            uint32_t turn = 0;
+            int it = 0;
+            bool alive = true;
+            for (int tl = 0; tl < my_tiles; ++tl) {
+                // (after a wait that ran out the warp keeps walking the items: the epilogue waits for its commits)
+                if (alive) alive = mbar_wait(smem_u32(&s_bfull[buf]), turn);     // the group's VLD threads have arrived
+                __syncwarp();
+                // the operand was written with ordinary stores by threads that have arrived on the
+                // barrier: one proxy fence here, between that synchronisation and the MMA's
+                // operand reads, orders them for all writers
+                fence_proxy_async_smem();
+                const uint64_t b_base = make_smem_desc(opnd_addr + (uint32_t)buf * L.opnd_bytes, 2048, 128);
+                const uint32_t b_hi = (uint32_t)(b_base >> 32);
+                for (int blk = 0; blk < items; ++blk, ++it) {
+                    const int acc = it & 1;
+                    const uint32_t d_tmem = tmem_base + kAccBase + acc * kAccCols;
+                    if (it >= 2) named_bar_sync(kBarAccFree + acc, 128 + 32);     // the epilogue has drained the accumulator
+                    __syncwarp();
+                    tc_fence_after_sync();
+                    // eight-row groups are 128 bytes apart; a step of 16 coefficients moves the start address on by two
+                    // core-matrix columns of 2048 bytes
+                    uint32_t b_lo = (uint32_t)b_base;
+                    uint32_t a_col = tmem_base + (uint32_t)(blk * (a.k / 2));
+                    int q = 0;
+                    auto step = [&] {
+                        mma_bf16_ts_guarded(d_tmem, a_col, b_lo, b_hi, idesc, q ? 1u : 0u, issuer);
+                        b_lo += 4096u >> 4;
+                        a_col += 8;
+                        ++q;
+                    };
+                    // a panel that the last item has read goes back to the VLD threads
+                    auto panel_read = [&] {
+                        if (blk == items - 1) mma_commit_guarded(smem_u32(&s_empty[buf][(q - 1) / (kPanelK / 16)]), issuer);
+                    };
+                    // (eight at a time: an instruction of this warp waits its turn among the others', and a turn of a rolled loop around one
+                    // MMA took 140 cycles)
+                    while (q + 8 <= n_k16) {
+#pragma unroll
+                        for (int i = 0; i < 8; ++i) step();
+                        panel_read();
+                    }
+                    if (q + 4 <= n_k16) {
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) step();
+                    }
+                    while (q < n_k16) step();
+                    if (n_k16 % 8 != 0) panel_read();
+                    mma_commit_guarded(smem_u32(&s_tfull[acc]), issuer);
+                }
+                if (++buf == G) { buf = 0; turn ^= 1u; }
             }
-            mma_commit_guarded(smem_u32(&s_tfull[w]), issuer);
-            buf += items == 2 ? 1 : 2;
-            if (buf >= G) { buf -= G; turn ^= 1u; }
+            if (!alive && issuer) tc_dev_set_status(a.status, TC_ERR_TIMEOUT);
         }
-        if (!alive && issuer) tc_dev_set_status(a.status, TC_ERR_TIMEOUT);
     }
 
     // ---- teardown ---------------------------------------------------------------------
@@ -739,7 +806,7 @@ static SmemLayout runs_layout(const tc_ctx *ctx, const DecodeArgs &a)
     // (a dense tile's segment is at most 3 % longer than the mean)
     const double tile_bytes = a.mean_tile_bytes > 0 ? a.mean_tile_bytes : std::max(2.5, (double)a.code_bits) * a.k * TC_TILE_PIXELS / 8;
     const uint32_t want = (uint32_t)std::min(1.03 * tile_bytes, 1e6);
-    return smem_layout(a.k, 1 << a.lut_bits, (group_work(a.splits, a.chunk_pixels) + 31) / 32, want, ctx->max_smem_optin - kStaticSmem);
+    return smem_layout(a.k, 1 << a.lut_bits, (group_work(a.splits, a.chunk_pixels) + 31) / 32, want, store_mode(a) != kRows16, ctx->max_smem_optin - kStaticSmem);
 }
 
 bool tc_decode_runs_supported(const tc_ctx *ctx, const DecodeArgs &a)
@@ -766,13 +833,12 @@ tc_status tc_launch_decode_runs(const tc_ctx *ctx, const DecodeArgs &a, cudaStre
     return cudaGetLastError() == cudaSuccess ? TC_OK : TC_ERR_CUDA;
 }
 
-// us that a tile takes a block: 2.0 with 64 coefficients at 1.1 bits each, 2.55 with 128, 5.0 with 256 (two VLD groups instead of four
-// and eight), 10.7 with 256 at 4.1 bits (8 to 42 tiles a block, after the first); 7.0 with 32 and 43 with 256 where pixels are stored one by one
+// us that a tile takes a block: 1.6 with 64 coefficients at 1.1 bits each, 1.8 with 128, 2.7 with 160 (two items a tile), 3.5 with 256; 2.9
+// with 128 at 4.1 bits, 5.8 with 256; 0.9 more for every 128 channels where rows start anywhere (40 tiles a block, less the first)
 double tc_decode_runs_tile_us(const DecodeArgs &a)
 {
-    if (!vector_stores(a)) return 2.0 + 0.165 * a.c;
     const double bits = a.mean_tile_bytes > 0 ? a.mean_tile_bytes * 8.0 / TC_TILE_PIXELS : (double)a.code_bits * a.k;
-    return 1.42 + 0.011 * std::max(0, a.k - 128) + 0.0075 * bits;
+    return 1.25 + (a.c > 128 ? 0.9 : 0.0) + 0.0035 * std::max(0, a.k - 128) + 0.003 * bits + (store_mode(a) == kRowsAny ? 0.9 * ((a.c + 127) / 128) : 0.0);
 }
 
 // Decodes tensors that tc_decode_runs_supported takes, all with the same `relu`, on `sms` SMs, in list_launches launches.

@@ -270,6 +270,40 @@ def test_staging_ring_of_the_resident_encoder(ctx, c, bits, ratio):
     m.close(); cb.close()
 
 
+# Run-skipping decoder, how channel rows leave: 16 and 8 bytes a thread and a pixel a thread (H*W a multiple of 8, of 4, of neither;
+# tensors that start anywhere), one item for the whole block and several, one block of 128 channels and two with remainders, last
+# tiles of a pixel, 64 and 127, images shorter than a tile.  The stream does not depend on how the pixels are laid out: one image of one row is the
+# same tensor through other stores.  Against the fp64 kernels too (neighbouring bf16 numbers).
+@pytest.mark.parametrize("c,h,w,n", [(16, 1, 1, 1), (16, 8, 8, 3), (32, 4, 3, 11), (48, 7, 7, 5), (64, 3, 43, 1), (80, 16, 16, 1), (128, 9, 7, 65), (128, 2, 2, 600),
+                                     (144, 2, 64, 3), (176, 14, 14, 7), (208, 5, 5, 51), (256, 1, 129, 1), (256, 8, 12, 199), (112, 1, 1, 19000)])
+def test_rows_of_the_run_skipping_decoder(ctx, c, h, w, n):
+    params = fm.layer_params(fm.LayerSpec(c, h, w, 0.9, None, 21000 + c + h))
+    cal = fm.make_maps(params, max(4, 30000 // (h * w)), calib=True, dtype=torch.bfloat16, device="cuda")
+    x = fm.make_maps(params, n, dtype=torch.bfloat16, device="cuda")
+    m = tc.tc_fit_pca(ctx, cal, 4)
+    cb = tc.tc_build_codebook(ctx, m, tc.tc_stats(ctx, m, None, cal).hist)
+    enc = tc.tc_encode(ctx, m, cb, x)
+    got = tc.tc_decode(ctx, m, cb, enc, x.shape, x.dtype)
+    assert tc.tc_get_status(ctx) == 0 and tc.tc_last_path(ctx, True) == 1
+    row = got.transpose(0, 1).reshape(c, -1)
+    for shape in ((1, c, 1, n * h * w), (n * h * w, c, 1, 1)):
+        assert torch.equal(row, tc.tc_decode(ctx, m, cb, enc, shape, x.dtype).transpose(0, 1).reshape(c, -1))
+    for offset in (1, 2, 4):
+        buf = torch.full((x.numel() + 16,), 7.0, dtype=x.dtype, device="cuda")
+        part = buf[offset:offset + x.numel()].view(x.shape)
+        tc.tc_decode(ctx, m, cb, enc, x.shape, x.dtype, out=part)
+        assert torch.equal(part, got)
+        assert bool((buf[:offset] == 7.0).all()) and bool((buf[offset + x.numel():] == 7.0).all())
+    assert tc.tc_get_status(ctx) == 0 and tc.tc_last_path(ctx, True) == 1
+    tc.tc_force_exact_path(ctx, 1)
+    want = tc.tc_decode(ctx, m, cb, enc, x.shape, x.dtype)
+    assert tc.tc_get_status(ctx) == 0
+    tc.tc_force_exact_path(ctx, 0)
+    a, b = got.float(), want.float()
+    assert bool(((a - b).abs() <= 2.0 ** -7 * b.abs() + 1e-6 * float(b.abs().max())).all())
+    m.close(); cb.close()
+
+
 # Run-skipping decoder, stream buffers sized by the rate: three groups and one work item per tile (128 and 112
 # channels), buffers above 16 KB, segments that fit no buffer, and hints that are too small or too large -- the hint
 # changes how tiles are staged, never the tensor.  Against the fp64 kernels on the same stream.
