@@ -268,6 +268,7 @@ __device__ __forceinline__ void decode_tiles(const DecodeArgs &a, const SmemLayo
     const int items = n_blocks;                                // work items per tile: its channel blocks
 
     // ---- set-up ---------------------------------------------------------------------
+    chain_next();
     if (tid < G * (kMaxPanels + 1)) {
         const int g = tid / (kMaxPanels + 1), p = tid - g * (kMaxPanels + 1);
         if (p < kMaxPanels) mbar_init(smem_u32(&s_empty[g][p]), 1);                     // the commit of the tile's last item
@@ -409,6 +410,7 @@ __device__ __forceinline__ void decode_tiles(const DecodeArgs &a, const SmemLayo
                 cp_async_commit();
             };
 
+            chain_wait();                                        // the stream
             const RawTile first = load_tile(grp);
             RawTile ahead = load_tile(grp + G);
             unsigned long long tile_base;
@@ -610,6 +612,7 @@ __device__ __forceinline__ void decode_tiles(const DecodeArgs &a, const SmemLayo
         const uint32_t tb_wr = tb + (uint32_t)(lane >> 2) * 256u + (uint32_t)(lane & 3) * 16u, swap = (uint32_t)(lane & 4) << 4;
         bool alive = true;
         const uint32_t trow = tmem_base + kAccBase + acc * kAccCols + ((uint32_t)(wq * 32) << 16);
+        chain_wait();                                            // earlier readers of the tensor
         // (after a wait that ran out the warps keep walking the items: the MMA warp waits for their arrivals)
         for (int it = acc; it < n_items; it += 2) {
             const unsigned int tile = block + (unsigned int)(items == 2 ? it >> 1 : it) * blocks;
@@ -829,8 +832,7 @@ tc_status tc_launch_decode_runs(const tc_ctx *ctx, const DecodeArgs &a, cudaStre
     if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)l.total) != cudaSuccess)
         return TC_ERR_CUDA;
     const unsigned int grid = (unsigned int)((a.n_tiles < ctx->sm_count) ? a.n_tiles : ctx->sm_count);
-    kernel<<<grid, kThreads, l.total, s>>>(a, l);
-    return cudaGetLastError() == cudaSuccess ? TC_OK : TC_ERR_CUDA;
+    return launch_first(a.alone, kernel, grid, kThreads, l.total, s, a, l) == cudaSuccess ? TC_OK : TC_ERR_CUDA;
 }
 
 // us that a tile takes a block: 1.6 with 64 coefficients at 1.1 bits each, 1.8 with 128, 2.7 with 160 (two items a tile), 3.5 with 256; 2.9

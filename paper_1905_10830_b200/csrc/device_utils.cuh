@@ -33,7 +33,8 @@ __device__ __forceinline__ unsigned long long global_timer_ns()
 
 // Kernels of one call that follow each other (launch_chained): a kernel lets the next one start setting up as soon
 // as all its own blocks run, and waits for what the one before it wrote -- and everything before that -- ahead of the
-// first access to it.  What it reads from the kernel before it does not go through the read-only path.
+// first access to it.  The last kernel of a call does so after its own wait: with the kernels of four calls' halves set up behind one
+// another a round trip of 256x14x14 f32 took 48 us instead of 43.  What it reads from the kernel before it does not go through the read-only path.
 __device__ __forceinline__ void chain_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 

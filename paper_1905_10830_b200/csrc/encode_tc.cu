@@ -251,6 +251,7 @@ __device__ __forceinline__ void encode_tiles(const EncodeArgs &a, const Plan &pl
     const int n_panels = (a.c + kPanelCh - 1) / kPanelCh;
 
     // ---- set-up ---------------------------------------------------------------------
+    chain_next();                                             // (a decoder that follows is set up meanwhile)
     if (tid < 2) s_overflow[tid] = 0;
     if (tid == 0) {
         for (int s = 0; s < n_stages; ++s) { mbar_init(smem_u32(&s_full[s]), 128); mbar_init(smem_u32(&s_empty[s]), 1); }
@@ -283,7 +284,6 @@ __device__ __forceinline__ void encode_tiles(const EncodeArgs &a, const Plan &pl
             s_bias[i] = b;
             s_bias_mid[i] = b - (float)(a.modal < 0 ? 0 : a.modal) / (float)(nsym - 1);   // the same, seen from the modal symbol's level
         }
-        for (long long i = (long long)block * kSetupThreads + setup_tid; i < a.other_words; i += (long long)blocks * kSetupThreads) a.other_state[i] = 0ull;
         if (enc_in_smem)
             for (int i = setup_tid; i < enc_entries; i += kSetupThreads) {
                 // per-layer table: (1 << length, code) pairs, so that appending a code to a register is
@@ -303,6 +303,7 @@ __device__ __forceinline__ void encode_tiles(const EncodeArgs &a, const Plan &pl
                 s_enc[2 * i + 1] = code;
                 (smem + L.len8)[i] = (unsigned char)len;
             }
+        for (long long i = (long long)block * kSetupThreads + setup_tid; i < a.other_words; i += (long long)blocks * kSetupThreads) a.other_state[i] = 0ull;
         tc_fence_before_sync();
         named_bar_sync(kSetupBar, kSetupThreads);
         tc_fence_after_sync();
@@ -1009,7 +1010,8 @@ tc_status tc_launch_encode_tc(const tc_ctx *ctx, const EncodeArgs &a, cudaStream
     const unsigned int grid = (unsigned int)((a.n_tiles < ctx->sm_count) ? a.n_tiles : ctx->sm_count);
     EncodeArgs args = a;
     void *params[] = {&args, &pl};
-    // cooperative launch: the grid must be co-resident, which is what makes the look-back safe
+    // cooperative launch: the grid must be co-resident, which is what makes the look-back safe (launched early as well it
+    // started no sooner)
     const cudaError_t err = cudaLaunchCooperativeKernel((void *)kernel, dim3(grid), dim3(kThreads), params, l.total, s);
     if (err != cudaSuccess) {
         if (getenv("TC_VERBOSE")) fprintf(stderr, "tc: encode launch failed: %s\n", cudaGetErrorString(err));

@@ -37,6 +37,7 @@ __global__ void __launch_bounds__(kPx * kRows) project_quantise_kernel(EncodeArg
     __shared__ __align__(16) double s_t[kRed][kOut + 2];
     const int tx = threadIdx.x, ty = threadIdx.y, t = ty * kPx + tx;
     chain_next();
+    chain_wait();
     const long long block = blockIdx.y * (long long)gridDim.x + blockIdx.x;
     for (long long i = block * (kPx * kRows) + t; i < a.clear_words; i += (long long)gridDim.x * gridDim.y * (kPx * kRows))
         reinterpret_cast<unsigned long long *>(a.ticket)[i] = 0ull;              // the coder's look-back state
@@ -160,6 +161,7 @@ __global__ void __launch_bounds__(kPx * kRows) reconstruct_kernel(DecodeArgs a, 
     };
     double acc[kPer] = {};
     chain_wait();                                      // the symbols
+    chain_next();
     fetch(0);
     for (int j0 = 0; j0 < a.k; j0 += kRed) {
         __syncthreads();                               // the previous step's operands have been used
@@ -233,6 +235,7 @@ __global__ void __launch_bounds__(TC_TILE_PIXELS * kMaxParts) pack_symbols_kerne
     if constexpr (kPerLayer)
         for (int i = t; i < nsym; i += blockDim.x) s_enc[i] = __ldg(a.enc + i);
     chain_wait();                                             // the symbols and the cleared look-back state
+    chain_next();
     if (t == 0 && rank == 0) {
         s_tile = (long long)atomicAdd(a.ticket, 1u);
         if constexpr (kCluster) {
@@ -592,6 +595,7 @@ __global__ void __launch_bounds__(kUnpackThreads) unpack_symbols_kernel(DecodeAr
         stage(tables, a.canon, (unsigned int)a.k * kCanonWords / 4u);
         if (sorted_staged) stage(s_sorted, a.sorted, (unsigned int)(a.k * nsym) / 16u);
     }
+    chain_wait();                                               // the stream; earlier readers of the workspace
     const long long tile = first_tile + blockIdx.x;
     const unsigned long long base = a.tile_off[tile], end = a.tile_off[tile + 1];
     const bool tile_ok = (base & 127ull) == 0 && (end & 127ull) == 0 && base <= end && end <= a.stream_bits;
@@ -770,9 +774,13 @@ tc_status tc_launch_project_quantise(const EncodeArgs &a, int dtype, uint8_t *sy
 {
     if (a.pixels <= 0) return TC_OK;
     const dim3 block(kPx, kRows), grid((unsigned int)((a.pixels + kPx - 1) / kPx), (unsigned int)((a.k + kOut - 1) / kOut));
-    if (dtype == TC_F32) project_quantise_kernel<float><<<grid, block, 0, s>>>(a, sym);
-    else project_quantise_kernel<__nv_bfloat16><<<grid, block, 0, s>>>(a, sym);
-    return cudaGetLastError() == cudaSuccess ? TC_OK : TC_ERR_CUDA;
+    void (*kernel)(EncodeArgs, uint8_t *) = dtype == TC_F32 ? project_quantise_kernel<float> : project_quantise_kernel<__nv_bfloat16>;
+    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSpreadMost) != cudaSuccess) return TC_ERR_CUDA;
+    // Early where that leaves the basis in L1: with several blocks an SM kept apart by shared memory wide layers lose (512x14x14 f32, 224
+    // blocks, 39.0 -> 43.6 us, 176x34x33 22.6 -> 24.3; 32x56x56 10.2 -> 8.3, 96x45x45 15.8 -> 15.3, 256x7x7 20.5 -> 18.8).
+    const long long blocks = (long long)grid.x * grid.y;
+    const size_t spread = a.alone && (blocks <= a.sms || a.c <= 128) ? spread_bytes(blocks, a.sms) : 0, own = 16 * 1024;      // (of static variables)
+    return launch_first(spread > 0, kernel, grid, block, spread > own ? spread - own : 0, s, a, sym) == cudaSuccess ? TC_OK : TC_ERR_CUDA;
 }
 
 tc_status tc_launch_reconstruct(const DecodeArgs &a, int dtype, const uint8_t *sym, cudaStream_t s)
@@ -861,8 +869,9 @@ static tc_status launch_unpack(const DecodeArgs &a, void *out, long long first_t
         : full ? unpack_symbols_kernel<kOperand, true, kOperand> : unpack_symbols_kernel<kOperand, true, false>;
     if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024) != cudaSuccess) return TC_ERR_CUDA;
     const size_t rows = full ? (size_t)(threads / 32) * kRowsWarpBytes : 0;
-    kernel<<<dim3((unsigned int)tiles, (unsigned int)parts), std::max(threads, least), tables + segment + rows, s>>>(a, out, first_tile, tables, segment);
-    return cudaGetLastError() == cudaSuccess ? TC_OK : TC_ERR_CUDA;
+    const size_t spread = a.alone ? spread_bytes(tiles * parts, sm_count) : 0, smem = std::max<size_t>(tables + segment + rows, spread);
+    return launch_first(spread > 0, kernel, dim3((unsigned int)tiles, (unsigned int)parts), std::max(threads, least), smem, s, a, out, first_tile, tables,
+                        segment) == cudaSuccess ? TC_OK : TC_ERR_CUDA;
 }
 
 tc_status tc_launch_unpack_symbols(const tc_ctx *ctx, const DecodeArgs &a, uint8_t *sym, cudaStream_t s)

@@ -200,7 +200,28 @@ inline cudaError_t launch_chained(bool early, void (*kernel)(P...), dim3 grid, d
     return err;
 }
 
-// The same, always early, in clusters of `blocks` along the grid's second dimension.
+// The first kernel of a call, early as well: launches that wait for one another's end start at multiples of 2.05 us here, and 4.1 apart at
+// least (a kernel that spins for 1 to 10 us, queued 300 times), which is a quarter of a small call's time.  The kernels ahead of it
+// in the stream may be anyone's: until it has called chain_wait such a kernel reads nothing but models and codebooks, which are
+// complete when the functions that make them return, and writes nothing.  Captured calls start after all that the graph
+// holds before them.  Small blocks that arrive early all pile onto the first SMs that have room (decode of 384x8x8 x 241, 121 blocks:
+// 25 -> 56 us), so they ask for as much shared memory as keeps them apart (spread_bytes; more than eight an SM start in their
+// turn: 64x56x56 x 64 with a table per channel, 1 568 blocks, 45 -> 56 us).
+constexpr size_t kSmBytes = 228 * 1024, kSpreadMost = 118 * 1024;
+inline size_t spread_bytes(long long blocks, int sm_count)
+{
+    const long long per_sm = (blocks + sm_count - 1) / sm_count;
+    return per_sm <= 1 ? kSpreadMost : per_sm <= 8 ? (kSmBytes / (size_t)(per_sm + 1) + 1023) & ~(size_t)1023 : 0;
+}
+template <typename... P, typename... A>
+inline cudaError_t launch_first(bool alone, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A &&...args)
+{
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    if (alone && cudaStreamIsCapturing(s, &capture) != cudaSuccess) { cudaGetLastError(); alone = false; }
+    return launch_chained(alone && capture == cudaStreamCaptureStatusNone, kernel, grid, block, smem, s, std::forward<A>(args)...);
+}
+
+// launch_chained, always early, in clusters of `blocks` along the grid's second dimension.
 template <typename... P, typename... A>
 inline cudaError_t launch_chained_cluster(int blocks, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A &&...args)
 {
