@@ -236,7 +236,8 @@ __device__ __forceinline__ void encode_tiles(const EncodeArgs &a, const Plan &pl
     __shared__ unsigned int s_padded[2][kSlots], s_stg_at[2][kSlots];   // bits of the tile, its place in the staging buffer
     __shared__ int s_store_cmd[2][kSlots];     // 1: copy the staged tile out, 2: nothing to copy, 3: stop
 
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    // (taken from lane 0: the compiler knows that the branches between the roles are the same for a whole warp)
+    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
     const int nsym = 1 << a.bits;
     constexpr bool enc_in_smem = !kPerChannel;
     constexpr bool kCanSkip = !kPerChannel && !kDebug && !kHist;     // blocks of modal symbols are passed over
@@ -308,7 +309,7 @@ __device__ __forceinline__ void encode_tiles(const EncodeArgs &a, const Plan &pl
         named_bar_sync(kSetupBar, kSetupThreads);
         tc_fence_after_sync();
     }
-    const uint32_t tmem_base = s_tmem_base;
+    const uint32_t tmem_base = __shfl_sync(0xffffffffu, s_tmem_base, 0);
 
     if (warp >= kLoaderWarp0 && warp < kMmaWarp) {
         // ================= loaders =================
@@ -396,8 +397,9 @@ __device__ __forceinline__ void encode_tiles(const EncodeArgs &a, const Plan &pl
                 tc_fence_after_sync();
                 const uint32_t d_tmem = tmem_base + acc * kAccCols;
                 uint32_t b_lo = (uint32_t)b_desc;
+#pragma unroll 4
                 for (int kp = 0; kp < n_panels; ++kp) {
-                    if (!mbar_wait(smem_u32(&s_full[s]), phase)) { alive = false; break; }
+                    if (alive) alive = mbar_wait(smem_u32(&s_full[s]), phase);
                     fence_proxy_async_smem();            // the loaders' copies, made visible to the tensor core
                     tc_fence_after_sync();
                     const uint32_t a_lo = a_desc_lo + (uint32_t)s * (kStageBytes >> 4);
