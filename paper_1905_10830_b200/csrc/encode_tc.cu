@@ -1,20 +1,24 @@
 // Fused tensor-core encode for bf16 tensors (Section 3: transform, quantiser, VLC).
 //
 // One persistent block per SM walks tiles of 128 consecutive pixels.  Warp roles:
-//   warps 0-7, 8-15  two epilogue groups (alternating tiles).  Within a group warps 0-3 own the
+//   warps 0-15       epilogue groups on tiles in turn: four of four warps up to 128 coefficients, a thread
+//                    per pixel, else two of eight.  Of these warps 0-3 own the
 //                    leading coefficients of the tile's 128 pixels and warps 4-7 the others, split
 //                    where the expected work of both is the same: TMEM -> registers, quantise, code.  A
 //                    thread packs its codes into a run of its own in shared memory, in one pass, and the
 //                    runs are joined once the tile's bit offsets are known (scan); tiles whose runs
 //                    would not fit take two passes over the accumulator, lengths first.
-//   warps 21, 22     one store warp per epilogue group: resolves the tile's stream offset by
-//                    look-back and copies the group's staging buffer out, while the group
+//   warps 21, 22     store warps, every other tile each: resolve the tile's stream offset by
+//                    look-back and copy the group's staging buffer out, while the group
 //                    already works on its next tile
 //   warps 16-19      loaders: 16- and 8-byte cp.async NCHW -> shared memory in the MMA's MN-major layout (128-byte swizzle)
 //   warp 20          one thread issues tcgen05.mma:  D[pixel][coef] = X_tile[pixel][c] * T[coef][c]
 // The basis T (bf16, K x C) stays resident in shared memory; the X tile streams through a ring
-// of 32-channel panels; the fp32 accumulators are double-buffered in tensor memory so that the
-// epilogue of one tile overlaps the loads and MMAs of the next.
+// of 32-channel panels; every group has an fp32 accumulator in tensor memory, so that the
+// epilogue of one tile overlaps the loads and MMAs of the next.  The time of a tile in a group is that of its chain (wait, codes,
+// scan, join, with barriers between), so the groups in flight set the rate where the accumulators leave room for four: us with two
+// groups of eight warps and with four of four, 96x112x112 x 128 203 -> 155, 64x56x56 x 512 at 4 and 8 bits 151 -> 122 and 173 -> 138,
+// 128x38x38 x 656 135 -> 110, 80x8x7 x 30965 169 -> 133, 32x44x44 x 2384 at 8 bits 373 -> 313.
 #include <algorithm>
 #include <cstdio>
 #include <cstdlib>
@@ -34,18 +38,19 @@ constexpr int kStageBytes = kPanelCh * TC_TILE_PIXELS * 2;   // 8 KB
 constexpr int kStaticSmem = 1024;                 // the static shared variables, up to the ring's alignment
 constexpr int kSlots = 4;                         // packed tiles of a group that may wait in its staging buffer
 constexpr int kMaxStagingBytes = 49152;           // a tile of 256 coefficients of 12 bits
-constexpr int kEpiWarps = 16;                     // 2 groups x (2 column halves x 4 lane quarters)
+constexpr int kEpiWarps = 16;                     // 2 groups x (2 column halves x 4 lane quarters), or 4 x 4 quarters
 constexpr int kLoaderWarp0 = kEpiWarps, kMmaWarp = kEpiWarps + 4;
 constexpr int kStoreWarp0 = kMmaWarp + 1;         // two store warps follow
 constexpr int kThreads = (kEpiWarps + 7) * 32;
 constexpr int kTmemCols = 512;
-constexpr int kSetupBar = 3;                      // named barrier of all warps but the loaders (1, 2: the epilogue groups)
-constexpr int kAccCols = 256;
+constexpr int kMaxGroups = 4;                     // epilogue groups (tiles in flight behind the MMAs)
+constexpr int kSetupBar = kMaxGroups + 1;         // named barrier of all warps but the loaders (1 ...: the epilogue groups)
 constexpr int kPairMaxBits = 6;                   // symbols of up to 6 bits can be coded two at a time (tables of up to 4096 entries)
 constexpr int kRunStep = 512;                     // bytes between a thread's words in the private runs (128 threads of a half)
 
 // How a launch uses the block: chosen on the host.
 struct Plan {
+    int groups;                // epilogue groups: two of eight warps, two threads a pixel, or four of four, a thread a pixel
     int stages;                // ring stages
     uint32_t staging_bytes;    // per epilogue group, a multiple of 16; 0: does not fit
     int run_words[2];          // words of a thread's private run, first and second half's threads; 0: two passes
@@ -66,12 +71,12 @@ __host__ __device__ inline SmemLayout smem_layout(int c, int k, const Plan &pl)
     l.ring = (uint32_t)(((size_t)k * c * 2 + 1023) & ~(size_t)1023);
     l.run_bytes = (uint32_t)(pl.run_words[0] + pl.run_words[1]) * kRunStep;      // per group
     l.staging = l.ring + (uint32_t)pl.stages * kStageBytes;                     // per group: the buffer, then the runs
-    l.enc = l.staging + 2u * (pl.staging_bytes + l.run_bytes);
+    l.enc = l.staging + (uint32_t)pl.groups * (pl.staging_bytes + l.run_bytes);
     l.len8 = l.enc + (uint32_t)pl.entries * 8;           // code lengths as bytes
     l.bias = (l.len8 + (uint32_t)pl.entries + 15u) & ~15u;
     l.bias_mid = l.bias + (uint32_t)k * 4;
     l.xch = l.bias_mid + (uint32_t)k * 4;               // per group: [2 halves][128] prefix and bits of every pixel, [3][128] chunk boundaries
-    l.total = l.xch + 2u * (2u * 128u * 4u + 3u * 128u * 2u);
+    l.total = l.xch + (uint32_t)pl.groups * (2u * 128u * 4u + 3u * 128u * 2u);
     return l;
 }
 
@@ -216,29 +221,32 @@ __device__ __noinline__ Sink code_again(Sink sink, uint32_t trow, int blk0, int 
 // but the modal symbol (the single bit 0): sixteen zero bits then.
 // kPair (per-layer tables, b <= 6): the code tables are indexed by two neighbouring symbols at once
 // (q0 | q1 << b), which halves the lookups.
+// kGroups: epilogue groups, two (a pixel's coefficients split between two threads) or four.
 // kHist (statistics, Section 3.1 "Variable length coding": the entropy needs the distribution of
 // the symbols): every symbol but the zero level is also counted, per coefficient channel, into one of the copies of a.hist, one
 // atomic each.
 // `block` of `blocks` that share the tensor's tiles.
-template <bool kPerChannel, bool kDebug, bool kPair, bool kHist, bool kRuns>
+template <bool kPerChannel, bool kDebug, bool kPair, bool kHist, bool kRuns, int kGroups>
 __device__ __forceinline__ void encode_tiles(const EncodeArgs &a, const Plan &pl, unsigned int block, unsigned int blocks)
 {
     extern __shared__ __align__(1024) unsigned char smem[];      // swizzled ring stages: aligned to their 1 KB atoms
-    __shared__ __align__(8) unsigned long long s_full[kMaxStages], s_empty[kMaxStages], s_tfull[2], s_tempty[2];
+    __shared__ __align__(8) unsigned long long s_full[kMaxStages], s_empty[kMaxStages], s_tfull[kGroups], s_tempty[kGroups];
     __shared__ __align__(8) unsigned long long s_basis_ready;
     __shared__ uint32_t s_tmem_base;
-    __shared__ unsigned int s_warp_sums[2][2][4], s_overflow[2];
-    __shared__ int s_go[2];                    // per group: its polling warp's waits for the tile have succeeded
-    __shared__ unsigned long long s_base[2];
-    __shared__ int s_write_ok[2];
+    __shared__ unsigned int s_warp_sums[kGroups][2][4], s_overflow[kGroups];
+    __shared__ int s_go[kGroups];                    // per group: its polling warp's waits for the tile have succeeded
+    __shared__ unsigned long long s_base[kGroups];
+    __shared__ int s_write_ok[kGroups];
     // staging hand-over to the store warp: slot n % kSlots for a group's n-th tile
-    __shared__ __align__(8) unsigned long long s_stg_full[2][kSlots], s_stg_free[2][kSlots];
-    __shared__ unsigned int s_padded[2][kSlots], s_stg_at[2][kSlots];   // bits of the tile, its place in the staging buffer
-    __shared__ int s_store_cmd[2][kSlots];     // 1: copy the staged tile out, 2: nothing to copy, 3: stop
+    __shared__ __align__(8) unsigned long long s_stg_full[kGroups][kSlots], s_stg_free[kGroups][kSlots];
+    __shared__ unsigned int s_padded[kGroups][kSlots], s_stg_at[kGroups][kSlots];   // bits of the tile, its place in the staging buffer
+    __shared__ int s_store_cmd[kGroups][kSlots];     // 1: copy the staged tile out, 2: nothing to copy, 3: stop
 
     // (taken from lane 0: the compiler knows that the branches between the roles are the same for a whole warp)
     const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
     const int nsym = 1 << a.bits;
+    constexpr int kGroupWarps = kEpiWarps / kGroups, kGroupThreads = 32 * kGroupWarps, kAccCols = kTmemCols / kGroups;
+    constexpr bool kHalves = kGroupWarps == 8;                   // two threads a pixel
     constexpr bool enc_in_smem = !kPerChannel;
     constexpr bool kCanSkip = !kPerChannel && !kDebug && !kHist;     // blocks of modal symbols are passed over
     const int enc_entries = pl.entries;
@@ -253,13 +261,13 @@ __device__ __forceinline__ void encode_tiles(const EncodeArgs &a, const Plan &pl
 
     // ---- set-up ---------------------------------------------------------------------
     chain_next();                                             // (a decoder that follows is set up meanwhile)
-    if (tid < 2) s_overflow[tid] = 0;
+    if (tid < kGroups) s_overflow[tid] = 0;
     if (tid == 0) {
         for (int s = 0; s < n_stages; ++s) { mbar_init(smem_u32(&s_full[s]), 128); mbar_init(smem_u32(&s_empty[s]), 1); }
-        for (int b = 0; b < 2; ++b) {
+        for (int b = 0; b < kGroups; ++b) {
             mbar_init(smem_u32(&s_tfull[b]), 1);
-            mbar_init(smem_u32(&s_tempty[b]), 8);                 // one arrival per warp of the group
-            for (int i = 0; i < kSlots; ++i) { mbar_init(smem_u32(&s_stg_full[b][i]), 8); mbar_init(smem_u32(&s_stg_free[b][i]), 1); }
+            mbar_init(smem_u32(&s_tempty[b]), kGroupWarps);                 // one arrival per warp of the group
+            for (int i = 0; i < kSlots; ++i) { mbar_init(smem_u32(&s_stg_full[b][i]), kGroupWarps); mbar_init(smem_u32(&s_stg_free[b][i]), 1); }
         }
         mbar_init(smem_u32(&s_basis_ready), 1);
         mbar_fence_init();
@@ -392,8 +400,8 @@ __device__ __forceinline__ void encode_tiles(const EncodeArgs &a, const Plan &pl
             uint32_t phase = 0;
             bool alive = mbar_wait(smem_u32(&s_basis_ready), 0u);
             for (long long tl = 0; tl < my_tiles && alive; ++tl) {
-                const int acc = (int)(tl & 1);
-                if (!mbar_wait(smem_u32(&s_tempty[acc]), (uint32_t)(((tl >> 1) & 1) ^ 1))) { alive = false; break; }
+                const int acc = (int)(tl % kGroups);
+                if (!mbar_wait(smem_u32(&s_tempty[acc]), (uint32_t)(((tl / kGroups) & 1) ^ 1))) { alive = false; break; }
                 tc_fence_after_sync();
                 const uint32_t d_tmem = tmem_base + acc * kAccCols;
                 uint32_t b_lo = (uint32_t)b_desc;
@@ -416,15 +424,17 @@ __device__ __forceinline__ void encode_tiles(const EncodeArgs &a, const Plan &pl
         }
     } else if (warp >= kStoreWarp0) {
         // ================= store warps =================
-        const int grp = warp - kStoreWarp0;
-        const uint32_t stg_addr = smem_u32(smem + L.staging + (uint32_t)grp * (pl.staging_bytes + L.run_bytes));
-        long long n = 0;
-        for (long long tl = grp; tl < my_tiles; tl += 2, ++n) {
+        unsigned int stopped = 0;                                // groups that hand over nothing more
+        for (long long tl = warp - kStoreWarp0; tl < my_tiles; tl += 2) {
+            const int grp = (int)(tl % kGroups);
+            const long long n = tl / kGroups;
+            const uint32_t stg_addr = smem_u32(smem + L.staging + (uint32_t)grp * (pl.staging_bytes + L.run_bytes));
             const long long tile = block + tl * blocks;
             const int slot = (int)(n % kSlots);
+            if (stopped >> grp & 1u) continue;
             if (!mbar_wait(smem_u32(&s_stg_full[grp][slot]), (uint32_t)((n / kSlots) & 1), 400u)) { if (lane == 0) tc_dev_set_status(a.status, TC_ERR_TIMEOUT); break; }
             const int cmd = s_store_cmd[grp][slot];
-            if (cmd == 3) break;
+            if (cmd == 3) { stopped |= 1u << grp; continue; }
             if (cmd == 1) {
                 const unsigned long long padded = s_padded[grp][slot];
                 const uint32_t src = stg_addr + s_stg_at[grp][slot];
@@ -451,12 +461,12 @@ __device__ __forceinline__ void encode_tiles(const EncodeArgs &a, const Plan &pl
         }
     } else {
         // ================= epilogue groups =================
-        const int grp = warp >> 3;                 // 0 or 1
-        const int wg = warp & 7;
-        const int half = wg >> 2;                  // which part of the coefficients
+        const int grp = warp / kGroupWarps;
+        const int wg = warp % kGroupWarps;
+        const int half = kHalves ? wg >> 2 : 0;    // which part of the coefficients
         const int wq = wg & 3;                     // TMEM lane quarter
         const int m = wq * 32 + lane;              // pixel within the tile = TMEM lane
-        const int tg = (tid & 255);                // thread within the group
+        const int tg = tid % kGroupThreads;        // thread within the group
         const int n_blk = a.k >> 4;                // blocks of 16 coefficients: the first split_blk belong to the first half's threads
         const int blk0 = half ? pl.split_blk : 0, blk1 = half ? n_blk : pl.split_blk;
         const int chunk_blks = a.splits > 1 ? n_blk / a.splits : n_blk;    // blocks per chunk of a pixel
@@ -493,7 +503,7 @@ __device__ __forceinline__ void encode_tiles(const EncodeArgs &a, const Plan &pl
             }
         };
 
-        for (long long tl = grp; tl < my_tiles && alive; tl += 2) {
+        for (long long tl = grp; tl < my_tiles && alive; tl += kGroups) {
             const long long tile = block + tl * blocks;
             const long long p = tile * TC_TILE_PIXELS + m;
             const bool valid = p < a.pixels;
@@ -501,13 +511,13 @@ __device__ __forceinline__ void encode_tiles(const EncodeArgs &a, const Plan &pl
             // tile before the last -- and lets the others in through a hardware barrier: a parked warp
             // issues nothing, whereas polling warps took two thirds of the SM's instructions.
             if (wg == 0) {
-                bool go = mbar_wait(smem_u32(&s_tfull[grp]), (uint32_t)((tl >> 1) & 1), 200u);
+                bool go = mbar_wait(smem_u32(&s_tfull[grp]), (uint32_t)((tl / kGroups) & 1), 200u);
                 const unsigned int back = prev_end > pl.staging_bytes ? 1u : 2u;      // (the tile before lies in the runs, too)
                 if (n_done >= back) go = go && mbar_wait(smem_u32(&s_stg_free[grp][(n_done - back) % kSlots]), ((n_done - back) / kSlots) & 1u);
                 if (lane == 0) s_go[grp] = go;
                 tc_fence_before_sync();
             }
-            named_bar_sync(bar_id, 256);
+            named_bar_sync(bar_id, kGroupThreads);
             tc_fence_after_sync();
             if (!s_go[grp]) { alive = false; break; }
             [[maybe_unused]] unsigned int n_clamped = 0;       // statistics mode: coefficients outside the quantiser's range
@@ -659,15 +669,15 @@ __device__ __forceinline__ void encode_tiles(const EncodeArgs &a, const Plan &pl
                 const unsigned int up = __shfl_up_sync(0xffffffffu, inc, d);
                 if (lane >= d) inc += up;
             }
-            xch[half * 128 + m] = ((inc - my_bits) << 12) | my_bits;       // at most 31 * 256 * 12 bits before, 256 * 12 own
+            if constexpr (kHalves) xch[half * 128 + m] = ((inc - my_bits) << 12) | my_bits;       // at most 31 * 256 * 12 bits before, 256 * 12 own
             if (lane == 31) s_warp_sums[grp][half][wq] = inc;
-            named_bar_sync(bar_id, 256);
-            const uint32_t theirs = xch[(half ^ 1) * 128 + m];
+            named_bar_sync(bar_id, kGroupThreads);
+            const uint32_t theirs = kHalves ? xch[(half ^ 1) * 128 + m] : 0u;
             const unsigned int other = theirs & 0xfffu, pixel_bits = my_bits + other;
             unsigned int before = 0, tile_bits = 0, warp_bits = 0;
 #pragma unroll
             for (int w = 0; w < 4; ++w) {
-                const unsigned int sw = s_warp_sums[grp][0][w] + s_warp_sums[grp][1][w];
+                const unsigned int sw = s_warp_sums[grp][0][w] + (kHalves ? s_warp_sums[grp][1][w] : 0u);
                 if (w < wq) before += sw;
                 if (w == wq) warp_bits = sw;
                 tile_bits += sw;
@@ -686,7 +696,7 @@ __device__ __forceinline__ void encode_tiles(const EncodeArgs &a, const Plan &pl
                 } else {
 #pragma unroll
                     for (int w = 0; w < 4; ++w)
-                        if (w < wq + (cpx >> 5)) chunk_end += s_warp_sums[grp][0][w] + s_warp_sums[grp][1][w];
+                        if (w < wq + (cpx >> 5)) chunk_end += s_warp_sums[grp][0][w] + (kHalves ? s_warp_sums[grp][1][w] : 0u);
                 }
                 if (valid && half == 0 && (m & (cpx - 1)) == 0) a.chunk_len[p >> (__ffs(cpx) - 1)] = (uint16_t)(chunk_end - pixel_off);
             } else if (valid && half == 0) {
@@ -724,7 +734,7 @@ __device__ __forceinline__ void encode_tiles(const EncodeArgs &a, const Plan &pl
                     const bool go = mbar_wait(smem_u32(&s_stg_free[grp][(n_done - 1) % kSlots]), ((n_done - 1) / kSlots) & 1u);
                     if (lane == 0) s_go[grp] = go;
                 }
-                named_bar_sync(bar_id, 256);
+                named_bar_sync(bar_id, kGroupThreads);
                 if (!s_go[grp]) { alive = false; break; }
             }
             prev_at = stg_at;
@@ -762,7 +772,7 @@ __device__ __forceinline__ void encode_tiles(const EncodeArgs &a, const Plan &pl
                         dst += 4;
                         tail = last << (32 - sh);
                     }
-                    named_bar_sync(bar_id, 256);      // all full words stored
+                    named_bar_sync(bar_id, kGroupThreads);      // all full words stored
                     if (tail && valid) asm volatile("red.shared.or.b32 [%0], %1;" ::"r"(dst), "r"(tail) : "memory");
                 } else {
                     SmemBitWriter<4> w;
@@ -771,7 +781,7 @@ __device__ __forceinline__ void encode_tiles(const EncodeArgs &a, const Plan &pl
                     tc_fence_before_sync();
                     __syncwarp();
                     if (lane == 0) mbar_arrive(smem_u32(&s_tempty[grp]));
-                    named_bar_sync(bar_id, 256);
+                    named_bar_sync(bar_id, kGroupThreads);
                     w.finish();
                 }
                 if (tg == 0) { s_padded[grp][n_done % kSlots] = (unsigned int)padded; s_stg_at[grp][n_done % kSlots] = stg_at; s_store_cmd[grp][n_done % kSlots] = 1; }
@@ -786,18 +796,18 @@ __device__ __forceinline__ void encode_tiles(const EncodeArgs &a, const Plan &pl
                 tc_fence_before_sync();
                 __syncwarp();
                 if (lane == 0) mbar_arrive(smem_u32(&s_tempty[grp]));
-                named_bar_sync(bar_id, 256);
+                named_bar_sync(bar_id, kGroupThreads);
                 w.finish();
                 if (tg == 0) { s_padded[grp][n_done % kSlots] = (unsigned int)padded; s_stg_at[grp][n_done % kSlots] = stg_at; s_store_cmd[grp][n_done % kSlots] = 1; }
             } else {
                 // rare: the tile does not fit -> resolve its position first and pack straight into (zeroed) global memory
                 resolve_base(tile, padded);
-                named_bar_sync(bar_id, 256);
+                named_bar_sync(bar_id, kGroupThreads);
                 if (s_write_ok[grp]) {
                     uint4 *z = reinterpret_cast<uint4 *>(a.stream + (s_base[grp] >> 5));
-                    for (unsigned int i = tg; i < (unsigned int)(padded >> 7); i += 256) z[i] = make_uint4(0u, 0u, 0u, 0u);
+                    for (unsigned int i = tg; i < (unsigned int)(padded >> 7); i += kGroupThreads) z[i] = make_uint4(0u, 0u, 0u, 0u);
                 }
-                named_bar_sync(bar_id, 256);
+                named_bar_sync(bar_id, kGroupThreads);
                 GlobalSink g;
                 g.on = valid && s_write_ok[grp];
                 g.w.init(a.stream, s_base[grp] + my_off);
@@ -834,10 +844,10 @@ __device__ __forceinline__ void encode_tiles(const EncodeArgs &a, const Plan &pl
     }
 }
 
-template <bool kPerChannel, bool kDebug, bool kPair, bool kHist, bool kRuns>
+template <bool kPerChannel, bool kDebug, bool kPair, bool kHist, bool kRuns, int kGroups>
 __global__ void __launch_bounds__(kThreads, 1) encode_tc_kernel(EncodeArgs a, Plan pl)
 {
-    encode_tiles<kPerChannel, kDebug, kPair, kHist, kRuns>(a, pl, blockIdx.x, gridDim.x);
+    encode_tiles<kPerChannel, kDebug, kPair, kHist, kRuns, kGroups>(a, pl, blockIdx.x, gridDim.x);
 }
 
 // Several tensors in one launch, each with blocks of its own.  A block's set-up and first tile take 13 us and a launch on a stream
@@ -848,16 +858,19 @@ struct EncodeList {
     unsigned int first[kListItems + 1];        // block that each item starts at; past the last item 2^32 - 1
     struct { EncodeArgs a; Plan pl; } item[kListItems];
 };
-template <bool kPerChannel, bool kPair, bool kRuns>
+template <bool kPerChannel, bool kPair, bool kRuns, int kGroups>
 __global__ void __launch_bounds__(kThreads, 1) encode_tc_list_kernel(const __grid_constant__ EncodeList list)
 {
     int i = 0;
     while (blockIdx.x >= list.first[i + 1]) ++i;
-    encode_tiles<kPerChannel, false, kPair, false, kRuns>(list.item[i].a, list.item[i].pl, blockIdx.x - list.first[i],
+    encode_tiles<kPerChannel, false, kPair, false, kRuns, kGroups>(list.item[i].a, list.item[i].pl, blockIdx.x - list.first[i],
                                                           min(list.first[i + 1], gridDim.x) - list.first[i]);
 }
 
 }  // namespace
+
+// Coefficients up to which four accumulators fit tensor memory and a thread codes a pixel.
+constexpr int kFourGroupsCoefs = 128;
 
 // What a launch does with the shared memory that the basis leaves, from the code lengths to expect of
 // the model's coefficients (a code without a one-bit symbol: b bits for each).  A tile's size varies
@@ -870,6 +883,7 @@ __global__ void __launch_bounds__(kThreads, 1) encode_tc_list_kernel(const __gri
 static Plan make_plan(const tc_ctx *ctx, const EncodeArgs &a)
 {
     const int n_blk = a.k / 16;
+    const bool plain = !a.hist && !a.dbg_coef && !a.dbg_sym;
     const bool modal = a.groups == 1 && a.modal >= 0;
     auto blk_bits = [&](int b) { return modal || a.groups != 1 ? a.blk_bits[b] : std::max(a.blk_bits[b], 16.f * a.bits); };
     Plan best{};
@@ -885,8 +899,9 @@ static Plan make_plan(const tc_ctx *ctx, const EncodeArgs &a)
     while (modal && best.skip_blk > 0 && 64.f * a.blk_odd[best.skip_blk - 1] < 1.2f) --best.skip_blk;
     // blocks of the two threads of a pixel: equal work, a coded block counted as three passed over
     auto cost = [&](int b0, int b1) { return 3 * std::max(0, std::min(b1, best.skip_blk) - b0) + (b1 - std::max(b0, std::min(b1, best.skip_blk))); };
-    best.split_blk = 1;
-    for (int x = 2; x <= n_blk; ++x)
+    best.groups = plain && a.k <= kFourGroupsCoefs && !a.two_groups ? 4 : 2;
+    best.split_blk = best.groups == 4 ? n_blk : 1;
+    for (int x = 2; x <= n_blk && best.groups == 2; ++x)
         if (std::max(cost(0, x), cost(x, n_blk)) < std::max(cost(0, best.split_blk), cost(best.split_blk, n_blk))) best.split_blk = x;
     double tile_bits = 0.0;
     int want_words[2];
@@ -909,7 +924,7 @@ static Plan make_plan(const tc_ctx *ctx, const EncodeArgs &a)
         for (int h = 0; h < 2; ++h) pl.run_words[h] = runs ? want_words[h] : 0;
         pl.staging_bytes = 0;
         const long long left = (long long)budget - smem_layout(a.c, a.k, pl).total;
-        const long long per_group = (left / 2) & ~15ll;
+        const long long per_group = (left / pl.groups) & ~15ll;
         if (per_group < 4096 || (per_group < (long long)want_staging && t != 7)) continue;
         pl.staging_bytes = (uint32_t)std::min<long long>(per_group, kMaxStagingBytes);
         return pl;
@@ -932,30 +947,43 @@ bool tc_encode_tc_supported(const tc_ctx *ctx, const EncodeArgs &a)
 }
 
 template <bool kPerChannel, bool kPair, bool kRuns>
-static void (*pick_kernel(bool debug, bool hist))(EncodeArgs, Plan)
+static void (*pick_kernel(bool debug, bool hist, int groups))(EncodeArgs, Plan)
 {
     if constexpr (!kPerChannel)
-        if (hist) return encode_tc_kernel<false, false, kPair, true, kRuns>;
-    return debug ? encode_tc_kernel<kPerChannel, true, kPair, false, kRuns> : encode_tc_kernel<kPerChannel, false, kPair, false, kRuns>;
+        if (hist) return encode_tc_kernel<false, false, kPair, true, kRuns, 2>;
+    if (debug) return encode_tc_kernel<kPerChannel, true, kPair, false, kRuns, 2>;
+    return groups == 4 ? encode_tc_kernel<kPerChannel, false, kPair, false, kRuns, 4> : encode_tc_kernel<kPerChannel, false, kPair, false, kRuns, 2>;
 }
 
-// Which kernel codes the tensor: bit 0 a table per channel, bit 1 symbol pairs, bit 2 private runs.
+// Which kernel codes the tensor: bit 0 a table per channel, bit 1 symbol pairs, bit 2 private runs, bit 3 four groups.
 static int kernel_class(const EncodeArgs &a, const Plan &pl)
 {
     const bool per_channel = a.groups != 1;
-    return (per_channel ? 1 : 0) | (!per_channel && pl.entries > (1 << a.bits) ? 2 : 0) | (pl.run_words[0] > 0 ? 4 : 0);
+    return (per_channel ? 1 : 0) | (!per_channel && pl.entries > (1 << a.bits) ? 2 : 0) | (pl.run_words[0] > 0 ? 4 : 0) | (pl.groups == 4 ? kEncodeFourGroups : 0);
+}
+template <int kGroups>
+static const void *list_kernel(int which)
+{
+    switch (which & 7) {
+    case 1: return (const void *)encode_tc_list_kernel<true, false, false, kGroups>;
+    case 5: return (const void *)encode_tc_list_kernel<true, false, true, kGroups>;
+    case 2: return (const void *)encode_tc_list_kernel<false, true, false, kGroups>;
+    case 6: return (const void *)encode_tc_list_kernel<false, true, true, kGroups>;
+    case 4: return (const void *)encode_tc_list_kernel<false, false, true, kGroups>;
+    default: return (const void *)encode_tc_list_kernel<false, false, false, kGroups>;
+    }
 }
 
 // of a tensor that tc_encode_tc_supported takes
 int tc_encode_tc_class(const tc_ctx *ctx, const EncodeArgs &a) { return kernel_class(a, make_plan(ctx, a)); }
 
-// us that a tile takes a block: 1.5 with 64 coefficients at 1.1 bits each, 2.1 with 128, 4.25 with 256, 2.3 with 96 at 2.8 bits, 7.5
-// with 256 at 4.1 (8 to 85 tiles a block, after the first)
+// us that a tile takes a block: 1.35 with 64 coefficients at 1.1 bits each, 2.0 with 128 at 1.9, 1.75 with 96 at 2.8 (four groups), 3.95
+// with 256 at 1.1, 6.9 at 4.1 (8 to 130 tiles a block, after the first)
 double tc_encode_tc_tile_us(const EncodeArgs &a)
 {
     double bits = 0.0;
     for (int b = 0; b < a.k / 16; ++b) bits += a.blk_bits[b];
-    return std::max(1.2, 0.0118 * a.k) + 0.0043 * bits;
+    return a.k <= kFourGroupsCoefs ? 0.8 + 0.0075 * a.k + 0.0022 * bits : 0.011 * a.k + 0.004 * bits;
 }
 
 // Encodes tensors of one class (tc_encode_tc_class) on `sms` SMs, in list_launches launches (40 of 128x14x14 x 32 in
@@ -984,9 +1012,7 @@ tc_status tc_launch_encode_tc_list(const tc_ctx *ctx, const std::vector<EncodeAr
             if (i < n) blocks += (unsigned int)work[i].blocks;
         }
         list.first[n] = ~0u;
-        const void *kernel = which == 1 ? (const void *)encode_tc_list_kernel<true, false, false> : which == 5 ? (const void *)encode_tc_list_kernel<true, false, true>
-                           : which == 2 ? (const void *)encode_tc_list_kernel<false, true, false> : which == 6 ? (const void *)encode_tc_list_kernel<false, true, true>
-                           : which == 4 ? (const void *)encode_tc_list_kernel<false, false, true> : (const void *)encode_tc_list_kernel<false, false, false>;
+        const void *kernel = which & kEncodeFourGroups ? list_kernel<4>(which) : list_kernel<2>(which);
         if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) { cudaGetLastError(); return TC_ERR_CUDA; }
         void *params[] = {&list};
         // cooperative, as for one tensor: the blocks of a tensor look back at one another
@@ -1004,9 +1030,9 @@ tc_status tc_launch_encode_tc(const tc_ctx *ctx, const EncodeArgs &a, cudaStream
     if (pl.staging_bytes == 0) return TC_ERR_UNSUPPORTED;
     const bool pair = !per_channel && pl.entries > (1 << a.bits), runs = pl.run_words[0] > 0;
     const SmemLayout l = smem_layout(a.c, a.k, pl);
-    void (*kernel)(EncodeArgs, Plan) = per_channel ? (runs ? pick_kernel<true, false, true>(debug, false) : pick_kernel<true, false, false>(debug, false))
-                                     : pair        ? (runs ? pick_kernel<false, true, true>(debug, a.hist) : pick_kernel<false, true, false>(debug, a.hist))
-                                                   : (runs ? pick_kernel<false, false, true>(debug, a.hist) : pick_kernel<false, false, false>(debug, a.hist));
+    void (*kernel)(EncodeArgs, Plan) = per_channel ? (runs ? pick_kernel<true, false, true>(debug, false, pl.groups) : pick_kernel<true, false, false>(debug, false, pl.groups))
+                                     : pair        ? (runs ? pick_kernel<false, true, true>(debug, a.hist, pl.groups) : pick_kernel<false, true, false>(debug, a.hist, pl.groups))
+                                                   : (runs ? pick_kernel<false, false, true>(debug, a.hist, pl.groups) : pick_kernel<false, false, false>(debug, a.hist, pl.groups));
     if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)l.total) != cudaSuccess)
         return TC_ERR_CUDA;
     const unsigned int grid = (unsigned int)((a.n_tiles < ctx->sm_count) ? a.n_tiles : ctx->sm_count);

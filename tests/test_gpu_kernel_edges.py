@@ -48,6 +48,28 @@ def test_resident_encoder_copies(ctx, c, h, w, n, bits, offset):
     m.close(); cb.close()
 
 
+# Resident-basis encoder with four groups a block (up to 128 coefficients): fewer tiles a block than groups and more than all groups'
+# slots hold, one chunk a pixel, parts of one and several pixels a chunk, every code table, private runs and two passes, maps of
+# more spread than the calibration's (tiles coded again, and straight into global memory).  The debug outputs take the kernel with two groups,
+# whose streams the parity cases check: the same bytes.
+@pytest.mark.parametrize("c,k,hw,n,bits,tables,cp,splits,spread", [
+    (16, 16, 12, 1, 4, 1, 0, 0, 1.0), (128, 128, 64, 1500, 4, 1, 0, 0, 1.0), (128, 128, 16, 1184, 8, 1, 0, 0, 1.0), (64, 64, 196, 2300, 4, 1, 0, 0, 2.5),
+    (96, 96, 196, 1300, 5, 1, 1, 2, 1.0), (128, 64, 100, 1600, 6, 1, 1, 4, 1.0), (80, 48, 64, 700, 3, 48, 0, 0, 1.0), (32, 32, 3136, 90, 7, 1, 16, 1, 3.0),
+    (112, 112, 4, 20000, 2, 1, 0, 0, 1.0), (128, 128, 196, 600, 8, 128, 0, 0, 2.0), (144, 128, 36, 900, 4, 1, 0, 0, 1.0)])
+def test_four_groups_a_block(ctx, c, k, hw, n, bits, tables, cp, splits, spread):
+    params = fm.layer_params(fm.LayerSpec(c, hw // 4, 4, 0.9, None, 22000 + c + k + bits))
+    cal = fm.make_maps(params, max(4, 30000 // hw), calib=True, dtype=torch.bfloat16, device="cuda")
+    x = fm.make_maps(params, n, dtype=torch.bfloat16, device="cuda") * spread
+    m = tc.tc_fit_pca(ctx, cal, bits, k=k)
+    cb = tc.tc_build_codebook(ctx, m, tc.tc_stats(ctx, m, None, cal, groups=tables).hist, groups=tables)
+    want = tc.tc_encode(ctx, m, cb, x, chunk_pixels=cp, pixel_splits=splits, debug=True)
+    assert tc.tc_get_status(ctx) == 0 and tc.tc_last_path(ctx) == 1
+    for _ in range(3):
+        assert _same_stream(tc.tc_encode(ctx, m, cb, x, chunk_pixels=cp, pixel_splits=splits), want)
+    assert tc.tc_get_status(ctx) == 0 and tc.tc_last_path(ctx) == 1
+    m.close(); cb.close()
+
+
 # Device eigensolver: every row / block shape of its kernel (blocks of 16 columns up to 512 rows, of 8
 # beyond; 33 and 65 columns leave column blocks that are empty), and spectra that reach below zero.
 @pytest.mark.parametrize("n,shift", [(16, 0.0), (31, 0.5), (33, 0.0), (65, 0.3), (130, 0.0), (300, 0.5), (384, 0.0), (513, 0.4), (640, 0.0)])
