@@ -826,14 +826,17 @@ tc_status tc_launch_pack_symbols(const tc_ctx *ctx, const EncodeArgs &a, const u
                         : (a.groups == 1 ? pack_symbols_kernel<true, false> : pack_symbols_kernel<false, false>);
     if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSpreadBytes) != cudaSuccess) return TC_ERR_CUDA;
     const dim3 grid((unsigned int)tiles, (unsigned int)tile_blocks), block(TC_TILE_PIXELS / tile_blocks * parts);
-    // Up to a block per SM: set up while the kernel before is still at work, with more than half of an SM's shared
-    // memory each -- small blocks that arrive early all pile onto the first SMs that have room (960x7x7 x 128, 49
-    // blocks: 49 us unchained, 65 chained, 48 chained and spread; 64x56x56 f32 17.2 unchained, 14.9 chained and spread).
-    // More blocks than that start when the SMs are free (80x27x19 x 37: 20 us, chained 26).
+    // Set up while the kernel before is still at work, kept apart by shared memory: small blocks that arrive early all pile onto the
+    // first SMs that have room (960x7x7 x 128, 49 blocks: 49 us unchained, 65 chained, 48 chained and spread; 64x56x56 f32 17.2
+    // unchained, 14.9 chained and spread; 400x7x7 x 800, 307 blocks, 87.8 -> 66.9; 80x27x27 x 64, 365 blocks of 256 threads, 25.2 ->
+    // 22.7).  Not large blocks of which some SMs get two: the first SMs that are free take two each (576x14x14 x 128, 196 blocks of 1 024
+    // threads: 55.4 -> 57.4).
     if (tile_blocks > 1)
         return launch_chained_cluster(tile_blocks, kernel, grid, block, std::max(staging, kSpreadBytes), s, a, sym, parts, first_tile, staging) == cudaSuccess ? TC_OK : TC_ERR_CUDA;
-    if (a.alone && tiles <= ctx->sm_count)
-        return launch_chained(true, kernel, grid, block, std::max(staging, kSpreadBytes), s, a, sym, parts, first_tile, staging) == cudaSuccess ? TC_OK : TC_ERR_CUDA;
+    const bool apart = tiles <= ctx->sm_count || tiles > 2ll * ctx->sm_count || block.x <= 512;
+    const size_t spread = a.alone && apart ? spread_bytes(tiles, ctx->sm_count) : 0;
+    if (spread > 0)
+        return launch_chained(true, kernel, grid, block, std::max<size_t>(staging, spread), s, a, sym, parts, first_tile, staging) == cudaSuccess ? TC_OK : TC_ERR_CUDA;
     kernel<<<grid, block, staging, s>>>(a, sym, parts, first_tile, staging);
     return cudaGetLastError() == cudaSuccess ? TC_OK : TC_ERR_CUDA;
 }
