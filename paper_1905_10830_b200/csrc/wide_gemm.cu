@@ -64,7 +64,8 @@ __global__ void __launch_bounds__(kThreads, 1) wide_gemm_kernel(GemmArgs a, cons
     extern __shared__ __align__(1024) unsigned char smem[];
     __shared__ __align__(8) unsigned long long s_full[kStages], s_empty[kStages], s_tfull[2], s_tempty[2];
     __shared__ uint32_t s_tmem_base;
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    // (taken from lane 0: the compiler knows that the branches between the roles are the same for a whole warp)
+    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
     const uint32_t ring = smem_u32(smem);
     chain_next();
     if (tid == 0) {
@@ -76,7 +77,7 @@ __global__ void __launch_bounds__(kThreads, 1) wide_gemm_kernel(GemmArgs a, cons
     tc_fence_before_sync();
     __syncthreads();
     tc_fence_after_sync();
-    const uint32_t tmem_base = s_tmem_base;
+    const uint32_t tmem_base = __shfl_sync(0xffffffffu, s_tmem_base, 0);
     chain_wait();                                             // the workspace operand; earlier readers of what this kernel writes
     // rows of both operands of unit u: (tile of pixels, block)
     auto tile_of = [&](long long u) { return (int)(u / a.blocks); };
@@ -118,8 +119,14 @@ __global__ void __launch_bounds__(kThreads, 1) wide_gemm_kernel(GemmArgs a, cons
                 tc_fence_after_sync();
                 const uint32_t a_lo = desc_lo + (uint32_t)s * (kStageBytes >> 4), b_lo = a_lo + (kStageA >> 4);
                 const int steps = min(kPanelK, a.k_depth - kp * kPanelK) >> 4;
-                for (int q = 0; q < steps; ++q)
+                auto step = [&](int q) {
                     mma_bf16_ss_guarded(tmem_base + acc * kMaxN, a_lo + 2 * q, desc_hi, b_lo + 2 * q, desc_hi, idesc, (kp | q) ? 1u : 0u, issuer);
+                };
+                if (steps == kPanelK / 16) {
+#pragma unroll
+                    for (int q = 0; q < kPanelK / 16; ++q) step(q);
+                } else
+                    for (int q = 0; q < steps; ++q) step(q);
                 mma_commit_guarded(smem_u32(&s_empty[s]), issuer);
                 if (++s == kStages) { s = 0; phase ^= 1u; }
             }
