@@ -148,7 +148,7 @@ struct BitReader {
     {
         uint32_t w;
         if constexpr (kShared) { w = lds_u32(next_addr); next_addr += 4; }
-        else { w = next < end ? __ldg(next) : 0u; ++next; }
+        else { w = stream_word(next, end); ++next; }
         return w;
     }
     // kShared: `base_addr` is the shared address of the segment; else `base` / `end_word` delimit it
@@ -371,7 +371,7 @@ __device__ __forceinline__ void decode_tiles(const DecodeArgs &a, const SmemLayo
                 RawTile rt{1, 0, 0};                             // (no tile: not valid)
                 if (tl >= my_tiles) return rt;
                 const long long tile = block + (long long)tl * blocks;
-                rt.at = __ldg(a.tile_off + tile + (lane & 1));
+                rt.at = a.tile_off[tile + (lane & 1)];
                 if (owner) {
                     const long long ch = tile * chunks_per_tile + (long long)t * (cp > 1 ? 1 : S);
                     if (cp > 1 || S == 1) { if (ch < a.n_chunks) rt.l01 = a.chunk_len[ch]; }
@@ -438,7 +438,7 @@ __device__ __forceinline__ void decode_tiles(const DecodeArgs &a, const SmemLayo
                 // with the tile before: its stream buffer may take the next tile's segment
                 named_bar_sync(bar_id, n_thr);
                 if (!cur.landed) {
-                    if (cur.ok) stage_tile(cur, __ldg(a.tile_off + tile), cur.room == 2 ? 0 : li & 1);
+                    if (cur.ok) stage_tile(cur, a.tile_off[tile], cur.room == 2 ? 0 : li & 1);
                     cp_async_wait<0>();
                     named_bar_sync(bar_id, n_thr);
                 }
@@ -552,7 +552,7 @@ __device__ __forceinline__ void decode_tiles(const DecodeArgs &a, const SmemLayo
                 } else {
                     BitReader<false> r;
                     if (active) {
-                        const uint32_t *seg = a.stream + (__ldg(a.tile_off + tile) >> 5);
+                        const uint32_t *seg = a.stream + (a.tile_off[tile] >> 5);
                         r.init(0u, seg, seg + (cur.bits >> 5), chunk_start);
                     } else r.idle();
                     decode_tile(r);

@@ -38,6 +38,15 @@ __device__ __forceinline__ unsigned long long global_timer_ns()
 __device__ __forceinline__ void chain_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
+// A word of a stream, 0 at or past `end`.  Not through the read-only path (see launch_first), and free to be scheduled among
+// stores as such a load is: its address comes from offsets that were read after the wait.
+__device__ __forceinline__ uint32_t stream_word(const uint32_t *next, const uint32_t *end)
+{
+    uint32_t w;
+    asm("{\n\t.reg .pred p;\n\tsetp.lt.u64 p, %1, %2;\n\tmov.u32 %0, 0;\n\t@p ld.global.u32 %0, [%1];\n\t}" : "=&r"(w) : "l"(next), "l"(end));
+    return w;
+}
+
 __device__ __forceinline__ double load_as_double(const float *p) { return (double)__ldg(p); }
 __device__ __forceinline__ double load_as_double(const __nv_bfloat16 *p)
 {

@@ -56,7 +56,7 @@ __global__ void __launch_bounds__(kPx * kRows) project_quantise_kernel(EncodeArg
         for (int i = 0; i < kRed / kRows; ++i) {
             const int ch = c0 + ty + kRows * i;
             const bool ok = p_ok && ch < a.c;
-            d[i] = ok ? load_as_double(xp + (long long)ch * a.hw) : 0.0;
+            d[i] = ok ? (double)(float)xp[(long long)ch * a.hw] : 0.0;
             mu[i] = ok ? __ldg(a.mean64 + ch) : 0.0;
         }
 #pragma unroll
@@ -439,7 +439,9 @@ constexpr uint32_t kRowBytes = 80;                            // 32 symbols of a
 constexpr uint32_t kRowsWarpBytes = 32 * kRowBytes;
 
 // MSB-first reader with a 64-bit window hi:lo (left-aligned) and the word behind it already loaded: a
-// refill never waits for memory.  Words at or past `end` read as zero.
+// refill never waits for memory.  Words at or past `end` read as zero.  kEarly: of a kernel that was launched early, for which the stream is
+// no read-only memory (64x56x56 x 64 with a table per channel 45.6 us through the read-only path, 46.8 past it).
+template <bool kEarly>
 struct AheadReader {
     const uint32_t *next, *end;
     uint32_t hi, lo, ahead;
@@ -447,7 +449,7 @@ struct AheadReader {
 
     __device__ __forceinline__ uint32_t fetch()
     {
-        const uint32_t v = next < end ? __ldg(next) : 0u;
+        const uint32_t v = kEarly ? stream_word(next, end) : next < end ? __ldg(next) : 0u;
         ++next;
         return v;
     }
@@ -559,7 +561,7 @@ __device__ __noinline__ void clear_rows(void *out, long long row0, int px0, int 
 // second lookup in the chain, 512x7x7 x 64 (25 tiles) 23.3 -> 27.3.
 // Two or four blocks a tile where that leaves no SM with two: the eight or sixteen warps of a tile share an SM's issue slots while others
 // idle (256x14x14 f32, per-channel codes, with the inverse 23.8 -> 21.5 us, 512x14x14 f32 45 -> 37, 768x7x7 x 16 26.7 -> 22.6).
-template <bool kOperand, bool kPerLayer, bool kFull>
+template <bool kOperand, bool kPerLayer, bool kFull, bool kEarly>
 __global__ void __launch_bounds__(kUnpackThreads) unpack_symbols_kernel(DecodeArgs a, void *out, long long first_tile, unsigned int table_bytes,
                                                                          unsigned int segment_bytes)
 {
@@ -761,7 +763,7 @@ __global__ void __launch_bounds__(kUnpackThreads) unpack_symbols_kernel(DecodeAr
         r.init(seg, walks ? off : 0u, walks ? seg + (uint32_t)((end - base) >> 3) : seg);
         walk(r);
     } else {
-        AheadReader r;
+        AheadReader<kEarly> r;
         r.init(a.stream, base + (walks ? off : 0u), walks ? end : base);
         walk(r);
     }
@@ -845,6 +847,12 @@ tc_status tc_launch_pack_symbols(const tc_ctx *ctx, const EncodeArgs &a, const u
 // the lookups in L2 that they save.
 constexpr unsigned int kSortedStaged = 16 * 1024;
 
+template <bool kOperand, bool kEarly>
+static void (*pick_unpack(bool per_channel, bool full))(DecodeArgs, void *, long long, unsigned int, unsigned int)
+{
+    return per_channel ? unpack_symbols_kernel<kOperand, false, false, kEarly> : full ? unpack_symbols_kernel<kOperand, true, kOperand, kEarly> : unpack_symbols_kernel<kOperand, true, false, kEarly>;
+}
+
 template <bool kOperand>
 static tc_status launch_unpack(const DecodeArgs &a, void *out, long long first_tile, long long end_tile, int sm_count, cudaStream_t s)
 {
@@ -867,12 +875,11 @@ static tc_status launch_unpack(const DecodeArgs &a, void *out, long long first_t
     const int threads = (chunks / parts + 31) / 32 * 32, least = tiles * parts < 4 * sm_count ? 256 : 32;
     // from 16 warps an SM on the shared-memory pipe is what bounds a per-layer decoder (see the kernel)
     const bool full = kOperand && a.groups == 1 && tiles * ((chunks + 31) / 32) >= 16 * (long long)sm_count;
-    void (*kernel)(DecodeArgs, void *, long long, unsigned int, unsigned int) =
-        a.groups != 1 ? unpack_symbols_kernel<kOperand, false, false>
-        : full ? unpack_symbols_kernel<kOperand, true, kOperand> : unpack_symbols_kernel<kOperand, true, false>;
+    const size_t spread = a.alone ? spread_bytes(tiles * parts, sm_count) : 0;
+    void (*kernel)(DecodeArgs, void *, long long, unsigned int, unsigned int) = spread > 0 ? pick_unpack<kOperand, true>(a.groups != 1, full) : pick_unpack<kOperand, false>(a.groups != 1, full);
     if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024) != cudaSuccess) return TC_ERR_CUDA;
     const size_t rows = full ? (size_t)(threads / 32) * kRowsWarpBytes : 0;
-    const size_t spread = a.alone ? spread_bytes(tiles * parts, sm_count) : 0, smem = std::max<size_t>(tables + segment + rows, spread);
+    const size_t smem = std::max<size_t>(tables + segment + rows, spread);
     return launch_first(spread > 0, kernel, dim3((unsigned int)tiles, (unsigned int)parts), std::max(threads, least), smem, s, a, out, first_tile, tables,
                         segment) == cudaSuccess ? TC_OK : TC_ERR_CUDA;
 }

@@ -204,7 +204,8 @@ inline cudaError_t launch_chained(bool early, void (*kernel)(P...), dim3 grid, d
 // The first kernel of a call, early as well: launches that wait for one another's end start at multiples of 2.05 us here, and 4.1 apart at
 // least (a kernel that spins for 1 to 10 us, queued 300 times), which is a quarter of a small call's time.  The kernels ahead of it
 // in the stream may be anyone's: until it has called chain_wait such a kernel reads nothing but models and codebooks, which are
-// complete when the functions that make them return, and writes nothing.  Captured calls start after all that the graph
+// complete when the functions that make them return, and writes nothing; afterwards it reads what
+// others wrote (maps, streams) not through the read-only path, whose lines may be older than the wait.  Captured calls start after all that the graph
 // holds before them.  Small blocks that arrive early all pile onto the first SMs that have room (decode of 384x8x8 x 241, 121 blocks:
 // 25 -> 56 us), so they ask for as much shared memory as keeps them apart (spread_bytes; more than eight an SM start in their
 // turn: 64x56x56 x 64 with a table per channel, 1 568 blocks, 45 -> 56 us).

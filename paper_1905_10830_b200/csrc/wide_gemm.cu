@@ -267,7 +267,7 @@ __global__ void __launch_bounds__(256) pixel_rows_kernel(const __nv_bfloat16 *x,
             uint2 v[kTurn / 16];
 #pragma unroll
             for (int i = 0; i < kTurn / 16; ++i)
-                if (c0 + cr + 16 * i < c) v[i] = __ldg(reinterpret_cast<const uint2 *>(src + (long long)(c0 + cr + 16 * i) * hw));
+                if (c0 + cr + 16 * i < c) v[i] = *reinterpret_cast<const uint2 *>(src + (long long)(c0 + cr + 16 * i) * hw);
 #pragma unroll
             for (int i = 0; i < kTurn / 16; ++i) {
                 uint32_t *d = reinterpret_cast<uint32_t *>(&s[cr + 16 * i][px]);
@@ -284,7 +284,7 @@ __global__ void __launch_bounds__(256) pixel_rows_kernel(const __nv_bfloat16 *x,
             __nv_bfloat16 v[kTurn / 4];
 #pragma unroll
             for (int i = 0; i < kTurn / 4; ++i)
-                if (c0 + cr + 4 * i < c) v[i] = __ldg(src + (long long)(c0 + cr + 4 * i) * hw);
+                if (c0 + cr + 4 * i < c) v[i] = src[(long long)(c0 + cr + 4 * i) * hw];
 #pragma unroll
             for (int i = 0; i < kTurn / 4; ++i) s[cr + 4 * i][px] = v[i];
         }
