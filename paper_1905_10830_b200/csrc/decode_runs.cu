@@ -812,6 +812,24 @@ static SmemLayout runs_layout(const tc_ctx *ctx, const DecodeArgs &a)
     return smem_layout(a.k, 1 << a.lut_bits, (group_work(a.splits, a.chunk_pixels) + 31) / 32, want, store_mode(a) != kRows16, ctx->max_smem_optin - kStaticSmem);
 }
 
+// The roles' registers are dealt from what a block is launched with: with fewer a thread than this the VLD warps would wait for theirs
+// for good, so a build whose kernels came out smaller does not run them.
+constexpr int kLaunchRegisters = 72;
+static_assert(16 * 80 + 8 * 72 + 4 * 40 <= 28 * kLaunchRegisters && kThreads == 28 * 32, "VLD, epilogue and MMA warpgroups");
+static bool registers_suffice()
+{
+    static const bool ok = [] {
+        for (const void *kernel : {(const void *)decode_runs_kernel<false>, (const void *)decode_runs_kernel<true>, (const void *)decode_runs_list_kernel<false>,
+                                   (const void *)decode_runs_list_kernel<true>}) {
+            cudaFuncAttributes at;
+            if (cudaFuncGetAttributes(&at, kernel) != cudaSuccess) { cudaGetLastError(); return false; }
+            if (at.numRegs < kLaunchRegisters) return false;
+        }
+        return true;
+    }();
+    return ok;
+}
+
 bool tc_decode_runs_supported(const tc_ctx *ctx, const DecodeArgs &a)
 {
     // K <= C leading components (PCA truncation): K is the reduction dimension of the MMA
@@ -820,7 +838,7 @@ bool tc_decode_runs_supported(const tc_ctx *ctx, const DecodeArgs &a)
     if (a.lut_bits > TC_MAX_CODE_LEN) return false;
     if (a.chunk_pixels > 1 ? a.splits != 1 : (a.splits != 1 && a.splits != 2 && a.splits != 4)) return false;
     if (a.splits > 1 && (a.k % a.splits != 0 || (a.k / a.splits) % 8 != 0)) return false;
-    return runs_layout(ctx, a).stream_buf > 0;
+    return runs_layout(ctx, a).stream_buf > 0 && registers_suffice();
 }
 
 tc_status tc_launch_decode_runs(const tc_ctx *ctx, const DecodeArgs &a, cudaStream_t s)
