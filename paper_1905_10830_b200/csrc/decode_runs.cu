@@ -714,6 +714,7 @@ __device__ __forceinline__ void decode_tiles(const DecodeArgs &a, const SmemLayo
             // symbols of the tile (the group's operand buffer).
             named_bar_sync(kBarBasis, 256 + 32);
             tc_fence_after_sync();
+            chain_wait();                                            // its waits run out two seconds from here, not from the launch
             const uint32_t issuer = (own_tid() & 31) == 0 ? 1u : 0u;
             const uint32_t idesc = make_idesc_bf16(128, TC_TILE_PIXELS, /*A K-major*/ false, /*B K-major*/ false);
             const int n_k16 = a.k >> 4;
