@@ -333,6 +333,9 @@ tc_status finish_codebook(tc_codebook *cb)
     TC_CUDA(cudaMalloc(&cb->d_block, lay.bytes));
     char *mem = (char *)cb->d_block;
     TC_CUDA(cudaMemcpy(mem, host.data(), lay.bytes, cudaMemcpyHostToDevice));
+    // (a copy from pageable memory may return while its last piece is on the way, and streams that do not wait for the legacy one may
+    // be next to read the tables: kernels that start early do so ahead of everything that their stream holds)
+    TC_CUDA(cudaStreamSynchronize(nullptr));
     cb->d_enc = (uint32_t *)(mem + enc_at);
     cb->d_lut32 = (uint32_t *)(mem + lut32_at);
     cb->d_canon = (uint32_t *)(mem + canon_at);

@@ -174,3 +174,28 @@ def test_a_long_kernel_ahead_is_no_timeout(ctx, late_copy):
     got = tc.tc_decode(ctx, m, cb, live, maps.shape[1:], BF16)
     assert tc.tc_get_status(ctx) == 0 and torch.equal(got, want)
     m.close(); cb.close()
+
+
+# Tables are read ahead of the wait: a codebook is complete when the call that makes it returns, also for streams that do not wait for the
+# legacy one.
+@pytest.mark.parametrize("c,tables,dtype,path", [(64, 1, BF16, 1), (256, 256, BF16, 1), (256, 256, F32, 0), (576, 1, BF16, 3)])
+def test_a_new_codebook_on_a_stream_of_its_own(ctx, c, tables, dtype, path):
+    m, cb, maps = _layer(ctx, c, 14, 14, 2, 8, tables, dtype, 1)
+    x, rng = maps[0], np.random.default_rng(c)
+    lengths = [np.stack([tc.tc_host_huffman_lengths(rng.integers(0, 10 ** rng.integers(1, 6), 256)) for _ in range(tables)]) for _ in range(TURNS)]
+    books = [tc.tc_codebook_import(ctx, l, 8) for l in lengths]
+    streams = [tc.tc_encode(ctx, m, b, x) for b in books]
+    want = tc.tc_decode(ctx, m, books[0], streams[0], x.shape, dtype)
+    assert tc.tc_get_status(ctx) == 0
+    got = [torch.empty_like(x) for _ in lengths]
+    side = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    with torch.cuda.stream(side):
+        made = [tc.tc_codebook_import(ctx, lengths[0], 8)]
+        for l, enc, out in zip(lengths, streams, got):
+            made.append(tc.tc_codebook_import(ctx, l, 8))
+            tc.tc_decode(ctx, m, made[-1], enc, x.shape, dtype, out=out)
+        assert tc.tc_get_status(ctx) == 0 and tc.tc_last_path(ctx, True) == path
+    assert all(torch.equal(g, want) for g in got)
+    for h in [m, cb] + books + made:
+        h.close()
