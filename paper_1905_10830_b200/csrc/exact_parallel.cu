@@ -772,6 +772,11 @@ __global__ void __launch_bounds__(kUnpackThreads) unpack_symbols_kernel(DecodeAr
 
 }  // namespace
 
+// Static shared memory of the kernels that are kept apart (-Xptxas -v); of the entropy decoder as kFull.
+constexpr size_t kProjectStatic = 15488, kPackStatic = 5696, kUnpackStatic = 2176, kUnpackFullStatic = 10368;
+// For the tests.
+extern "C" size_t tc_spread_bytes(long long blocks, int sm_count, size_t own) { return spread_bytes(blocks, sm_count, own); }
+
 tc_status tc_launch_project_quantise(const EncodeArgs &a, int dtype, uint8_t *sym, cudaStream_t s)
 {
     if (a.pixels <= 0) return TC_OK;
@@ -781,8 +786,8 @@ tc_status tc_launch_project_quantise(const EncodeArgs &a, int dtype, uint8_t *sy
     // Early where that leaves the basis in L1: with several blocks an SM kept apart by shared memory wide layers lose (512x14x14 f32, 224
     // blocks, 39.0 -> 43.6 us, 176x34x33 22.6 -> 24.3; 32x56x56 10.2 -> 8.3, 96x45x45 15.8 -> 15.3, 256x7x7 20.5 -> 18.8).
     const long long blocks = (long long)grid.x * grid.y;
-    const size_t spread = a.alone && (blocks <= a.sms || a.c <= 128) ? spread_bytes(blocks, a.sms) : 0, own = 16 * 1024;      // (of static variables)
-    return launch_first(spread > 0, kernel, grid, block, spread > own ? spread - own : 0, s, a, sym) == cudaSuccess ? TC_OK : TC_ERR_CUDA;
+    const size_t spread = a.alone && (blocks <= a.sms || a.c <= 128) ? spread_bytes(blocks, a.sms, kProjectStatic) : 0;
+    return launch_first(spread > 0, kernel, grid, block, spread, s, a, sym) == cudaSuccess ? TC_OK : TC_ERR_CUDA;
 }
 
 tc_status tc_launch_reconstruct(const DecodeArgs &a, int dtype, const uint8_t *sym, cudaStream_t s)
@@ -807,7 +812,6 @@ int tc_pack_symbols_parts(const EncodeArgs &a)
 // Coefficients from which a tile is worth a cluster: its barriers cost 2 us (64x56x56 f32 14.3 -> 15.8 us, 128 to 256 coefficients
 // even, 384x7x7 x 64 20.5 -> 18.5).
 constexpr int kClusterCoefs = 384;
-constexpr unsigned int kSpreadBytes = 118 * 1024;             // two of these do not fit an SM
 
 tc_status tc_launch_pack_symbols(const tc_ctx *ctx, const EncodeArgs &a, const uint8_t *sym, long long first_tile, long long end_tile, cudaStream_t s)
 {
@@ -826,7 +830,7 @@ tc_status tc_launch_pack_symbols(const tc_ctx *ctx, const EncodeArgs &a, const u
     void (*kernel)(EncodeArgs, const uint8_t *, int, long long, unsigned int) =
         tile_blocks > 1 ? (a.groups == 1 ? pack_symbols_kernel<true, true> : pack_symbols_kernel<false, true>)
                         : (a.groups == 1 ? pack_symbols_kernel<true, false> : pack_symbols_kernel<false, false>);
-    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSpreadBytes) != cudaSuccess) return TC_ERR_CUDA;
+    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSpreadMost) != cudaSuccess) return TC_ERR_CUDA;
     const dim3 grid((unsigned int)tiles, (unsigned int)tile_blocks), block(TC_TILE_PIXELS / tile_blocks * parts);
     // Set up while the kernel before is still at work, kept apart by shared memory: small blocks that arrive early all pile onto the
     // first SMs that have room (960x7x7 x 128, 49 blocks: 49 us unchained, 65 chained, 48 chained and spread; 64x56x56 f32 17.2
@@ -834,9 +838,9 @@ tc_status tc_launch_pack_symbols(const tc_ctx *ctx, const EncodeArgs &a, const u
     // 22.7).  Not large blocks of which some SMs get two: the first SMs that are free take two each (576x14x14 x 128, 196 blocks of 1 024
     // threads: 55.4 -> 57.4).
     if (tile_blocks > 1)
-        return launch_chained_cluster(tile_blocks, kernel, grid, block, std::max(staging, kSpreadBytes), s, a, sym, parts, first_tile, staging) == cudaSuccess ? TC_OK : TC_ERR_CUDA;
+        return launch_chained_cluster(tile_blocks, kernel, grid, block, std::max<size_t>(staging, kSpreadMost), s, a, sym, parts, first_tile, staging) == cudaSuccess ? TC_OK : TC_ERR_CUDA;
     const bool apart = tiles <= ctx->sm_count || tiles > 2ll * ctx->sm_count || block.x <= 512;
-    const size_t spread = a.alone && apart ? spread_bytes(tiles, ctx->sm_count) : 0;
+    const size_t spread = a.alone && apart ? spread_bytes(tiles, ctx->sm_count, kPackStatic) : 0;
     if (spread > 0)
         return launch_chained(true, kernel, grid, block, std::max<size_t>(staging, spread), s, a, sym, parts, first_tile, staging) == cudaSuccess ? TC_OK : TC_ERR_CUDA;
     kernel<<<grid, block, staging, s>>>(a, sym, parts, first_tile, staging);
@@ -875,7 +879,7 @@ static tc_status launch_unpack(const DecodeArgs &a, void *out, long long first_t
     const int threads = (chunks / parts + 31) / 32 * 32, least = tiles * parts < 4 * sm_count ? 256 : 32;
     // from 16 warps an SM on the shared-memory pipe is what bounds a per-layer decoder (see the kernel)
     const bool full = kOperand && a.groups == 1 && tiles * ((chunks + 31) / 32) >= 16 * (long long)sm_count;
-    const size_t spread = a.alone ? spread_bytes(tiles * parts, sm_count) : 0;
+    const size_t spread = a.alone ? spread_bytes(tiles * parts, sm_count, full ? kUnpackFullStatic : kUnpackStatic) : 0;
     void (*kernel)(DecodeArgs, void *, long long, unsigned int, unsigned int) = spread > 0 ? pick_unpack<kOperand, true>(a.groups != 1, full) : pick_unpack<kOperand, false>(a.groups != 1, full);
     if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024) != cudaSuccess) return TC_ERR_CUDA;
     const size_t rows = full ? (size_t)(threads / 32) * kRowsWarpBytes : 0;

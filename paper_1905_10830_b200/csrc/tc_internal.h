@@ -209,11 +209,15 @@ inline cudaError_t launch_chained(bool early, void (*kernel)(P...), dim3 grid, d
 // holds before them.  Small blocks that arrive early all pile onto the first SMs that have room (decode of 384x8x8 x 241, 121 blocks:
 // 25 -> 56 us), so they ask for as much shared memory as keeps them apart (spread_bytes; more than eight an SM start in their
 // turn: 64x56x56 x 64 with a table per channel, 1 568 blocks, 45 -> 56 us).
-constexpr size_t kSmBytes = 228 * 1024, kSpreadMost = 118 * 1024;
-inline size_t spread_bytes(long long blocks, int sm_count)
+constexpr size_t kSmBytes = 228 * 1024, kBlockBytes = 1024, kSpreadMost = 118 * 1024;       // of an SM; what the system keeps of a block's
+// Dynamic shared memory with which as many blocks fit an SM as it would get of `blocks` and no more, `own` bytes being static variables (0: no
+// spreading).  (The static ones left out of it, seven fitted an SM that was to take eight: decode of 16x16x16 x 592 with a table per channel 28.8 ->
+// 40.2 us, 64x16x16 x 592 33.4 -> 37.3.)
+inline size_t spread_bytes(long long blocks, int sm_count, size_t own)
 {
     const long long per_sm = (blocks + sm_count - 1) / sm_count;
-    return per_sm <= 1 ? kSpreadMost : per_sm <= 8 ? (kSmBytes / (size_t)(per_sm + 1) + 1023) & ~(size_t)1023 : 0;
+    if (per_sm <= 1) return kSpreadMost;
+    return per_sm <= 8 ? (kSmBytes / (size_t)(per_sm + 1) / 1024 + 1) * 1024 - kBlockBytes - own : 0;
 }
 template <typename... P, typename... A>
 inline cudaError_t launch_first(bool alone, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A &&...args)

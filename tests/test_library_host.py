@@ -71,3 +71,19 @@ def test_host_eigh_repeated_eigenvalues(lib):
     ev, vt = tc.tc_host_eigh(np.diag([2.0, 2.0, 1.0, 2.0]))
     assert np.allclose(ev, [2, 2, 2, 1])
     assert np.allclose(vt @ vt.T, np.eye(4), atol=1e-14)
+
+
+# Shared memory that keeps the blocks of kernels that start early apart: as many as an SM would get fit it, and not one more.
+@pytest.mark.parametrize("own", [2176, 5696, 10368, 15488])
+def test_blocks_kept_apart_fit_their_sm(lib, own):
+    import ctypes as C
+    spread = lib.tc_spread_bytes
+    spread.restype, spread.argtypes = C.c_size_t, [C.c_longlong, C.c_int, C.c_size_t]
+    sms, sm, block = 148, 228 * 1024, 1024                     # bytes of an SM, and what the system keeps of a block's
+    for blocks in (1, 2, 147, 148):
+        assert 2 * (spread(blocks, sms, own) + own + block) > sm and spread(blocks, sms, own) + own <= 227 * 1024
+    for per_sm in range(2, 9):
+        for blocks in ((per_sm - 1) * sms + 1, per_sm * sms):
+            each = spread(blocks, sms, own) + own + block
+            assert per_sm * each <= sm < (per_sm + 1) * each
+    assert spread(8 * sms + 1, sms, own) == 0
