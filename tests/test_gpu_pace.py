@@ -1,0 +1,56 @@
+"""Calls that a choice of launch once made several times slower than the work they hold: times beside those of calls with more work, or the same
+work laid out otherwise."""
+import pytest
+import torch
+
+import paper_1905_10830_b200 as tc
+from synth import featuremaps as fm
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def ctx():
+    c = tc.tc_create(0)
+    yield c
+    c.close()
+
+
+def _queued_us(*calls, times=20, rounds=9):
+    """us of each call among others of its kind, the least of several rounds taken in turn."""
+    best = [float("inf")] * len(calls)
+    for _ in range(rounds):
+        for i, call in enumerate(calls):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            call()
+            torch.cuda.synchronize()
+            torch.cuda._sleep(400_000)                         # the calls are queued by the time that the first runs
+            a.record()
+            for _ in range(times):
+                call()
+            b.record()
+            torch.cuda.synchronize()
+            best[i] = min(best[i], a.elapsed_time(b) * 1e3 / times)
+    return best
+
+
+def _layer(ctx, c, h, w, n, bits, tables, dtype):
+    params = fm.layer_params(fm.LayerSpec(c, h, w, 0.93, None, 41000 + c))
+    cal = fm.make_maps(params, max(4, 30000 // (h * w)), calib=True, dtype=dtype, device="cuda")
+    x = fm.make_maps(params, n, dtype=dtype, device="cuda")
+    m = tc.tc_fit_pca(ctx, cal, bits)
+    cb = tc.tc_build_codebook(ctx, m, tc.tc_stats(ctx, m, None, cal, groups=tables).hist, groups=tables)
+    return m, cb, x
+
+
+# The exact inverse behind the entropy decoder: its blocks, early, all on some of the SMs took as long for 10 tiles as for 20 (47.0 and 49.4 us;
+# 31.6 and 49.4 kept apart).
+def test_exact_decodes_of_half_the_tiles(ctx):
+    m, cb, x = _layer(ctx, 256, 8, 16, 20, 5, 1, torch.float32)
+    half, whole = (tc.tc_encode(ctx, m, cb, v) for v in (x[:10], x))
+    out = torch.empty_like(x)
+    few, many = _queued_us(lambda: tc.tc_decode(ctx, m, cb, half, x[:10].shape, x.dtype, out=out[:10]),
+                           lambda: tc.tc_decode(ctx, m, cb, whole, x.shape, x.dtype, out=out))
+    assert tc.tc_get_status(ctx) == 0 and tc.tc_last_path(ctx, True) == 0
+    assert few < 0.8 * many, (few, many)
+    m.close(); cb.close()
