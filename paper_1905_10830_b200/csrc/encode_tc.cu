@@ -206,6 +206,33 @@ __device__ __noinline__ Sink code_again(Sink sink, uint32_t trow, int blk0, int 
     return sink;
 }
 
+// The issuing warp's way through the tiles of a block: the accumulators in turn, the panels of a tile through the ring of stages.  Once a wait has run
+// out it issues nothing more -- what has not landed is not multiplied, and its stage not handed back to be loaded while it is read -- and
+// it leaves only when what it has issued is done: the block frees tensor memory next.  (Not by leaving the inner loop at the wait, which keeps it from being unrolled.)
+#pragma nv_exec_check_disable
+template <int kGroups, typename Basis, typename Accumulator, typename Landed, typename Panel, typename Done, typename Drain>
+__host__ __device__ __forceinline__ bool issue_tiles(long long tiles, int panels, int stages, Basis basis, Accumulator accumulator, Landed landed, Panel panel,
+                                                     Done done, Drain drain)
+{
+    if (!basis()) return false;
+    bool alive = true;
+    int s = 0;
+    uint32_t phase = 0;
+    for (long long tl = 0; tl < tiles && alive; ++tl) {
+        const int acc = (int)(tl % kGroups);
+        if (!accumulator(acc, (uint32_t)(((tl / kGroups) & 1) ^ 1))) { alive = false; break; }
+#pragma unroll 4
+        for (int kp = 0; kp < panels; ++kp) {
+            if (alive) alive = landed(s, phase);
+            panel(kp, s, alive);
+            if (++s == stages) { s = 0; phase ^= 1u; }
+        }
+        if (alive) done(acc);
+    }
+    drain();
+    return alive;
+}
+
 // The epilogue's two ways (kRuns):
 //   one pass: every thread packs the codes of its coefficients, as they are quantised, into a private
 //     run of words in shared memory (word w of all threads side by side: no bank conflicts); when
@@ -381,47 +408,45 @@ __device__ __forceinline__ void encode_tiles(const EncodeArgs &a, const Plan &pl
                 if (++s == n_stages) { s = 0; phase ^= 1u; }
             }
         }
-        if (!alive) {
-            cp_async_wait_all();
-            tc_dev_set_status(a.status, TC_ERR_TIMEOUT);
-        }
+        cp_async_wait_all();                       // (of a block whose other waits ran out, too)
+        if (!alive) tc_dev_set_status(a.status, TC_ERR_TIMEOUT);
     } else if (warp == kMmaWarp) {
         // ================= MMA issuer =================
-        // The whole warp walks the loop and waits on the barriers; lane 0 issues, through instructions
+        // The whole warp walks the loop (issue_tiles) and waits on the barriers; lane 0 issues, through instructions
         // that carry their own guard (a branch taken by one lane around every MMA costs about 90
         // cycles per instruction).
-        {
-            const uint32_t issuer = lane == 0 ? 1u : 0u;
-            const uint32_t idesc = make_idesc_bf16(TC_TILE_PIXELS, a.k, /*A MN-major*/ true, /*B K-major*/ false);
-            const uint64_t a_desc = make_smem_desc_mn_sw128(ring_addr, kStageBytes / 2, 1024);
-            const uint64_t b_desc = make_smem_desc(basis_addr, 128, (uint32_t)(a.c / 8) * 128u);
-            const uint32_t a_desc_lo = (uint32_t)a_desc, a_desc_hi = (uint32_t)(a_desc >> 32), b_desc_hi = (uint32_t)(b_desc >> 32);
-            int s = 0;
-            uint32_t phase = 0;
-            bool alive = mbar_wait(smem_u32(&s_basis_ready), 0u);
-            for (long long tl = 0; tl < my_tiles && alive; ++tl) {
-                const int acc = (int)(tl % kGroups);
-                if (!mbar_wait(smem_u32(&s_tempty[acc]), (uint32_t)(((tl / kGroups) & 1) ^ 1))) { alive = false; break; }
+        const uint32_t issuer = lane == 0 ? 1u : 0u;
+        const uint32_t idesc = make_idesc_bf16(TC_TILE_PIXELS, a.k, /*A MN-major*/ true, /*B K-major*/ false);
+        const uint64_t a_desc = make_smem_desc_mn_sw128(ring_addr, kStageBytes / 2, 1024);
+        const uint64_t b_desc = make_smem_desc(basis_addr, 128, (uint32_t)(a.c / 8) * 128u);
+        const uint32_t a_desc_lo = (uint32_t)a_desc, a_desc_hi = (uint32_t)(a_desc >> 32), b_desc_hi = (uint32_t)(b_desc >> 32);
+        uint32_t d_tmem = 0, b_lo = 0;
+        const bool alive = issue_tiles<kGroups>(
+            my_tiles, n_panels, n_stages,
+            [&] { return mbar_wait(smem_u32(&s_basis_ready), 0u); },
+            [&](int acc, uint32_t parity) {
+                if (!mbar_wait(smem_u32(&s_tempty[acc]), parity)) return false;
                 tc_fence_after_sync();
-                const uint32_t d_tmem = tmem_base + acc * kAccCols;
-                uint32_t b_lo = (uint32_t)b_desc;
-#pragma unroll 4
-                for (int kp = 0; kp < n_panels; ++kp) {
-                    if (alive) alive = mbar_wait(smem_u32(&s_full[s]), phase);
-                    fence_proxy_async_smem();            // the loaders' copies, made visible to the tensor core
-                    tc_fence_after_sync();
-                    const uint32_t a_lo = a_desc_lo + (uint32_t)s * (kStageBytes >> 4);
-                    mma_bf16_ss_guarded(d_tmem, a_lo, a_desc_hi, b_lo, b_desc_hi, idesc, kp ? 1u : 0u, issuer);
-                    if ((kp + 1) * kPanelCh <= a.c)          // else half a panel
-                        mma_bf16_ss_guarded(d_tmem, a_lo + (2048u >> 4), a_desc_hi, b_lo + (256u >> 4), b_desc_hi, idesc, 1u, issuer);
-                    b_lo += (kPanelCh / 8) * (128u >> 4);
-                    mma_commit_guarded(smem_u32(&s_empty[s]), issuer);
-                    if (++s == n_stages) { s = 0; phase ^= 1u; }
-                }
-                if (alive) mma_commit_guarded(smem_u32(&s_tfull[acc]), issuer);
-            }
-            if (!alive && issuer) tc_dev_set_status(a.status, TC_ERR_TIMEOUT);
-        }
+                d_tmem = tmem_base + acc * kAccCols;
+                b_lo = (uint32_t)b_desc;
+                return true;
+            },
+            [&](int s, uint32_t parity) { return mbar_wait(smem_u32(&s_full[s]), parity); },
+            [&](int kp, int s, bool issue) {
+                const uint32_t on = issue ? issuer : 0u;
+                fence_proxy_async_smem();            // the loaders' copies, made visible to the tensor core
+                tc_fence_after_sync();
+                const uint32_t a_lo = a_desc_lo + (uint32_t)s * (kStageBytes >> 4);
+                mma_bf16_ss_guarded(d_tmem, a_lo, a_desc_hi, b_lo, b_desc_hi, idesc, kp ? 1u : 0u, on);
+                if ((kp + 1) * kPanelCh <= a.c)          // else half a panel
+                    mma_bf16_ss_guarded(d_tmem, a_lo + (2048u >> 4), a_desc_hi, b_lo + (256u >> 4), b_desc_hi, idesc, 1u, on);
+                b_lo += (kPanelCh / 8) * (128u >> 4);
+                mma_commit_guarded(smem_u32(&s_empty[s]), on);
+            },
+            [&](int acc) { mma_commit_guarded(smem_u32(&s_tfull[acc]), issuer); },
+            // (the basis has come: its barrier is in its second phase)
+            [&] { mma_commit_guarded(smem_u32(&s_basis_ready), issuer); mbar_wait(smem_u32(&s_basis_ready), 1u); });
+        if (!alive && issuer) tc_dev_set_status(a.status, TC_ERR_TIMEOUT);
     } else if (warp >= kStoreWarp0) {
         // ================= store warps =================
         unsigned int stopped = 0;                                // groups that hand over nothing more
@@ -868,6 +893,22 @@ __global__ void __launch_bounds__(kThreads, 1) encode_tc_list_kernel(const __gri
 }
 
 }  // namespace
+
+// For the tests: what the issuing warp does when its wait number `fails` (0 ...; none if negative) runs out, one event an entry: 100 + stage (a panel's
+// products and its stage handed back), 200 + accumulator (handed on), 300 (the wait for all of it), -1 (the wait that ran out).  The number of events.
+extern "C" int tc_issue_events(int groups, long long tiles, int panels, int stages, int fails, int32_t *events, int room)
+{
+    int n = 0;
+    auto put = [&](int32_t e) { if (n < room) events[n] = e; ++n; };
+    auto wait = [&] { if (fails-- != 0) return true; put(-1); return false; };
+    auto on_barrier = [&](int, uint32_t) { return wait(); };
+    auto panel = [&](int, int s, bool issue) { if (issue) put(100 + s); };
+    auto done = [&](int acc) { put(200 + acc); };
+    auto drain = [&] { put(300); };
+    if (groups == 4) issue_tiles<4>(tiles, panels, stages, wait, on_barrier, on_barrier, panel, done, drain);
+    else issue_tiles<2>(tiles, panels, stages, wait, on_barrier, on_barrier, panel, done, drain);
+    return n;
+}
 
 // Coefficients up to which four accumulators fit tensor memory and a thread codes a pixel.
 constexpr int kFourGroupsCoefs = 128;

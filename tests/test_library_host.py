@@ -87,3 +87,28 @@ def test_blocks_kept_apart_fit_their_sm(lib, own):
             each = spread(blocks, sms, own) + own + block
             assert per_sm * each <= sm < (per_sm + 1) * each
     assert spread(8 * sms + 1, sms, own) == 0
+
+
+# The resident-basis encoder's issuing warp when one of its waits runs out: no products of what has not landed, no stage handed back, no
+# accumulator handed on, and it leaves when what it has issued is done.
+@pytest.mark.parametrize("groups,tiles,panels,stages", [(4, 1, 1, 8), (4, 9, 4, 6), (2, 3, 8, 8), (2, 5, 7, 6)])
+def test_nothing_is_issued_after_a_wait_that_ran_out(lib, groups, tiles, panels, stages):
+    import ctypes as C
+    call = lib.tc_issue_events
+    call.restype, call.argtypes = C.c_int, [C.c_int, C.c_longlong, C.c_int, C.c_int, C.c_int, C.POINTER(C.c_int32), C.c_int]
+    room = (C.c_int32 * 4096)()
+
+    def events(fails):
+        n = call(groups, tiles, panels, stages, fails, room, len(room))
+        assert 0 < n <= len(room)
+        return list(room[:n])
+    want, at = [], 0
+    for tl in range(tiles):
+        want += [100 + (at + i) % stages for i in range(panels)] + [200 + tl % groups]
+        at += panels
+    assert events(-1) == want + [300]
+    assert events(0) == [-1]                                   # the basis: nothing has been issued
+    for fails in range(1, 1 + tiles * (1 + panels)):
+        tl, i = divmod(fails - 1, 1 + panels)                  # wait i of a tile: its accumulator, then its panels
+        issued = want[:tl * (panels + 1) + max(0, i - 1)]
+        assert events(fails) == issued + [-1, 300]
