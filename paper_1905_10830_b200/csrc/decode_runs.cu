@@ -246,7 +246,7 @@ template <bool kRelu>
 __device__ __forceinline__ void decode_tiles(const DecodeArgs &a, const SmemLayout &L, unsigned int block, unsigned int blocks)
 {
     extern __shared__ __align__(128) unsigned char smem[];
-    __shared__ __align__(8) unsigned long long s_empty[kMaxGroups][kMaxPanels], s_bfull[kMaxGroups], s_tfull[2];
+    __shared__ __align__(8) unsigned long long s_empty[kMaxGroups][kMaxPanels], s_bfull[kMaxGroups], s_tfull[2], s_drained;
     __shared__ uint32_t s_tmem_base;
     // [group][tile parity][thread set][warp]: bits per warp, for the start positions.  Two copies: a warp
     // that is done with its tile early writes the next tile's sum while a slower warp may still
@@ -274,6 +274,7 @@ __device__ __forceinline__ void decode_tiles(const DecodeArgs &a, const SmemLayo
         if (p < kMaxPanels) mbar_init(smem_u32(&s_empty[g][p]), 1);                     // the commit of the tile's last item
         else mbar_init(smem_u32(&s_bfull[g]), (uint32_t)group_warps);                   // operand complete: one arrival per warp
         if (tid < 2) mbar_init(smem_u32(&s_tfull[tid]), 1);
+        if (tid == 2) mbar_init(smem_u32(&s_drained), 1);
         mbar_fence_init();
     }
     if (warp == kMmaWarp) { tmem_alloc(smem_u32(&s_tmem_base), kTmemCols); tmem_relinquish(); }
@@ -770,6 +771,9 @@ __device__ __forceinline__ void decode_tiles(const DecodeArgs &a, const SmemLayo
                 }
                 if (++buf == G) { buf = 0; turn ^= 1u; }
             }
+            // the block frees tensor memory next: not ahead of MMAs that nobody waits for (an epilogue whose own wait ran out)
+            mma_commit_guarded(smem_u32(&s_drained), issuer);
+            mbar_wait(smem_u32(&s_drained), 0u);
             if (!alive && issuer) tc_dev_set_status(a.status, TC_ERR_TIMEOUT);
         }
     }
