@@ -77,25 +77,28 @@ struct SmemLayout {
     uint32_t opnd_bytes;                                      // one operand buffer (one per VLD group)
     uint32_t stream_buf;                                      // bytes per staged stream buffer (two per group; 0: does not fit)
     int groups;                                               // VLD groups
+    int mode;                                                 // how the tensor's values leave (see store_mode)
 };
+enum { kRows16, kRows8, kRowsAny, kMaps };
 
 // group_warps: warps of a VLD group.  As many groups as warps and shared memory allow beside stream
 // buffers of `want_bytes`, what a tile's segment is expected to take (two groups: for what is left, at least 4 KB).  A segment
 // that does not fit its buffer is read from global memory word by word, which costs more than a group less: with room
 // for 2.5 bits per symbol whatever the rate, 512 maps of 28x28 at 8 bits (4.8 to 4.3 bits per value) took 115 us at
 // 128 channels, 186 at 176 and 200 at 192; sized by the rate 95, 153 and 163, and 256 maps of 64x56x56 121 -> 101.
-inline SmemLayout smem_layout(int k, int lut_entries, int group_warps, uint32_t want_bytes, bool row_blocks, int budget)
+inline SmemLayout smem_layout(int k, int lut_entries, int group_warps, uint32_t want_bytes, int mode, int budget)
 {
     SmemLayout l;
     l.lut = 0;                                                // 32-bit entries: bf16(symbol - center) << 16 | length
     l.opnd = ((uint32_t)lut_entries * 4u + 1023u) & ~1023u;
     l.opnd_bytes = (uint32_t)k * TC_TILE_PIXELS * 2;
     const int most = kVldWarps / group_warps < kMaxGroups ? kVldWarps / group_warps : kMaxGroups;
+    l.mode = mode;
     l.stream_buf = 0;
     l.total = 0;
     for (l.groups = most; l.groups >= 2; --l.groups) {
         l.tbuf = l.opnd + (uint32_t)l.groups * l.opnd_bytes;
-        l.sbuf = l.tbuf + (row_blocks ? 8u * kTrWarpBytes : 0u);
+        l.sbuf = l.tbuf + (mode != kRows16 ? 8u * kTrWarpBytes : 0u);
         const long long left = (long long)budget - l.sbuf - kStreamSlack;
         const long long room = (left / (2ll * l.groups)) & ~127ll;
         if (room < 4096 || (room < (long long)want_bytes && l.groups > 2)) continue;
@@ -219,10 +222,15 @@ struct BitReader {
 //            64 of eight rows an instruction, a row's four pieces in succession;
 //   kRows8:  the same of groups of four: through a block of the warp in shared memory, a row an instruction, 8 bytes a thread;
 //   kRowsAny: rows that start anywhere (H*W no multiple of 4, an unaligned tensor): through the block, a pixel a thread, a row in four
-//            instructions in succession.
-enum { kRows16, kRows8, kRowsAny };
-__host__ __device__ inline int store_mode(const DecodeArgs &a)
+//            instructions in succession;
+//   kMaps:   maps of up to four pixels: their rows are all over memory, but 32 channels of a map lie in a line or two: a channel a thread (two where
+//            a map is a pixel), a map or a pixel an instruction.  As rows they took several times as long (us as rows and so: 208x1x1 x 229248, 96
+//            coefficients, 444 and 50; 112x1x2 x 54144 65 and 23; 256x1x3 x 32720 129 and 40; 160x2x2 x 40800 67 and 46).  Five pixels leave faster
+//            as rows, as do 16 channels, of which a line holds several maps (16x1x2 x 46848: rows 21, so 23).
+constexpr int kSmallMap = 4;
+inline int store_mode(const DecodeArgs &a)
 {
+    if (a.hw <= kSmallMap && a.c > 16) return kMaps;
     if ((a.hw & 3) != 0 || ((uintptr_t)a.xhat & 7u) != 0) return kRowsAny;
     return (a.hw & 7) == 0 && ((uintptr_t)a.xhat & 15u) == 0 ? kRows16 : kRows8;
 }
@@ -231,6 +239,23 @@ __host__ __device__ inline int store_mode(const DecodeArgs &a)
 // pixels 8 q + 2 g + {0, 1}.
 __device__ __forceinline__ uint32_t column_of(uint32_t p) { return (p & ~31u) | ((p & 6u) << 2) | ((p >> 2) & 6u) | (p & 1u); }
 __device__ __forceinline__ uint32_t pixel_of(uint32_t n) { return (n & ~31u) | ((n & 6u) << 2) | ((n >> 2) & 6u) | (n & 1u); }
+
+// two accumulator values -> two bf16: x_hat = step * acc + bias (one packed fused multiply-add)
+template <bool kRelu>
+__device__ __forceinline__ uint32_t decoded_pair(uint32_t x0, uint32_t x1, float step, float bias)
+{
+    float f0, f1;
+    asm("{\n\t.reg .b64 v, s, b;\n\t"
+        "mov.b64 v, {%2, %3};\n\t"
+        "mov.b64 s, {%4, %4};\n\t"
+        "mov.b64 b, {%5, %5};\n\t"
+        "fma.rn.f32x2 v, v, s, b;\n\t"
+        "mov.b64 {%0, %1}, v;\n\t}"
+        : "=f"(f0), "=f"(f1) : "r"(x0), "r"(x1), "f"(step), "f"(bias));
+    if constexpr (kRelu) { f0 = fmaxf(f0, 0.f); f1 = fmaxf(f1, 0.f); }   // the layer's non-linearity, when it follows the decoder
+    const __nv_bfloat162 h = __floats2bfloat162_rn(f0, f1);
+    return *reinterpret_cast<const uint32_t *>(&h);
+}
 
 // The thread's index, read anew: what a role derives from its own reading is not worked out ahead of the other roles and kept through them (with
 // registers as short as here such values went to local memory, that is to L2: L1 is what shared memory leaves of it).
@@ -567,32 +592,102 @@ __device__ __forceinline__ void decode_tiles(const DecodeArgs &a, const SmemLayo
             cp_async_wait<0>();
             if (!alive) tc_dev_set_status(a.status, TC_ERR_TIMEOUT);
         }
+    } else if (warp < kMmaWarp && L.mode == kMaps) {
+        // ================= epilogue, maps of up to kSmallMap pixels =================
+        // As below, but for a thread's 16 columns of its own channel at a time.
+        const int warp = own_tid() >> 5, lane = own_tid() & 31;
+        const int set = (warp - kEpiWarp0) >> 2, wq = warp & 3;
+        const int n_items = my_tiles * items;
+        const bool shared = n_items == 1;                         // one item only: half of the pixels each
+        const int acc = shared ? 0 : set;
+        const int hw = (int)a.hw, map = a.c * hw;
+        const int ch = (items == 2 ? set * 128 : 0) + wq * 32 + lane;
+        const bool ch_ok = ch < a.c;
+        const float step = (float)(a.step * a.basis_scale), bias = ch_ok ? __ldg(a.dec_bias + ch) : 0.f;
+        // bytes that leave at a time: a map's row of the channel, or one pixel of two channels (the neighbouring lane's), or of one
+        const bool fours = hw == 4 && ((uintptr_t)a.xhat & 7u) == 0, twos = hw == 2 && ((uintptr_t)a.xhat & 3u) == 0;
+        const bool pairs = hw == 1 && ((uintptr_t)a.xhat & 3u) == 0;
+        const int odd = lane & 1;
+        const uint32_t places = smem_u32(smem + L.tbuf) + (uint32_t)(warp - kEpiWarp0) * kTrWarpBytes;       // of a tile's pixels in the tensor, where neither holds
+        const uint32_t trow = tmem_base + kAccBase + acc * kAccCols + ((uint32_t)(wq * 32) << 16);
+        bool alive = true;
+        chain_wait();                                            // earlier readers of the tensor
+        for (int it = acc; it < n_items; it += 2) {
+            const long long tile = block + (long long)(items == 2 ? it >> 1 : it) * blocks, img = tile * TC_TILE_PIXELS / hw;
+            const int sp = (int)(tile * TC_TILE_PIXELS - img * hw);
+            const int n_valid = ch_ok ? (int)min((long long)TC_TILE_PIXELS, a.pixels - tile * TC_TILE_PIXELS) : 0;
+            __nv_bfloat16 *const out = reinterpret_cast<__nv_bfloat16 *>(a.xhat) + img * map + (long long)ch * hw;
+            if (wq == 0) {
+                if (alive) alive = mbar_wait(smem_u32(&s_tfull[acc]), (uint32_t)((it >> 1) & 1), 50u);
+                tc_fence_before_sync();
+            }
+            named_bar_sync(kBarEpi + set, 128);
+            tc_fence_after_sync();
+            if (!pairs && !fours && !twos) {
+                int to[4];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const int x = sp + 4 * lane + i, m = hw == 3 ? (x * 171) >> 9 : x >> (hw >> 1);          // x / hw
+                    to[i] = m * map + (x - m * hw);
+                }
+                sts_v4(places + 16u * lane, to[0], to[1], to[2], to[3]);
+                __syncwarp();
+            }
+#pragma unroll 1
+            for (int c0 = shared ? 64 * set : 0; c0 < (shared ? 64 * set + 64 : TC_TILE_PIXELS); c0 += 16) {
+                uint32_t r[16];
+                tmem_ld_32x32b_x16(trow + c0, r);
+                tmem_ld_wait(r);
+                const int px0 = (int)pixel_of((uint32_t)c0);      // column c0 + 8 g + 2 q + {0, 1}: pixel px0 + 8 q + 2 g + {0, 1}
+                int at = (pairs ? px0 + odd : fours ? px0 >> 2 : px0 >> 1) * map - (pairs ? odd : 0);
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    uint32_t w[2];
+#pragma unroll
+                    for (int g = 0; g < 2; ++g) w[g] = decoded_pair<kRelu>(r[8 * g + 2 * q], r[8 * g + 2 * q + 1], step, bias);
+                    const int px = px0 + 8 * q;
+                    if (pairs) {
+#pragma unroll
+                        for (int g = 0; g < 2; ++g) {
+                            const uint32_t theirs = __shfl_xor_sync(0xffffffffu, w[g], 1);
+                            const uint32_t v = __byte_perm(w[g], theirs, odd ? 0x3276 : 0x5410);
+                            if (px + 2 * g + odd < n_valid) *reinterpret_cast<uint32_t *>(out + (at + 2 * g * map)) = v;
+                        }
+                        at += 8 * map;
+                    } else if (fours) {
+                        if (px < n_valid) *reinterpret_cast<uint2 *>(out + at) = make_uint2(w[0], w[1]);
+                        at += 2 * map;
+                    } else if (twos) {
+#pragma unroll
+                        for (int g = 0; g < 2; ++g)
+                            if (px + 2 * g < n_valid) *reinterpret_cast<uint32_t *>(out + (at + g * map)) = w[g];
+                        at += 4 * map;
+                    } else {
+                        int to[4];
+                        asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(to[0]), "=r"(to[1]), "=r"(to[2]), "=r"(to[3]) : "r"(places + 4u * px));
+#pragma unroll
+                        for (int i = 0; i < 4; ++i)
+                            if (px + i < n_valid) *reinterpret_cast<unsigned short *>(out + to[i]) = (unsigned short)(w[i >> 1] >> (16 * (i & 1)));
+                    }
+                }
+            }
+            tc_fence_before_sync();
+            if (!shared) named_bar_arrive(kBarAccFree + acc, 128 + 32);
+        }
+        if (!alive && lane == 0) tc_dev_set_status(a.status, TC_ERR_TIMEOUT);
     } else if (warp < kMmaWarp) {
         // ================= epilogue =================
         // An item is a tile's 128 pixels of one block of 128 channels.  Four warps serve each accumulator, so that the waits of one
         // item run beside the work of another; a warp stores the 32 channels of its quarter of TMEM, 16 at a time.
         const int warp = own_tid() >> 5, lane = own_tid() & 31;
-        const int mode = store_mode(a);
+        const int mode = L.mode;
         const int set = (warp - kEpiWarp0) >> 2, wq = warp & 3;
         const int n_items = my_tiles * items;
         const bool shared = n_items == 1;                         // one item only: half of the channels each
         const int acc = shared ? 0 : set;
         const float step = (float)(a.step * a.basis_scale);        // the operand holds basis / basis_scale
         __nv_bfloat16 *out = reinterpret_cast<__nv_bfloat16 *>(a.xhat);
-        // two accumulator values -> two bf16: x_hat = step * acc + bias (one packed fused multiply-add)
-        auto convert = [&](uint32_t x0, uint32_t x1, float bias) {
-            float f0, f1;
-            asm("{\n\t.reg .b64 v, s, b;\n\t"
-                "mov.b64 v, {%2, %3};\n\t"
-                "mov.b64 s, {%4, %4};\n\t"
-                "mov.b64 b, {%5, %5};\n\t"
-                "fma.rn.f32x2 v, v, s, b;\n\t"
-                "mov.b64 {%0, %1}, v;\n\t}"
-                : "=f"(f0), "=f"(f1) : "r"(x0), "r"(x1), "f"(step), "f"(bias));
-            if constexpr (kRelu) { f0 = fmaxf(f0, 0.f); f1 = fmaxf(f1, 0.f); }   // the layer's non-linearity, when it follows the decoder
-            const __nv_bfloat162 h = __floats2bfloat162_rn(f0, f1);
-            return *reinterpret_cast<const uint32_t *>(&h);
-        };
+        auto convert = [&](uint32_t x0, uint32_t x1, float bias) { return decoded_pair<kRelu>(x0, x1, step, bias); };
         // Position of this lane's first pixel of a tile: image and offset inside it of the block's first tile, moved on from
         // tile to tile by a constant number of pixels (a division of 64-bit numbers per item was a fifth of
         // the epilogue's instructions).
@@ -814,7 +909,7 @@ static SmemLayout runs_layout(const tc_ctx *ctx, const DecodeArgs &a)
     // (a dense tile's segment is at most 3 % longer than the mean)
     const double tile_bytes = a.mean_tile_bytes > 0 ? a.mean_tile_bytes : std::max(2.5, (double)a.code_bits) * a.k * TC_TILE_PIXELS / 8;
     const uint32_t want = (uint32_t)std::min(1.03 * tile_bytes, 1e6);
-    return smem_layout(a.k, 1 << a.lut_bits, (group_work(a.splits, a.chunk_pixels) + 31) / 32, want, store_mode(a) != kRows16, ctx->max_smem_optin - kStaticSmem);
+    return smem_layout(a.k, 1 << a.lut_bits, (group_work(a.splits, a.chunk_pixels) + 31) / 32, want, store_mode(a), ctx->max_smem_optin - kStaticSmem);
 }
 
 // The roles' registers are dealt from what a block is launched with: with fewer a thread than this the VLD warps would wait for theirs
@@ -859,11 +954,11 @@ tc_status tc_launch_decode_runs(const tc_ctx *ctx, const DecodeArgs &a, cudaStre
 }
 
 // us that a tile takes a block: 1.6 with 64 coefficients at 1.1 bits each, 1.8 with 128, 2.7 with 160 (two items a tile), 3.5 with 256; 2.9
-// with 128 at 4.1 bits, 5.8 with 256; 0.9 more for every 128 channels where rows start anywhere (40 tiles a block, less the first)
+// with 128 at 4.1 bits, 5.8 with 256; 0.9 more for every 128 channels where rows start anywhere, 0.5 of small maps (40 tiles a block, less the first)
 double tc_decode_runs_tile_us(const DecodeArgs &a)
 {
     const double bits = a.mean_tile_bytes > 0 ? a.mean_tile_bytes * 8.0 / TC_TILE_PIXELS : (double)a.code_bits * a.k;
-    return 1.25 + (a.c > 128 ? 0.9 : 0.0) + 0.0035 * std::max(0, a.k - 128) + 0.003 * bits + (store_mode(a) == kRowsAny ? 0.9 * ((a.c + 127) / 128) : 0.0);
+    return 1.25 + (a.c > 128 ? 0.9 : 0.0) + 0.0035 * std::max(0, a.k - 128) + 0.003 * bits + (store_mode(a) == kRowsAny ? 0.9 : store_mode(a) == kMaps ? 0.5 : 0.0) * ((a.c + 127) / 128);
 }
 
 // Decodes tensors that tc_decode_runs_supported takes, all with the same `relu`, on `sms` SMs, in list_launches launches.

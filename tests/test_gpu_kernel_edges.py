@@ -326,6 +326,22 @@ def test_rows_of_the_run_skipping_decoder(ctx, c, h, w, n):
     m.close(); cb.close()
 
 
+# Maps of up to four pixels, whose channels leave side by side: 2, 4 and 8 bytes a thread (tensors that start anywhere), one item and several, a
+# last tile of a pixel or a map, channels that end inside a warp's 32, maps that begin in the tile before (three pixels), the non-linearity.
+@pytest.mark.parametrize("c,h,w,n", [(16, 1, 2, 5), (48, 3, 1, 43), (128, 1, 3, 700), (144, 1, 3, 1), (176, 1, 1, 129), (208, 4, 1, 33), (256, 1, 2, 20000), (240, 2, 2, 6000),
+                                     (80, 1, 1, 38000), (112, 1, 3, 25000)])
+def test_small_maps_of_the_run_skipping_decoder(ctx, c, h, w, n):
+    test_rows_of_the_run_skipping_decoder(ctx, c, h, w, n)
+    params = fm.layer_params(fm.LayerSpec(c, h, w, 0.9, None, 23000 + c))
+    cal, x = (fm.make_maps(params, m, calib=m > n, dtype=torch.bfloat16, device="cuda") for m in (max(n + 1, 12000), n))
+    m = tc.tc_fit_pca(ctx, cal, 5)
+    cb = tc.tc_build_codebook(ctx, m, tc.tc_stats(ctx, m, None, cal).hist)
+    enc = tc.tc_encode(ctx, m, cb, x)
+    got = [tc.tc_decode(ctx, m, cb, enc, x.shape, x.dtype, relu=r) for r in (False, True)]
+    assert tc.tc_get_status(ctx) == 0 and tc.tc_last_path(ctx, True) == 1 and torch.equal(got[0].clamp(min=0), got[1])
+    m.close(); cb.close()
+
+
 # Run-skipping decoder, stream buffers sized by the rate: three groups and one work item per tile (128 and 112
 # channels), buffers above 16 KB, segments that fit no buffer, and hints that are too small or too large -- the hint
 # changes how tiles are staged, never the tensor.  Against the fp64 kernels on the same stream.

@@ -54,3 +54,17 @@ def test_exact_decodes_of_half_the_tiles(ctx):
     assert tc.tc_get_status(ctx) == 0 and tc.tc_last_path(ctx, True) == 0
     assert few < 0.8 * many, (few, many)
     m.close(); cb.close()
+
+
+# Decodes of one stream as maps of a pixel, two and three take about what larger maps of as many pixels take (208 channels as 1x3 82 us, as 14x12 26 when
+# channels of small maps left as rows; twice the time is the line).
+@pytest.mark.parametrize("w", [1, 2, 3])
+def test_decodes_of_small_maps(ctx, w):
+    m, cb, x = _layer(ctx, 208, 14, 12, 600, 4, 1, torch.bfloat16)
+    enc = tc.tc_encode(ctx, m, cb, x)
+    small = (x.shape[0] * 168 // w, 208, 1, w)
+    out, as_small = torch.empty_like(x), torch.empty(small, dtype=x.dtype, device="cuda")
+    large, us = _queued_us(lambda: tc.tc_decode(ctx, m, cb, enc, x.shape, x.dtype, out=out), lambda: tc.tc_decode(ctx, m, cb, enc, small, x.dtype, out=as_small))
+    assert tc.tc_get_status(ctx) == 0 and tc.tc_last_path(ctx, True) == 1
+    assert us < 2.0 * large, (us, large)
+    m.close(); cb.close()
