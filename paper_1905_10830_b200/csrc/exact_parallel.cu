@@ -772,8 +772,14 @@ __global__ void __launch_bounds__(kUnpackThreads) unpack_symbols_kernel(DecodeAr
 
 }  // namespace
 
-// Static shared memory of the kernels that are kept apart (-Xptxas -v); of the entropy decoder as kFull.
-constexpr size_t kProjectStatic = 15488, kReconstructStatic = 12544, kPackStatic = 5696, kUnpackStatic = 2176, kUnpackFullStatic = 10368;
+// Static shared memory of a kernel that is kept apart, asked for once: a byte or two of another variant's let one block more onto an SM.
+static size_t static_bytes(const void *kernel)
+{
+    cudaFuncAttributes at;
+    if (cudaFuncGetAttributes(&at, kernel) == cudaSuccess) return at.sharedSizeBytes;
+    cudaGetLastError();
+    return 0;
+}
 // For the tests.
 extern "C" size_t tc_spread_bytes(long long blocks, int sm_count, size_t own) { return spread_bytes(blocks, sm_count, own); }
 
@@ -786,7 +792,8 @@ tc_status tc_launch_project_quantise(const EncodeArgs &a, int dtype, uint8_t *sy
     // Early where that leaves the basis in L1: with several blocks an SM kept apart by shared memory wide layers lose (512x14x14 f32, 224
     // blocks, 39.0 -> 43.6 us, 176x34x33 22.6 -> 24.3; 32x56x56 10.2 -> 8.3, 96x45x45 15.8 -> 15.3, 256x7x7 20.5 -> 18.8).
     const long long blocks = (long long)grid.x * grid.y;
-    const size_t spread = a.alone && (blocks <= a.sms || a.c <= 128) ? spread_bytes(blocks, a.sms, kProjectStatic) : 0;
+    static const size_t own[2] = {static_bytes((const void *)project_quantise_kernel<float>), static_bytes((const void *)project_quantise_kernel<__nv_bfloat16>)};
+    const size_t spread = a.alone && (blocks <= a.sms || a.c <= 128) ? spread_bytes(blocks, a.sms, own[dtype != TC_F32]) : 0;
     return launch_first(spread > 0, kernel, grid, block, spread, s, a, sym) == cudaSuccess ? TC_OK : TC_ERR_CUDA;
 }
 
@@ -800,7 +807,8 @@ tc_status tc_launch_reconstruct(const DecodeArgs &a, int dtype, const uint8_t *s
     // an SM gets several (f32, us without and with: 256x8x16 x 10 47.0 and 31.6, 128x8x16 x 20 27.7 and 20.0, 64x8x16 x 36 18.1 and 15.1; fewer or
     // lighter ones lose by it, 32x8x16 x 17 13.4 and 14.2, 64x8x16 x 26 13.3 and 13.9).
     const long long blocks = (long long)grid.x * grid.y;
-    const size_t spread = a.alone && blocks > (a.k >= 128 ? 2 : 3) * (long long)a.sms ? spread_bytes(blocks, a.sms, kReconstructStatic) : 0;
+    static const size_t own[2] = {static_bytes((const void *)reconstruct_kernel<float>), static_bytes((const void *)reconstruct_kernel<__nv_bfloat16>)};
+    const size_t spread = a.alone && blocks > (a.k >= 128 ? 2 : 3) * (long long)a.sms ? spread_bytes(blocks, a.sms, own[dtype != TC_F32]) : 0;
     return launch_chained(a.alone, kernel, grid, block, spread, s, a, sym) == cudaSuccess ? TC_OK : TC_ERR_CUDA;
 }
 
@@ -846,7 +854,8 @@ tc_status tc_launch_pack_symbols(const tc_ctx *ctx, const EncodeArgs &a, const u
     if (tile_blocks > 1)
         return launch_chained_cluster(tile_blocks, kernel, grid, block, std::max<size_t>(staging, kSpreadMost), s, a, sym, parts, first_tile, staging) == cudaSuccess ? TC_OK : TC_ERR_CUDA;
     const bool apart = tiles <= ctx->sm_count || tiles > 2ll * ctx->sm_count || block.x <= 512;
-    const size_t spread = a.alone && apart ? spread_bytes(tiles, ctx->sm_count, kPackStatic) : 0;
+    static const size_t own[2] = {static_bytes((const void *)pack_symbols_kernel<true, false>), static_bytes((const void *)pack_symbols_kernel<false, false>)};
+    const size_t spread = a.alone && apart ? spread_bytes(tiles, ctx->sm_count, own[a.groups != 1]) : 0;
     if (spread > 0)
         return launch_chained(true, kernel, grid, block, std::max<size_t>(staging, spread), s, a, sym, parts, first_tile, staging) == cudaSuccess ? TC_OK : TC_ERR_CUDA;
     kernel<<<grid, block, staging, s>>>(a, sym, parts, first_tile, staging);
@@ -885,7 +894,9 @@ static tc_status launch_unpack(const DecodeArgs &a, void *out, long long first_t
     const int threads = (chunks / parts + 31) / 32 * 32, least = tiles * parts < 4 * sm_count ? 256 : 32;
     // from 16 warps an SM on the shared-memory pipe is what bounds a per-layer decoder (see the kernel)
     const bool full = kOperand && a.groups == 1 && tiles * ((chunks + 31) / 32) >= 16 * (long long)sm_count;
-    const size_t spread = a.alone ? spread_bytes(tiles * parts, sm_count, full ? kUnpackFullStatic : kUnpackStatic) : 0;
+    static const size_t own[3] = {static_bytes((const void *)pick_unpack<kOperand, true>(false, false)), static_bytes((const void *)pick_unpack<kOperand, true>(false, true)),
+                                  static_bytes((const void *)pick_unpack<kOperand, true>(true, false))};
+    const size_t spread = a.alone ? spread_bytes(tiles * parts, sm_count, own[a.groups != 1 ? 2 : full]) : 0;
     void (*kernel)(DecodeArgs, void *, long long, unsigned int, unsigned int) = spread > 0 ? pick_unpack<kOperand, true>(a.groups != 1, full) : pick_unpack<kOperand, false>(a.groups != 1, full);
     if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024) != cudaSuccess) return TC_ERR_CUDA;
     const size_t rows = full ? (size_t)(threads / 32) * kRowsWarpBytes : 0;
