@@ -850,12 +850,14 @@ tc_status tc_launch_pack_symbols(const tc_ctx *ctx, const EncodeArgs &a, const u
     // first SMs that have room (960x7x7 x 128, 49 blocks: 49 us unchained, 65 chained, 48 chained and spread; 64x56x56 f32 17.2
     // unchained, 14.9 chained and spread; 400x7x7 x 800, 307 blocks, 87.8 -> 66.9; 80x27x27 x 64, 365 blocks of 256 threads, 25.2 ->
     // 22.7).  Not large blocks of which some SMs get two: the first SMs that are free take two each (576x14x14 x 128, 196 blocks of 1 024
-    // threads: 55.4 -> 57.4).
+    // threads: 55.4 -> 57.4).  Nor so many that little L1 is left, with tables per channel, which are looked up through it, from four an SM on (us in
+    // turn and early: 784x14x14, 185 blocks a pass, at 7 bits 766 and 583, 400x14x14, 299, 285 and 227; 240x1x1 x 124928, 488 blocks, at 8 bits 211 and
+    // 231, 144x1x1 x 109568, 856, 81 and 111; one table: 192x7x7, 456 blocks, 80.1 and 77.2, 208x7x7 x 2100, 804, 74.8 and 82.0).
     if (tile_blocks > 1)
         return launch_chained_cluster(tile_blocks, kernel, grid, block, std::max<size_t>(staging, kSpreadMost), s, a, sym, parts, first_tile, staging) == cudaSuccess ? TC_OK : TC_ERR_CUDA;
     const bool apart = tiles <= ctx->sm_count || tiles > 2ll * ctx->sm_count || block.x <= 512;
     static const size_t own[2] = {static_bytes((const void *)pack_symbols_kernel<true, false>), static_bytes((const void *)pack_symbols_kernel<false, false>)};
-    const size_t spread = a.alone && apart ? spread_bytes(tiles, ctx->sm_count, own[a.groups != 1]) : 0;
+    const size_t spread = a.alone && apart && tiles <= (a.groups == 1 ? 5ll : 3ll) * ctx->sm_count ? spread_bytes(tiles, ctx->sm_count, own[a.groups != 1]) : 0;
     if (spread > 0)
         return launch_chained(true, kernel, grid, block, std::max<size_t>(staging, spread), s, a, sym, parts, first_tile, staging) == cudaSuccess ? TC_OK : TC_ERR_CUDA;
     kernel<<<grid, block, staging, s>>>(a, sym, parts, first_tile, staging);
@@ -880,9 +882,11 @@ static tc_status launch_unpack(const DecodeArgs &a, void *out, long long first_t
     if (chunks > kUnpackThreads) return TC_ERR_UNSUPPORTED;
     // beside the tables (at most 48 KB and the symbols) room for a segment of three bits per symbol, at most 48 KB
     unsigned int tables = (unsigned int)(a.groups == 1 ? std::max<size_t>((size_t)4 << a.lut_bits, 16) : (size_t)a.k * kCanonWords * 4);
+    bool tables_staged = true;
     if (a.groups != 1) {
         const unsigned int sorted = (unsigned int)a.k << a.bits;                   // bytes
-        if (sorted % 16 == 0 && ((uintptr_t)a.sorted & 15u) == 0 && sorted <= kSortedStaged) tables += sorted;
+        tables_staged = sorted % 16 == 0 && ((uintptr_t)a.sorted & 15u) == 0 && sorted <= kSortedStaged;
+        if (tables_staged) tables += sorted;
     }
     const unsigned int segment = (unsigned int)std::min<long long>((long long)a.k * TC_TILE_PIXELS * 3 / 8, 48 * 1024);
     // Two or four blocks a tile of 256 chunks and more, as long as every block has an SM (320x7x7 x 180, 69 tiles in four blocks each:
@@ -896,7 +900,9 @@ static tc_status launch_unpack(const DecodeArgs &a, void *out, long long first_t
     const bool full = kOperand && a.groups == 1 && tiles * ((chunks + 31) / 32) >= 16 * (long long)sm_count;
     static const size_t own[3] = {static_bytes((const void *)pick_unpack<kOperand, true>(false, false)), static_bytes((const void *)pick_unpack<kOperand, true>(false, true)),
                                   static_bytes((const void *)pick_unpack<kOperand, true>(true, false))};
-    const size_t spread = a.alone ? spread_bytes(tiles * parts, sm_count, own[a.groups != 1 ? 2 : full]) : 0;
+    // In its turn where the symbols are looked up through L1, which spreading would take from them (us in turn and early: 240x13x13 x 183 at 8 bits 45.4
+    // and 48.8, 176x7x7 x 352 31.5 and 33.2, 848x16x16 x 526 at 5 bits 579 and 612; staged: 144x12x12 x 97 20.6 and 18.4, 512x56x56 19.6 and 18.3).
+    const size_t spread = a.alone && tables_staged ? spread_bytes(tiles * parts, sm_count, own[a.groups != 1 ? 2 : full]) : 0;
     void (*kernel)(DecodeArgs, void *, long long, unsigned int, unsigned int) = spread > 0 ? pick_unpack<kOperand, true>(a.groups != 1, full) : pick_unpack<kOperand, false>(a.groups != 1, full);
     if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024) != cudaSuccess) return TC_ERR_CUDA;
     const size_t rows = full ? (size_t)(threads / 32) * kRowsWarpBytes : 0;
