@@ -924,7 +924,7 @@ constexpr int kFourGroupsCoefs = 128;
 static Plan make_plan(const tc_ctx *ctx, const EncodeArgs &a)
 {
     const int n_blk = a.k / 16;
-    const bool plain = !a.hist && !a.dbg_coef && !a.dbg_sym;
+    const bool four_groups = a.k <= kFourGroupsCoefs && !a.hist && !a.dbg_coef && !a.dbg_sym && a.epilogue_groups != 2;
     const bool modal = a.groups == 1 && a.modal >= 0;
     auto blk_bits = [&](int b) { return modal || a.groups != 1 ? a.blk_bits[b] : std::max(a.blk_bits[b], 16.f * a.bits); };
     Plan best{};
@@ -940,7 +940,7 @@ static Plan make_plan(const tc_ctx *ctx, const EncodeArgs &a)
     while (modal && best.skip_blk > 0 && 64.f * a.blk_odd[best.skip_blk - 1] < 1.2f) --best.skip_blk;
     // blocks of the two threads of a pixel: equal work, a coded block counted as three passed over
     auto cost = [&](int b0, int b1) { return 3 * std::max(0, std::min(b1, best.skip_blk) - b0) + (b1 - std::max(b0, std::min(b1, best.skip_blk))); };
-    best.groups = plain && a.k <= kFourGroupsCoefs && !a.two_groups ? 4 : 2;
+    best.groups = four_groups ? 4 : 2;
     best.split_blk = best.groups == 4 ? n_blk : 1;
     for (int x = 2; x <= n_blk && best.groups == 2; ++x)
         if (std::max(cost(0, x), cost(x, n_blk)) < std::max(cost(0, best.split_blk), cost(best.split_blk, n_blk))) best.split_blk = x;
@@ -974,6 +974,8 @@ static Plan make_plan(const tc_ctx *ctx, const EncodeArgs &a)
     return best;
 }
 
+static bool coded_in_pairs(const EncodeArgs &a, const Plan &pl) { return a.groups == 1 && pl.entries > (1 << a.bits); }
+
 bool tc_encode_tc_supported(const tc_ctx *ctx, const EncodeArgs &a)
 {
     // K <= C leading components (PCA truncation): K is the N dimension of the MMA
@@ -1000,7 +1002,7 @@ static void (*pick_kernel(bool debug, bool hist, int groups))(EncodeArgs, Plan)
 static int kernel_class(const EncodeArgs &a, const Plan &pl)
 {
     const bool per_channel = a.groups != 1;
-    return (per_channel ? 1 : 0) | (!per_channel && pl.entries > (1 << a.bits) ? 2 : 0) | (pl.run_words[0] > 0 ? 4 : 0) | (pl.groups == 4 ? kEncodeFourGroups : 0);
+    return (per_channel ? 1 : 0) | (coded_in_pairs(a, pl) ? 2 : 0) | (pl.run_words[0] > 0 ? 4 : 0) | (pl.groups == 4 ? kEncodeFourGroups : 0);
 }
 template <int kGroups>
 static const void *list_kernel(int which)
@@ -1015,19 +1017,64 @@ static const void *list_kernel(int which)
     }
 }
 
-// of a tensor that tc_encode_tc_supported takes
-int tc_encode_tc_class(const tc_ctx *ctx, const EncodeArgs &a) { return kernel_class(a, make_plan(ctx, a)); }
+constexpr double kShortListUs = 18.0, kSharedListUs = 40.0;       // see tc_encode_tc_list_classes
 
 // us that a tile takes a block: 1.35 with 64 coefficients at 1.1 bits each, 2.0 with 128 at 1.9, 1.75 with 96 at 2.8 (four groups), 3.95
 // with 256 at 1.1, 6.9 at 4.1 (8 to 130 tiles a block, after the first)
-double tc_encode_tc_tile_us(const EncodeArgs &a)
+double tc_encode_tc_tile_us(const EncodeArgs &a, int which)
 {
     double bits = 0.0;
     for (int b = 0; b < a.k / 16; ++b) bits += a.blk_bits[b];
-    return a.k <= kFourGroupsCoefs ? 0.8 + 0.0075 * a.k + 0.0022 * bits : 0.011 * a.k + 0.004 * bits;
+    return which & kEncodeFourGroups ? 0.8 + 0.0075 * a.k + 0.0022 * bits : std::max(1.2, 0.011 * a.k) + 0.004 * bits;
 }
 
-// Encodes tensors of one class (tc_encode_tc_class) on `sms` SMs, in list_launches launches (40 of 128x14x14 x 32 in
+// Narrow tensors code faster with four groups a block, but in a short list a block gets a tile or two (fifteen small tensors
+// of 16 to 144 channels, 25 us of work), and where wider ones take a launch anyway theirs as well costs more than that
+// (47.6 -> 54.5 us in two launches; six tensors of 32 to 256 channels, 2 us of work, 17.0 -> 30; 16 layers, 100 us of work: 130.6 -> 124.3).
+void tc_encode_tc_list_classes(const tc_ctx *ctx, std::vector<EncodeArgs> &args, std::vector<int> &kind)
+{
+    double all_us = 0.0, class_us[kEncodeClasses] = {};
+    for (size_t i = 0; i < args.size(); ++i) {
+        if (kind[i] < 0) continue;
+        args[i].epilogue_groups = 4;
+        kind[i] = kernel_class(args[i], make_plan(ctx, args[i]));
+        const double us = (double)args[i].n_tiles * tc_encode_tc_tile_us(args[i], kind[i]) / ctx->sm_count;
+        class_us[kind[i]] += us;
+        all_us += us;
+    }
+    for (size_t i = 0; i < args.size(); ++i) {
+        if (kind[i] < 0 || !(kind[i] & kEncodeFourGroups)) continue;
+        args[i].epilogue_groups = 2;
+        const int two = kernel_class(args[i], make_plan(ctx, args[i]));        // (not the same one less a bit: there is more room)
+        if (all_us <= kShortListUs || (class_us[two] > 0.0 && class_us[two] + class_us[kind[i]] <= kSharedListUs)) kind[i] = two;
+        else args[i].epilogue_groups = 4;
+    }
+}
+
+// For the tests: the classes of a list of `n` tensors (1: a call with one tensor), each of `tiles` tiles and with `coef_bits` expected of each coefficient,
+// on a device of `sm_count` SMs and `smem` bytes of shared memory a block.
+extern "C" void tc_encode_classes(int n, const int *c, const int *k, const int *bits, const int *tables, const long long *tiles, const float *coef_bits, int sm_count,
+                                  int smem, int *out)
+{
+    tc_ctx ctx;
+    ctx.sm_count = sm_count;
+    ctx.max_smem_optin = smem;
+    std::vector<EncodeArgs> args(n);
+    std::vector<std::vector<float>> blk_bits(n), blk_odd(n);
+    std::vector<int> kind(n, 0);
+    for (int i = 0; i < n; ++i) {
+        EncodeArgs &a = args[i];
+        a.c = c[i]; a.k = k[i]; a.bits = bits[i]; a.groups = tables[i]; a.n_tiles = tiles[i]; a.modal = 0;
+        blk_bits[i].assign(k[i] / 16, 16.f * coef_bits[i]);
+        blk_odd[i].assign(k[i] / 16, 16.f * std::min(1.f, coef_bits[i] - 1.f));
+        a.blk_bits = blk_bits[i].data(); a.blk_odd = blk_odd[i].data();
+    }
+    if (n > 1) tc_encode_tc_list_classes(&ctx, args, kind);
+    else kind[0] = kernel_class(args[0], make_plan(&ctx, args[0]));
+    std::copy(kind.begin(), kind.end(), out);
+}
+
+// Encodes tensors of one class (tc_encode_tc_list_classes) on `sms` SMs, in list_launches launches (40 of 128x14x14 x 32 in
 // two of 20 each: 57 us, in one of 32 and one of 8: 62).
 tc_status tc_launch_encode_tc_list(const tc_ctx *ctx, const std::vector<EncodeArgs> &tensors, int sms, cudaStream_t s)
 {
@@ -1044,7 +1091,7 @@ tc_status tc_launch_encode_tc_list(const tc_ctx *ctx, const std::vector<EncodeAr
             list.item[i].pl = make_plan(ctx, a);
             which = kernel_class(a, list.item[i].pl);
             smem = std::max(smem, smem_layout(a.c, a.k, list.item[i].pl).total);
-            work[i] = {a.n_tiles, tc_encode_tc_tile_us(a), 1};
+            work[i] = {a.n_tiles, tc_encode_tc_tile_us(a, which), 1};
         }
         deal_blocks(work, sms);
         unsigned int blocks = 0;
@@ -1069,7 +1116,7 @@ tc_status tc_launch_encode_tc(const tc_ctx *ctx, const EncodeArgs &a, cudaStream
     if (a.hist && (per_channel || debug)) return TC_ERR_UNSUPPORTED;      // statistics run with a per-layer table
     Plan pl = make_plan(ctx, a);
     if (pl.staging_bytes == 0) return TC_ERR_UNSUPPORTED;
-    const bool pair = !per_channel && pl.entries > (1 << a.bits), runs = pl.run_words[0] > 0;
+    const bool pair = coded_in_pairs(a, pl), runs = pl.run_words[0] > 0;
     const SmemLayout l = smem_layout(a.c, a.k, pl);
     void (*kernel)(EncodeArgs, Plan) = per_channel ? (runs ? pick_kernel<true, false, true>(debug, false, pl.groups) : pick_kernel<true, false, false>(debug, false, pl.groups))
                                      : pair        ? (runs ? pick_kernel<false, true, true>(debug, a.hist, pl.groups) : pick_kernel<false, true, false>(debug, a.hist, pl.groups))

@@ -1347,30 +1347,21 @@ tc_status tc_encode_many(tc_ctx *ctx, const tc_encode_item *items, int32_t n_ite
     std::vector<int> kind(n_items, -1);
     std::vector<std::vector<int>> members(kEncodeClasses);
     std::vector<std::vector<ListWork>> tiles(kEncodeClasses);
-    double others_us = 0.0, others = 0.0, class_us[kEncodeClasses] = {};
+    double others_us = 0.0, others = 0.0;
     std::vector<int> order;
     for (int i = 0; i < n_items; ++i) {
         const tc_encode_item &it = items[i];
         if (work[i] == 0.0) continue;
         args[i] = encode_args(ctx, it.model, it.codebook, it.x, shape[i].cp, shape[i].splits, it.stream_out, it.capacity, it.chunk_len,
                               it.tile_off, nullptr, nullptr, nullptr, nullptr, 0);
-        if (!resident_encode(ctx, it.x, args[i])) continue;
-        kind[i] = tc_encode_tc_class(ctx, args[i]);
-        class_us[kind[i]] += (double)args[i].n_tiles * tc_encode_tc_tile_us(args[i]) / ctx->sm_count;
+        if (resident_encode(ctx, it.x, args[i])) kind[i] = 0;
     }
-    // Narrow tensors code faster with four groups a block, but a launch more costs a short list more than that (fifteen small tensors
-    // of 16 to 144 channels, 25 us of work: 47.6 -> 54.5 us in two launches; 16 layers, 100 us of work: 130.6 -> 124.3).
-    for (int i = 0; i < n_items; ++i) {
-        const int two = kind[i] & ~kEncodeFourGroups;
-        if (kind[i] < 0 || two == kind[i] || class_us[two] == 0.0 || class_us[two] + class_us[kind[i]] > 40.0) continue;
-        args[i].two_groups = true;
-        kind[i] = tc_encode_tc_class(ctx, args[i]);
-    }
+    tc_encode_tc_list_classes(ctx, args, kind);
     for (int i : by_descending_work(n_items, work)) {
         const tc_encode_item &it = items[i];
         if (kind[i] >= 0) {
             members[kind[i]].push_back(i);
-            tiles[kind[i]].push_back({args[i].n_tiles, tc_encode_tc_tile_us(args[i]), 0});
+            tiles[kind[i]].push_back({args[i].n_tiles, tc_encode_tc_tile_us(args[i], kind[i]), 0});
         } else {
             order.push_back(i);
             others += work[i];

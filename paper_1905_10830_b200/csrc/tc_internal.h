@@ -128,7 +128,7 @@ struct EncodeArgs {
     unsigned long long *tile_state;   // look-back state, zeroed before launch
     unsigned int *ticket;             // zeroed before launch; the look-back words follow it
     bool alone;                       // no other stream of this call (see launch_chained)
-    bool two_groups;                  // resident-basis encoder: share a launch with wider tensors
+    int epilogue_groups;              // resident-basis encoder: 2 or 4 a block, as a list has it; 0: four where they fit
     int sms;                          // SMs that a persistent kernel of its own takes at most in a list
     long long clear_words;            // 64-bit words from `ticket` on that the first of several kernels zeroes (0: they are zero)
     unsigned long long *other_state;  // resident-basis encoder: look-back state that no tile of this call uses,
@@ -297,9 +297,10 @@ bool tc_tensor_map_sw128(CUtensorMap *map, const void *base, long long rows, int
 tc_status tc_launch_reconstruct(const DecodeArgs &a, int dtype, const uint8_t *sym, cudaStream_t s);
 bool tc_encode_tc_supported(const tc_ctx *ctx, const EncodeArgs &a);
 tc_status tc_launch_encode_tc(const tc_ctx *ctx, const EncodeArgs &a, cudaStream_t s);
-int tc_encode_tc_class(const tc_ctx *ctx, const EncodeArgs &a);
+// Kernels of a list's tensors, those with kind[i] >= 0 on entry, which tc_encode_tc_supported takes.
+void tc_encode_tc_list_classes(const tc_ctx *ctx, std::vector<EncodeArgs> &args, std::vector<int> &kind);
 constexpr int kEncodeClasses = 16, kEncodeFourGroups = 8;     // classes; the bit of those with four epilogue groups a block
-double tc_encode_tc_tile_us(const EncodeArgs &a);
+double tc_encode_tc_tile_us(const EncodeArgs &a, int which);
 tc_status tc_launch_encode_tc_list(const tc_ctx *ctx, const std::vector<EncodeArgs> &tensors, int sms, cudaStream_t s);
 bool tc_decode_tc_supported(const tc_ctx *ctx, const DecodeArgs &a);
 tc_status tc_launch_decode_tc(const tc_ctx *ctx, const DecodeArgs &a, cudaStream_t s);

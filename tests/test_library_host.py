@@ -112,3 +112,28 @@ def test_nothing_is_issued_after_a_wait_that_ran_out(lib, groups, tiles, panels,
         tl, i = divmod(fails - 1, 1 + panels)                  # wait i of a tile: its accumulator, then its panels
         issued = want[:tl * (panels + 1) + max(0, i - 1)]
         assert events(fails) == issued + [-1, 300]
+
+
+@pytest.fixture(scope="module")
+def encode_classes(lib):
+    """Kernel classes of tensors (c, k, bits, tables, tiles, bits per coefficient) of a list, or of a call with one: bit 0 a table per channel, bit 1 symbol
+    pairs, bit 2 private runs, bit 3 four epilogue groups a block."""
+    import ctypes as C
+
+    def run(*tensors):
+        n, out = len(tensors), (C.c_int * len(tensors))()
+        ints = [(C.c_int * n)(*[t[j] for t in tensors]) for j in range(4)]
+        lib.tc_encode_classes(n, *ints, (C.c_longlong * n)(*[t[4] for t in tensors]), (C.c_float * n)(*[t[5] for t in tensors]), 148, 227 * 1024, out)
+        return list(out)
+    return run
+
+
+# Lists: short ones in one launch; longer ones, where wide tensors take a launch anyway, in theirs -- the class with two groups being that of the plan with two
+# groups, which has room for private runs where four leave none -- and long ones with four groups for narrow tensors.
+def test_epilogue_groups_of_lists(encode_classes):
+    assert encode_classes((32, 32, 4, 1, 17, 1.3), (256, 256, 4, 1, 55, 1.3), (64, 64, 4, 1, 50, 1.3)) == [6, 6, 6]
+    narrow, wide = (240, 128, 6, 1, 500, 4.5), (256, 256, 4, 1, 700, 1.3)
+    assert encode_classes((*narrow[:4], 5000, 4.5)) == [10]
+    assert encode_classes(narrow, wide) == [6, 6]
+    assert encode_classes((128, 128, 4, 1, 1500, 1.3), (64, 64, 4, 1, 500, 1.3)) == [14, 14]
+    assert encode_classes((128, 128, 4, 1, 5000, 1.3), (256, 256, 4, 1, 3000, 1.3)) == [14, 6]
