@@ -910,8 +910,12 @@ extern "C" int tc_issue_events(int groups, long long tiles, int panels, int stag
     return n;
 }
 
-// Coefficients up to which four accumulators fit tensor memory and a thread codes a pixel.
-constexpr int kFourGroupsCoefs = 128;
+// Four groups: up to as many coefficients as let their accumulators fit tensor memory, and where a block has more tiles than these (less one up
+// to 64 coefficients), since few tiles are coded sooner by eight warps each than by four (us with two and with four groups, a tile a block:
+// 128x16x16 at 96 coefficients 10.6 and 12.4, 80x28x28 x 3 10.4 and 12.4; two: 128x16x16 x 124 16.5 and 18.2; four: 240x14x14 x 300 at 128
+// 23.2 and 24.9; five: 128x14x14 x 432 23.2 and 21.4).  Also where their buffers leave no room for private runs, which two would have:
+// dense codes of 128 coefficients of wide layers (256x14x14 x 1500 at 6 bits 73.4 and 74.0, at 8 bits 80.0 and 77.3, 240x14x14 x 1500 at 5 bits 72.6 and 69.1).
+constexpr int kFourGroupsCoefs = 128, kTwoGroupsTiles = 4;
 
 // What a launch does with the shared memory that the basis leaves, from the code lengths to expect of
 // the model's coefficients (a code without a one-bit symbol: b bits for each).  A tile's size varies
@@ -924,7 +928,8 @@ constexpr int kFourGroupsCoefs = 128;
 static Plan make_plan(const tc_ctx *ctx, const EncodeArgs &a)
 {
     const int n_blk = a.k / 16;
-    const bool four_groups = a.k <= kFourGroupsCoefs && !a.hist && !a.dbg_coef && !a.dbg_sym && a.epilogue_groups != 2;
+    const bool few = a.n_tiles <= (long long)(a.k > 64 ? kTwoGroupsTiles : kTwoGroupsTiles - 1) * ctx->sm_count;
+    const bool four_groups = a.k <= kFourGroupsCoefs && !a.hist && !a.dbg_coef && !a.dbg_sym && (a.epilogue_groups ? a.epilogue_groups == 4 : !few);
     const bool modal = a.groups == 1 && a.modal >= 0;
     auto blk_bits = [&](int b) { return modal || a.groups != 1 ? a.blk_bits[b] : std::max(a.blk_bits[b], 16.f * a.bits); };
     Plan best{};

@@ -128,7 +128,7 @@ struct EncodeArgs {
     unsigned long long *tile_state;   // look-back state, zeroed before launch
     unsigned int *ticket;             // zeroed before launch; the look-back words follow it
     bool alone;                       // no other stream of this call (see launch_chained)
-    int epilogue_groups;              // resident-basis encoder: 2 or 4 a block, as a list has it; 0: four where they fit
+    int epilogue_groups;              // resident-basis encoder: 2 or 4 a block, as a list has it; 0: by the tensor's tiles
     int sms;                          // SMs that a persistent kernel of its own takes at most in a list
     long long clear_words;            // 64-bit words from `ticket` on that the first of several kernels zeroes (0: they are zero)
     unsigned long long *other_state;  // resident-basis encoder: look-back state that no tile of this call uses,

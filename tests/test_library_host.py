@@ -128,6 +128,12 @@ def encode_classes(lib):
     return run
 
 
+# Four epilogue groups where a block has several tiles, two where it has few and above 128 coefficients.
+@pytest.mark.parametrize("k,tiles,four", [(64, 1, 0), (64, 3 * 148, 0), (64, 3 * 148 + 1, 1), (128, 4 * 148, 0), (128, 4 * 148 + 1, 1), (16, 10 ** 7, 1), (144, 10 ** 7, 0)])
+def test_epilogue_groups_by_tiles(encode_classes, k, tiles, four):
+    assert encode_classes((max(k, 160), k, 4, 1, tiles, 1.3)) == [6 + 8 * four]
+
+
 # Lists: short ones in one launch; longer ones, where wide tensors take a launch anyway, in theirs -- the class with two groups being that of the plan with two
 # groups, which has room for private runs where four leave none -- and long ones with four groups for narrow tensors.
 def test_epilogue_groups_of_lists(encode_classes):
