@@ -451,6 +451,8 @@ int tc_last_path(const tc_ctx *ctx, int decode)
     if (!ctx) return -1;
     return decode ? ctx->last_decode_path : ctx->last_encode_path;
 }
+// For the tests: whether it was the run-skipping decoder that the last call of path 1 took, and not those that take over where it does not run.
+extern "C" int tc_last_decode_skipped_runs(const tc_ctx *ctx) { return ctx->last_decode_path == 1 && ctx->last_decode_runs; }
 
 tc_status tc_get_status(tc_ctx *ctx, void *cuda_stream)
 {
@@ -1166,6 +1168,7 @@ static tc_status decode_with_scratch(tc_ctx *ctx, const tc_model *m, const tc_co
     const DecodeArgs a = decode_args(ctx, m, cb, stream, stream_bytes, chunk_len, tile_off, params, cs, x_hat, list_sms);
     if (runs_decode(ctx, x_hat, a)) {                   // (it also takes dense tiles; in lists these share launches)
         ctx->last_decode_path = 1;
+        ctx->last_decode_runs = true;
         return tc_launch_decode_runs(ctx, a, (cudaStream_t)cuda_stream);
     }
     bool resident = (ctx->force_exact == 0 || ctx->force_exact == 3) && x_hat->dtype == TC_BF16 && tc_decode_tc_supported(ctx, a);
@@ -1180,6 +1183,7 @@ static tc_status decode_with_scratch(tc_ctx *ctx, const tc_model *m, const tc_co
         resident = false;
     if (resident) {
         ctx->last_decode_path = 1;
+        ctx->last_decode_runs = false;
         if (product) return tc_launch_decode_wide_gemm(ctx, a, sym_scratch, (cudaStream_t)cuda_stream);
         return tc_launch_decode_tc(ctx, a, (cudaStream_t)cuda_stream);
     }
@@ -1461,7 +1465,7 @@ tc_status tc_decode_many(tc_ctx *ctx, const tc_decode_item *items, int32_t n_ite
     tc_status first_error = launch_shared(ctx, classes, sms, s, n_streams, streams.used, [&](const std::vector<DecodeArgs> &c, int mine, cudaStream_t on) {
         return tc_launch_decode_runs_list(ctx, c, mine, on);
     });
-    if (n_classes) ctx->last_decode_path = 1;
+    if (n_classes) { ctx->last_decode_path = 1; ctx->last_decode_runs = true; }
     for (size_t r = 0; r < order.size(); ++r) {
         const int i = order[r];
         const tc_decode_item &it = items[i];

@@ -53,6 +53,7 @@ struct tc_ctx {
     bool force_jacobi = false;            // the eigensolver for devices that cannot hold the clusters
     int last_encode_path = 0;             // 0 = fp64 kernels, 1 = tensor-core kernels (resident basis), 2 = fp32 kernels, 3 = tensor-core kernels (streamed basis)
     int last_decode_path = 0;
+    bool last_decode_runs = false;        // path 1 by the run-skipping decoder
     tc_codebook *stats_cb[9] = {};        // tc_stats: fixed-length code tables (one per bit width) for streams coded without a codebook
 };
 
@@ -183,8 +184,8 @@ struct DecodeArgs {
 };
 
 // ---- encode dispatch shared by tc_encode and tc_encode_noalloc (tc_api.cu) --------------------
-// Launch of a kernel that may be set up while the one before it in the stream still runs (it calls chain_wait).  Only for
-// the second and later kernels of one call: its first one starts after everything that the stream held before.  Not with
+// Launch of a kernel that may be set up while the one before it in the stream still runs (`early`; it calls chain_wait): as it is for the second and
+// later kernels of a call, behind kernels of this library, and by launch_first for a call's first kernel, behind anyone's.  Not with
 // other streams of the call at work (`early` false): a product's blocks that wait hold shared memory their kernels could
 // use (decode of a network's 16 layers 274 us, 250 without).
 template <typename... P, typename... A>

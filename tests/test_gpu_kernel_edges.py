@@ -1,4 +1,6 @@
 """Kernel branches that the parity cases do not separate, each at the sizes where it can go wrong."""
+import ctypes
+
 import numpy as np
 import pytest
 import torch
@@ -323,6 +325,30 @@ def test_rows_of_the_run_skipping_decoder(ctx, c, h, w, n):
     tc.tc_force_exact_path(ctx, 0)
     a, b = got.float(), want.float()
     assert bool(((a - b).abs() <= 2.0 ** -7 * b.abs() + 1e-6 * float(b.abs().max())).all())
+    m.close(); cb.close()
+
+
+# The run-skipping decoder is what runs on this build: kernels that come out with too few registers for its roles, or buffers that do not fit, leave
+# the tensor to decoders that report the same path and are several times slower.
+@pytest.mark.parametrize("c,h,w,n,bits,k,cp,splits", [(16, 1, 1, 1, 2, 0, 0, 0), (64, 56, 56, 4, 4, 0, 0, 0), (128, 14, 14, 9, 8, 0, 0, 0), (176, 7, 7, 40, 5, 0, 0, 0), (256, 14, 14, 9, 4, 0, 0, 0),
+                                                      (256, 14, 14, 9, 8, 0, 0, 0), (256, 9, 7, 30, 8, 0, 0, 0), (256, 3, 1, 500, 6, 0, 0, 0), (240, 14, 14, 5, 6, 48, 0, 0), (256, 14, 14, 4, 4, 0, 1, 4),
+                                                      (128, 14, 14, 4, 5, 0, 16, 1)])
+def test_the_run_skipping_decoder_runs(ctx, c, h, w, n, bits, k, cp, splits):
+    params = fm.layer_params(fm.LayerSpec(c, h, w, 0.9, None, 24000 + c))
+    cal = fm.make_maps(params, max(4, 30000 // (h * w)), calib=True, dtype=torch.bfloat16, device="cuda")
+    x = fm.make_maps(params, n, dtype=torch.bfloat16, device="cuda")
+    m = tc.tc_fit_pca(ctx, cal, bits, k=k)
+    cb = tc.tc_build_codebook(ctx, m, tc.tc_stats(ctx, m, None, cal).hist)
+    enc = tc.tc_encode(ctx, m, cb, x, chunk_pixels=cp, pixel_splits=splits)
+    runs = tc.load_library().tc_last_decode_skipped_runs
+    runs.argtypes = [ctypes.c_void_p]
+    for switch, want in ((0, 1), (3, 0), (0, 1)):
+        tc.tc_force_exact_path(ctx, switch)
+        for relu in (False, True):
+            tc.tc_decode(ctx, m, cb, enc, x.shape, x.dtype, relu=relu)
+            assert tc.tc_get_status(ctx) == 0 and runs(ctx.ptr) == want and (not want or tc.tc_last_path(ctx, True) == 1)
+    tc.tc_decode_many(ctx, [(m, cb, enc, x.shape, x.dtype)] * 2)
+    assert tc.tc_get_status(ctx) == 0 and tc.tc_last_path(ctx, True) == 1 and runs(ctx.ptr) == 1
     m.close(); cb.close()
 
 
