@@ -31,7 +31,7 @@
 // panel, and a VLD thread of the group's next tile waits only for the panels that it writes.
 //
 // What bounds it is the VLD groups' instructions and their chains (256x14x14 x 4096 at 4 bits: 139 us with the products and the stores
-// left out, 163 in all; 218 before the items, stores and registers took their present form).  Every warp takes its turn at the issue
+// left out, 160 in all; 219 before the items, stores and registers took their present form).  Every warp takes its turn at the issue
 // slots, an instruction in about twelve cycles, so that the MMA warp's loop is unrolled; and what does not fit the registers goes to local
 // memory and comes back from L2 (shared memory leaves the L1 no room): hence the split of the registers below.
 //
@@ -505,8 +505,8 @@ __device__ __forceinline__ void decode_tiles(const DecodeArgs &a, const SmemLayo
 
                 // Walks this thread's chunks.  Control flow is kept uniform across the warp: the lanes
                 // of a warp step together (a lane that has finished its chunk idles until all have),
-                // panels are waited for and filled by all lanes at once when any lane needs the next
-                // one, and a wait that runs out is seen by every lane -- lanes that wander off on
+                // the panels of a chunk are waited for and filled by all lanes at once, before its first
+                // symbol, and a wait that runs out is seen by every lane -- lanes that wander off on
                 // their own would run the rest of the tile one after the other.
                 auto decode_tile = [&](auto &r) {
                     uint32_t expect = 0;               // bits the chunks decoded so far should have taken

@@ -31,10 +31,12 @@ __device__ __forceinline__ unsigned long long global_timer_ns()
     return t;
 }
 
-// Kernels of one call that follow each other (launch_chained): a kernel lets the next one start setting up as soon
-// as all its own blocks run, and waits for what the one before it wrote -- and everything before that -- ahead of the
-// first access to it.  The last kernel of a call does so after its own wait: with the kernels of four calls' halves set up behind one
-// another a round trip of 256x14x14 f32 took 48 us instead of 43.  What it reads from the kernel before it does not go through the read-only path.
+// Kernels that follow each other (launch_chained, launch_first): a kernel lets the next one start setting up once all its own blocks run
+// (chain_next), and every thread that touches what others wrote or read waits for the kernel before it, and so for everything before that, ahead of the
+// first access to it (chain_wait).  What it reads of theirs does not go through the read-only path.
+// chain_next is a kernel's first act, also of the persistent decoder, encoder and tiled product where they end a call: whoever starts then waits in
+// its turn.  Only the exact inverse and the entropy coder of stored symbols, which end a call, do so behind their wait: with the kernels of four calls'
+// halves set up behind one another a round trip of 256x14x14 f32 took 48 us instead of 43.
 __device__ __forceinline__ void chain_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 

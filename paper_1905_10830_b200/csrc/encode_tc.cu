@@ -1035,7 +1035,7 @@ double tc_encode_tc_tile_us(const EncodeArgs &a, int which)
 
 // Narrow tensors code faster with four groups a block, but in a short list a block gets a tile or two (fifteen small tensors
 // of 16 to 144 channels, 25 us of work), and where wider ones take a launch anyway theirs as well costs more than that
-// (47.6 -> 54.5 us in two launches; six tensors of 32 to 256 channels, 2 us of work, 17.0 -> 30; 16 layers, 100 us of work: 130.6 -> 124.3).
+// (47.6 -> 54.5 us in two launches; eleven of 16 to 144, 8 us of work, 25.4 -> 38.8; 16 layers, 100 us of work: 130.6 -> 124.3).
 void tc_encode_tc_list_classes(const tc_ctx *ctx, std::vector<EncodeArgs> &args, std::vector<int> &kind)
 {
     double all_us = 0.0, class_us[kEncodeClasses] = {};
