@@ -806,10 +806,10 @@ tc_status tc_launch_reconstruct(const DecodeArgs &a, int dtype, const uint8_t *s
     // Its blocks are there before the entropy decoder's are done, whose shared memory keeps them off the SMs with one, and pile onto others: kept apart where
     // an SM gets several (f32, us without and with: 256x8x16 x 10 47.0 and 31.6, 128x8x16 x 20 27.7 and 20.0, 64x8x16 x 36 18.1 and 15.1; fewer or
     // lighter ones lose by it, 32x8x16 x 17 13.4 and 14.2, 64x8x16 x 26 13.3 and 13.9; so do those that would fill all places, of which the decoder's blocks still have
-    // some, 337x8x16 x 13, 3.9 blocks an SM, 111 and 117, 480x8x16 x 9, 3.65, 84.4 and 77.5; more than four are even).
+    // some, 337x8x16 x 13, 7.7 blocks an SM, 111 and 117, 480x8x16 x 9, 7.3, 84.4 and 77.5; more than eight are even).
     const long long blocks = (long long)grid.x * grid.y;
     static const size_t own[2] = {static_bytes((const void *)reconstruct_kernel<float>), static_bytes((const void *)reconstruct_kernel<__nv_bfloat16>)};
-    const size_t spread = a.alone && blocks > (a.k >= 128 ? 2 : 3) * (long long)a.sms && 4 * blocks <= 15ll * a.sms ? spread_bytes(blocks, a.sms, own[dtype != TC_F32]) : 0;
+    const size_t spread = a.alone && blocks > (a.k >= 128 ? 2 : 3) * (long long)a.sms && 2 * blocks <= 15ll * a.sms ? spread_bytes(blocks, a.sms, own[dtype != TC_F32]) : 0;
     return launch_chained(a.alone, kernel, grid, block, spread, s, a, sym) == cudaSuccess ? TC_OK : TC_ERR_CUDA;
 }
 
