@@ -772,14 +772,6 @@ __global__ void __launch_bounds__(kUnpackThreads) unpack_symbols_kernel(DecodeAr
 
 }  // namespace
 
-// Static shared memory of a kernel that is kept apart, asked for once: a byte or two of another variant's let one block more onto an SM.
-static size_t static_bytes(const void *kernel)
-{
-    cudaFuncAttributes at;
-    if (cudaFuncGetAttributes(&at, kernel) == cudaSuccess) return at.sharedSizeBytes;
-    cudaGetLastError();
-    return 0;
-}
 // For the tests.
 extern "C" size_t tc_spread_bytes(long long blocks, int sm_count, size_t own) { return spread_bytes(blocks, sm_count, own); }
 
