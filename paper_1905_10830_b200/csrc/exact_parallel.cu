@@ -895,14 +895,16 @@ static tc_status launch_unpack(const DecodeArgs &a, void *out, long long first_t
                                   static_bytes((const void *)pick_unpack<kOperand, true>(true, false))};
     // In its turn where the symbols are looked up through L1, which spreading would take from them (us in turn and early: 240x13x13 x 183 at 8 bits 45.4
     // and 48.8, 176x7x7 x 352 31.5 and 33.2, 848x16x16 x 526 at 5 bits 579 and 612; staged: 144x12x12 x 97 20.6 and 18.4, 512x56x56 19.6 and 18.3).
-    const size_t spread = a.alone && tables_staged ? spread_bytes(tiles * parts, sm_count, own[a.groups != 1 ? 2 : full]) : 0;
+    // And with long chunks of codes per channel (768x1x1 x 3072 in chunks of 3072 220 and 230, 192x28x28 of 6144 377 and 401).
+    const bool long_chunks = a.k / a.splits * a.chunk_pixels > 512;
+    const size_t spread = a.alone && tables_staged && (a.groups == 1 || !long_chunks) ? spread_bytes(tiles * parts, sm_count, own[a.groups != 1 ? 2 : full]) : 0;
     // In its turn as well where an operand's segments are expected not to fit their buffer and are read through L1, of which a product ahead leaves
     // little to blocks that start under it, and that takes longer than the launch saves: long chunks, or several blocks an SM (us in turn and early:
     // 384x14x14 x 651 at 7.5 bits a value 206 and 259, 944x34x5 x 44 at 7.3 bits, chunks of 944 symbols, 102.6 and 107.6; 704x28x28 at 4.4 bits, chunks of 176,
     // 26.8 and 23.1, 400x14x14 x 10 at 3.9 bits, chunks of 400, 39.1 and 36.1).
     const double tile_bytes = a.mean_tile_bytes > 0 ? (double)a.mean_tile_bytes : (double)a.code_bits * a.k * TC_TILE_PIXELS / 8;
     const bool through_l1 = kOperand && a.groups == 1 && tile_bytes > 1.05 * segment;
-    const bool early = spread > 0 && !(through_l1 && (tiles * parts > sm_count || a.k / a.splits * a.chunk_pixels > 512));
+    const bool early = spread > 0 && !(through_l1 && (tiles * parts > sm_count || long_chunks));
     void (*kernel)(DecodeArgs, void *, long long, unsigned int, unsigned int) = spread > 0 ? pick_unpack<kOperand, true>(a.groups != 1, full) : pick_unpack<kOperand, false>(a.groups != 1, full);
     if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024) != cudaSuccess) return TC_ERR_CUDA;
     const size_t rows = full ? (size_t)(threads / 32) * kRowsWarpBytes : 0;
