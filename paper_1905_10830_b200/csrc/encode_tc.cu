@@ -910,12 +910,14 @@ extern "C" int tc_issue_events(int groups, long long tiles, int panels, int stag
     return n;
 }
 
-// Four groups: up to as many coefficients as let their accumulators fit tensor memory, and where a block has more tiles than these (less one up
-// to 64 coefficients), since few tiles are coded sooner by eight warps each than by four (us with two and with four groups, a tile a block:
-// 128x16x16 at 96 coefficients 10.6 and 12.4, 80x28x28 x 3 10.4 and 12.4; two: 128x16x16 x 124 16.5 and 18.2; four: 240x14x14 x 300 at 128
-// 23.2 and 24.9; five: 128x14x14 x 432 23.2 and 21.4).  Also where their buffers leave no room for private runs, which two would have:
-// dense codes of 128 coefficients of wide layers (256x14x14 x 1500 at 6 bits 73.4 and 74.0, at 8 bits 80.0 and 77.3, 240x14x14 x 1500 at 5 bits 72.6 and 69.1).
-constexpr int kFourGroupsCoefs = 128, kTwoGroupsTiles = 4;
+// Four groups: up to as many coefficients as let their accumulators fit tensor memory, and where a block has more tiles than two, one below 64
+// coefficients, since few tiles are coded sooner by eight warps each than by four; 16 coefficients are not split between warps and take four always
+// (us with two and with four groups, a tile a block: 128x16x16 at 96 coefficients 10.6 and 12.4, 80x28x28 x 3 10.4 and 12.4, 96x7x8 x 6 at 16 10.3 and 9.3;
+// two: 128x16x16 x 124 16.5 and 18.2; three: 16x12x7 x 528 12.3 and 11.8; five: 128x14x14 x 432 23.2 and 21.4.  Four's time over two's, 300 drawn
+// layers: 80 coefficients and more 1.06, 1.05, 0.98 at one, two and three tiles; 64 1.04, 1.01, 1.01; 32 and 48 1.01, 0.99, 0.98; 16 0.99, 0.97, 0.97).
+// Also where their buffers leave no room for private runs, which two would have: dense codes of 128 coefficients of wide layers (256x14x14 x 1500 at
+// 6 bits 73.4 and 74.0, at 8 bits 80.0 and 77.3, 240x14x14 x 1500 at 5 bits 72.6 and 69.1; four tiles a block 240x14x14 x 300 23.2 and 24.9).
+constexpr int kFourGroupsCoefs = 128;
 
 // What a launch does with the shared memory that the basis leaves, from the code lengths to expect of
 // the model's coefficients (a code without a one-bit symbol: b bits for each).  A tile's size varies
@@ -928,7 +930,7 @@ constexpr int kFourGroupsCoefs = 128, kTwoGroupsTiles = 4;
 static Plan make_plan(const tc_ctx *ctx, const EncodeArgs &a)
 {
     const int n_blk = a.k / 16;
-    const bool few = a.n_tiles <= (long long)(a.k > 64 ? kTwoGroupsTiles : kTwoGroupsTiles - 1) * ctx->sm_count;
+    const bool few = a.n_tiles <= (long long)std::min(2, a.k / 32) * ctx->sm_count;
     const bool four_groups = a.k <= kFourGroupsCoefs && !a.hist && !a.dbg_coef && !a.dbg_sym && (a.epilogue_groups ? a.epilogue_groups == 4 : !few);
     const bool modal = a.groups == 1 && a.modal >= 0;
     auto blk_bits = [&](int b) { return modal || a.groups != 1 ? a.blk_bits[b] : std::max(a.blk_bits[b], 16.f * a.bits); };

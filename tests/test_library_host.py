@@ -129,7 +129,7 @@ def encode_classes(lib):
 
 
 # Four epilogue groups where a block has several tiles, two where it has few and above 128 coefficients.
-@pytest.mark.parametrize("k,tiles,four", [(64, 1, 0), (64, 3 * 148, 0), (64, 3 * 148 + 1, 1), (128, 4 * 148, 0), (128, 4 * 148 + 1, 1), (16, 10 ** 7, 1), (144, 10 ** 7, 0)])
+@pytest.mark.parametrize("k,tiles,four", [(16, 1, 1), (32, 1, 0), (48, 148, 0), (48, 149, 1), (64, 2 * 148, 0), (64, 2 * 148 + 1, 1), (128, 2 * 148, 0), (128, 2 * 148 + 1, 1), (16, 10 ** 7, 1), (144, 10 ** 7, 0)])
 def test_epilogue_groups_by_tiles(encode_classes, k, tiles, four):
     assert encode_classes((max(k, 160), k, 4, 1, tiles, 1.3)) == [6 + 8 * four]
 
