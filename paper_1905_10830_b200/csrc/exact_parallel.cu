@@ -784,8 +784,8 @@ tc_status tc_launch_project_quantise(const EncodeArgs &a, int dtype, uint8_t *sy
     // Early where that leaves the basis in L1: with several blocks an SM kept apart by shared memory wide layers lose (512x14x14 f32, 224
     // blocks, 39.0 -> 43.6 us, 176x34x33 22.6 -> 24.3; 32x56x56 10.2 -> 8.3, 96x45x45 15.8 -> 15.3, 256x7x7 20.5 -> 18.8).
     const long long blocks = (long long)grid.x * grid.y;
-    static const size_t own[2] = {static_bytes((const void *)project_quantise_kernel<float>), static_bytes((const void *)project_quantise_kernel<__nv_bfloat16>)};
-    const size_t spread = a.alone && (blocks <= a.sms || a.c <= 128) ? spread_bytes(blocks, a.sms, own[dtype != TC_F32]) : 0;
+    static std::atomic<size_t> own[2];
+    const size_t spread = a.alone && (blocks <= a.sms || a.c <= 128) ? spread_bytes(blocks, a.sms, static_bytes(own[dtype != TC_F32], (const void *)kernel)) : 0;
     return launch_first(spread > 0, kernel, grid, block, spread, s, a, sym) == cudaSuccess ? TC_OK : TC_ERR_CUDA;
 }
 
@@ -800,8 +800,8 @@ tc_status tc_launch_reconstruct(const DecodeArgs &a, int dtype, const uint8_t *s
     // lighter ones lose by it, 32x8x16 x 17 13.4 and 14.2, 64x8x16 x 26 13.3 and 13.9; so do those that would fill all places, of which the decoder's blocks still have
     // some, 337x8x16 x 13, 7.7 blocks an SM, 111 and 117, 480x8x16 x 9, 7.3, 84.4 and 77.5; more than eight are even).
     const long long blocks = (long long)grid.x * grid.y;
-    static const size_t own[2] = {static_bytes((const void *)reconstruct_kernel<float>), static_bytes((const void *)reconstruct_kernel<__nv_bfloat16>)};
-    const size_t spread = a.alone && blocks > (a.k >= 128 ? 2 : 3) * (long long)a.sms && 2 * blocks <= 15ll * a.sms ? spread_bytes(blocks, a.sms, own[dtype != TC_F32]) : 0;
+    static std::atomic<size_t> own[2];
+    const size_t spread = a.alone && blocks > (a.k >= 128 ? 2 : 3) * (long long)a.sms && 2 * blocks <= 15ll * a.sms ? spread_bytes(blocks, a.sms, static_bytes(own[dtype != TC_F32], (const void *)kernel)) : 0;
     return launch_chained(a.alone, kernel, grid, block, spread, s, a, sym) == cudaSuccess ? TC_OK : TC_ERR_CUDA;
 }
 
@@ -849,8 +849,8 @@ tc_status tc_launch_pack_symbols(const tc_ctx *ctx, const EncodeArgs &a, const u
     if (tile_blocks > 1)
         return launch_chained_cluster(tile_blocks, kernel, grid, block, std::max<size_t>(staging, kSpreadMost), s, a, sym, parts, first_tile, staging) == cudaSuccess ? TC_OK : TC_ERR_CUDA;
     const bool apart = tiles <= ctx->sm_count || tiles > 2ll * ctx->sm_count || block.x <= 512;
-    static const size_t own[2] = {static_bytes((const void *)pack_symbols_kernel<true, false>), static_bytes((const void *)pack_symbols_kernel<false, false>)};
-    const size_t spread = a.alone && apart && tiles <= (a.groups == 1 ? 5ll : 3ll) * ctx->sm_count ? spread_bytes(tiles, ctx->sm_count, own[a.groups != 1]) : 0;
+    static std::atomic<size_t> own[2];
+    const size_t spread = a.alone && apart && tiles <= (a.groups == 1 ? 5ll : 3ll) * ctx->sm_count ? spread_bytes(tiles, ctx->sm_count, static_bytes(own[a.groups != 1], (const void *)kernel)) : 0;
     if (spread > 0)
         return launch_chained(true, kernel, grid, block, std::max<size_t>(staging, spread), s, a, sym, parts, first_tile, staging) == cudaSuccess ? TC_OK : TC_ERR_CUDA;
     kernel<<<grid, block, staging, s>>>(a, sym, parts, first_tile, staging);
@@ -891,13 +891,13 @@ static tc_status launch_unpack(const DecodeArgs &a, void *out, long long first_t
     const int threads = (chunks / parts + 31) / 32 * 32, least = tiles * parts < 4 * sm_count ? 256 : 32;
     // from 16 warps an SM on the shared-memory pipe is what bounds a per-layer decoder (see the kernel)
     const bool full = kOperand && a.groups == 1 && tiles * ((chunks + 31) / 32) >= 16 * (long long)sm_count;
-    static const size_t own[3] = {static_bytes((const void *)pick_unpack<kOperand, true>(false, false)), static_bytes((const void *)pick_unpack<kOperand, true>(false, true)),
-                                  static_bytes((const void *)pick_unpack<kOperand, true>(true, false))};
+    static std::atomic<size_t> own[3];
+    auto own_bytes = [&] { return static_bytes(own[a.groups != 1 ? 2 : full], (const void *)pick_unpack<kOperand, true>(a.groups != 1, full)); };
     // In its turn where the symbols are looked up through L1, which spreading would take from them (us in turn and early: 240x13x13 x 183 at 8 bits 45.4
     // and 48.8, 176x7x7 x 352 31.5 and 33.2, 848x16x16 x 526 at 5 bits 579 and 612; staged: 144x12x12 x 97 20.6 and 18.4, 512x56x56 19.6 and 18.3).
     // And with long chunks of codes per channel (768x1x1 x 3072 in chunks of 3072 220 and 230, 192x28x28 of 6144 377 and 401).
     const bool long_chunks = a.k / a.splits * a.chunk_pixels > 512;
-    const size_t spread = a.alone && tables_staged && (a.groups == 1 || !long_chunks) ? spread_bytes(tiles * parts, sm_count, own[a.groups != 1 ? 2 : full]) : 0;
+    const size_t spread = a.alone && tables_staged && (a.groups == 1 || !long_chunks) ? spread_bytes(tiles * parts, sm_count, own_bytes()) : 0;
     // In its turn as well where an operand's segments are expected not to fit their buffer and are read through L1, of which a product ahead leaves
     // little to blocks that start under it, and that takes longer than the launch saves: long chunks, or several blocks an SM (us in turn and early:
     // 384x14x14 x 651 at 7.5 bits a value 206 and 259, 944x34x5 x 44 at 7.3 bits, chunks of 944 symbols, 102.6 and 107.6; 704x28x28 at 4.4 bits, chunks of 176,

@@ -6,6 +6,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
 #include <utility>
 #include <vector>
 
@@ -220,13 +221,15 @@ inline size_t spread_bytes(long long blocks, int sm_count, size_t own)
     if (per_sm <= 1) return kSpreadMost;
     return per_sm <= 8 ? (kSmBytes / (size_t)(per_sm + 1) / 1024 + 1) * 1024 - kBlockBytes - own : 0;
 }
-// Static shared memory of a kernel that is kept apart, asked for once: a byte or two of another variant's let one block more onto an SM.
-inline size_t static_bytes(const void *kernel)
+// Static shared memory of a kernel that is kept apart, asked for at its first launch (`known`, of that kernel): a byte or two of another variant's let
+// one block more onto an SM.
+inline size_t static_bytes(std::atomic<size_t> &known, const void *kernel)
 {
+    size_t bytes = known.load(std::memory_order_relaxed);
     cudaFuncAttributes at;
-    if (cudaFuncGetAttributes(&at, kernel) == cudaSuccess) return at.sharedSizeBytes;
-    cudaGetLastError();
-    return 0;
+    if (bytes == 0 && cudaFuncGetAttributes(&at, kernel) == cudaSuccess) known.store(bytes = at.sharedSizeBytes, std::memory_order_relaxed);
+    else if (bytes == 0) cudaGetLastError();
+    return bytes;
 }
 template <typename... P, typename... A>
 inline cudaError_t launch_first(bool alone, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A &&...args)

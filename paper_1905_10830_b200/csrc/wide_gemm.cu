@@ -376,8 +376,8 @@ tc_status tc_launch_encode_wide_gemm(const tc_ctx *ctx, const EncodeArgs &a, voi
         // Early for a tensor of one pass (400x7x7 x 3243, three of them, 296 -> 300 us); kept apart up to five blocks an SM (us in turn, early on the first SMs
         // that are free, and so: 128x1x1 x 18688, 4.0 an SM, 26.1, 32.2, 24.1; 64x7x7 x 404, 2.1, 20.9, 22.6, 20.4; 160x1x1 x 16512, 5.2, 24.6, 24.8, 28.4).
         const long long blocks = (long long)grid.x * grid.y;
-        static const size_t own = static_bytes((const void *)pixel_rows_kernel);
-        const size_t spread = a.alone && blocks <= 5ll * a.sms ? spread_bytes(blocks, a.sms, own) : 0;
+        static std::atomic<size_t> own;
+        const size_t spread = a.alone && blocks <= 5ll * a.sms ? spread_bytes(blocks, a.sms, static_bytes(own, (const void *)pixel_rows_kernel)) : 0;
         if (cudaFuncSetAttribute(pixel_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSpreadMost) != cudaSuccess) return TC_ERR_CUDA;
         if (launch_first(a.alone && per_pass >= a.n_tiles, pixel_rows_kernel, grid, 256, spread, s, (const __nv_bfloat16 *)a.x, a.c, a.hw, p0, p1, rows,
                          (unsigned long long *)a.ticket, t0 == 0 ? a.clear_words : 0ll) != cudaSuccess) return TC_ERR_CUDA;
