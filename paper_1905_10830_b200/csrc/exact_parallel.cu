@@ -845,12 +845,13 @@ tc_status tc_launch_pack_symbols(const tc_ctx *ctx, const EncodeArgs &a, const u
     // 22.7).  Not large blocks of which some SMs get two: the first SMs that are free take two each (576x14x14 x 128, 196 blocks of 1 024
     // threads: 55.4 -> 57.4).  Nor so many that little L1 is left, with tables per channel, which are looked up through it, from four an SM on (us in
     // turn and early: 784x14x14, 185 blocks a pass, at 7 bits 766 and 583, 400x14x14, 299, 285 and 227; 240x1x1 x 124928, 488 blocks, at 8 bits 211 and
-    // 231, 144x1x1 x 109568, 856, 81 and 111; one table: 192x7x7, 456 blocks, 80.1 and 77.2, 208x7x7 x 2100, 804, 74.8 and 82.0).
+    // 231, 144x1x1 x 109568, 856, 81 and 111; with one table from six on above
+    // 128 coefficients: 192x7x7, 456 blocks, 80.1 and 77.2, 208x7x7 x 2100, 804, 74.8 and 82.0, 32x27x19 x 282, 1131, 37.4 and 35.0).
     if (tile_blocks > 1)
         return launch_chained_cluster(tile_blocks, kernel, grid, block, std::max<size_t>(staging, kSpreadMost), s, a, sym, parts, first_tile, staging) == cudaSuccess ? TC_OK : TC_ERR_CUDA;
     const bool apart = tiles <= ctx->sm_count || tiles > 2ll * ctx->sm_count || block.x <= 512;
     static std::atomic<size_t> own[2];
-    const size_t spread = a.alone && apart && tiles <= (a.groups == 1 ? 5ll : 3ll) * ctx->sm_count ? spread_bytes(tiles, ctx->sm_count, static_bytes(own[a.groups != 1], (const void *)kernel)) : 0;
+    const size_t spread = a.alone && apart && tiles <= (a.groups != 1 ? 3ll : a.k <= 128 ? 8ll : 5ll) * ctx->sm_count ? spread_bytes(tiles, ctx->sm_count, static_bytes(own[a.groups != 1], (const void *)kernel)) : 0;
     if (spread > 0)
         return launch_chained(true, kernel, grid, block, std::max<size_t>(staging, spread), s, a, sym, parts, first_tile, staging) == cudaSuccess ? TC_OK : TC_ERR_CUDA;
     kernel<<<grid, block, staging, s>>>(a, sym, parts, first_tile, staging);
