@@ -1051,7 +1051,7 @@ void tc_encode_tc_list_classes(const tc_ctx *ctx, std::vector<EncodeArgs> &args,
         all_us += us;
     }
     for (size_t i = 0; i < args.size(); ++i) {
-        if (kind[i] < 0 || !(kind[i] & kEncodeFourGroups)) continue;
+        if (kind[i] < 0 || !(kind[i] & kEncodeFourGroups) || (all_us > kShortListUs && class_us[kind[i]] > kSharedListUs)) continue;
         args[i].epilogue_groups = 2;
         const int two = kernel_class(args[i], make_plan(ctx, args[i]));        // (not the same one less a bit: there is more room)
         if (all_us <= kShortListUs || (class_us[two] > 0.0 && class_us[two] + class_us[kind[i]] <= kSharedListUs)) kind[i] = two;

@@ -794,7 +794,6 @@ tc_status tc_launch_reconstruct(const DecodeArgs &a, int dtype, const uint8_t *s
     if (a.pixels <= 0) return TC_OK;
     const dim3 block(kPx, kRows), grid((unsigned int)((a.pixels + kPx - 1) / kPx), (unsigned int)((a.c + kOut - 1) / kOut));
     void (*kernel)(DecodeArgs, const uint8_t *) = dtype == TC_F32 ? reconstruct_kernel<float> : reconstruct_kernel<__nv_bfloat16>;
-    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSpreadMost) != cudaSuccess) return TC_ERR_CUDA;
     // Its blocks are there before the entropy decoder's are done, whose shared memory keeps them off the SMs with one, and pile onto others: kept apart where
     // an SM gets several (f32, us without and with: 256x8x16 x 10 47.0 and 31.6, 128x8x16 x 20 27.7 and 20.0, 64x8x16 x 36 18.1 and 15.1; fewer or
     // lighter ones lose by it, 32x8x16 x 17 13.4 and 14.2, 64x8x16 x 26 13.3 and 13.9; so do those that would fill all places, of which the decoder's blocks still have
@@ -802,6 +801,7 @@ tc_status tc_launch_reconstruct(const DecodeArgs &a, int dtype, const uint8_t *s
     const long long blocks = (long long)grid.x * grid.y;
     static std::atomic<size_t> own[2];
     const size_t spread = a.alone && blocks > (a.k >= 128 ? 2 : 3) * (long long)a.sms && 2 * blocks <= 15ll * a.sms ? spread_bytes(blocks, a.sms, static_bytes(own[dtype != TC_F32], (const void *)kernel)) : 0;
+    if (spread > 0 && cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSpreadMost) != cudaSuccess) return TC_ERR_CUDA;
     return launch_chained(a.alone, kernel, grid, block, spread, s, a, sym) == cudaSuccess ? TC_OK : TC_ERR_CUDA;
 }
 

@@ -378,7 +378,7 @@ tc_status tc_launch_encode_wide_gemm(const tc_ctx *ctx, const EncodeArgs &a, voi
         const long long blocks = (long long)grid.x * grid.y;
         static std::atomic<size_t> own;
         const size_t spread = a.alone && blocks <= 5ll * a.sms ? spread_bytes(blocks, a.sms, static_bytes(own, (const void *)pixel_rows_kernel)) : 0;
-        if (cudaFuncSetAttribute(pixel_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSpreadMost) != cudaSuccess) return TC_ERR_CUDA;
+        if (spread > 0 && cudaFuncSetAttribute(pixel_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSpreadMost) != cudaSuccess) return TC_ERR_CUDA;
         if (launch_first(a.alone && per_pass >= a.n_tiles, pixel_rows_kernel, grid, 256, spread, s, (const __nv_bfloat16 *)a.x, a.c, a.hw, p0, p1, rows,
                          (unsigned long long *)a.ticket, t0 == 0 ? a.clear_words : 0ll) != cudaSuccess) return TC_ERR_CUDA;
         GemmArgs g{};
